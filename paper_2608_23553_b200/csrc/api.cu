@@ -126,13 +126,26 @@ Layout make_layout(const Index &ix, const Params &p)
     L.cand = take(B * (size_t)p.maxc * sizeof(int32_t));
     L.n_cand = take(B * sizeof(int32_t));
     L.ci = take(B * (size_t)p.maxc * sizeof(int32_t));
-    const size_t two_phase = coarse_supported(p.nq) ? B * (size_t)p.maxc * sizeof(int32_t) : 0;
+    const bool filter = filter_used(ix, p);
+    const size_t two_phase = (coarse_supported(p.nq) || filter) ? B * (size_t)p.maxc * sizeof(int32_t) : 0;
     L.lo = take(two_phase);
     L.hi = take(two_phase);
     L.cont = take(two_phase);
-    L.cand_rng = take(2 * two_phase);
+    L.cand_rng = take(filter ? 0 : 2 * two_phase);
     L.cont_rng = take(2 * two_phase);
     L.n_cont = take(B * sizeof(int32_t));
+    L.flt_theta = take(filter ? B * nq * sizeof(int32_t) : 0);
+    L.flt_tab = take(filter ? B * filter_table_pitch(ix) : 0);
+    L.flt_hist = take(filter ? B * (size_t)filter_hist_bins() * sizeof(int32_t) : 0);
+    L.flt_thr = take(filter ? B * sizeof(int32_t) : 0);
+    L.flt_slot = L.lo;                  // (the filtered pipeline has no lower bounds)
+    L.flt_tau = take(filter ? B * sizeof(int32_t) : 0);
+    L.flt_parts = take(filter ? filter_parts_bytes(ix, p) : 0);
+    L.flt_counts = take(filter ? B * (size_t)filter_count_slots() * sizeof(int32_t) : 0);
+    L.kept = take(filter ? two_phase : 0);
+    L.kept_rng = take(filter ? 2 * two_phase : 0);
+    L.n_kept = take(filter ? B * sizeof(int32_t) : 0);
+    L.n_seed = take(filter ? B * sizeof(int32_t) : 0);
     L.pruned = take(B * p.n_prune * sizeof(int32_t));
     L.word_rank = take(B * (size_t)L.words * sizeof(int32_t));
     // partial-score table: dense rows per candidate (always for the RaBitQ refinement), or the hashed form
@@ -253,6 +266,13 @@ static int run(const Index &ix, const Params &p, int first, int last, const floa
     int32_t *n_cand = (int32_t *)(ws + L.n_cand);
     int32_t *ci = (int32_t *)(ws + L.ci);
     const bool two_phase = coarse_supported(p.nq) && !partial && !rabitq;
+    const bool filter = filter_used(ix, p) && !partial && !rabitq;      // (stage 3's first cut)
+    // blocks per query for the exact scores of a short list (two to three times n_prune documents): one per SM in a large
+    // batch, more when n_prune is large (about one block per eight survivors wanted; Large, n_prune 4096: 2.75 ms with
+    // 444-592 blocks against 3.26 ms with 148, Mid unchanged), four per SM when a single query has the GPU to itself
+    int exact_blocks = (4 * ix.sm_count + p.B - 1) / p.B;
+    if (exact_blocks < ix.sm_count) exact_blocks = ix.sm_count;
+    if (exact_blocks < p.n_prune / 8) exact_blocks = p.n_prune / 8;
     uint8_t *table8 = two_phase ? (uint8_t *)(ws + L.table8) : nullptr;
     int32_t *lo = (int32_t *)(ws + L.lo);
     int32_t *hi = (int32_t *)(ws + L.hi);
@@ -348,34 +368,54 @@ static int run(const Index &ix, const Params &p, int first, int last, const floa
             prof_mark(SLOT_CI, st);
             if ((rc = launch_select(ix, p, cand, n_cand, ci, pruned, n_pruned, pruned_ci, sel_scratch, st))) return rc;
             prof_mark(SLOT_SELECT, st);
-        } else if (two_phase) {
-            if (first > 1) {                       // the table came from the caller: derive its coarse copy
+        } else {
+            if (two_phase && first > 1) {          // the table came from the caller: derive its coarse copy
                 if ((rc = launch_coarse_table(ix, p, table, table8, st))) return rc;
                 prof_mark(SLOT_MISC, st);
             }
-            // bounds for every candidate, contenders for the top n_prune, exact CI and selection among those
-            if ((rc = launch_coarse_bounds(ix, p, table8, cand, n_cand, lo, hi, (int2 *)(ws + L.cand_rng), st))) return rc;
-            prof_mark(SLOT_CI, st);
-            if ((rc = launch_contenders(ix, p, cand, n_cand, lo, hi, cont, n_cont, ci, (const int2 *)(ws + L.cand_rng),
-                                        (int2 *)(ws + L.cont_rng), st))) return rc;
-            prof_mark(SLOT_SELECT, st);
-            // blocks per query for the few contenders (typically two to three times n_prune documents): one per SM
-            // in a large batch, more when n_prune is large (about one block per eight survivors wanted; Large,
-            // n_prune 4096: 2.75 ms with 444-592 blocks against 3.26 ms with 148, Mid unchanged), four per SM when a
-            // single query has the GPU to itself
-            int exact_blocks = (4 * ix.sm_count + p.B - 1) / p.B;
-            if (exact_blocks < ix.sm_count) exact_blocks = ix.sm_count;
-            if (exact_blocks < p.n_prune / 8) exact_blocks = p.n_prune / 8;
-            if ((rc = launch_centroid_interaction(ix, p, table, cont, n_cont, ci, exact_blocks, SLOT_CI_EXACT,
-                                                  ix.T < 0x7fffffffLL ? (const int2 *)(ws + L.cont_rng) : nullptr, st)))
+            // the documents that the steps below look at, and their token ranges
+            const int32_t *docs = cand, *n_docs = n_cand;
+            const int2 *docs_rng = ix.T < 0x7fffffffLL ? (const int2 *)(ws + L.cand_rng) : nullptr;
+            int2 *cont_rng = docs_rng ? (int2 *)(ws + L.cont_rng) : nullptr;
+            if (docs_rng && two_phase && !filter &&
+                (rc = launch_cand_ranges(ix, p, cand, n_cand, (int2 *)(ws + L.cand_rng), st)))
                 return rc;
-            prof_mark(SLOT_CI_EXACT, st);
-            if ((rc = launch_select(ix, p, cont, n_cont, ci, pruned, n_pruned, pruned_ci, nullptr, st))) return rc;
-            prof_mark(SLOT_SELECT, st);
-        } else {
-            if ((rc = launch_centroid_interaction(ix, p, table, cand, n_cand, ci, 0, SLOT_CI, nullptr, st))) return rc;
-            prof_mark(SLOT_CI, st);
-            if ((rc = launch_select(ix, p, cand, n_cand, ci, pruned, n_pruned, pruned_ci, sel_scratch, st))) return rc;
+            if (filter) {
+                if ((rc = launch_filter_scan(ix, p, L, table, table8, cand, n_cand, hi, cont, cont_rng, ws, st)))
+                    return rc;
+                if ((rc = launch_centroid_interaction(ix, p, table, cont, (const int32_t *)(ws + L.n_seed), ci, exact_blocks,
+                                                      SLOT_CI, cont_rng, st)))
+                    return rc;
+                prof_mark(SLOT_CI, st);
+                int32_t *kept = (int32_t *)(ws + L.kept), *n_kept = (int32_t *)(ws + L.n_kept);
+                int2 *kept_rng = (int2 *)(ws + L.kept_rng);
+                if ((rc = launch_filter_keep(ix, p, L, cand, n_cand, hi, ci, kept, kept_rng, n_kept, ws, st))) return rc;
+                prof_mark(SLOT_SELECT, st);
+                docs = kept; n_docs = n_kept; docs_rng = kept_rng;
+                if (two_phase) {                   // upper bounds of the kept ones from the 8-bit table
+                    if ((rc = launch_coarse_bounds(ix, p, table8, docs, n_docs, nullptr, hi, docs_rng, st))) return rc;
+                    prof_mark(SLOT_CI, st);
+                    if ((rc = launch_filter_contenders(ix, p, L, docs, docs_rng, n_docs, hi, cont, cont_rng, n_cont, ws, st)))
+                        return rc;
+                    prof_mark(SLOT_SELECT, st);
+                    docs = cont; n_docs = n_cont; docs_rng = cont_rng;
+                }
+            } else if (two_phase) {
+                // bounds for every candidate, contenders for the top n_prune, exact CI and selection among those
+                if ((rc = launch_coarse_bounds(ix, p, table8, docs, n_docs, lo, hi, docs_rng, st))) return rc;
+                prof_mark(SLOT_CI, st);
+                if ((rc = launch_contenders(ix, p, docs, n_docs, lo, hi, cont, n_cont, ci, docs_rng, cont_rng, st))) return rc;
+                prof_mark(SLOT_SELECT, st);
+                docs = cont; n_docs = n_cont; docs_rng = cont_rng;
+            }
+            const bool short_list = two_phase || filter;
+            if ((rc = launch_centroid_interaction(ix, p, table, docs, n_docs, ci, short_list ? exact_blocks : 0,
+                                                  short_list ? SLOT_CI_EXACT : SLOT_CI, docs_rng, st)))
+                return rc;
+            prof_mark(short_list ? SLOT_CI_EXACT : SLOT_CI, st);
+            if ((rc = launch_select(ix, p, docs, n_docs, ci, pruned, n_pruned, pruned_ci, short_list ? nullptr : sel_scratch,
+                                    st)))
+                return rc;
             prof_mark(SLOT_SELECT, st);
         }
     }
@@ -409,14 +449,16 @@ static int run(const Index &ix, const Params &p, int first, int last, const floa
         }
         if (first <= 3 && last >= 3) {
             if (taps->ci) {
-                if (two_phase) {                   // the search only needed exact CI for the contenders: the tap asks
+                if (two_phase || filter) {         // the search only needed exact CI for the contenders: the tap asks
                                                    // for every candidate, so the exact kernel runs over all of them
                     if ((rc = launch_centroid_interaction(ix, p, table, cand, n_cand, taps->ci, 0, SLOT_MISC, nullptr, st)))
                         return rc;
                 } else if ((rc = copy_d2d(taps->ci, ci, cand_bytes, st))) return rc;
             }
             if (taps->n_contenders &&
-                (rc = copy_d2d(taps->n_contenders, two_phase ? n_cont : n_cand, B * sizeof(int32_t), st)))
+                (rc = copy_d2d(taps->n_contenders,
+                               two_phase ? n_cont : filter ? (int32_t *)(ws + L.n_kept) : n_cand,
+                               B * sizeof(int32_t), st)))
                 return rc;
             if (taps->pruned && (rc = copy_d2d(taps->pruned, pruned, pruned_bytes, st))) return rc;
             if (taps->n_pruned && (rc = copy_d2d(taps->n_pruned, n_pruned, B * sizeof(int32_t), st))) return rc;

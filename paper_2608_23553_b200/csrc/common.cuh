@@ -57,7 +57,7 @@ struct Params {
     int64_t maxc;                     // candidate capacity per query
 };
 
-constexpr int MAX_GUARDS = 48;
+constexpr int MAX_GUARDS = 64;
 struct Layout {
     // debug builds (CHIMERA_DEBUG) put a 256-byte guard region behind every region below; guards[i] is its offset
     size_t guards[MAX_GUARDS];
@@ -87,6 +87,18 @@ struct Layout {
     size_t cand_rng;      // int2   [B][maxc]         (first token, length) of each candidate (bound scan)
     size_t cont_rng;      // int2   [B][maxc]         the same for the contenders
     size_t n_cont;        // int32  [B]
+    size_t flt_theta;     // int32  [B][nq]           first cut (g3_filter.cu): thresholds,
+    size_t flt_tab;       // uint8  [B][pitch]        one number per centroid,
+    size_t flt_hist;      // int32  [B][bins]         histogram of the bounds,
+    size_t flt_parts;     // int32  histograms and counters of the threshold kernel's blocks (few queries)
+    size_t flt_thr;       // int32  [B]               hi0 from which a candidate is a seed,
+    size_t flt_slot;      // int32  [B][maxc]         place of each seed in the seed list,
+    size_t flt_tau;       // int32  [B]               n_prune-th largest exact CI of the seeds,
+    size_t flt_counts;    // int32  [B][slots]        kept candidates per slice
+    size_t kept;          // int32  [B][maxc]         candidates that pass it, ascending
+    size_t kept_rng;      // int2   [B][maxc]         their token ranges
+    size_t n_kept;        // int32  [B]
+    size_t n_seed;        // int32  [B]
     size_t pruned;        // int32  [B][n_prune]
     size_t word_rank;     // int32  [B][words]        candidates before each bitmap word (document -> candidate index)
     size_t partial_m;     // int32  [B][maxc][nq]     per (candidate, query token) best retrieved-token score, or
@@ -175,17 +187,40 @@ int launch_partial_scores(const Index &ix, const Params &p, const Layout &L, con
                           const int32_t *table, const int32_t *probes, const uint32_t *bitmap,
                           const int32_t *word_rank, const int32_t *n_cand, int32_t *partial_m, int32_t *fprime, uint32_t *status,
                           cudaStream_t st);
+int launch_filter_contenders(const Index &ix, const Params &p, const Layout &L, const int32_t *kept, const int2 *kept_rng,
+                             const int32_t *n_kept, const int32_t *hi, int32_t *cont, int2 *cont_rng, int32_t *n_cont,
+                             char *ws, cudaStream_t st);
 bool coarse_supported(int nq);
 int launch_coarse_table(const Index &ix, const Params &p, const int32_t *table, uint8_t *table8, cudaStream_t st);
-// rng: int2 [B][maxc] scratch for the candidates' token ranges (may be NULL: per-document offset lookups instead).
+// The candidates' token ranges (corpora with fewer than 2^31 tokens).
+int launch_cand_ranges(const Index &ix, const Params &p, const int32_t *cand, const int32_t *n_cand, int2 *rng,
+                       cudaStream_t st);
+// rng: those ranges (may be NULL: per-document offset lookups instead; (CI, 0) stands for a document whose exact CI is
+// known).  lo may be NULL with ranges.
 int launch_coarse_bounds(const Index &ix, const Params &p, const uint8_t *table8, const int32_t *cand,
-                         const int32_t *n_cand, int32_t *lo, int32_t *hi, int2 *rng, cudaStream_t st);
+                         const int32_t *n_cand, int32_t *lo, int32_t *hi, const int2 *rng, cudaStream_t st);
+// First cut of the candidates by an upper bound from one number per token (g3_filter.cu).  launch_filter_scan leaves the
+// bounds in hi0 and the best ~1.5 n_prune candidates in seed / seed_rng (their number in the workspace's n_seed);
+// launch_filter_keep takes the seeds' exact CI and writes the candidates that can still be in the top n_prune, ascending;
+// launch_filter_contenders narrows them down by the 8-bit upper bounds.
+bool filter_used(const Index &ix, const Params &p);
+size_t filter_table_pitch(const Index &ix);
+int filter_hist_bins();
+int filter_count_slots();
+size_t filter_parts_bytes(const Index &ix, const Params &p);
+int launch_filter_scan(const Index &ix, const Params &p, const Layout &L, const int32_t *table, const uint8_t *table8,
+                       const int32_t *cand, const int32_t *n_cand, int32_t *hi0, int32_t *seed,
+                       int2 *seed_rng, char *ws, cudaStream_t st);
+int launch_filter_keep(const Index &ix, const Params &p, const Layout &L, const int32_t *cand,
+                       const int32_t *n_cand, const int32_t *hi0, const int32_t *seed_ci, int32_t *kept,
+                       int2 *kept_rng, int32_t *n_kept, char *ws, cudaStream_t st);
 // scratch: an int32 [B][maxc] array that is free during this step.
 // rng / cont_rng (may be NULL): the candidates' token ranges and where to put those of the contenders.
 int launch_contenders(const Index &ix, const Params &p, const int32_t *cand, const int32_t *n_cand, const int32_t *lo,
                       const int32_t *hi, int32_t *cont, int32_t *n_cont, int32_t *scratch, const int2 *rng,
                       int2 *cont_rng, cudaStream_t st);
-// rng (may be NULL): the token ranges of the listed documents, in list order.
+// rng (may be NULL, used when blocks_cap > 0): the token ranges of the listed documents, in list order; (CI, 0) stands
+// for a document whose CI is known.
 int launch_centroid_interaction(const Index &ix, const Params &p, const int32_t *table, const int32_t *cand,
                                 const int32_t *n_cand, int32_t *ci, int blocks_cap, int slot, const int2 *rng,
                                 cudaStream_t st);

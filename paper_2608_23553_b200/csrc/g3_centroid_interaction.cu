@@ -23,17 +23,19 @@
 #include <limits.h>
 
 #include "common.cuh"
+#include "g3_select.cuh"
 
 namespace chimera {
 
 constexpr int CI_THREADS = 256;
 constexpr int CI_WARPS = CI_THREADS / 32;
 
+// rng: NULL, or the documents' token ranges (first token, length); (CI, 0) stands for a document whose CI is known.
 template <int NQW>   // 32-column groups handled per lane
 __global__ void __launch_bounds__(CI_THREADS)
 ci_kernel(const int32_t *__restrict__ table, int64_t K, int nq, const int32_t *__restrict__ cand,
           const int32_t *__restrict__ n_cand, int64_t maxc, const int32_t *__restrict__ cids,
-          const int64_t *__restrict__ doc_off, int32_t *__restrict__ ci)
+          const int64_t *__restrict__ doc_off, const int2 *__restrict__ rng, int32_t *__restrict__ ci)
 {
     const int b = blockIdx.y;
     const int lane = threadIdx.x & 31;
@@ -43,8 +45,20 @@ ci_kernel(const int32_t *__restrict__ table, int64_t K, int nq, const int32_t *_
     int32_t *out = ci + (int64_t)b * maxc;
     const int warps_per_query = gridDim.x * CI_WARPS;
     for (int j = blockIdx.x * CI_WARPS + (threadIdx.x >> 5); j < n; j += warps_per_query) {
-        const int64_t d = DBG_DOC(cb[j]);
-        const int64_t t0 = doc_off[d], t1 = doc_off[d + 1];
+        int64_t t0, t1;
+        if (rng) {
+            const int2 r = rng[(int64_t)b * maxc + j];
+            if (r.y == 0) {
+                if (lane == 0) out[j] = r.x;
+                continue;
+            }
+            t0 = r.x;
+            t1 = t0 + r.y;
+        } else {
+            const int64_t d = DBG_DOC(cb[j]);
+            t0 = doc_off[d];
+            t1 = doc_off[d + 1];
+        }
         int m[NQW];
 #pragma unroll
         for (int w = 0; w < NQW; ++w) m[w] = INT_MIN;
@@ -170,20 +184,25 @@ ci_wide_rng_kernel(const int32_t *__restrict__ table, int64_t K, const int2 *__r
     const int j_end = j_begin + per_warp < n ? j_begin + per_warp : n;
     for (int jb = j_begin; jb < j_end; jb += 32) {
         const int cnt_docs = j_end - jb < 32 ? j_end - jb : 32;
-        const int2 mine = lane < cnt_docs ? rb[jb + lane] : make_int2(0, 1);
+        int2 mine = lane < cnt_docs ? rb[jb + lane] : make_int2(0, 1);
         int my_sum = 0;
+        if (mine.y == 0) {                                 // its CI is known and passes through
+            my_sum = mine.x;
+            mine.x = 0;
+        }
         int32_t nx_cid;
         {
             const int t0 = __shfl_sync(0xffffffffu, mine.x, 0), len = __shfl_sync(0xffffffffu, mine.y, 0);
-            nx_cid = cids[DBG_TOK((int64_t)t0 + (lane < len - 1 ? lane : len - 1))];
+            nx_cid = cids[DBG_TOK((int64_t)t0 + (lane < len - 1 ? lane : len > 0 ? len - 1 : 0))];
         }
         for (int di = 0; di < cnt_docs; ++di) {
             const int t0 = __shfl_sync(0xffffffffu, mine.x, di), len = __shfl_sync(0xffffffffu, mine.y, di);
             int32_t cidv = nx_cid;
             if (di + 1 < cnt_docs) {
                 const int n0 = __shfl_sync(0xffffffffu, mine.x, di + 1), nl = __shfl_sync(0xffffffffu, mine.y, di + 1);
-                nx_cid = cids[DBG_TOK((int64_t)n0 + (lane < nl - 1 ? lane : nl - 1))];
+                nx_cid = cids[DBG_TOK((int64_t)n0 + (lane < nl - 1 ? lane : nl > 0 ? nl - 1 : 0))];
             }
+            if (len == 0) continue;
             int4 m = make_int4(INT_MIN, INT_MIN, INT_MIN, INT_MIN);
             for (int base = 0; base < len; base += 32) {
                 const int cnt = len - base < 32 ? len - base : 32;
@@ -249,9 +268,6 @@ __device__ __forceinline__ int32_t coarse_hi(int packed, int nq)
 {
     return ((packed & 0xffff) << 16) + nq * ((1 << 16) - 1) + ((packed >> 16) & 0xff) * ((1 << 16) + 1);
 }
-// The histogram key of a lower bound in the contender step: floor(lo / 2^16) clamped at 0 -- a valid, slightly smaller
-// lower bound (documents with an empty column fall to the bottom, which only lowers the threshold).
-__device__ __forceinline__ int coarse_key(int32_t lo) { return lo < 0 ? 0 : lo >> 16; }
 // Running maxima of a lane's 16 columns in eight registers of two 16-bit fields each, updated from two rows at a time
 // with the three-input packed 16-bit maximum.  A field compares as (column byte << 8 | whatever lies below it), so the
 // winner's HIGH byte is the column's maximum and no widening is needed: the odd bytes of a word already sit in the high
@@ -437,15 +453,19 @@ ci_coarse_rng_body(const uint8_t *__restrict__ table8, int64_t K, const int2 *__
 
     for (int jb = j_begin; jb < j_end; jb += 32) {
         const int cnt = j_end - jb < 32 ? j_end - jb : 32;
-        const int2 mine = lane < cnt ? rb[jb + lane] : make_int2(0, 1);
+        int2 mine = lane < cnt ? rb[jb + lane] : make_int2(0, 1);
         int my_lo = 0, my_hi = 0;
+        if (mine.y == 0) {                             // its exact CI is known: both bounds
+            my_lo = my_hi = mine.x;
+            mine.x = 0;
+        }
         int32_t nx_cid[SLABS];
         {
             const int t0 = __shfl_sync(0xffffffffu, mine.x, 0), len = __shfl_sync(0xffffffffu, mine.y, 0);
 #pragma unroll
             for (int k = 0; k < SLABS; ++k) {
                 const int i = 32 * k + lane;
-                nx_cid[k] = cids[DBG_TOK((int64_t)t0 + (i < len - 1 ? i : len - 1))];
+                nx_cid[k] = cids[DBG_TOK((int64_t)t0 + (i < len - 1 ? i : len > 0 ? len - 1 : 0))];
             }
         }
         for (int di = 0; di < cnt; ++di) {
@@ -462,9 +482,10 @@ ci_coarse_rng_body(const uint8_t *__restrict__ table8, int64_t K, const int2 *__
 #pragma unroll
                 for (int k = 0; k < SLABS; ++k) {
                     const int i = 32 * k + lane;
-                    nx_cid[k] = cids[DBG_TOK((int64_t)n0 + (i < nl - 1 ? i : nl - 1))];
+                    nx_cid[k] = cids[DBG_TOK((int64_t)n0 + (i < nl - 1 ? i : nl > 0 ? nl - 1 : 0))];
                 }
             }
+            if (len == 0) continue;
             uint32_t m[8];
 #pragma unroll
             for (int r = 0; r < 8; ++r) m[r] = 0u;
@@ -531,7 +552,7 @@ ci_coarse_rng_body(const uint8_t *__restrict__ table8, int64_t K, const int2 *__
             }
         }
         if (lane < cnt) {
-            lo[(int64_t)b * maxc + jb + lane] = my_lo;
+            if (lo) lo[(int64_t)b * maxc + jb + lane] = my_lo;
             hi[(int64_t)b * maxc + jb + lane] = my_hi;
         }
     }
@@ -559,22 +580,25 @@ ci_coarse_rng_kernel_b4(const uint8_t *__restrict__ table8, int64_t K, const int
 
 bool coarse_supported(int nq) { return nq == 32 || nq == 64; }
 
+int launch_cand_ranges(const Index &ix, const Params &p, const int32_t *cand, const int32_t *n_cand, int2 *rng,
+                       cudaStream_t st)
+{
+    int64_t rb = ((int64_t)ix.sm_count * 8 + p.B - 1) / p.B;
+    const int64_t rwant = (p.maxc + 255) / 256;
+    if (rb > rwant) rb = rwant;
+    if (rb < 1) rb = 1;
+    cand_range_kernel<<<dim3((unsigned)rb, (unsigned)p.B), 256, 0, st>>>(cand, n_cand, p.maxc, ix.doc_off, rng);
+    CHIMERA_CUDA(cudaGetLastError());
+    count_launch(SLOT_CI);
+    return CHIMERA_OK;
+}
+
 int launch_coarse_bounds(const Index &ix, const Params &p, const uint8_t *table8, const int32_t *cand,
-                         const int32_t *n_cand, int32_t *lo, int32_t *hi, int2 *rng, cudaStream_t st)
+                         const int32_t *n_cand, int32_t *lo, int32_t *hi, const int2 *rng, cudaStream_t st)
 {
     const size_t table_bytes = (size_t)ix.K * p.nq;
-    // the candidates' token ranges, for this scan and for the exact scoring of the contenders afterwards
-    const bool use_rng = ix.T < 0x7fffffffLL && rng != nullptr;
-    if (use_rng) {
-        int64_t rb = ((int64_t)ix.sm_count * 8 + p.B - 1) / p.B;
-        const int64_t rwant = (p.maxc + 255) / 256;
-        if (rb > rwant) rb = rwant;
-        if (rb < 1) rb = 1;
-        cand_range_kernel<<<dim3((unsigned)rb, (unsigned)p.B), 256, 0, st>>>(cand, n_cand, p.maxc, ix.doc_off, rng);
-        CHIMERA_CUDA(cudaGetLastError());
-        count_launch(SLOT_CI);
-    }
-    if (table_bytes <= 160 * 1024) {
+    const bool use_rng = rng != nullptr;
+    if (table_bytes <= 160 * 1024 && lo != nullptr) {
         // the whole 8-bit table of a query fits in shared memory: stage it once per block and look rows up there
         constexpr int T = 512;
         int64_t gx = (4LL * ix.sm_count + p.B - 1) / p.B;       // every block re-reads the table: few, long blocks
@@ -663,7 +687,8 @@ int launch_centroid_interaction(const Index &ix, const Params &p, const int32_t 
     if (gx < 1) gx = 1;
     dim3 grid(gx, (unsigned)p.B);
     const int nqw = (p.nq + 31) / 32;
-    if (rng != nullptr && (p.nq == 32 || p.nq == 64)) {       // the listed documents' token ranges are known
+    const int2 *grng = blocks_cap > 0 ? rng : nullptr;
+    if (rng != nullptr && blocks_cap > 0 && (p.nq == 32 || p.nq == 64)) {       // the listed documents' token ranges are known
         if (p.nq == 32)
             ci_wide_rng_kernel<8><<<grid, CI_THREADS, 0, st>>>(table, ix.K, rng, n_cand, p.maxc, ix.cids, ci);
         else
@@ -677,99 +702,17 @@ int launch_centroid_interaction(const Index &ix, const Params &p, const int32_t 
     else if (p.nq == 64)
         ci_wide_kernel<16><<<grid, CI_THREADS, 0, st>>>(table, ix.K, cand, n_cand, p.maxc, ix.cids, ix.doc_off, ci);
     else if (nqw == 1)
-        ci_kernel<1><<<grid, CI_THREADS, 0, st>>>(table, ix.K, p.nq, cand, n_cand, p.maxc, ix.cids, ix.doc_off, ci);
+        ci_kernel<1><<<grid, CI_THREADS, 0, st>>>(table, ix.K, p.nq, cand, n_cand, p.maxc, ix.cids, ix.doc_off, grng, ci);
     else if (nqw == 2)
-        ci_kernel<2><<<grid, CI_THREADS, 0, st>>>(table, ix.K, p.nq, cand, n_cand, p.maxc, ix.cids, ix.doc_off, ci);
+        ci_kernel<2><<<grid, CI_THREADS, 0, st>>>(table, ix.K, p.nq, cand, n_cand, p.maxc, ix.cids, ix.doc_off, grng, ci);
     else
-        ci_kernel<4><<<grid, CI_THREADS, 0, st>>>(table, ix.K, p.nq, cand, n_cand, p.maxc, ix.cids, ix.doc_off, ci);
+        ci_kernel<4><<<grid, CI_THREADS, 0, st>>>(table, ix.K, p.nq, cand, n_cand, p.maxc, ix.cids, ix.doc_off, grng, ci);
     CHIMERA_CUDA(cudaGetLastError());
     count_launch(slot);
     return CHIMERA_OK;
 }
 
 // ------------------------------------------------------------------------------------------------ selection ------
-constexpr int SEL_THREADS = 1024;
-
-// Exclusive prefix sum over the block (SEL_THREADS threads); *total gets the block sum.  Two barriers.
-__device__ __forceinline__ int sel_block_scan(int v, int *total, int *warp_part /* [32] */)
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int incl = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        int t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += t;
-    }
-    __syncthreads();                     // warp_part may still be read from a previous call
-    if (lane == 31) warp_part[warp] = incl;
-    __syncthreads();
-    int pw = warp_part[lane];            // 32 warps
-    int pincl = pw;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        int t = __shfl_up_sync(0xffffffffu, pincl, o);
-        if (lane >= o) pincl += t;
-    }
-    *total = __shfl_sync(0xffffffffu, pincl, 31);
-    int before = __shfl_sync(0xffffffffu, pincl - pw, warp);
-    return before + incl - v;
-}
-
-// Radix select (11 + 11 + 10 bits, most significant first) of the `want`-th largest value of sb[0..n) in the order of
-// u = value ^ 0x80000000.  Needs n >= want >= 1.  Returns that value's u; *need_eq = how many entries equal to it
-// belong to the top `want` (the rest of the top `want` are strictly greater).  Whole block, uniform.
-template <class Load>     // load(j) = value j (int32)
-__device__ __forceinline__ uint32_t radix_select(Load load, int n, int want_in, int *hist, int *warp_part,
-                                                 uint32_t *s_prefix, int *s_want, int *need_eq)
-{
-    if (threadIdx.x == 0) { *s_prefix = 0u; *s_want = want_in; }
-    const int shifts[3] = {21, 10, 0};
-    const int widths[3] = {11, 11, 10};
-    uint32_t known_mask = 0u;
-    for (int pass = 0; pass < 3; ++pass) {
-        const int shift = shifts[pass], bins = 1 << widths[pass];
-        for (int i = threadIdx.x; i < 2048; i += SEL_THREADS) hist[i] = 0;
-        __syncthreads();
-        const uint32_t prefix = *s_prefix;
-        const int want = *s_want;
-        // eight independent loads per thread before their histogram updates (the loop is latency-bound otherwise)
-        for (int base = 0; base < n; base += 8 * SEL_THREADS) {
-            uint32_t u[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const int j = base + e * SEL_THREADS + threadIdx.x;
-                u[e] = j < n ? ((uint32_t)load(j) ^ 0x80000000u) : 0u;
-            }
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const int j = base + e * SEL_THREADS + threadIdx.x;
-                if (j < n && (u[e] & known_mask) == prefix) atomicAdd(&hist[(u[e] >> shift) & (bins - 1)], 1);
-            }
-        }
-        __syncthreads();
-        // descending bins: thread t owns bins (bins-1-2t) and (bins-2-2t)
-        int hi_bin = bins - 1 - 2 * (int)threadIdx.x, lo_bin = hi_bin - 1;
-        int h_hi = hi_bin >= 0 ? hist[hi_bin] : 0;
-        int h_lo = lo_bin >= 0 ? hist[lo_bin] : 0;
-        int total;
-        int before = sel_block_scan(h_hi + h_lo, &total, warp_part);
-        // the wanted rank falls in the first bin whose cumulative count reaches `want`
-        if (before < want && want <= before + h_hi + h_lo) {
-            if (want <= before + h_hi) {
-                *s_prefix = prefix | ((uint32_t)hi_bin << shift);
-                *s_want = want - before;
-            } else {
-                *s_prefix = prefix | ((uint32_t)lo_bin << shift);
-                *s_want = want - before - h_hi;
-            }
-        }
-        known_mask |= (uint32_t)(bins - 1) << shift;
-        __syncthreads();
-    }
-    *need_eq = *s_want;
-    return *s_prefix;
-}
-
 // grid (B).  pruned[b][0..n_prune) ascending ids, -1 padded; n_pruned[b]; pruned_ci (optional): the score of each
 // kept document, INT_MIN beside every -1.
 __global__ void __launch_bounds__(SEL_THREADS)
@@ -846,7 +789,6 @@ select_kernel(const int32_t *__restrict__ cand, const int32_t *__restrict__ n_ca
 // coarse_key(lo) = floor(lo / 2^16), clamped at 0, is a key of at most 14 bits and 2^16 key <= lo: one histogram sweep
 // over CONT_BINS bins (two neighbouring keys share a bin for q_len 64; tau is then the smaller of the two, still a
 // valid lower threshold) finds tau without radix passes.
-constexpr int CONT_BINS = 8192;
 __global__ void __launch_bounds__(SEL_THREADS)
 contender_kernel(const int32_t *__restrict__ cand, const int32_t *__restrict__ n_cand, const int32_t *__restrict__ lo,
                  const int32_t *__restrict__ hi, int64_t maxc, int n_prune, int nq, int32_t *__restrict__ cont,
@@ -1136,7 +1078,6 @@ int launch_contenders(const Index &ix, const Params &p, const int32_t *cand, con
                       const int32_t *hi, int32_t *cont, int32_t *n_cont, int32_t *scratch, const int2 *rng,
                       int2 *cont_rng, cudaStream_t st)
 {
-    if (ix.T >= 0x7fffffffLL) { rng = nullptr; cont_rng = nullptr; }      // the bound scan wrote no ranges
     if (4 * p.B <= ix.sm_count && p.maxc >= CONT_BINS + CONT_SPLIT + 1) {
         // few queries: CONT_SPLIT blocks each
         CHIMERA_CUDA(cudaMemset2DAsync(scratch, sizeof(int32_t) * (size_t)p.maxc, 0, sizeof(int32_t) * CONT_BINS,

@@ -1,0 +1,829 @@
+// Stage 3, first cut: an upper bound on CI from ONE number per document token, so that the row lookups of the later
+// phases (g3_centroid_interaction.cu) run over a small part of the candidates only.
+//
+// For any thresholds theta_i,  max_t S[c_t, i] <= theta_i + sum_t (S[c_t, i] - theta_i)+ , so with
+//     e(c) = sum_i (S[c, i] - theta_i)+                    (one number per centroid and query)
+//     CI(d) = sum_i max_t S[c_t, i]  <=  sum_i theta_i + sum_t e(c_t) = hi0(d).
+// theta_i is set so that about FILTER_LAMBDA of a document's tokens exceed it: lower thresholds count a column's second
+// and third best tokens as well, higher ones replace the column's true maximum by theta.  Any choice is correct; with one
+// token per column of a long document the bound keeps 7-13 % of the candidates when 1 % are wanted (65,536 and 262,144
+// centroids, candidates of 85-512 tokens), with half or one and a half times as many up to twice that.
+//
+//   filter_theta_kernel    theta_i from a sample of the table's rows
+//   filter_excess_kernel   e(c) of every centroid, rounded up (16 bits, or 6-bit codes five to a word for large K)
+//   filter_scan_kernel     hi0 of every candidate: the query's whole e table in shared memory, one lookup per token
+//   filter_seed_kernel     the ~1.5 n_prune candidates with the largest hi0 (their order does not matter)
+//   (their exact CI: g3_centroid_interaction.cu)
+//   filter_count_kernel,   tau = the n_prune-th largest of those, a lower bound on the n_prune-th largest CI; keeps every
+//   filter_write_kernel    candidate with hi0 >= tau, ascending, with its token range
+//   (q_len 32 / 64: upper bounds of the kept ones from the 8-bit table: g3_centroid_interaction.cu)
+//   filter_contend_kernel  and of those the ones whose bound reaches tau
+//   (exact CI of what is left, except for the seeds, and the exact selection: g3_centroid_interaction.cu)
+// Every document of the exact top n_prune has an upper bound >= CI >= tau, so it is never dropped and the result is the
+// same as without these cuts.
+#include <limits.h>
+
+#include "g3_select.cuh"
+
+namespace chimera {
+
+constexpr double FILTER_LAMBDA = 1.0;     // wanted tokens of a document above theta, per query token
+constexpr int FILTER_SAMPLE = 4096;       // table rows sampled per query for theta
+constexpr int KEEP_SPLIT = 32;            // most blocks per query of the selection kernels
+constexpr int FILTER_BINS = 2048;         // histogram bins of sum_t e(c_t), 2^17 (one 128th) each
+constexpr int64_t FILTER_SMEM = 208 * 1024;   // shared memory of the scan's block that its e table may take
+
+// 6-bit codes of e in units of 2^16 (1/256): exact up to 20, then steps of about 7 % (the sums of a document's far
+// tokens are 1-30, a token of a probed centroid adds about 180), a few large ones for centroids near several query
+// tokens, and the largest possible value (127 * 257).
+struct FilterLevels { uint16_t v[64]; };
+constexpr FilterLevels filter_levels()
+{
+    FilterLevels l{};
+    for (int j = 0; j <= 20; ++j) l.v[j] = (uint16_t)j;
+    for (int j = 21; j < 60; ++j) l.v[j] = (uint16_t)(l.v[j - 1] + (l.v[j - 1] * 19 >> 8) + 1);
+    l.v[60] = 1024; l.v[61] = 2048; l.v[62] = 8192; l.v[63] = 32640;
+    return l;
+}
+__constant__ FilterLevels c_levels = filter_levels();
+
+// How the e table of a query is kept: 16 = 16-bit values (K <= 106,496), 6 = 6-bit codes (K <= 266,240), 0 = not at all.
+static int filter_codec(int64_t K)
+{
+    if (K * 2 <= FILTER_SMEM) return 16;
+    if ((K + 4) / 5 * 4 <= FILTER_SMEM) return 6;
+    return 0;
+}
+
+// When the cut runs.  The table has to fit one SM's shared memory; a token position has to fit 32 bits and a document's
+// sum of e 31 bits; and there has to be enough to scan that the additional launches pay: 13 against 8 kernels for q_len
+// 32 / 64, whose other form scans 8-bit rows (one query of 60 M tokens, 14 M of them candidates': 248 us with the cut, 225
+// without; one of 16 queries with 48 M candidate tokens each: 5.4 against 6.7 ms), 9 against 6 for the others, which
+// look up exact rows (8 queries of 20 M tokens: 3.3 against 5.8 ms).
+bool filter_used(const Index &ix, const Params &p)
+{
+    if (filter_codec(ix.K) == 0 || ix.T >= 0x7fffff00LL || ix.max_doclen > 32000) return false;
+    if (p.maxc < 4 * (int64_t)p.n_prune) return false;
+    return (double)p.B * (double)p.maxc * ((double)ix.T / (double)ix.N) >= (coarse_supported(p.nq) ? 2e8 : 2e7);
+}
+size_t filter_table_pitch(const Index &ix)
+{
+    const int codec = filter_codec(ix.K);
+    const size_t bytes = codec == 16 ? (size_t)ix.K * 2 : codec == 6 ? (size_t)(ix.K + 4) / 5 * 4 : 0;
+    return (bytes + 15) & ~(size_t)15;
+}
+int filter_hist_bins() { return FILTER_BINS; }
+int filter_count_slots() { return KEEP_SPLIT; }
+// Blocks per query of the selection kernels: about four per SM, slices of 4,096 candidates or more.
+static int filter_split(const Index &ix, const Params &p)
+{
+    int64_t g = (4LL * ix.sm_count + p.B - 1) / p.B;
+    if (g > (p.maxc + 4095) / 4096) g = (p.maxc + 4095) / 4096;
+    return (int)(g > KEEP_SPLIT ? KEEP_SPLIT : g < 1 ? 1 : g);
+}
+
+// Blocks per query and column group of the theta kernel, and the bytes they share.
+static int filter_parts(const Index &ix, const Params &p) { return 4 * p.B <= ix.sm_count ? 8 : 1; }
+size_t filter_parts_bytes(const Index &ix, const Params &p)
+{
+    return filter_parts(ix, p) > 1 ? sizeof(int32_t) * (size_t)p.B * ((p.nq + 31) / 32) * (256 * 32 + 1) : 0;
+}
+
+// ------------------------------------------------------------------------------------------------ thresholds ------
+// grid (ceil(nq / 32), B, parts), lane = query token.  theta[b][i] = the smallest t (in units of 2^16) such that at most
+// `rank` of the m sampled rows (every step-th one) have S >= t 2^16.  With few queries the sample is split over several
+// blocks that add their histograms up in `parts_hist` ([B][groups][256 * 32], zero before and afterwards); the last one to
+// finish (`done`, likewise) reads the sum.  Also clears what the scan and the seed selection add to.
+__global__ void __launch_bounds__(SEL_THREADS)
+filter_theta_kernel(const int32_t *__restrict__ table, int64_t K, int nq, int m, int step, int rank,
+                    int32_t *__restrict__ theta, int32_t *__restrict__ hist_out, int32_t *__restrict__ n_seed,
+                    int32_t *__restrict__ parts_hist, int32_t *__restrict__ done)
+{
+    __shared__ int hist[256 * 32];
+    __shared__ int s_last;
+    const int b = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int col = blockIdx.x * 32 + lane;
+    for (int i = threadIdx.x; i < 256 * 32; i += SEL_THREADS) hist[i] = 0;
+    if (blockIdx.x == 0 && blockIdx.z == 0) {
+        for (int i = threadIdx.x; i < FILTER_BINS; i += SEL_THREADS) hist_out[(int64_t)b * FILTER_BINS + i] = 0;
+        if (threadIdx.x == 0) n_seed[b] = 0;
+    }
+    __syncthreads();
+    const int32_t *tb = table + (int64_t)b * K * nq + col;
+    const int64_t row = (int64_t)step * nq;
+    for (int r0 = blockIdx.z * 32 + warp; r0 < m; r0 += gridDim.z * 32 * 16) {
+        int32_t v[16];
+#pragma unroll
+        for (int u = 0; u < 16; ++u) {
+            const int r = r0 + gridDim.z * 32 * u;
+            v[u] = (r < m && col < nq) ? tb[r * row] : -1;
+        }
+#pragma unroll
+        for (int u = 0; u < 16; ++u) {
+            const int k = v[u] >> 16;
+            if (k > 0) atomicAdd(&hist[(k > 255 ? 255 : k) * 32 + lane], 1);
+        }
+    }
+    __syncthreads();
+    if (gridDim.z > 1) {
+        int32_t *ph = parts_hist + ((int64_t)b * gridDim.x + blockIdx.x) * 256 * 32;
+        for (int i = threadIdx.x; i < 256 * 32; i += SEL_THREADS)
+            if (hist[i]) atomicAdd(&ph[i], hist[i]);
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) s_last = atomicAdd(&done[(int64_t)b * gridDim.x + blockIdx.x], 1) == (int)gridDim.z - 1;
+        __syncthreads();
+        if (!s_last) return;
+        __threadfence();
+        for (int i = threadIdx.x; i < 256 * 32; i += SEL_THREADS) {
+            hist[i] = __ldcg(&ph[i]);
+            ph[i] = 0;
+        }
+        if (threadIdx.x == 0) done[(int64_t)b * gridDim.x + blockIdx.x] = 0;
+        __syncthreads();
+    }
+    // warp w finds column w's threshold: lane l holds buckets 255 - 8 l ... 248 - 8 l, descending
+    int h[8], mine = 0;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) { h[e] = hist[(255 - 8 * lane - e) * 32 + warp]; mine += h[e]; }
+    int incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+    }
+    int above = incl - mine, best = 256;                     // the lowest t whose count is within the rank
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        above += h[e];
+        if (above <= rank) best = 255 - 8 * lane - e;
+    }
+    best = __reduce_min_sync(0xffffffffu, best);
+    if (best < 1) best = 1;
+    if (lane == 0 && blockIdx.x * 32 + warp < nq) theta[(int64_t)b * nq + blockIdx.x * 32 + warp] = best;
+}
+
+// ------------------------------------------------------------------------------------------------ excess table ----
+// Smallest code whose level is >= e.
+__device__ __forceinline__ int filter_encode(const uint8_t *enc, int e)
+{
+    return e < 512 ? enc[e] : e <= 1024 ? 60 : e <= 2048 ? 61 : e <= 8192 ? 62 : 63;
+}
+__device__ __forceinline__ void filter_fill_encoder(uint8_t *enc)
+{
+    for (int e = threadIdx.x; e < 512; e += blockDim.x) {
+        int j = 0;
+        while (c_levels.v[j] < e) ++j;
+        enc[e] = (uint8_t)j;
+    }
+    __syncthreads();
+}
+
+// e(c) in units of 2^16 from a row of the 8-bit table: S < 2^16 (u + 1), and for u = 255 S <= 2^16 * 257.  tm1[k]: the
+// thresholds minus one, the even bytes of word k in tm1[k].x and the odd ones in tm1[k].y (16-bit fields), so that
+// sum_i (u_i + 1 - t_i)+ = sum_i max(u_i, t_i - 1) - sum_i (t_i - 1).
+template <int WORDS>
+__device__ __forceinline__ int filter_row_excess(const uint4 *row, const uint2 *tm1, int sum_tm1)
+{
+    uint32_t acc = 0;
+    int full = 0;
+#pragma unroll
+    for (int q = 0; q < WORDS / 4; ++q) {
+        const uint4 v = __ldg(row + q);
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const uint2 t = tm1[4 * q + k];
+            acc += __vmaxu2(w[k] & 0x00ff00ffu, t.x);
+            acc += __vmaxu2((w[k] >> 8) & 0x00ff00ffu, t.y);
+            full += __popc((((w[k] & 0x7f7f7f7fu) + 0x01010101u) & w[k]) & 0x80808080u);
+        }
+    }
+    return (int)(acc & 0xffffu) + (int)(acc >> 16) - sum_tm1 + full;      // fields <= 32 * 256
+}
+
+// grid (blocks, B).  One thread per centroid (16-bit values) or per five centroids (6-bit codes): a stream of the 8-bit
+// table (Mid, batch 256: 537 MB).
+template <int WORDS, int CODEC>
+__global__ void __launch_bounds__(256)
+filter_excess_kernel(const uint8_t *__restrict__ table8, int64_t K, const int32_t *__restrict__ theta,
+                     uint8_t *__restrict__ out, size_t pitch)
+{
+    __shared__ uint2 tm1[WORDS];
+    __shared__ int s_sum;
+    __shared__ uint8_t enc[512];
+    const int b = blockIdx.y;
+    const int32_t *th = theta + (int64_t)b * 4 * WORDS;
+    if (threadIdx.x < WORDS) {
+        const int32_t *t = th + 4 * threadIdx.x;
+        tm1[threadIdx.x] = make_uint2((uint32_t)(t[0] - 1) | (uint32_t)(t[2] - 1) << 16,
+                                      (uint32_t)(t[1] - 1) | (uint32_t)(t[3] - 1) << 16);
+    }
+    if (threadIdx.x == 0) {
+        int s = 0;
+        for (int i = 0; i < 4 * WORDS; ++i) s += th[i] - 1;
+        s_sum = s;
+    }
+    if (CODEC == 6) filter_fill_encoder(enc);
+    __syncthreads();
+    const uint4 *tb = reinterpret_cast<const uint4 *>(table8 + (int64_t)b * K * 4 * WORDS);
+    uint8_t *ob = out + (size_t)b * pitch;
+    const int sum = s_sum;
+    if (CODEC == 16) {
+        for (int64_t c = (int64_t)blockIdx.x * 256 + threadIdx.x; c < K; c += (int64_t)gridDim.x * 256)
+            reinterpret_cast<uint16_t *>(ob)[c] = (uint16_t)filter_row_excess<WORDS>(tb + c * (WORDS / 4), tm1, sum);
+    } else {
+        const int64_t words = (K + 4) / 5;
+        for (int64_t w = (int64_t)blockIdx.x * 256 + threadIdx.x; w < words; w += (int64_t)gridDim.x * 256) {
+            uint32_t packed = 0;
+#pragma unroll
+            for (int r = 0; r < 5; ++r) {
+                const int64_t c = w * 5 + r < K ? w * 5 + r : K - 1;
+                packed |= (uint32_t)filter_encode(enc, filter_row_excess<WORDS>(tb + c * (WORDS / 4), tm1, sum)) << (6 * r + (r > 2));
+            }
+            reinterpret_cast<uint32_t *>(ob)[w] = packed;
+        }
+    }
+}
+
+// The same from the exact table, for any q_len: one warp per row, values rounded up to units of 2^us.
+template <int CODEC>
+__global__ void __launch_bounds__(256)
+filter_excess_exact_kernel(const int32_t *__restrict__ table, int64_t K, int nq, const int32_t *__restrict__ theta, int us,
+                           uint8_t *__restrict__ out, size_t pitch)
+{
+    __shared__ uint8_t enc[512];
+    if (CODEC == 6) filter_fill_encoder(enc);
+    const int b = blockIdx.y, lane = threadIdx.x & 31;
+    int th[4];
+#pragma unroll
+    for (int w = 0; w < 4; ++w) th[w] = lane + 32 * w < nq ? theta[(int64_t)b * nq + lane + 32 * w] << 16 : 0;
+    const int32_t *tb = table + (int64_t)b * K * nq;
+    uint8_t *ob = out + (size_t)b * pitch;
+    constexpr int PER = CODEC == 16 ? 8 : 5;                          // rows per warp and iteration
+    const int64_t groups = (K + PER - 1) / PER;
+    for (int64_t g = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); g < groups; g += (int64_t)gridDim.x * 8) {
+        int e[PER];
+#pragma unroll
+        for (int r = 0; r < PER; ++r) e[r] = 0;
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+            if (32 * w < nq) {
+                int v[PER];
+#pragma unroll
+                for (int r = 0; r < PER; ++r)
+                    v[r] = (lane + 32 * w < nq && g * PER + r < K) ? __ldg(tb + (g * PER + r) * nq + lane + 32 * w) : 0;
+#pragma unroll
+                for (int r = 0; r < PER; ++r) e[r] += max(v[r] - th[w], 0);
+            }
+        }
+        uint32_t packed = 0;
+        int val = 0;
+#pragma unroll
+        for (int r = 0; r < PER; ++r) {
+            // the sum of 127 columns stays below 2^31; + the rounding, so add in unsigned
+            const uint32_t s = ((uint32_t)__reduce_add_sync(0xffffffffu, e[r]) + ((1u << us) - 1)) >> us;
+            if (CODEC == 16) { if (lane == r) val = (int)s; }
+            else packed |= (uint32_t)filter_encode(enc, (int)s) << (6 * r + (r > 2));
+        }
+        if (CODEC == 16) {
+            if (lane < PER && g * PER + lane < K) reinterpret_cast<uint16_t *>(ob)[g * PER + lane] = (uint16_t)val;
+        } else if (lane == 0) {
+            reinterpret_cast<uint32_t *>(ob)[g] = packed;
+        }
+    }
+}
+
+// ------------------------------------------------------------------------------------------------ scan ------------
+// grid (blocks per query, B), one block of 1,024 threads per SM, the query's e table in shared memory.  Eight lanes take
+// a document: each loads four consecutive centroid ids with one 16-byte load (a group reads a 128-byte line), looks
+// the four up in shared memory (32 random banks: about 3.5 wavefronts per 32 tokens, against one L1 line per token for
+// the row lookups of the later phases) and adds.  A warp holds four documents and has the loads of its next 64 tokens
+// per document -- of the same documents or of the next four -- in flight while the present ones are looked up.
+// The instruction pipe is the limit, so lanes must not idle: the block takes its candidates in windows of 1,024, one
+// thread per candidate finds the token range (loads issued a window ahead), and a counting sort by number of 32-token
+// chunks gives every warp four documents of about the same length.
+//   hi0   [B][maxc]         sum_i theta_i + sum_t e(c_t) in units of 2^us
+//   hist  [B][FILTER_BINS]  of sum_t e(c_t) in units of 2^17
+constexpr int SCAN_THREADS_F = 1024;
+constexpr int SCAN_SORT_BINS = 64;
+
+template <int CODEC>
+__global__ void __launch_bounds__(SCAN_THREADS_F, 1)
+filter_scan_kernel(const uint8_t *__restrict__ tab, size_t pitch, const int32_t *__restrict__ theta, int nq, int us,
+                   const int32_t *__restrict__ cand, const int64_t *__restrict__ doc_off,
+                   const int32_t *__restrict__ n_cand, int64_t maxc, const int32_t *__restrict__ cids, int64_t T,
+                   int32_t *__restrict__ hi0, int32_t *__restrict__ hist)
+{
+    extern __shared__ uint4 s_tab[];
+    __shared__ uint32_t s_level[64];
+    __shared__ int s_hist[FILTER_BINS];
+    __shared__ int s_sort[SCAN_SORT_BINS];
+    __shared__ uint2 s_rng[SCAN_THREADS_F];
+    __shared__ uint16_t s_idx[SCAN_THREADS_F];
+    __shared__ int s_theta;
+    const int b = blockIdx.y, tid = threadIdx.x;
+    const int n = n_cand[b];
+    const int per = (n + (int)gridDim.x - 1) / (int)gridDim.x;
+    const int j0 = blockIdx.x * per, j1 = j0 + per < n ? j0 + per : n;
+    if (j0 >= n) return;
+    const int lane = tid & 31, warp = tid >> 5, grp = lane >> 3, sub = lane & 7;
+    const int32_t *cb = cand + (int64_t)b * maxc;
+    int32_t *out = hi0 + (int64_t)b * maxc;
+
+    // token range of this thread's candidate of a window; an empty one past the end
+    auto range_of = [&](int32_t d) {
+        if (d < 0) return make_int2(0, 0);
+        d = DBG_DOC(d);
+        const int64_t t0 = __ldg(doc_off + d);
+        return make_int2((int)t0, (int)(__ldg(doc_off + d + 1) - t0));
+    };
+    auto cand_of = [&](int base) { return base + tid < j1 ? __ldg(cb + base + tid) : -1; };
+    int2 nx_rng = range_of(cand_of(j0));
+    int32_t nx_cand = cand_of(j0 + SCAN_THREADS_F);
+
+    const uint4 *src = reinterpret_cast<const uint4 *>(tab + (size_t)b * pitch);
+#pragma unroll 4
+    for (int i = tid; i < (int)(pitch / 16); i += SCAN_THREADS_F) s_tab[i] = __ldg(src + i);
+    for (int i = tid; i < FILTER_BINS; i += SCAN_THREADS_F) s_hist[i] = 0;
+    if (tid < 64) { s_level[tid] = c_levels.v[tid]; s_sort[tid] = 0; }
+    if (tid < 32) {
+        int s = 0;
+        for (int i = tid; i < nq; i += 32) s += theta[(int64_t)b * nq + i];
+        s = __reduce_add_sync(0xffffffffu, s);
+        if (tid == 0) s_theta = s << (16 - us);
+    }
+    __syncthreads();
+    const uint16_t *tab16 = reinterpret_cast<const uint16_t *>(s_tab);
+    const uint32_t *tab6 = reinterpret_cast<const uint32_t *>(s_tab);
+
+    // Positions count from the 16-byte boundary at or below cids.  Whole 16-byte groups inside the array are [edge_lo, edge_hi):
+    // only the corpus's first and last documents can reach beyond, and the thread that owns one adds those tokens itself.
+    const uint32_t mis = (uint32_t)(((uintptr_t)cids >> 2) & 3);
+    const int4 *c4 = reinterpret_cast<const int4 *>(cids - mis);
+    const uint32_t edge_lo = mis ? 4u : 0u, edge_hi = (mis + (uint32_t)T) & ~3u;
+    auto load4 = [&](uint32_t q, uint32_t hi) { return q < hi ? __ldg(c4 + (q >> 2)) : make_int4(0, 0, 0, 0); };
+    auto value = [&](int32_t c) -> int {
+        c = DBG_CID(c);
+        if (CODEC == 16) return tab16[c];
+        // c / 5 in the high word, (c % 5) / 5 in the low one: its top five bits are the bit positions 0, 6, 12, 19, 25
+        const unsigned long long pr = (unsigned long long)(uint32_t)c * 858993460u;
+        return (int)s_level[(tab6[pr >> 32] >> ((uint32_t)pr >> 27)) & 63];
+    };
+    auto add4 = [&](int acc, const int4 &v, int rem) {
+        const int x = value(v.x), y = value(v.y), z = value(v.z), w = value(v.w);
+        acc += rem > 0 ? x : 0;
+        acc += rem > 1 ? y : 0;
+        acc += rem > 2 ? z : 0;
+        acc += rem > 3 ? w : 0;
+        return acc;
+    };
+
+    for (int base = j0; base < j1; base += SCAN_THREADS_F) {
+        const int cnt = j1 - base < SCAN_THREADS_F ? j1 - base : SCAN_THREADS_F;
+        // counting sort by chunk count, long documents first
+        const int2 r = nx_rng;
+        nx_rng = range_of(nx_cand);
+        nx_cand = cand_of(base + 2 * SCAN_THREADS_F);
+        uint32_t lo = mis + (uint32_t)r.x, hi = lo + (uint32_t)r.y;
+        int extra = 0;
+        for (; lo < edge_lo && lo < hi; ++lo) extra += value(cids[lo - mis]);
+        for (; hi > edge_hi && hi > lo; --hi) extra += value(cids[hi - 1 - mis]);
+        if (hi <= lo) lo = hi = 0;
+        int key = (int)((hi - (lo & ~3u) + 31) >> 5);
+        key = SCAN_SORT_BINS - 1 - (key < SCAN_SORT_BINS ? key : SCAN_SORT_BINS - 1);
+        int place = 0;
+        if (tid < cnt) place = atomicAdd(&s_sort[key], 1);
+        __syncthreads();
+        if (warp == 0) {
+            const int a = s_sort[2 * lane], c = s_sort[2 * lane + 1];
+            int incl = a + c;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int t = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += t;
+            }
+            s_sort[2 * lane] = incl - a - c;
+            s_sort[2 * lane + 1] = incl - c;
+        }
+        __syncthreads();
+        if (tid < cnt) {
+            place += s_sort[key];
+            s_rng[place] = make_uint2(lo, hi);
+            s_idx[place] = (uint16_t)tid;
+        }
+        __syncthreads();
+        if (tid < SCAN_SORT_BINS) s_sort[tid] = 0;
+
+        int k = warp * 4 + grp;
+        uint2 cur = k < cnt ? s_rng[k] : make_uint2(0, 0);
+        uint32_t q = (cur.x & ~3u) + 4 * sub;
+        int4 a0 = load4(q, cur.y), a1 = load4(q + 32, cur.y);
+        for (int kw = warp * 4; kw < cnt; kw += SCAN_THREADS_F / 8) {
+            const int kn = k + SCAN_THREADS_F / 8;
+            const uint2 nxt = kn < cnt ? s_rng[kn] : make_uint2(0, 0);
+            const uint32_t qn = (nxt.x & ~3u) + 4 * sub;
+            // steps of 64 tokens, as many as the longest of the four documents needs
+            const int most = __reduce_max_sync(0xffffffffu, (int)(cur.y - (q - 4 * sub)));
+            int acc = 0, rem = (int)(cur.y - q);
+            if (sub == 0) {                                  // ids of the document before, in front of the first token
+                const int lead = (int)(cur.x & 3u);
+                if (lead > 0) acc -= value(a0.x);
+                if (lead > 1) acc -= value(a0.y);
+                if (lead > 2) acc -= value(a0.z);
+            }
+            for (int c = 0; c < most; c += 64) {
+                int4 n0, n1;
+                const bool last = c + 64 >= most;
+                const uint32_t ql = last ? qn : q + 64, hl = last ? nxt.y : cur.y;
+                n0 = load4(ql, hl);
+                n1 = load4(ql + 32, hl);
+                acc = add4(acc, a0, rem);
+                if (c + 32 < most) acc = add4(acc, a1, rem - 32);
+                rem -= 64;
+                a0 = n0;
+                a1 = n1;
+                q = ql;
+            }
+            acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+            acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+            acc += __shfl_xor_sync(0xffffffffu, acc, 4);
+            if (sub == 0 && k < cnt) {
+                const int bin = acc >> (17 - us);
+                atomicAdd(&s_hist[bin < FILTER_BINS ? bin : FILTER_BINS - 1], 1);
+                out[base + s_idx[k]] = s_theta + acc;
+            }
+            k = kn;
+            cur = nxt;
+        }
+        __syncthreads();
+        if (extra > 0) out[base + tid] += extra;             // (the histogram keeps the smaller value: it only picks seeds)
+    }
+    int32_t *hb = hist + (int64_t)b * FILTER_BINS;
+    for (int i = tid; i < FILTER_BINS; i += SCAN_THREADS_F)
+        if (s_hist[i]) atomicAdd(&hb[i], s_hist[i]);
+}
+
+// ------------------------------------------------------------------------------------------------ seeds -----------
+// (first token, length) of a document.
+__device__ __forceinline__ int2 filter_range(const int64_t *doc_off, int32_t d)
+{
+    d = DBG_DOC(d);
+    const int64_t t0 = __ldg(doc_off + d);
+    return make_int2((int)t0, (int)(__ldg(doc_off + d + 1) - t0));
+}
+
+// A Q.24 threshold in units of 2^us, rounded up (hi0 is a whole number of them).
+__device__ __forceinline__ int32_t units_up(int32_t tau, int us) { return (int32_t)(((long long)tau + (1 << us) - 1) >> us); }
+
+// grid (split, B): candidates with the largest hi0, 1.5 n_prune of them and the rest of the
+// last histogram bin, with their token ranges, in no particular order; seed_thr[b] = the hi0 they
+// start at, seed_slot[candidate] = where each one went.  n_seed (cleared before) stays 0 when a query has so few
+// candidates that all are kept.
+__global__ void __launch_bounds__(SEL_THREADS)
+filter_seed_kernel(const int32_t *__restrict__ cand, const int32_t *__restrict__ n_cand, const int64_t *__restrict__ doc_off,
+                   const int32_t *__restrict__ hi0, int64_t maxc, const int32_t *__restrict__ theta, int nq, int us,
+                   const int32_t *__restrict__ hist, int n_prune, int32_t *__restrict__ seed,
+                   int2 *__restrict__ seed_rng, int32_t *__restrict__ n_seed, int32_t *__restrict__ seed_thr,
+                   int32_t *__restrict__ seed_slot)
+{
+    __shared__ int warp_part[32];
+    __shared__ int s_bin, s_theta;
+    const int b = blockIdx.y, n = n_cand[b];
+    const int want = n_prune + n_prune / 2 + 32;
+    if (n <= want) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) seed_thr[b] = INT_MAX;
+        return;
+    }
+    const int32_t *hb = hist + (int64_t)b * FILTER_BINS;
+    constexpr int PER = FILTER_BINS / SEL_THREADS;
+    const int first_bin = FILTER_BINS - 1 - PER * (int)threadIdx.x;
+    int h[PER], mine = 0;
+#pragma unroll
+    for (int e = 0; e < PER; ++e) { h[e] = hb[first_bin - e]; mine += h[e]; }
+    int total;
+    int before = sel_block_scan(mine, &total, warp_part);
+    if (before < want && want <= before + mine) {
+#pragma unroll
+        for (int e = 0; e < PER; ++e) {
+            if (before < want && want <= before + h[e]) s_bin = first_bin - e;
+            before += h[e];
+        }
+    }
+    if (threadIdx.x < 32) {
+        int s = 0;
+        for (int i = threadIdx.x; i < nq; i += 32) s += theta[(int64_t)b * nq + i];
+        s = __reduce_add_sync(0xffffffffu, s);
+        if (threadIdx.x == 0) s_theta = s;
+    }
+    __syncthreads();
+    const int32_t thr = (s_theta << (16 - us)) + (s_bin << (17 - us));
+    if (blockIdx.x == 0 && threadIdx.x == 0) seed_thr[b] = thr;
+    const int32_t *ub = hi0 + (int64_t)b * maxc;
+    const int32_t *cb = cand + (int64_t)b * maxc;
+    const int per = (n + (int)gridDim.x - 1) / (int)gridDim.x;
+    const int j0 = blockIdx.x * per, j1 = j0 + per < n ? j0 + per : n;
+    const int lane = threadIdx.x & 31;
+    for (int base = j0 + (threadIdx.x & ~31); base < j1; base += 8 * SEL_THREADS) {
+        int32_t v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int j = base + u * SEL_THREADS + lane;
+            v[u] = j < j1 ? ub[j] : INT_MIN;
+        }
+        unsigned mask[8];
+        int found = 0;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            mask[u] = __ballot_sync(0xffffffffu, v[u] >= thr);
+            found += __popc(mask[u]);
+        }
+        if (found == 0) continue;
+        int at = 0;
+        if (lane == 0) at = atomicAdd(&n_seed[b], found);    // one slot request per 256 candidates
+        at = __shfl_sync(0xffffffffu, at, 0);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            if (v[u] >= thr) {
+                const int32_t d = cb[base + u * SEL_THREADS + lane];
+                const int64_t o = (int64_t)b * maxc + at + __popc(mask[u] & ((1u << lane) - 1));
+                seed[o] = d;
+                seed_slot[(int64_t)b * maxc + base + u * SEL_THREADS + lane] = (int32_t)(o - (int64_t)b * maxc);
+                seed_rng[o] = filter_range(doc_off, d);
+            }
+            at += __popc(mask[u]);
+        }
+    }
+}
+
+// ------------------------------------------------------------------------------------------------ keep ------------
+// Ordered compaction of a slice [j0, j1) by a whole block: every element with v >= thr, in order.  A warp takes 256
+// consecutive elements per round (eight coalesced loads), one block scan per 8,192.  emit(j, v, position).
+template <class Emit>
+__device__ __forceinline__ int block_compact(const int32_t *__restrict__ v, int j0, int j1, int32_t thr, int run,
+                                             int *warp_part, Emit emit)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int base = j0; base < j1; base += 8 * SEL_THREADS) {
+        const int w0 = base + warp * 256 + lane;
+        int32_t x[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) x[u] = w0 + 32 * u < j1 ? v[w0 + 32 * u] : INT_MIN;
+        unsigned mask[8];
+        int found = 0;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            mask[u] = __ballot_sync(0xffffffffu, w0 + 32 * u < j1 && x[u] >= thr);
+            found += __popc(mask[u]);
+        }
+        int tot;
+        int pos = run + sel_block_scan(lane == 0 ? found : 0, &tot, warp_part);
+        pos = __shfl_sync(0xffffffffu, pos, 0);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            if (mask[u] >> lane & 1u) emit(w0 + 32 * u, x[u], pos + __popc(mask[u] & ((1u << lane) - 1)));
+            pos += __popc(mask[u]);
+        }
+        run += tot;
+    }
+    return run;
+}
+__device__ __forceinline__ void slice_of(int n, int *j0, int *j1)
+{
+    const int per = (n + (int)gridDim.x - 1) / (int)gridDim.x;
+    *j0 = blockIdx.x * per < n ? blockIdx.x * per : n;
+    *j1 = *j0 + per < n ? *j0 + per : n;
+}
+// Elements of the slices before this block's (counts[slice]; none when there is one slice).
+__device__ __forceinline__ int slices_before(const int32_t *counts)
+{
+    int run = 0;
+    for (int s = 0; s < (int)blockIdx.x; ++s) run += counts[s];
+    return run;
+}
+template <class T>
+__device__ __forceinline__ int block_count(const T *__restrict__ v, int j0, int j1, T thr, int *warp_part)
+{
+    int keep = 0;
+    for (int base = j0; base < j1; base += 8 * SEL_THREADS) {
+        T x[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int j = base + u * SEL_THREADS + threadIdx.x;
+            x[u] = j < j1 ? v[j] : thr - 1;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) keep += x[u] >= thr ? 1 : 0;
+    }
+    int total;
+    sel_block_scan(keep, &total, warp_part);
+    return total;
+}
+
+// grid (split, B).  tau = the n_prune-th largest exact CI of the seeds -> tau[b]; how many candidates of each slice have
+// hi0 >= tau -> counts[b][slice].  Fewer seeds than n_prune (then there are few candidates): everything is kept.
+__global__ void __launch_bounds__(SEL_THREADS)
+filter_count_kernel(const int32_t *__restrict__ n_cand, const int32_t *__restrict__ hi0, int64_t maxc,
+                    const int32_t *__restrict__ seed_ci, const int32_t *__restrict__ n_seed, int n_prune, int us,
+                    int32_t *__restrict__ tau_out, int32_t *__restrict__ counts)
+{
+    __shared__ int hist[2048];
+    __shared__ int warp_part[32];
+    __shared__ uint32_t s_prefix;
+    __shared__ int s_want;
+    const int b = blockIdx.y;
+    int32_t tau = INT_MIN + 1;
+    if (n_seed[b] >= n_prune) {
+        const int32_t *sb = seed_ci + (int64_t)b * maxc;
+        int need_eq;
+        const uint32_t u = radix_select([&](int j) { return sb[j]; }, n_seed[b], n_prune, hist, warp_part, &s_prefix,
+                                        &s_want, &need_eq);
+        tau = (int32_t)(u ^ 0x80000000u);
+    }
+    int j0, j1;
+    slice_of(n_cand[b], &j0, &j1);
+    const int total = block_count<int32_t>(hi0 + (int64_t)b * maxc, j0, j1, units_up(tau, us), warp_part);
+    if (threadIdx.x == 0) {
+        counts[(int64_t)b * KEEP_SPLIT + blockIdx.x] = total;
+        if (blockIdx.x == 0) tau_out[b] = tau;
+    }
+}
+
+// Same grid: the kept candidates, ascending, behind those of the slices before, with their token ranges.  A seed's exact CI
+// is known already: its range is (CI, 0), which the later kernels pass through.
+__global__ void __launch_bounds__(SEL_THREADS)
+filter_write_kernel(const int32_t *__restrict__ cand, const int32_t *__restrict__ n_cand,
+                    const int64_t *__restrict__ doc_off, const int32_t *__restrict__ hi0, int64_t maxc,
+                    const int32_t *__restrict__ seed_thr, const int32_t *__restrict__ seed_slot,
+                    const int32_t *__restrict__ seed_ci, const int32_t *__restrict__ tau, int us,
+                    const int32_t *__restrict__ counts, int32_t *__restrict__ kept, int2 *__restrict__ kept_rng,
+                    int32_t *__restrict__ n_kept)
+{
+    __shared__ int warp_part[32];
+    const int b = blockIdx.y;
+    const int64_t row = (int64_t)b * maxc;
+    const int32_t thr = seed_thr[b];
+    int j0, j1;
+    slice_of(n_cand[b], &j0, &j1);
+    const int run = block_compact(hi0 + row, j0, j1, units_up(tau[b], us), slices_before(counts + (int64_t)b * KEEP_SPLIT),
+                                  warp_part, [&](int j, int32_t v, int pos) {
+        const int32_t d = cand[row + j];
+        kept[row + pos] = d;
+        kept_rng[row + pos] = v >= thr ? make_int2(seed_ci[row + seed_slot[row + j]], 0) : filter_range(doc_off, d);
+    });
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) n_kept[b] = run;
+}
+
+// grid (split, B): contenders = kept candidates whose 8-bit upper bound reaches tau, with their ranges, ascending.  With
+// several slices the count kernel runs first.
+__global__ void __launch_bounds__(SEL_THREADS)
+filter_contend_count_kernel(const int32_t *__restrict__ n_kept, const int32_t *__restrict__ hi, int64_t maxc,
+                            const int32_t *__restrict__ tau, int32_t *__restrict__ counts)
+{
+    __shared__ int warp_part[32];
+    const int b = blockIdx.y;
+    int j0, j1;
+    slice_of(n_kept[b], &j0, &j1);
+    const int total = block_count<int32_t>(hi + (int64_t)b * maxc, j0, j1, tau[b], warp_part);
+    if (threadIdx.x == 0) counts[(int64_t)b * KEEP_SPLIT + blockIdx.x] = total;
+}
+__global__ void __launch_bounds__(SEL_THREADS)
+filter_contend_kernel(const int32_t *__restrict__ kept, const int2 *__restrict__ kept_rng, const int32_t *__restrict__ n_kept,
+                      const int32_t *__restrict__ hi, int64_t maxc, const int32_t *__restrict__ tau,
+                      const int32_t *__restrict__ counts, int32_t *__restrict__ cont, int2 *__restrict__ cont_rng,
+                      int32_t *__restrict__ n_cont)
+{
+    __shared__ int warp_part[32];
+    const int b = blockIdx.y;
+    const int64_t row = (int64_t)b * maxc;
+    int j0, j1;
+    slice_of(n_kept[b], &j0, &j1);
+    const int run = block_compact(hi + row, j0, j1, tau[b], slices_before(counts + (int64_t)b * KEEP_SPLIT), warp_part,
+                                  [&](int j, int32_t, int pos) {
+        cont[row + pos] = kept[row + j];
+        cont_rng[row + pos] = kept_rng[row + j];
+    });
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) n_cont[b] = run;
+}
+
+// ------------------------------------------------------------------------------------------------ launchers -------
+// Units of e and hi0: 2^us.  2^16 from the 8-bit table and for the 6-bit codes; the exact table gives finer ones, as fine as
+// 16 bits hold for q_len columns.
+static int filter_unit(const Index &ix, const Params &p, bool from_table8)
+{
+    return from_table8 || filter_codec(ix.K) != 16 ? 16 : p.nq <= 63 ? 14 : 15;
+}
+
+int launch_filter_scan(const Index &ix, const Params &p, const Layout &L, const int32_t *table, const uint8_t *table8,
+                       const int32_t *cand, const int32_t *n_cand, int32_t *hi0, int32_t *seed,
+                       int2 *seed_rng, char *ws, cudaStream_t st)
+{
+    int32_t *theta = (int32_t *)(ws + L.flt_theta), *hist = (int32_t *)(ws + L.flt_hist);
+    int32_t *n_seed = (int32_t *)(ws + L.n_seed);
+    uint8_t *tab = (uint8_t *)(ws + L.flt_tab);
+    const int codec = filter_codec(ix.K);
+    const size_t pitch = filter_table_pitch(ix);
+    const int step = (int)(ix.K / FILTER_SAMPLE > 1 ? ix.K / FILTER_SAMPLE : 1);
+    const int m = (int)((ix.K + step - 1) / step < 2 * FILTER_SAMPLE ? (ix.K + step - 1) / step : 2 * FILTER_SAMPLE);
+    // the length of the documents that compete for the top: about halfway between the candidates' mean (somewhat above
+    // the corpus's: long documents are probed more often) and the longest, outliers aside
+    const double mean = (double)ix.T / (double)ix.N, most = (double)ix.max_doclen;
+    const double len = 0.5 * ((1.2 * mean < most ? 1.2 * mean : most) + (2.4 * mean < most ? 2.4 * mean : most));
+    int rank = (int)(FILTER_LAMBDA / len * m + 0.5);
+    if (rank < 1) rank = 1;
+    const unsigned groups = (unsigned)((p.nq + 31) / 32);
+    const int parts = filter_parts(ix, p);
+    int32_t *parts_hist = (int32_t *)(ws + L.flt_parts), *done = parts_hist + (size_t)p.B * groups * 256 * 32;
+    if (parts > 1)
+        CHIMERA_CUDA(cudaMemsetAsync(parts_hist, 0, filter_parts_bytes(ix, p), st));
+    filter_theta_kernel<<<dim3(groups, (unsigned)p.B, (unsigned)parts), SEL_THREADS, 0, st>>>(
+        table, ix.K, p.nq, m, step, rank, theta, hist, n_seed, parts_hist, done);
+    CHIMERA_CUDA(cudaGetLastError());
+
+    const int us = filter_unit(ix, p, table8 != nullptr);
+    int64_t gx = (8LL * ix.sm_count + p.B - 1) / p.B;
+    if (table8 != nullptr) {
+        const int64_t want = ((codec == 16 ? ix.K : (ix.K + 4) / 5) + 255) / 256;
+        if (gx > want) gx = want;
+        const dim3 grid((unsigned)gx, (unsigned)p.B);
+        if (p.nq == 32 && codec == 16) filter_excess_kernel<8, 16><<<grid, 256, 0, st>>>(table8, ix.K, theta, tab, pitch);
+        else if (p.nq == 32) filter_excess_kernel<8, 6><<<grid, 256, 0, st>>>(table8, ix.K, theta, tab, pitch);
+        else if (codec == 16) filter_excess_kernel<16, 16><<<grid, 256, 0, st>>>(table8, ix.K, theta, tab, pitch);
+        else filter_excess_kernel<16, 6><<<grid, 256, 0, st>>>(table8, ix.K, theta, tab, pitch);
+    } else {
+        const int64_t want = (ix.K + 39) / 40;
+        if (gx > want) gx = want;
+        const dim3 grid((unsigned)gx, (unsigned)p.B);
+        if (codec == 16)
+            filter_excess_exact_kernel<16><<<grid, 256, 0, st>>>(table, ix.K, p.nq, theta, us, tab, pitch);
+        else
+            filter_excess_exact_kernel<6><<<grid, 256, 0, st>>>(table, ix.K, p.nq, theta, us, tab, pitch);
+    }
+    CHIMERA_CUDA(cudaGetLastError());
+
+    // Blocks per query: one block is resident per SM.  About eight waves over the batch even out the queries; few blocks
+    // per query keep many queries in step over the same documents, whose centroid ids then come from L2.
+    gx = (8LL * ix.sm_count + p.B - 1) / p.B;
+    if (gx > ix.sm_count) gx = ix.sm_count;
+    const int64_t want = (p.maxc + 511) / 512;
+    if (gx > want) gx = want;
+    const dim3 grid((unsigned)gx, (unsigned)p.B);
+    if (codec == 16) {
+        CHIMERA_CUDA(cudaFuncSetAttribute(filter_scan_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pitch));
+        filter_scan_kernel<16><<<grid, SCAN_THREADS_F, pitch, st>>>(tab, pitch, theta, p.nq, us, cand, ix.doc_off, n_cand, p.maxc,
+                                                                    ix.cids, ix.T, hi0, hist);
+    } else {
+        CHIMERA_CUDA(cudaFuncSetAttribute(filter_scan_kernel<6>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pitch));
+        filter_scan_kernel<6><<<grid, SCAN_THREADS_F, pitch, st>>>(tab, pitch, theta, p.nq, us, cand, ix.doc_off, n_cand, p.maxc,
+                                                                   ix.cids, ix.T, hi0, hist);
+    }
+    CHIMERA_CUDA(cudaGetLastError());
+    filter_seed_kernel<<<dim3((unsigned)filter_split(ix, p), (unsigned)p.B), SEL_THREADS, 0, st>>>(
+        cand, n_cand, ix.doc_off, hi0, p.maxc, theta, p.nq, us, hist, p.n_prune, seed, seed_rng, n_seed,
+        (int32_t *)(ws + L.flt_thr), (int32_t *)(ws + L.flt_slot));
+    CHIMERA_CUDA(cudaGetLastError());
+    count_launch(SLOT_CI, 4);
+    return CHIMERA_OK;
+}
+
+int launch_filter_keep(const Index &ix, const Params &p, const Layout &L, const int32_t *cand,
+                       const int32_t *n_cand, const int32_t *hi0, const int32_t *seed_ci, int32_t *kept,
+                       int2 *kept_rng, int32_t *n_kept, char *ws, cudaStream_t st)
+{
+    const int32_t *n_seed = (const int32_t *)(ws + L.n_seed);
+    int32_t *counts = (int32_t *)(ws + L.flt_counts);
+    const int us = filter_unit(ix, p, coarse_supported(p.nq));
+    int32_t *tau = (int32_t *)(ws + L.flt_tau);
+    const int32_t *thr = (const int32_t *)(ws + L.flt_thr), *slot = (const int32_t *)(ws + L.flt_slot);
+    const dim3 grid((unsigned)filter_split(ix, p), (unsigned)p.B);
+    filter_count_kernel<<<grid, SEL_THREADS, 0, st>>>(n_cand, hi0, p.maxc, seed_ci, n_seed, p.n_prune, us, tau, counts);
+    CHIMERA_CUDA(cudaGetLastError());
+    filter_write_kernel<<<grid, SEL_THREADS, 0, st>>>(cand, n_cand, ix.doc_off, hi0, p.maxc, thr, slot, seed_ci, tau, us,
+                                                      counts, kept, kept_rng, n_kept);
+    CHIMERA_CUDA(cudaGetLastError());
+    count_launch(SLOT_SELECT, 2);
+    return CHIMERA_OK;
+}
+
+int launch_filter_contenders(const Index &ix, const Params &p, const Layout &L, const int32_t *kept, const int2 *kept_rng,
+                             const int32_t *n_kept, const int32_t *hi, int32_t *cont, int2 *cont_rng, int32_t *n_cont,
+                             char *ws, cudaStream_t st)
+{
+    int32_t *counts = (int32_t *)(ws + L.flt_counts);
+    const int32_t *tau = (const int32_t *)(ws + L.flt_tau);
+    // one block per query keeps up in a large batch; a single query's list is spread
+    const int split = 4 * p.B <= ix.sm_count ? filter_split(ix, p) : 1;
+    const dim3 grid((unsigned)split, (unsigned)p.B);
+    if (split > 1) {
+        filter_contend_count_kernel<<<grid, SEL_THREADS, 0, st>>>(n_kept, hi, p.maxc, tau, counts);
+        CHIMERA_CUDA(cudaGetLastError());
+        count_launch(SLOT_SELECT);
+    }
+    filter_contend_kernel<<<grid, SEL_THREADS, 0, st>>>(kept, kept_rng, n_kept, hi, p.maxc, tau, counts, cont, cont_rng,
+                                                        n_cont);
+    CHIMERA_CUDA(cudaGetLastError());
+    count_launch(SLOT_SELECT);
+    return CHIMERA_OK;
+}
+
+}  // namespace chimera
