@@ -109,6 +109,8 @@ Layout make_layout(const Index &ix, const Params &p)
     L.out_ids = take(B * p.k * sizeof(int32_t));
     L.out_scores = take(B * p.k * sizeof(float));
     L.qdig = take(3 * B * nq * 128);
+    const size_t rows4 = residual_umma_supported(p.nq) ? B * (size_t)residual_rows(p.nq) : 0;
+    L.qdig4 = take(3 * rows4 * 128);
     L.table = take(B * (size_t)ix.K * nq * sizeof(int32_t));
     L.table8 = take(coarse_supported(p.nq) ? B * (size_t)ix.K * nq : 0);
     L.pq_stride = probe_queue_stride(ix, p);
@@ -160,7 +162,7 @@ Layout make_layout(const Index &ix, const Params &p)
     }
     L.graph_vis = take(ix.graph ? graph_scratch_bytes(ix, (int64_t)p.B * p.nq) : 0);
     L.q_rot = take(ix.rot_t ? B * nq * ix.D * sizeof(float) : 0);
-    L.qdig_rot = take(ix.rot_t ? 3 * B * nq * 128 : 0);
+    L.qdig_rot = take(ix.rot_t ? 3 * rows4 * 128 : 0);
     L.n_pruned = take(B * sizeof(int32_t));
     L.pruned_ci = take(B * p.n_prune * sizeof(int32_t));
     L.sel_scratch = take(select_split_scratch_bytes(ix, p));
@@ -257,6 +259,7 @@ static int run(const Index &ix, const Params &p, int first, int last, const floa
     char *ws = (char *)workspace;
     uint32_t *status = (uint32_t *)(ws + L.status);
     int8_t *qdig = (int8_t *)(ws + L.qdig);
+    int8_t *qdig4 = residual_umma_supported(p.nq) ? (int8_t *)(ws + L.qdig4) : nullptr;
     int32_t *table = (int32_t *)(ws + L.table);
     unsigned long long *part = (unsigned long long *)(ws + L.part);
     int32_t *probes = (int32_t *)(ws + L.probes);
@@ -328,9 +331,9 @@ static int run(const Index &ix, const Params &p, int first, int last, const floa
     const bool together = first <= 1 && last >= 2 && !graph && L.pq_stride > 0;
     if (first <= 1 && last >= 1 && !graph) {
         if (together)
-            rc = launch_score_table_probes(ix, p, L, queries, qdig, table, table8, ws, status, st);
+            rc = launch_score_table_probes(ix, p, L, queries, qdig, qdig4, table, table8, ws, status, st);
         else
-            rc = launch_score_table(ix, p, queries, qdig, table, table8, status, st);
+            rc = launch_score_table(ix, p, queries, qdig, qdig4, table, table8, status, st);
         if (rc) return rc;
         prof_mark(SLOT_G1, st);
     }
@@ -352,7 +355,7 @@ static int run(const Index &ix, const Params &p, int first, int last, const floa
         if (rabitq) {
             // the paper's pipeline on its own codec: rotate the queries, refine by partial 1-bit scores
             if ((rc = launch_rotate(ix, p, queries, q_rot, st))) return rc;
-            if ((rc = launch_digits(q_rot, (int64_t)p.B * p.nq, ix.D, qdig_rot, status, st))) return rc;
+            if ((rc = launch_digits(q_rot, (int64_t)p.B * p.nq, ix.D, 1, nullptr, qdig_rot, p.nq, status, st))) return rc;
             count_launch(SLOT_G1);
             prof_mark(SLOT_G1, st);
             if ((rc = launch_rabitq_partial(ix, p, L, q_rot, probes, bitmap, word_rank, n_cand, partial_m, ci, st)))
@@ -424,10 +427,10 @@ static int run(const Index &ix, const Params &p, int first, int last, const floa
             if ((rc = launch_rabitq_scores_umma(ix, p, q_rot, qdig_rot, pruned, score4, status, st))) return rc;
         } else if (residual_umma_supported(p.nq)) {
             if (first > 1) {                       // stage 1 did not run in this call: build the query digit planes
-                if ((rc = launch_digits(queries, (int64_t)p.B * p.nq, ix.D, qdig, status, st))) return rc;
+                if ((rc = launch_digits(queries, (int64_t)p.B * p.nq, ix.D, ix.nbits, nullptr, qdig4, p.nq, status, st))) return rc;
                 count_launch(SLOT_G4);
             }
-            if ((rc = launch_residual_scores_umma(ix, p, queries, qdig, table, pruned, score4, status, st))) return rc;
+            if ((rc = launch_residual_scores_umma(ix, p, queries, qdig4, table, pruned, score4, status, st))) return rc;
         } else if ((rc = launch_residual_scores(ix, p, queries, table, pruned, score4, st))) {
             return rc;
         }

@@ -20,7 +20,7 @@ struct Index {
     const int32_t *cids = nullptr;    // [T]        borrowed
     const uint8_t *codes = nullptr;   // [T, CB]    borrowed
     int64_t *doc_off = nullptr;       // [N+1]      owned: first token of each document
-    int8_t *cdig = nullptr;           // [3][K][128] owned: balanced base-256 digits of rint(c * 2^22), zero padded
+    int8_t *cdig = nullptr;           // [3][K][128] owned: balanced base-256 digits of rint(c * 2^22), zero padded, digit_dim() order
     int64_t *ivf_off = nullptr;       // [K+1]      owned
     int32_t *ivf_doc = nullptr;       // [ivf_len]  owned: unique document ids per centroid, unordered
     int64_t ivf_len = 0;
@@ -67,6 +67,7 @@ struct Layout {
     size_t out_ids;       // int32  [B, k]            (host-entry staging)
     size_t out_scores;    // float  [B, k]
     size_t qdig;          // int8   [3][B*nq][128]
+    size_t qdig4;         // int8   [3][B*residual_rows(nq)][128]  the same for stage 4 (q_len <= 64)
     size_t table;         // int32  [B][K][nq]
     size_t table8;        // uint8  [B][K][nq]        coarse copy: min((S + 2^24 + 64) >> 17, 255)
     size_t part;          // uint64 [B][n_part][P][nq] partial top-P keys
@@ -106,7 +107,7 @@ struct Layout {
     int64_t hash_slots;   // slots per query of that table; 0 = the dense form
     size_t graph_vis;     // uint32 [B*nq][K/32]      visited centroids of the graph search (only with a centroid graph)
     size_t q_rot;         // float  [B, nq, D]        rotated queries (RaBitQ pipeline)
-    size_t qdig_rot;      // int8   [3][B*nq][128]    their digit planes
+    size_t qdig_rot;      // int8   [3][B*residual_rows(nq)][128]  their digit planes for stage 4
     size_t n_pruned;      // int32  [B]
     size_t pruned_ci;     // int32  [B][n_prune] stage-3 score of each survivor (document-sharded search)
     size_t sel_scratch;   // int32  histograms and slice counts of the multi-block selection (few queries per call)
@@ -152,12 +153,15 @@ void count_launch(int slot, int n = 1);
 // Stage launchers (one per .cu file).  Each only enqueues kernels on `st` and returns a chimera_status.
 // ---------------------------------------------------------------------------------------------------------------
 int build_index_device(Index &ix, const float *centroids, const int32_t *doclens, cudaStream_t st);
-// rows x D float32 in [-1, 1] -> three int8 digit planes [3][rows][128] (zero padded); out-of-range elements set
-// ST_BAD_QUERY.
-int launch_digits(const float *x, int64_t rows, int D, int8_t *dig, uint32_t *status, cudaStream_t st);
+// rows x D float32 in [-1, 1] -> three int8 digit planes [3][rows][128] (zero padded, dimensions in digit_dim() order);
+// out-of-range elements set ST_BAD_QUERY.
+// dig4 (may be NULL): the same planes for stage 4, rows = query tokens (q_len of them per query) in score_row() order,
+// padded to residual_rows(q_len) per query; the padding is not written.  dig may be NULL then.
+int launch_digits(const float *x, int64_t rows, int D, int nbits, int8_t *dig, int8_t *dig4, int q_len, uint32_t *status,
+                  cudaStream_t st);
 
 // table8 may be NULL (no coarse copy wanted).
-int launch_score_table(const Index &ix, const Params &p, const float *queries, int8_t *qdig, int32_t *table,
+int launch_score_table(const Index &ix, const Params &p, const float *queries, int8_t *qdig, int8_t *qdig4, int32_t *table,
                        uint8_t *table8, uint32_t *status, cudaStream_t st);
 int launch_probes(const Index &ix, const Params &p, const Layout &L, const int32_t *table, unsigned long long *part,
                   int32_t *probes, cudaStream_t st);
@@ -169,6 +173,7 @@ int probe_queue_stride(const Index &ix, const Params &p);
 int probe_queue_cap();
 int probe_sample_groups(const Index &ix, int stride);
 int launch_score_table_probes(const Index &ix, const Params &p, const Layout &L, const float *queries, int8_t *qdig,
+                              int8_t *qdig4,
                               int32_t *table, uint8_t *table8, char *ws, uint32_t *status, cudaStream_t st);
 int launch_probe_sample(const Index &ix, const Params &p, const Layout &L, const int32_t *table, char *ws,
                         int n_sample_tiles, cudaStream_t st);
@@ -240,7 +245,7 @@ int launch_shard_merge_topk(const int32_t *all_ids, const float *all_scores, int
                             float *out_scores, cudaStream_t st);
 int launch_residual_scores(const Index &ix, const Params &p, const float *queries, const int32_t *table,
                            const int32_t *pruned, float *score4, cudaStream_t st);
-// Tensor-core variant of stage 4 for q_len <= 64; qdig = the query digit planes of stage 1.
+// Tensor-core variant of stage 4 for q_len <= 64; qdig4 = the query digit planes in its own row order.
 bool residual_umma_supported(int nq);
 int launch_residual_scores_umma(const Index &ix, const Params &p, const float *queries, const int8_t *qdig,
                                 const int32_t *table, const int32_t *pruned, float *score4, uint32_t *status,
@@ -294,6 +299,21 @@ template <class I> __device__ __forceinline__ I dbg_index(I x, long long n) { re
 #endif
 // Host side (api.cu): publish the running search's limits / fill and check the guard regions (no-ops in release builds).
 int debug_begin_search(const Index &ix, const Params &p, const Layout &L, void *workspace, cudaStream_t st);
+
+// Order of the dimensions in a digit row: position -> dimension.  A contraction does not care as long as both operands
+// agree, so the order is the one in which packed codes expand with one shift and one mask per four dimensions (stage 4):
+// (word >> 2 j) & 0x03030303 holds dimensions j, 4 + j, 8 + j, 12 + j of the word's 16 2-bit codes, and
+// (word >> j) & 0x01010101 dimensions j, 8 + j, 16 + j, 24 + j of its 32 1-bit codes.
+__host__ __device__ __forceinline__ int digit_dim(int pos, int nbits)
+{
+    return nbits == 2 ? (pos & ~15) | (pos & 3) << 2 | (pos >> 2 & 3) : (pos & ~31) | (pos & 3) << 3 | (pos >> 2 & 7);
+}
+
+// Stage 4 on the tensor cores: rows per query of its digit planes, and the row of query token i.  Within 16 tokens, tokens
+// 4 g ... 4 g + 3 sit in rows 2 g, 2 g + 1, 8 + 2 g, 8 + 2 g + 1: the accumulator columns that the same thread reads back,
+// so that its four score-table entries are one 16-byte load.
+__host__ __device__ __forceinline__ int residual_rows(int q_len) { return q_len <= 32 ? 32 : 64; }
+__host__ __device__ __forceinline__ int score_row(int i) { return (i & ~15) | (i & 2) << 2 | (i >> 1 & 6) | (i & 1); }
 
 // ---------------------------------------------------------------------------------------------------------------
 // Device helpers.

@@ -157,7 +157,7 @@ score_table_umma(const int8_t *__restrict__ cdig, const __grid_constant__ CUtens
 #pragma unroll
                 for (int x = 0; x < 32; ++x) r[x] = 0u;
             }
-            tmem_st32(lane_addr + p * 32, r);
+            tmem_st(lane_addr + p * 32, r);
         }
         asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
     }
@@ -425,11 +425,11 @@ static int launch_g1_tiles(const Index &ix, const Params &p, const CUtensorMap &
     return CHIMERA_OK;
 }
 
-int launch_score_table(const Index &ix, const Params &p, const float *queries, int8_t *qdig, int32_t *table,
+int launch_score_table(const Index &ix, const Params &p, const float *queries, int8_t *qdig, int8_t *qdig4, int32_t *table,
                        uint8_t *table8, uint32_t *status, cudaStream_t st)
 {
     const int64_t rows = (int64_t)p.B * p.nq;
-    int rc = launch_digits(queries, rows, ix.D, qdig, status, st);
+    int rc = launch_digits(queries, rows, ix.D, ix.nbits, qdig, qdig4, p.nq, status, st);
     if (rc) return rc;
     CUtensorMap map_q;
     if ((rc = make_plane_map(&map_q, qdig, rows, G1_N, 3))) return rc;        // one load brings a tile's three planes
@@ -446,11 +446,11 @@ int launch_score_table(const Index &ix, const Params &p, const float *queries, i
 // by a scan of their rows), and the nprobe best keys of each queue.  The result is the exact top nprobe by (score
 // descending, centroid id ascending): a centroid that belongs to it has a score >= the bound, so it is queued.
 // A query with a token whose queue overflowed is redone by the table scan of the separate probe stage.
-int launch_score_table_probes(const Index &ix, const Params &p, const Layout &L, const float *queries, int8_t *qdig,
+int launch_score_table_probes(const Index &ix, const Params &p, const Layout &L, const float *queries, int8_t *qdig, int8_t *qdig4,
                               int32_t *table, uint8_t *table8, char *ws, uint32_t *status, cudaStream_t st)
 {
     const int64_t rows = (int64_t)p.B * p.nq;
-    int rc = launch_digits(queries, rows, ix.D, qdig, status, st);
+    int rc = launch_digits(queries, rows, ix.D, ix.nbits, qdig, qdig4, p.nq, status, st);
     if (rc) return rc;
     CUtensorMap map_q;
     if ((rc = make_plane_map(&map_q, qdig, rows, G1_N, 3))) return rc;

@@ -8,15 +8,19 @@
 // int32; the three planes are recombined in fp32 (relative error 2^-24).
 //
 // A CTA owns one query and a run of its surviving documents, whose tokens form one stream cut into tiles of 128
-// (MMA M).  Per tile: every thread expands the packed code of one token into 128 int8 values (two integer
-// multiplications and two masks per four dimensions) and writes them with one tcgen05.st into its lane of the A
-// operand IN TENSOR MEMORY (32 columns behind the accumulators; through shared memory the same row cost eight
-// 16-byte stores per thread, and the load/store pipe is what this kernel is short of); one thread issues D/32 MMAs
-// (N = 3 * padded q_len: the three digit planes side by side, loaded once per CTA by TMA); the accumulators come back
-// with tcgen05.ld, get the centroid term from the stage-1 table, and go to shared memory, where each warp folds its
-// 32 tokens into per-document maxima (a warp whose tokens are all of one document reads 16 bytes per lane and row
-// quarter instead of a word per row).  Tensor memory: 128 or 256 columns per CTA, so several CTAs share an SM and
-// overlap each other's phases.  All mbarrier waits are bounded.
+// (MMA M).  The kernel is bound by the instructions and latencies around the MMAs (tensor pipe 12 %), so:
+//   - codes expand with one shift and one mask per four dimensions (the query's digits are stored in the order in which
+//     codes expand, digit_dim()) and go into tensor memory as the A operand with one tcgen05.st per thread;
+//   - each warp takes 16 query tokens of a quarter's 32 token rows (two warps per quarter for q_len <= 32, four above) and
+//     reads the accumulators back in the 16x256b shape, i.e. already spread over (row, four query tokens): the maxima are
+//     folded in registers, without a transposition through shared memory, and the score-table entries of the centroid
+//     term come as one 16-byte load per row, four lanes to a row (a thread per row would touch 32 lines with each load);
+//   - the accumulators of tile t are read back before the tile's only block barrier, and behind it tile t + 1's MMAs, code
+//     and row loads run while tile t is folded.
+// Measured (batch 256, Mid, n_prune 1024): 2.24 -> 1.56 ms against one warp per quarter, value rows in shared memory and
+// two barriers per tile; 64 long-document queries of 64 tokens: 5.9 -> 3.75 ms.  Residency: q_len <= 32 three CTAs of 256
+// threads (85 registers, no spills; four with 64 registers: 1.78 ms; the RaBitQ variant, which holds no score-table
+// entries, four: 1.18 against 1.32 ms), q_len <= 64 two of 512 threads.  All mbarrier waits are bounded.
 #include <math.h>
 
 #include "common.cuh"
@@ -24,7 +28,7 @@
 
 namespace chimera {
 
-constexpr int G4U_THREADS = 128;
+constexpr int G4U_COLS = 16;              // query tokens per draining warp
 constexpr int G4U_TOK = 128;             // tokens per tile (MMA M)
 constexpr int G4U_MAX_DOCS = 32;         // documents per CTA, at most
 
@@ -38,46 +42,28 @@ __device__ __forceinline__ float f_unorder(uint32_t o)
     return __uint_as_float((o & 0x80000000u) ? (o & 0x7fffffffu) : ~o);
 }
 
-// One code byte (four 2-bit bucket indices, dimension 4g+t in bits [2t, 2t+1]) -> four int8 values, one per byte.
-// Both multiplications only place copies at disjoint bit positions, so they are shifts-and-ors without carries.
-__device__ __forceinline__ uint32_t spread2(uint32_t byte)
-{
-    const uint32_t x = (byte * 0x1001u) & 0x000F000Fu;       // low nibble at bit 0, high nibble at bit 16
-    return (x * 0x41u) & 0x03030303u;                        // second index of each nibble moved up one byte
-}
-// Four 1-bit codes (a nibble, dimension t in bit t) -> four int8 values 0/1: bit t lands at bit 8t of the product
-// (the other copies fall on bits that the mask drops; all partial products occupy distinct bits).
-__device__ __forceinline__ uint32_t spread1(uint32_t nibble) { return (nibble * 0x00204081u) & 0x01010101u; }
-
 // RQ = true scores RaBitQ 1-bit codes instead (Sec. 2.2; the GPU half of the paper's document scoring): the same
 // contraction T = sum_x Xq[x] b[x] against the digit planes of the ROTATED query, then
 // est = inv_dot_t * (c * (float)(2 T - SQ_i)) with SQ_i = sum_x Xq_i[x] and c = 1 / (sqrt(D) 2^22); no centroid term;
 // query tokens are summed in increasing order in fp32 so that the score is reproducible bit for bit.
-template <int NQP, int NBITS, bool RQ>
-__global__ void __launch_bounds__(G4U_THREADS)
+// FULL: q_len is NQP and dim is 128, the common sizes: no row or code is partial and every address is aligned.
+template <int NQP, int NBITS, bool RQ, bool FULL>
+__global__ void __launch_bounds__(128 * (NQP / G4U_COLS), NQP == 32 ? (RQ ? 4 : 3) : 2)
 residual_maxsim_umma(const __grid_constant__ CUtensorMap map_q, const float *__restrict__ queries,
-                     const int32_t *__restrict__ table, int64_t K, int nq, int D, int CW, float delta, float kappa,
+                     const int32_t *__restrict__ table, int64_t K, int nq_arg, int D_arg, int CW_arg, float delta, float kappa,
                      const int32_t *__restrict__ pruned, int n_prune, int docs_per_cta,
                      const int32_t *__restrict__ cids, const uint32_t *__restrict__ codes,
                      const float *__restrict__ factors, const int64_t *__restrict__ doc_off,
                      float *__restrict__ score4, uint32_t *status, long long wait_limit, int skip_loads)
 {
+    const int nq = FULL ? NQP : nq_arg, D = FULL ? 128 : D_arg, CW = FULL ? (NBITS == 2 ? 8 : 4) : CW_arg;
     constexpr int N = 3 * NQP;                               // MMA N: three digit planes side by side
     constexpr uint32_t TMEM_COLS = N <= 96 ? 128 : 256;
     constexpr uint32_t A_COL = N;                            // the expanded codes: 32 columns behind the accumulators
     static_assert(N + 32 <= TMEM_COLS, "accumulators and the A operand share the allocation");
     constexpr uint32_t B_BYTES = N * 128;
-    // Value rows (one per token, floats) in shared memory.  PACKED (q_len <= 32, residual codes): a row is exactly 128
-    // bytes and its 16-byte groups are XOR-swizzled with the row number, so the row-per-thread writes and the
-    // lane = column reads are both conflict-free without padding: 16 KB, which with the query planes and the
-    // per-document maxima keeps the CTA at 32 KB and lets the SM run with a small shared-memory carve-out, i.e. more L1
-    // for the scattered score-table rows (Mid, batch 256: 2.72 -> 2.41 ms against padded rows; forcing the largest
-    // carve-out brings 2.71 ms back).  The RaBitQ variant gathers no rows and is faster with padded rows (pitch
-    // NQP + 4, read with lane = column: conflict-free), as are 64-token queries.
-    constexpr bool ON_A = NQP == 32 && !RQ;
-    constexpr int VP = ON_A ? 32 : NQP + 4;
-    constexpr uint32_t V_BYTES = sizeof(float) * G4U_TOK * VP;       // a multiple of 1024 for every variant
-    static_assert(V_BYTES % 1024 == 0, "the query planes behind the value rows stay 1024-byte aligned");
+    constexpr int WPQ = NQP / G4U_COLS;                      // warps per lane quarter: each drains 16 query tokens
+    constexpr int G4U_THREADS = 128 * WPQ;
     constexpr uint32_t IDESC = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) |
                                ((uint32_t)(G4U_TOK >> 4) << 24);
 
@@ -90,13 +76,14 @@ residual_maxsim_umma(const __grid_constant__ CUtensorMap map_q, const float *__r
     __shared__ int s_sq[NQP];                                // RQ: sum_x rint(q_p[x] * 2^22) per query token
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t *gen = smem_raw + (base - smem_u32(smem_raw));   // generic pointer to the aligned area
-    float *vals = reinterpret_cast<float *>(gen);                                            // [128][VP]
-    const uint32_t sB = base + V_BYTES;                                                      // [3][NQP][128] int8
-    uint32_t *docmax = reinterpret_cast<uint32_t *>(gen + V_BYTES + B_BYTES);                // [MAX_DOCS][NQP]
+    const uint32_t sB = base;                                                      // [3][NQP][128] int8
+    uint32_t *docmax = reinterpret_cast<uint32_t *>(gen + B_BYTES);                // [MAX_DOCS][NQP]
     const uint32_t bars = smem_u32(docmax + G4U_MAX_DOCS * NQP);
     const uint32_t bar_b = (bars + 7u) & ~7u, bar_mma = bar_b + 8;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int quarter = warp & 3, part = warp >> 2;          // lanes of tensor memory, columns / code words of this warp
+    const int row = tid & 127;                               // this thread's token of a tile (shared by the WPQ parts)
     const int b = blockIdx.y;
     const int j0 = blockIdx.x * docs_per_cta;
     int nd = n_prune - j0;
@@ -142,9 +129,9 @@ residual_maxsim_umma(const __grid_constant__ CUtensorMap map_q, const float *__r
         float sum = 0.f;
         int si = 0;
         if (i < nq) {
-            const int quarter = D >> 2;               // D is a multiple of 32
-            const float4 *src = reinterpret_cast<const float4 *>(queries + ((int64_t)b * nq + i) * D + (tid & 3) * quarter);
-            for (int x = 0; x < (quarter >> 2); ++x) {
+            const int fourth = D >> 2;                // D is a multiple of 32
+            const float4 *src = reinterpret_cast<const float4 *>(queries + ((int64_t)b * nq + i) * D + (tid & 3) * fourth);
+            for (int x = 0; x < (fourth >> 2); ++x) {
                 const float4 v = __ldg(src + x);
                 sum += (v.x + v.y) + (v.z + v.w);
                 si += __float2int_rn(fminf(fmaxf(v.x, -1.0f), 1.0f) * 4194304.0f) +
@@ -169,251 +156,218 @@ residual_maxsim_umma(const __grid_constant__ CUtensorMap map_q, const float *__r
     // skip_loads (test hook): no load is issued, so the first wait below runs into its limit with nothing in flight
     if (tid == 0 && !skip_loads) {   // the query's three digit planes, side by side: rows [p * NQP, (p + 1) * NQP)
         mbar_expect_tx(bar_b, B_BYTES);
-        for (int p = 0; p < 3; ++p) tma_load_3d(sB + p * NQP * 128, &map_q, 0, b * nq, p, bar_b);
+        for (int p = 0; p < 3; ++p) tma_load_3d(sB + p * NQP * 128, &map_q, 0, b * NQP, p, bar_b);
     }
 
-    const int32_t *tb = table + (int64_t)b * K * nq;
-    const bool vec_rows = (nq & 3) == 0;
-    const bool wide_rows = (nq & 7) == 0;          // rows are then 32-byte aligned (the table is 256-byte aligned)
-    const int k_steps = D >> 5;
-    const float code_scale = delta * (1.0f / 4194304.0f);    // delta * 2^-22
+    const char *tb = reinterpret_cast<const char *>(table + (int64_t)b * K * nq);
+    const uint32_t row_bytes = 4u * (uint32_t)nq;
+    const bool vec_rows = (nq & 3) == 0;           // 16-byte groups of a row are aligned
+    const int k_steps = FULL ? 4 : D >> 5;
+    const float code_scale = delta * 4.0f;                    // delta * 2^-22, times 2^24
     bool alive = true;
-    constexpr int MAXCW = 8;                                  // 32 code bytes per token at most
+    // Code words of a token that one thread expands: a token has at most 32 code bytes (2 bits per dimension) or 16 (1 bit).
+    constexpr int TW = (NBITS == 2 ? 8 : 4) / WPQ;
+    constexpr int ACOLS = 32 / WPQ;                           // columns of the A operand they fill
+    const int w0 = part * TW;
 
-    // Token of stream position s (this thread's row of a tile): local document, centroid id, packed code words.
-    int dl_hint = 0;
-    auto fetch = [&](int tile, int &dl, int32_t &cid, uint32_t (&cw)[MAXCW]) {
-        const int s = tile * G4U_TOK + tid;
-        dl = -1;
+    // Token of stream position s (this thread's row of a tile): centroid id (-1 past the stream's end) and its part of the
+    // packed code.  Positions only move forward, so the document is found by stepping on.
+    int at_doc = -1, at_end = 0;
+    const uint32_t *at_code = nullptr;                        // of position 0, were it in the same document
+    const int32_t *at_cid = nullptr;                          // (RQ: the token's factor, whose bits > 0 take the id's place)
+    auto fetch = [&](int tile, int32_t &cid, uint32_t (&cw)[TW]) {
+        const int s = tile * G4U_TOK + row;
         cid = -1;
-        if (s < total) {
-            while (dl_hint + 1 < nd && s_off[dl_hint + 1] <= s) ++dl_hint;    // positions only move forward
-            dl = dl_hint;
-            const long long t = DBG_TOK(s_t0[dl] + (s - s_off[dl]));
-            cid = RQ ? __float_as_int(factors[t]) : cids[t];     // RQ: the slot carries the token's factor bits (> 0)
-            const uint32_t *src = codes + t * CW;
-            if (NBITS == 2 && CW == 8) {                  // 32-byte codes (32-byte aligned): one load
-                asm volatile("ld.global.nc.v8.u32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                             : "=r"(cw[0]), "=r"(cw[1]), "=r"(cw[2]), "=r"(cw[3]), "=r"(cw[4]), "=r"(cw[5]), "=r"(cw[6]),
-                               "=r"(cw[7])
-                             : "l"(src));
-            } else if ((CW & 3) == 0) {                   // 16-byte aligned codes
+        if (s >= total) return;
+        if (s >= at_end) {
+            do ++at_doc; while (s_off[at_doc + 1] <= s);
+            at_end = s_off[at_doc + 1];
+            const long long t = s_t0[at_doc] - s_off[at_doc];
+            at_code = codes + t * CW + w0;
+            at_cid = (RQ ? reinterpret_cast<const int32_t *>(factors) : cids) + t;
+        }
+#ifdef CHIMERA_DEBUG
+        const long long dbg_t = s_t0[at_doc] + s - s_off[at_doc];
+        if (DBG_TOK(dbg_t) != dbg_t) return;                  // (reported; the row keeps no token)
+#endif
+        cid = __ldg(at_cid + s);
+        const uint32_t *src = at_code + (long long)s * CW;
+        if (FULL ? TW == 4 : TW == 4 && (CW & 3) == 0) {
+            const uint4 v = __ldg(reinterpret_cast<const uint4 *>(src));
+            cw[0] = v.x; cw[1] = v.y; cw[TW > 2 ? 2 : 0] = v.z; cw[TW > 3 ? 3 : 0] = v.w;
+        } else if (FULL ? TW >= 2 : TW >= 2 && (CW & 1) == 0) {
 #pragma unroll
-                for (int w = 0; w < MAXCW; w += 4)
-                    if (w < CW) {
-                        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(src + w));
-                        cw[w] = v.x; cw[w + 1] = v.y; cw[w + 2] = v.z; cw[w + 3] = v.w;
-                    }
-            } else if ((CW & 1) == 0) {
+            for (int w = 0; w < TW; w += 2)
+                if (FULL || w0 + w < CW) {
+                    const uint2 v = __ldg(reinterpret_cast<const uint2 *>(src + w));
+                    cw[w] = v.x; cw[w + 1 < TW ? w + 1 : w] = v.y;
+                }
+        } else {
 #pragma unroll
-                for (int w = 0; w < MAXCW; w += 2)
-                    if (w < CW) {
-                        const uint2 v = __ldg(reinterpret_cast<const uint2 *>(src + w));
-                        cw[w] = v.x; cw[w + 1] = v.y;
-                    }
-            } else {
-#pragma unroll
-                for (int w = 0; w < MAXCW; ++w)
-                    if (w < CW) cw[w] = __ldg(src + w);
-            }
+            for (int w = 0; w < TW; ++w)
+                if (FULL || w0 + w < CW) cw[w] = __ldg(src + w);
         }
     };
 
-    int dl, dl_next = -1;
-    int32_t cid, cid_next = -1;
-    uint32_t cw[MAXCW], cw_next[MAXCW];
-    if (n_tiles > 0) fetch(0, dl_next, cid_next, cw_next);
-
-    for (int tile = 0; tile < n_tiles; ++tile) {
-        dl = dl_next;
-        cid = cid_next;
+    // Expands this thread's part of a token into lane `row` of the A operand in tensor memory.  A row without a token keeps
+    // whatever cw holds (its products take part in no maximum); columns past the code are not multiplied.
+    auto expand = [&](const uint32_t (&cw)[TW]) {
+        uint32_t a[ACOLS];
 #pragma unroll
-        for (int w = 0; w < MAXCW; ++w) cw[w] = cw_next[w];
-
-        // ---- expand this thread's token into lane `tid` of the A operand in tensor memory (128 int8 = 32 columns) ----
-        {
-            uint32_t row[32];
+        for (int w = 0; w < TW; ++w) {
+            const uint32_t word = cw[w];
+            if (NBITS == 2) {
 #pragma unroll
-            for (int x = 0; x < 32; ++x) row[x] = 0u;
-            if (dl >= 0) {
+                for (int h = 0; h < 4; ++h) a[4 * w + h] = (word >> (2 * h)) & 0x03030303u;
+            } else {
 #pragma unroll
-                for (int w = 0; w < MAXCW; ++w) {
-                    if (w < CW) {
-                        const uint32_t word = cw[w];
-                        if (NBITS == 2) {
-                            row[4 * w + 0] = spread2(word & 255u);
-                            row[4 * w + 1] = spread2((word >> 8) & 255u);
-                            row[4 * w + 2] = spread2((word >> 16) & 255u);
-                            row[4 * w + 3] = spread2(word >> 24);
-                        } else if (w < 4) {                  // 1 bit per dimension: at most four words
-#pragma unroll
-                            for (int h = 0; h < 8; ++h) row[8 * w + h] = spread1((word >> (4 * h)) & 15u);
-                        }
-                    }
-                }
+                for (int h = 0; h < 8; ++h) a[8 * w + h] = (word >> h) & 0x01010101u;
             }
-            tmem_st32(tmem + ((uint32_t)(warp * 32) << 16) + A_COL, row);
-            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
         }
+        tmem_st(tmem + ((uint32_t)(quarter * 32) << 16) + A_COL + part * ACOLS, a);
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+    };
+    auto issue = [&]() {                                      // one thread
+        tc_fence_after();
+        const uint64_t db = umma_desc(sB);
+        for (int k = 0; k < k_steps; ++k) umma_i8_ts(tmem, tmem + A_COL + 8 * k, db + 2 * k, IDESC, k > 0 ? 1u : 0u);
+        umma_commit(bar_mma);
+    };
+
+    int fold_doc = -1, fold_end = 0;                          // document of the warp's first token in the tile being folded
+    int32_t cid = -1, cid_next = -1;
+    uint32_t cw[TW] = {};
+    const int grp = lane & 3, sub = lane >> 2;                // fold: four query tokens, a row of every eight
+    const int col0 = part * G4U_COLS + 4 * grp;
+    // The MMAs of tile t + 1 run while tile t is folded: accumulators are read back and the A operand is rewritten as soon
+    // as tile t's MMAs are done, in front of the tile's only block barrier.
+    if (n_tiles > 0) {
+        fetch(0, cid, cw);
+        expand(cw);
+        if (n_tiles > 1) fetch(1, cid_next, cw);
         tc_fence_before();
         __syncthreads();
-
-        // ---- one thread issues the MMAs --------------------------------------------------------------------------
         if (tid == 0) {
-            bool ok = true;
-            if (tile == 0) ok = mbar_wait(bar_b, 0, wait_limit);
-            if (ok) {
-                tc_fence_after();
-                const uint64_t db = umma_desc(sB);
-                for (int k = 0; k < k_steps; ++k) umma_i8_ts(tmem, tmem + A_COL + 8 * k, db + 2 * k, IDESC, k > 0 ? 1u : 0u);
-                umma_commit(bar_mma);
-            } else {
-                s_abort = 1;
-            }
+            if (mbar_wait(bar_b, 0, wait_limit)) issue();
+            else s_abort = 1;
         }
         __syncwarp();
+    }
 
-        // ---- while the tensor core works: this token's row of the score table, and the next tile's token -----------
-        int4 sv[NQP / 4];
-        if (!RQ && cid >= 0) {
-            const int32_t *srow = tb + (int64_t)DBG_CID(cid) * nq;
+    // Score-table entries of a tile's tokens, in the layout in which the accumulators come back: rows sub, sub + 8, ... of the
+    // warp's 32 tokens, query tokens col0 ... col0 + 3.  Four lanes read 64 bytes of a row, so a load of the warp touches
+    // eight lines; one thread per row would touch 32 with each.
+    int32_t sv[4][4];
+    auto load_rows = [&](int32_t cid) {
 #pragma unroll
-            for (int g = 0; g < NQP / 4; ++g) {
-                const int col = 4 * g;
-                if (wide_rows && col + 7 < nq) {
-                    // 32 bytes per load: half as many line lookups per row as with 16-byte pieces
-                    if ((g & 1) == 0)
-                        asm volatile("ld.global.nc.v8.s32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                                     : "=r"(sv[g].x), "=r"(sv[g].y), "=r"(sv[g].z), "=r"(sv[g].w), "=r"(sv[g + 1].x),
-                                       "=r"(sv[g + 1].y), "=r"(sv[g + 1].z), "=r"(sv[g + 1].w)
-                                     : "l"(srow + col));
-                } else if (wide_rows && (g & 1) == 1 && col + 3 < nq) {
-                    // second half of a 32-byte load issued at g - 1
-                } else if (vec_rows && col + 3 < nq) {
-                    sv[g] = __ldg(reinterpret_cast<const int4 *>(srow + col));
-                } else {
-                    sv[g].x = col + 0 < nq ? __ldg(srow + col + 0) : 0;
-                    sv[g].y = col + 1 < nq ? __ldg(srow + col + 1) : 0;
-                    sv[g].z = col + 2 < nq ? __ldg(srow + col + 2) : 0;
-                    sv[g].w = col + 3 < nq ? __ldg(srow + col + 3) : 0;
-                }
+        for (int j = 0; j < 4; ++j) {
+            int32_t c = __shfl_sync(0xffffffffu, cid, sub + 8 * j);
+            c = DBG_CID(c > 0 ? c : 0);                       // (rows without a token take part in no maximum)
+            const int32_t *src = reinterpret_cast<const int32_t *>(tb + (uint64_t)(uint32_t)c * row_bytes) + col0;
+            if (FULL || (vec_rows && col0 < nq)) {
+                const int4 q = __ldg(reinterpret_cast<const int4 *>(src));
+                sv[j][0] = q.x; sv[j][1] = q.y; sv[j][2] = q.z; sv[j][3] = q.w;
+            } else {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) sv[j][e] = col0 + e < nq ? __ldg(src + e) : 0;
             }
         }
-        if (tile + 1 < n_tiles) {
-            fetch(tile + 1, dl_next, cid_next, cw_next);
-            // the next token's score-table row is a scattered 4 * q_len-byte read that misses L2 (a batch's tables
-            // are far larger): ask for it now so that HBM latency passes during this tile's epilogue
-            // (measured: a gain for q_len <= 32, a loss for the two-line rows of longer queries)
-            if (!RQ && NQP == 32 && cid_next >= 0) {
-                const char *row = reinterpret_cast<const char *>(tb + (int64_t)DBG_CID(cid_next) * nq);
-                for (int off = 0; off < nq * 4; off += 128) asm volatile("prefetch.global.L2 [%0];" ::"l"(row + off));
-            }
+    };
+    if (!RQ) load_rows(cid);
+
+    for (int tile = 0; tile < n_tiles; ++tile) {
+        // the next token's scattered score-table row misses L2 (a batch's tables are far larger): ask for it now
+        // (measured: a gain for q_len <= 32, a loss for the two-line rows of longer queries)
+        if (!RQ && NQP == 32 && part == 0 && cid_next >= 0) {
+            const char *next = tb + (uint64_t)(uint32_t)DBG_CID(cid_next) * row_bytes;
+            for (int off = 0; off < nq * 4; off += 128) asm volatile("prefetch.global.L2 [%0];" ::"l"(next + off));
         }
 
         const bool ok = mbar_wait(bar_mma, tile & 1, wait_limit);
+        tc_fence_after();
+        __syncwarp();
+
+        // ---- accumulators -> code products of rows sub + 8 j, query tokens col0 ... col0 + 3 --------------------------------
+        const uint32_t lane_addr = tmem + ((uint32_t)(quarter * 32) << 16) + part * G4U_COLS;
+        int32_t T[4][4];
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+            int32_t a0[8], a1[8], a2[8];
+            tmem_ld_16x16(lane_addr + (uint32_t)(half * 16 << 16) + 0 * NQP, a0);
+            tmem_ld_16x16(lane_addr + (uint32_t)(half * 16 << 16) + 1 * NQP, a1);
+            tmem_ld_16x16(lane_addr + (uint32_t)(half * 16 << 16) + 2 * NQP, a2);
+            tmem_ld_wait();
+#pragma unroll
+            for (int o = 0; o < 8; ++o)
+                // |sum_x u_x Xq_x| <= 3 * 2^22 * |q|_1 < 2^31: the plane recombination fits int32
+                T[2 * half + (o >> 1 & 1)][(o & 1) + (o >> 2) * 2] = (a2[o] * 256 + a1[o]) * 256 + a0[o];
+        }
+
+        // ---- the next tile's codes, its MMAs, the token after it ----------------------------------------------------------
+        if (tile + 1 < n_tiles) expand(cw);
+        tc_fence_before();
         if (!__syncthreads_and(ok && !*(volatile int *)&s_abort)) {
             if (tid == 0) atomicOr(status, ST_TIMEOUT);
             alive = false;
             break;
         }
-        tc_fence_after();
+        if (tid == 0 && tile + 1 < n_tiles) issue();
         __syncwarp();
+        int32_t cid_far = -1;
+        if (tile + 2 < n_tiles) fetch(tile + 2, cid_far, cw);
 
-        // ---- accumulators -> values of this thread's token for every query token -----------------------------------
-        const uint32_t lane_addr = tmem + ((uint32_t)(warp * 32) << 16);
-        float *vrow = vals + tid * VP;
+        // ---- values (times 2^24: S is an integer there, and a power of two changes no rounding); the next tile's rows --------
+        float v[4][4];
 #pragma unroll
-        for (int ch = 0; ch < NQP / 16; ++ch) {
-            int32_t a0[16], a1[16], a2[16];
-            tmem_ld16(lane_addr + 0 * NQP + ch * 16, a0);
-            tmem_ld16(lane_addr + 1 * NQP + ch * 16, a1);
-            tmem_ld16(lane_addr + 2 * NQP + ch * 16, a2);
-            tmem_ld_wait();
-            if (cid >= 0) {
+        for (int j = 0; j < 4; ++j) {
+            const float f = RQ ? __int_as_float(__shfl_sync(0xffffffffu, cid, sub + 8 * j)) : 0.f;
 #pragma unroll
-                for (int g = 0; g < 4; ++g) {
-                    const int4 q4 = RQ ? make_int4(0, 0, 0, 0) : sv[ch * 4 + g];
-                    const int32_t se[4] = {q4.x, q4.y, q4.z, q4.w};
-                    float val[4];
+            for (int e = 0; e < 4; ++e)
+                v[j][e] = RQ ? __fmul_rn(f, __fmul_rn(kappa, (float)(2 * T[j][e] - s_sq[col0 + e])))
+                             : fmaf(code_scale, (float)T[j][e], (float)sv[j][e]);
+        }
+        if (!RQ) load_rows(cid_next);
+
+        // ---- fold the warp's 32 tokens into the per-document maxima ---------------------------------------------------------
+        // maximum over the eight lanes of a column group: each exchange keeps half of the columns, the last one is whole
+        auto publish = [&](int doc, float m0, float m1, float m2, float m3) {
+            const bool up = (lane & 16) != 0, up2 = (lane & 8) != 0;
+            const float h0 = fmaxf(up ? m2 : m0, __shfl_xor_sync(0xffffffffu, up ? m0 : m2, 16));
+            const float h1 = fmaxf(up ? m3 : m1, __shfl_xor_sync(0xffffffffu, up ? m1 : m3, 16));
+            float x = fmaxf(up2 ? h1 : h0, __shfl_xor_sync(0xffffffffu, up2 ? h0 : h1, 8));
+            x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, 4));
+            if ((lane & 4) == 0) atomicMax(&docmax[doc * NQP + col0 + (up ? 2 : 0) + (up2 ? 1 : 0)], f_order(x));
+        };
+        const int s0 = tile * G4U_TOK + quarter * 32;          // first token of the warp
+        if (s0 < total) {
+            if (s0 >= fold_end) {
+                do fold_end = s_off[++fold_doc + 1]; while (fold_end <= s0);
+            }
+            if (fold_end >= s0 + 32) {
+                // all 32 tokens are of one document (most of a long document's)
+                float m[4];
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const int o = 4 * g + e;
-                        // |sum_x u_x Xq_x| <= 3 * 2^22 * |q|_1 < 2^31: the plane recombination fits int32
-                        const int32_t T = a0[o] + a1[o] * 256 + a2[o] * 65536;
-                        if (RQ)
-                            val[e] = __fmul_rn(__int_as_float(cid), __fmul_rn(kappa, (float)(2 * T - s_sq[ch * 16 + o])));
-                        else
-                            val[e] = fmaf(code_scale, (float)T, (float)se[e] * (1.0f / 16777216.0f));
-                    }
-                    const int grp = ch * 4 + g;               // 16-byte group of the row
-                    *reinterpret_cast<float4 *>(vrow + 4 * (ON_A ? grp ^ (tid & 7) : grp)) =
-                        make_float4(val[0], val[1], val[2], val[3]);
+                for (int e = 0; e < 4; ++e) m[e] = fmaxf(fmaxf(v[0][e], v[1][e]), fmaxf(v[2][e], v[3][e]));
+                publish(fold_doc, m[0], m[1], m[2], m[3]);
+            } else {
+                // several documents, or the stream's end: one document after the other
+                int a = 0;                                     // rows [a, b1) of the warp's 32
+                for (int doc = fold_doc; doc < nd && a < 32; ++doc) {
+                    const int b1 = s_off[doc + 1] - s0;
+                    if (b1 <= a) continue;                     // (a slot without a document)
+                    float m[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+                    for (int jj = 0; jj < 4; ++jj)
+                        if (sub + 8 * jj >= a && sub + 8 * jj < b1)
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) m[e] = fmaxf(m[e], v[jj][e]);
+                    publish(doc, m[0], m[1], m[2], m[3]);
+                    a = b1;
                 }
             }
         }
-        tc_fence_before();
-        __syncwarp();
-
-        // ---- fold this warp's 32 tokens into the per-document maxima (lane = query token) -------------------------
-        {
-            const int prev = __shfl_up_sync(0xffffffffu, dl, 1);
-            const uint32_t valid = __ballot_sync(0xffffffffu, dl >= 0);
-            uint32_t starts = __ballot_sync(0xffffffffu, dl >= 0 && (lane == 0 || dl != prev));
-            const int n_rows = __popc(valid);                 // valid rows are a prefix of the warp's rows
-            if (ON_A && starts == 1u && valid == 0xffffffffu) {
-                // The warp's 32 tokens belong to one document (most tiles of a long document): lane = (four columns,
-                // a quarter of the rows), eight 16-byte loads per lane instead of 32 scalar ones, then two exchange
-                // steps among the four lanes of a column group.
-                const int grp = lane & 7, sub = lane >> 3;
-                const float *vb = vals + warp * 32 * VP;
-                float4 m = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const int r = sub + 4 * j;
-                    const float4 v = *reinterpret_cast<const float4 *>(vb + r * VP + ((grp ^ (r & 7)) << 2));
-                    m.x = fmaxf(m.x, v.x); m.y = fmaxf(m.y, v.y); m.z = fmaxf(m.z, v.z); m.w = fmaxf(m.w, v.w);
-                }
-#pragma unroll
-                for (int o = 8; o <= 16; o <<= 1) {
-                    m.x = fmaxf(m.x, __shfl_xor_sync(0xffffffffu, m.x, o));
-                    m.y = fmaxf(m.y, __shfl_xor_sync(0xffffffffu, m.y, o));
-                    m.z = fmaxf(m.z, __shfl_xor_sync(0xffffffffu, m.z, o));
-                    m.w = fmaxf(m.w, __shfl_xor_sync(0xffffffffu, m.w, o));
-                }
-                const int doc = __shfl_sync(0xffffffffu, dl, 0);
-                // lane (grp, sub) publishes column 4 grp + sub
-                const float mine = sub == 0 ? m.x : sub == 1 ? m.y : sub == 2 ? m.z : m.w;
-                atomicMax(&docmax[doc * NQP + 4 * grp + sub], f_order(mine));
-                starts = 0u;
-            }
-            while (starts) {
-                const int a = __ffs(starts) - 1;
-                starts &= starts - 1;
-                const int e = starts ? __ffs(starts) - 1 : n_rows;
-                const int doc = __shfl_sync(0xffffffffu, dl, a);
-                float m0, m1 = 0.f;
-                if (ON_A) {
-                    // column `lane` of row r sits in group (lane / 4) ^ (r & 7)
-                    const float *vw = vals + warp * 32 * VP + (lane & 3);
-                    m0 = vw[a * VP + ((((lane >> 2) ^ a) & 7) << 2)];
-                    for (int r = a + 1; r < e; ++r) m0 = fmaxf(m0, vw[r * VP + ((((lane >> 2) ^ r) & 7) << 2)]);
-                } else {
-                    const float *vp = vals + (warp * 32 + a) * VP + lane;
-                    m0 = vp[0];
-                    m1 = NQP > 32 ? vp[32] : 0.f;
-                    for (int r = a + 1; r < e; ++r) {
-                        vp += VP;
-                        m0 = fmaxf(m0, vp[0]);
-                        if (NQP > 32) m1 = fmaxf(m1, vp[32]);
-                    }
-                }
-                atomicMax(&docmax[doc * NQP + lane], f_order(m0));
-                if (NQP > 32) atomicMax(&docmax[doc * NQP + 32 + lane], f_order(m1));
-            }
-            // the value rows of this warp are rewritten by the next tile's epilogue, each lane its own row, while the
-            // fold above reads the rows of other lanes: all lanes finish reading first
-            __syncwarp();
-        }
+        cid = cid_next;
+        cid_next = cid_far;
     }
 
     if (n_tiles == 0 && tid == 0 && !skip_loads) mbar_wait(bar_b, 0, wait_limit);   // never leave with the TMA load in flight
@@ -429,8 +383,8 @@ residual_maxsim_umma(const __grid_constant__ CUtensorMap map_q, const float *__r
                 if (d >= 0 && lane == 0)
                     for (int i = 0; i < nq; ++i) v = __fadd_rn(v, f_unorder(docmax[dl * NQP + i]));
             } else if (d >= 0) {
-                if (lane < nq) v = f_unorder(docmax[dl * NQP + lane]) + kappa * s_sumq[lane];
-                if (NQP > 32 && 32 + lane < nq) v += f_unorder(docmax[dl * NQP + 32 + lane]) + kappa * s_sumq[32 + lane];
+                if (lane < nq) v = f_unorder(docmax[dl * NQP + lane]) * (1.0f / 16777216.0f) + kappa * s_sumq[lane];
+                if (NQP > 32 && 32 + lane < nq) v += f_unorder(docmax[dl * NQP + 32 + lane]) * (1.0f / 16777216.0f) + kappa * s_sumq[32 + lane];
             }
             v = warp_sum(v);
             if (lane == 0) score4[(int64_t)b * n_prune + j0 + dl] = d >= 0 ? v : -INFINITY;
@@ -443,7 +397,7 @@ residual_maxsim_umma(const __grid_constant__ CUtensorMap map_q, const float *__r
 }
 
 template <int NQP, int NBITS, bool RQ>
-static int launch_g4_umma(const Index &ix, const Params &p, const float *queries, const int8_t *qdig,
+static int launch_g4_umma(const Index &ix, const Params &p, const float *queries, const int8_t *qdig4,
                           const int32_t *table, const int32_t *pruned, float *score4, uint32_t *status, cudaStream_t st)
 {
     constexpr int N = 3 * NQP;
@@ -451,18 +405,17 @@ static int launch_g4_umma(const Index &ix, const Params &p, const float *queries
     // RQ: the kappa slot carries c = 1 / (sqrt(D) * 2^22)
     const float kappa = RQ ? (float)(1.0 / (sqrt((double)ix.D) * 4194304.0)) : ix.res_lo + 0.5f * delta;
     CUtensorMap map_q;
-    int rc = make_plane_map(&map_q, qdig, (int64_t)p.B * p.nq, NQP);
+    int rc = make_plane_map(&map_q, qdig4, (int64_t)p.B * NQP, NQP);
     if (rc) return rc;
-    // value rows (128-byte rows for q_len <= 32 with residual codes, padded rows otherwise), query planes, maxima
-    size_t smem = 1024 + sizeof(float) * G4U_TOK * (NQP == 32 && !RQ ? 32 : NQP + 4) + (size_t)N * 128 +
-                  sizeof(uint32_t) * G4U_MAX_DOCS * NQP + 32;
+    // query planes, maxima
+    size_t smem = 1024 + (size_t)N * 128 + sizeof(uint32_t) * G4U_MAX_DOCS * NQP + 32;
     // No more CTAs may become resident on an SM than its 512 tensor-memory columns serve: one more would sit in
-    // tcgen05.alloc with its registers and shared memory until another leaves (64-token queries: three CTAs of 66 KB
-    // fit an SM, two get tensor memory; measured 5.97 -> 8.92 ms).  Registers cap the 128-column residual variants at
-    // four; the 256-column variants ask for a third of an SM's shared memory plus one byte.  (The 128-column RaBitQ
-    // variant, whose tiles are short, measured the same with and without such a cap and has none.)
+    // tcgen05.alloc with its registers and shared memory until another leaves.  Registers cap the 128-column variants at
+    // four or fewer and the 256-column ones at two; the latter ask for a third of an SM's shared memory plus one byte
+    // besides, so that a build with fewer registers does not change that.
     if (N > 96 && smem < 227 * 1024 / 3 + 1) smem = 227 * 1024 / 3 + 1;
-    auto kern = residual_maxsim_umma<NQP, NBITS, RQ>;
+    auto kern = p.nq == NQP && ix.D == 128 ? residual_maxsim_umma<NQP, NBITS, RQ, true>
+                                           : residual_maxsim_umma<NQP, NBITS, RQ, false>;
     CHIMERA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     // documents per CTA: about four CTAs per SM in total, at most 32 documents each (with few queries per call a CTA
     // gets one or two documents, so that the call's latency is a tile or two and not a chain of them)
@@ -472,7 +425,7 @@ static int launch_g4_umma(const Index &ix, const Params &p, const float *queries
     if (dpc > p.n_prune) dpc = p.n_prune;
     dim3 grid((unsigned)((p.n_prune + dpc - 1) / dpc), (unsigned)p.B);
     const uint32_t *code_words = reinterpret_cast<const uint32_t *>(RQ ? ix.rq_bits : ix.codes);
-    kern<<<grid, G4U_THREADS, smem, st>>>(map_q, queries, table, ix.K, p.nq, ix.D, RQ ? ix.D / 32 : ix.CB / 4, delta,
+    kern<<<grid, 128 * (NQP / G4U_COLS), smem, st>>>(map_q, queries, table, ix.K, p.nq, ix.D, RQ ? ix.D / 32 : ix.CB / 4, delta,
                                           kappa, pruned, p.n_prune, (int)dpc, ix.cids, code_words, ix.rq_inv, ix.doc_off,
                                           score4, status, wait_limit_cycles(), fault_skip_tma_loads());
     CHIMERA_CUDA(cudaGetLastError());
@@ -482,16 +435,16 @@ static int launch_g4_umma(const Index &ix, const Params &p, const float *queries
 
 bool residual_umma_supported(int nq) { return nq <= 64; }
 
-int launch_residual_scores_umma(const Index &ix, const Params &p, const float *queries, const int8_t *qdig,
+int launch_residual_scores_umma(const Index &ix, const Params &p, const float *queries, const int8_t *qdig4,
                                 const int32_t *table, const int32_t *pruned, float *score4, uint32_t *status,
                                 cudaStream_t st)
 {
     if (ix.nbits == 2) {
-        if (p.nq <= 32) return launch_g4_umma<32, 2, false>(ix, p, queries, qdig, table, pruned, score4, status, st);
-        return launch_g4_umma<64, 2, false>(ix, p, queries, qdig, table, pruned, score4, status, st);
+        if (p.nq <= 32) return launch_g4_umma<32, 2, false>(ix, p, queries, qdig4, table, pruned, score4, status, st);
+        return launch_g4_umma<64, 2, false>(ix, p, queries, qdig4, table, pruned, score4, status, st);
     }
-    if (p.nq <= 32) return launch_g4_umma<32, 1, false>(ix, p, queries, qdig, table, pruned, score4, status, st);
-    return launch_g4_umma<64, 1, false>(ix, p, queries, qdig, table, pruned, score4, status, st);
+    if (p.nq <= 32) return launch_g4_umma<32, 1, false>(ix, p, queries, qdig4, table, pruned, score4, status, st);
+    return launch_g4_umma<64, 1, false>(ix, p, queries, qdig4, table, pruned, score4, status, st);
 }
 
 // Complete 1-bit scores of the surviving documents on the RaBitQ codes; q_rot / qdig_rot belong to the rotated queries.

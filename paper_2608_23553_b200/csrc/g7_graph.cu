@@ -24,15 +24,15 @@ constexpr int GP_WARPS = 4;              // query tokens (warps) per block
 constexpr int GP_PIPE = 8;               // centroid rows in flight per warp while scoring
 
 // Xc[c][d] = rint(centroid * 2^22), recombined from the three balanced base-256 digit planes of the index.
-__global__ void xc_kernel(const int8_t *__restrict__ cdig, int64_t K, int D, int32_t *__restrict__ xc)
+__global__ void xc_kernel(const int8_t *__restrict__ cdig, int64_t K, int D, int nbits, int32_t *__restrict__ xc)
 {
     const int64_t n = K * D;
     const int64_t plane = K * 128;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
         const int64_t c = e / D;
-        const int d = (int)(e % D);
-        const int64_t at = c * 128 + d;
-        xc[e] = (int)cdig[at] + 256 * (int)cdig[plane + at] + 65536 * (int)cdig[2 * plane + at];
+        const int i = (int)(e % D);                          // (D is a multiple of 32: positions below D hold all dimensions)
+        const int64_t at = c * 128 + i;
+        xc[c * D + digit_dim(i, nbits)] = (int)cdig[at] + 256 * (int)cdig[plane + at] + 65536 * (int)cdig[2 * plane + at];
     }
 }
 
@@ -83,7 +83,7 @@ int build_graph(Index &ix, const float *centroids, int R, cudaStream_t st)
         drop();
         return fail(CHIMERA_CUDA_ERROR, "cudaMalloc (centroid graph): %s", cudaGetErrorString(e));
     }
-    xc_kernel<<<(unsigned)(8 * ix.sm_count), 256, 0, st>>>(ix.cdig, ix.K, ix.D, xc);
+    xc_kernel<<<(unsigned)(8 * ix.sm_count), 256, 0, st>>>(ix.cdig, ix.K, ix.D, ix.nbits, xc);
     uint32_t *status = (uint32_t *)(ws + L.status);
     int8_t *qdig = (int8_t *)(ws + L.qdig);
     int32_t *table = (int32_t *)(ws + L.table);
@@ -96,7 +96,7 @@ int build_graph(Index &ix, const float *centroids, int R, cudaStream_t st)
         if (e == cudaSuccess && rows < rows_per_call)
             e = cudaMemsetAsync(qbuf + (size_t)rows * ix.D, 0, sizeof(float) * (size_t)(rows_per_call - rows) * ix.D, st);
         if (e != cudaSuccess) { rc = fail(CHIMERA_CUDA_ERROR, "copy (centroid graph): %s", cudaGetErrorString(e)); break; }
-        if ((rc = launch_score_table(ix, p, qbuf, qdig, table, nullptr, status, st))) break;
+        if ((rc = launch_score_table(ix, p, qbuf, qdig, nullptr, table, nullptr, status, st))) break;
         if ((rc = launch_probes(ix, p, L, table, part, probes, st))) break;
         graph_rows_kernel<<<(unsigned)((rows + 127) / 128), 128, 0, st>>>(probes, c0, rows, R, graph);
     }

@@ -110,15 +110,15 @@ static int exclusive_scan(const int32_t *in, int64_t n, int64_t *out, int64_t *t
 // ------------------------------------------------------------------------------------------------ digit planes ---
 // X = rint(x * 2^22) split into balanced base-256 digits X = d0 + 256 d1 + 65536 d2, d0, d1 in [-128, 127],
 // |d2| <= 64.  Planes have a fixed row pitch of DIGIT_PITCH (128) bytes, dimensions >= D are zero:
-// plane p of row r, dimension d sits at dig[(p * rows + r) * 128 + d].
+// plane p of row r, dimension digit_dim(i) sits at dig[(p * rows + r) * 128 + i].
 // Rows must also be (at most) unit-norm: later stages rely on |S_fx| <= 2^24 + 2^16, which holds when both factors
 // have sum_d X[d]^2 <= 2^44 + 2^35 (norm <= 1 + 2^-10).  A longer row sets the same status bit as an element out of
 // range.  A block of 256 threads holds two rows (one thread per padded dimension).
 constexpr int DIGIT_PITCH = 128;
 constexpr long long MAX_ROW_SQUARE_SUM = (1LL << 44) + (1LL << 35);
 
-__global__ void digits_kernel(const float *__restrict__ x, int64_t rows, int D, int8_t *__restrict__ dig,
-                              uint32_t *status)
+__global__ void digits_kernel(const float *__restrict__ x, int64_t rows, int D, int nbits, int8_t *__restrict__ dig,
+                              int8_t *__restrict__ dig4, int q_len, uint32_t *status)
 {
     __shared__ unsigned long long row_sq[2];
     const int64_t n = rows * DIGIT_PITCH;
@@ -126,7 +126,7 @@ __global__ void digits_kernel(const float *__restrict__ x, int64_t rows, int D, 
     if (threadIdx.x < 2) row_sq[threadIdx.x] = 0ull;
     __syncthreads();
     const int64_t r = i / DIGIT_PITCH;
-    const int d = (int)(i % DIGIT_PITCH);
+    const int d = digit_dim((int)(i % DIGIT_PITCH), nbits);
     int d0 = 0, d1 = 0, d2 = 0;
     unsigned long long sq = 0ull;
     if (i < n && d < D) {
@@ -143,10 +143,18 @@ __global__ void digits_kernel(const float *__restrict__ x, int64_t rows, int D, 
         d1 = ((X1 + 128) & 255) - 128;
         d2 = (X1 - d1) >> 8;
     }
-    if (i < n) {
+    if (i < n && dig) {
         dig[i] = (int8_t)d0;
         dig[n + i] = (int8_t)d1;
         dig[2 * n + i] = (int8_t)d2;
+    }
+    if (i < n && dig4) {
+        const int per = residual_rows(q_len);
+        const int64_t b = r / q_len, n4 = rows / q_len * per * DIGIT_PITCH;
+        const int64_t at = (b * per + score_row((int)(r - b * q_len))) * DIGIT_PITCH + i % DIGIT_PITCH;
+        dig4[at] = (int8_t)d0;
+        dig4[n4 + at] = (int8_t)d1;
+        dig4[2 * n4 + at] = (int8_t)d2;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
@@ -156,10 +164,11 @@ __global__ void digits_kernel(const float *__restrict__ x, int64_t rows, int D, 
         atomicOr(status, ST_BAD_QUERY);
 }
 
-int launch_digits(const float *x, int64_t rows, int D, int8_t *dig, uint32_t *status, cudaStream_t st)
+int launch_digits(const float *x, int64_t rows, int D, int nbits, int8_t *dig, int8_t *dig4, int q_len, uint32_t *status,
+                  cudaStream_t st)
 {
     const int64_t n = rows * DIGIT_PITCH;
-    digits_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(x, rows, D, dig, status);
+    digits_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(x, rows, D, nbits, dig, dig4, q_len, status);
     CHIMERA_CUDA(cudaGetLastError());
     return CHIMERA_OK;
 }
@@ -333,7 +342,7 @@ int build_index_device(Index &ix, const float *centroids, const int32_t *doclens
     // centroid digit planes
     BUILD_CUDA(cudaMalloc(&ix.cdig, (size_t)3 * ix.K * DIGIT_PITCH));
     BUILD_CUDA(cudaMemsetAsync(flags, 0, sizeof(int32_t), st));
-    rc = launch_digits(centroids, ix.K, ix.D, ix.cdig, (uint32_t *)flags, st);
+    rc = launch_digits(centroids, ix.K, ix.D, ix.nbits, ix.cdig, nullptr, 1, (uint32_t *)flags, st);
     if (rc) { cleanup(); return rc; }
 
     // inverted file
