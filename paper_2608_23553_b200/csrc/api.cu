@@ -149,17 +149,11 @@ Layout make_layout(const Index &ix, const Params &p)
     L.n_kept = take(filter ? B * sizeof(int32_t) : 0);
     L.n_seed = take(filter ? B * sizeof(int32_t) : 0);
     L.pruned = take(B * p.n_prune * sizeof(int32_t));
-    L.word_rank = take(B * (size_t)L.words * sizeof(int32_t));
-    // partial-score table: dense rows per candidate (always for the RaBitQ refinement), or the hashed form
-    L.hash_slots = partial_hash_slots(ix, p);
-    {
-        const size_t dense = B * (size_t)p.maxc * nq * sizeof(int32_t);
-        const size_t hashed = B * (size_t)L.hash_slots * sizeof(unsigned long long);
-        size_t bytes = 0;
-        if (ix.tok_id) bytes = L.hash_slots ? hashed : dense;
-        if (ix.rot_t && bytes < dense) bytes = dense;
-        L.partial_m = take(bytes);
-    }
+    L.ranks = take(ix.tok_id ? B * (size_t)L.words * sizeof(uint2) : 0);
+    // retrieved-token scores of the refinements: visit lists, or dense rows per candidate
+    L.visit_nodes = visit_list_nodes(ix, p);
+    L.partial_m = take(!ix.tok_id ? 0 : L.visit_nodes ? B * ((size_t)L.visit_nodes * 8 + (size_t)p.maxc * 4)
+                                                      : B * (size_t)p.maxc * nq * sizeof(int32_t));
     L.graph_vis = take(ix.graph ? graph_scratch_bytes(ix, (int64_t)p.B * p.nq) : 0);
     L.q_rot = take(ix.rot_t ? B * nq * ix.D * sizeof(float) : 0);
     L.qdig_rot = take(ix.rot_t ? 3 * rows4 * 128 : 0);
@@ -285,8 +279,8 @@ static int run(const Index &ix, const Params &p, int first, int last, const floa
     int32_t *n_pruned = (int32_t *)(ws + L.n_pruned);
     int32_t *pruned_ci = (int32_t *)(ws + L.pruned_ci);
     int32_t *sel_scratch = select_split_used(ix, p) ? (int32_t *)(ws + L.sel_scratch) : nullptr;
-    int32_t *word_rank = (int32_t *)(ws + L.word_rank);
-    int32_t *partial_m = (int32_t *)(ws + L.partial_m);
+    uint2 *ranks = (uint2 *)(ws + L.ranks);
+    void *partial_m = ws + L.partial_m;
     float *q_rot = (float *)(ws + L.q_rot);
     int8_t *qdig_rot = (int8_t *)(ws + L.qdig_rot);
     float *score4 = (float *)(ws + L.score4);
@@ -348,7 +342,8 @@ static int run(const Index &ix, const Params &p, int first, int last, const floa
             return rc;
         }
         prof_mark(SLOT_PROBE, st);
-        if ((rc = launch_gather(ix, p, L, probes, bitmap, chunk_cnt, cand, n_cand, word_rank, status, st))) return rc;
+        if ((rc = launch_gather(ix, p, L, probes, bitmap, chunk_cnt, cand, n_cand,
+                                partial || rabitq ? ranks : nullptr, status, st))) return rc;
         prof_mark(SLOT_GATHER, st);
     }
     if (first <= 3 && last >= 3) {
@@ -358,15 +353,14 @@ static int run(const Index &ix, const Params &p, int first, int last, const floa
             if ((rc = launch_digits(q_rot, (int64_t)p.B * p.nq, ix.D, 1, nullptr, qdig_rot, p.nq, status, st))) return rc;
             count_launch(SLOT_G1);
             prof_mark(SLOT_G1, st);
-            if ((rc = launch_rabitq_partial(ix, p, L, q_rot, probes, bitmap, word_rank, n_cand, partial_m, ci, st)))
+            if ((rc = launch_rabitq_partial(ix, p, L, q_rot, probes, ranks, n_cand, partial_m, ci, st)))
                 return rc;
             prof_mark(SLOT_CI, st);
             if ((rc = launch_select(ix, p, cand, n_cand, ci, pruned, n_pruned, pruned_ci, sel_scratch, st))) return rc;
             prof_mark(SLOT_SELECT, st);
         } else if (partial) {
             // the paper's candidate refinement: partial scores from the retrieved tokens only, then the same selection
-            if ((rc = launch_partial_scores(ix, p, L, queries, table, probes, bitmap, word_rank, n_cand, partial_m, ci,
-                                            status, st)))
+            if ((rc = launch_partial_scores(ix, p, L, queries, table, probes, ranks, n_cand, partial_m, ci, st)))
                 return rc;
             prof_mark(SLOT_CI, st);
             if ((rc = launch_select(ix, p, cand, n_cand, ci, pruned, n_pruned, pruned_ci, sel_scratch, st))) return rc;

@@ -101,10 +101,11 @@ struct Layout {
     size_t n_kept;        // int32  [B]
     size_t n_seed;        // int32  [B]
     size_t pruned;        // int32  [B][n_prune]
-    size_t word_rank;     // int32  [B][words]        candidates before each bitmap word (document -> candidate index)
-    size_t partial_m;     // int32  [B][maxc][nq]     per (candidate, query token) best retrieved-token score, or
-                          // uint64 [B][hash_slots]   the same as an open-addressing table (see partial_hash_slots)
-    int64_t hash_slots;   // slots per query of that table; 0 = the dense form
+    size_t ranks;         // uint2  [B][words]        bitmap word, candidates before it (document -> candidate index);
+                          //                          only with token lists
+    size_t partial_m;     // int32  [B][maxc][nq]     per (candidate, query token) best retrieved-token score, or the visit
+                          //                          lists in its place (g3_visits.cuh)
+    int64_t visit_nodes;  // nodes per query of those lists; 0 = the table
     size_t graph_vis;     // uint32 [B*nq][K/32]      visited centroids of the graph search (only with a centroid graph)
     size_t q_rot;         // float  [B, nq, D]        rotated queries (RaBitQ pipeline)
     size_t qdig_rot;      // int8   [3][B*residual_rows(nq)][128]  their digit planes for stage 4
@@ -179,19 +180,15 @@ int launch_probe_sample(const Index &ix, const Params &p, const Layout &L, const
                         int n_sample_tiles, cudaStream_t st);
 int launch_probe_merge(const Index &ix, const Params &p, const Layout &L, const int32_t *table, char *ws, cudaStream_t st);
 int launch_gather(const Index &ix, const Params &p, const Layout &L, const int32_t *probes, uint32_t *bitmap,
-                  int32_t *chunk_cnt, int32_t *cand, int32_t *n_cand, int32_t *word_rank, uint32_t *status,
+                  int32_t *chunk_cnt, int32_t *cand, int32_t *n_cand, uint2 *ranks, uint32_t *status,
                   cudaStream_t st);
 // Token-level posting lists for the partial-score refinement (allocates; index_build.cu).
 int build_token_lists(Index &ix, cudaStream_t st);
 // Candidate refinement with partial scores (Algorithm 2): fprime[b][j] for every candidate.
-// Slots per query (a power of two) of the hashed score table of the partial-score refinement, 0 when the dense table
-// is used (no token lists, few queries per call, keys that do not fit 32 bits, or a dense table less than four times
-// as large).
-int64_t partial_hash_slots(const Index &ix, const Params &p);
+int64_t visit_list_nodes(const Index &ix, const Params &p);
 int launch_partial_scores(const Index &ix, const Params &p, const Layout &L, const float *queries,
-                          const int32_t *table, const int32_t *probes, const uint32_t *bitmap,
-                          const int32_t *word_rank, const int32_t *n_cand, int32_t *partial_m, int32_t *fprime, uint32_t *status,
-                          cudaStream_t st);
+                          const int32_t *table, const int32_t *probes, const uint2 *ranks, const int32_t *n_cand,
+                          void *partial_m, int32_t *fprime, cudaStream_t st);
 int launch_filter_contenders(const Index &ix, const Params &p, const Layout &L, const int32_t *kept, const int2 *kept_rng,
                              const int32_t *n_kept, const int32_t *hi, int32_t *cont, int2 *cont_rng, int32_t *n_cont,
                              char *ws, cudaStream_t st);
@@ -263,8 +260,8 @@ int launch_graph_probes(const Index &ix, const float *queries, int64_t n_tokens,
 int attach_rabitq(Index &ix, const float *rotation, cudaStream_t st);
 int launch_rotate(const Index &ix, const Params &p, const float *queries, float *q_rot, cudaStream_t st);
 int launch_rabitq_partial(const Index &ix, const Params &p, const Layout &L, const float *q_rot,
-                          const int32_t *probes, const uint32_t *bitmap, const int32_t *word_rank,
-                          const int32_t *n_cand, int32_t *partial_m, int32_t *fprime_bits, cudaStream_t st);
+                          const int32_t *probes, const uint2 *ranks, const int32_t *n_cand, void *partial_m,
+                          int32_t *fprime_bits, cudaStream_t st);
 int launch_topk(const Index &ix, const Params &p, const int32_t *pruned, const float *score4, int32_t *out_ids,
                 float *out_scores, cudaStream_t st);
 

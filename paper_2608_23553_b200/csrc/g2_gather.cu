@@ -114,7 +114,7 @@ chunk_scan_kernel(int32_t *__restrict__ chunk_cnt, int n_chunks, int64_t maxc, i
 __global__ void __launch_bounds__(CHUNK_THREADS)
 compact_kernel(const uint32_t *__restrict__ bitmap, int64_t words, int n_chunks,
                const int32_t *__restrict__ chunk_cnt, int64_t maxc, int32_t *__restrict__ cand,
-               int32_t *__restrict__ word_rank)
+               uint2 *__restrict__ ranks)
 {
     const int b = blockIdx.y;
     const uint32_t *bm = bitmap + (int64_t)b * words;
@@ -138,8 +138,8 @@ compact_kernel(const uint32_t *__restrict__ bitmap, int64_t words, int n_chunks,
 #pragma unroll
     for (int j = 0; j < WORDS_PER_THREAD; ++j) {
         uint32_t bits = w[j];
-        if (w0 + j < words)
-            word_rank[(int64_t)b * words + w0 + j] = (int32_t)(use_stage ? base + pos : pos);
+        if (ranks && w0 + j < words)          // the word and the candidates before it: document -> candidate index
+            ranks[(int64_t)b * words + w0 + j] = make_uint2(w[j], (uint32_t)(use_stage ? base + pos : pos));
         while (bits) {
             int t = __ffs(bits) - 1;
             bits &= bits - 1;
@@ -157,7 +157,7 @@ compact_kernel(const uint32_t *__restrict__ bitmap, int64_t words, int n_chunks,
 }
 
 int launch_gather(const Index &ix, const Params &p, const Layout &L, const int32_t *probes, uint32_t *bitmap,
-                  int32_t *chunk_cnt, int32_t *cand, int32_t *n_cand, int32_t *word_rank, uint32_t *status,
+                  int32_t *chunk_cnt, int32_t *cand, int32_t *n_cand, uint2 *ranks, uint32_t *status,
                   cudaStream_t st)
 {
     CHIMERA_CUDA(cudaMemsetAsync(bitmap, 0, sizeof(uint32_t) * (size_t)L.words * p.B, st));
@@ -170,7 +170,7 @@ int launch_gather(const Index &ix, const Params &p, const Layout &L, const int32
     CHIMERA_CUDA(cudaGetLastError());
     chunk_scan_kernel<<<(unsigned)p.B, 32, 0, st>>>(chunk_cnt, L.n_chunks, p.maxc, n_cand, status);
     CHIMERA_CUDA(cudaGetLastError());
-    compact_kernel<<<gc, CHUNK_THREADS, 0, st>>>(bitmap, L.words, L.n_chunks, chunk_cnt, p.maxc, cand, word_rank);
+    compact_kernel<<<gc, CHUNK_THREADS, 0, st>>>(bitmap, L.words, L.n_chunks, chunk_cnt, p.maxc, cand, ranks);
     CHIMERA_CUDA(cudaGetLastError());
     count_launch(SLOT_GATHER, 4);
     return CHIMERA_OK;

@@ -13,44 +13,75 @@
 // no separate summation pass is needed.  The table is indexed by candidate rank (bitmap word prefix + popcount), so it has
 // one 4*q_len-byte row per candidate rather than per document.
 //
-// Only about one cell per candidate is ever touched (a candidate owns about one retrieved token), so on large corpora
-// the table is kept as an open-addressing hash table instead: key = rank * q_len + i + 1 in the high word of a 64-bit
-// slot, the running maximum in the low word; a slot's key never changes once set, so the maximum is one 64-bit
-// atomicMax on the slot.  The slots of a query (a power of two, at least twice the largest possible number of
-// visits: q_len * nprobe * longest list) are a few MB against tens of MB of dense rows: the clear is that much
-// shorter and the read-modify-writes of the queries in flight stay in L2.
-#include "common.cuh"
+// Batches on large corpora keep the visits as lists instead of the table (g3_visits.cuh); few queries per call keep the
+// table, whose update is one atomic and whose sum needs no second kernel.
+#include "g3_visits.cuh"
 
 namespace chimera {
 
 constexpr int PS_THREADS = 128;
-constexpr int HASH_MAX_PROBES = 256;     // linear probing gives up after this many slots (load factor <= 1/2)
 
-int64_t partial_hash_slots(const Index &ix, const Params &p)
+// Nodes per query of the visit lists, 0 when the table of maxima is used: no token lists, few queries per call (latency
+// counts), more nodes than their index holds, a table less than four times as large, or candidates with several visits
+// each, whose lists would be walked node by node (a mean of two: long documents under many probes stay with the table).
+int64_t visit_list_nodes(const Index &ix, const Params &p)
 {
-    if (!ix.tok_id || ix.max_tok_list <= 0) return 0;
-    if ((int64_t)p.maxc * p.nq >= 0xffffffffLL) return 0;                  // keys must fit 32 bits
-    if (4 * p.B <= ix.sm_count) return 0;      // few queries per call: latency counts, and a dense cell is one atomic
-                                               // where a slot is a load, a compare-and-swap and a maximum (Mid, one query:
-                                               // 36 us dense, 46 us hashed)
-    const int64_t visits = (int64_t)p.nq * p.P * ix.max_tok_list;          // distinct cells are at most the visits
-    int64_t slots = 1024;
-    while (slots < 2 * visits) slots <<= 1;
-    if (slots * 8 * 4 > (int64_t)p.maxc * p.nq * 4) return 0;              // worth it from a quarter of the dense size down
-                                                                           // (long documents, 32 MB against 51 MB: slower)
-    return slots;
+    if (!ix.tok_id || ix.max_tok_list <= 0 || 4 * p.B <= ix.sm_count) return 0;
+    const int64_t nodes = (int64_t)p.nq * p.P * ix.max_tok_list;
+    if (nodes > VISIT_MAX_NODES) return 0;
+    if (4 * (nodes * 8 + p.maxc * 4) > (int64_t)p.maxc * p.nq * 4) return 0;
+    const double len = (double)ix.T / (double)ix.N, probed = (double)p.nq * p.P / (double)ix.K;
+    return len * probed <= 1.6 ? nodes : 0;              // (visits per candidate: x / (1 - exp(-x)) = 2 at x = 1.6)
 }
 
-// grid (blocks, B): zero a query's slots and the first n_cand[b] partial scores.
-__global__ void __launch_bounds__(256)
-hash_clear_kernel(unsigned long long *__restrict__ H, int64_t slots, int32_t *__restrict__ fprime,
-                  const int32_t *__restrict__ n_cand, int64_t maxc)
+// Blocks per query token of the refinement kernels: one per probed list until the batch fills the GPU sixteen times over.
+int refine_splits(const Index &ix, const Params &p)
 {
-    const int b = blockIdx.y;
-    uint4 *row = reinterpret_cast<uint4 *>(H + (int64_t)b * slots);         // slots is a multiple of 1024
-    const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t e = tid; e < slots / 2; e += stride) row[e] = make_uint4(0u, 0u, 0u, 0u);
-    for (int64_t e = tid; e < n_cand[b]; e += stride) fprime[(int64_t)b * maxc + e] = 0;
+    int s = (int)((16LL * 8 * ix.sm_count + (int64_t)p.B * p.nq - 1) / ((int64_t)p.B * p.nq));
+    return s < 1 ? 1 : s > p.P ? p.P : s;
+}
+
+// grid (blocks, B): empty lists for the first n_cand[b] candidates.
+__global__ void __launch_bounds__(256)
+visit_clear_kernel(int32_t *__restrict__ head, const int32_t *__restrict__ n_cand, int64_t maxc)
+{
+    const int b = blockIdx.y, n = n_cand[b];
+    for (int e = blockIdx.x * 256 + threadIdx.x; e < n; e += gridDim.x * 256) head[(int64_t)b * maxc + e] = 0;
+}
+// grid (blocks, B): fprime[b][j] of every candidate, one thread each.
+template <bool FLOAT>
+__global__ void __launch_bounds__(256)
+visit_sum_kernel(const int32_t *__restrict__ head, const unsigned long long *__restrict__ node, int64_t cap,
+                 const int32_t *__restrict__ n_cand, int64_t maxc, int32_t *__restrict__ fprime)
+{
+    const int b = blockIdx.y, n = n_cand[b];
+    const unsigned long long *nodes = node + (int64_t)b * cap;
+    for (int j = blockIdx.x * 256 + threadIdx.x; j < n; j += gridDim.x * 256)
+        fprime[(int64_t)b * maxc + j] = visit_sum<FLOAT>(head[(int64_t)b * maxc + j], nodes);
+}
+VisitLists visit_lists(const Params &p, const Layout &L, void *mem)
+{
+    VisitLists v;
+    v.cap = L.visit_nodes;
+    v.node = (unsigned long long *)mem;
+    v.head = (int32_t *)(v.node + (int64_t)p.B * v.cap);
+    return v;
+}
+int launch_visit_clear(const Index &ix, const Params &p, const VisitLists &v, const int32_t *n_cand, cudaStream_t st)
+{
+    int64_t gx = (8LL * ix.sm_count + p.B - 1) / p.B;
+    visit_clear_kernel<<<dim3((unsigned)gx, (unsigned)p.B), 256, 0, st>>>(v.head, n_cand, p.maxc);
+    CHIMERA_CUDA(cudaGetLastError());
+    return CHIMERA_OK;
+}
+int launch_visit_sum(const Index &ix, const Params &p, const VisitLists &v, bool floats, const int32_t *n_cand,
+                     int32_t *fprime, cudaStream_t st)
+{
+    const dim3 grid((unsigned)((16LL * ix.sm_count + p.B - 1) / p.B), (unsigned)p.B);
+    if (floats) visit_sum_kernel<true><<<grid, 256, 0, st>>>(v.head, v.node, v.cap, n_cand, p.maxc, fprime);
+    else visit_sum_kernel<false><<<grid, 256, 0, st>>>(v.head, v.node, v.cap, n_cand, p.maxc, fprime);
+    CHIMERA_CUDA(cudaGetLastError());
+    return CHIMERA_OK;
 }
 
 // grid (blocks, B): zero the first n_cand[b] rows of M and the first n_cand[b] partial scores.
@@ -71,42 +102,40 @@ partial_clear_kernel(int32_t *__restrict__ M, int32_t *__restrict__ fprime, cons
     for (int64_t e = tid; e < n_cand[b]; e += stride) fprime[(int64_t)b * maxc + e] = 0;
 }
 
-// grid (nq * P, B): one block per (query token, probed list).
-template <int NBITS, bool HASH>
+// grid (nq * splits, B): a block takes the lists p, p + splits, ... of a query token (splits = nprobe when few queries are
+// served, so that a block is one list; 1 in a large batch, where preparing the query token once per list costs more).
+template <int NBITS, bool LISTS>
 __global__ void __launch_bounds__(PS_THREADS)
 partial_score_kernel(const float *__restrict__ queries, const int32_t *__restrict__ table, int64_t K, int nq, int D,
                      int CW, int P, float delta, float kappa, const int32_t *__restrict__ probes,
                      const int64_t *__restrict__ tok_off, const int32_t *__restrict__ tok_id,
                      const int32_t *__restrict__ tok_doc, const uint32_t *__restrict__ codes,
-                     const uint32_t *__restrict__ bitmap, const int32_t *__restrict__ word_rank, int64_t words,
-                     int64_t maxc, int32_t *__restrict__ M, int32_t *__restrict__ fprime, int64_t slots,
-                     uint32_t *__restrict__ status)
+                     const uint2 *__restrict__ ranks, int64_t words, int64_t maxc, int32_t *__restrict__ M,
+                     int32_t *__restrict__ fprime, VisitLists lists, int64_t longest, int splits)
 {
     __shared__ int32_t xq[128];
     __shared__ long long s_sq;
     const int b = blockIdx.y;
-    const int i = blockIdx.x / P;
-    const int32_t c = DBG_CID(probes[((int64_t)b * nq + i) * P + blockIdx.x % P]);
+    const int i = blockIdx.x / splits;
     const float *q = queries + ((int64_t)b * nq + i) * D;
     for (int x = threadIdx.x; x < D; x += PS_THREADS) {
         float v = fminf(fmaxf(q[x], -1.0f), 1.0f);
         xq[x] = __float2int_rn(v * 4194304.0f);
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        long long s = 0;
-        for (int x = 0; x < D; ++x) s += xq[x];
-        s_sq = s;
+    if (threadIdx.x < 32) {                            // |Xq| <= 2^22: a lane's four stay below 2^25, the sum below 2^30
+        int s = 0;
+        for (int x = threadIdx.x; x < D; x += 32) s += xq[x];
+        s = __reduce_add_sync(0xffffffffu, s);
+        if (threadIdx.x == 0) s_sq = s;
     }
     __syncthreads();
-    const int32_t s_c = table[((int64_t)b * K + c) * nq + i];
     const double d4 = __dmul_rn((double)delta, 4.0);
     const double kterm = __dmul_rn(__dmul_rn((double)kappa, 4.0), (double)s_sq);
-    const uint32_t *bm = bitmap + (int64_t)b * words;
-    const int32_t *wr = word_rank + (int64_t)b * words;
-    int32_t *Mb = M + (int64_t)b * maxc * nq;
-    unsigned long long *Hb = reinterpret_cast<unsigned long long *>(M) + (int64_t)b * slots;
-    const uint32_t slot_mask = (uint32_t)(slots - 1);
+    const uint2 *rk = ranks + (int64_t)b * words;
+    int32_t *Mb = LISTS ? nullptr : M + (int64_t)b * maxc * nq;
+    int32_t *heads = LISTS ? lists.head + (int64_t)b * maxc : nullptr;
+    unsigned long long *nodes = LISTS ? lists.node + (int64_t)b * lists.cap : nullptr;
     constexpr int DPW = 32 / NBITS;
     constexpr uint32_t MASK = (1u << NBITS) - 1u;
     // One visit: the token's packed code (16-byte loads where the code size allows) against the query token's integers.
@@ -146,95 +175,85 @@ partial_score_kernel(const float *__restrict__ queries, const int32_t *__restric
             }
         return T;
     };
-    // (the document's bitmap word and its rank come as arguments: they depend on the list entry alone, so their loads
-    // are issued with the code loads instead of after the score is known -- one memory latency less per visit)
-    auto update = [&](uint32_t d, int T, uint32_t bm_word, int32_t wr_word) {
-        const double r = __dadd_rn(__dmul_rn(d4, (double)T), kterm);
-        const long long dist = (long long)s_c + __double2ll_rn(r);
+    // (the document's bitmap word and rank come as an argument: they depend on the list entry alone, so their load is
+    // issued with the code loads instead of after the score is known -- one memory latency less per visit)
+    int32_t s_c;
+    uint32_t v0;                                       // node of the list's first entry
+    int64_t e0;
+    auto update = [&](int64_t e, uint32_t d, int T, uint2 r) {
+        const double x = __dadd_rn(__dmul_rn(d4, (double)T), kterm);
+        const long long dist = (long long)s_c + __double2ll_rn(x);
         if (dist > 0) {                                // the table starts at 0 (Algorithm 2)
-            const int64_t rank = wr_word + __popc(bm_word & ((1u << (d & 31)) - 1u));
+            const int64_t rank = (int64_t)r.y + __popc(r.x & ((1u << (d & 31)) - 1u));
             if (rank < maxc && DBG_RANK_OK(rank)) {
-                // F' = sum_i M[., i] is kept up to date with the increments: M only grows, integer adds commute
-                int32_t old = 0;
-                if (HASH) {
-                    const uint32_t key = (uint32_t)(rank * nq + i) + 1u;
-                    const unsigned long long mine = ((unsigned long long)key << 32) | (uint32_t)dist;
-                    uint32_t h = (key * 2654435761u) & slot_mask;
-                    int probes = 0;
-                    for (; probes < HASH_MAX_PROBES; ++probes, h = (h + 1u) & slot_mask) {
-                        unsigned long long cur = Hb[h];
-                        if (cur == 0ull) {
-                            cur = atomicCAS(&Hb[h], 0ull, mine);
-                            if (cur == 0ull) break;                         // new cell: the old maximum is 0
-                        }
-                        if ((uint32_t)(cur >> 32) == key) {                 // this cell's slot (its key is final)
-                            old = (int32_t)(uint32_t)atomicMax(&Hb[h], mine);
-                            break;
-                        }
-                    }
-                    if (probes == HASH_MAX_PROBES) {                        // cannot happen below half load; reported
-                        atomicOr(status, ST_OVERFLOW);
-                        old = (int32_t)dist;                                // no increment
-                    }
+                if (LISTS) {
+                    visit_push(heads + rank, nodes, v0 + (uint32_t)(e - e0), i, (uint32_t)dist);
                 } else {
-                    old = atomicMax(&Mb[rank * nq + i], (int32_t)dist);
+                    // F' = sum_i M[., i] is kept up to date with the increments: M only grows, integer adds commute
+                    const int32_t old = atomicMax(&Mb[rank * nq + i], (int32_t)dist);
+                    if ((int32_t)dist > old) atomicAdd(&fprime[(int64_t)b * maxc + rank], (int32_t)dist - old);
                 }
-                if ((int32_t)dist > old) atomicAdd(&fprime[(int64_t)b * maxc + rank], (int32_t)dist - old);
             }
         }
     };
-    // two visits per thread and iteration, their loads issued together
-    const int64_t e1 = tok_off[c + 1];
-    int64_t e = tok_off[c] + threadIdx.x;
-    for (; e + PS_THREADS < e1; e += 2 * PS_THREADS) {
-        const int64_t ta = DBG_TOK(tok_id[e]), tb2 = DBG_TOK(tok_id[e + PS_THREADS]);
-        const uint32_t da = (uint32_t)DBG_DOC(tok_doc[e]), db = (uint32_t)DBG_DOC(tok_doc[e + PS_THREADS]);
-        const uint32_t bma = __ldg(bm + (da >> 5)), bmb = __ldg(bm + (db >> 5));
-        const int32_t wra = __ldg(wr + (da >> 5)), wrb = __ldg(wr + (db >> 5));
-        const int Ta = code_dot(ta), Tb = code_dot(tb2);
-        update(da, Ta, bma, wra);
-        update(db, Tb, bmb, wrb);
-    }
-    if (e < e1) {
-        const uint32_t d = (uint32_t)DBG_DOC(tok_doc[e]);
-        const uint32_t bmd = __ldg(bm + (d >> 5));
-        const int32_t wrd = __ldg(wr + (d >> 5));
-        update(d, code_dot(DBG_TOK(tok_id[e])), bmd, wrd);
+    for (int p = blockIdx.x % splits; p < P; p += splits) {
+        const int32_t c = DBG_CID(probes[((int64_t)b * nq + i) * P + p]);
+        s_c = table[((int64_t)b * K + c) * nq + i];
+        v0 = (uint32_t)((i * P + p) * longest);
+        e0 = tok_off[c];
+        const int64_t e1 = tok_off[c + 1];
+        int64_t e = e0 + threadIdx.x;
+        // two visits per thread and iteration, their loads issued together
+        for (; e + PS_THREADS < e1; e += 2 * PS_THREADS) {
+            const int64_t ta = DBG_TOK(tok_id[e]), tb2 = DBG_TOK(tok_id[e + PS_THREADS]);
+            const uint32_t da = (uint32_t)DBG_DOC(tok_doc[e]), db = (uint32_t)DBG_DOC(tok_doc[e + PS_THREADS]);
+            const uint2 ra = __ldg(rk + (da >> 5)), rb = __ldg(rk + (db >> 5));
+            const int Ta = code_dot(ta), Tb = code_dot(tb2);
+            update(e, da, Ta, ra);
+            update(e + PS_THREADS, db, Tb, rb);
+        }
+        if (e < e1) {
+            const uint32_t d = (uint32_t)DBG_DOC(tok_doc[e]);
+            const uint2 r = __ldg(rk + (d >> 5));
+            update(e, d, code_dot(DBG_TOK(tok_id[e])), r);
+        }
     }
 }
 
 int launch_partial_scores(const Index &ix, const Params &p, const Layout &L, const float *queries,
-                          const int32_t *table, const int32_t *probes, const uint32_t *bitmap,
-                          const int32_t *word_rank, const int32_t *n_cand, int32_t *partial_m, int32_t *fprime,
-                          uint32_t *status, cudaStream_t st)
+                          const int32_t *table, const int32_t *probes, const uint2 *ranks, const int32_t *n_cand,
+                          void *partial_m, int32_t *fprime, cudaStream_t st)
 {
     const float delta = (ix.res_hi - ix.res_lo) / (float)(1 << ix.nbits);
     const float kappa = ix.res_lo + 0.5f * delta;
-    int64_t per_query = ((int64_t)ix.sm_count * 8 + p.B - 1) / p.B;
-    if (per_query < 1) per_query = 1;
-    dim3 gclr((unsigned)per_query, (unsigned)p.B);
-    const bool hashed = L.hash_slots > 0;
-    if (hashed)
-        hash_clear_kernel<<<gclr, 256, 0, st>>>(reinterpret_cast<unsigned long long *>(partial_m), L.hash_slots, fprime,
-                                                n_cand, p.maxc);
-    else
-        partial_clear_kernel<<<gclr, 256, 0, st>>>(partial_m, fprime, n_cand, p.maxc, p.nq);
-    CHIMERA_CUDA(cudaGetLastError());
-    dim3 grid((unsigned)(p.nq * p.P), (unsigned)p.B);
-    const uint32_t *codes = reinterpret_cast<const uint32_t *>(ix.codes);
-#define PS_LAUNCH(NB, HS)                                                                                              \
-    partial_score_kernel<NB, HS><<<grid, PS_THREADS, 0, st>>>(queries, table, ix.K, p.nq, ix.D, ix.CB / 4, p.P, delta, \
-                                                              kappa, probes, ix.tok_off, ix.tok_id, ix.tok_doc, codes, \
-                                                              bitmap, word_rank, L.words, p.maxc, partial_m, fprime,   \
-                                                              L.hash_slots, status)
-    if (ix.nbits == 2) {
-        if (hashed) PS_LAUNCH(2, true); else PS_LAUNCH(2, false);
+    const bool use_lists = L.visit_nodes > 0;
+    const VisitLists lists = visit_lists(p, L, partial_m);
+    int32_t *M = (int32_t *)partial_m;
+    int rc;
+    if (use_lists) {
+        if ((rc = launch_visit_clear(ix, p, lists, n_cand, st))) return rc;
     } else {
-        if (hashed) PS_LAUNCH(1, true); else PS_LAUNCH(1, false);
+        int64_t per_query = ((int64_t)ix.sm_count * 8 + p.B - 1) / p.B;
+        partial_clear_kernel<<<dim3((unsigned)per_query, (unsigned)p.B), 256, 0, st>>>(M, fprime, n_cand, p.maxc, p.nq);
+        CHIMERA_CUDA(cudaGetLastError());
+    }
+    const int splits = refine_splits(ix, p);
+    dim3 grid((unsigned)(p.nq * splits), (unsigned)p.B);
+    const uint32_t *codes = reinterpret_cast<const uint32_t *>(ix.codes);
+#define PS_LAUNCH(NB, LS)                                                                                              \
+    partial_score_kernel<NB, LS><<<grid, PS_THREADS, 0, st>>>(queries, table, ix.K, p.nq, ix.D, ix.CB / 4, p.P, delta, \
+                                                              kappa, probes, ix.tok_off, ix.tok_id, ix.tok_doc, codes, \
+                                                              ranks, L.words, p.maxc, M, fprime, lists, ix.max_tok_list, \
+                                                              splits)
+    if (ix.nbits == 2) {
+        if (use_lists) PS_LAUNCH(2, true); else PS_LAUNCH(2, false);
+    } else {
+        if (use_lists) PS_LAUNCH(1, true); else PS_LAUNCH(1, false);
     }
 #undef PS_LAUNCH
     CHIMERA_CUDA(cudaGetLastError());
-    count_launch(SLOT_CI, 2);
+    if (use_lists && (rc = launch_visit_sum(ix, p, lists, false, n_cand, fprime, st))) return rc;
+    count_launch(SLOT_CI, use_lists ? 3 : 2);
     return CHIMERA_OK;
 }
 

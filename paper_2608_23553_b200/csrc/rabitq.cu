@@ -6,11 +6,12 @@
 // over query tokens in increasing order, so every result is reproducible bit for bit.
 //
 // This file: attaching the codes to an index, the rotation kernel, and candidate refinement by partial 1-bit scores
-// (Algorithm 2; one block per (query token, posting list) as in the paper's design, atomicMax as in Algorithm 4).
+// (Algorithm 2; a block per (query token, posting list) as in the paper's design; the maxima of Algorithm 4 as visit
+// lists for batches on large corpora, g3_visits.cuh, otherwise a table of rows updated with atomicMax).
 // The complete 1-bit scores of the survivors run on the tensor cores (g4_residual_umma.cu, RQ variant).
 #include <math.h>
 
-#include "common.cuh"
+#include "g3_visits.cuh"
 
 namespace chimera {
 
@@ -74,13 +75,15 @@ rabitq_clear_kernel(int32_t *__restrict__ M, const int32_t *__restrict__ n_cand,
     }
 }
 
-// grid (nq * P, B): one block per (query token, probed list); M holds float bits (>= 0, so integer order = float order).
+// grid (nq * splits, B): lists p, p + splits, ... of a query token per block; M holds float bits (>= 0, so integer order =
+// float order).
+template <bool LISTS>
 __global__ void __launch_bounds__(RP_THREADS)
 rabitq_partial_kernel(const float *__restrict__ q_rot, int nq, int D, int P, float c, const int32_t *__restrict__ probes,
                       const int64_t *__restrict__ tok_off, const int32_t *__restrict__ tok_id,
                       const int32_t *__restrict__ tok_doc, const uint32_t *__restrict__ bits,
-                      const float *__restrict__ inv_dot, const uint32_t *__restrict__ bitmap,
-                      const int32_t *__restrict__ word_rank, int64_t words, int64_t maxc, int32_t *__restrict__ M)
+                      const float *__restrict__ inv_dot, const uint2 *__restrict__ ranks, int64_t words, int64_t maxc,
+                      int32_t *__restrict__ M, VisitLists lists, int64_t longest, int splits)
 {
     // Sec. 4.1's look-up-table form of the binary inner product: for every group of four dimensions the 16 partial
     // sums of the query token's integers are tabulated once per block (D/4 * 16 entries: cheap next to a list of a few
@@ -90,16 +93,16 @@ rabitq_partial_kernel(const float *__restrict__ q_rot, int nq, int D, int P, flo
     __shared__ int32_t lut[32 * 16];
     __shared__ int s_sq;
     const int b = blockIdx.y;
-    const int i = blockIdx.x / P;
-    const int32_t cen = DBG_CID(probes[((int64_t)b * nq + i) * P + blockIdx.x % P]);
+    const int i = blockIdx.x / splits;
     const float *q = q_rot + ((int64_t)b * nq + i) * D;
     for (int x = threadIdx.x; x < D; x += RP_THREADS)
         xq[x] = __float2int_rn(fminf(fmaxf(q[x], -1.0f), 1.0f) * 4194304.0f);
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (threadIdx.x < 32) {
         int s = 0;
-        for (int x = 0; x < D; ++x) s += xq[x];
-        s_sq = s;
+        for (int x = threadIdx.x; x < D; x += 32) s += xq[x];
+        s = __reduce_add_sync(0xffffffffu, s);
+        if (threadIdx.x == 0) s_sq = s;
     }
     for (int e = threadIdx.x; e < (D >> 2) * 16; e += RP_THREADS) {
         const int g = e >> 4, v = e & 15;
@@ -111,9 +114,10 @@ rabitq_partial_kernel(const float *__restrict__ q_rot, int nq, int D, int P, flo
     __syncthreads();
     const int sq = s_sq;
     const int CW = D >> 5;
-    const uint32_t *bm = bitmap + (int64_t)b * words;
-    const int32_t *wr = word_rank + (int64_t)b * words;
-    int32_t *Mb = M + (int64_t)b * maxc * nq;
+    const uint2 *rk = ranks + (int64_t)b * words;
+    int32_t *Mb = LISTS ? nullptr : M + (int64_t)b * maxc * nq;
+    int32_t *heads = LISTS ? lists.head + (int64_t)b * maxc : nullptr;
+    unsigned long long *nodes = LISTS ? lists.node + (int64_t)b * lists.cap : nullptr;
     auto code_dot = [&](int64_t t) -> int {
         uint32_t word[4];                              // D <= 128: at most four words
         if (CW == 4) {                                 // 16-byte rows (the attach call checks the alignment)
@@ -134,32 +138,40 @@ rabitq_partial_kernel(const float *__restrict__ q_rot, int nq, int D, int P, flo
     };
     // (the token's factor, the document's bitmap word and its rank come as arguments: they depend on the list entry
     // alone, so their loads are issued with the code loads instead of one after the other behind the score)
-    auto update = [&](uint32_t d, float factor, int T, uint32_t bm_word, int32_t wr_word) {
+    uint32_t v0;                                       // node of the list's first entry
+    int64_t e0;
+    auto update = [&](int64_t e, uint32_t d, float factor, int T, uint2 r) {
         const float est = __fmul_rn(factor, __fmul_rn(c, (float)(2 * T - sq)));
         if (est > 0.0f) {                              // the table starts at 0 (Algorithm 2)
-            const int64_t rank = wr_word + __popc(bm_word & ((1u << (d & 31)) - 1u));
-            if (rank < maxc && DBG_RANK_OK(rank)) atomicMax(&Mb[rank * nq + i], __float_as_int(est));
+            const int64_t rank = (int64_t)r.y + __popc(r.x & ((1u << (d & 31)) - 1u));
+            if (rank < maxc && DBG_RANK_OK(rank)) {
+                if (LISTS) visit_push(heads + rank, nodes, v0 + (uint32_t)(e - e0), i, __float_as_uint(est));
+                else atomicMax(&Mb[rank * nq + i], __float_as_int(est));
+            }
         }
     };
-    const int64_t e1 = tok_off[cen + 1];
-    int64_t e = tok_off[cen] + threadIdx.x;
-    for (; e + RP_THREADS < e1; e += 2 * RP_THREADS) {         // two visits per iteration, their loads issued together
-        const int64_t ta = DBG_TOK(tok_id[e]), tb = DBG_TOK(tok_id[e + RP_THREADS]);
-        const uint32_t da = (uint32_t)DBG_DOC(tok_doc[e]), db = (uint32_t)DBG_DOC(tok_doc[e + RP_THREADS]);
-        const float fa = __ldg(inv_dot + ta), fb = __ldg(inv_dot + tb);
-        const uint32_t bma = __ldg(bm + (da >> 5)), bmb = __ldg(bm + (db >> 5));
-        const int32_t wra = __ldg(wr + (da >> 5)), wrb = __ldg(wr + (db >> 5));
-        const int Ta = code_dot(ta), Tb = code_dot(tb);
-        update(da, fa, Ta, bma, wra);
-        update(db, fb, Tb, bmb, wrb);
-    }
-    if (e < e1) {
-        const int64_t t = DBG_TOK(tok_id[e]);
-        const uint32_t d = (uint32_t)DBG_DOC(tok_doc[e]);
-        const float f = __ldg(inv_dot + t);
-        const uint32_t bmd = __ldg(bm + (d >> 5));
-        const int32_t wrd = __ldg(wr + (d >> 5));
-        update(d, f, code_dot(t), bmd, wrd);
+    for (int p = blockIdx.x % splits; p < P; p += splits) {
+        const int32_t cen = DBG_CID(probes[((int64_t)b * nq + i) * P + p]);
+        v0 = (uint32_t)((i * P + p) * longest);
+        e0 = tok_off[cen];
+        const int64_t e1 = tok_off[cen + 1];
+        int64_t e = e0 + threadIdx.x;
+        for (; e + RP_THREADS < e1; e += 2 * RP_THREADS) {         // two visits per iteration, their loads issued together
+            const int64_t ta = DBG_TOK(tok_id[e]), tb = DBG_TOK(tok_id[e + RP_THREADS]);
+            const uint32_t da = (uint32_t)DBG_DOC(tok_doc[e]), db = (uint32_t)DBG_DOC(tok_doc[e + RP_THREADS]);
+            const float fa = __ldg(inv_dot + ta), fb = __ldg(inv_dot + tb);
+            const uint2 ra = __ldg(rk + (da >> 5)), rb = __ldg(rk + (db >> 5));
+            const int Ta = code_dot(ta), Tb = code_dot(tb);
+            update(e, da, fa, Ta, ra);
+            update(e + RP_THREADS, db, fb, Tb, rb);
+        }
+        if (e < e1) {
+            const int64_t t = DBG_TOK(tok_id[e]);
+            const uint32_t d = (uint32_t)DBG_DOC(tok_doc[e]);
+            const float f = __ldg(inv_dot + t);
+            const uint2 r = __ldg(rk + (d >> 5));
+            update(e, d, f, code_dot(t), r);
+        }
     }
 }
 
@@ -190,21 +202,39 @@ rabitq_sum_kernel(const int32_t *__restrict__ M, const int32_t *__restrict__ n_c
 }
 
 int launch_rabitq_partial(const Index &ix, const Params &p, const Layout &L, const float *q_rot,
-                          const int32_t *probes, const uint32_t *bitmap, const int32_t *word_rank,
-                          const int32_t *n_cand, int32_t *partial_m, int32_t *fprime_bits, cudaStream_t st)
+                          const int32_t *probes, const uint2 *ranks, const int32_t *n_cand, void *partial_m,
+                          int32_t *fprime_bits, cudaStream_t st)
 {
-    int64_t per_query = ((int64_t)ix.sm_count * 8 + p.B - 1) / p.B;
-    if (per_query < 1) per_query = 1;
-    dim3 gclr((unsigned)per_query, (unsigned)p.B);
-    rabitq_clear_kernel<<<gclr, 256, 0, st>>>(partial_m, n_cand, p.maxc, p.nq);
-    CHIMERA_CUDA(cudaGetLastError());
+    const bool use_lists = L.visit_nodes > 0;
+    const VisitLists lists = visit_lists(p, L, partial_m);
+    int32_t *M = (int32_t *)partial_m;
+    const dim3 gclr((unsigned)(((int64_t)ix.sm_count * 8 + p.B - 1) / p.B), (unsigned)p.B);
+    int rc;
+    if (use_lists) {
+        if ((rc = launch_visit_clear(ix, p, lists, n_cand, st))) return rc;
+    } else {
+        rabitq_clear_kernel<<<gclr, 256, 0, st>>>(M, n_cand, p.maxc, p.nq);
+        CHIMERA_CUDA(cudaGetLastError());
+    }
     const float c = (float)(1.0 / (sqrt((double)ix.D) * 4194304.0));
-    rabitq_partial_kernel<<<dim3((unsigned)(p.nq * p.P), (unsigned)p.B), RP_THREADS, 0, st>>>(
-        q_rot, p.nq, ix.D, p.P, c, probes, ix.tok_off, ix.tok_id, ix.tok_doc,
-        reinterpret_cast<const uint32_t *>(ix.rq_bits), ix.rq_inv, bitmap, word_rank, L.words, p.maxc, partial_m);
+    const int splits = refine_splits(ix, p);
+    const dim3 grid((unsigned)(p.nq * splits), (unsigned)p.B);
+    const uint32_t *bits = reinterpret_cast<const uint32_t *>(ix.rq_bits);
+    if (use_lists)
+        rabitq_partial_kernel<true><<<grid, RP_THREADS, 0, st>>>(q_rot, p.nq, ix.D, p.P, c, probes, ix.tok_off, ix.tok_id,
+                                                                 ix.tok_doc, bits, ix.rq_inv, ranks, L.words, p.maxc, M,
+                                                                 lists, ix.max_tok_list, splits);
+    else
+        rabitq_partial_kernel<false><<<grid, RP_THREADS, 0, st>>>(q_rot, p.nq, ix.D, p.P, c, probes, ix.tok_off, ix.tok_id,
+                                                                  ix.tok_doc, bits, ix.rq_inv, ranks, L.words, p.maxc, M,
+                                                                  lists, ix.max_tok_list, splits);
     CHIMERA_CUDA(cudaGetLastError());
-    rabitq_sum_kernel<<<gclr, 256, 0, st>>>(partial_m, n_cand, p.maxc, p.nq, fprime_bits);
-    CHIMERA_CUDA(cudaGetLastError());
+    if (use_lists) {
+        if ((rc = launch_visit_sum(ix, p, lists, true, n_cand, fprime_bits, st))) return rc;
+    } else {
+        rabitq_sum_kernel<<<gclr, 256, 0, st>>>(M, n_cand, p.maxc, p.nq, fprime_bits);
+        CHIMERA_CUDA(cudaGetLastError());
+    }
     count_launch(SLOT_CI, 3);
     return CHIMERA_OK;
 }
