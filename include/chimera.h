@@ -166,8 +166,9 @@ int chimera_run_stages(const chimera_index *index, int32_t first_stage, int32_t 
 
 /* Build the token-level posting lists (per centroid: its tokens and their documents; Sec. 3.2 step 1 keeps posting
  * lists at token level) that chimera_search_partial needs.  Allocates 8 bytes per token plus 8 per centroid inside the
- * index (cudaMalloc), synchronises the stream.  Idempotent.  Workspace sizes grow afterwards (a score table of
- * n_queries x max_candidates x q_len int32), so query chimera_workspace_bytes again.
+ * index (cudaMalloc) and, where that takes no more than a quarter of the free device memory, a copy of the codes in the
+ * order of the lists; synchronises the stream.  Idempotent.  Workspace sizes grow afterwards (visit lists, or a score
+ * table of n_queries x max_candidates x q_len int32), so query chimera_workspace_bytes again.
  * Errors: INVALID_ARG, UNSUPPORTED (more than 2^31 - 1 tokens), CUDA_ERROR (nothing stays allocated). */
 int chimera_index_enable_partial(chimera_index *index, void *stream);
 
@@ -192,7 +193,8 @@ int chimera_search_partial(const chimera_index *index, const float *queries, int
  *   rotation  device, [dim, dim] float32 row-major orthonormal matrix P.  Copied (transposed).
  *   bits      device, [T, dim/8] uint8, document-major: bit t of byte g is dimension 8g+t.  REFERENCED, not copied.
  *   inv_dot   device, [T] float32, 1 / <o_p, o_p-bar> = sqrt(dim) / sum_x |o_p[x]|.  REFERENCED, not copied.
- * Also builds the token-level posting lists (as chimera_index_enable_partial).  Synchronises the stream.
+ * Also builds the token-level posting lists (as chimera_index_enable_partial) and, where that takes no more than a quarter
+ * of the free device memory, copies of bits and inv_dot in their order.  Synchronises the stream.
  * Errors: INVALID_ARG, CUDA_ERROR. */
 int chimera_index_attach_rabitq(chimera_index *index, const float *rotation, const uint8_t *bits,
                                 const float *inv_dot, void *stream);

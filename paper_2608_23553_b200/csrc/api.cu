@@ -353,14 +353,14 @@ static int run(const Index &ix, const Params &p, int first, int last, const floa
             if ((rc = launch_digits(q_rot, (int64_t)p.B * p.nq, ix.D, 1, nullptr, qdig_rot, p.nq, status, st))) return rc;
             count_launch(SLOT_G1);
             prof_mark(SLOT_G1, st);
-            if ((rc = launch_rabitq_partial(ix, p, L, q_rot, probes, ranks, n_cand, partial_m, ci, st)))
+            if ((rc = launch_rabitq_partial(ix, p, L, qdig_rot, probes, ranks, n_cand, partial_m, ci, st)))
                 return rc;
             prof_mark(SLOT_CI, st);
             if ((rc = launch_select(ix, p, cand, n_cand, ci, pruned, n_pruned, pruned_ci, sel_scratch, st))) return rc;
             prof_mark(SLOT_SELECT, st);
         } else if (partial) {
             // the paper's candidate refinement: partial scores from the retrieved tokens only, then the same selection
-            if ((rc = launch_partial_scores(ix, p, L, queries, table, probes, ranks, n_cand, partial_m, ci, st)))
+            if ((rc = launch_partial_scores(ix, p, L, qdig, table, probes, ranks, n_cand, partial_m, ci, st)))
                 return rc;
             prof_mark(SLOT_CI, st);
             if ((rc = launch_select(ix, p, cand, n_cand, ci, pruned, n_pruned, pruned_ci, sel_scratch, st))) return rc;
@@ -531,7 +531,10 @@ int chimera_index_enable_partial(chimera_index *index, void *stream)
 {
     Index *ix = reinterpret_cast<Index *>(index);
     if (!ix) return fail(CHIMERA_INVALID_ARG, "index is NULL");
-    return build_token_lists(*ix, (cudaStream_t)stream);
+    int rc = build_token_lists(*ix, (cudaStream_t)stream);
+    if (rc || (rc = copy_in_list_order(*ix, ix->codes, ix->CB / 4, (void **)&ix->list_codes, (cudaStream_t)stream))) return rc;
+    CHIMERA_CUDA(cudaStreamSynchronize((cudaStream_t)stream));
+    return CHIMERA_OK;
 }
 
 int chimera_search_partial(const chimera_index *index, const float *queries, int32_t n_queries, int32_t q_len,
@@ -559,6 +562,21 @@ int chimera_index_attach_rabitq(chimera_index *index, const float *rotation, con
     if (rc) return rc;
     ix->rq_bits = bits;
     ix->rq_inv = inv_dot;
+    // (codes attached before, if any, are replaced)
+    cudaFree(ix->list_bits);
+    cudaFree(ix->list_inv);
+    ix->list_bits = nullptr;
+    ix->list_inv = nullptr;
+    if ((rc = copy_in_list_order(*ix, bits, ix->D / 32, (void **)&ix->list_bits, (cudaStream_t)stream))) return rc;
+    if ((rc = copy_in_list_order(*ix, inv_dot, 1, (void **)&ix->list_inv, (cudaStream_t)stream))) return rc;
+    if (!ix->list_bits || !ix->list_inv) {                   // both or neither
+        CHIMERA_CUDA(cudaStreamSynchronize((cudaStream_t)stream));
+        cudaFree(ix->list_bits);
+        cudaFree(ix->list_inv);
+        ix->list_bits = nullptr;
+        ix->list_inv = nullptr;
+    }
+    CHIMERA_CUDA(cudaStreamSynchronize((cudaStream_t)stream));
     return CHIMERA_OK;
 }
 
@@ -719,6 +737,9 @@ int chimera_destroy_index(chimera_index *index)
     cudaFree(ix->tok_off);
     cudaFree(ix->tok_id);
     cudaFree(ix->tok_doc);
+    cudaFree(ix->list_codes);
+    cudaFree(ix->list_bits);
+    cudaFree(ix->list_inv);
     cudaFree(ix->doc_off);
     cudaFree(ix->cdig);
     cudaFree(ix->ivf_off);

@@ -30,6 +30,9 @@ struct Index {
     int32_t *tok_id = nullptr;        // [T]        owned: token ids per centroid, unordered
     int32_t *tok_doc = nullptr;       // [T]        owned: document of each listed token
     int64_t max_tok_list = 0;         // longest token list
+    uint8_t *list_codes = nullptr;    // [T, CB]    owned, optional: the codes in list order (see copy_in_list_order)
+    uint8_t *list_bits = nullptr;     // [T, D/8]   owned, optional: the RaBitQ codes in list order
+    float *list_inv = nullptr;        // [T]        owned, optional: their factors
     // RaBitQ 1-bit codes (only after chimera_index_attach_rabitq)
     const uint8_t *rq_bits = nullptr; // [T, D/8]   borrowed: sign bits of the rotated tokens
     const float *rq_inv = nullptr;    // [T]        borrowed: 1 / <o_p, o_p-bar>
@@ -184,9 +187,13 @@ int launch_gather(const Index &ix, const Params &p, const Layout &L, const int32
                   cudaStream_t st);
 // Token-level posting lists for the partial-score refinement (allocates; index_build.cu).
 int build_token_lists(Index &ix, cudaStream_t st);
+// A copy of src ([T][words] 32-bit words, document-major) in the order of the token lists, so that a list's codes are one
+// contiguous run instead of a scattered sector each; *out stays NULL when it would take more than a quarter of the free
+// memory (the kernels then gather through the token ids).
+int copy_in_list_order(const Index &ix, const void *src, int words, void **out, cudaStream_t st);
 // Candidate refinement with partial scores (Algorithm 2): fprime[b][j] for every candidate.
 int64_t visit_list_nodes(const Index &ix, const Params &p);
-int launch_partial_scores(const Index &ix, const Params &p, const Layout &L, const float *queries,
+int launch_partial_scores(const Index &ix, const Params &p, const Layout &L, const int8_t *qdig,
                           const int32_t *table, const int32_t *probes, const uint2 *ranks, const int32_t *n_cand,
                           void *partial_m, int32_t *fprime, cudaStream_t st);
 int launch_filter_contenders(const Index &ix, const Params &p, const Layout &L, const int32_t *kept, const int2 *kept_rng,
@@ -259,7 +266,7 @@ int launch_graph_probes(const Index &ix, const float *queries, int64_t n_tokens,
 // rabitq.cu
 int attach_rabitq(Index &ix, const float *rotation, cudaStream_t st);
 int launch_rotate(const Index &ix, const Params &p, const float *queries, float *q_rot, cudaStream_t st);
-int launch_rabitq_partial(const Index &ix, const Params &p, const Layout &L, const float *q_rot,
+int launch_rabitq_partial(const Index &ix, const Params &p, const Layout &L, const int8_t *qdig_rot,
                           const int32_t *probes, const uint2 *ranks, const int32_t *n_cand, void *partial_m,
                           int32_t *fprime_bits, cudaStream_t st);
 int launch_topk(const Index &ix, const Params &p, const int32_t *pruned, const float *score4, int32_t *out_ids,

@@ -104,82 +104,32 @@ partial_clear_kernel(int32_t *__restrict__ M, int32_t *__restrict__ fprime, cons
 
 // grid (nq * splits, B): a block takes the lists p, p + splits, ... of a query token (splits = nprobe when few queries are
 // served, so that a block is one list; 1 in a large batch, where preparing the query token once per list costs more).
+// codes: in list order (tok_id NULL), or the index's document-major codes.
 template <int NBITS, bool LISTS>
 __global__ void __launch_bounds__(PS_THREADS)
-partial_score_kernel(const float *__restrict__ queries, const int32_t *__restrict__ table, int64_t K, int nq, int D,
-                     int CW, int P, float delta, float kappa, const int32_t *__restrict__ probes,
+partial_score_kernel(const int8_t *__restrict__ qdig, const int32_t *__restrict__ table, int64_t K, int nq, int B, int CW,
+                     int P, float delta, float kappa, const int32_t *__restrict__ probes,
                      const int64_t *__restrict__ tok_off, const int32_t *__restrict__ tok_id,
                      const int32_t *__restrict__ tok_doc, const uint32_t *__restrict__ codes,
                      const uint2 *__restrict__ ranks, int64_t words, int64_t maxc, int32_t *__restrict__ M,
                      int32_t *__restrict__ fprime, VisitLists lists, int64_t longest, int splits)
 {
-    __shared__ int32_t xq[128];
-    __shared__ long long s_sq;
+    __shared__ __align__(16) QueryDigits dig;
     const int b = blockIdx.y;
     const int i = blockIdx.x / splits;
-    const float *q = queries + ((int64_t)b * nq + i) * D;
-    for (int x = threadIdx.x; x < D; x += PS_THREADS) {
-        float v = fminf(fmaxf(q[x], -1.0f), 1.0f);
-        xq[x] = __float2int_rn(v * 4194304.0f);
-    }
-    __syncthreads();
-    if (threadIdx.x < 32) {                            // |Xq| <= 2^22: a lane's four stay below 2^25, the sum below 2^30
-        int s = 0;
-        for (int x = threadIdx.x; x < D; x += 32) s += xq[x];
-        s = __reduce_add_sync(0xffffffffu, s);
-        if (threadIdx.x == 0) s_sq = s;
-    }
+    load_query_digits(dig, qdig, (int64_t)B * nq, (int64_t)b * nq + i);
     __syncthreads();
     const double d4 = __dmul_rn((double)delta, 4.0);
-    const double kterm = __dmul_rn(__dmul_rn((double)kappa, 4.0), (double)s_sq);
+    const double kterm = __dmul_rn(__dmul_rn((double)kappa, 4.0), (double)query_sum(dig));
     const uint2 *rk = ranks + (int64_t)b * words;
     int32_t *Mb = LISTS ? nullptr : M + (int64_t)b * maxc * nq;
     int32_t *heads = LISTS ? lists.head + (int64_t)b * maxc : nullptr;
     unsigned long long *nodes = LISTS ? lists.node + (int64_t)b * lists.cap : nullptr;
-    constexpr int DPW = 32 / NBITS;
-    constexpr uint32_t MASK = (1u << NBITS) - 1u;
-    // One visit: the token's packed code (16-byte loads where the code size allows) against the query token's integers.
-    auto code_dot = [&](int64_t t) -> int {
-        const uint32_t *cw = codes + t * CW;
-        uint32_t word[8];                              // at most 32 code bytes per token
-        if (NBITS == 2 && CW == 8) {                   // 32-byte codes (32-byte aligned): one load
-            asm volatile("ld.global.nc.v8.u32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                         : "=r"(word[0]), "=r"(word[1]), "=r"(word[2]), "=r"(word[3]), "=r"(word[4]), "=r"(word[5]),
-                           "=r"(word[6]), "=r"(word[7])
-                         : "l"(cw));
-        } else if ((CW & 3) == 0) {
-#pragma unroll
-            for (int w = 0; w < 8; w += 4)
-                if (w < CW) {
-                    const uint4 v = __ldg(reinterpret_cast<const uint4 *>(cw + w));
-                    word[w] = v.x; word[w + 1] = v.y; word[w + 2] = v.z; word[w + 3] = v.w;
-                }
-        } else if ((CW & 1) == 0) {
-#pragma unroll
-            for (int w = 0; w < 8; w += 2)
-                if (w < CW) {
-                    const uint2 v = __ldg(reinterpret_cast<const uint2 *>(cw + w));
-                    word[w] = v.x; word[w + 1] = v.y;
-                }
-        } else {
-#pragma unroll
-            for (int w = 0; w < 8; ++w)
-                if (w < CW) word[w] = __ldg(cw + w);
-        }
-        int T = 0;                                     // |T| <= 3 * 2^22 * |q|_1 < 2^31 for unit-norm queries
-#pragma unroll
-        for (int w = 0; w < 8; ++w)
-            if (w < CW) {
-#pragma unroll
-                for (int s = 0; s < DPW; ++s) T += xq[w * DPW + s] * (int)((word[w] >> (s * NBITS)) & MASK);
-            }
-        return T;
-    };
-    // (the document's bitmap word and rank come as an argument: they depend on the list entry alone, so their load is
-    // issued with the code loads instead of after the score is known -- one memory latency less per visit)
     int32_t s_c;
     uint32_t v0;                                       // node of the list's first entry
     int64_t e0;
+    // (the document's bitmap word and rank come as an argument: they depend on the list entry alone, so their load is
+    // issued with the code loads instead of after the score is known -- one memory latency less per visit)
     auto update = [&](int64_t e, uint32_t d, int T, uint2 r) {
         const double x = __dadd_rn(__dmul_rn(d4, (double)T), kterm);
         const long long dist = (long long)s_c + __double2ll_rn(x);
@@ -202,25 +152,26 @@ partial_score_kernel(const float *__restrict__ queries, const int32_t *__restric
         v0 = (uint32_t)((i * P + p) * longest);
         e0 = tok_off[c];
         const int64_t e1 = tok_off[c + 1];
-        int64_t e = e0 + threadIdx.x;
-        // two visits per thread and iteration, their loads issued together
-        for (; e + PS_THREADS < e1; e += 2 * PS_THREADS) {
-            const int64_t ta = DBG_TOK(tok_id[e]), tb2 = DBG_TOK(tok_id[e + PS_THREADS]);
-            const uint32_t da = (uint32_t)DBG_DOC(tok_doc[e]), db = (uint32_t)DBG_DOC(tok_doc[e + PS_THREADS]);
-            const uint2 ra = __ldg(rk + (da >> 5)), rb = __ldg(rk + (db >> 5));
-            const int Ta = code_dot(ta), Tb = code_dot(tb2);
-            update(e, da, Ta, ra);
-            update(e + PS_THREADS, db, Tb, rb);
-        }
-        if (e < e1) {
-            const uint32_t d = (uint32_t)DBG_DOC(tok_doc[e]);
-            const uint2 r = __ldg(rk + (d >> 5));
-            update(e, d, code_dot(DBG_TOK(tok_id[e])), r);
+        // two visits per thread and iteration, their loads issued together (the second one past the end repeats the first)
+        for (int64_t e = e0 + threadIdx.x; e < e1; e += 2 * PS_THREADS) {
+            const int64_t at[2] = {e, e + PS_THREADS < e1 ? e + PS_THREADS : e};
+            uint32_t d[2], w[2][CODE_WORDS<NBITS>];
+            uint2 r[2];
+#pragma unroll
+            for (int n = 0; n < 2; ++n) {
+                load_code<NBITS>(w[n], codes + DBG_TOK(tok_id ? (int64_t)tok_id[at[n]] : at[n]) * CW, CW);
+                d[n] = (uint32_t)DBG_DOC(tok_doc[at[n]]);
+                r[n] = __ldg(rk + (d[n] >> 5));
+            }
+            int T[2];
+            code_dots<NBITS, 2>(T, w, CW, dig);
+            update(at[0], d[0], T[0], r[0]);
+            if (at[1] != e) update(at[1], d[1], T[1], r[1]);
         }
     }
 }
 
-int launch_partial_scores(const Index &ix, const Params &p, const Layout &L, const float *queries,
+int launch_partial_scores(const Index &ix, const Params &p, const Layout &L, const int8_t *qdig,
                           const int32_t *table, const int32_t *probes, const uint2 *ranks, const int32_t *n_cand,
                           void *partial_m, int32_t *fprime, cudaStream_t st)
 {
@@ -239,10 +190,11 @@ int launch_partial_scores(const Index &ix, const Params &p, const Layout &L, con
     }
     const int splits = refine_splits(ix, p);
     dim3 grid((unsigned)(p.nq * splits), (unsigned)p.B);
-    const uint32_t *codes = reinterpret_cast<const uint32_t *>(ix.codes);
+    const uint32_t *codes = reinterpret_cast<const uint32_t *>(ix.list_codes ? ix.list_codes : ix.codes);
+    const int32_t *ids = ix.list_codes ? nullptr : ix.tok_id;
 #define PS_LAUNCH(NB, LS)                                                                                              \
-    partial_score_kernel<NB, LS><<<grid, PS_THREADS, 0, st>>>(queries, table, ix.K, p.nq, ix.D, ix.CB / 4, p.P, delta, \
-                                                              kappa, probes, ix.tok_off, ix.tok_id, ix.tok_doc, codes, \
+    partial_score_kernel<NB, LS><<<grid, PS_THREADS, 0, st>>>(qdig, table, ix.K, p.nq, p.B, ix.CB / 4, p.P, delta, \
+                                                              kappa, probes, ix.tok_off, ids, ix.tok_doc, codes, \
                                                               ranks, L.words, p.maxc, M, fprime, lists, ix.max_tok_list, \
                                                               splits)
     if (ix.nbits == 2) {

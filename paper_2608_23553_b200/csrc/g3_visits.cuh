@@ -34,6 +34,91 @@ __device__ __forceinline__ void visit_push(int32_t *head /* of the candidate */,
     nodes[v] = (unsigned long long)score << 32 | next << VISIT_I_BITS | (uint32_t)i;
 }
 
+// ---- products of packed codes with a query token --------------------------------------------------------------------------
+// T = sum_x Xq[x] u[x] from the token's three digit planes (balanced base-256 digits, digit_dim() order: a shift and a mask
+// give the code values that one word of digits multiplies) with byte dot products: 4.75 instructions per four dimensions
+// instead of twelve for value-by-value multiplication.
+struct QueryDigits { int32_t plane[3][32]; };            // in shared memory, 16-byte aligned
+
+// rows of a digit plane array [3][n_rows][128]; whole block (128 threads or more), followed by a barrier of the caller's.
+__device__ __forceinline__ void load_query_digits(QueryDigits &s, const int8_t *dig, int64_t n_rows, int64_t row)
+{
+    const int t = threadIdx.x;
+    if (t < 96) s.plane[t >> 5][t & 31] = reinterpret_cast<const int32_t *>(dig + ((t >> 5) * n_rows + row) * 128)[t & 31];
+}
+// sum_x Xq[x] (whole warp, after the barrier).
+__device__ __forceinline__ int query_sum(const QueryDigits &s)
+{
+    const int lane = threadIdx.x & 31, ones = 0x01010101;
+    return __reduce_add_sync(0xffffffffu, __dp4a(s.plane[0][lane], ones, 0) + 256 * __dp4a(s.plane[1][lane], ones, 0) +
+                                              65536 * __dp4a(s.plane[2][lane], ones, 0));
+}
+template <int NBITS> constexpr int CODE_WORDS = NBITS == 2 ? 8 : 4;      // 128 dimensions
+// A token's CW code words (rows are as aligned as their size allows).
+template <int NBITS>
+__device__ __forceinline__ void load_code(uint32_t (&w)[CODE_WORDS<NBITS>], const uint32_t *src, int CW)
+{
+    constexpr int MAX = CODE_WORDS<NBITS>;
+    if (NBITS == 2 && CW == 8) {                         // 32-byte codes (32-byte aligned): one load
+        asm volatile("ld.global.nc.v8.u32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                     : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[MAX - 4]), "=r"(w[MAX - 3]), "=r"(w[MAX - 2]),
+                       "=r"(w[MAX - 1])
+                     : "l"(src));
+    } else if ((CW & 3) == 0) {
+#pragma unroll
+        for (int k = 0; k < MAX; k += 4)
+            if (k < CW) {
+                const uint4 v = __ldg(reinterpret_cast<const uint4 *>(src + k));
+                w[k] = v.x; w[k + 1] = v.y; w[k + 2] = v.z; w[k + 3] = v.w;
+            }
+    } else if ((CW & 1) == 0) {
+#pragma unroll
+        for (int k = 0; k < MAX; k += 2)
+            if (k < CW) {
+                const uint2 v = __ldg(reinterpret_cast<const uint2 *>(src + k));
+                w[k] = v.x; w[k + 1] = v.y;
+            }
+    } else {
+#pragma unroll
+        for (int k = 0; k < MAX; ++k)
+            if (k < CW) w[k] = __ldg(src + k);
+    }
+}
+// T of N tokens at once (they share the reads of the digits).  |T| <= 3 * 2^22 * |q|_1 < 2^31 for unit-norm queries.
+template <int NBITS, int N>
+__device__ __forceinline__ void code_dots(int (&T)[N], const uint32_t (&w)[N][CODE_WORDS<NBITS>], int CW, const QueryDigits &s)
+{
+    constexpr int PER = 4 * NBITS == 8 ? 4 : 8;          // words of digits per code word
+    constexpr uint32_t MASK = NBITS == 2 ? 0x03030303u : 0x01010101u;
+    int acc[N][3] = {};
+#pragma unroll
+    for (int k = 0; k < CODE_WORDS<NBITS>; ++k) {
+        if (k < CW) {
+#pragma unroll
+            for (int h = 0; h < PER; h += 4) {
+                int4 d[3];
+#pragma unroll
+                for (int p = 0; p < 3; ++p) d[p] = *reinterpret_cast<const int4 *>(&s.plane[p][PER * k + h]);
+#pragma unroll
+                for (int n = 0; n < N; ++n) {
+                    const uint32_t word = w[n][k] >> (NBITS * h);
+                    const int u[4] = {(int)(word & MASK), (int)(word >> NBITS & MASK), (int)(word >> 2 * NBITS & MASK),
+                                      (int)(word >> 3 * NBITS & MASK)};
+#pragma unroll
+                    for (int p = 0; p < 3; ++p) {
+                        acc[n][p] = __dp4a(u[0], d[p].x, acc[n][p]);
+                        acc[n][p] = __dp4a(u[1], d[p].y, acc[n][p]);
+                        acc[n][p] = __dp4a(u[2], d[p].z, acc[n][p]);
+                        acc[n][p] = __dp4a(u[3], d[p].w, acc[n][p]);
+                    }
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int n = 0; n < N; ++n) T[n] = acc[n][0] + 256 * acc[n][1] + 65536 * acc[n][2];
+}
+
 // Largest score per query token, summed in increasing query token.  FLOAT: the scores are float bits > 0 (whose order is
 // that of the integers) and the sum is a chain of fp32 additions from 0.
 template <bool FLOAT>

@@ -292,6 +292,35 @@ int build_token_lists(Index &ix, cudaStream_t st)
     return CHIMERA_OK;
 }
 
+// dst[e] = src[tok_id[e]], rows of `words` 32-bit words: consecutive threads write consecutive words.
+__global__ void __launch_bounds__(256)
+list_order_kernel(const uint32_t *__restrict__ src, const int32_t *__restrict__ tok_id, int64_t T, int words,
+                  uint32_t *__restrict__ dst)
+{
+    const int64_t n = T * words, stride = (int64_t)gridDim.x * 256;
+    for (int64_t k = (int64_t)blockIdx.x * 256 + threadIdx.x; k < n; k += stride) {
+        const int64_t e = k / words;
+        dst[k] = __ldg(src + (int64_t)tok_id[e] * words + (k - e * words));
+    }
+}
+
+int copy_in_list_order(const Index &ix, const void *src, int words, void **out, cudaStream_t st)
+{
+    const size_t bytes = (size_t)ix.T * words * 4;
+    size_t avail = 0, all = 0;
+    CHIMERA_CUDA(cudaMemGetInfo(&avail, &all));
+    if (*out != nullptr || bytes > avail / 4) return CHIMERA_OK;
+    if (cudaMalloc(out, bytes) != cudaSuccess) {             // (an option: without it the searches gather)
+        cudaGetLastError();
+        *out = nullptr;
+        return CHIMERA_OK;
+    }
+    list_order_kernel<<<(unsigned)(16 * ix.sm_count), 256, 0, st>>>(reinterpret_cast<const uint32_t *>(src), ix.tok_id, ix.T,
+                                                                    words, reinterpret_cast<uint32_t *>(*out));
+    CHIMERA_CUDA(cudaGetLastError());
+    return CHIMERA_OK;
+}
+
 // ------------------------------------------------------------------------------------------------ driver ---------
 int build_index_device(Index &ix, const float *centroids, const int32_t *doclens, cudaStream_t st)
 {

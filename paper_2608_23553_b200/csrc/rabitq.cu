@@ -76,70 +76,30 @@ rabitq_clear_kernel(int32_t *__restrict__ M, const int32_t *__restrict__ n_cand,
 }
 
 // grid (nq * splits, B): lists p, p + splits, ... of a query token per block; M holds float bits (>= 0, so integer order =
-// float order).
+// float order).  bits / inv_dot: in list order (tok_id NULL), or the caller's document-major arrays.
 template <bool LISTS>
 __global__ void __launch_bounds__(RP_THREADS)
-rabitq_partial_kernel(const float *__restrict__ q_rot, int nq, int D, int P, float c, const int32_t *__restrict__ probes,
-                      const int64_t *__restrict__ tok_off, const int32_t *__restrict__ tok_id,
-                      const int32_t *__restrict__ tok_doc, const uint32_t *__restrict__ bits,
-                      const float *__restrict__ inv_dot, const uint2 *__restrict__ ranks, int64_t words, int64_t maxc,
-                      int32_t *__restrict__ M, VisitLists lists, int64_t longest, int splits)
+rabitq_partial_kernel(const int8_t *__restrict__ qdig, int nq, int B, int CW, int P, float c,
+                      const int32_t *__restrict__ probes, const int64_t *__restrict__ tok_off,
+                      const int32_t *__restrict__ tok_id, const int32_t *__restrict__ tok_doc,
+                      const uint32_t *__restrict__ bits, const float *__restrict__ inv_dot,
+                      const uint2 *__restrict__ ranks, int64_t words, int64_t maxc, int32_t *__restrict__ M,
+                      VisitLists lists, int64_t longest, int splits)
 {
-    // Sec. 4.1's look-up-table form of the binary inner product: for every group of four dimensions the 16 partial
-    // sums of the query token's integers are tabulated once per block (D/4 * 16 entries: cheap next to a list of a few
-    // hundred tokens), so a token costs D/4 table reads and adds instead of a data-dependent loop over its set bits.
-    // Integer sums: the same T in any order.
-    __shared__ int32_t xq[128];
-    __shared__ int32_t lut[32 * 16];
-    __shared__ int s_sq;
+    __shared__ __align__(16) QueryDigits dig;
     const int b = blockIdx.y;
     const int i = blockIdx.x / splits;
-    const float *q = q_rot + ((int64_t)b * nq + i) * D;
-    for (int x = threadIdx.x; x < D; x += RP_THREADS)
-        xq[x] = __float2int_rn(fminf(fmaxf(q[x], -1.0f), 1.0f) * 4194304.0f);
+    load_query_digits(dig, qdig, (int64_t)B * residual_rows(nq), (int64_t)b * residual_rows(nq) + score_row(i));
     __syncthreads();
-    if (threadIdx.x < 32) {
-        int s = 0;
-        for (int x = threadIdx.x; x < D; x += 32) s += xq[x];
-        s = __reduce_add_sync(0xffffffffu, s);
-        if (threadIdx.x == 0) s_sq = s;
-    }
-    for (int e = threadIdx.x; e < (D >> 2) * 16; e += RP_THREADS) {
-        const int g = e >> 4, v = e & 15;
-        int s = 0;
-#pragma unroll
-        for (int t = 0; t < 4; ++t) s += ((v >> t) & 1) ? xq[4 * g + t] : 0;
-        lut[e] = s;
-    }
-    __syncthreads();
-    const int sq = s_sq;
-    const int CW = D >> 5;
+    const int sq = query_sum(dig);
     const uint2 *rk = ranks + (int64_t)b * words;
     int32_t *Mb = LISTS ? nullptr : M + (int64_t)b * maxc * nq;
     int32_t *heads = LISTS ? lists.head + (int64_t)b * maxc : nullptr;
     unsigned long long *nodes = LISTS ? lists.node + (int64_t)b * lists.cap : nullptr;
-    auto code_dot = [&](int64_t t) -> int {
-        uint32_t word[4];                              // D <= 128: at most four words
-        if (CW == 4) {                                 // 16-byte rows (the attach call checks the alignment)
-            const uint4 v = __ldg(reinterpret_cast<const uint4 *>(bits + t * 4));
-            word[0] = v.x; word[1] = v.y; word[2] = v.z; word[3] = v.w;
-        } else {
-#pragma unroll
-            for (int w = 0; w < 4; ++w) word[w] = w < CW ? __ldg(bits + t * CW + w) : 0u;
-        }
-        int T = 0;
-#pragma unroll
-        for (int w = 0; w < 4; ++w)
-            if (w < CW) {
-#pragma unroll
-                for (int k = 0; k < 8; ++k) T += lut[(8 * w + k) * 16 + ((word[w] >> (4 * k)) & 15u)];
-            }
-        return T;
-    };
-    // (the token's factor, the document's bitmap word and its rank come as arguments: they depend on the list entry
-    // alone, so their loads are issued with the code loads instead of one after the other behind the score)
     uint32_t v0;                                       // node of the list's first entry
     int64_t e0;
+    // (the token's factor, the document's bitmap word and its rank come as arguments: they depend on the list entry
+    // alone, so their loads are issued with the code loads instead of one after the other behind the score)
     auto update = [&](int64_t e, uint32_t d, float factor, int T, uint2 r) {
         const float est = __fmul_rn(factor, __fmul_rn(c, (float)(2 * T - sq)));
         if (est > 0.0f) {                              // the table starts at 0 (Algorithm 2)
@@ -155,22 +115,24 @@ rabitq_partial_kernel(const float *__restrict__ q_rot, int nq, int D, int P, flo
         v0 = (uint32_t)((i * P + p) * longest);
         e0 = tok_off[cen];
         const int64_t e1 = tok_off[cen + 1];
-        int64_t e = e0 + threadIdx.x;
-        for (; e + RP_THREADS < e1; e += 2 * RP_THREADS) {         // two visits per iteration, their loads issued together
-            const int64_t ta = DBG_TOK(tok_id[e]), tb = DBG_TOK(tok_id[e + RP_THREADS]);
-            const uint32_t da = (uint32_t)DBG_DOC(tok_doc[e]), db = (uint32_t)DBG_DOC(tok_doc[e + RP_THREADS]);
-            const float fa = __ldg(inv_dot + ta), fb = __ldg(inv_dot + tb);
-            const uint2 ra = __ldg(rk + (da >> 5)), rb = __ldg(rk + (db >> 5));
-            const int Ta = code_dot(ta), Tb = code_dot(tb);
-            update(e, da, fa, Ta, ra);
-            update(e + RP_THREADS, db, fb, Tb, rb);
-        }
-        if (e < e1) {
-            const int64_t t = DBG_TOK(tok_id[e]);
-            const uint32_t d = (uint32_t)DBG_DOC(tok_doc[e]);
-            const float f = __ldg(inv_dot + t);
-            const uint2 r = __ldg(rk + (d >> 5));
-            update(e, d, f, code_dot(t), r);
+        // two visits per thread and iteration, their loads issued together (the second one past the end repeats the first)
+        for (int64_t e = e0 + threadIdx.x; e < e1; e += 2 * RP_THREADS) {
+            const int64_t at[2] = {e, e + RP_THREADS < e1 ? e + RP_THREADS : e};
+            uint32_t d[2], w[2][CODE_WORDS<1>];
+            uint2 r[2];
+            float f[2];
+#pragma unroll
+            for (int n = 0; n < 2; ++n) {
+                const int64_t t = DBG_TOK(tok_id ? (int64_t)tok_id[at[n]] : at[n]);
+                load_code<1>(w[n], bits + t * CW, CW);
+                f[n] = __ldg(inv_dot + t);
+                d[n] = (uint32_t)DBG_DOC(tok_doc[at[n]]);
+                r[n] = __ldg(rk + (d[n] >> 5));
+            }
+            int T[2];
+            code_dots<1, 2>(T, w, CW, dig);
+            update(at[0], d[0], f[0], T[0], r[0]);
+            if (at[1] != e) update(at[1], d[1], f[1], T[1], r[1]);
         }
     }
 }
@@ -201,7 +163,7 @@ rabitq_sum_kernel(const int32_t *__restrict__ M, const int32_t *__restrict__ n_c
     }
 }
 
-int launch_rabitq_partial(const Index &ix, const Params &p, const Layout &L, const float *q_rot,
+int launch_rabitq_partial(const Index &ix, const Params &p, const Layout &L, const int8_t *qdig_rot,
                           const int32_t *probes, const uint2 *ranks, const int32_t *n_cand, void *partial_m,
                           int32_t *fprime_bits, cudaStream_t st)
 {
@@ -219,14 +181,16 @@ int launch_rabitq_partial(const Index &ix, const Params &p, const Layout &L, con
     const float c = (float)(1.0 / (sqrt((double)ix.D) * 4194304.0));
     const int splits = refine_splits(ix, p);
     const dim3 grid((unsigned)(p.nq * splits), (unsigned)p.B);
-    const uint32_t *bits = reinterpret_cast<const uint32_t *>(ix.rq_bits);
+    const uint32_t *bits = reinterpret_cast<const uint32_t *>(ix.list_bits ? ix.list_bits : ix.rq_bits);
+    const float *inv = ix.list_bits ? ix.list_inv : ix.rq_inv;
+    const int32_t *ids = ix.list_bits ? nullptr : ix.tok_id;
     if (use_lists)
-        rabitq_partial_kernel<true><<<grid, RP_THREADS, 0, st>>>(q_rot, p.nq, ix.D, p.P, c, probes, ix.tok_off, ix.tok_id,
-                                                                 ix.tok_doc, bits, ix.rq_inv, ranks, L.words, p.maxc, M,
+        rabitq_partial_kernel<true><<<grid, RP_THREADS, 0, st>>>(qdig_rot, p.nq, p.B, ix.D / 32, p.P, c, probes, ix.tok_off, ids,
+                                                                 ix.tok_doc, bits, inv, ranks, L.words, p.maxc, M,
                                                                  lists, ix.max_tok_list, splits);
     else
-        rabitq_partial_kernel<false><<<grid, RP_THREADS, 0, st>>>(q_rot, p.nq, ix.D, p.P, c, probes, ix.tok_off, ix.tok_id,
-                                                                  ix.tok_doc, bits, ix.rq_inv, ranks, L.words, p.maxc, M,
+        rabitq_partial_kernel<false><<<grid, RP_THREADS, 0, st>>>(qdig_rot, p.nq, p.B, ix.D / 32, p.P, c, probes, ix.tok_off, ids,
+                                                                  ix.tok_doc, bits, inv, ranks, L.words, p.maxc, M,
                                                                   lists, ix.max_tok_list, splits);
     CHIMERA_CUDA(cudaGetLastError());
     if (use_lists) {
