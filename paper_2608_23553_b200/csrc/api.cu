@@ -123,8 +123,8 @@ Layout make_layout(const Index &ix, const Params &p)
     L.pq_cnt = take(L.pq_stride ? B * nq * sizeof(int32_t) : 0);
     L.pq_keys = take(L.pq_stride ? B * nq * (size_t)L.pq_cap * sizeof(unsigned long long) : 0);
     L.pq_ovf = take(L.pq_stride ? B * sizeof(int32_t) : 0);
-    L.bitmap = take(B * (size_t)L.words * sizeof(uint32_t));
-    L.chunk_cnt = take(B * (size_t)(L.n_chunks + 1) * sizeof(int32_t));
+    L.bitmap = take(B * ((size_t)L.words + (nq + 31) / 32) * sizeof(uint32_t));
+    L.chunk_cnt = take(B * (size_t)L.n_chunks * sizeof(int32_t));
     L.cand = take(B * (size_t)p.maxc * sizeof(int32_t));
     L.n_cand = take(B * sizeof(int32_t));
     L.ci = take(B * (size_t)p.maxc * sizeof(int32_t));
@@ -264,6 +264,8 @@ static int run(const Index &ix, const Params &p, int first, int last, const floa
     int32_t *ci = (int32_t *)(ws + L.ci);
     const bool two_phase = coarse_supported(p.nq) && !partial && !rabitq;
     const bool filter = filter_used(ix, p) && !partial && !rabitq;      // (stage 3's first cut)
+    // the candidates' token ranges, where the 8-bit scan reads them for every candidate
+    int2 *scan_rng = two_phase && !filter && ix.T < 0x7fffffffLL ? (int2 *)(ws + L.cand_rng) : nullptr;
     // blocks per query for the exact scores of a short list (two to three times n_prune documents): one per SM in a large
     // batch, more when n_prune is large (about one block per eight survivors wanted; Large, n_prune 4096: 2.75 ms with
     // 444-592 blocks against 3.26 ms with 148, Mid unchanged), four per SM when a single query has the GPU to itself
@@ -323,11 +325,16 @@ static int run(const Index &ix, const Params &p, int first, int last, const floa
     // stages 1 and 2a of one call run together when the layout provides for it: the probes come out of the score
     // table's epilogue and the table is not read again
     const bool together = first <= 1 && last >= 2 && !graph && L.pq_stride > 0;
+    // a small bitmap, and the probe kernel's counters behind it, are cleared on the side by the first kernel of stage 1 (one
+    // operation less in the chain)
+    const int64_t bitmap_words = (int64_t)p.B * (L.words + (p.nq + 31) / 32);
+    const int64_t clear_words = first <= 1 && !graph && bitmap_words <= (1 << 19) ? bitmap_words : 0;
+    int32_t *probes_done = clear_words > 0 ? (int32_t *)bitmap + (int64_t)p.B * L.words : nullptr;
     if (first <= 1 && last >= 1 && !graph) {
         if (together)
-            rc = launch_score_table_probes(ix, p, L, queries, qdig, qdig4, table, table8, ws, status, st);
+            rc = launch_score_table_probes(ix, p, L, queries, qdig, qdig4, table, table8, ws, status, st, bitmap, clear_words);
         else
-            rc = launch_score_table(ix, p, queries, qdig, qdig4, table, table8, status, st);
+            rc = launch_score_table(ix, p, queries, qdig, qdig4, table, table8, status, st, bitmap, clear_words);
         if (rc) return rc;
         prof_mark(SLOT_G1, st);
     }
@@ -338,12 +345,13 @@ static int run(const Index &ix, const Params &p, int first, int last, const floa
                 return rc;
         } else if (together) {
             if ((rc = launch_probe_merge(ix, p, L, table, ws, st))) return rc;
-        } else if ((rc = launch_probes(ix, p, L, table, part, probes, st))) {
+        } else if ((rc = launch_probes(ix, p, L, table, part, probes, probes_done, st))) {
             return rc;
         }
         prof_mark(SLOT_PROBE, st);
-        if ((rc = launch_gather(ix, p, L, probes, bitmap, chunk_cnt, cand, n_cand,
-                                partial || rabitq ? ranks : nullptr, status, st))) return rc;
+        if ((rc = launch_gather(ix, p, L, probes, bitmap, clear_words > 0, chunk_cnt, cand, n_cand, partial || rabitq ? ranks : nullptr,
+                                scan_rng, scan_rng && contenders_split(ix, p) ? ci : nullptr, status, st)))
+            return rc;
         prof_mark(SLOT_GATHER, st);
     }
     if (first <= 3 && last >= 3) {
@@ -374,8 +382,8 @@ static int run(const Index &ix, const Params &p, int first, int last, const floa
             const int32_t *docs = cand, *n_docs = n_cand;
             const int2 *docs_rng = ix.T < 0x7fffffffLL ? (const int2 *)(ws + L.cand_rng) : nullptr;
             int2 *cont_rng = docs_rng ? (int2 *)(ws + L.cont_rng) : nullptr;
-            if (docs_rng && two_phase && !filter &&
-                (rc = launch_cand_ranges(ix, p, cand, n_cand, (int2 *)(ws + L.cand_rng), st)))
+            if (scan_rng && first > 2 &&               // (else the gather wrote them)
+                (rc = launch_cand_ranges(ix, p, cand, n_cand, scan_rng, ci, st)))
                 return rc;
             if (filter) {
                 if ((rc = launch_filter_scan(ix, p, L, table, table8, cand, n_cand, hi, cont, cont_rng, ws, st)))

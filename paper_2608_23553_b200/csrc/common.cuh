@@ -80,8 +80,8 @@ struct Layout {
     size_t pq_cnt;        // int32  [B*nq]            keys queued for the row,
     size_t pq_keys;       // uint64 [B*nq][pq_cap]    the keys,
     size_t pq_ovf;        // int32  [B]               1 = a queue of this query overflowed (redo by the table scan)
-    size_t bitmap;        // uint32 [B][words]
-    size_t chunk_cnt;     // int32  [B][n_chunks + 1]
+    size_t bitmap;        // uint32 [B][words], followed by the probe kernel's counters int32 [B][ceil(nq / 32)]
+    size_t chunk_cnt;     // int32  [B][n_chunks]
     size_t cand;          // int32  [B][maxc]
     size_t n_cand;        // int32  [B]
     size_t ci;            // int32  [B][maxc]         exact CI of the contenders (of every candidate: generic q_len / tap)
@@ -154,6 +154,35 @@ enum Slot { SLOT_G1 = 0, SLOT_PROBE, SLOT_GATHER, SLOT_CI, SLOT_SELECT, SLOT_G4,
 void count_launch(int slot, int n = 1);
 
 // ---------------------------------------------------------------------------------------------------------------
+// Launches of a search.  A search is a chain of up to two dozen short kernels on one stream, so the gaps between them are a
+// good part of a small call.  Every kernel is launched as a programmatic dependent of the one before it: its blocks are
+// placed as soon as that kernel's have exited, and pdl_entry(), the first thing every kernel does, waits until
+// that kernel has finished and its writes are visible (one query against 10,000 documents: 142 -> 107 us).  EVERY kernel
+// launched this way has to begin with pdl_entry(), on all its threads: the next kernel relies on this one to have waited.
+// ---------------------------------------------------------------------------------------------------------------
+template <class... P, class... A>
+void launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A &&...args)
+{
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);       // (errors: cudaGetLastError() behind every launch)
+}
+#ifdef __CUDACC__
+__device__ __forceinline__ void pdl_entry() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// (No kernel lets its successor in earlier, with griddepcontrol.launch_dependents: blocks that wait hold shared memory, and
+// with it L1, of the kernel they wait for.  Measured with the trigger behind pdl_entry(), in all kernels: Mid, batch 256, 9.2
+// -> 12.1 ms; in the short ones only: 9.2 -> 9.6 ms, one query 184 -> 214 us.)
+#endif
+
+// ---------------------------------------------------------------------------------------------------------------
 // Stage launchers (one per .cu file).  Each only enqueues kernels on `st` and returns a chimera_status.
 // ---------------------------------------------------------------------------------------------------------------
 int build_index_device(Index &ix, const float *centroids, const int32_t *doclens, cudaStream_t st);
@@ -161,14 +190,17 @@ int build_index_device(Index &ix, const float *centroids, const int32_t *doclens
 // out-of-range elements set ST_BAD_QUERY.
 // dig4 (may be NULL): the same planes for stage 4, rows = query tokens (q_len of them per query) in score_row() order,
 // padded to residual_rows(q_len) per query; the padding is not written.  dig may be NULL then.
+// clear / clear_n (may be NULL / 0): 32-bit words set to zero on the side, for a later kernel of the same call.
 int launch_digits(const float *x, int64_t rows, int D, int nbits, int8_t *dig, int8_t *dig4, int q_len, uint32_t *status,
-                  cudaStream_t st);
+                  cudaStream_t st, uint32_t *clear = nullptr, int64_t clear_n = 0);
 
 // table8 may be NULL (no coarse copy wanted).
 int launch_score_table(const Index &ix, const Params &p, const float *queries, int8_t *qdig, int8_t *qdig4, int32_t *table,
-                       uint8_t *table8, uint32_t *status, cudaStream_t st);
+                       uint8_t *table8, uint32_t *status, cudaStream_t st, uint32_t *clear = nullptr, int64_t clear_n = 0);
+// done (may be NULL): counters int32 [B][ceil(nq / 32)], zero before; the probe kernel's last block then folds its lists
+// itself instead of a second kernel.
 int launch_probes(const Index &ix, const Params &p, const Layout &L, const int32_t *table, unsigned long long *part,
-                  int32_t *probes, cudaStream_t st);
+                  int32_t *probes, int32_t *done, cudaStream_t st);
 // Stages 1 and 2a together (g1_score_table.cu), used when the layout has pq_stride > 0, and its probe-side pieces
 // (g2_probe.cu): the sample's top nprobe and bounds; the final top nprobe from sample list and queues, with the table
 // scan as the fallback for queries whose queue overflowed.
@@ -178,13 +210,18 @@ int probe_queue_cap();
 int probe_sample_groups(const Index &ix, int stride);
 int launch_score_table_probes(const Index &ix, const Params &p, const Layout &L, const float *queries, int8_t *qdig,
                               int8_t *qdig4,
-                              int32_t *table, uint8_t *table8, char *ws, uint32_t *status, cudaStream_t st);
+                              int32_t *table, uint8_t *table8, char *ws, uint32_t *status, cudaStream_t st,
+                              uint32_t *clear = nullptr, int64_t clear_n = 0);
 int launch_probe_sample(const Index &ix, const Params &p, const Layout &L, const int32_t *table, char *ws,
                         int n_sample_tiles, cudaStream_t st);
 int launch_probe_merge(const Index &ix, const Params &p, const Layout &L, const int32_t *table, char *ws, cudaStream_t st);
+// bitmap_clear: the bitmap is zero already.  ranks, rng (the candidates' token ranges), cont_scratch (rows of which the
+// contender step's histogram is cleared): each may be NULL.
 int launch_gather(const Index &ix, const Params &p, const Layout &L, const int32_t *probes, uint32_t *bitmap,
-                  int32_t *chunk_cnt, int32_t *cand, int32_t *n_cand, uint2 *ranks, uint32_t *status,
-                  cudaStream_t st);
+                  bool bitmap_clear, int32_t *chunk_cnt, int32_t *cand, int32_t *n_cand, uint2 *ranks, int2 *rng,
+                  int32_t *cont_scratch, uint32_t *status, cudaStream_t st);
+bool contenders_split(const Index &ix, const Params &p);
+int contender_hist_entries();
 // Token-level posting lists for the partial-score refinement (allocates; index_build.cu).
 int build_token_lists(Index &ix, cudaStream_t st);
 // A copy of src ([T][words] 32-bit words, document-major) in the order of the token lists, so that a list's codes are one
@@ -201,9 +238,10 @@ int launch_filter_contenders(const Index &ix, const Params &p, const Layout &L, 
                              char *ws, cudaStream_t st);
 bool coarse_supported(int nq);
 int launch_coarse_table(const Index &ix, const Params &p, const int32_t *table, uint8_t *table8, cudaStream_t st);
-// The candidates' token ranges (corpora with fewer than 2^31 tokens).
+// The candidates' token ranges (corpora with fewer than 2^31 tokens); also clears the contender step's histograms at the
+// head of its scratch rows (int32 [B][maxc]) where launch_contenders will use them.
 int launch_cand_ranges(const Index &ix, const Params &p, const int32_t *cand, const int32_t *n_cand, int2 *rng,
-                       cudaStream_t st);
+                       int32_t *cont_scratch, cudaStream_t st);
 // rng: those ranges (may be NULL: per-document offset lookups instead; (CI, 0) stands for a document whose exact CI is
 // known).  lo may be NULL with ranges.
 int launch_coarse_bounds(const Index &ix, const Params &p, const uint8_t *table8, const int32_t *cand,
@@ -327,6 +365,13 @@ __device__ __forceinline__ int warp_sum(int v)
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
+}
+// (first token, length) of a document (corpora with fewer than 2^31 tokens).
+__device__ __forceinline__ int2 doc_range(const int64_t *doc_off, int32_t d)
+{
+    d = DBG_DOC(d);
+    const int64_t t0 = __ldg(doc_off + d);
+    return make_int2((int)t0, (int)(__ldg(doc_off + d + 1) - t0));
 }
 __device__ __forceinline__ float warp_sum(float v)
 {

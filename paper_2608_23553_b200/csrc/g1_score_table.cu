@@ -87,6 +87,7 @@ score_table_umma(const int8_t *__restrict__ cdig, const __grid_constant__ CUtens
                  int64_t q_rows, int n_tiles, int tiles_per_split, int32_t *__restrict__ table,
                  uint8_t *__restrict__ table8, uint32_t *status, long long wait_limit, int skip_loads, G1Tiles tiles)
 {
+    pdl_entry();
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint32_t s_tmem_base;
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -410,7 +411,7 @@ static int launch_g1_tiles(const Index &ix, const Params &p, const CUtensorMap &
     do {                                                                                                               \
         CHIMERA_CUDA(cudaFuncSetAttribute(score_table_umma<KS, FILTER>, cudaFuncAttributeMaxDynamicSharedMemorySize,   \
                                           (int)G1_SMEM));                                                              \
-        score_table_umma<KS, FILTER><<<grid, G1_THREADS, G1_SMEM, st>>>(ix.cdig, map_q, ix.K, p.nq, rows, n_tiles,     \
+        launch(score_table_umma<KS, FILTER>, grid, G1_THREADS, G1_SMEM, st, ix.cdig, map_q, ix.K, p.nq, rows, n_tiles,     \
                                                                         tiles_per_split, table, table8, status, limit, \
                                                                         skip, tiles);                                  \
     } while (0)
@@ -426,10 +427,10 @@ static int launch_g1_tiles(const Index &ix, const Params &p, const CUtensorMap &
 }
 
 int launch_score_table(const Index &ix, const Params &p, const float *queries, int8_t *qdig, int8_t *qdig4, int32_t *table,
-                       uint8_t *table8, uint32_t *status, cudaStream_t st)
+                       uint8_t *table8, uint32_t *status, cudaStream_t st, uint32_t *clear, int64_t clear_n)
 {
     const int64_t rows = (int64_t)p.B * p.nq;
-    int rc = launch_digits(queries, rows, ix.D, ix.nbits, qdig, qdig4, p.nq, status, st);
+    int rc = launch_digits(queries, rows, ix.D, ix.nbits, qdig, qdig4, p.nq, status, st, clear, clear_n);
     if (rc) return rc;
     CUtensorMap map_q;
     if ((rc = make_plane_map(&map_q, qdig, rows, G1_N, 3))) return rc;        // one load brings a tile's three planes
@@ -447,10 +448,11 @@ int launch_score_table(const Index &ix, const Params &p, const float *queries, i
 // descending, centroid id ascending): a centroid that belongs to it has a score >= the bound, so it is queued.
 // A query with a token whose queue overflowed is redone by the table scan of the separate probe stage.
 int launch_score_table_probes(const Index &ix, const Params &p, const Layout &L, const float *queries, int8_t *qdig, int8_t *qdig4,
-                              int32_t *table, uint8_t *table8, char *ws, uint32_t *status, cudaStream_t st)
+                              int32_t *table, uint8_t *table8, char *ws, uint32_t *status, cudaStream_t st,
+                              uint32_t *clear, int64_t clear_n)
 {
     const int64_t rows = (int64_t)p.B * p.nq;
-    int rc = launch_digits(queries, rows, ix.D, ix.nbits, qdig, qdig4, p.nq, status, st);
+    int rc = launch_digits(queries, rows, ix.D, ix.nbits, qdig, qdig4, p.nq, status, st, clear, clear_n);
     if (rc) return rc;
     CUtensorMap map_q;
     if ((rc = make_plane_map(&map_q, qdig, rows, G1_N, 3))) return rc;

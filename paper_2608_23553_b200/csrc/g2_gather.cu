@@ -2,8 +2,9 @@
 // (Sec. 3.2 step 1: L_q is the union of the probed lists, S the set of their source documents).
 //
 // The inverted file stores, per centroid, the unique ids of those documents.  Each probed list is streamed once and
-// sets one bit per document in a per-query bitmap (the dedup); the bitmap is then compacted into an ascending id
-// list with a three-kernel count / scan / write pass.
+// sets one bit per document in a per-query bitmap (the dedup); the bitmap is then compacted into an ascending id list with
+// the documents' token ranges: a count per chunk of the bitmap and an ordered write, or, for few queries on small corpora, the
+// write alone over shorter chunks, each of which counts the words before its own.
 #include "common.cuh"
 
 namespace chimera {
@@ -13,6 +14,7 @@ __global__ void __launch_bounds__(128)
 mark_kernel(const int32_t *__restrict__ probes, int n_lists, const int64_t *__restrict__ ivf_off,
             const int32_t *__restrict__ ivf_doc, uint32_t *__restrict__ bitmap, int64_t words)
 {
+    pdl_entry();
     const int b = blockIdx.y;
     const int32_t c = DBG_CID(probes[(int64_t)b * n_lists + blockIdx.x]);
     uint32_t *bm = bitmap + (int64_t)b * words;
@@ -36,8 +38,44 @@ mark_kernel(const int32_t *__restrict__ probes, int n_lists, const int64_t *__re
     }
 }
 
+// The same with the bitmap in shared memory, for small corpora: their lists set the same few words over and over, and
+// atomics on one L2 line come one after the other (10,000 documents, 128 lists of 625: 17 us, here 6.5).  grid (blocks, B): a
+// block takes every gridDim.x-th list and adds its bits to the query's bitmap at the end.
+__global__ void __launch_bounds__(512)
+mark_shared_kernel(const int32_t *__restrict__ probes, int n_lists, const int64_t *__restrict__ ivf_off,
+                   const int32_t *__restrict__ ivf_doc, uint32_t *__restrict__ bitmap, int words)
+{
+    pdl_entry();
+    extern __shared__ uint32_t bits[];
+    const int b = blockIdx.y;
+    for (int w = threadIdx.x; w < words; w += 512) bits[w] = 0u;
+    __syncthreads();
+    // a warp per list
+    for (int l = blockIdx.x + gridDim.x * (threadIdx.x >> 5); l < n_lists; l += gridDim.x * 16) {
+        const int32_t c = DBG_CID(probes[(int64_t)b * n_lists + l]);
+        const int64_t hi = ivf_off[c + 1];
+        for (int64_t e0 = ivf_off[c] + (threadIdx.x & 31); e0 < hi; e0 += 8 * 32) {
+            uint32_t d[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                d[u] = e0 + 32 * u < hi ? (uint32_t)ivf_doc[e0 + 32 * u] : 0xffffffffu;
+                if (d[u] != 0xffffffffu && !DBG_DOC_OK(d[u])) d[u] = 0xffffffffu;
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (d[u] != 0xffffffffu) {
+                    const uint32_t bit = 1u << (d[u] & 31);
+                    if (!(bits[d[u] >> 5] & bit)) atomicOr(&bits[d[u] >> 5], bit);
+                }
+        }
+    }
+    __syncthreads();
+    for (int w = threadIdx.x; w < words; w += 512)
+        if (bits[w]) atomicOr(&bitmap[(int64_t)b * words + w], bits[w]);
+}
+
 constexpr int CHUNK_THREADS = 256;
-constexpr int WORDS_PER_THREAD = BITMAP_CHUNK_WORDS / CHUNK_THREADS;   // 4 consecutive words per thread
+constexpr int WORDS_PER_THREAD = BITMAP_CHUNK_WORDS / CHUNK_THREADS;   // at most: 4 consecutive words per thread
 constexpr int COMPACT_STAGE = 8192;      // ids a chunk stages in shared memory (a chunk covers 32,768 documents)
 
 __device__ __forceinline__ int block_exclusive_scan_256(int v, int *total)
@@ -67,6 +105,7 @@ __device__ __forceinline__ int block_exclusive_scan_256(int v, int *total)
 __global__ void __launch_bounds__(CHUNK_THREADS)
 count_kernel(const uint32_t *__restrict__ bitmap, int64_t words, int n_chunks, int32_t *__restrict__ chunk_cnt)
 {
+    pdl_entry();
     const int b = blockIdx.y;
     const uint32_t *bm = bitmap + (int64_t)b * words;
     int64_t w0 = (int64_t)blockIdx.x * BITMAP_CHUNK_WORDS + threadIdx.x * WORDS_PER_THREAD;
@@ -76,59 +115,60 @@ count_kernel(const uint32_t *__restrict__ bitmap, int64_t words, int n_chunks, i
         if (w0 + j < words) c += __popc(bm[w0 + j]);
     int total;
     block_exclusive_scan_256(c, &total);
-    if (threadIdx.x == 0) chunk_cnt[(int64_t)b * (n_chunks + 1) + blockIdx.x] = total;
+    if (threadIdx.x == 0) chunk_cnt[(int64_t)b * n_chunks + blockIdx.x] = total;
 }
 
-// grid (B), one warp: exclusive scan of the chunk counts in place; entry n_chunks and n_cand[b] get the total
-// (clamped to maxc; an overflow sets the status bit).
-__global__ void __launch_bounds__(32)
-chunk_scan_kernel(int32_t *__restrict__ chunk_cnt, int n_chunks, int64_t maxc, int32_t *__restrict__ n_cand,
-                  uint32_t *status)
-{
-    const int b = blockIdx.x, lane = threadIdx.x;
-    int32_t *cc = chunk_cnt + (int64_t)b * (n_chunks + 1);
-    int run = 0;
-    for (int base = 0; base < n_chunks; base += 32) {
-        int i = base + lane;
-        int v = i < n_chunks ? cc[i] : 0;
-        int incl = v;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            int t = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += t;
-        }
-        if (i < n_chunks) cc[i] = run + incl - v;
-        run += __shfl_sync(0xffffffffu, incl, 31);
-    }
-    if (lane == 0) {
-        cc[n_chunks] = run;
-        if ((int64_t)run > maxc) {
-            atomicOr(status, ST_OVERFLOW);
-            run = (int)maxc;
-        }
-        n_cand[b] = run;
-    }
-}
-
-// grid (n_chunks, B): write the ids of the set bits of each chunk, ascending, at its scanned offset.
+// grid (n_chunks, B): write the ids of the set bits of each chunk, ascending, behind those of the chunks before it (whose
+// counts are in chunk_cnt; NULL: their words are counted here), and the documents' token ranges (rng may be NULL).  The last
+// chunk's block reports the query's candidates (clamped to maxc; an overflow sets the status bit).  cont_hist (may be NULL):
+// scratch rows whose first `hist_n` entries are cleared for a later kernel.
 __global__ void __launch_bounds__(CHUNK_THREADS)
-compact_kernel(const uint32_t *__restrict__ bitmap, int64_t words, int n_chunks,
+compact_kernel(const uint32_t *__restrict__ bitmap, int64_t words, int n_chunks, int chunk_words,
                const int32_t *__restrict__ chunk_cnt, int64_t maxc, int32_t *__restrict__ cand,
-               uint2 *__restrict__ ranks)
+               int32_t *__restrict__ n_cand, uint2 *__restrict__ ranks, const int64_t *__restrict__ doc_off,
+               int2 *__restrict__ rng, int32_t *__restrict__ cont_hist, int hist_n, uint32_t *status)
 {
+    pdl_entry();
+    __shared__ int s_base;
+    if (threadIdx.x == 0) s_base = 0;
+    if (cont_hist)
+        for (int i = blockIdx.x * CHUNK_THREADS + threadIdx.x; i < hist_n; i += gridDim.x * CHUNK_THREADS)
+            cont_hist[(int64_t)blockIdx.y * maxc + i] = 0;
+    __syncthreads();
+    {
+        int before = 0;
+        if (chunk_cnt) {
+            for (int c = threadIdx.x; c < (int)blockIdx.x; c += CHUNK_THREADS)
+                before += chunk_cnt[(int64_t)blockIdx.y * n_chunks + c];
+        } else {
+            const uint32_t *bm = bitmap + (int64_t)blockIdx.y * words;
+            const int n = (int)blockIdx.x * chunk_words;
+#pragma unroll 8
+            for (int w = threadIdx.x; w < n; w += CHUNK_THREADS) before += __popc(bm[w]);
+        }
+        before = __reduce_add_sync(0xffffffffu, before);
+        if ((threadIdx.x & 31) == 0 && before) atomicAdd(&s_base, before);
+    }
     const int b = blockIdx.y;
     const uint32_t *bm = bitmap + (int64_t)b * words;
-    int64_t w0 = (int64_t)blockIdx.x * BITMAP_CHUNK_WORDS + threadIdx.x * WORDS_PER_THREAD;
+    const int wpt = chunk_words > CHUNK_THREADS ? chunk_words / CHUNK_THREADS : 1;
+    const int64_t w0 = (int64_t)blockIdx.x * chunk_words + threadIdx.x * wpt;
+    const int mine = (int)threadIdx.x * wpt < chunk_words ? wpt : 0;      // words of this thread
     uint32_t w[WORDS_PER_THREAD];
     int c = 0;
 #pragma unroll
     for (int j = 0; j < WORDS_PER_THREAD; ++j) {
-        w[j] = (w0 + j < words) ? bm[w0 + j] : 0u;
+        w[j] = (j < mine && w0 + j < words) ? bm[w0 + j] : 0u;
         c += __popc(w[j]);
     }
     int total;
-    const int local = block_exclusive_scan_256(c, &total);
-    const int64_t base = chunk_cnt[(int64_t)b * (n_chunks + 1) + blockIdx.x];
+    const int local = block_exclusive_scan_256(c, &total);      // (its barrier is also the one behind s_base)
+    const int64_t base = s_base;
+    if (threadIdx.x == 0 && (int)blockIdx.x == n_chunks - 1) {
+        const int64_t all = base + total;
+        if (all > maxc) atomicOr(status, ST_OVERFLOW);
+        n_cand[b] = (int32_t)(all < maxc ? all : maxc);
+    }
     int32_t *out = cand + (int64_t)b * maxc;
     // A thread's ids are consecutive in the output but the threads' runs are ~30 ids apart, so direct stores are
     // scattered 4-byte writes: when the chunk's ids fit, they are staged in shared memory and copied out coalesced.
@@ -138,41 +178,62 @@ compact_kernel(const uint32_t *__restrict__ bitmap, int64_t words, int n_chunks,
 #pragma unroll
     for (int j = 0; j < WORDS_PER_THREAD; ++j) {
         uint32_t bits = w[j];
-        if (ranks && w0 + j < words)          // the word and the candidates before it: document -> candidate index
+        if (ranks && j < mine && w0 + j < words)          // the word and the candidates before it: document -> candidate index
             ranks[(int64_t)b * words + w0 + j] = make_uint2(w[j], (uint32_t)(use_stage ? base + pos : pos));
         while (bits) {
             int t = __ffs(bits) - 1;
             bits &= bits - 1;
             const int32_t id = (int32_t)(((w0 + j) << 5) + t);
-            if (use_stage) staged[pos] = id;
-            else if (pos < maxc) out[pos] = id;
+            if (use_stage) {
+                staged[pos] = id;
+            } else if (pos < maxc) {
+                out[pos] = id;
+                if (rng) rng[(int64_t)b * maxc + pos] = doc_range(doc_off, id);
+            }
             ++pos;
         }
     }
     if (use_stage) {
         __syncthreads();
         for (int e = threadIdx.x; e < total; e += CHUNK_THREADS)
-            if (base + e < maxc) out[base + e] = staged[e];
+            if (base + e < maxc) {
+                out[base + e] = staged[e];
+                if (rng) rng[(int64_t)b * maxc + base + e] = doc_range(doc_off, staged[e]);
+            }
     }
 }
 
 int launch_gather(const Index &ix, const Params &p, const Layout &L, const int32_t *probes, uint32_t *bitmap,
-                  int32_t *chunk_cnt, int32_t *cand, int32_t *n_cand, uint2 *ranks, uint32_t *status,
-                  cudaStream_t st)
+                  bool bitmap_clear, int32_t *chunk_cnt, int32_t *cand, int32_t *n_cand, uint2 *ranks, int2 *rng,
+                  int32_t *cont_scratch, uint32_t *status, cudaStream_t st)
 {
-    CHIMERA_CUDA(cudaMemsetAsync(bitmap, 0, sizeof(uint32_t) * (size_t)L.words * p.B, st));
+    if (!bitmap_clear) CHIMERA_CUDA(cudaMemsetAsync(bitmap, 0, sizeof(uint32_t) * (size_t)L.words * p.B, st));
     const int n_lists = p.nq * p.P;
-    mark_kernel<<<dim3((unsigned)n_lists, (unsigned)p.B), 128, 0, st>>>(probes, n_lists, ix.ivf_off, ix.ivf_doc,
-                                                                         bitmap, L.words);
+    const bool few = 4 * p.B <= ix.sm_count;
+    // bitmaps of up to 48 KB whose words are set 32 times or more on average
+    if (L.words <= 12 * 1024 && (double)n_lists * ((double)ix.ivf_len / (double)ix.K) >= 32.0 * (double)L.words) {
+        const int gx = few ? (n_lists < 16 ? n_lists : 16) : 1;
+        launch(mark_shared_kernel, dim3((unsigned)gx, (unsigned)p.B), 512, sizeof(uint32_t) * (size_t)L.words, st, probes, n_lists,
+               ix.ivf_off, ix.ivf_doc, bitmap, (int)L.words);
+    } else {
+        launch(mark_kernel, dim3((unsigned)n_lists, (unsigned)p.B), 128, 0, st, probes, n_lists, ix.ivf_off, ix.ivf_doc,
+               bitmap, L.words);
+    }
     CHIMERA_CUDA(cudaGetLastError());
-    dim3 gc((unsigned)L.n_chunks, (unsigned)p.B);
-    count_kernel<<<gc, CHUNK_THREADS, 0, st>>>(bitmap, L.words, L.n_chunks, chunk_cnt);
+    const dim3 gc((unsigned)L.n_chunks, (unsigned)p.B);
+    // few queries on up to half a million documents: one launch of many short chunks, which count the words before them
+    const bool one_pass = few && L.words <= 16 * 1024;
+    constexpr int SHORT_CHUNK = 64;
+    const dim3 gs((unsigned)((L.words + SHORT_CHUNK - 1) / SHORT_CHUNK), (unsigned)p.B);
+    if (!one_pass) {
+        launch(count_kernel, gc, CHUNK_THREADS, 0, st, bitmap, L.words, L.n_chunks, chunk_cnt);
+        CHIMERA_CUDA(cudaGetLastError());
+    }
+    launch(compact_kernel, one_pass ? gs : gc, CHUNK_THREADS, 0, st, bitmap, L.words, one_pass ? (int)gs.x : L.n_chunks,
+           one_pass ? SHORT_CHUNK : BITMAP_CHUNK_WORDS, one_pass ? nullptr : chunk_cnt, p.maxc, cand,
+           n_cand, ranks, ix.doc_off, rng, cont_scratch, contender_hist_entries(), status);
     CHIMERA_CUDA(cudaGetLastError());
-    chunk_scan_kernel<<<(unsigned)p.B, 32, 0, st>>>(chunk_cnt, L.n_chunks, p.maxc, n_cand, status);
-    CHIMERA_CUDA(cudaGetLastError());
-    compact_kernel<<<gc, CHUNK_THREADS, 0, st>>>(bitmap, L.words, L.n_chunks, chunk_cnt, p.maxc, cand, ranks);
-    CHIMERA_CUDA(cudaGetLastError());
-    count_launch(SLOT_GATHER, 4);
+    count_launch(SLOT_GATHER, one_pass ? 2 : 3);
     return CHIMERA_OK;
 }
 

@@ -29,67 +29,17 @@ __device__ __forceinline__ void list_insert(unsigned long long *list, int P, uns
     list[j * STRIDE] = key;
 }
 
-// grid (probe_blocks, B, ceil(nq / 32)).  part: [B][n_part][P][nq], n_part = probe_blocks (one list per block).
-// only_flagged: NULL, or int32[B]: blocks of queries whose entry is 0 return at once.
-__global__ void __launch_bounds__(PROBE_THREADS)
-probe_partial(const int32_t *__restrict__ table, int64_t K, int nq, int P, int rows_per_block, int n_part,
-              unsigned long long *__restrict__ part, const int32_t *__restrict__ only_flagged)
-{
-    extern __shared__ unsigned long long lists[];    // [P][PROBE_THREADS]
-    if (only_flagged && !only_flagged[blockIdx.y]) return;      // (fallback use: only the flagged queries)
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int col = blockIdx.z * 32 + lane;
-    const int b = blockIdx.y;
-    unsigned long long *mine = lists + threadIdx.x;
-    for (int j = 0; j < P; ++j) mine[j * PROBE_THREADS] = 0ull;
-    const int64_t r0 = (int64_t)blockIdx.x * rows_per_block;
-    int64_t r1 = r0 + rows_per_block;
-    if (r1 > K) r1 = K;
-    if (col < nq) {
-        const int32_t *tb = table + (int64_t)b * K * nq + col;
-        int64_t r = r0 + warp;
-        // sixteen independent loads in flight per thread (the stream is bound by bytes in flight)
-        for (; r + 15 * PROBE_WARPS < r1; r += 16 * PROBE_WARPS) {
-            int32_t sc[16];
-#pragma unroll
-            for (int u = 0; u < 16; ++u) sc[u] = tb[(r + u * PROBE_WARPS) * nq];
-#pragma unroll
-            for (int u = 0; u < 16; ++u) list_insert(mine, P, key_int(sc[u], (int32_t)(r + u * PROBE_WARPS)));
-        }
-        for (; r < r1; r += PROBE_WARPS) list_insert(mine, P, key_int(tb[r * nq], (int32_t)r));
-    }
-    // fold the block's eight lists into warp 0's, then write one list per block and column
-    __syncthreads();
-    if (warp == 0 && col < nq) {
-        for (int w = 1; w < PROBE_WARPS; ++w) {
-            const unsigned long long *src = lists + w * 32 + lane;
-            for (int j = 0; j < P; ++j) {
-                unsigned long long key = src[j * PROBE_THREADS];
-                if (key <= mine[(P - 1) * PROBE_THREADS]) break;
-                list_insert(mine, P, key);
-            }
-        }
-        unsigned long long *dst = part + (((int64_t)b * n_part + blockIdx.x) * P) * nq + col;
-        for (int j = 0; j < P; ++j) dst[(int64_t)j * nq] = mine[j * PROBE_THREADS];
-    }
-}
-
-// grid (1, B, ceil(nq / 32)), THREADS threads.  Folds n_part sorted lists per column into one; writes
-// probes[b][col][0..P).  Warp w takes lists w, w + W, ... (W = THREADS / 32 warps, lane = column); the warps' lists are
-// then folded pairwise in a tree.  With one query per call this kernel is a single block, so it is latency that counts:
-// up to eight list heads are loaded together, and 32 warps share the lists when nprobe is small enough for the
-// shared-memory lists of 1024 threads.
+// Folds n_part sorted lists per column into one; writes probes[b][col][0..P).  Warp w takes lists w, w + W, ... (W =
+// THREADS / 32 warps, lane = column); the warps' lists are then folded pairwise in a tree.  With one query per call this is a
+// single block, so it is latency that counts: up to eight list heads are loaded together.
 template <int THREADS>
-__global__ void __launch_bounds__(THREADS)
-probe_final(const unsigned long long *__restrict__ part, int nq, int P, int n_part, int32_t *__restrict__ probes,
-            const int32_t *__restrict__ only_flagged)
+__device__ __forceinline__ void probe_fold(unsigned long long *lists /* [P][THREADS] */,
+                                           const unsigned long long *__restrict__ part, int b, int nq, int P, int n_part,
+                                           int32_t *__restrict__ probes)
 {
-    extern __shared__ unsigned long long lists[];      // [P][THREADS]
-    if (only_flagged && !only_flagged[blockIdx.y]) return;
     constexpr int W = THREADS / 32;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int col = blockIdx.z * 32 + lane;
-    const int b = blockIdx.y;
     unsigned long long *mine = lists + threadIdx.x;
     for (int j = 0; j < P; ++j) mine[j * THREADS] = 0ull;
     if (col < nq) {
@@ -153,6 +103,75 @@ probe_final(const unsigned long long *__restrict__ part, int nq, int P, int n_pa
     }
 }
 
+// grid (probe_blocks, B, ceil(nq / 32)).  part: [B][n_part][P][nq], n_part = probe_blocks (one list per block).
+// only_flagged: NULL, or int32[B]: blocks of queries whose entry is 0 return at once.  done: NULL, or counters [B][groups], zero
+// before: the block of a query that finishes last folds the lists (few blocks per query), else probe_final does.
+__global__ void __launch_bounds__(PROBE_THREADS)
+probe_partial(const int32_t *__restrict__ table, int64_t K, int nq, int P, int rows_per_block, int n_part,
+              unsigned long long *__restrict__ part, const int32_t *__restrict__ only_flagged, int32_t *__restrict__ done,
+              int32_t *__restrict__ probes)
+{
+    pdl_entry();
+    extern __shared__ unsigned long long lists[];    // [P][PROBE_THREADS]
+    __shared__ int s_last;
+    if (only_flagged && !only_flagged[blockIdx.y]) return;      // (fallback use: only the flagged queries)
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int col = blockIdx.z * 32 + lane;
+    const int b = blockIdx.y;
+    unsigned long long *mine = lists + threadIdx.x;
+    for (int j = 0; j < P; ++j) mine[j * PROBE_THREADS] = 0ull;
+    const int64_t r0 = (int64_t)blockIdx.x * rows_per_block;
+    int64_t r1 = r0 + rows_per_block;
+    if (r1 > K) r1 = K;
+    if (col < nq) {
+        const int32_t *tb = table + (int64_t)b * K * nq + col;
+        int64_t r = r0 + warp;
+        // sixteen independent loads in flight per thread (the stream is bound by bytes in flight)
+        for (; r + 15 * PROBE_WARPS < r1; r += 16 * PROBE_WARPS) {
+            int32_t sc[16];
+#pragma unroll
+            for (int u = 0; u < 16; ++u) sc[u] = tb[(r + u * PROBE_WARPS) * nq];
+#pragma unroll
+            for (int u = 0; u < 16; ++u) list_insert(mine, P, key_int(sc[u], (int32_t)(r + u * PROBE_WARPS)));
+        }
+        for (; r < r1; r += PROBE_WARPS) list_insert(mine, P, key_int(tb[r * nq], (int32_t)r));
+    }
+    // fold the block's eight lists into warp 0's, then write one list per block and column
+    __syncthreads();
+    if (warp == 0 && col < nq) {
+        for (int w = 1; w < PROBE_WARPS; ++w) {
+            const unsigned long long *src = lists + w * 32 + lane;
+            for (int j = 0; j < P; ++j) {
+                unsigned long long key = src[j * PROBE_THREADS];
+                if (key <= mine[(P - 1) * PROBE_THREADS]) break;
+                list_insert(mine, P, key);
+            }
+        }
+        unsigned long long *dst = part + (((int64_t)b * n_part + blockIdx.x) * P) * nq + col;
+        for (int j = 0; j < P; ++j) dst[(int64_t)j * nq] = mine[j * PROBE_THREADS];
+    }
+    if (!done) return;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(&done[b * gridDim.z + blockIdx.z], 1) == (int)gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    probe_fold<PROBE_THREADS>(lists, part, b, nq, P, n_part, probes);
+}
+
+// grid (1, B, ceil(nq / 32)), THREADS threads: the fold in a launch of its own, with up to 32 warps.
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS)
+probe_final(const unsigned long long *__restrict__ part, int nq, int P, int n_part, int32_t *__restrict__ probes,
+            const int32_t *__restrict__ only_flagged)
+{
+    pdl_entry();
+    extern __shared__ unsigned long long lists[];      // [P][THREADS]
+    if (only_flagged && !only_flagged[blockIdx.y]) return;
+    probe_fold<THREADS>(lists, part, blockIdx.y, nq, P, n_part, probes);
+}
+
 // The widest block whose lists (nprobe keys of 8 bytes per thread) fit the default 48 KB of shared memory, at least
 // PROBE_THREADS (whose lists may need the opt-in limit: 128 KB at nprobe = 64).
 static int launch_probe_final(const unsigned long long *part, int B, int nq, int P, int n_part, int32_t *probes,
@@ -161,34 +180,90 @@ static int launch_probe_final(const unsigned long long *part, int B, int nq, int
     const dim3 grid(1, (unsigned)B, (unsigned)((nq + 31) / 32));
     const size_t per_thread = sizeof(unsigned long long) * (size_t)P;
     if (per_thread * 1024 <= 48 * 1024) {
-        probe_final<1024><<<grid, 1024, per_thread * 1024, st>>>(part, nq, P, n_part, probes, only_flagged);
+        launch(probe_final<1024>, grid, 1024, per_thread * 1024, st, part, nq, P, n_part, probes, only_flagged);
     } else if (per_thread * 512 <= 48 * 1024) {
-        probe_final<512><<<grid, 512, per_thread * 512, st>>>(part, nq, P, n_part, probes, only_flagged);
+        launch(probe_final<512>, grid, 512, per_thread * 512, st, part, nq, P, n_part, probes, only_flagged);
     } else {
         const size_t smem = per_thread * PROBE_THREADS;
         if (smem > 48 * 1024)
             CHIMERA_CUDA(cudaFuncSetAttribute(probe_final<PROBE_THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)smem));
-        probe_final<PROBE_THREADS><<<grid, PROBE_THREADS, smem, st>>>(part, nq, P, n_part, probes, only_flagged);
+        launch(probe_final<PROBE_THREADS>, grid, PROBE_THREADS, smem, st, part, nq, P, n_part, probes, only_flagged);
     }
     CHIMERA_CUDA(cudaGetLastError());
     return CHIMERA_OK;
 }
 
-int launch_probes(const Index &ix, const Params &p, const Layout &L, const int32_t *table, unsigned long long *part,
-                  int32_t *probes, cudaStream_t st)
+// Small tables and few queries, where latency counts: a block per query token reads its column (warp w rows 1024 w ... 1024 w +
+// 1023, 32 scores per lane in registers), every warp extracts its nprobe largest keys, the first warp those of the block.
+// One launch and a handful of memory latencies (1,024 centroids: 9 us against 22 us for the list kernels).
+constexpr int PROBE_COL_ROWS = 1024;
+__global__ void __launch_bounds__(1024)
+probe_column_kernel(const int32_t *__restrict__ table, int64_t K, int nq, int P, int32_t *__restrict__ probes)
 {
+    pdl_entry();
+    extern __shared__ unsigned long long best_of[];                       // [warps][P]
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+    const int col = blockIdx.x, b = blockIdx.y;
+    const int32_t *tb = table + (int64_t)b * K * nq + col;
+    const int r0 = warp * PROBE_COL_ROWS + lane;
+    int32_t v[32];
+#pragma unroll
+    for (int u = 0; u < 32; ++u) v[u] = r0 + 32 * u < K ? __ldg(tb + (int64_t)(r0 + 32 * u) * nq) : INT32_MIN;
+    unsigned long long prev = ~0ull;
+    for (int j = 0; j < P; ++j) {
+        // the lane's largest key below the one before: the largest score, the first row of it
+        unsigned long long best = 0ull;
+#pragma unroll
+        for (int u = 0; u < 32; ++u) {
+            const unsigned long long k = r0 + 32 * u < K ? key_int(v[u], r0 + 32 * u) : 0ull;
+            if (k < prev && k > best) best = k;
+        }
+        prev = warp_max(best);
+        if (lane == 0) best_of[warp * P + j] = prev;
+    }
+    __syncthreads();
+    if (warp != 0) return;
+    int32_t my_id = 0;
+    prev = ~0ull;
+    for (int j = 0; j < P; ++j) {
+        unsigned long long best = 0ull;
+        for (int k = lane; k < warps * P; k += 32) {
+            const unsigned long long x = best_of[k];
+            if (x < prev && x > best) best = x;
+        }
+        prev = warp_max(best);
+        if (lane == j) my_id = key_id(prev);
+    }
+    if (lane < P) probes[((int64_t)b * nq + col) * P + lane] = my_id;
+}
+
+int launch_probes(const Index &ix, const Params &p, const Layout &L, const int32_t *table, unsigned long long *part,
+                  int32_t *probes, int32_t *done, cudaStream_t st)
+{
+    // tables below the sizes of the joint form (a column's rows are a sector each: up to 64 MB of sectors in all)
+    if (L.pq_stride == 0 && p.P <= 32 && ix.K <= 32 * PROBE_COL_ROWS && (double)p.B * p.nq * (double)ix.K <= 2e6) {
+        const unsigned warps = (unsigned)((ix.K + PROBE_COL_ROWS - 1) / PROBE_COL_ROWS);
+        launch(probe_column_kernel, dim3((unsigned)p.nq, (unsigned)p.B), 32 * warps, sizeof(unsigned long long) * warps * p.P, st,
+               table, ix.K, p.nq, p.P, probes);
+        CHIMERA_CUDA(cudaGetLastError());
+        count_launch(SLOT_PROBE);
+        return CHIMERA_OK;
+    }
     const size_t smem = sizeof(unsigned long long) * (size_t)p.P * PROBE_THREADS;
     if (smem > 48 * 1024)
         CHIMERA_CUDA(cudaFuncSetAttribute(probe_partial, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const int rows_per_block = (int)((ix.K + L.probe_blocks - 1) / L.probe_blocks);
     const unsigned col_groups = (unsigned)((p.nq + 31) / 32);
     dim3 g1((unsigned)L.probe_blocks, (unsigned)p.B, col_groups);
-    probe_partial<<<g1, PROBE_THREADS, smem, st>>>(table, ix.K, p.nq, p.P, rows_per_block, L.n_part, part, nullptr);
+    launch(probe_partial, g1, PROBE_THREADS, smem, st, table, ix.K, p.nq, p.P, rows_per_block, L.n_part, part, nullptr,
+           done, probes);
     CHIMERA_CUDA(cudaGetLastError());
-    const int rc = launch_probe_final(part, p.B, p.nq, p.P, L.n_part, probes, st);
-    if (rc) return rc;
-    count_launch(SLOT_PROBE, 2);
+    if (!done) {
+        const int rc = launch_probe_final(part, p.B, p.nq, p.P, L.n_part, probes, st);
+        if (rc) return rc;
+    }
+    count_launch(SLOT_PROBE, done ? 1 : 2);
     return CHIMERA_OK;
 }
 
@@ -237,6 +312,7 @@ __global__ void __launch_bounds__(32 * PQ_WARPS)
 sample_max_kernel(const int32_t *__restrict__ table, int64_t K, int nq, int64_t sample_rows, int stride, int G,
                   int rows_per_group, int32_t *__restrict__ gmax)
 {
+    pdl_entry();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int col = blockIdx.z * 32 + lane;
     const int b = blockIdx.y;
@@ -267,6 +343,7 @@ __global__ void __launch_bounds__(32 * PQ_WARPS)
 sample_bound_kernel(const int32_t *__restrict__ gmax, int G, int nq, int P, int64_t rows, int32_t *__restrict__ thr,
                     int32_t *__restrict__ cnt, int32_t *__restrict__ ovf)
 {
+    pdl_entry();
     const int lane = threadIdx.x & 31;
     const int64_t row = (int64_t)blockIdx.x * PQ_WARPS + (threadIdx.x >> 5);
     if (row >= rows) return;
@@ -306,6 +383,7 @@ sample_push_kernel(const int32_t *__restrict__ table, int64_t K, int nq, int64_t
                    int rows_per_group, const int32_t *__restrict__ thr, int32_t *__restrict__ cnt,
                    unsigned long long *__restrict__ keys, int cap)
 {
+    pdl_entry();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int col = blockIdx.z * 32 + lane;
     const int b = blockIdx.y;
@@ -342,6 +420,7 @@ probe_merge_kernel(int nq, int P, int64_t rows, const int32_t *__restrict__ cnt,
                    const unsigned long long *__restrict__ keys, int cap, int32_t *__restrict__ probes,
                    int32_t *__restrict__ ovf)
 {
+    pdl_entry();
     const int lane = threadIdx.x & 31;
     const int64_t row = (int64_t)blockIdx.x * PQ_WARPS + (threadIdx.x >> 5);
     if (row >= rows) return;
@@ -381,13 +460,13 @@ int launch_probe_sample(const Index &ix, const Params &p, const Layout &L, const
     int32_t *ovf = (int32_t *)(ws + L.pq_ovf);
     unsigned long long *keys = (unsigned long long *)(ws + L.pq_keys);
     const dim3 grid((unsigned)((G + PQ_WARPS - 1) / PQ_WARPS), (unsigned)p.B, (unsigned)((p.nq + 31) / 32));
-    sample_max_kernel<<<grid, 32 * PQ_WARPS, 0, st>>>(table, ix.K, p.nq, sample_rows, L.pq_stride, G, rows_per_group,
+    launch(sample_max_kernel, grid, 32 * PQ_WARPS, 0, st, table, ix.K, p.nq, sample_rows, L.pq_stride, G, rows_per_group,
                                                       gmax);
     CHIMERA_CUDA(cudaGetLastError());
-    sample_bound_kernel<<<(unsigned)((rows + PQ_WARPS - 1) / PQ_WARPS), 32 * PQ_WARPS, 0, st>>>(gmax, G, p.nq, p.P, rows,
+    launch(sample_bound_kernel, (unsigned)((rows + PQ_WARPS - 1) / PQ_WARPS), 32 * PQ_WARPS, 0, st, gmax, G, p.nq, p.P, rows,
                                                                                                 thr, cnt, ovf);
     CHIMERA_CUDA(cudaGetLastError());
-    sample_push_kernel<<<grid, 32 * PQ_WARPS, 0, st>>>(table, ix.K, p.nq, sample_rows, L.pq_stride, G, rows_per_group,
+    launch(sample_push_kernel, grid, 32 * PQ_WARPS, 0, st, table, ix.K, p.nq, sample_rows, L.pq_stride, G, rows_per_group,
                                                        thr, cnt, keys, L.pq_cap);
     CHIMERA_CUDA(cudaGetLastError());
     count_launch(SLOT_PROBE, 3);
@@ -402,7 +481,7 @@ int launch_probe_merge(const Index &ix, const Params &p, const Layout &L, const 
     int32_t *ovf = (int32_t *)(ws + L.pq_ovf);
     unsigned long long *part = (unsigned long long *)(ws + L.part);
     int32_t *probes = (int32_t *)(ws + L.probes);
-    probe_merge_kernel<<<(unsigned)((rows + PQ_WARPS - 1) / PQ_WARPS), 32 * PQ_WARPS, 0, st>>>(p.nq, p.P, rows, cnt, keys,
+    launch(probe_merge_kernel, (unsigned)((rows + PQ_WARPS - 1) / PQ_WARPS), 32 * PQ_WARPS, 0, st, p.nq, p.P, rows, cnt, keys,
                                                                                                L.pq_cap, probes, ovf);
     CHIMERA_CUDA(cudaGetLastError());
     // queries with an overflowed queue (none, except for inputs with masses of equal scores): the table scan, whose
@@ -412,8 +491,7 @@ int launch_probe_merge(const Index &ix, const Params &p, const Layout &L, const 
         CHIMERA_CUDA(cudaFuncSetAttribute(probe_partial, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const int rows_per_block = (int)((ix.K + L.probe_blocks - 1) / L.probe_blocks);
     const unsigned col_groups = (unsigned)((p.nq + 31) / 32);
-    probe_partial<<<dim3((unsigned)L.probe_blocks, (unsigned)p.B, col_groups), PROBE_THREADS, smem, st>>>(
-        table, ix.K, p.nq, p.P, rows_per_block, L.n_part, part, ovf);
+    launch(probe_partial, dim3((unsigned)L.probe_blocks, (unsigned)p.B, col_groups), PROBE_THREADS, smem, st, table, ix.K, p.nq, p.P, rows_per_block, L.n_part, part, ovf, nullptr, probes);
     CHIMERA_CUDA(cudaGetLastError());
     const int rc = launch_probe_final(part, p.B, p.nq, p.P, L.n_part, probes, st, ovf);
     if (rc) return rc;
@@ -497,8 +575,8 @@ extern "C" int chimera_probes_static(const int32_t *score_table, int64_t n_centr
     const unsigned col_groups = (unsigned)((q_len + 31) / 32);
     // probe_partial writes every entry probe_final reads (all n_part lists x nprobe keys x q_len columns), so nothing
     // of the previous call's contents survives into this call's result and nothing needs clearing.
-    probe_partial<<<dim3((unsigned)blocks, (unsigned)n_queries, col_groups), PROBE_THREADS, smem, st>>>(
-        score_table, n_centroids, q_len, nprobe, rows_per_block, n_part, part, nullptr);
+    launch(probe_partial, dim3((unsigned)blocks, (unsigned)n_queries, col_groups), PROBE_THREADS, smem, st, score_table, n_centroids, q_len, nprobe,
+           rows_per_block, n_part, part, nullptr, nullptr, out_probes);
     CHIMERA_CUDA(cudaGetLastError());
     return launch_probe_final(part, n_queries, q_len, nprobe, n_part, out_probes, st);
 }

@@ -37,6 +37,7 @@ ci_kernel(const int32_t *__restrict__ table, int64_t K, int nq, const int32_t *_
           const int32_t *__restrict__ n_cand, int64_t maxc, const int32_t *__restrict__ cids,
           const int64_t *__restrict__ doc_off, const int2 *__restrict__ rng, int32_t *__restrict__ ci)
 {
+    pdl_entry();
     const int b = blockIdx.y;
     const int lane = threadIdx.x & 31;
     const int n = n_cand[b];
@@ -104,6 +105,7 @@ ci_wide_kernel(const int32_t *__restrict__ table, int64_t K, const int32_t *__re
                const int32_t *__restrict__ n_cand, int64_t maxc, const int32_t *__restrict__ cids,
                const int64_t *__restrict__ doc_off, int32_t *__restrict__ ci)
 {
+    pdl_entry();
     constexpr int NQ = 4 * LPR;
     constexpr int TPL = 32 / LPR;                 // tokens per warp-wide load
     constexpr int UNROLL = 8;
@@ -167,6 +169,7 @@ ci_wide_rng_kernel(const int32_t *__restrict__ table, int64_t K, const int2 *__r
                    const int32_t *__restrict__ n_docs, int64_t maxc, const int32_t *__restrict__ cids,
                    int32_t *__restrict__ ci)
 {
+    pdl_entry();
     constexpr int NQ = 4 * LPR;
     constexpr int TPL = 32 / LPR;                 // tokens per warp-wide load
     constexpr int UNROLL = 8;
@@ -293,6 +296,7 @@ ci_coarse_kernel(const uint8_t *__restrict__ table8, int64_t K, const int32_t *_
                  const int32_t *__restrict__ n_cand, int64_t maxc, const int32_t *__restrict__ cids,
                  const int64_t *__restrict__ doc_off, int32_t *__restrict__ lo, int32_t *__restrict__ hi)
 {
+    pdl_entry();
     extern __shared__ int4 smem_table[];
     constexpr int WARPS = THREADS / 32;
     constexpr int NQ = 16 * LPR;
@@ -408,9 +412,13 @@ ci_coarse_kernel(const uint8_t *__restrict__ table8, int64_t K, const int32_t *_
 // tokens with one coalesced load per 32 documents instead of the dependent chain id -> offsets per document.
 __global__ void __launch_bounds__(256)
 cand_range_kernel(const int32_t *__restrict__ cand, const int32_t *__restrict__ n_cand, int64_t maxc,
-                  const int64_t *__restrict__ doc_off, int2 *__restrict__ rng)
+                  const int64_t *__restrict__ doc_off, int2 *__restrict__ rng, int32_t *__restrict__ cont_hist)
 {
+    pdl_entry();
     const int b = blockIdx.y;
+    if (cont_hist)                                        // the contender step's histogram (at the head of its scratch row)
+        for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < CONT_BINS; i += gridDim.x * blockDim.x)
+            cont_hist[(int64_t)b * maxc + i] = 0;
     const int n = n_cand[b];
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
         const int64_t d = DBG_DOC(cand[(int64_t)b * maxc + j]);
@@ -567,6 +575,7 @@ ci_coarse_rng_kernel(const uint8_t *__restrict__ table8, int64_t K, const int2 *
                      const int32_t *__restrict__ n_cand, int64_t maxc, const int32_t *__restrict__ cids,
                      int32_t *__restrict__ lo, int32_t *__restrict__ hi)
 {
+    pdl_entry();
     ci_coarse_rng_body<LPR>(table8, K, rng, n_cand, maxc, cids, lo, hi);
 }
 template <int LPR>
@@ -575,19 +584,26 @@ ci_coarse_rng_kernel_b4(const uint8_t *__restrict__ table8, int64_t K, const int
                         const int32_t *__restrict__ n_cand, int64_t maxc, const int32_t *__restrict__ cids,
                         int32_t *__restrict__ lo, int32_t *__restrict__ hi)
 {
+    pdl_entry();
     ci_coarse_rng_body<LPR>(table8, K, rng, n_cand, maxc, cids, lo, hi);
 }
 
 bool coarse_supported(int nq) { return nq == 32 || nq == 64; }
 
+// Several blocks per query in the contender step: few queries with long candidate lists (one block reads 100,000 candidates
+// in about 40 us, and 16,384 in the time of the two more launches).
+int contender_hist_entries() { return CONT_BINS; }
+bool contenders_split(const Index &ix, const Params &p) { return 4 * p.B <= ix.sm_count && p.maxc > 16384; }
+
 int launch_cand_ranges(const Index &ix, const Params &p, const int32_t *cand, const int32_t *n_cand, int2 *rng,
-                       cudaStream_t st)
+                       int32_t *cont_hist, cudaStream_t st)
 {
     int64_t rb = ((int64_t)ix.sm_count * 8 + p.B - 1) / p.B;
     const int64_t rwant = (p.maxc + 255) / 256;
     if (rb > rwant) rb = rwant;
     if (rb < 1) rb = 1;
-    cand_range_kernel<<<dim3((unsigned)rb, (unsigned)p.B), 256, 0, st>>>(cand, n_cand, p.maxc, ix.doc_off, rng);
+    launch(cand_range_kernel, dim3((unsigned)rb, (unsigned)p.B), 256, 0, st, cand, n_cand, p.maxc, ix.doc_off, rng,
+           contenders_split(ix, p) ? cont_hist : nullptr);
     CHIMERA_CUDA(cudaGetLastError());
     count_launch(SLOT_CI);
     return CHIMERA_OK;
@@ -604,18 +620,20 @@ int launch_coarse_bounds(const Index &ix, const Params &p, const uint8_t *table8
         int64_t gx = (4LL * ix.sm_count + p.B - 1) / p.B;       // every block re-reads the table: few, long blocks
         int64_t want = (p.maxc + T / 32 - 1) / (T / 32);
         if (gx > want) gx = want;
-        if (gx > 64) gx = 64;
+        if (4 * p.B <= ix.sm_count) gx = (ix.sm_count + p.B - 1) / p.B;        // few queries: a block per SM
+        else if (gx > 64) gx = 64;
+        if (gx > want) gx = want;
         if (gx < 1) gx = 1;
         dim3 grid((unsigned)gx, (unsigned)p.B);
         if (p.nq == 32) {
             CHIMERA_CUDA(cudaFuncSetAttribute(ci_coarse_kernel<2, true, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)table_bytes));
-            ci_coarse_kernel<2, true, T><<<grid, T, table_bytes, st>>>(table8, ix.K, cand, n_cand, p.maxc, ix.cids,
+            launch(ci_coarse_kernel<2, true, T>, grid, T, table_bytes, st, table8, ix.K, cand, n_cand, p.maxc, ix.cids,
                                                                        ix.doc_off, lo, hi);
         } else {
             CHIMERA_CUDA(cudaFuncSetAttribute(ci_coarse_kernel<4, true, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)table_bytes));
-            ci_coarse_kernel<4, true, T><<<grid, T, table_bytes, st>>>(table8, ix.K, cand, n_cand, p.maxc, ix.cids,
+            launch(ci_coarse_kernel<4, true, T>, grid, T, table_bytes, st, table8, ix.K, cand, n_cand, p.maxc, ix.cids,
                                                                        ix.doc_off, lo, hi);
         }
         CHIMERA_CUDA(cudaGetLastError());
@@ -640,18 +658,18 @@ int launch_coarse_bounds(const Index &ix, const Params &p, const uint8_t *table8
     dim3 grid(gx, (unsigned)p.B);
     if (use_rng) {
         if (p.nq == 32)
-            ci_coarse_rng_kernel<2><<<grid, CI_THREADS, 0, st>>>(table8, ix.K, rng, n_cand, p.maxc, ix.cids, lo, hi);
+            launch(ci_coarse_rng_kernel<2>, grid, CI_THREADS, 0, st, table8, ix.K, rng, n_cand, p.maxc, ix.cids, lo, hi);
         else
-            ci_coarse_rng_kernel_b4<4><<<grid, CI_THREADS, 0, st>>>(table8, ix.K, rng, n_cand, p.maxc, ix.cids, lo, hi);
+            launch(ci_coarse_rng_kernel_b4<4>, grid, CI_THREADS, 0, st, table8, ix.K, rng, n_cand, p.maxc, ix.cids, lo, hi);
         CHIMERA_CUDA(cudaGetLastError());
         count_launch(SLOT_CI);
         return CHIMERA_OK;
     }
     if (p.nq == 32)
-        ci_coarse_kernel<2, false, CI_THREADS><<<grid, CI_THREADS, 0, st>>>(table8, ix.K, cand, n_cand, p.maxc, ix.cids,
+        launch(ci_coarse_kernel<2, false, CI_THREADS>, grid, CI_THREADS, 0, st, table8, ix.K, cand, n_cand, p.maxc, ix.cids,
                                                                           ix.doc_off, lo, hi);
     else
-        ci_coarse_kernel<4, false, CI_THREADS><<<grid, CI_THREADS, 0, st>>>(table8, ix.K, cand, n_cand, p.maxc, ix.cids,
+        launch(ci_coarse_kernel<4, false, CI_THREADS>, grid, CI_THREADS, 0, st, table8, ix.K, cand, n_cand, p.maxc, ix.cids,
                                                                           ix.doc_off, lo, hi);
     CHIMERA_CUDA(cudaGetLastError());
     count_launch(SLOT_CI);
@@ -661,6 +679,7 @@ int launch_coarse_bounds(const Index &ix, const Params &p, const uint8_t *table8
 // table [rows] int32 -> table8 [rows] uint8 (only needed when stage 1 did not run in this call).
 __global__ void coarse_table_kernel(const int32_t *__restrict__ table, int64_t n, uint8_t *__restrict__ table8)
 {
+    pdl_entry();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) {
         const int v = table[i] >> 16;
@@ -670,7 +689,7 @@ __global__ void coarse_table_kernel(const int32_t *__restrict__ table, int64_t n
 int launch_coarse_table(const Index &ix, const Params &p, const int32_t *table, uint8_t *table8, cudaStream_t st)
 {
     const int64_t n = (int64_t)p.B * ix.K * p.nq;
-    coarse_table_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(table, n, table8);
+    launch(coarse_table_kernel, (unsigned)((n + 255) / 256), 256, 0, st, table, n, table8);
     CHIMERA_CUDA(cudaGetLastError());
     count_launch(SLOT_MISC);
     return CHIMERA_OK;
@@ -690,23 +709,23 @@ int launch_centroid_interaction(const Index &ix, const Params &p, const int32_t 
     const int2 *grng = blocks_cap > 0 ? rng : nullptr;
     if (rng != nullptr && blocks_cap > 0 && (p.nq == 32 || p.nq == 64)) {       // the listed documents' token ranges are known
         if (p.nq == 32)
-            ci_wide_rng_kernel<8><<<grid, CI_THREADS, 0, st>>>(table, ix.K, rng, n_cand, p.maxc, ix.cids, ci);
+            launch(ci_wide_rng_kernel<8>, grid, CI_THREADS, 0, st, table, ix.K, rng, n_cand, p.maxc, ix.cids, ci);
         else
-            ci_wide_rng_kernel<16><<<grid, CI_THREADS, 0, st>>>(table, ix.K, rng, n_cand, p.maxc, ix.cids, ci);
+            launch(ci_wide_rng_kernel<16>, grid, CI_THREADS, 0, st, table, ix.K, rng, n_cand, p.maxc, ix.cids, ci);
         CHIMERA_CUDA(cudaGetLastError());
         count_launch(slot);
         return CHIMERA_OK;
     }
     if (p.nq == 32)
-        ci_wide_kernel<8><<<grid, CI_THREADS, 0, st>>>(table, ix.K, cand, n_cand, p.maxc, ix.cids, ix.doc_off, ci);
+        launch(ci_wide_kernel<8>, grid, CI_THREADS, 0, st, table, ix.K, cand, n_cand, p.maxc, ix.cids, ix.doc_off, ci);
     else if (p.nq == 64)
-        ci_wide_kernel<16><<<grid, CI_THREADS, 0, st>>>(table, ix.K, cand, n_cand, p.maxc, ix.cids, ix.doc_off, ci);
+        launch(ci_wide_kernel<16>, grid, CI_THREADS, 0, st, table, ix.K, cand, n_cand, p.maxc, ix.cids, ix.doc_off, ci);
     else if (nqw == 1)
-        ci_kernel<1><<<grid, CI_THREADS, 0, st>>>(table, ix.K, p.nq, cand, n_cand, p.maxc, ix.cids, ix.doc_off, grng, ci);
+        launch(ci_kernel<1>, grid, CI_THREADS, 0, st, table, ix.K, p.nq, cand, n_cand, p.maxc, ix.cids, ix.doc_off, grng, ci);
     else if (nqw == 2)
-        ci_kernel<2><<<grid, CI_THREADS, 0, st>>>(table, ix.K, p.nq, cand, n_cand, p.maxc, ix.cids, ix.doc_off, grng, ci);
+        launch(ci_kernel<2>, grid, CI_THREADS, 0, st, table, ix.K, p.nq, cand, n_cand, p.maxc, ix.cids, ix.doc_off, grng, ci);
     else
-        ci_kernel<4><<<grid, CI_THREADS, 0, st>>>(table, ix.K, p.nq, cand, n_cand, p.maxc, ix.cids, ix.doc_off, grng, ci);
+        launch(ci_kernel<4>, grid, CI_THREADS, 0, st, table, ix.K, p.nq, cand, n_cand, p.maxc, ix.cids, ix.doc_off, grng, ci);
     CHIMERA_CUDA(cudaGetLastError());
     count_launch(slot);
     return CHIMERA_OK;
@@ -720,6 +739,7 @@ select_kernel(const int32_t *__restrict__ cand, const int32_t *__restrict__ n_ca
               int64_t maxc, int n_prune, int32_t *__restrict__ pruned, int32_t *__restrict__ n_pruned,
               int32_t *__restrict__ pruned_ci)
 {
+    pdl_entry();
     __shared__ int hist[2048];
     __shared__ int warp_part[32];
     __shared__ uint32_t s_prefix;
@@ -794,6 +814,7 @@ contender_kernel(const int32_t *__restrict__ cand, const int32_t *__restrict__ n
                  const int32_t *__restrict__ hi, int64_t maxc, int n_prune, int nq, int32_t *__restrict__ cont,
                  int32_t *__restrict__ n_cont, const int2 *__restrict__ rng, int2 *__restrict__ cont_rng)
 {
+    pdl_entry();
     __shared__ int hist[CONT_BINS];
     __shared__ int warp_part[32];
     __shared__ int s_bin;
@@ -882,6 +903,7 @@ shard_select_kernel(const int32_t *__restrict__ all_ids, const int32_t *__restri
                     int n_prune, long long doc_base, long long n_local, int32_t *__restrict__ pruned,
                     int32_t *__restrict__ n_pruned)
 {
+    pdl_entry();
     __shared__ int hist[2048];
     __shared__ int warp_part[32];
     __shared__ uint32_t s_prefix;
@@ -947,7 +969,7 @@ shard_select_kernel(const int32_t *__restrict__ all_ids, const int32_t *__restri
 int launch_shard_select(const Params &p, const int32_t *all_ids, const int32_t *all_ci, int world, int64_t doc_base,
                         int64_t n_local, int32_t *pruned, int32_t *n_pruned, cudaStream_t st)
 {
-    shard_select_kernel<<<(unsigned)p.B, SEL_THREADS, 0, st>>>(all_ids, all_ci, world, p.B, p.n_prune,
+    launch(shard_select_kernel, (unsigned)p.B, SEL_THREADS, 0, st, all_ids, all_ci, world, p.B, p.n_prune,
                                                                (long long)doc_base, (long long)n_local, pruned,
                                                                n_pruned);
     CHIMERA_CUDA(cudaGetLastError());
@@ -973,6 +995,7 @@ __global__ void __launch_bounds__(SEL_THREADS)
 contender_hist_kernel(const int32_t *__restrict__ n_cand, const int32_t *__restrict__ lo, int64_t maxc, int n_prune,
                       int nq, int32_t *__restrict__ scratch)
 {
+    pdl_entry();
     __shared__ int hist[CONT_BINS];
     const int b = blockIdx.y, n = n_cand[b];
     if (n <= n_prune) return;                          // everything is a contender: no threshold needed
@@ -994,6 +1017,7 @@ __global__ void __launch_bounds__(SEL_THREADS)
 contender_count_kernel(const int32_t *__restrict__ n_cand, const int32_t *__restrict__ hi, int64_t maxc, int n_prune,
                        int nq, int32_t *__restrict__ scratch)
 {
+    pdl_entry();
     __shared__ int warp_part[32];
     __shared__ int s_bin;
     const int b = blockIdx.y, n = n_cand[b];
@@ -1037,6 +1061,7 @@ contender_write_kernel(const int32_t *__restrict__ cand, const int32_t *__restri
                        int32_t *__restrict__ cont, int32_t *__restrict__ n_cont, const int2 *__restrict__ rng,
                        int2 *__restrict__ cont_rng)
 {
+    pdl_entry();
     __shared__ int warp_part[32];
     const int b = blockIdx.y, n = n_cand[b], g = blockIdx.x;
     const int32_t *gh = scratch + (int64_t)b * maxc;
@@ -1078,21 +1103,19 @@ int launch_contenders(const Index &ix, const Params &p, const int32_t *cand, con
                       const int32_t *hi, int32_t *cont, int32_t *n_cont, int32_t *scratch, const int2 *rng,
                       int2 *cont_rng, cudaStream_t st)
 {
-    if (4 * p.B <= ix.sm_count && p.maxc >= CONT_BINS + CONT_SPLIT + 1) {
-        // few queries: CONT_SPLIT blocks each
-        CHIMERA_CUDA(cudaMemset2DAsync(scratch, sizeof(int32_t) * (size_t)p.maxc, 0, sizeof(int32_t) * CONT_BINS,
-                                       (size_t)p.B, st));
+    if (rng != nullptr && contenders_split(ix, p)) {
+        // few queries: CONT_SPLIT blocks each (the kernel that wrote the ranges has cleared the histograms)
         const dim3 grid(CONT_SPLIT, (unsigned)p.B);
-        contender_hist_kernel<<<grid, SEL_THREADS, 0, st>>>(n_cand, lo, p.maxc, p.n_prune, p.nq, scratch);
+        launch(contender_hist_kernel, grid, SEL_THREADS, 0, st, n_cand, lo, p.maxc, p.n_prune, p.nq, scratch);
         CHIMERA_CUDA(cudaGetLastError());
-        contender_count_kernel<<<grid, SEL_THREADS, 0, st>>>(n_cand, hi, p.maxc, p.n_prune, p.nq, scratch);
+        launch(contender_count_kernel, grid, SEL_THREADS, 0, st, n_cand, hi, p.maxc, p.n_prune, p.nq, scratch);
         CHIMERA_CUDA(cudaGetLastError());
-        contender_write_kernel<<<grid, SEL_THREADS, 0, st>>>(cand, n_cand, hi, p.maxc, scratch, cont, n_cont, rng, cont_rng);
+        launch(contender_write_kernel, grid, SEL_THREADS, 0, st, cand, n_cand, hi, p.maxc, scratch, cont, n_cont, rng, cont_rng);
         CHIMERA_CUDA(cudaGetLastError());
         count_launch(SLOT_SELECT, 3);
         return CHIMERA_OK;
     }
-    contender_kernel<<<(unsigned)p.B, SEL_THREADS, 0, st>>>(cand, n_cand, lo, hi, p.maxc, p.n_prune, p.nq, cont,
+    launch(contender_kernel, (unsigned)p.B, SEL_THREADS, 0, st, cand, n_cand, lo, hi, p.maxc, p.n_prune, p.nq, cont,
                                                             n_cont, rng, cont_rng);
     CHIMERA_CUDA(cudaGetLastError());
     count_launch(SLOT_SELECT);
@@ -1142,6 +1165,7 @@ __global__ void __launch_bounds__(SEL_THREADS)
 sels_hist_kernel(const int32_t *__restrict__ n_cand, const int32_t *__restrict__ ci, int64_t maxc, int n_prune,
                  int32_t *__restrict__ scratch)
 {
+    pdl_entry();
     __shared__ int hist[2048];
     __shared__ int warp_part[32];
     __shared__ int s_out[2];
@@ -1194,6 +1218,7 @@ __global__ void __launch_bounds__(SEL_THREADS)
 sels_count_kernel(const int32_t *__restrict__ n_cand, const int32_t *__restrict__ ci, int64_t maxc, int n_prune,
                   int32_t *__restrict__ scratch)
 {
+    pdl_entry();
     __shared__ int warp_part[32];
     __shared__ int s_out[2];
     const int b = blockIdx.y, n = n_cand[b];
@@ -1223,6 +1248,7 @@ sels_write_kernel(const int32_t *__restrict__ cand, const int32_t *__restrict__ 
                   int64_t maxc, int n_prune, const int32_t *__restrict__ scratch, int32_t *__restrict__ pruned,
                   int32_t *__restrict__ n_pruned, int32_t *__restrict__ pruned_ci)
 {
+    pdl_entry();
     __shared__ int warp_part[32];
     __shared__ int s_out[2];
     const int b = blockIdx.y, n = n_cand[b], g = blockIdx.x;
@@ -1306,17 +1332,17 @@ int launch_select(const Index &ix, const Params &p, const int32_t *cand, const i
     if (scratch != nullptr && select_split_used(ix, p) && p.maxc >= 16384 && p.maxc < (int64_t)SELS_SPLIT * 32767) {
         CHIMERA_CUDA(cudaMemsetAsync(scratch, 0, select_split_scratch_bytes(ix, p), st));
         const dim3 grid(SELS_SPLIT, (unsigned)p.B);
-        sels_hist_kernel<0><<<grid, SEL_THREADS, 0, st>>>(n_cand, ci, p.maxc, p.n_prune, scratch);
-        sels_hist_kernel<1><<<grid, SEL_THREADS, 0, st>>>(n_cand, ci, p.maxc, p.n_prune, scratch);
-        sels_hist_kernel<2><<<grid, SEL_THREADS, 0, st>>>(n_cand, ci, p.maxc, p.n_prune, scratch);
-        sels_count_kernel<<<grid, SEL_THREADS, 0, st>>>(n_cand, ci, p.maxc, p.n_prune, scratch);
-        sels_write_kernel<<<grid, SEL_THREADS, 0, st>>>(cand, n_cand, ci, p.maxc, p.n_prune, scratch, pruned, n_pruned,
+        launch(sels_hist_kernel<0>, grid, SEL_THREADS, 0, st, n_cand, ci, p.maxc, p.n_prune, scratch);
+        launch(sels_hist_kernel<1>, grid, SEL_THREADS, 0, st, n_cand, ci, p.maxc, p.n_prune, scratch);
+        launch(sels_hist_kernel<2>, grid, SEL_THREADS, 0, st, n_cand, ci, p.maxc, p.n_prune, scratch);
+        launch(sels_count_kernel, grid, SEL_THREADS, 0, st, n_cand, ci, p.maxc, p.n_prune, scratch);
+        launch(sels_write_kernel, grid, SEL_THREADS, 0, st, cand, n_cand, ci, p.maxc, p.n_prune, scratch, pruned, n_pruned,
                                                         pruned_ci);
         CHIMERA_CUDA(cudaGetLastError());
         count_launch(SLOT_SELECT, 5);
         return CHIMERA_OK;
     }
-    select_kernel<<<(unsigned)p.B, SEL_THREADS, 0, st>>>(cand, n_cand, ci, p.maxc, p.n_prune, pruned, n_pruned,
+    launch(select_kernel, (unsigned)p.B, SEL_THREADS, 0, st, cand, n_cand, ci, p.maxc, p.n_prune, pruned, n_pruned,
                                                          pruned_ci);
     CHIMERA_CUDA(cudaGetLastError());
     count_launch(SLOT_SELECT);

@@ -99,6 +99,7 @@ filter_theta_kernel(const int32_t *__restrict__ table, int64_t K, int nq, int m,
                     int32_t *__restrict__ theta, int32_t *__restrict__ hist_out, int32_t *__restrict__ n_seed,
                     int32_t *__restrict__ parts_hist, int32_t *__restrict__ done)
 {
+    pdl_entry();
     __shared__ int hist[256 * 32];
     __shared__ int s_last;
     const int b = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -209,6 +210,7 @@ __global__ void __launch_bounds__(256)
 filter_excess_kernel(const uint8_t *__restrict__ table8, int64_t K, const int32_t *__restrict__ theta,
                      uint8_t *__restrict__ out, size_t pitch)
 {
+    pdl_entry();
     __shared__ uint2 tm1[WORDS];
     __shared__ int s_sum;
     __shared__ uint8_t enc[512];
@@ -252,6 +254,7 @@ __global__ void __launch_bounds__(256)
 filter_excess_exact_kernel(const int32_t *__restrict__ table, int64_t K, int nq, const int32_t *__restrict__ theta, int us,
                            uint8_t *__restrict__ out, size_t pitch)
 {
+    pdl_entry();
     __shared__ uint8_t enc[512];
     if (CODEC == 6) filter_fill_encoder(enc);
     const int b = blockIdx.y, lane = threadIdx.x & 31;
@@ -315,6 +318,7 @@ filter_scan_kernel(const uint8_t *__restrict__ tab, size_t pitch, const int32_t 
                    const int32_t *__restrict__ n_cand, int64_t maxc, const int32_t *__restrict__ cids, int64_t T,
                    int32_t *__restrict__ hi0, int32_t *__restrict__ hist)
 {
+    pdl_entry();
     extern __shared__ uint4 s_tab[];
     __shared__ uint32_t s_level[64];
     __shared__ int s_hist[FILTER_BINS];
@@ -465,14 +469,6 @@ filter_scan_kernel(const uint8_t *__restrict__ tab, size_t pitch, const int32_t 
 }
 
 // ------------------------------------------------------------------------------------------------ seeds -----------
-// (first token, length) of a document.
-__device__ __forceinline__ int2 filter_range(const int64_t *doc_off, int32_t d)
-{
-    d = DBG_DOC(d);
-    const int64_t t0 = __ldg(doc_off + d);
-    return make_int2((int)t0, (int)(__ldg(doc_off + d + 1) - t0));
-}
-
 // A Q.24 threshold in units of 2^us, rounded up (hi0 is a whole number of them).
 __device__ __forceinline__ int32_t units_up(int32_t tau, int us) { return (int32_t)(((long long)tau + (1 << us) - 1) >> us); }
 
@@ -487,6 +483,7 @@ filter_seed_kernel(const int32_t *__restrict__ cand, const int32_t *__restrict__
                    int2 *__restrict__ seed_rng, int32_t *__restrict__ n_seed, int32_t *__restrict__ seed_thr,
                    int32_t *__restrict__ seed_slot)
 {
+    pdl_entry();
     __shared__ int warp_part[32];
     __shared__ int s_bin, s_theta;
     const int b = blockIdx.y, n = n_cand[b];
@@ -549,7 +546,7 @@ filter_seed_kernel(const int32_t *__restrict__ cand, const int32_t *__restrict__
                 const int64_t o = (int64_t)b * maxc + at + __popc(mask[u] & ((1u << lane) - 1));
                 seed[o] = d;
                 seed_slot[(int64_t)b * maxc + base + u * SEL_THREADS + lane] = (int32_t)(o - (int64_t)b * maxc);
-                seed_rng[o] = filter_range(doc_off, d);
+                seed_rng[o] = doc_range(doc_off, d);
             }
             at += __popc(mask[u]);
         }
@@ -627,6 +624,7 @@ filter_count_kernel(const int32_t *__restrict__ n_cand, const int32_t *__restric
                     const int32_t *__restrict__ seed_ci, const int32_t *__restrict__ n_seed, int n_prune, int us,
                     int32_t *__restrict__ tau_out, int32_t *__restrict__ counts)
 {
+    pdl_entry();
     __shared__ int hist[2048];
     __shared__ int warp_part[32];
     __shared__ uint32_t s_prefix;
@@ -659,6 +657,7 @@ filter_write_kernel(const int32_t *__restrict__ cand, const int32_t *__restrict_
                     const int32_t *__restrict__ counts, int32_t *__restrict__ kept, int2 *__restrict__ kept_rng,
                     int32_t *__restrict__ n_kept)
 {
+    pdl_entry();
     __shared__ int warp_part[32];
     const int b = blockIdx.y;
     const int64_t row = (int64_t)b * maxc;
@@ -669,7 +668,7 @@ filter_write_kernel(const int32_t *__restrict__ cand, const int32_t *__restrict_
                                   warp_part, [&](int j, int32_t v, int pos) {
         const int32_t d = cand[row + j];
         kept[row + pos] = d;
-        kept_rng[row + pos] = v >= thr ? make_int2(seed_ci[row + seed_slot[row + j]], 0) : filter_range(doc_off, d);
+        kept_rng[row + pos] = v >= thr ? make_int2(seed_ci[row + seed_slot[row + j]], 0) : doc_range(doc_off, d);
     });
     if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) n_kept[b] = run;
 }
@@ -680,6 +679,7 @@ __global__ void __launch_bounds__(SEL_THREADS)
 filter_contend_count_kernel(const int32_t *__restrict__ n_kept, const int32_t *__restrict__ hi, int64_t maxc,
                             const int32_t *__restrict__ tau, int32_t *__restrict__ counts)
 {
+    pdl_entry();
     __shared__ int warp_part[32];
     const int b = blockIdx.y;
     int j0, j1;
@@ -693,6 +693,7 @@ filter_contend_kernel(const int32_t *__restrict__ kept, const int2 *__restrict__
                       const int32_t *__restrict__ counts, int32_t *__restrict__ cont, int2 *__restrict__ cont_rng,
                       int32_t *__restrict__ n_cont)
 {
+    pdl_entry();
     __shared__ int warp_part[32];
     const int b = blockIdx.y;
     const int64_t row = (int64_t)b * maxc;
@@ -736,8 +737,7 @@ int launch_filter_scan(const Index &ix, const Params &p, const Layout &L, const 
     int32_t *parts_hist = (int32_t *)(ws + L.flt_parts), *done = parts_hist + (size_t)p.B * groups * 256 * 32;
     if (parts > 1)
         CHIMERA_CUDA(cudaMemsetAsync(parts_hist, 0, filter_parts_bytes(ix, p), st));
-    filter_theta_kernel<<<dim3(groups, (unsigned)p.B, (unsigned)parts), SEL_THREADS, 0, st>>>(
-        table, ix.K, p.nq, m, step, rank, theta, hist, n_seed, parts_hist, done);
+    launch(filter_theta_kernel, dim3(groups, (unsigned)p.B, (unsigned)parts), SEL_THREADS, 0, st, table, ix.K, p.nq, m, step, rank, theta, hist, n_seed, parts_hist, done);
     CHIMERA_CUDA(cudaGetLastError());
 
     const int us = filter_unit(ix, p, table8 != nullptr);
@@ -746,18 +746,18 @@ int launch_filter_scan(const Index &ix, const Params &p, const Layout &L, const 
         const int64_t want = ((codec == 16 ? ix.K : (ix.K + 4) / 5) + 255) / 256;
         if (gx > want) gx = want;
         const dim3 grid((unsigned)gx, (unsigned)p.B);
-        if (p.nq == 32 && codec == 16) filter_excess_kernel<8, 16><<<grid, 256, 0, st>>>(table8, ix.K, theta, tab, pitch);
-        else if (p.nq == 32) filter_excess_kernel<8, 6><<<grid, 256, 0, st>>>(table8, ix.K, theta, tab, pitch);
-        else if (codec == 16) filter_excess_kernel<16, 16><<<grid, 256, 0, st>>>(table8, ix.K, theta, tab, pitch);
-        else filter_excess_kernel<16, 6><<<grid, 256, 0, st>>>(table8, ix.K, theta, tab, pitch);
+        if (p.nq == 32 && codec == 16) launch(filter_excess_kernel<8, 16>, grid, 256, 0, st, table8, ix.K, theta, tab, pitch);
+        else if (p.nq == 32) launch(filter_excess_kernel<8, 6>, grid, 256, 0, st, table8, ix.K, theta, tab, pitch);
+        else if (codec == 16) launch(filter_excess_kernel<16, 16>, grid, 256, 0, st, table8, ix.K, theta, tab, pitch);
+        else launch(filter_excess_kernel<16, 6>, grid, 256, 0, st, table8, ix.K, theta, tab, pitch);
     } else {
         const int64_t want = (ix.K + 39) / 40;
         if (gx > want) gx = want;
         const dim3 grid((unsigned)gx, (unsigned)p.B);
         if (codec == 16)
-            filter_excess_exact_kernel<16><<<grid, 256, 0, st>>>(table, ix.K, p.nq, theta, us, tab, pitch);
+            launch(filter_excess_exact_kernel<16>, grid, 256, 0, st, table, ix.K, p.nq, theta, us, tab, pitch);
         else
-            filter_excess_exact_kernel<6><<<grid, 256, 0, st>>>(table, ix.K, p.nq, theta, us, tab, pitch);
+            launch(filter_excess_exact_kernel<6>, grid, 256, 0, st, table, ix.K, p.nq, theta, us, tab, pitch);
     }
     CHIMERA_CUDA(cudaGetLastError());
 
@@ -770,16 +770,15 @@ int launch_filter_scan(const Index &ix, const Params &p, const Layout &L, const 
     const dim3 grid((unsigned)gx, (unsigned)p.B);
     if (codec == 16) {
         CHIMERA_CUDA(cudaFuncSetAttribute(filter_scan_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pitch));
-        filter_scan_kernel<16><<<grid, SCAN_THREADS_F, pitch, st>>>(tab, pitch, theta, p.nq, us, cand, ix.doc_off, n_cand, p.maxc,
+        launch(filter_scan_kernel<16>, grid, SCAN_THREADS_F, pitch, st, tab, pitch, theta, p.nq, us, cand, ix.doc_off, n_cand, p.maxc,
                                                                     ix.cids, ix.T, hi0, hist);
     } else {
         CHIMERA_CUDA(cudaFuncSetAttribute(filter_scan_kernel<6>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pitch));
-        filter_scan_kernel<6><<<grid, SCAN_THREADS_F, pitch, st>>>(tab, pitch, theta, p.nq, us, cand, ix.doc_off, n_cand, p.maxc,
+        launch(filter_scan_kernel<6>, grid, SCAN_THREADS_F, pitch, st, tab, pitch, theta, p.nq, us, cand, ix.doc_off, n_cand, p.maxc,
                                                                    ix.cids, ix.T, hi0, hist);
     }
     CHIMERA_CUDA(cudaGetLastError());
-    filter_seed_kernel<<<dim3((unsigned)filter_split(ix, p), (unsigned)p.B), SEL_THREADS, 0, st>>>(
-        cand, n_cand, ix.doc_off, hi0, p.maxc, theta, p.nq, us, hist, p.n_prune, seed, seed_rng, n_seed,
+    launch(filter_seed_kernel, dim3((unsigned)filter_split(ix, p), (unsigned)p.B), SEL_THREADS, 0, st, cand, n_cand, ix.doc_off, hi0, p.maxc, theta, p.nq, us, hist, p.n_prune, seed, seed_rng, n_seed,
         (int32_t *)(ws + L.flt_thr), (int32_t *)(ws + L.flt_slot));
     CHIMERA_CUDA(cudaGetLastError());
     count_launch(SLOT_CI, 4);
@@ -796,9 +795,9 @@ int launch_filter_keep(const Index &ix, const Params &p, const Layout &L, const 
     int32_t *tau = (int32_t *)(ws + L.flt_tau);
     const int32_t *thr = (const int32_t *)(ws + L.flt_thr), *slot = (const int32_t *)(ws + L.flt_slot);
     const dim3 grid((unsigned)filter_split(ix, p), (unsigned)p.B);
-    filter_count_kernel<<<grid, SEL_THREADS, 0, st>>>(n_cand, hi0, p.maxc, seed_ci, n_seed, p.n_prune, us, tau, counts);
+    launch(filter_count_kernel, grid, SEL_THREADS, 0, st, n_cand, hi0, p.maxc, seed_ci, n_seed, p.n_prune, us, tau, counts);
     CHIMERA_CUDA(cudaGetLastError());
-    filter_write_kernel<<<grid, SEL_THREADS, 0, st>>>(cand, n_cand, ix.doc_off, hi0, p.maxc, thr, slot, seed_ci, tau, us,
+    launch(filter_write_kernel, grid, SEL_THREADS, 0, st, cand, n_cand, ix.doc_off, hi0, p.maxc, thr, slot, seed_ci, tau, us,
                                                       counts, kept, kept_rng, n_kept);
     CHIMERA_CUDA(cudaGetLastError());
     count_launch(SLOT_SELECT, 2);
@@ -815,11 +814,11 @@ int launch_filter_contenders(const Index &ix, const Params &p, const Layout &L, 
     const int split = 4 * p.B <= ix.sm_count ? filter_split(ix, p) : 1;
     const dim3 grid((unsigned)split, (unsigned)p.B);
     if (split > 1) {
-        filter_contend_count_kernel<<<grid, SEL_THREADS, 0, st>>>(n_kept, hi, p.maxc, tau, counts);
+        launch(filter_contend_count_kernel, grid, SEL_THREADS, 0, st, n_kept, hi, p.maxc, tau, counts);
         CHIMERA_CUDA(cudaGetLastError());
         count_launch(SLOT_SELECT);
     }
-    filter_contend_kernel<<<grid, SEL_THREADS, 0, st>>>(kept, kept_rng, n_kept, hi, p.maxc, tau, counts, cont, cont_rng,
+    launch(filter_contend_kernel, grid, SEL_THREADS, 0, st, kept, kept_rng, n_kept, hi, p.maxc, tau, counts, cont, cont_rng,
                                                         n_cont);
     CHIMERA_CUDA(cudaGetLastError());
     count_launch(SLOT_SELECT);

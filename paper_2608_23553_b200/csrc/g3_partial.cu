@@ -45,6 +45,7 @@ int refine_splits(const Index &ix, const Params &p)
 __global__ void __launch_bounds__(256)
 visit_clear_kernel(int32_t *__restrict__ head, const int32_t *__restrict__ n_cand, int64_t maxc)
 {
+    pdl_entry();
     const int b = blockIdx.y, n = n_cand[b];
     for (int e = blockIdx.x * 256 + threadIdx.x; e < n; e += gridDim.x * 256) head[(int64_t)b * maxc + e] = 0;
 }
@@ -54,6 +55,7 @@ __global__ void __launch_bounds__(256)
 visit_sum_kernel(const int32_t *__restrict__ head, const unsigned long long *__restrict__ node, int64_t cap,
                  const int32_t *__restrict__ n_cand, int64_t maxc, int32_t *__restrict__ fprime)
 {
+    pdl_entry();
     const int b = blockIdx.y, n = n_cand[b];
     const unsigned long long *nodes = node + (int64_t)b * cap;
     for (int j = blockIdx.x * 256 + threadIdx.x; j < n; j += gridDim.x * 256)
@@ -70,7 +72,7 @@ VisitLists visit_lists(const Params &p, const Layout &L, void *mem)
 int launch_visit_clear(const Index &ix, const Params &p, const VisitLists &v, const int32_t *n_cand, cudaStream_t st)
 {
     int64_t gx = (8LL * ix.sm_count + p.B - 1) / p.B;
-    visit_clear_kernel<<<dim3((unsigned)gx, (unsigned)p.B), 256, 0, st>>>(v.head, n_cand, p.maxc);
+    launch(visit_clear_kernel, dim3((unsigned)gx, (unsigned)p.B), 256, 0, st, v.head, n_cand, p.maxc);
     CHIMERA_CUDA(cudaGetLastError());
     return CHIMERA_OK;
 }
@@ -78,8 +80,8 @@ int launch_visit_sum(const Index &ix, const Params &p, const VisitLists &v, bool
                      int32_t *fprime, cudaStream_t st)
 {
     const dim3 grid((unsigned)((16LL * ix.sm_count + p.B - 1) / p.B), (unsigned)p.B);
-    if (floats) visit_sum_kernel<true><<<grid, 256, 0, st>>>(v.head, v.node, v.cap, n_cand, p.maxc, fprime);
-    else visit_sum_kernel<false><<<grid, 256, 0, st>>>(v.head, v.node, v.cap, n_cand, p.maxc, fprime);
+    if (floats) launch(visit_sum_kernel<true>, grid, 256, 0, st, v.head, v.node, v.cap, n_cand, p.maxc, fprime);
+    else launch(visit_sum_kernel<false>, grid, 256, 0, st, v.head, v.node, v.cap, n_cand, p.maxc, fprime);
     CHIMERA_CUDA(cudaGetLastError());
     return CHIMERA_OK;
 }
@@ -89,6 +91,7 @@ __global__ void __launch_bounds__(256)
 partial_clear_kernel(int32_t *__restrict__ M, int32_t *__restrict__ fprime, const int32_t *__restrict__ n_cand,
                      int64_t maxc, int nq)
 {
+    pdl_entry();
     const int b = blockIdx.y;
     const int64_t n = (int64_t)n_cand[b] * nq;
     int4 *row = reinterpret_cast<int4 *>(M + (int64_t)b * maxc * nq);      // rows are 16-byte aligned when nq % 4 == 0
@@ -114,6 +117,7 @@ partial_score_kernel(const int8_t *__restrict__ qdig, const int32_t *__restrict_
                      const uint2 *__restrict__ ranks, int64_t words, int64_t maxc, int32_t *__restrict__ M,
                      int32_t *__restrict__ fprime, VisitLists lists, int64_t longest, int splits)
 {
+    pdl_entry();
     __shared__ __align__(16) QueryDigits dig;
     const int b = blockIdx.y;
     const int i = blockIdx.x / splits;
@@ -185,7 +189,7 @@ int launch_partial_scores(const Index &ix, const Params &p, const Layout &L, con
         if ((rc = launch_visit_clear(ix, p, lists, n_cand, st))) return rc;
     } else {
         int64_t per_query = ((int64_t)ix.sm_count * 8 + p.B - 1) / p.B;
-        partial_clear_kernel<<<dim3((unsigned)per_query, (unsigned)p.B), 256, 0, st>>>(M, fprime, n_cand, p.maxc, p.nq);
+        launch(partial_clear_kernel, dim3((unsigned)per_query, (unsigned)p.B), 256, 0, st, M, fprime, n_cand, p.maxc, p.nq);
         CHIMERA_CUDA(cudaGetLastError());
     }
     const int splits = refine_splits(ix, p);
@@ -193,7 +197,7 @@ int launch_partial_scores(const Index &ix, const Params &p, const Layout &L, con
     const uint32_t *codes = reinterpret_cast<const uint32_t *>(ix.list_codes ? ix.list_codes : ix.codes);
     const int32_t *ids = ix.list_codes ? nullptr : ix.tok_id;
 #define PS_LAUNCH(NB, LS)                                                                                              \
-    partial_score_kernel<NB, LS><<<grid, PS_THREADS, 0, st>>>(qdig, table, ix.K, p.nq, p.B, ix.CB / 4, p.P, delta, \
+    launch(partial_score_kernel<NB, LS>, grid, PS_THREADS, 0, st, qdig, table, ix.K, p.nq, p.B, ix.CB / 4, p.P, delta, \
                                                               kappa, probes, ix.tok_off, ids, ix.tok_doc, codes, \
                                                               ranks, L.words, p.maxc, M, fprime, lists, ix.max_tok_list, \
                                                               splits)

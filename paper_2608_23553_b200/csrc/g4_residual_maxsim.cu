@@ -25,6 +25,7 @@ residual_maxsim_kernel(const float *__restrict__ queries, const int32_t *__restr
                        const int32_t *__restrict__ cids, const uint32_t *__restrict__ codes,
                        const int64_t *__restrict__ doc_off, float *__restrict__ score4)
 {
+    pdl_entry();
     constexpr int NQP = 4 * CT;
     constexpr int TY = G4_THREADS / CT;       // token rows of the thread grid
     constexpr int TT = 4 * TY;                // document tokens per tile
@@ -157,7 +158,7 @@ static int launch_g4(const Index &ix, const Params &p, const float *queries, con
     if (per_query > p.n_prune) per_query = p.n_prune;
     if (per_query < 1) per_query = 1;
     dim3 grid((unsigned)per_query, (unsigned)p.B);
-    kern<<<grid, G4_THREADS, smem, st>>>(queries, table, ix.K, p.nq, ix.D, ix.CB / 4, delta, kappa, pruned, p.n_prune,
+    launch(kern, grid, G4_THREADS, smem, st, queries, table, ix.K, p.nq, ix.D, ix.CB / 4, delta, kappa, pruned, p.n_prune,
                                          ix.cids, reinterpret_cast<const uint32_t *>(ix.codes), ix.doc_off, score4);
     CHIMERA_CUDA(cudaGetLastError());
     count_launch(SLOT_G4);

@@ -56,6 +56,7 @@ residual_maxsim_umma(const __grid_constant__ CUtensorMap map_q, const float *__r
                      const float *__restrict__ factors, const int64_t *__restrict__ doc_off,
                      float *__restrict__ score4, uint32_t *status, long long wait_limit, int skip_loads)
 {
+    pdl_entry();
     const int nq = FULL ? NQP : nq_arg, D = FULL ? 128 : D_arg, CW = FULL ? (NBITS == 2 ? 8 : 4) : CW_arg;
     constexpr int N = 3 * NQP;                               // MMA N: three digit planes side by side
     constexpr uint32_t TMEM_COLS = N <= 96 ? 128 : 256;
@@ -417,15 +418,18 @@ static int launch_g4_umma(const Index &ix, const Params &p, const float *queries
     auto kern = p.nq == NQP && ix.D == 128 ? residual_maxsim_umma<NQP, NBITS, RQ, true>
                                            : residual_maxsim_umma<NQP, NBITS, RQ, false>;
     CHIMERA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    // documents per CTA: about four CTAs per SM in total, at most 32 documents each (with few queries per call a CTA
-    // gets one or two documents, so that the call's latency is a tile or two and not a chain of them)
-    int64_t dpc = ((int64_t)p.n_prune * p.B + 4LL * ix.sm_count - 1) / (4LL * ix.sm_count);
+    // documents per CTA: whole waves of resident CTAs, as few as documents-per-CTA limit allows (a second wave of a few CTAs
+    // costs as much as a full one: 37 queries of 777 survivors in 2.1 waves of 32 documents, or in three of 22)
+    const int64_t slots = (int64_t)(NQP == 32 ? (RQ ? 4 : 3) : 2) * ix.sm_count, docs = (int64_t)p.n_prune * p.B;
+    const int64_t waves = (docs + slots * G4U_MAX_DOCS - 1) / (slots * G4U_MAX_DOCS);
+    int64_t per_query = waves * slots / p.B;               // CTAs per query
+    if (per_query < 1) per_query = 1;
+    int64_t dpc = (p.n_prune + per_query - 1) / per_query;
     if (dpc < 1) dpc = 1;
     if (dpc > G4U_MAX_DOCS) dpc = G4U_MAX_DOCS;
-    if (dpc > p.n_prune) dpc = p.n_prune;
     dim3 grid((unsigned)((p.n_prune + dpc - 1) / dpc), (unsigned)p.B);
     const uint32_t *code_words = reinterpret_cast<const uint32_t *>(RQ ? ix.rq_bits : ix.codes);
-    kern<<<grid, 128 * (NQP / G4U_COLS), smem, st>>>(map_q, queries, table, ix.K, p.nq, ix.D, RQ ? ix.D / 32 : ix.CB / 4, delta,
+    launch(kern, grid, 128 * (NQP / G4U_COLS), smem, st, map_q, queries, table, ix.K, p.nq, ix.D, RQ ? ix.D / 32 : ix.CB / 4, delta,
                                           kappa, pruned, p.n_prune, (int)dpc, ix.cids, code_words, ix.rq_inv, ix.doc_off,
                                           score4, status, wait_limit_cycles(), fault_skip_tma_loads());
     CHIMERA_CUDA(cudaGetLastError());

@@ -38,6 +38,7 @@ __global__ void __launch_bounds__(TOPK_THREADS)
 topk_kernel(const int32_t *__restrict__ pruned, const float *__restrict__ score4, int n_prune, int n_pow2, int k,
             int seg_len, long long seg_stride, int32_t *__restrict__ out_ids, float *__restrict__ out_scores)
 {
+    pdl_entry();
     extern __shared__ unsigned long long keys[];
     const int b = blockIdx.x;
     for (int j = threadIdx.x; j < n_pow2; j += TOPK_THREADS) {
@@ -80,6 +81,7 @@ __global__ void __launch_bounds__(TOPK_THREADS)
 topk_small_kernel(const int32_t *__restrict__ pruned, const float *__restrict__ score4, int n_prune, int k,
                   int seg_len, long long seg_stride, int32_t *__restrict__ out_ids, float *__restrict__ out_scores)
 {
+    pdl_entry();
     __shared__ unsigned long long warp_max[32];
     __shared__ unsigned long long s_win;
     const int b = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -176,6 +178,7 @@ __global__ void __launch_bounds__(TOPK_THREADS)
 topk_runs_kernel(const int32_t *__restrict__ pruned, const float *__restrict__ score4, int n_prune, int k, int seg_len,
                  long long seg_stride, int32_t *__restrict__ out_ids, float *__restrict__ out_scores)
 {
+    pdl_entry();
     extern __shared__ unsigned long long runs[];           // [32][RUN] then [16][RUN]
     unsigned long long *buf0 = runs, *buf1 = runs + 32 * RUN;
     const int b = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -233,20 +236,19 @@ static int launch_topk_entries(const int32_t *ids, const float *scores, int B, i
 {
     if (k <= 16 && n <= 16 * TOPK_THREADS) {
         if (n <= TOPK_THREADS)
-            topk_small_kernel<1><<<(unsigned)B, TOPK_THREADS, 0, st>>>(ids, scores, n, k, seg_len, seg_stride, out_ids,
+            launch(topk_small_kernel<1>, (unsigned)B, TOPK_THREADS, 0, st, ids, scores, n, k, seg_len, seg_stride, out_ids,
                                                                        out_scores);
         else if (n <= 4 * TOPK_THREADS)
-            topk_small_kernel<4><<<(unsigned)B, TOPK_THREADS, 0, st>>>(ids, scores, n, k, seg_len, seg_stride, out_ids,
+            launch(topk_small_kernel<4>, (unsigned)B, TOPK_THREADS, 0, st, ids, scores, n, k, seg_len, seg_stride, out_ids,
                                                                        out_scores);
         else
-            topk_small_kernel<16><<<(unsigned)B, TOPK_THREADS, 0, st>>>(ids, scores, n, k, seg_len, seg_stride, out_ids,
+            launch(topk_small_kernel<16>, (unsigned)B, TOPK_THREADS, 0, st, ids, scores, n, k, seg_len, seg_stride, out_ids,
                                                                         out_scores);
         CHIMERA_CUDA(cudaGetLastError());
         return CHIMERA_OK;
     }
     if (k <= RUN && n <= 32 * RUN) {
-        topk_runs_kernel<<<(unsigned)B, TOPK_THREADS, sizeof(unsigned long long) * 48 * RUN, st>>>(
-            ids, scores, n, k, seg_len, seg_stride, out_ids, out_scores);
+        launch(topk_runs_kernel, (unsigned)B, TOPK_THREADS, sizeof(unsigned long long) * 48 * RUN, st, ids, scores, n, k, seg_len, seg_stride, out_ids, out_scores);
         CHIMERA_CUDA(cudaGetLastError());
         return CHIMERA_OK;
     }
@@ -256,7 +258,7 @@ static int launch_topk_entries(const int32_t *ids, const float *scores, int B, i
     if (smem > 128 * 1024) return fail(CHIMERA_UNSUPPORTED, "top-k over %d entries per query does not fit shared memory", n);
     if (smem > 48 * 1024)
         CHIMERA_CUDA(cudaFuncSetAttribute(topk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    topk_kernel<<<(unsigned)B, TOPK_THREADS, smem, st>>>(ids, scores, n, n_pow2, k, seg_len, seg_stride, out_ids,
+    launch(topk_kernel, (unsigned)B, TOPK_THREADS, smem, st, ids, scores, n, n_pow2, k, seg_len, seg_stride, out_ids,
                                                          out_scores);
     CHIMERA_CUDA(cudaGetLastError());
     return CHIMERA_OK;

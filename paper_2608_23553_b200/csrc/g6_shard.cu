@@ -11,6 +11,7 @@ namespace chimera {
 __global__ void shard_export_kernel(const int32_t *__restrict__ pruned, const int32_t *__restrict__ pruned_ci, int64_t n,
                                     long long doc_base, int32_t *__restrict__ out_ids, int32_t *__restrict__ out_ci)
 {
+    pdl_entry();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) {
         const int32_t d = pruned[i];
@@ -21,6 +22,7 @@ __global__ void shard_export_kernel(const int32_t *__restrict__ pruned, const in
 
 __global__ void add_base_kernel(int32_t *__restrict__ ids, int64_t n, long long doc_base)
 {
+    pdl_entry();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n && ids[i] >= 0) ids[i] = (int32_t)(ids[i] + doc_base);
 }
@@ -29,7 +31,7 @@ int launch_shard_export(const Params &p, const int32_t *pruned, const int32_t *p
                         int32_t *out_ids, int32_t *out_ci, cudaStream_t st)
 {
     const int64_t n = (int64_t)p.B * p.n_prune;
-    shard_export_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(pruned, pruned_ci, n, (long long)doc_base, out_ids,
+    launch(shard_export_kernel, (unsigned)((n + 255) / 256), 256, 0, st, pruned, pruned_ci, n, (long long)doc_base, out_ids,
                                                                      out_ci);
     CHIMERA_CUDA(cudaGetLastError());
     count_launch(SLOT_MISC);
@@ -38,7 +40,7 @@ int launch_shard_export(const Params &p, const int32_t *pruned, const int32_t *p
 
 int launch_add_base(int32_t *ids, int64_t n, int64_t doc_base, cudaStream_t st)
 {
-    add_base_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(ids, n, (long long)doc_base);
+    launch(add_base_kernel, (unsigned)((n + 255) / 256), 256, 0, st, ids, n, (long long)doc_base);
     CHIMERA_CUDA(cudaGetLastError());
     count_launch(SLOT_MISC);
     return CHIMERA_OK;

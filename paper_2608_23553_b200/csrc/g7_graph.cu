@@ -97,7 +97,7 @@ int build_graph(Index &ix, const float *centroids, int R, cudaStream_t st)
             e = cudaMemsetAsync(qbuf + (size_t)rows * ix.D, 0, sizeof(float) * (size_t)(rows_per_call - rows) * ix.D, st);
         if (e != cudaSuccess) { rc = fail(CHIMERA_CUDA_ERROR, "copy (centroid graph): %s", cudaGetErrorString(e)); break; }
         if ((rc = launch_score_table(ix, p, qbuf, qdig, nullptr, table, nullptr, status, st))) break;
-        if ((rc = launch_probes(ix, p, L, table, part, probes, st))) break;
+        if ((rc = launch_probes(ix, p, L, table, part, probes, nullptr, st))) break;
         graph_rows_kernel<<<(unsigned)((rows + 127) / 128), 128, 0, st>>>(probes, c0, rows, R, graph);
     }
     if (rc == CHIMERA_OK) {
@@ -135,6 +135,7 @@ graph_probe_kernel(const float *__restrict__ queries, int64_t n_tokens, int D, c
                    int nprobe, uint32_t *__restrict__ visited, int64_t vwords, int32_t *__restrict__ out_probes,
                    int32_t *__restrict__ out_scores, int32_t *__restrict__ out_nvis)
 {
+    pdl_entry();
     const int lane = threadIdx.x & 31;
     const int64_t token = (int64_t)blockIdx.x * GP_WARPS + (threadIdx.x >> 5);
     if (token >= n_tokens) return;                       // whole warps leave together
@@ -260,7 +261,7 @@ int launch_graph_probes(const Index &ix, const float *queries, int64_t n_tokens,
     const int64_t vwords = (ix.K + 31) / 32;
     CHIMERA_CUDA(cudaMemsetAsync(visited, 0, graph_scratch_bytes(ix, n_tokens), st));
     const unsigned blocks = (unsigned)((n_tokens + GP_WARPS - 1) / GP_WARPS);
-    graph_probe_kernel<<<blocks, GP_WARPS * 32, 0, st>>>(queries, n_tokens, ix.D, ix.xc, ix.graph, ix.graph_deg, ix.K,
+    launch(graph_probe_kernel, blocks, GP_WARPS * 32, 0, st, queries, n_tokens, ix.D, ix.xc, ix.graph, ix.graph_deg, ix.K,
                                                          g.n_entries, g.beam, g.max_expansions, nprobe, visited, vwords,
                                                          out_probes, out_scores, out_nvis);
     CHIMERA_CUDA(cudaGetLastError());

@@ -118,8 +118,11 @@ constexpr int DIGIT_PITCH = 128;
 constexpr long long MAX_ROW_SQUARE_SUM = (1LL << 44) + (1LL << 35);
 
 __global__ void digits_kernel(const float *__restrict__ x, int64_t rows, int D, int nbits, int8_t *__restrict__ dig,
-                              int8_t *__restrict__ dig4, int q_len, uint32_t *status)
+                              int8_t *__restrict__ dig4, int q_len, uint32_t *status, uint32_t *__restrict__ clear,
+                              int64_t clear_n)
 {
+    pdl_entry();
+    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < clear_n; k += (int64_t)gridDim.x * blockDim.x) clear[k] = 0u;
     __shared__ unsigned long long row_sq[2];
     const int64_t n = rows * DIGIT_PITCH;
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -165,10 +168,11 @@ __global__ void digits_kernel(const float *__restrict__ x, int64_t rows, int D, 
 }
 
 int launch_digits(const float *x, int64_t rows, int D, int nbits, int8_t *dig, int8_t *dig4, int q_len, uint32_t *status,
-                  cudaStream_t st)
+                  cudaStream_t st, uint32_t *clear, int64_t clear_n)
 {
     const int64_t n = rows * DIGIT_PITCH;
-    digits_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(x, rows, D, nbits, dig, dig4, q_len, status);
+    launch(digits_kernel, (unsigned)((n + 255) / 256), 256, 0, st, x, rows, D, nbits, dig, dig4, q_len, status, clear,
+           clear_n);
     CHIMERA_CUDA(cudaGetLastError());
     return CHIMERA_OK;
 }

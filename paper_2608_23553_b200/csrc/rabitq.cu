@@ -37,6 +37,7 @@ int attach_rabitq(Index &ix, const float *rotation, cudaStream_t st)
 __global__ void __launch_bounds__(128)
 rotate_kernel(const float *__restrict__ rot_t, const float *__restrict__ q, int D, float *__restrict__ out)
 {
+    pdl_entry();
     __shared__ float qrow[128];
     const int64_t row = blockIdx.x;
     const int r = threadIdx.x;
@@ -51,7 +52,7 @@ rotate_kernel(const float *__restrict__ rot_t, const float *__restrict__ q, int 
 
 int launch_rotate(const Index &ix, const Params &p, const float *queries, float *q_rot, cudaStream_t st)
 {
-    rotate_kernel<<<(unsigned)((int64_t)p.B * p.nq), 128, 0, st>>>(ix.rot_t, queries, ix.D, q_rot);
+    launch(rotate_kernel, (unsigned)((int64_t)p.B * p.nq), 128, 0, st, ix.rot_t, queries, ix.D, q_rot);
     CHIMERA_CUDA(cudaGetLastError());
     count_launch(SLOT_G1);
     return CHIMERA_OK;
@@ -63,6 +64,7 @@ constexpr int RP_THREADS = 128;
 __global__ void __launch_bounds__(256)
 rabitq_clear_kernel(int32_t *__restrict__ M, const int32_t *__restrict__ n_cand, int64_t maxc, int nq)
 {
+    pdl_entry();
     const int b = blockIdx.y;
     const int64_t n = (int64_t)n_cand[b] * nq;
     int32_t *row = M + (int64_t)b * maxc * nq;
@@ -86,6 +88,7 @@ rabitq_partial_kernel(const int8_t *__restrict__ qdig, int nq, int B, int CW, in
                       const uint2 *__restrict__ ranks, int64_t words, int64_t maxc, int32_t *__restrict__ M,
                       VisitLists lists, int64_t longest, int splits)
 {
+    pdl_entry();
     __shared__ __align__(16) QueryDigits dig;
     const int b = blockIdx.y;
     const int i = blockIdx.x / splits;
@@ -142,6 +145,7 @@ __global__ void __launch_bounds__(256)
 rabitq_sum_kernel(const int32_t *__restrict__ M, const int32_t *__restrict__ n_cand, int64_t maxc, int nq,
                   int32_t *__restrict__ fprime_bits)
 {
+    pdl_entry();
     const int b = blockIdx.y;
     const int n = n_cand[b];
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
@@ -175,7 +179,7 @@ int launch_rabitq_partial(const Index &ix, const Params &p, const Layout &L, con
     if (use_lists) {
         if ((rc = launch_visit_clear(ix, p, lists, n_cand, st))) return rc;
     } else {
-        rabitq_clear_kernel<<<gclr, 256, 0, st>>>(M, n_cand, p.maxc, p.nq);
+        launch(rabitq_clear_kernel, gclr, 256, 0, st, M, n_cand, p.maxc, p.nq);
         CHIMERA_CUDA(cudaGetLastError());
     }
     const float c = (float)(1.0 / (sqrt((double)ix.D) * 4194304.0));
@@ -185,18 +189,18 @@ int launch_rabitq_partial(const Index &ix, const Params &p, const Layout &L, con
     const float *inv = ix.list_bits ? ix.list_inv : ix.rq_inv;
     const int32_t *ids = ix.list_bits ? nullptr : ix.tok_id;
     if (use_lists)
-        rabitq_partial_kernel<true><<<grid, RP_THREADS, 0, st>>>(qdig_rot, p.nq, p.B, ix.D / 32, p.P, c, probes, ix.tok_off, ids,
+        launch(rabitq_partial_kernel<true>, grid, RP_THREADS, 0, st, qdig_rot, p.nq, p.B, ix.D / 32, p.P, c, probes, ix.tok_off, ids,
                                                                  ix.tok_doc, bits, inv, ranks, L.words, p.maxc, M,
                                                                  lists, ix.max_tok_list, splits);
     else
-        rabitq_partial_kernel<false><<<grid, RP_THREADS, 0, st>>>(qdig_rot, p.nq, p.B, ix.D / 32, p.P, c, probes, ix.tok_off, ids,
+        launch(rabitq_partial_kernel<false>, grid, RP_THREADS, 0, st, qdig_rot, p.nq, p.B, ix.D / 32, p.P, c, probes, ix.tok_off, ids,
                                                                   ix.tok_doc, bits, inv, ranks, L.words, p.maxc, M,
                                                                   lists, ix.max_tok_list, splits);
     CHIMERA_CUDA(cudaGetLastError());
     if (use_lists) {
         if ((rc = launch_visit_sum(ix, p, lists, true, n_cand, fprime_bits, st))) return rc;
     } else {
-        rabitq_sum_kernel<<<gclr, 256, 0, st>>>(M, n_cand, p.maxc, p.nq, fprime_bits);
+        launch(rabitq_sum_kernel, gclr, 256, 0, st, M, n_cand, p.maxc, p.nq, fprime_bits);
         CHIMERA_CUDA(cudaGetLastError());
     }
     count_launch(SLOT_CI, 3);
