@@ -109,7 +109,7 @@ Layout make_layout(const Index &ix, const Params &p)
     L.out_ids = take(B * p.k * sizeof(int32_t));
     L.out_scores = take(B * p.k * sizeof(float));
     L.qdig = take(3 * B * nq * 128);
-    const size_t rows4 = residual_umma_supported(p.nq) ? B * (size_t)residual_rows(p.nq) : 0;
+    const size_t rows4 = B * (size_t)residual_rows(p.nq);
     L.qdig4 = take(3 * rows4 * 128);
     L.table = take(B * (size_t)ix.K * nq * sizeof(int32_t));
     L.table8 = take(coarse_supported(p.nq) ? B * (size_t)ix.K * nq : 0);
@@ -240,7 +240,7 @@ static int run(const Index &ix, const Params &p, int first, int last, const floa
     // results are still there (document-sharded search: the exchange happens between the two calls)
     if (partial && !ix.tok_id)
         return fail(CHIMERA_INVALID_ARG, "partial-score refinement needs chimera_index_enable_partial first");
-    if (rabitq && (!ix.rot_t || !residual_umma_supported(p.nq)))
+    if (rabitq && (!ix.rot_t || p.nq > 64))
         return fail(CHIMERA_INVALID_ARG, "the RaBitQ pipeline needs chimera_index_attach_rabitq and q_len <= 64");
     if (!workspace || ((uintptr_t)workspace & 255)) return fail(CHIMERA_INVALID_ARG, "workspace is NULL or not 256-byte aligned");
     const Layout L = make_layout(ix, p);
@@ -253,7 +253,7 @@ static int run(const Index &ix, const Params &p, int first, int last, const floa
     char *ws = (char *)workspace;
     uint32_t *status = (uint32_t *)(ws + L.status);
     int8_t *qdig = (int8_t *)(ws + L.qdig);
-    int8_t *qdig4 = residual_umma_supported(p.nq) ? (int8_t *)(ws + L.qdig4) : nullptr;
+    int8_t *qdig4 = (int8_t *)(ws + L.qdig4);
     int32_t *table = (int32_t *)(ws + L.table);
     unsigned long long *part = (unsigned long long *)(ws + L.part);
     int32_t *probes = (int32_t *)(ws + L.probes);
@@ -427,14 +427,12 @@ static int run(const Index &ix, const Params &p, int first, int last, const floa
     if (first <= 4 && last >= 4) {
         if (rabitq) {
             if ((rc = launch_rabitq_scores_umma(ix, p, q_rot, qdig_rot, pruned, score4, status, st))) return rc;
-        } else if (residual_umma_supported(p.nq)) {
+        } else {
             if (first > 1) {                       // stage 1 did not run in this call: build the query digit planes
                 if ((rc = launch_digits(queries, (int64_t)p.B * p.nq, ix.D, ix.nbits, nullptr, qdig4, p.nq, status, st))) return rc;
                 count_launch(SLOT_G4);
             }
             if ((rc = launch_residual_scores_umma(ix, p, queries, qdig4, table, pruned, score4, status, st))) return rc;
-        } else if ((rc = launch_residual_scores(ix, p, queries, table, pruned, score4, st))) {
-            return rc;
         }
         prof_mark(SLOT_G4, st);
     }

@@ -70,7 +70,7 @@ struct Layout {
     size_t out_ids;       // int32  [B, k]            (host-entry staging)
     size_t out_scores;    // float  [B, k]
     size_t qdig;          // int8   [3][B*nq][128]
-    size_t qdig4;         // int8   [3][B*residual_rows(nq)][128]  the same for stage 4 (q_len <= 64)
+    size_t qdig4;         // int8   [3][B*residual_rows(nq)][128]  the same for stage 4
     size_t table;         // int32  [B][K][nq]
     size_t table8;        // uint8  [B][K][nq]        coarse copy: min((S + 2^24 + 64) >> 17, 255)
     size_t part;          // uint64 [B][n_part][P][nq] partial top-P keys
@@ -247,7 +247,7 @@ int launch_cand_ranges(const Index &ix, const Params &p, const int32_t *cand, co
 int launch_coarse_bounds(const Index &ix, const Params &p, const uint8_t *table8, const int32_t *cand,
                          const int32_t *n_cand, int32_t *lo, int32_t *hi, const int2 *rng, cudaStream_t st);
 // First cut of the candidates by an upper bound from one number per token (g3_filter.cu).  launch_filter_scan leaves the
-// bounds in hi0 and the best ~1.5 n_prune candidates in seed / seed_rng (their number in the workspace's n_seed);
+// bounds in hi0 and the best ~2 n_prune candidates in seed / seed_rng (their number in the workspace's n_seed);
 // launch_filter_keep takes the seeds' exact CI and writes the candidates that can still be in the top n_prune, ascending;
 // launch_filter_contenders narrows them down by the 8-bit upper bounds.
 bool filter_used(const Index &ix, const Params &p);
@@ -285,10 +285,7 @@ int launch_shard_select(const Params &p, const int32_t *all_ids, const int32_t *
 int launch_add_base(int32_t *ids, int64_t n, int64_t doc_base, cudaStream_t st);
 int launch_shard_merge_topk(const int32_t *all_ids, const float *all_scores, int world, int B, int k, int32_t *out_ids,
                             float *out_scores, cudaStream_t st);
-int launch_residual_scores(const Index &ix, const Params &p, const float *queries, const int32_t *table,
-                           const int32_t *pruned, float *score4, cudaStream_t st);
-// Tensor-core variant of stage 4 for q_len <= 64; qdig4 = the query digit planes in its own row order.
-bool residual_umma_supported(int nq);
+// qdig4 = the query digit planes in stage 4's own row order.
 int launch_residual_scores_umma(const Index &ix, const Params &p, const float *queries, const int8_t *qdig,
                                 const int32_t *table, const int32_t *pruned, float *score4, uint32_t *status,
                                 cudaStream_t st);
@@ -354,7 +351,7 @@ __host__ __device__ __forceinline__ int digit_dim(int pos, int nbits)
 // Stage 4 on the tensor cores: rows per query of its digit planes, and the row of query token i.  Within 16 tokens, tokens
 // 4 g ... 4 g + 3 sit in rows 2 g, 2 g + 1, 8 + 2 g, 8 + 2 g + 1: the accumulator columns that the same thread reads back,
 // so that its four score-table entries are one 16-byte load.
-__host__ __device__ __forceinline__ int residual_rows(int q_len) { return q_len <= 32 ? 32 : 64; }
+__host__ __device__ __forceinline__ int residual_rows(int q_len) { return q_len <= 32 ? 32 : q_len <= 64 ? 64 : 128; }
 __host__ __device__ __forceinline__ int score_row(int i) { return (i & ~15) | (i & 2) << 2 | (i >> 1 & 6) | (i & 1); }
 
 // ---------------------------------------------------------------------------------------------------------------

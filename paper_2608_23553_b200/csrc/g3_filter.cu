@@ -12,7 +12,7 @@
 //   filter_theta_kernel    theta_i from a sample of the table's rows
 //   filter_excess_kernel   e(c) of every centroid, rounded up (16 bits, or 6-bit codes five to a word for large K)
 //   filter_scan_kernel     hi0 of every candidate: the query's whole e table in shared memory, one lookup per token
-//   filter_seed_kernel     the ~1.5 n_prune candidates with the largest hi0 (their order does not matter)
+//   filter_seed_kernel     the ~2 n_prune candidates with the largest hi0 (their order does not matter)
 //   (their exact CI: g3_centroid_interaction.cu)
 //   filter_count_kernel,   tau = the n_prune-th largest of those, a lower bound on the n_prune-th largest CI; keeps every
 //   filter_write_kernel    candidate with hi0 >= tau, ascending, with its token range
@@ -320,7 +320,7 @@ filter_scan_kernel(const uint8_t *__restrict__ tab, size_t pitch, const int32_t 
 {
     pdl_entry();
     extern __shared__ uint4 s_tab[];
-    __shared__ uint32_t s_level[64];
+    __shared__ uint16_t s_level[64];                     // two to a bank: no conflicts
     __shared__ int s_hist[FILTER_BINS];
     __shared__ int s_sort[SCAN_SORT_BINS];
     __shared__ uint2 s_rng[SCAN_THREADS_F];
@@ -374,11 +374,12 @@ filter_scan_kernel(const uint8_t *__restrict__ tab, size_t pitch, const int32_t 
         const unsigned long long pr = (unsigned long long)(uint32_t)c * 858993460u;
         return (int)s_level[(tab6[pr >> 32] >> ((uint32_t)pr >> 27)) & 63];
     };
-    auto add4 = [&](int acc, const int4 &v, int rem) {
+    // the values of positions lead ... rem - 1 of a group of four
+    auto add4 = [&](int acc, const int4 &v, int rem, int lead) {
         const int x = value(v.x), y = value(v.y), z = value(v.z), w = value(v.w);
-        acc += rem > 0 ? x : 0;
-        acc += rem > 1 ? y : 0;
-        acc += rem > 2 ? z : 0;
+        acc += rem > 0 && lead <= 0 ? x : 0;
+        acc += rem > 1 && lead <= 1 ? y : 0;
+        acc += rem > 2 && lead <= 2 ? z : 0;
         acc += rem > 3 ? w : 0;
         return acc;
     };
@@ -430,20 +431,16 @@ filter_scan_kernel(const uint8_t *__restrict__ tab, size_t pitch, const int32_t 
             // steps of 64 tokens, as many as the longest of the four documents needs
             const int most = __reduce_max_sync(0xffffffffu, (int)(cur.y - (q - 4 * sub)));
             int acc = 0, rem = (int)(cur.y - q);
-            if (sub == 0) {                                  // ids of the document before, in front of the first token
-                const int lead = (int)(cur.x & 3u);
-                if (lead > 0) acc -= value(a0.x);
-                if (lead > 1) acc -= value(a0.y);
-                if (lead > 2) acc -= value(a0.z);
-            }
+            int lead = sub == 0 ? (int)(cur.x & 3u) : 0;     // ids of the document before, in front of the first token
             for (int c = 0; c < most; c += 64) {
                 int4 n0, n1;
                 const bool last = c + 64 >= most;
                 const uint32_t ql = last ? qn : q + 64, hl = last ? nxt.y : cur.y;
                 n0 = load4(ql, hl);
                 n1 = load4(ql + 32, hl);
-                acc = add4(acc, a0, rem);
-                if (c + 32 < most) acc = add4(acc, a1, rem - 32);
+                acc = add4(acc, a0, rem, lead);
+                if (c + 32 < most) acc = add4(acc, a1, rem - 32, 0);
+                lead = 0;
                 rem -= 64;
                 a0 = n0;
                 a1 = n1;
@@ -472,7 +469,7 @@ filter_scan_kernel(const uint8_t *__restrict__ tab, size_t pitch, const int32_t 
 // A Q.24 threshold in units of 2^us, rounded up (hi0 is a whole number of them).
 __device__ __forceinline__ int32_t units_up(int32_t tau, int us) { return (int32_t)(((long long)tau + (1 << us) - 1) >> us); }
 
-// grid (split, B): candidates with the largest hi0, 1.5 n_prune of them and the rest of the
+// grid (split, B): candidates with the largest hi0, 2 n_prune of them and the rest of the
 // last histogram bin, with their token ranges, in no particular order; seed_thr[b] = the hi0 they
 // start at, seed_slot[candidate] = where each one went.  n_seed (cleared before) stays 0 when a query has so few
 // candidates that all are kept.
@@ -487,7 +484,7 @@ filter_seed_kernel(const int32_t *__restrict__ cand, const int32_t *__restrict__
     __shared__ int warp_part[32];
     __shared__ int s_bin, s_theta;
     const int b = blockIdx.y, n = n_cand[b];
-    const int want = n_prune + n_prune / 2 + 32;
+    const int want = 2 * n_prune + 32;
     if (n <= want) {
         if (blockIdx.x == 0 && threadIdx.x == 0) seed_thr[b] = INT_MAX;
         return;

@@ -1,4 +1,4 @@
-// Stage 4 on the tensor cores (q_len <= 64): residual-decode MaxSim of the surviving documents (Definition 1 on the
+// Stage 4 on the tensor cores: residual-decode MaxSim of the surviving documents (Definition 1 on the
 // decoded tokens),
 //   score(d) = sum_i max_{t in d} <q_i, c_{cid_t} + r^(code_t)>
 //            = sum_i [ max_t ( S[cid_t, i] + delta * sum_x q_i[x] u_t[x] ) + (lo + delta/2) * sum_x q_i[x] ].
@@ -20,7 +20,9 @@
 // Measured (batch 256, Mid, n_prune 1024): 2.24 -> 1.56 ms against one warp per quarter, value rows in shared memory and
 // two barriers per tile; 64 long-document queries of 64 tokens: 5.9 -> 3.75 ms.  Residency: q_len <= 32 three CTAs of 256
 // threads (85 registers, no spills; four with 64 registers: 1.78 ms; the RaBitQ variant, which holds no score-table
-// entries, four: 1.18 against 1.32 ms), q_len <= 64 two of 512 threads.  All mbarrier waits are bounded.
+// entries, four: 1.18 against 1.32 ms), q_len <= 64 two of 512 threads.  Longer queries
+// take two launches (8 queries of 100 tokens, n_prune 1024: 1.91 ms with an FMA kernel, 0.26 with these).  All mbarrier waits are
+// bounded.
 #include <math.h>
 
 #include "common.cuh"
@@ -50,14 +52,17 @@ __device__ __forceinline__ float f_unorder(uint32_t o)
 template <int NQP, int NBITS, bool RQ, bool FULL>
 __global__ void __launch_bounds__(128 * (NQP / G4U_COLS), NQP == 32 ? (RQ ? 4 : 3) : 2)
 residual_maxsim_umma(const __grid_constant__ CUtensorMap map_q, const float *__restrict__ queries,
-                     const int32_t *__restrict__ table, int64_t K, int nq_arg, int D_arg, int CW_arg, float delta, float kappa,
+                     const int32_t *__restrict__ table, int64_t K, int nq_arg, int q_base, int nq_all_arg, int q_rows, int D_arg,
+                     int CW_arg, float delta, float kappa,
                      const int32_t *__restrict__ pruned, int n_prune, int docs_per_cta,
                      const int32_t *__restrict__ cids, const uint32_t *__restrict__ codes,
                      const float *__restrict__ factors, const int64_t *__restrict__ doc_off,
                      float *__restrict__ score4, uint32_t *status, long long wait_limit, int skip_loads)
 {
     pdl_entry();
-    const int nq = FULL ? NQP : nq_arg, D = FULL ? 128 : D_arg, CW = FULL ? (NBITS == 2 ? 8 : 4) : CW_arg;
+    // this launch's query tokens are q_base ... q_base + nq - 1 of the query's nq_all (its digit planes have q_rows rows)
+    const int nq = FULL ? NQP : nq_arg, nq_all = FULL ? NQP : nq_all_arg;
+    const int D = FULL ? 128 : D_arg, CW = FULL ? (NBITS == 2 ? 8 : 4) : CW_arg;
     constexpr int N = 3 * NQP;                               // MMA N: three digit planes side by side
     constexpr uint32_t TMEM_COLS = N <= 96 ? 128 : 256;
     constexpr uint32_t A_COL = N;                            // the expanded codes: 32 columns behind the accumulators
@@ -131,7 +136,7 @@ residual_maxsim_umma(const __grid_constant__ CUtensorMap map_q, const float *__r
         int si = 0;
         if (i < nq) {
             const int fourth = D >> 2;                // D is a multiple of 32
-            const float4 *src = reinterpret_cast<const float4 *>(queries + ((int64_t)b * nq + i) * D + (tid & 3) * fourth);
+            const float4 *src = reinterpret_cast<const float4 *>(queries + ((int64_t)b * nq_all + q_base + i) * D + (tid & 3) * fourth);
             for (int x = 0; x < (fourth >> 2); ++x) {
                 const float4 v = __ldg(src + x);
                 sum += (v.x + v.y) + (v.z + v.w);
@@ -157,12 +162,12 @@ residual_maxsim_umma(const __grid_constant__ CUtensorMap map_q, const float *__r
     // skip_loads (test hook): no load is issued, so the first wait below runs into its limit with nothing in flight
     if (tid == 0 && !skip_loads) {   // the query's three digit planes, side by side: rows [p * NQP, (p + 1) * NQP)
         mbar_expect_tx(bar_b, B_BYTES);
-        for (int p = 0; p < 3; ++p) tma_load_3d(sB + p * NQP * 128, &map_q, 0, b * NQP, p, bar_b);
+        for (int p = 0; p < 3; ++p) tma_load_3d(sB + p * NQP * 128, &map_q, 0, b * q_rows + q_base, p, bar_b);
     }
 
-    const char *tb = reinterpret_cast<const char *>(table + (int64_t)b * K * nq);
-    const uint32_t row_bytes = 4u * (uint32_t)nq;
-    const bool vec_rows = (nq & 3) == 0;           // 16-byte groups of a row are aligned
+    const char *tb = reinterpret_cast<const char *>(table + (int64_t)b * K * nq_all + q_base);
+    const uint32_t row_bytes = 4u * (uint32_t)nq_all;
+    const bool vec_rows = (nq_all & 3) == 0;       // 16-byte groups of a row are aligned (q_base is a multiple of 64)
     const int k_steps = FULL ? 4 : D >> 5;
     const float code_scale = delta * 4.0f;                    // delta * 2^-22, times 2^24
     bool alive = true;
@@ -265,7 +270,7 @@ residual_maxsim_umma(const __grid_constant__ CUtensorMap map_q, const float *__r
             int32_t c = __shfl_sync(0xffffffffu, cid, sub + 8 * j);
             c = DBG_CID(c > 0 ? c : 0);                       // (rows without a token take part in no maximum)
             const int32_t *src = reinterpret_cast<const int32_t *>(tb + (uint64_t)(uint32_t)c * row_bytes) + col0;
-            if (FULL || (vec_rows && col0 < nq)) {
+            if (FULL || (vec_rows && col0 + 3 < nq)) {
                 const int4 q = __ldg(reinterpret_cast<const int4 *>(src));
                 sv[j][0] = q.x; sv[j][1] = q.y; sv[j][2] = q.z; sv[j][3] = q.w;
             } else {
@@ -388,7 +393,10 @@ residual_maxsim_umma(const __grid_constant__ CUtensorMap map_q, const float *__r
                 if (NQP > 32 && 32 + lane < nq) v += f_unorder(docmax[dl * NQP + 32 + lane]) * (1.0f / 16777216.0f) + kappa * s_sumq[32 + lane];
             }
             v = warp_sum(v);
-            if (lane == 0) score4[(int64_t)b * n_prune + j0 + dl] = d >= 0 ? v : -INFINITY;
+            if (lane == 0) {
+                float *out = score4 + (int64_t)b * n_prune + j0 + dl;
+                *out = d >= 0 ? (q_base > 0 ? *out + v : v) : -INFINITY;      // (the first tokens' launch came before)
+            }
         }
     }
     if (warp == 0) {
@@ -398,7 +406,7 @@ residual_maxsim_umma(const __grid_constant__ CUtensorMap map_q, const float *__r
 }
 
 template <int NQP, int NBITS, bool RQ>
-static int launch_g4_umma(const Index &ix, const Params &p, const float *queries, const int8_t *qdig4,
+static int launch_g4_umma(const Index &ix, const Params &p, int q_base, int nq, const float *queries, const int8_t *qdig4,
                           const int32_t *table, const int32_t *pruned, float *score4, uint32_t *status, cudaStream_t st)
 {
     constexpr int N = 3 * NQP;
@@ -406,7 +414,7 @@ static int launch_g4_umma(const Index &ix, const Params &p, const float *queries
     // RQ: the kappa slot carries c = 1 / (sqrt(D) * 2^22)
     const float kappa = RQ ? (float)(1.0 / (sqrt((double)ix.D) * 4194304.0)) : ix.res_lo + 0.5f * delta;
     CUtensorMap map_q;
-    int rc = make_plane_map(&map_q, qdig4, (int64_t)p.B * NQP, NQP);
+    int rc = make_plane_map(&map_q, qdig4, (int64_t)p.B * residual_rows(p.nq), NQP);
     if (rc) return rc;
     // query planes, maxima
     size_t smem = 1024 + (size_t)N * 128 + sizeof(uint32_t) * G4U_MAX_DOCS * NQP + 32;
@@ -415,7 +423,7 @@ static int launch_g4_umma(const Index &ix, const Params &p, const float *queries
     // four or fewer and the 256-column ones at two; the latter ask for a third of an SM's shared memory plus one byte
     // besides, so that a build with fewer registers does not change that.
     if (N > 96 && smem < 227 * 1024 / 3 + 1) smem = 227 * 1024 / 3 + 1;
-    auto kern = p.nq == NQP && ix.D == 128 ? residual_maxsim_umma<NQP, NBITS, RQ, true>
+    auto kern = p.nq == NQP && nq == NQP && ix.D == 128 ? residual_maxsim_umma<NQP, NBITS, RQ, true>
                                            : residual_maxsim_umma<NQP, NBITS, RQ, false>;
     CHIMERA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     // documents per CTA: whole waves of resident CTAs, as few as documents-per-CTA limit allows (a second wave of a few CTAs
@@ -429,7 +437,8 @@ static int launch_g4_umma(const Index &ix, const Params &p, const float *queries
     if (dpc > G4U_MAX_DOCS) dpc = G4U_MAX_DOCS;
     dim3 grid((unsigned)((p.n_prune + dpc - 1) / dpc), (unsigned)p.B);
     const uint32_t *code_words = reinterpret_cast<const uint32_t *>(RQ ? ix.rq_bits : ix.codes);
-    launch(kern, grid, 128 * (NQP / G4U_COLS), smem, st, map_q, queries, table, ix.K, p.nq, ix.D, RQ ? ix.D / 32 : ix.CB / 4, delta,
+    launch(kern, grid, 128 * (NQP / G4U_COLS), smem, st, map_q, queries, table, ix.K, nq, q_base, p.nq,
+           residual_rows(p.nq), ix.D, RQ ? ix.D / 32 : ix.CB / 4, delta,
                                           kappa, pruned, p.n_prune, (int)dpc, ix.cids, code_words, ix.rq_inv, ix.doc_off,
                                           score4, status, wait_limit_cycles(), fault_skip_tma_loads());
     CHIMERA_CUDA(cudaGetLastError());
@@ -437,26 +446,34 @@ static int launch_g4_umma(const Index &ix, const Params &p, const float *queries
     return CHIMERA_OK;
 }
 
-bool residual_umma_supported(int nq) { return nq <= 64; }
+// More than 64 query tokens: the first 64, then the rest added to their scores (MMA N would exceed 256 with all of them).
+template <int NBITS>
+static int launch_g4_parts(const Index &ix, const Params &p, const float *queries, const int8_t *qdig4, const int32_t *table,
+                           const int32_t *pruned, float *score4, uint32_t *status, cudaStream_t st)
+{
+    for (int q_base = 0; q_base < p.nq; q_base += 64) {
+        const int nq = p.nq - q_base < 64 ? p.nq - q_base : 64;
+        const int rc = nq <= 32 ? launch_g4_umma<32, NBITS, false>(ix, p, q_base, nq, queries, qdig4, table, pruned, score4, status, st)
+                                : launch_g4_umma<64, NBITS, false>(ix, p, q_base, nq, queries, qdig4, table, pruned, score4, status, st);
+        if (rc) return rc;
+    }
+    return CHIMERA_OK;
+}
 
 int launch_residual_scores_umma(const Index &ix, const Params &p, const float *queries, const int8_t *qdig4,
                                 const int32_t *table, const int32_t *pruned, float *score4, uint32_t *status,
                                 cudaStream_t st)
 {
-    if (ix.nbits == 2) {
-        if (p.nq <= 32) return launch_g4_umma<32, 2, false>(ix, p, queries, qdig4, table, pruned, score4, status, st);
-        return launch_g4_umma<64, 2, false>(ix, p, queries, qdig4, table, pruned, score4, status, st);
-    }
-    if (p.nq <= 32) return launch_g4_umma<32, 1, false>(ix, p, queries, qdig4, table, pruned, score4, status, st);
-    return launch_g4_umma<64, 1, false>(ix, p, queries, qdig4, table, pruned, score4, status, st);
+    return ix.nbits == 2 ? launch_g4_parts<2>(ix, p, queries, qdig4, table, pruned, score4, status, st)
+                         : launch_g4_parts<1>(ix, p, queries, qdig4, table, pruned, score4, status, st);
 }
 
 // Complete 1-bit scores of the surviving documents on the RaBitQ codes; q_rot / qdig_rot belong to the rotated queries.
 int launch_rabitq_scores_umma(const Index &ix, const Params &p, const float *q_rot, const int8_t *qdig_rot,
                               const int32_t *pruned, float *score4, uint32_t *status, cudaStream_t st)
 {
-    if (p.nq <= 32) return launch_g4_umma<32, 1, true>(ix, p, q_rot, qdig_rot, nullptr, pruned, score4, status, st);
-    return launch_g4_umma<64, 1, true>(ix, p, q_rot, qdig_rot, nullptr, pruned, score4, status, st);
+    if (p.nq <= 32) return launch_g4_umma<32, 1, true>(ix, p, 0, p.nq, q_rot, qdig_rot, nullptr, pruned, score4, status, st);
+    return launch_g4_umma<64, 1, true>(ix, p, 0, p.nq, q_rot, qdig_rot, nullptr, pruned, score4, status, st);
 }
 
 }  // namespace chimera
