@@ -325,6 +325,8 @@ static int run(const Index &ix, const Params &p, int first, int last, const floa
     // stages 1 and 2a of one call run together when the layout provides for it: the probes come out of the score
     // table's epilogue and the table is not read again
     const bool together = first <= 1 && last >= 2 && !graph && L.pq_stride > 0;
+    // the RaBitQ pipeline reads nothing of the table but the probes
+    const bool keep_table = !rabitq || (taps && taps->score_table);
     // a small bitmap, and the probe kernel's counters behind it, are cleared on the side by the first kernel of stage 1 (one
     // operation less in the chain)
     const int64_t bitmap_words = (int64_t)p.B * (L.words + (p.nq + 31) / 32);
@@ -332,7 +334,8 @@ static int run(const Index &ix, const Params &p, int first, int last, const floa
     int32_t *probes_done = clear_words > 0 ? (int32_t *)bitmap + (int64_t)p.B * L.words : nullptr;
     if (first <= 1 && last >= 1 && !graph) {
         if (together)
-            rc = launch_score_table_probes(ix, p, L, queries, qdig, qdig4, table, table8, ws, status, st, bitmap, clear_words);
+            rc = launch_score_table_probes(ix, p, L, queries, qdig, qdig4, table, keep_table, table8, ws, status, st, bitmap,
+                                           clear_words);
         else
             rc = launch_score_table(ix, p, queries, qdig, qdig4, table, table8, status, st, bitmap, clear_words);
         if (rc) return rc;
@@ -340,11 +343,11 @@ static int run(const Index &ix, const Params &p, int first, int last, const floa
     }
     if (first <= 2 && last >= 2) {
         if (graph) {
-            if ((rc = launch_graph_probes(ix, queries, (int64_t)p.B * p.nq, p.P, *graph, (uint32_t *)(ws + L.graph_vis),
+            if ((rc = launch_graph_probes(ix, queries, (int64_t)p.B * p.nq, p.P, *graph, (uint32_t *)(ws + L.graph_vis), false,
                                           probes, nullptr, nullptr, st)))
                 return rc;
         } else if (together) {
-            if ((rc = launch_probe_merge(ix, p, L, table, ws, st))) return rc;
+            if ((rc = launch_probe_merge(ix, p, L, table, keep_table ? nullptr : qdig, ws, status, st))) return rc;
         } else if ((rc = launch_probes(ix, p, L, table, part, probes, probes_done, st))) {
             return rc;
         }
@@ -645,7 +648,7 @@ int chimera_graph_probes(const chimera_index *index, const float *queries, int32
     const int64_t tokens = (int64_t)n_queries * q_len;
     if (scratch_bytes < graph_scratch_bytes(*ix, tokens))
         return fail(CHIMERA_WORKSPACE_TOO_SMALL, "scratch has %zu bytes, %zu needed", scratch_bytes, graph_scratch_bytes(*ix, tokens));
-    return launch_graph_probes(*ix, queries, tokens, nprobe, g, (uint32_t *)scratch, out_probes, out_scores, out_n_visited,
+    return launch_graph_probes(*ix, queries, tokens, nprobe, g, (uint32_t *)scratch, true, out_probes, out_scores, out_n_visited,
                                (cudaStream_t)stream);
 }
 

@@ -203,18 +203,22 @@ int launch_probes(const Index &ix, const Params &p, const Layout &L, const int32
                   int32_t *probes, int32_t *done, cudaStream_t st);
 // Stages 1 and 2a together (g1_score_table.cu), used when the layout has pq_stride > 0, and its probe-side pieces
 // (g2_probe.cu): the sample's top nprobe and bounds; the final top nprobe from sample list and queues, with the table
-// scan as the fallback for queries whose queue overflowed.
+// scan as the fallback for queries whose queue overflowed.  keep_table: the table is wanted beside the probes; without it
+// only the sample's tiles are written, and launch_probe_merge (given the query digits) has the rest made for those queries.
 int probe_sample_stride(int64_t K, int nq, int P);       // host arithmetic only
 int probe_queue_stride(const Index &ix, const Params &p);
 int probe_queue_cap();
 int probe_sample_groups(const Index &ix, int stride);
 int launch_score_table_probes(const Index &ix, const Params &p, const Layout &L, const float *queries, int8_t *qdig,
                               int8_t *qdig4,
-                              int32_t *table, uint8_t *table8, char *ws, uint32_t *status, cudaStream_t st,
+                              int32_t *table, bool keep_table, uint8_t *table8, char *ws, uint32_t *status, cudaStream_t st,
                               uint32_t *clear = nullptr, int64_t clear_n = 0);
+int launch_score_table_redo(const Index &ix, const Params &p, const Layout &L, const int8_t *qdig, int32_t *table,
+                            const int32_t *redo, uint32_t *status, cudaStream_t st);
 int launch_probe_sample(const Index &ix, const Params &p, const Layout &L, const int32_t *table, char *ws,
                         int n_sample_tiles, cudaStream_t st);
-int launch_probe_merge(const Index &ix, const Params &p, const Layout &L, const int32_t *table, char *ws, cudaStream_t st);
+int launch_probe_merge(const Index &ix, const Params &p, const Layout &L, int32_t *table, const int8_t *redo_qdig, char *ws,
+                       uint32_t *status, cudaStream_t st);
 // bitmap_clear: the bitmap is zero already.  ranks, rng (the candidates' token ranges), cont_scratch (rows of which the
 // contender step's histogram is cleared): each may be NULL.
 int launch_gather(const Index &ix, const Params &p, const Layout &L, const int32_t *probes, uint32_t *bitmap,
@@ -295,9 +299,11 @@ int launch_rabitq_scores_umma(const Index &ix, const Params &p, const float *q_r
 int build_graph(Index &ix, const float *centroids, int degree, cudaStream_t st);
 size_t graph_scratch_bytes(const Index &ix, int64_t n_tokens);
 int check_graph_params(const Index &ix, const GraphSearch &g, int nprobe);
-// visited: graph_scratch_bytes(ix, n_tokens) bytes; out_scores / out_nvis may be NULL.
+// visited: graph_scratch_bytes(ix, n_tokens) bytes of scratch, holding the visited sets afterwards if want_visited;
+// out_scores / out_nvis may be NULL.
 int launch_graph_probes(const Index &ix, const float *queries, int64_t n_tokens, int nprobe, const GraphSearch &g,
-                        uint32_t *visited, int32_t *out_probes, int32_t *out_scores, int32_t *out_nvis, cudaStream_t st);
+                        uint32_t *visited, bool want_visited, int32_t *out_probes, int32_t *out_scores, int32_t *out_nvis,
+                        cudaStream_t st);
 // rabitq.cu
 int attach_rabitq(Index &ix, const float *rotation, cudaStream_t st);
 int launch_rotate(const Index &ix, const Params &p, const float *queries, float *q_rot, cudaStream_t st);

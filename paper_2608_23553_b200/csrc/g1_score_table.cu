@@ -46,16 +46,16 @@ constexpr uint32_t G1_SMEM = G1_STAGES * G1_B_STAGE + 1024 /* alignment slack */
 static_assert(G1_ACC_COLS + 96 <= G1_TMEM_COLS, "accumulators and centroid digits share the allocation");
 
 // floor((T + 2^19) / 2^20) with T = a0 + 2^8 a1 + 2^16 a2 + 2^24 a3 + 2^32 a4, in 32-bit arithmetic.  Split T as
-// u + 2^16 v with u = a0 + 2^8 a1 (|a0| < 2^23, |a1| < 2^23: no overflow together with the rounding constant) and
+// u + 2^16 v with u = a0 + 2^8 a1 (|a0| < 2^23, |a1| < 2^23: no overflow) and
 // v = a2 + 2^8 a3 + 2^16 a4.  v is about T / 2^16, which fits 32 bits whenever the result does (|S| < 2^31 means
 // |T| < 2^51; here |T| < 2^45), so computing it modulo 2^32 loses nothing.  Nested floor divisions compose:
 // floor((x + 2^16 v) / 2^20) = floor((floor(x / 2^16) + v) / 2^4) for any integers x, v; arithmetic right shifts are
 // floor divisions.
 __device__ __forceinline__ int32_t combine_digits(int32_t a0, int32_t a1, int32_t a2, int32_t a3, int32_t a4)
 {
-    const int32_t u = a0 + (a1 << 8) + (1 << 19);
+    const int32_t u = a0 + (a1 << 8);
     const int32_t v = a2 + (int32_t)((uint32_t)a3 << 8) + (int32_t)((uint32_t)a4 << 16);
-    return ((u >> 16) + v) >> 4;
+    return ((u >> 16) + v + 8) >> 4;                    // the rounding constant is a multiple of 2^16
 }
 
 __device__ __forceinline__ void mbar_arrive(uint32_t bar)
@@ -70,19 +70,22 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar)
 // FILTER (only with the "others"): thr[row] holds, for every query-token row, a lower bound on the score of the row's
 // nprobe-th best centroid (found on the sample); every score >= thr[row] goes, as a (score, centroid) key, into that
 // row's queue (keys[row][cap], counted in cnt[row]; entries past cap are dropped and the count tells).  The top nprobe
-// of a row are then in its queue, so the probe stage never reads the table again.
+// of a row are then in its queue, so the probe stage never reads the table again, and a search that needs only the
+// probes passes no table (the RaBitQ pipeline: 2.1 GB less to write at Mid, batch 256).
+// redo: a flag per query (nonzero: its rows of these tiles are wanted after all); a CTA without such a query returns.
 struct G1Tiles {
     int tile_stride, sample;
     const int32_t *thr;
     int32_t *cnt;
     unsigned long long *keys;
     int cap;
+    const int32_t *redo;
 };
 
 // grid (centroid tiles of the launch, n_splits).  Each CTA: one centroid tile, query-row tiles
 // [blockIdx.y * tiles_per_split, ...).  KS = D / 32 MMA steps per digit-plane product.
-template <int KS, bool FILTER>
-__global__ void __launch_bounds__(G1_THREADS)
+template <int KS, bool FILTER, bool TABLE>
+__global__ void __launch_bounds__(G1_THREADS, 2)
 score_table_umma(const int8_t *__restrict__ cdig, const __grid_constant__ CUtensorMap map_q, int64_t K, int nq,
                  int64_t q_rows, int n_tiles, int tiles_per_split, int32_t *__restrict__ table,
                  uint8_t *__restrict__ table8, uint32_t *status, long long wait_limit, int skip_loads, G1Tiles tiles)
@@ -105,6 +108,13 @@ score_table_umma(const int8_t *__restrict__ cdig, const __grid_constant__ CUtens
     int t_end = t_begin + tiles_per_split;
     if (t_end > n_tiles) t_end = n_tiles;
     const int my_tiles = t_end > t_begin ? t_end - t_begin : 0;
+    if (!FILTER && tiles.redo != nullptr) {
+        const int64_t r_end = (int64_t)t_end * G1_N < q_rows ? (int64_t)t_end * G1_N : q_rows;
+        int wanted = 0;
+        if (my_tiles > 0)
+            for (int64_t b = (int64_t)t_begin * G1_N / nq + tid; b <= (r_end - 1) / nq; b += G1_THREADS) wanted |= tiles.redo[b];
+        if (!__syncthreads_or(wanted)) return;
+    }
 
     if (tid == 0) {
         for (int s = 0; s < G1_STAGES; ++s) mbar_init(bar_full + 8 * s, 1);
@@ -230,15 +240,14 @@ score_table_umma(const int8_t *__restrict__ cdig, const __grid_constant__ CUtens
         const uint32_t lane_addr = tmem + ((uint32_t)(quad * 32) << 16);
         const uint32_t unq = (uint32_t)nq, rows32 = (uint32_t)q_rows;
         const int first_chunk = 2 * (warp >> 2);
+        const uint32_t col0 = (uint32_t)first_chunk * 8;
         unsigned long long pend_key = 0ull, *pend_dst = nullptr;   // FILTER: this thread's last key, not stored yet
         int pend_slot = 0;
         for (int it = 0; it < my_tiles; ++it) {
-            const int t = t_begin + it;
-            // FILTER: the thresholds of this warp's 16 query-token rows (the same for every lane), asked for before
-            // the wait
+            const uint32_t r0 = (uint32_t)(t_begin + it) * G1_N + col0;      // this warp's first query-token row
+            // FILTER: the thresholds of this warp's 16 query-token rows (the same for every lane), asked for before the wait
             int32_t thr_v[16];
             if (FILTER) {
-                const uint32_t r0 = (uint32_t)t * G1_N + (uint32_t)first_chunk * 8;
 #pragma unroll
                 for (int g = 0; g < 4; ++g) {
                     int4 v = make_int4(0x7fffffff, 0x7fffffff, 0x7fffffff, 0x7fffffff);     // rows past the end
@@ -254,70 +263,65 @@ score_table_umma(const int8_t *__restrict__ cdig, const __grid_constant__ CUtens
             tc_fence_after();
             int32_t accs[2][5][8];
 #pragma unroll
-            for (int ch = 0; ch < 2; ++ch)
-#pragma unroll
-                for (int w = 0; w < 5; ++w) tmem_ld8(lane_addr + w * G1_N + (first_chunk + ch) * 8, accs[ch][w]);
+            for (int w = 0; w < 5; ++w) {
+                tmem_ld8(lane_addr + w * G1_N + col0, accs[0][w]);
+                tmem_ld8(lane_addr + w * G1_N + col0 + 8, accs[1][w]);
+            }
             tmem_ld_wait();
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_empty);             // the accumulators may be overwritten from here on
 
-            // (query, token) coordinates of the tile's first row: one 32-bit division per tile
-            const uint32_t tile_qb = ((uint32_t)t * G1_N) / unq, tile_qi = (uint32_t)t * G1_N - tile_qb * unq;
-            uint32_t w8_carry[2] = {0u, 0u};                  // 8-bit words of the even chunk of the pair
+            // (query, token) coordinates of that row (rows fit 32 bits: n_queries * q_len < 2^23)
+            uint32_t qb = TABLE ? r0 / unq : 0u, qi = TABLE ? r0 - qb * unq : 0u;
+            uint32_t w8[4];                                    // their 8-bit copies
 #pragma unroll
             for (int ch = 0; ch < 2; ++ch) {
-                const int chunk = first_chunk + ch;
                 int32_t out[8];
 #pragma unroll
                 for (int e = 0; e < 8; ++e)
                     out[e] = combine_digits(accs[ch][0][e], accs[ch][1][e], accs[ch][2][e], accs[ch][3][e], accs[ch][4][e]);
-                // first query-token row of this chunk and its (query, token) coordinates (rows fit 32 bits:
-                // n_queries * q_len < 2^23)
-                const uint32_t r0 = (uint32_t)t * G1_N + (uint32_t)chunk * 8;
-                uint32_t qb = tile_qb, qi = tile_qi + (uint32_t)chunk * 8;      // chunk * 8 < 32: few subtractions
-                while (qi >= unq) { qi -= unq; ++qb; }
+                const uint32_t rc = r0 + 8 * ch;               // first query-token row of this chunk
                 if (FILTER && c < K) {
                     bool any = false;
 #pragma unroll
                     for (int e = 0; e < 8; ++e) any |= out[e] >= thr_v[ch * 8 + e];
-                    if (any) {                  // about nprobe x tile_stride keys per row in all: one lane of a warp
-                                                // every few chunks
+                    if (any) {                  // about nprobe x tile_stride keys per row in all: one lane of a warp every
+                                                // few chunks, and then hardly ever two values of the lane
+                        uint32_t pass = 0u;
 #pragma unroll
-                        for (int e = 0; e < 8; ++e) {
-                            if (out[e] >= thr_v[ch * 8 + e]) {  // (rows past the end have the largest threshold and
-                                                                //  zero digits: they never pass)
-                                // The slot comes back from the atomic hundreds of cycles later; the key is stored
-                                // only when this thread's next key turns up (or at the end), so nobody waits for it.
-                                if (pend_key && pend_slot < tiles.cap) pend_dst[pend_slot] = pend_key;
-                                const uint32_t row = r0 + e;
-                                pend_key = key_int(out[e], (int32_t)c);
-                                pend_dst = tiles.keys + (int64_t)row * tiles.cap;
-                                pend_slot = atomicAdd(tiles.cnt + row, 1);
-                            }
+                        for (int e = 0; e < 8; ++e) pass |= out[e] >= thr_v[ch * 8 + e] ? 1u << e : 0u;
+                        while (pass) {          // (rows past the end have the largest threshold: they never pass)
+                            const int e = __ffs(pass) - 1;
+                            pass &= pass - 1;
+                            int32_t v = out[0];
+#pragma unroll
+                            for (int x = 1; x < 8; ++x) v = e == x ? out[x] : v;
+                            // The slot comes back from the atomic hundreds of cycles later; the key is stored only when
+                            // this thread's next key turns up (or at the end), so nobody waits for it.
+                            if (pend_key && pend_slot < tiles.cap) pend_dst[pend_slot] = pend_key;
+                            const uint32_t row = rc + e;
+                            pend_key = key_int(v, (int32_t)c);
+                            pend_dst = tiles.keys + (int64_t)row * tiles.cap;
+                            pend_slot = atomicAdd(tiles.cnt + row, 1);
                         }
                     }
                 }
-                if (c < K && r0 < rows32) {
+                if (TABLE && c < K && rc < rows32) {
                     if (table8 != nullptr) {
-                        // coarse copy for the bound phase of stage 3: clamp(S >> 16, 0, 255); q_len is a multiple
-                        // of 16 here, so the 8 rows of a chunk belong to one query and the store is 8-byte aligned
-                        uint32_t w[2];
+                        // coarse copy for the bound phase of stage 3: clamp(S >> 16, 0, 255); q_len is a multiple of 16 here,
+                        // so the 16 rows of a warp belong to one query: one 16-byte store for both chunks
 #pragma unroll
                         for (int g = 0; g < 2; ++g) {
                             uint32_t v[4];
 #pragma unroll
                             for (int e = 0; e < 4; ++e) v[e] = (uint32_t)__vimin_s32_relu(out[4 * g + e] >> 16, 255);
-                            w[g] = __byte_perm(__byte_perm(v[0], v[1], 0x0040), __byte_perm(v[2], v[3], 0x0040), 0x5410);
+                            w8[2 * ch + g] =
+                                __byte_perm(__byte_perm(v[0], v[1], 0x0040), __byte_perm(v[2], v[3], 0x0040), 0x5410);
                         }
-                        // a warp's two chunks are adjacent (16 query tokens of one query): one 16-byte store for the pair
-                        if (ch == 0) {
-                            w8_carry[0] = w[0];
-                            w8_carry[1] = w[1];
-                        } else {
+                        if (ch == 1)
                             *reinterpret_cast<uint4 *>(table8 + ((int64_t)qb * K + c) * nq + qi - 8) =
-                                make_uint4(w8_carry[0], w8_carry[1], w[0], w[1]);
-                        }
+                                make_uint4(w8[0], w8[1], w8[2], w8[3]);
                     }
                     if ((nq & 7) == 0) {
                         // the chunk's eight values are consecutive tokens of one query, 32-byte aligned: one store
@@ -326,10 +330,12 @@ score_table_umma(const int8_t *__restrict__ cdig, const __grid_constant__ CUtens
                                      "r"(out[0]), "r"(out[1]), "r"(out[2]), "r"(out[3]), "r"(out[4]), "r"(out[5]),
                                      "r"(out[6]), "r"(out[7])
                                      : "memory");
+                        qi += 8;
+                        if (qi >= unq) { qi -= unq; ++qb; }
                     } else if ((nq & 3) == 0) {
 #pragma unroll
                         for (int e = 0; e < 8; e += 4) {
-                            if (r0 + e < rows32)                          // q_rows is a multiple of 4 here
+                            if (rc + e < rows32)                          // q_rows is a multiple of 4 here
                                 *reinterpret_cast<int4 *>(table + ((int64_t)qb * K + c) * nq + qi) =
                                     make_int4(out[e], out[e + 1], out[e + 2], out[e + 3]);
                             qi += 4;
@@ -338,7 +344,7 @@ score_table_umma(const int8_t *__restrict__ cdig, const __grid_constant__ CUtens
                     } else {
 #pragma unroll
                         for (int e = 0; e < 8; ++e) {
-                            if (r0 + e < rows32) table[((int64_t)qb * K + c) * nq + qi] = out[e];
+                            if (rc + e < rows32) table[((int64_t)qb * K + c) * nq + qi] = out[e];
                             if (++qi == unq) { qi = 0; ++qb; }
                         }
                     }
@@ -392,7 +398,7 @@ int make_plane_map(CUtensorMap *map, const int8_t *planes, int64_t rows, int box
 }
 
 // One launch of the kernel over `c_tiles` centroid tiles (see G1Tiles for which).
-template <bool FILTER>
+template <bool FILTER, bool TABLE>
 static int launch_g1_tiles(const Index &ix, const Params &p, const CUtensorMap &map_q, int c_tiles, int32_t *table,
                            uint8_t *table8, uint32_t *status, const G1Tiles &tiles, cudaStream_t st)
 {
@@ -400,7 +406,8 @@ static int launch_g1_tiles(const Index &ix, const Params &p, const CUtensorMap &
     const int n_tiles = (int)((rows + G1_N - 1) / G1_N);
     // about eight waves of two CTAs per SM, so the last wave is mostly full; a launch over few centroid tiles (the
     // sample) fills one wave instead, because a CTA's start-up costs as much as three tiles
-    int splits = c_tiles < 2 * ix.sm_count ? (2 * ix.sm_count) / c_tiles : (16 * ix.sm_count + c_tiles - 1) / c_tiles;
+    // -- unless it will hardly ever have anything to do (redo): then one CTA per centroid tile
+    int splits = tiles.redo ? 1 : c_tiles < 2 * ix.sm_count ? (2 * ix.sm_count) / c_tiles : (16 * ix.sm_count + c_tiles - 1) / c_tiles;
     if (splits > n_tiles) splits = n_tiles;
     if (splits < 1) splits = 1;
     const int tiles_per_split = (n_tiles + splits - 1) / splits;
@@ -409,9 +416,9 @@ static int launch_g1_tiles(const Index &ix, const Params &p, const CUtensorMap &
     const int skip = fault_skip_tma_loads();
 #define CHIMERA_G1_LAUNCH(KS)                                                                                          \
     do {                                                                                                               \
-        CHIMERA_CUDA(cudaFuncSetAttribute(score_table_umma<KS, FILTER>, cudaFuncAttributeMaxDynamicSharedMemorySize,   \
+        CHIMERA_CUDA(cudaFuncSetAttribute(score_table_umma<KS, FILTER, TABLE>, cudaFuncAttributeMaxDynamicSharedMemorySize,   \
                                           (int)G1_SMEM));                                                              \
-        launch(score_table_umma<KS, FILTER>, grid, G1_THREADS, G1_SMEM, st, ix.cdig, map_q, ix.K, p.nq, rows, n_tiles,     \
+        launch(score_table_umma<KS, FILTER, TABLE>, grid, G1_THREADS, G1_SMEM, st, ix.cdig, map_q, ix.K, p.nq, rows, n_tiles,     \
                                                                         tiles_per_split, table, table8, status, limit, \
                                                                         skip, tiles);                                  \
     } while (0)
@@ -434,8 +441,8 @@ int launch_score_table(const Index &ix, const Params &p, const float *queries, i
     if (rc) return rc;
     CUtensorMap map_q;
     if ((rc = make_plane_map(&map_q, qdig, rows, G1_N, 3))) return rc;        // one load brings a tile's three planes
-    const G1Tiles all = {0, 0, nullptr, nullptr, nullptr, 0};
-    if ((rc = launch_g1_tiles<false>(ix, p, map_q, (int)((ix.K + G1_M - 1) / G1_M), table, table8, status, all, st)))
+    const G1Tiles all = {0, 0, nullptr, nullptr, nullptr, 0, nullptr};
+    if ((rc = launch_g1_tiles<false, true>(ix, p, map_q, (int)((ix.K + G1_M - 1) / G1_M), table, table8, status, all, st)))
         return rc;
     count_launch(SLOT_G1, 2);
     return CHIMERA_OK;
@@ -448,7 +455,7 @@ int launch_score_table(const Index &ix, const Params &p, const float *queries, i
 // descending, centroid id ascending): a centroid that belongs to it has a score >= the bound, so it is queued.
 // A query with a token whose queue overflowed is redone by the table scan of the separate probe stage.
 int launch_score_table_probes(const Index &ix, const Params &p, const Layout &L, const float *queries, int8_t *qdig, int8_t *qdig4,
-                              int32_t *table, uint8_t *table8, char *ws, uint32_t *status, cudaStream_t st,
+                              int32_t *table, bool keep_table, uint8_t *table8, char *ws, uint32_t *status, cudaStream_t st,
                               uint32_t *clear, int64_t clear_n)
 {
     const int64_t rows = (int64_t)p.B * p.nq;
@@ -462,13 +469,28 @@ int launch_score_table_probes(const Index &ix, const Params &p, const Layout &L,
     int32_t *thr = (int32_t *)(ws + L.pq_thr), *cnt = (int32_t *)(ws + L.pq_cnt);
     unsigned long long *keys = (unsigned long long *)(ws + L.pq_keys);
 
-    const G1Tiles sample = {stride, 1, nullptr, nullptr, nullptr, 0};
-    if ((rc = launch_g1_tiles<false>(ix, p, map_q, n_sample, table, table8, status, sample, st))) return rc;
+    const G1Tiles sample = {stride, 1, nullptr, nullptr, nullptr, 0, nullptr};
+    if ((rc = launch_g1_tiles<false, true>(ix, p, map_q, n_sample, table, table8, status, sample, st))) return rc;
     if ((rc = launch_probe_sample(ix, p, L, table, ws, n_sample, st))) return rc;
-    const G1Tiles rest = {stride, 0, thr, cnt, keys, L.pq_cap};
-    if ((rc = launch_g1_tiles<true>(ix, p, map_q, c_tiles - n_sample, table, table8, status, rest, st))) return rc;
+    const G1Tiles rest = {stride, 0, thr, cnt, keys, L.pq_cap, nullptr};
+    rc = keep_table ? launch_g1_tiles<true, true>(ix, p, map_q, c_tiles - n_sample, table, table8, status, rest, st)
+                    : launch_g1_tiles<true, false>(ix, p, map_q, c_tiles - n_sample, nullptr, nullptr, status, rest, st);
+    if (rc) return rc;
     count_launch(SLOT_G1, 3);
     return CHIMERA_OK;
+}
+
+// The tiles that launch_score_table_probes left out of the table (keep_table false), for the queries that `redo` flags.
+int launch_score_table_redo(const Index &ix, const Params &p, const Layout &L, const int8_t *qdig, int32_t *table,
+                            const int32_t *redo, uint32_t *status, cudaStream_t st)
+{
+    CUtensorMap map_q;
+    const int rc = make_plane_map(&map_q, qdig, (int64_t)p.B * p.nq, G1_N, 3);
+    if (rc) return rc;
+    const int c_tiles = (int)((ix.K + G1_M - 1) / G1_M);
+    const int n_sample = (c_tiles + L.pq_stride - 1) / L.pq_stride;
+    const G1Tiles rest = {L.pq_stride, 0, nullptr, nullptr, nullptr, 0, redo};
+    return launch_g1_tiles<false, true>(ix, p, map_q, c_tiles - n_sample, table, nullptr, status, rest, st);
 }
 
 }  // namespace chimera

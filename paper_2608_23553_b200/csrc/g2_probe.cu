@@ -473,7 +473,8 @@ int launch_probe_sample(const Index &ix, const Params &p, const Layout &L, const
     return CHIMERA_OK;
 }
 
-int launch_probe_merge(const Index &ix, const Params &p, const Layout &L, const int32_t *table, char *ws, cudaStream_t st)
+int launch_probe_merge(const Index &ix, const Params &p, const Layout &L, int32_t *table, const int8_t *redo_qdig, char *ws,
+                       uint32_t *status, cudaStream_t st)
 {
     const int64_t rows = (int64_t)p.B * p.nq;
     const int32_t *cnt = (const int32_t *)(ws + L.pq_cnt);
@@ -485,7 +486,12 @@ int launch_probe_merge(const Index &ix, const Params &p, const Layout &L, const 
                                                                                                L.pq_cap, probes, ovf);
     CHIMERA_CUDA(cudaGetLastError());
     // queries with an overflowed queue (none, except for inputs with masses of equal scores): the table scan, whose
-    // blocks return at once for every other query
+    // blocks return at once for every other query -- and first their part of the table, when it was not kept
+    if (redo_qdig) {
+        const int rc = launch_score_table_redo(ix, p, L, redo_qdig, table, ovf, status, st);
+        if (rc) return rc;
+        count_launch(SLOT_PROBE);
+    }
     const size_t smem = sizeof(unsigned long long) * (size_t)p.P * PROBE_THREADS;
     if (smem > 48 * 1024)
         CHIMERA_CUDA(cudaFuncSetAttribute(probe_partial, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));

@@ -2,14 +2,14 @@
 // first, ties towards the smaller document id; missing entries are (-1, -inf).
 //
 // One block per query.  Each (score, id) becomes a 64-bit key whose unsigned order is (score desc, id asc); the keys
-// are sorted descending with a bitonic network in shared memory (n_prune <= 16384 keys = 128 KB) and the first k are
-// decoded back.  For k <= 16 the keys stay in registers instead and the block extracts its maximum k times (two
+// (those that reach the k-th score, when k is small beside them) are sorted descending with a bitonic network in shared
+// memory (n_prune <= 16384 keys = 128 KB) and the first k are decoded back.  For k <= 16 the keys stay in registers instead and the block extracts its maximum k times (two
 // barriers per result instead of the network's log^2 stages), and for k <= 128 over at most 4096 entries the warps sort
 // 128-key runs in registers and merge them pairwise, keeping the better half each time: the shorter chains matter
 // when one query is served at a time.
 #include <math.h>
 
-#include "common.cuh"
+#include "g3_select.cuh"
 
 namespace chimera {
 
@@ -34,12 +34,34 @@ __device__ __forceinline__ int64_t entry_index(int j, int b, int seg_len, long l
     return (int64_t)(j / seg_len) * seg_stride + (int64_t)b * seg_len + j % seg_len;
 }
 
+// Descending bitonic sort of n_pow2 keys in shared memory; whole block.
+__device__ __forceinline__ void bitonic_sort(unsigned long long *keys, int n_pow2)
+{
+    for (int size = 2; size <= n_pow2; size <<= 1) {
+        for (int stride = size >> 1; stride > 0; stride >>= 1) {
+            for (int t = threadIdx.x; t < (n_pow2 >> 1); t += TOPK_THREADS) {
+                int lo = 2 * t - (t & (stride - 1));      // index with the stride bit clear
+                int hi = lo + stride;
+                bool descending = (lo & size) == 0;
+                unsigned long long a = keys[lo], c = keys[hi];
+                if ((a < c) == descending) { keys[lo] = c; keys[hi] = a; }
+            }
+            __syncthreads();
+        }
+    }
+}
+
+// SELECT (at least four times as many entries as wanted): the k-th largest score by radix select, then only the entries
+// that reach it are sorted (16,384 entries, k = 1,000: 185 us for sorting all, XX with the selection).  More ties at that
+// score than the second array holds: everything is sorted after all.
+template <bool SELECT>
 __global__ void __launch_bounds__(TOPK_THREADS)
-topk_kernel(const int32_t *__restrict__ pruned, const float *__restrict__ score4, int n_prune, int n_pow2, int k,
+topk_kernel(const int32_t *__restrict__ pruned, const float *__restrict__ score4, int n_prune, int n_pow2, int cap, int k,
             int seg_len, long long seg_stride, int32_t *__restrict__ out_ids, float *__restrict__ out_scores)
 {
     pdl_entry();
-    extern __shared__ unsigned long long keys[];
+    extern __shared__ unsigned long long topk_keys[];
+    unsigned long long *keys = topk_keys;
     const int b = blockIdx.x;
     for (int j = threadIdx.x; j < n_pow2; j += TOPK_THREADS) {
         unsigned long long key = 0ull;
@@ -52,17 +74,36 @@ topk_kernel(const int32_t *__restrict__ pruned, const float *__restrict__ score4
         keys[j] = key;
     }
     __syncthreads();
-    for (int size = 2; size <= n_pow2; size <<= 1) {
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            for (int t = threadIdx.x; t < (n_pow2 >> 1); t += TOPK_THREADS) {
-                int lo = 2 * t - (t & (stride - 1));      // index with the stride bit clear
-                int hi = lo + stride;
-                bool descending = (lo & size) == 0;
-                unsigned long long a = keys[lo], c = keys[hi];
-                if ((a < c) == descending) { keys[lo] = c; keys[hi] = a; }
+    if (SELECT) {
+        __shared__ int hist[2048];
+        __shared__ int warp_part[32];
+        __shared__ uint32_t s_prefix;
+        __shared__ int s_want, s_count;
+        if (threadIdx.x == 0) s_count = 0;
+        int need_eq;
+        const uint32_t thr = radix_select([&](int j) { return (int)((uint32_t)(keys[j] >> 32) ^ 0x80000000u); }, n_prune, k, hist,
+                                          warp_part, &s_prefix, &s_want, &need_eq);
+        unsigned long long *best = keys + n_pow2;         // room for 2 * pow2(k)
+        for (int j = threadIdx.x; j < n_prune; j += TOPK_THREADS)
+            if ((uint32_t)(keys[j] >> 32) >= thr) {
+                const int at = atomicAdd(&s_count, 1);
+                if (at < cap) best[at] = keys[j];
             }
+        __syncthreads();
+        const int cnt = s_count;
+        if (cnt <= cap) {
+            int m = 2;
+            while (m < cnt) m <<= 1;
+            for (int j = cnt + threadIdx.x; j < m; j += TOPK_THREADS) best[j] = 0ull;
             __syncthreads();
+            bitonic_sort(best, m);
+            keys = best;
+            n_pow2 = m;
+        } else {
+            bitonic_sort(keys, n_pow2);
         }
+    } else {
+        bitonic_sort(keys, n_pow2);
     }
     for (int r = threadIdx.x; r < k; r += TOPK_THREADS) {
         unsigned long long key = r < n_pow2 ? keys[r] : 0ull;
@@ -256,10 +297,14 @@ static int launch_topk_entries(const int32_t *ids, const float *scores, int B, i
     while (n_pow2 < n) n_pow2 <<= 1;
     const size_t smem = sizeof(unsigned long long) * (size_t)n_pow2;
     if (smem > 128 * 1024) return fail(CHIMERA_UNSUPPORTED, "top-k over %d entries per query does not fit shared memory", n);
-    if (smem > 48 * 1024)
-        CHIMERA_CUDA(cudaFuncSetAttribute(topk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    launch(topk_kernel, (unsigned)B, TOPK_THREADS, smem, st, ids, scores, n, n_pow2, k, seg_len, seg_stride, out_ids,
-                                                         out_scores);
+    int cap = 4;
+    while (cap < 2 * k) cap <<= 1;
+    const bool select = n >= 4 * k && n > 2048;
+    const size_t bytes = smem + (select ? sizeof(unsigned long long) * (size_t)cap : 0);
+    auto kern = select ? topk_kernel<true> : topk_kernel<false>;
+    if (bytes > 48 * 1024 - 16 * 1024)                    // (the selection has 8 KB of its own)
+        CHIMERA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    launch(kern, (unsigned)B, TOPK_THREADS, bytes, st, ids, scores, n, n_pow2, cap, k, seg_len, seg_stride, out_ids, out_scores);
     CHIMERA_CUDA(cudaGetLastError());
     return CHIMERA_OK;
 }

@@ -20,8 +20,9 @@
 
 namespace chimera {
 
-constexpr int GP_WARPS = 4;              // query tokens (warps) per block
-constexpr int GP_PIPE = 8;               // centroid rows in flight per warp while scoring
+constexpr int GP_WARPS = 4;              // warps per query token
+constexpr int GP_PIPE = 4;               // centroid rows in flight per warp while scoring
+constexpr int GP_BATCH = GP_WARPS * 32;  // centroids per step
 
 // Xc[c][d] = rint(centroid * 2^22), recombined from the three balanced base-256 digit planes of the index.
 __global__ void xc_kernel(const int8_t *__restrict__ cdig, int64_t K, int D, int nbits, int32_t *__restrict__ xc)
@@ -128,17 +129,25 @@ __device__ __forceinline__ unsigned long long gp_key(int32_t score, int32_t id)
 __device__ __forceinline__ int32_t gp_id(unsigned long long key) { return 0x7FFFFFFF - (int32_t)((uint32_t)key >> 1); }
 __device__ __forceinline__ int32_t gp_score(unsigned long long key) { return (int32_t)((uint32_t)(key >> 32) ^ 0x80000000u); }
 
-// grid (ceil(tokens / GP_WARPS)); visited: [tokens][vwords] zeroed by the caller.
-__global__ void __launch_bounds__(GP_WARPS * 32)
-graph_probe_kernel(const float *__restrict__ queries, int64_t n_tokens, int D, const int32_t *__restrict__ xc,
+// grid (tokens), one block of four warps per query token.  The search is a chain -- best unexpanded member -> its neighbours ->
+// which are new -> their rows -> their scores -> the list -- so it is latency that counts: the visited set is a bitmap in
+// shared memory (SHARED; written out at the end when wanted), all warps fetch and score the new centroids of a step
+// together, and warp 0 keeps the list in registers and looks only at scores that rank inside it.  With one warp per token,
+// a bitmap in global memory and every score offered in turn, Mid's 2,048 tokens of a batch of 64 took 860 us; now XX.
+// visited (NULL: not wanted; !SHARED: [tokens][vwords] zeroed by the caller).
+template <bool SHARED>
+__global__ void __launch_bounds__(GP_WARPS * 32, 8)
+graph_probe_kernel(const float *__restrict__ queries, int D, const int32_t *__restrict__ xc,
                    const int32_t *__restrict__ graph, int R, int64_t K, int n_entries, int beam, int max_exp,
                    int nprobe, uint32_t *__restrict__ visited, int64_t vwords, int32_t *__restrict__ out_probes,
                    int32_t *__restrict__ out_scores, int32_t *__restrict__ out_nvis)
 {
     pdl_entry();
-    const int lane = threadIdx.x & 31;
-    const int64_t token = (int64_t)blockIdx.x * GP_WARPS + (threadIdx.x >> 5);
-    if (token >= n_tokens) return;                       // whole warps leave together
+    extern __shared__ uint32_t s_vis[];
+    __shared__ int32_t s_ids[GP_BATCH], s_sc[GP_BATCH];
+    __shared__ int s_n, s_next;                          // centroids of the step; the member to expand (-1: none)
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t token = blockIdx.x;
     const bool has_dims = 4 * lane < D;                  // lane owns dimensions 4 lane .. 4 lane + 3
     int xq[4] = {0, 0, 0, 0};
     if (has_dims) {
@@ -148,13 +157,17 @@ graph_probe_kernel(const float *__restrict__ queries, int64_t n_tokens, int D, c
         xq[2] = __float2int_rn(fminf(fmaxf(v.z, -1.0f), 1.0f) * 4194304.0f);
         xq[3] = __float2int_rn(fminf(fmaxf(v.w, -1.0f), 1.0f) * 4194304.0f);
     }
-    uint32_t *vis = visited + token * vwords;
-    unsigned long long key0 = 0ull, key1 = 0ull;         // list slots lane and 32 + lane, best first
+    uint32_t *vis = SHARED ? s_vis : visited + token * vwords;
+    if (SHARED)
+        for (int w = tid; w < (int)vwords; w += GP_WARPS * 32) s_vis[w] = 0u;
+    if (tid == 0) s_n = 0;
+    __syncthreads();
+
+    unsigned long long key0 = 0ull, key1 = 0ull;         // warp 0: list slots lane and 32 + lane, best first
     int n_vis = 0;
 
-    // offer a scored centroid (warp-uniform arguments) to the list
-    auto offer = [&](int32_t n, int32_t s) {
-        const unsigned long long x = gp_key(s, n);
+    // offer a scored centroid (warp-uniform argument) to the list
+    auto offer = [&](unsigned long long x) {
         const int pos = __popc(__ballot_sync(0xffffffffu, (key0 >> 1) > (x >> 1))) +
                         __popc(__ballot_sync(0xffffffffu, (key1 >> 1) > (x >> 1)));
         if (pos >= beam) return;                          // ranks behind a full list
@@ -178,66 +191,93 @@ graph_probe_kernel(const float *__restrict__ queries, int64_t n_tokens, int D, c
         const long long t = ((long long)hi << 24) + (long long)lo;
         return (int32_t)((t + (1LL << 19)) >> 20);
     };
-    // visit up to 32 centroids, one per lane: mark, then score the unvisited ones GP_PIPE rows at a time
-    auto visit = [&](int32_t n, bool valid) {
-        bool fresh = false;
-        if (valid) {
-            n = DBG_CID(n);
-            const uint32_t bit = 1u << (n & 31);
-            fresh = (atomicOr(&vis[n >> 5], bit) & bit) == 0u;
-        }
-        uint32_t todo = __ballot_sync(0xffffffffu, fresh);
-        n_vis += __popc(todo);
-        while (todo) {
-            int32_t ids[GP_PIPE];
+    // this thread's centroid of the step: into s_ids when it was never visited (order does not matter: the list is the best
+    // `beam` of everything offered)
+    auto collect = [&](int32_t n) {
+        n = DBG_CID(n);
+        const uint32_t bit = 1u << (n & 31);
+        if ((atomicOr(&vis[n >> 5], bit) & bit) == 0u) s_ids[atomicAdd(&s_n, 1)] = n;
+    };
+    // the step's centroids (at most GP_BATCH): scored by all warps, offered by warp 0.  Two barriers; s_n is 0 afterwards.
+    auto score_and_offer = [&]() {
+        __syncthreads();
+        const int cnt = s_n;
+        for (int k0 = warp; k0 < cnt; k0 += GP_WARPS * GP_PIPE) {
             int4 rows[GP_PIPE];
-            int cnt = 0;
 #pragma unroll
             for (int u = 0; u < GP_PIPE; ++u) {
-                if (todo) {
-                    const int src = __ffs(todo) - 1;
-                    todo &= todo - 1;
-                    ids[u] = __shfl_sync(0xffffffffu, n, src);
-                    rows[u] = make_int4(0, 0, 0, 0);
-                    if (has_dims) rows[u] = __ldg(reinterpret_cast<const int4 *>(xc + (int64_t)ids[u] * D) + lane);
-                    cnt = u + 1;
-                }
+                const int k = k0 + GP_WARPS * u;
+                rows[u] = make_int4(0, 0, 0, 0);
+                if (k < cnt && has_dims) rows[u] = __ldg(reinterpret_cast<const int4 *>(xc + (int64_t)s_ids[k] * D) + lane);
             }
 #pragma unroll
-            for (int u = 0; u < GP_PIPE; ++u)
-                if (u < cnt) offer(ids[u], finish_score(rows[u]));
+            for (int u = 0; u < GP_PIPE; ++u) {
+                const int k = k0 + GP_WARPS * u;
+                if (k < cnt) {
+                    const int32_t sc = finish_score(rows[u]);
+                    if (lane == 0) s_sc[k] = sc;
+                }
+            }
+        }
+        __syncthreads();
+        if (warp == 0) {
+            n_vis += cnt;
+            for (int k0 = 0; k0 < cnt; k0 += 32) {
+                const int k = k0 + lane;
+                const unsigned long long mine = k < cnt ? gp_key(s_sc[k], s_ids[k]) : 0ull;
+                for (uint32_t left = __ballot_sync(0xffffffffu, k < cnt); left;) {
+                    // the keys that rank inside the list as it is now (it only gets better)
+                    const unsigned long long last = beam <= 32 ? __shfl_sync(0xffffffffu, key0, beam - 1)
+                                                               : __shfl_sync(0xffffffffu, key1, beam - 33);
+                    left &= __ballot_sync(0xffffffffu, (mine >> 1) > (last >> 1));
+                    if (!left) break;
+                    const int src = __ffs(left) - 1;
+                    left &= left - 1;
+                    offer(__shfl_sync(0xffffffffu, mine, src));
+                }
+            }
+            if (lane == 0) s_n = 0;
         }
     };
 
-    for (int j0 = 0; j0 < n_entries; j0 += 32) {
-        const int j = j0 + lane;
-        visit((int32_t)(((long long)j * K) / n_entries), j < n_entries);
+    for (int j0 = 0; j0 < n_entries; j0 += GP_WARPS * 32) {
+        const int j = j0 + tid;
+        if (j < n_entries) collect((int32_t)(((long long)j * K) / n_entries));
+        score_and_offer();
+        __syncthreads();
     }
     for (int done = 0; done < max_exp; ++done) {
-        const uint32_t u0 = __ballot_sync(0xffffffffu, (key0 & 1ull) != 0ull);
-        const uint32_t u1 = __ballot_sync(0xffffffffu, (key1 & 1ull) != 0ull);
-        if ((u0 | u1) == 0u) break;                      // every member expanded
-        int32_t p;
-        if (u0) {
-            const int src = __ffs(u0) - 1;
-            p = gp_id(__shfl_sync(0xffffffffu, key0, src));
-            if (lane == src) key0 &= ~1ull;
-        } else {
-            const int src = __ffs(u1) - 1;
-            p = gp_id(__shfl_sync(0xffffffffu, key1, src));
-            if (lane == src) key1 &= ~1ull;
+        if (warp == 0) {
+            const uint32_t u0 = __ballot_sync(0xffffffffu, (key0 & 1ull) != 0ull);
+            const uint32_t u1 = __ballot_sync(0xffffffffu, (key1 & 1ull) != 0ull);
+            int32_t p = -1;                              // every member expanded
+            if (u0) {
+                const int src = __ffs(u0) - 1;
+                p = gp_id(__shfl_sync(0xffffffffu, key0, src));
+                if (lane == src) key0 &= ~1ull;
+            } else if (u1) {
+                const int src = __ffs(u1) - 1;
+                p = gp_id(__shfl_sync(0xffffffffu, key1, src));
+                if (lane == src) key1 &= ~1ull;
+            }
+            if (lane == 0) s_next = p;
         }
-        for (int r0 = 0; r0 < R; r0 += 32) {
-            const int r = r0 + lane;
-            visit(r < R ? graph[(int64_t)p * R + r] : 0, r < R);
+        __syncthreads();
+        const int32_t p = s_next;
+        if (p < 0) break;
+        if (tid < R) collect(__ldg(graph + (int64_t)p * R + tid));          // (R <= 63)
+        score_and_offer();
+    }
+    if (warp == 0) {
+        for (int r = lane; r < nprobe; r += 32) {
+            const unsigned long long k = r < 32 ? key0 : key1;   // r = lane or lane + 32
+            out_probes[token * nprobe + r] = k ? gp_id(k) : -1;
+            if (out_scores) out_scores[token * nprobe + r] = k ? gp_score(k) : INT32_MIN;
         }
+        if (out_nvis && lane == 0) out_nvis[token] = n_vis;
     }
-    for (int r = lane; r < nprobe; r += 32) {
-        const unsigned long long k = r < 32 ? key0 : key1;   // r = lane or lane + 32
-        out_probes[token * nprobe + r] = k ? gp_id(k) : -1;
-        if (out_scores) out_scores[token * nprobe + r] = k ? gp_score(k) : INT32_MIN;
-    }
-    if (out_nvis && lane == 0) out_nvis[token] = n_vis;
+    if (SHARED && visited)
+        for (int w = tid; w < (int)vwords; w += GP_WARPS * 32) visited[token * vwords + w] = s_vis[w];
 }
 
 size_t graph_scratch_bytes(const Index &ix, int64_t n_tokens)
@@ -256,14 +296,18 @@ int check_graph_params(const Index &ix, const GraphSearch &g, int nprobe)
 }
 
 int launch_graph_probes(const Index &ix, const float *queries, int64_t n_tokens, int nprobe, const GraphSearch &g,
-                        uint32_t *visited, int32_t *out_probes, int32_t *out_scores, int32_t *out_nvis, cudaStream_t st)
+                        uint32_t *visited, bool want_visited, int32_t *out_probes, int32_t *out_scores, int32_t *out_nvis,
+                        cudaStream_t st)
 {
     const int64_t vwords = (ix.K + 31) / 32;
-    CHIMERA_CUDA(cudaMemsetAsync(visited, 0, graph_scratch_bytes(ix, n_tokens), st));
-    const unsigned blocks = (unsigned)((n_tokens + GP_WARPS - 1) / GP_WARPS);
-    launch(graph_probe_kernel, blocks, GP_WARPS * 32, 0, st, queries, n_tokens, ix.D, ix.xc, ix.graph, ix.graph_deg, ix.K,
-                                                         g.n_entries, g.beam, g.max_expansions, nprobe, visited, vwords,
-                                                         out_probes, out_scores, out_nvis);
+    const size_t smem = sizeof(uint32_t) * (size_t)vwords;
+    const bool shared = smem <= 128 * 1024;              // a million centroids
+    auto kern = shared ? graph_probe_kernel<true> : graph_probe_kernel<false>;
+    if (shared) CHIMERA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    else CHIMERA_CUDA(cudaMemsetAsync(visited, 0, graph_scratch_bytes(ix, n_tokens), st));
+    launch(kern, (unsigned)n_tokens, GP_WARPS * 32, shared ? smem : 0, st, queries, ix.D, ix.xc, ix.graph, ix.graph_deg, ix.K,
+           g.n_entries, g.beam, g.max_expansions, nprobe, shared && !want_visited ? nullptr : visited, vwords, out_probes,
+           out_scores, out_nvis);
     CHIMERA_CUDA(cudaGetLastError());
     count_launch(SLOT_PROBE, 1);
     return CHIMERA_OK;

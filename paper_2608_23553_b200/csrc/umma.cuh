@@ -134,7 +134,6 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, int32_t (&r)[8])
                  : "r"(taddr)
                  : "memory");
 }
-
 __device__ __forceinline__ void tmem_alloc(uint32_t *smem_dst, uint32_t ncols)      // whole warp
 {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(smem_dst)), "r"(ncols)
