@@ -112,7 +112,7 @@ Layout make_layout(const Index &ix, const Params &p)
     const size_t rows4 = B * (size_t)residual_rows(p.nq);
     L.qdig4 = take(3 * rows4 * 128);
     L.table = take(B * (size_t)ix.K * nq * sizeof(int32_t));
-    L.table8 = take(coarse_supported(p.nq) ? B * (size_t)ix.K * nq : 0);
+    L.table8 = take(coarse_supported(p.nq) || filter_used(ix, p) ? B * (size_t)ix.K * coarse_pitch(p.nq) : 0);
     L.pq_stride = probe_queue_stride(ix, p);
     L.pq_groups = L.pq_stride ? probe_sample_groups(ix, L.pq_stride) : 0;
     L.part = take(B * L.n_part * p.P * nq * sizeof(unsigned long long));
@@ -389,7 +389,7 @@ static int run(const Index &ix, const Params &p, int first, int last, const floa
                 (rc = launch_cand_ranges(ix, p, cand, n_cand, scan_rng, ci, st)))
                 return rc;
             if (filter) {
-                if ((rc = launch_filter_scan(ix, p, L, table, table8, cand, n_cand, hi, cont, cont_rng, ws, st)))
+                if ((rc = launch_filter_scan(ix, p, L, table, (uint8_t *)(ws + L.table8), cand, n_cand, hi, cont, cont_rng, ws, st)))
                     return rc;
                 if ((rc = launch_centroid_interaction(ix, p, table, cont, (const int32_t *)(ws + L.n_seed), ci, exact_blocks,
                                                       SLOT_CI, cont_rng, st)))
@@ -400,14 +400,14 @@ static int run(const Index &ix, const Params &p, int first, int last, const floa
                 if ((rc = launch_filter_keep(ix, p, L, cand, n_cand, hi, ci, kept, kept_rng, n_kept, ws, st))) return rc;
                 prof_mark(SLOT_SELECT, st);
                 docs = kept; n_docs = n_kept; docs_rng = kept_rng;
-                if (two_phase) {                   // upper bounds of the kept ones from the 8-bit table
-                    if ((rc = launch_coarse_bounds(ix, p, table8, docs, n_docs, nullptr, hi, docs_rng, st))) return rc;
-                    prof_mark(SLOT_CI, st);
-                    if ((rc = launch_filter_contenders(ix, p, L, docs, docs_rng, n_docs, hi, cont, cont_rng, n_cont, ws, st)))
-                        return rc;
-                    prof_mark(SLOT_SELECT, st);
-                    docs = cont; n_docs = n_cont; docs_rng = cont_rng;
-                }
+                // upper bounds of the kept ones from the 8-bit table
+                if ((rc = launch_coarse_bounds(ix, p, (uint8_t *)(ws + L.table8), docs, n_docs, nullptr, hi, docs_rng, st)))
+                    return rc;
+                prof_mark(SLOT_CI, st);
+                if ((rc = launch_filter_contenders(ix, p, L, docs, docs_rng, n_docs, hi, cont, cont_rng, n_cont, ws, st)))
+                    return rc;
+                prof_mark(SLOT_SELECT, st);
+                docs = cont; n_docs = n_cont; docs_rng = cont_rng;
             } else if (two_phase) {
                 // bounds for every candidate, contenders for the top n_prune, exact CI and selection among those
                 if ((rc = launch_coarse_bounds(ix, p, table8, docs, n_docs, lo, hi, docs_rng, st))) return rc;
@@ -463,7 +463,7 @@ static int run(const Index &ix, const Params &p, int first, int last, const floa
             }
             if (taps->n_contenders &&
                 (rc = copy_d2d(taps->n_contenders,
-                               two_phase ? n_cont : filter ? (int32_t *)(ws + L.n_kept) : n_cand,
+                               two_phase || filter ? n_cont : n_cand,
                                B * sizeof(int32_t), st)))
                 return rc;
             if (taps->pruned && (rc = copy_d2d(taps->pruned, pruned, pruned_bytes, st))) return rc;

@@ -241,6 +241,7 @@ int launch_filter_contenders(const Index &ix, const Params &p, const Layout &L, 
                              const int32_t *n_kept, const int32_t *hi, int32_t *cont, int2 *cont_rng, int32_t *n_cont,
                              char *ws, cudaStream_t st);
 bool coarse_supported(int nq);
+int coarse_pitch(int nq);       // bytes of an 8-bit row
 int launch_coarse_table(const Index &ix, const Params &p, const int32_t *table, uint8_t *table8, cudaStream_t st);
 // The candidates' token ranges (corpora with fewer than 2^31 tokens); also clears the contender step's histograms at the
 // head of its scratch rows (int32 [B][maxc]) where launch_contenders will use them.
@@ -259,7 +260,7 @@ size_t filter_table_pitch(const Index &ix);
 int filter_hist_bins();
 int filter_count_slots();
 size_t filter_parts_bytes(const Index &ix, const Params &p);
-int launch_filter_scan(const Index &ix, const Params &p, const Layout &L, const int32_t *table, const uint8_t *table8,
+int launch_filter_scan(const Index &ix, const Params &p, const Layout &L, const int32_t *table, uint8_t *table8,
                        const int32_t *cand, const int32_t *n_cand, int32_t *hi0, int32_t *seed,
                        int2 *seed_rng, char *ws, cudaStream_t st);
 int launch_filter_keep(const Index &ix, const Params &p, const Layout &L, const int32_t *cand,

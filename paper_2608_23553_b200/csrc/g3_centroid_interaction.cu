@@ -30,7 +30,9 @@ namespace chimera {
 constexpr int CI_THREADS = 256;
 constexpr int CI_WARPS = CI_THREADS / 32;
 
-// rng: NULL, or the documents' token ranges (first token, length); (CI, 0) stands for a document whose CI is known.
+// Any q_len.  rng: NULL, or the documents' token ranges (first token, length); (CI, 0) stands for a document whose CI is
+// known.  L2 is the limit (rows of 84 bytes, 59,000 documents of 173 tokens: 1.1 GB of sectors in 332 us); the next 32
+// centroid ids are loaded ahead of the rows.
 template <int NQW>   // 32-column groups handled per lane
 __global__ void __launch_bounds__(CI_THREADS)
 ci_kernel(const int32_t *__restrict__ table, int64_t K, int nq, const int32_t *__restrict__ cand,
@@ -38,6 +40,7 @@ ci_kernel(const int32_t *__restrict__ table, int64_t K, int nq, const int32_t *_
           const int64_t *__restrict__ doc_off, const int2 *__restrict__ rng, int32_t *__restrict__ ci)
 {
     pdl_entry();
+    constexpr int U = NQW == 1 ? 16 : 8;                     // rows in flight (16 of short rows: 48 us where 8 take 63)
     const int b = blockIdx.y;
     const int lane = threadIdx.x & 31;
     const int n = n_cand[b];
@@ -63,18 +66,18 @@ ci_kernel(const int32_t *__restrict__ table, int64_t K, int nq, const int32_t *_
         int m[NQW];
 #pragma unroll
         for (int w = 0; w < NQW; ++w) m[w] = INT_MIN;
+        // lanes past the end repeat the last token: a duplicate cannot change a maximum
+        int32_t next = t0 < t1 ? cids[t0 + lane < t1 ? t0 + lane : t1 - 1] : 0;
         for (int64_t base = t0; base < t1; base += 32) {
             const int cnt = (int)((t1 - base) < 32 ? (t1 - base) : 32);
-            // lanes past the end repeat the last token: a duplicate cannot change a maximum
-            const int32_t cidv = cids[base + (lane < cnt ? lane : cnt - 1)];
-            for (int t = 0; t < cnt; t += 8) {
-                int32_t c[8];
+            const int32_t cidv = next;
+            if (base + 32 < t1) next = cids[base + 32 + lane < t1 ? base + 32 + lane : t1 - 1];
+            for (int t = 0; t < cnt; t += U) {
+                int32_t v[U][NQW];
 #pragma unroll
-                for (int u = 0; u < 8; ++u) c[u] = __shfl_sync(0xffffffffu, cidv, t + u);   // t + u <= 31
-                int32_t v[8][NQW];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const int32_t *row = tb + (int64_t)DBG_CID(c[u]) * nq;
+                for (int u = 0; u < U; ++u) {
+                    const int32_t c = __shfl_sync(0xffffffffu, cidv, t + u);                // t + u <= 31
+                    const int32_t *row = tb + (int64_t)DBG_CID(c) * nq;
 #pragma unroll
                     for (int w = 0; w < NQW; ++w) {
                         int col = lane + 32 * w;
@@ -82,7 +85,7 @@ ci_kernel(const int32_t *__restrict__ table, int64_t K, int nq, const int32_t *_
                     }
                 }
 #pragma unroll
-                for (int u = 0; u < 8; ++u)
+                for (int u = 0; u < U; ++u)
 #pragma unroll
                     for (int w = 0; w < NQW; ++w) m[w] = max(m[w], v[u][w]);
             }
@@ -432,9 +435,10 @@ cand_range_kernel(const int32_t *__restrict__ cand, const int32_t *__restrict__ 
 // load), the ranges are handed out by shuffle, and while document i is scanned the first centroid ids of document
 // i + 1 are already being fetched -- a one-level prefetch where the per-document chain used to have three levels.
 // The 32 results of a group are written back coalesced.
+// nq: the columns that count; those up to 16 LPR are zero in every row (lower bounds are for nq == 16 LPR only).
 template <int LPR>
 __device__ __forceinline__ void
-ci_coarse_rng_body(const uint8_t *__restrict__ table8, int64_t K, const int2 *__restrict__ rng,
+ci_coarse_rng_body(const uint8_t *__restrict__ table8, int64_t K, int nq, const int2 *__restrict__ rng,
                      const int32_t *__restrict__ n_cand, int64_t maxc, const int32_t *__restrict__ cids,
                      int32_t *__restrict__ lo, int32_t *__restrict__ hi)
 {
@@ -445,8 +449,8 @@ ci_coarse_rng_body(const uint8_t *__restrict__ table8, int64_t K, const int2 *__
     // Measured (bound scan, batch 256): for 32-byte rows one slab without that prefetch is the fastest of the four
     // combinations (Mid 14.21 ms against 14.45 ms for two slabs with it, 14.54 / 14.75 ms for the mixed ones; Large
     // 28.2 against 28.7 ms); for 64-byte rows two slabs with the prefetch are (long documents: 28.8 against 29.1 ms).
-    constexpr int SLABS = LPR == 2 ? 1 : 2;
-    constexpr bool PREFETCH_L2 = LPR != 2;
+    constexpr int SLABS = LPR == 4 ? 2 : 1;
+    constexpr bool PREFETCH_L2 = LPR == 4;
     const int b = blockIdx.y;
     const int lane = threadIdx.x & 31;
     const int grp = lane / LPR, sub = lane % LPR;
@@ -549,14 +553,18 @@ ci_coarse_rng_body(const uint8_t *__restrict__ table8, int64_t K, const int2 *__
                     dup_mask |= (uint32_t)o;
                 }
             }
-            const int u_lo = coarse_field_lo(m[0]), u_hi = coarse_field_hi(m[0]);
             int packed = 0;                                         // sum of maxima | saturated << 16 | zeros << 24
-            if ((lane & dup_mask) == 0)
-                packed = (u_lo + u_hi) + (((u_lo >= 255) + (u_hi >= 255)) << 16) + (((u_lo == 0) + (u_hi == 0)) << 24);
+#pragma unroll
+            for (int r = 0; r < (LPR == 8 ? 2 : 1); ++r) {
+                const int u_lo = coarse_field_lo(m[r]), u_hi = coarse_field_hi(m[r]);
+                if ((lane & dup_mask) == 0)
+                    packed += (u_lo + u_hi) + (((u_lo >= 255) + (u_hi >= 255)) << 16) +
+                              (LPR == 8 ? 0 : ((u_lo == 0) + (u_hi == 0)) << 24);
+            }
             packed = __reduce_add_sync(0xffffffffu, packed);
             if (lane == di) {                                       // lane di keeps the result of document di
                 my_lo = coarse_lo(packed);
-                my_hi = coarse_hi(packed, NQ);
+                my_hi = coarse_hi(packed, nq);
             }
         }
         if (lane < cnt) {
@@ -576,7 +584,7 @@ ci_coarse_rng_kernel(const uint8_t *__restrict__ table8, int64_t K, const int2 *
                      int32_t *__restrict__ lo, int32_t *__restrict__ hi)
 {
     pdl_entry();
-    ci_coarse_rng_body<LPR>(table8, K, rng, n_cand, maxc, cids, lo, hi);
+    ci_coarse_rng_body<LPR>(table8, K, 16 * LPR, rng, n_cand, maxc, cids, lo, hi);
 }
 template <int LPR>
 __global__ void __launch_bounds__(CI_THREADS, 4)
@@ -585,10 +593,23 @@ ci_coarse_rng_kernel_b4(const uint8_t *__restrict__ table8, int64_t K, const int
                         int32_t *__restrict__ lo, int32_t *__restrict__ hi)
 {
     pdl_entry();
-    ci_coarse_rng_body<LPR>(table8, K, rng, n_cand, maxc, cids, lo, hi);
+    ci_coarse_rng_body<LPR>(table8, K, 16 * LPR, rng, n_cand, maxc, cids, lo, hi);
+}
+
+// Other query lengths, rows padded to 32, 64 or 128 bytes (made beside the first cut's excess table): 28 M lookups for 8
+// queries of 100 tokens in 213 us, where the exact rows took 860.
+template <int LPR>
+__global__ void __launch_bounds__(CI_THREADS, LPR == 2 ? 4 : 3)
+ci_coarse_rng_kernel_pad(const uint8_t *__restrict__ table8, int64_t K, int nq, const int2 *__restrict__ rng,
+                         const int32_t *__restrict__ n_cand, int64_t maxc, const int32_t *__restrict__ cids,
+                         int32_t *__restrict__ hi)
+{
+    pdl_entry();
+    ci_coarse_rng_body<LPR>(table8, K, nq, rng, n_cand, maxc, cids, nullptr, hi);
 }
 
 bool coarse_supported(int nq) { return nq == 32 || nq == 64; }
+int coarse_pitch(int nq) { return nq <= 32 ? 32 : nq <= 64 ? 64 : 128; }
 
 // Several blocks per query in the contender step: few queries with long candidate lists (one block reads 100,000 candidates
 // in about 40 us, and 16,384 in the time of the two more launches).
@@ -612,7 +633,7 @@ int launch_cand_ranges(const Index &ix, const Params &p, const int32_t *cand, co
 int launch_coarse_bounds(const Index &ix, const Params &p, const uint8_t *table8, const int32_t *cand,
                          const int32_t *n_cand, int32_t *lo, int32_t *hi, const int2 *rng, cudaStream_t st)
 {
-    const size_t table_bytes = (size_t)ix.K * p.nq;
+    const size_t table_bytes = (size_t)ix.K * coarse_pitch(p.nq);
     const bool use_rng = rng != nullptr;
     if (table_bytes <= 160 * 1024 && lo != nullptr) {
         // the whole 8-bit table of a query fits in shared memory: stage it once per block and look rows up there
@@ -657,7 +678,10 @@ int launch_coarse_bounds(const Index &ix, const Params &p, const uint8_t *table8
     const unsigned gx = (unsigned)per_query;
     dim3 grid(gx, (unsigned)p.B);
     if (use_rng) {
-        if (p.nq == 32)
+        if (!coarse_supported(p.nq)) {
+            auto kern = p.nq <= 32 ? ci_coarse_rng_kernel_pad<2> : p.nq <= 64 ? ci_coarse_rng_kernel_pad<4> : ci_coarse_rng_kernel_pad<8>;
+            launch(kern, grid, CI_THREADS, 0, st, table8, ix.K, p.nq, rng, n_cand, p.maxc, ix.cids, hi);
+        } else if (p.nq == 32)
             launch(ci_coarse_rng_kernel<2>, grid, CI_THREADS, 0, st, table8, ix.K, rng, n_cand, p.maxc, ix.cids, lo, hi);
         else
             launch(ci_coarse_rng_kernel_b4<4>, grid, CI_THREADS, 0, st, table8, ix.K, rng, n_cand, p.maxc, ix.cids, lo, hi);
@@ -720,12 +744,10 @@ int launch_centroid_interaction(const Index &ix, const Params &p, const int32_t 
         launch(ci_wide_kernel<8>, grid, CI_THREADS, 0, st, table, ix.K, cand, n_cand, p.maxc, ix.cids, ix.doc_off, ci);
     else if (p.nq == 64)
         launch(ci_wide_kernel<16>, grid, CI_THREADS, 0, st, table, ix.K, cand, n_cand, p.maxc, ix.cids, ix.doc_off, ci);
-    else if (nqw == 1)
-        launch(ci_kernel<1>, grid, CI_THREADS, 0, st, table, ix.K, p.nq, cand, n_cand, p.maxc, ix.cids, ix.doc_off, grng, ci);
-    else if (nqw == 2)
-        launch(ci_kernel<2>, grid, CI_THREADS, 0, st, table, ix.K, p.nq, cand, n_cand, p.maxc, ix.cids, ix.doc_off, grng, ci);
-    else
-        launch(ci_kernel<4>, grid, CI_THREADS, 0, st, table, ix.K, p.nq, cand, n_cand, p.maxc, ix.cids, ix.doc_off, grng, ci);
+    else {
+        auto kern = nqw == 1 ? ci_kernel<1> : nqw == 2 ? ci_kernel<2> : ci_kernel<4>;
+        launch(kern, grid, CI_THREADS, 0, st, table, ix.K, p.nq, cand, n_cand, p.maxc, ix.cids, ix.doc_off, grng, ci);
+    }
     CHIMERA_CUDA(cudaGetLastError());
     count_launch(slot);
     return CHIMERA_OK;

@@ -16,7 +16,7 @@
 //   (their exact CI: g3_centroid_interaction.cu)
 //   filter_count_kernel,   tau = the n_prune-th largest of those, a lower bound on the n_prune-th largest CI; keeps every
 //   filter_write_kernel    candidate with hi0 >= tau, ascending, with its token range
-//   (q_len 32 / 64: upper bounds of the kept ones from the 8-bit table: g3_centroid_interaction.cu)
+//   (upper bounds of the kept ones from the 8-bit table: g3_centroid_interaction.cu)
 //   filter_contend_kernel  and of those the ones whose bound reaches tau
 //   (exact CI of what is left, except for the seeds, and the exact selection: g3_centroid_interaction.cu)
 // Every document of the exact top n_prune has an upper bound >= CI >= tau, so it is never dropped and the result is the
@@ -58,8 +58,8 @@ static int filter_codec(int64_t K)
 // When the cut runs.  The table has to fit one SM's shared memory; a token position has to fit 32 bits and a document's
 // sum of e 31 bits; and there has to be enough to scan that the additional launches pay: 13 against 8 kernels for q_len
 // 32 / 64, whose other form scans 8-bit rows (one query of 60 M tokens, 14 M of them candidates': 248 us with the cut, 225
-// without; one of 16 queries with 48 M candidate tokens each: 5.4 against 6.7 ms), 9 against 6 for the others, which
-// look up exact rows (8 queries of 20 M tokens: 3.3 against 5.8 ms).
+// without; one of 16 queries with 48 M candidate tokens each: 5.4 against 6.7 ms), 11 against 6 for the others, which
+// look up exact rows (8 queries of 20 M tokens: 1.1 against 5.8 ms).
 bool filter_used(const Index &ix, const Params &p)
 {
     if (filter_codec(ix.K) == 0 || ix.T >= 0x7fffff00LL || ix.max_doclen > 32000) return false;
@@ -248,37 +248,51 @@ filter_excess_kernel(const uint8_t *__restrict__ table8, int64_t K, const int32_
     }
 }
 
-// The same from the exact table, for any q_len: one warp per row, values rounded up to units of 2^us.
-template <int CODEC>
+// The same from the exact table, for any q_len: one warp per row, values rounded up to units of 2^us.  The 8-bit rows that
+// the second bound looks up are made on the way (table8: [B][K][pitch8], a lane's columns side by side, zeros for those
+// past nq: the bound is a sum over columns, whatever their order).
+template <int CODEC, int NQW>      // NQW = pitch8 / 32
 __global__ void __launch_bounds__(256)
 filter_excess_exact_kernel(const int32_t *__restrict__ table, int64_t K, int nq, const int32_t *__restrict__ theta, int us,
-                           uint8_t *__restrict__ out, size_t pitch)
+                           uint8_t *__restrict__ table8, uint8_t *__restrict__ out, size_t pitch)
 {
     pdl_entry();
     __shared__ uint8_t enc[512];
     if (CODEC == 6) filter_fill_encoder(enc);
     const int b = blockIdx.y, lane = threadIdx.x & 31;
-    int th[4];
+    constexpr int pitch8 = 32 * NQW;
+    uint8_t *t8 = table8 + (int64_t)b * K * pitch8;
+    int th[NQW];
 #pragma unroll
-    for (int w = 0; w < 4; ++w) th[w] = lane + 32 * w < nq ? theta[(int64_t)b * nq + lane + 32 * w] << 16 : 0;
+    for (int w = 0; w < NQW; ++w) th[w] = lane + 32 * w < nq ? theta[(int64_t)b * nq + lane + 32 * w] << 16 : 0;
     const int32_t *tb = table + (int64_t)b * K * nq;
     uint8_t *ob = out + (size_t)b * pitch;
     constexpr int PER = CODEC == 16 ? 8 : 5;                          // rows per warp and iteration
     const int64_t groups = (K + PER - 1) / PER;
     for (int64_t g = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); g < groups; g += (int64_t)gridDim.x * 8) {
         int e[PER];
+        uint32_t coarse[PER];
 #pragma unroll
-        for (int r = 0; r < PER; ++r) e[r] = 0;
+        for (int r = 0; r < PER; ++r) { e[r] = 0; coarse[r] = 0u; }
 #pragma unroll
-        for (int w = 0; w < 4; ++w) {
-            if (32 * w < nq) {
-                int v[PER];
+        for (int w = 0; w < NQW; ++w) {
+            int v[PER];
 #pragma unroll
-                for (int r = 0; r < PER; ++r)
-                    v[r] = (lane + 32 * w < nq && g * PER + r < K) ? __ldg(tb + (g * PER + r) * nq + lane + 32 * w) : 0;
+            for (int r = 0; r < PER; ++r)
+                v[r] = (lane + 32 * w < nq && g * PER + r < K) ? __ldg(tb + (g * PER + r) * nq + lane + 32 * w) : 0;
 #pragma unroll
-                for (int r = 0; r < PER; ++r) e[r] += max(v[r] - th[w], 0);
+            for (int r = 0; r < PER; ++r) {
+                coarse[r] |= (uint32_t)__vimin_s32_relu(v[r] >> 16, 255) << (8 * w);
+                e[r] += max(v[r] - th[w], 0);     // (a column past the end has neither a value nor a threshold)
             }
+        }
+#pragma unroll
+        for (int r = 0; r < PER; ++r) {
+            if (g * PER + r >= K) break;
+            uint8_t *row = t8 + (g * PER + r) * pitch8;
+            if constexpr (NQW == 1) row[lane] = (uint8_t)coarse[r];
+            else if constexpr (NQW == 2) reinterpret_cast<uint16_t *>(row)[lane] = (uint16_t)coarse[r];
+            else reinterpret_cast<uint32_t *>(row)[lane] = coarse[r];
         }
         uint32_t packed = 0;
         int val = 0;
@@ -469,13 +483,15 @@ filter_scan_kernel(const uint8_t *__restrict__ tab, size_t pitch, const int32_t 
 // A Q.24 threshold in units of 2^us, rounded up (hi0 is a whole number of them).
 __device__ __forceinline__ int32_t units_up(int32_t tau, int us) { return (int32_t)(((long long)tau + (1 << us) - 1) >> us); }
 
-// grid (split, B): candidates with the largest hi0, 2 n_prune of them and the rest of the
+// grid (split, B): candidates with the largest hi0, 2 n_prune of them (wide: q_len 32 or 64, whose exact rows are read in
+// 16-byte pieces) or 1.5 n_prune (other lengths, where an exact row costs three to four times its 8-bit copy: 37 queries of
+// 21 tokens 1,255 against 1,309 us; on the wide ones 1.5 costs more in the later cuts than it saves) and the rest of the
 // last histogram bin, with their token ranges, in no particular order; seed_thr[b] = the hi0 they
 // start at, seed_slot[candidate] = where each one went.  n_seed (cleared before) stays 0 when a query has so few
 // candidates that all are kept.
 __global__ void __launch_bounds__(SEL_THREADS)
 filter_seed_kernel(const int32_t *__restrict__ cand, const int32_t *__restrict__ n_cand, const int64_t *__restrict__ doc_off,
-                   const int32_t *__restrict__ hi0, int64_t maxc, const int32_t *__restrict__ theta, int nq, int us,
+                   const int32_t *__restrict__ hi0, int64_t maxc, const int32_t *__restrict__ theta, int nq, bool wide, int us,
                    const int32_t *__restrict__ hist, int n_prune, int32_t *__restrict__ seed,
                    int2 *__restrict__ seed_rng, int32_t *__restrict__ n_seed, int32_t *__restrict__ seed_thr,
                    int32_t *__restrict__ seed_slot)
@@ -484,7 +500,7 @@ filter_seed_kernel(const int32_t *__restrict__ cand, const int32_t *__restrict__
     __shared__ int warp_part[32];
     __shared__ int s_bin, s_theta;
     const int b = blockIdx.y, n = n_cand[b];
-    const int want = 2 * n_prune + 32;
+    const int want = (wide ? 2 * n_prune : n_prune + n_prune / 2) + 32;
     if (n <= want) {
         if (blockIdx.x == 0 && threadIdx.x == 0) seed_thr[b] = INT_MAX;
         return;
@@ -712,7 +728,7 @@ static int filter_unit(const Index &ix, const Params &p, bool from_table8)
     return from_table8 || filter_codec(ix.K) != 16 ? 16 : p.nq <= 63 ? 14 : 15;
 }
 
-int launch_filter_scan(const Index &ix, const Params &p, const Layout &L, const int32_t *table, const uint8_t *table8,
+int launch_filter_scan(const Index &ix, const Params &p, const Layout &L, const int32_t *table, uint8_t *table8,
                        const int32_t *cand, const int32_t *n_cand, int32_t *hi0, int32_t *seed,
                        int2 *seed_rng, char *ws, cudaStream_t st)
 {
@@ -737,9 +753,10 @@ int launch_filter_scan(const Index &ix, const Params &p, const Layout &L, const 
     launch(filter_theta_kernel, dim3(groups, (unsigned)p.B, (unsigned)parts), SEL_THREADS, 0, st, table, ix.K, p.nq, m, step, rank, theta, hist, n_seed, parts_hist, done);
     CHIMERA_CUDA(cudaGetLastError());
 
-    const int us = filter_unit(ix, p, table8 != nullptr);
+    const bool ready = coarse_supported(p.nq);           // stage 1 has written the 8-bit table
+    const int us = filter_unit(ix, p, ready);
     int64_t gx = (8LL * ix.sm_count + p.B - 1) / p.B;
-    if (table8 != nullptr) {
+    if (ready) {
         const int64_t want = ((codec == 16 ? ix.K : (ix.K + 4) / 5) + 255) / 256;
         if (gx > want) gx = want;
         const dim3 grid((unsigned)gx, (unsigned)p.B);
@@ -751,10 +768,13 @@ int launch_filter_scan(const Index &ix, const Params &p, const Layout &L, const 
         const int64_t want = (ix.K + 39) / 40;
         if (gx > want) gx = want;
         const dim3 grid((unsigned)gx, (unsigned)p.B);
-        if (codec == 16)
-            launch(filter_excess_exact_kernel<16>, grid, 256, 0, st, table, ix.K, p.nq, theta, us, tab, pitch);
-        else
-            launch(filter_excess_exact_kernel<6>, grid, 256, 0, st, table, ix.K, p.nq, theta, us, tab, pitch);
+        auto kern = codec == 16 ? (p.nq <= 32   ? filter_excess_exact_kernel<16, 1>
+                                   : p.nq <= 64 ? filter_excess_exact_kernel<16, 2>
+                                                : filter_excess_exact_kernel<16, 4>)
+                                : (p.nq <= 32   ? filter_excess_exact_kernel<6, 1>
+                                   : p.nq <= 64 ? filter_excess_exact_kernel<6, 2>
+                                                : filter_excess_exact_kernel<6, 4>);
+        launch(kern, grid, 256, 0, st, table, ix.K, p.nq, theta, us, table8, tab, pitch);
     }
     CHIMERA_CUDA(cudaGetLastError());
 
@@ -775,7 +795,7 @@ int launch_filter_scan(const Index &ix, const Params &p, const Layout &L, const 
                                                                    ix.cids, ix.T, hi0, hist);
     }
     CHIMERA_CUDA(cudaGetLastError());
-    launch(filter_seed_kernel, dim3((unsigned)filter_split(ix, p), (unsigned)p.B), SEL_THREADS, 0, st, cand, n_cand, ix.doc_off, hi0, p.maxc, theta, p.nq, us, hist, p.n_prune, seed, seed_rng, n_seed,
+    launch(filter_seed_kernel, dim3((unsigned)filter_split(ix, p), (unsigned)p.B), SEL_THREADS, 0, st, cand, n_cand, ix.doc_off, hi0, p.maxc, theta, p.nq, ready, us, hist, p.n_prune, seed, seed_rng, n_seed,
         (int32_t *)(ws + L.flt_thr), (int32_t *)(ws + L.flt_slot));
     CHIMERA_CUDA(cudaGetLastError());
     count_launch(SLOT_CI, 4);

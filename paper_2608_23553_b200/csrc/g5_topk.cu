@@ -52,7 +52,7 @@ __device__ __forceinline__ void bitonic_sort(unsigned long long *keys, int n_pow
 }
 
 // SELECT (at least four times as many entries as wanted): the k-th largest score by radix select, then only the entries
-// that reach it are sorted (16,384 entries, k = 1,000: 185 us for sorting all, XX with the selection).  More ties at that
+// that reach it are sorted (16,384 entries, k = 1,000: 185 us for sorting all, 41 with the selection).  More ties at that
 // score than the second array holds: everything is sorted after all.
 template <bool SELECT>
 __global__ void __launch_bounds__(TOPK_THREADS)

@@ -19,6 +19,8 @@ pytestmark = pytest.mark.gpu
     (96, 1, 21, 700, 20_000, 1, 99, 21, 2, 200, 0, 1),            # exact table, q_len < 32
     (32, 2, 100, 3_000, 12_345, 10, 70, 45, 1, 500, 1, 1),        # ... four column groups
     (32, 2, 40, 107_001, 8_000, 90, 120, 25, 16, 64, 0, 1),       # ... 6-bit codes
+    (64, 2, 47, 2_000, 9_000, 20, 90, 60, 1, 300, 0, 1),          # ... rows of an odd number of values, two per lane
+    (32, 2, 127, 1_000, 6_000, 20, 70, 80, 1, 200, 0, 1),         # ... four per lane, the longest query
     (64, 2, 32, 6_000, 24_000, 1, 70, 256, 1, 5_900, 0, 1),        # queries with fewer candidates than 1.5 n_prune
     (32, 2, 32, 300, 20_000, 1, 80, 260, 1, 333, 0, 50),          # every document 50 times: masses of equal scores
 ])
