@@ -18,7 +18,7 @@ def _index(cent, cids, codes, doclens):
 
 
 @pytest.mark.parametrize("n,k,distinct", [
-    (4097, 129, 0), (16384, 1000, 0), (16384, 4096, 0), (9001, 129, 0), (8192, 2048, 0),
+    (256, 64, 0), (255, 63, 0), (300, 17, 3), (4096, 100, 0), (4097, 129, 0), (16384, 1000, 0), (16384, 4096, 0), (9001, 129, 0), (8192, 2048, 0),
     (16384, 1000, 12),                     # about 1,365 entries per value: the ties fit the second array
     (5000, 513, 5),                        # they do not
 ])
