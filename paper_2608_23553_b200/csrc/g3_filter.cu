@@ -74,10 +74,12 @@ size_t filter_table_pitch(const Index &ix)
 }
 int filter_hist_bins() { return FILTER_BINS; }
 int filter_count_slots() { return KEEP_SPLIT; }
-// Blocks per query of the selection kernels: about four per SM, slices of 4,096 candidates or more.
+// Blocks per query of the selection kernels: slices of 4,096 candidates or more, and no more blocks than are resident at once
+// (two of 1,024 threads per SM): every block of a query first finds tau, or the seeds' histogram bin, for itself, so a second
+// wave costs as much as the first (256 queries in 3 x 256 blocks: 214 us for the keep steps, in 256: 183).
 static int filter_split(const Index &ix, const Params &p)
 {
-    int64_t g = (4LL * ix.sm_count + p.B - 1) / p.B;
+    int64_t g = 2LL * ix.sm_count / p.B;
     if (g > (p.maxc + 4095) / 4096) g = (p.maxc + 4095) / 4096;
     return (int)(g > KEEP_SPLIT ? KEEP_SPLIT : g < 1 ? 1 : g);
 }
