@@ -1106,13 +1106,21 @@ contender_write_kernel(const int32_t *__restrict__ cand, const int32_t *__restri
         int keep = 0;
 #pragma unroll
         for (int e = 0; e < 4; ++e) keep += (q0 + e < j1 && hv[e] >= tau) ? 1 : 0;
+        int32_t id[4];                                       // (asked for in front of the scan's barriers)
+        int2 r[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            if (q0 + e < j1 && hv[e] >= tau) {
+                id[e] = cb[q0 + e];
+                r[e] = orng ? rb[q0 + e] : make_int2(0, 0);
+            }
         int tot;
         int pos = run + sel_block_scan(keep, &tot, warp_part);
 #pragma unroll
         for (int e = 0; e < 4; ++e)
             if (q0 + e < j1 && hv[e] >= tau) {
-                out[pos] = cb[q0 + e];
-                if (orng) orng[pos] = rb[q0 + e];
+                out[pos] = id[e];
+                if (orng) orng[pos] = r[e];
                 ++pos;
             }
         run += tot;
