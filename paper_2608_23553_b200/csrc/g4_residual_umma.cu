@@ -48,8 +48,10 @@ __device__ __forceinline__ float f_unorder(uint32_t o)
 // contraction T = sum_x Xq[x] b[x] against the digit planes of the ROTATED query, then
 // est = inv_dot_t * (c * (float)(2 T - SQ_i)) with SQ_i = sum_x Xq_i[x] and c = 1 / (sqrt(D) 2^22); no centroid term;
 // query tokens are summed in increasing order in fp32 so that the score is reproducible bit for bit.
-// FULL: q_len is NQP and dim is 128, the common sizes: no row or code is partial and every address is aligned.
-template <int NQP, int NBITS, bool RQ, bool FULL>
+// DIM > 0: q_len is NQP and dim is DIM, so that no row is partial and the code's extent is known when this is compiled (0: any
+// sizes; 64 queries of 64 tokens, long documents: dim 96 took 4.36 ms without a variant of its own, 3.96 with it; 64 queries
+// of 32 tokens, Mid with dim 96: 0.60, now 0.41).
+template <int NQP, int NBITS, bool RQ, int DIM>
 __global__ void __launch_bounds__(128 * (NQP / G4U_COLS), NQP == 32 ? (RQ ? 4 : 3) : 2)
 residual_maxsim_umma(const __grid_constant__ CUtensorMap map_q, const float *__restrict__ queries,
                      const int32_t *__restrict__ table, int64_t K, int nq_arg, int q_base, int nq_all_arg, int q_rows, int D_arg,
@@ -61,8 +63,9 @@ residual_maxsim_umma(const __grid_constant__ CUtensorMap map_q, const float *__r
 {
     pdl_entry();
     // this launch's query tokens are q_base ... q_base + nq - 1 of the query's nq_all (its digit planes have q_rows rows)
+    constexpr bool FULL = DIM > 0;
     const int nq = FULL ? NQP : nq_arg, nq_all = FULL ? NQP : nq_all_arg;
-    const int D = FULL ? 128 : D_arg, CW = FULL ? (NBITS == 2 ? 8 : 4) : CW_arg;
+    const int D = FULL ? DIM : D_arg, CW = FULL ? DIM * NBITS / 32 : CW_arg;
     constexpr int N = 3 * NQP;                               // MMA N: three digit planes side by side
     constexpr uint32_t TMEM_COLS = N <= 96 ? 128 : 256;
     constexpr uint32_t A_COL = N;                            // the expanded codes: 32 columns behind the accumulators
@@ -168,7 +171,7 @@ residual_maxsim_umma(const __grid_constant__ CUtensorMap map_q, const float *__r
     const char *tb = reinterpret_cast<const char *>(table + (int64_t)b * K * nq_all + q_base);
     const uint32_t row_bytes = 4u * (uint32_t)nq_all;
     const bool vec_rows = (nq_all & 3) == 0;       // 16-byte groups of a row are aligned (q_base is a multiple of 64)
-    const int k_steps = FULL ? 4 : D >> 5;
+    const int k_steps = D >> 5;
     const float code_scale = delta * 4.0f;                    // delta * 2^-22, times 2^24
     bool alive = true;
     // Code words of a token that one thread expands: a token has at most 32 code bytes (2 bits per dimension) or 16 (1 bit).
@@ -198,20 +201,21 @@ residual_maxsim_umma(const __grid_constant__ CUtensorMap map_q, const float *__r
 #endif
         cid = __ldg(at_cid + s);
         const uint32_t *src = at_code + (long long)s * CW;
-        if (FULL ? TW == 4 : TW == 4 && (CW & 3) == 0) {
+        if (w0 >= CW) {                                       // (this warp's part lies behind a short code)
+        } else if (TW == 4 && (CW & 3) == 0) {
             const uint4 v = __ldg(reinterpret_cast<const uint4 *>(src));
             cw[0] = v.x; cw[1] = v.y; cw[TW > 2 ? 2 : 0] = v.z; cw[TW > 3 ? 3 : 0] = v.w;
-        } else if (FULL ? TW >= 2 : TW >= 2 && (CW & 1) == 0) {
+        } else if (TW >= 2 && (CW & 1) == 0) {
 #pragma unroll
             for (int w = 0; w < TW; w += 2)
-                if (FULL || w0 + w < CW) {
+                if (w0 + w < CW) {
                     const uint2 v = __ldg(reinterpret_cast<const uint2 *>(src + w));
                     cw[w] = v.x; cw[w + 1 < TW ? w + 1 : w] = v.y;
                 }
         } else {
 #pragma unroll
             for (int w = 0; w < TW; ++w)
-                if (FULL || w0 + w < CW) cw[w] = __ldg(src + w);
+                if (w0 + w < CW) cw[w] = __ldg(src + w);
         }
     };
 
@@ -423,8 +427,12 @@ static int launch_g4_umma(const Index &ix, const Params &p, int q_base, int nq, 
     // four or fewer and the 256-column ones at two; the latter ask for a third of an SM's shared memory plus one byte
     // besides, so that a build with fewer registers does not change that.
     if (N > 96 && smem < 227 * 1024 / 3 + 1) smem = 227 * 1024 / 3 + 1;
-    auto kern = p.nq == NQP && nq == NQP && ix.D == 128 ? residual_maxsim_umma<NQP, NBITS, RQ, true>
-                                           : residual_maxsim_umma<NQP, NBITS, RQ, false>;
+    auto kern = residual_maxsim_umma<NQP, NBITS, RQ, 0>;
+    if (p.nq == NQP && nq == NQP)                            // dim is a multiple of 32 up to 128
+        kern = ix.D == 128  ? residual_maxsim_umma<NQP, NBITS, RQ, 128>
+               : ix.D == 96 ? residual_maxsim_umma<NQP, NBITS, RQ, 96>
+               : ix.D == 64 ? residual_maxsim_umma<NQP, NBITS, RQ, 64>
+                            : residual_maxsim_umma<NQP, NBITS, RQ, 32>;
     CHIMERA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     // documents per CTA: whole waves of resident CTAs, as few as documents-per-CTA limit allows (a second wave of a few CTAs
     // costs as much as a full one: 37 queries of 777 survivors in 2.1 waves of 32 documents, or in three of 22)

@@ -1,5 +1,6 @@
 """Branches that only sizes or ties reach: the top-k that sorts the best entries only, the graph search whose visited set
-does not fit shared memory, and the RaBitQ search whose score table is made only for the queries that turn out to need it."""
+does not fit shared memory, the RaBitQ search whose score table is made only for the queries that turn out to need it, and
+stage 4 for every dimension."""
 import numpy as np
 import pytest
 import torch
@@ -10,15 +11,16 @@ from helpers import random_corpus, unit_rows
 pytestmark = pytest.mark.gpu
 
 
-def _index(cent, cids, codes, doclens):
+def _index(cent, cids, codes, doclens, nbits=2):
     import paper_2608_23553_b200 as pkg
     dev = torch.device("cuda:0")
     return pkg.Index(torch.from_numpy(cent).to(dev), torch.from_numpy(cids).to(dev), torch.from_numpy(codes).to(dev),
-                     torch.from_numpy(doclens).to(dev), 2)
+                     torch.from_numpy(doclens).to(dev), nbits)
 
 
 @pytest.mark.parametrize("n,k,distinct", [
-    (256, 64, 0), (255, 63, 0), (300, 17, 3), (4096, 100, 0), (4097, 129, 0), (16384, 1000, 0), (16384, 4096, 0), (9001, 129, 0), (8192, 2048, 0),
+    (256, 64, 0), (255, 63, 0), (300, 17, 3), (4096, 100, 0), (4097, 129, 0), (16384, 1000, 0),
+    (16384, 4096, 0), (9001, 129, 0), (8192, 2048, 0),
     (16384, 1000, 12),                     # about 1,365 entries per value: the ties fit the second array
     (5000, 513, 5),                        # they do not
 ])
@@ -84,3 +86,20 @@ def test_rabitq_makes_the_table_for_queries_whose_queue_overflows():
         assert np.array_equal(taps.probes[b].cpu().numpy(), oracle.probes(oracle.score_table(q[b], cent), nprobe))
         res = oracle.pipeline_rabitq(q[b], oix, rq, nprobe, 60, 10)
         assert np.array_equal(ids[b].cpu().numpy(), res.ids) and np.array_equal(sc[b].cpu().numpy(), res.scores)
+
+
+@pytest.mark.parametrize("nq", [32, 64])
+@pytest.mark.parametrize("D,nbits", [(32, 1), (32, 2), (64, 1), (64, 2), (96, 1), (96, 2), (128, 1)])
+def test_stage_4_of_every_dimension(D, nbits, nq):
+    """Every document survives, the corpus's last one included, whose code ends with the array."""
+    from parity import check_query, taps_to_numpy
+    N, nprobe = 97, 16
+    cent, cids, codes, doclens = random_corpus(D + nbits, N, 16, D, nbits, len_lo=1, len_hi=150)
+    gix = _index(cent, cids, codes, doclens, nbits)
+    q = np.stack([unit_rows(np.random.default_rng(7 + b), nq, D) for b in range(2)])
+    taps = gix.alloc_taps(2, nq, nprobe, N, table=False)
+    ids, sc = gix.search(torch.from_numpy(q).cuda(), nprobe, N, 20, taps=taps)
+    assert gix.status() == 0
+    oix, tn = oracle.make_index(cent, cids, codes, doclens, nbits), taps_to_numpy(taps)
+    for b in range(2):
+        check_query(tn, b, oracle.pipeline(q[b], oix, nprobe, N, 20), ids[b].cpu().numpy(), sc[b].cpu().numpy(), 20, N, table=False)
