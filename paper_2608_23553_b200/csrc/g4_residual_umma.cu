@@ -48,14 +48,13 @@ __device__ __forceinline__ float f_unorder(uint32_t o)
 // contraction T = sum_x Xq[x] b[x] against the digit planes of the ROTATED query, then
 // est = inv_dot_t * (c * (float)(2 T - SQ_i)) with SQ_i = sum_x Xq_i[x] and c = 1 / (sqrt(D) 2^22); no centroid term;
 // query tokens are summed in increasing order in fp32 so that the score is reproducible bit for bit.
-// DIM > 0: q_len is NQP and dim is DIM, so that no row is partial and the code's extent is known when this is compiled (0: any
-// sizes; 64 queries of 64 tokens, long documents: dim 96 took 4.36 ms without a variant of its own, 3.96 with it; 64 queries
-// of 32 tokens, Mid with dim 96: 0.60, now 0.41).
-template <int NQP, int NBITS, bool RQ, int DIM>
+// DIM: the dimension, so that a code's extent is known when this is compiled (64 queries of 64 tokens, long documents: dim 96
+// took 4.36 ms without, 3.96 with it; 64 queries of 32 tokens, Mid with dim 96: 0.60, now 0.41).  FULL: q_len is NQP, no row is
+// partial.
+template <int NQP, int NBITS, bool RQ, int DIM, bool FULL>
 __global__ void __launch_bounds__(128 * (NQP / G4U_COLS), NQP == 32 ? (RQ ? 4 : 3) : 2)
 residual_maxsim_umma(const __grid_constant__ CUtensorMap map_q, const float *__restrict__ queries,
-                     const int32_t *__restrict__ table, int64_t K, int nq_arg, int q_base, int nq_all_arg, int q_rows, int D_arg,
-                     int CW_arg, float delta, float kappa,
+                     const int32_t *__restrict__ table, int64_t K, int nq_arg, int q_base, int nq_all_arg, int q_rows, float delta, float kappa,
                      const int32_t *__restrict__ pruned, int n_prune, int docs_per_cta,
                      const int32_t *__restrict__ cids, const uint32_t *__restrict__ codes,
                      const float *__restrict__ factors, const int64_t *__restrict__ doc_off,
@@ -63,9 +62,8 @@ residual_maxsim_umma(const __grid_constant__ CUtensorMap map_q, const float *__r
 {
     pdl_entry();
     // this launch's query tokens are q_base ... q_base + nq - 1 of the query's nq_all (its digit planes have q_rows rows)
-    constexpr bool FULL = DIM > 0;
     const int nq = FULL ? NQP : nq_arg, nq_all = FULL ? NQP : nq_all_arg;
-    const int D = FULL ? DIM : D_arg, CW = FULL ? DIM * NBITS / 32 : CW_arg;
+    constexpr int D = DIM, CW = DIM * NBITS / 32;
     constexpr int N = 3 * NQP;                               // MMA N: three digit planes side by side
     constexpr uint32_t TMEM_COLS = N <= 96 ? 128 : 256;
     constexpr uint32_t A_COL = N;                            // the expanded codes: 32 columns behind the accumulators
@@ -427,12 +425,13 @@ static int launch_g4_umma(const Index &ix, const Params &p, int q_base, int nq, 
     // four or fewer and the 256-column ones at two; the latter ask for a third of an SM's shared memory plus one byte
     // besides, so that a build with fewer registers does not change that.
     if (N > 96 && smem < 227 * 1024 / 3 + 1) smem = 227 * 1024 / 3 + 1;
-    auto kern = residual_maxsim_umma<NQP, NBITS, RQ, 0>;
-    if (p.nq == NQP && nq == NQP)                            // dim is a multiple of 32 up to 128
-        kern = ix.D == 128  ? residual_maxsim_umma<NQP, NBITS, RQ, 128>
-               : ix.D == 96 ? residual_maxsim_umma<NQP, NBITS, RQ, 96>
-               : ix.D == 64 ? residual_maxsim_umma<NQP, NBITS, RQ, 64>
-                            : residual_maxsim_umma<NQP, NBITS, RQ, 32>;
+    const bool full = p.nq == NQP && nq == NQP;
+    auto kern = full ? residual_maxsim_umma<NQP, NBITS, RQ, 128, true> : residual_maxsim_umma<NQP, NBITS, RQ, 128, false>;
+    switch (ix.D) {                                          // (a multiple of 32 up to 128)
+    case 32: kern = full ? residual_maxsim_umma<NQP, NBITS, RQ, 32, true> : residual_maxsim_umma<NQP, NBITS, RQ, 32, false>; break;
+    case 64: kern = full ? residual_maxsim_umma<NQP, NBITS, RQ, 64, true> : residual_maxsim_umma<NQP, NBITS, RQ, 64, false>; break;
+    case 96: kern = full ? residual_maxsim_umma<NQP, NBITS, RQ, 96, true> : residual_maxsim_umma<NQP, NBITS, RQ, 96, false>; break;
+    }
     CHIMERA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     // documents per CTA: whole waves of resident CTAs, as few as documents-per-CTA limit allows (a second wave of a few CTAs
     // costs as much as a full one: 37 queries of 777 survivors in 2.1 waves of 32 documents, or in three of 22)
@@ -446,9 +445,8 @@ static int launch_g4_umma(const Index &ix, const Params &p, int q_base, int nq, 
     dim3 grid((unsigned)((p.n_prune + dpc - 1) / dpc), (unsigned)p.B);
     const uint32_t *code_words = reinterpret_cast<const uint32_t *>(RQ ? ix.rq_bits : ix.codes);
     launch(kern, grid, 128 * (NQP / G4U_COLS), smem, st, map_q, queries, table, ix.K, nq, q_base, p.nq,
-           residual_rows(p.nq), ix.D, RQ ? ix.D / 32 : ix.CB / 4, delta,
-                                          kappa, pruned, p.n_prune, (int)dpc, ix.cids, code_words, ix.rq_inv, ix.doc_off,
-                                          score4, status, wait_limit_cycles(), fault_skip_tma_loads());
+           residual_rows(p.nq), delta, kappa, pruned, p.n_prune, (int)dpc, ix.cids, code_words, ix.rq_inv, ix.doc_off, score4,
+           status, wait_limit_cycles(), fault_skip_tma_loads());
     CHIMERA_CUDA(cudaGetLastError());
     count_launch(SLOT_G4);
     return CHIMERA_OK;
