@@ -169,7 +169,7 @@ int chimera_run_stages(const chimera_index *index, int32_t first_stage, int32_t 
  * index (cudaMalloc) and, where that takes no more than a quarter of the free device memory, a copy of the codes in the
  * order of the lists; synchronises the stream.  Idempotent.  Workspace sizes grow afterwards (visit lists, or a score
  * table of n_queries x max_candidates x q_len int32), so query chimera_workspace_bytes again.
- * Errors: INVALID_ARG, UNSUPPORTED (more than 2^31 - 1 tokens), CUDA_ERROR (nothing stays allocated). */
+ * Errors: INVALID_ARG, UNSUPPORTED (more than 2^31 - 1 tokens), CUDA_ERROR (the index can be used as before the call). */
 int chimera_index_enable_partial(chimera_index *index, void *stream);
 
 /* The search with the paper's own candidate refinement in place of stage 3 (Sec. 3.2 step 2, Algorithm 2; aggregation
@@ -194,8 +194,9 @@ int chimera_search_partial(const chimera_index *index, const float *queries, int
  *   bits      device, [T, dim/8] uint8, document-major: bit t of byte g is dimension 8g+t.  REFERENCED, not copied.
  *   inv_dot   device, [T] float32, 1 / <o_p, o_p-bar> = sqrt(dim) / sum_x |o_p[x]|.  REFERENCED, not copied.
  * Also builds the token-level posting lists (as chimera_index_enable_partial) and, where that takes no more than a quarter
- * of the free device memory, copies of bits and inv_dot in their order.  Synchronises the stream.
- * Errors: INVALID_ARG, CUDA_ERROR. */
+ * of the free device memory, copies of bits and inv_dot in their order.  Synchronises the stream.  A second call replaces
+ * the codes.
+ * Errors: INVALID_ARG, CUDA_ERROR (the index keeps the codes and the rotation that it had, if any). */
 int chimera_index_attach_rabitq(chimera_index *index, const float *rotation, const uint8_t *bits,
                                 const float *inv_dot, void *stream);
 

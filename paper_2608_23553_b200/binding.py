@@ -188,11 +188,11 @@ class Index:
 
     def attach_rabitq(self, rotation: torch.Tensor, bits: torch.Tensor, inv_dot: torch.Tensor):
         """Attach RaBitQ 1-bit codes (kept referenced) for search(..., rabitq=True)."""
-        self._rq = (rotation.contiguous().to(torch.float32), bits.contiguous().to(torch.uint8),
-                    inv_dot.contiguous().to(torch.float32))
+        rq = (rotation.contiguous().to(torch.float32), bits.contiguous().to(torch.uint8),
+              inv_dot.contiguous().to(torch.float32))
         with torch.cuda.device(self.device):
-            _check(lib().chimera_index_attach_rabitq(self._h, _ptr(self._rq[0]), _ptr(self._rq[1]), _ptr(self._rq[2]),
-                                                     _stream()))
+            _check(lib().chimera_index_attach_rabitq(self._h, _ptr(rq[0]), _ptr(rq[1]), _ptr(rq[2]), _stream()))
+        self._rq = rq                        # (a failed call leaves the library with the arrays it had)
         self._ws = None
 
     def build_graph(self, degree: int):

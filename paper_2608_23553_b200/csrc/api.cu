@@ -541,8 +541,10 @@ int chimera_index_enable_partial(chimera_index *index, void *stream)
     Index *ix = reinterpret_cast<Index *>(index);
     if (!ix) return fail(CHIMERA_INVALID_ARG, "index is NULL");
     int rc = build_token_lists(*ix, (cudaStream_t)stream);
-    if (rc || (rc = copy_in_list_order(*ix, ix->codes, ix->CB / 4, (void **)&ix->list_codes, (cudaStream_t)stream))) return rc;
-    CHIMERA_CUDA(cudaStreamSynchronize((cudaStream_t)stream));
+    if (rc || ix->list_codes) return rc;
+    ListOrderCopy codes = {ix->codes, ix->CB / 4, nullptr};
+    if ((rc = copy_in_list_order(*ix, &codes, 1, (cudaStream_t)stream))) return rc;
+    ix->list_codes = (uint8_t *)codes.dst;
     return CHIMERA_OK;
 }
 
@@ -567,25 +569,24 @@ int chimera_index_attach_rabitq(chimera_index *index, const float *rotation, con
     if (((uintptr_t)bits & 15) || ((uintptr_t)inv_dot & 3)) return fail(CHIMERA_INVALID_ARG, "bits must be 16-byte aligned");
     int rc = build_token_lists(*ix, (cudaStream_t)stream);
     if (rc) return rc;
-    rc = attach_rabitq(*ix, rotation, (cudaStream_t)stream);
-    if (rc) return rc;
-    ix->rq_bits = bits;
-    ix->rq_inv = inv_dot;
-    // (codes attached before, if any, are replaced)
+    // Codes attached before, if any, are replaced: their copies go first, to make room.  Whatever fails below leaves the index
+    // with the codes and the rotation that it had (and no copies of them).
     cudaFree(ix->list_bits);
-    cudaFree(ix->list_inv);
     ix->list_bits = nullptr;
     ix->list_inv = nullptr;
-    if ((rc = copy_in_list_order(*ix, bits, ix->D / 32, (void **)&ix->list_bits, (cudaStream_t)stream))) return rc;
-    if ((rc = copy_in_list_order(*ix, inv_dot, 1, (void **)&ix->list_inv, (cudaStream_t)stream))) return rc;
-    if (!ix->list_bits || !ix->list_inv) {                   // both or neither
-        CHIMERA_CUDA(cudaStreamSynchronize((cudaStream_t)stream));
-        cudaFree(ix->list_bits);
-        cudaFree(ix->list_inv);
-        ix->list_bits = nullptr;
-        ix->list_inv = nullptr;
+    ListOrderCopy copies[2] = {{bits, ix->D / 32, nullptr}, {inv_dot, 1, nullptr}};
+    if ((rc = copy_in_list_order(*ix, copies, 2, (cudaStream_t)stream))) return rc;
+    float *rot_t = nullptr;
+    if ((rc = transpose_rotation(*ix, rotation, &rot_t, (cudaStream_t)stream))) {
+        cudaFree(copies[0].dst);
+        return rc;
     }
-    CHIMERA_CUDA(cudaStreamSynchronize((cudaStream_t)stream));
+    cudaFree(ix->rot_t);
+    ix->rot_t = rot_t;
+    ix->rq_bits = bits;
+    ix->rq_inv = inv_dot;
+    ix->list_bits = (uint8_t *)copies[0].dst;
+    ix->list_inv = (float *)copies[1].dst;
     return CHIMERA_OK;
 }
 
@@ -748,7 +749,6 @@ int chimera_destroy_index(chimera_index *index)
     cudaFree(ix->tok_doc);
     cudaFree(ix->list_codes);
     cudaFree(ix->list_bits);
-    cudaFree(ix->list_inv);
     cudaFree(ix->doc_off);
     cudaFree(ix->cdig);
     cudaFree(ix->ivf_off);

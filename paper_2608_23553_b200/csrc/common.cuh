@@ -32,7 +32,7 @@ struct Index {
     int64_t max_tok_list = 0;         // longest token list
     uint8_t *list_codes = nullptr;    // [T, CB]    owned, optional: the codes in list order (see copy_in_list_order)
     uint8_t *list_bits = nullptr;     // [T, D/8]   owned, optional: the RaBitQ codes in list order
-    float *list_inv = nullptr;        // [T]        owned, optional: their factors
+    float *list_inv = nullptr;        // [T]        their factors, in the same allocation: both or neither
     // RaBitQ 1-bit codes (only after chimera_index_attach_rabitq)
     const uint8_t *rq_bits = nullptr; // [T, D/8]   borrowed: sign bits of the rotated tokens
     const float *rq_inv = nullptr;    // [T]        borrowed: 1 / <o_p, o_p-bar>
@@ -228,10 +228,16 @@ bool contenders_split(const Index &ix, const Params &p);
 int contender_hist_entries();
 // Token-level posting lists for the partial-score refinement (allocates; index_build.cu).
 int build_token_lists(Index &ix, cudaStream_t st);
-// A copy of src ([T][words] 32-bit words, document-major) in the order of the token lists, so that a list's codes are one
-// contiguous run instead of a scattered sector each; *out stays NULL when it would take more than a quarter of the free
-// memory (the kernels then gather through the token ids).
-int copy_in_list_order(const Index &ix, const void *src, int words, void **out, cudaStream_t st);
+// Copies of `n` arrays ([T][words] 32-bit words each, document-major) in the order of the token lists, so that a list's
+// codes are one contiguous run instead of a scattered sector each.  One allocation (the first copy's address) holds all of
+// them; they are complete when the call returns.  Every dst stays NULL, with CHIMERA_OK, when they would take more than a
+// quarter of the free memory (the kernels then gather through the token ids), and on every error.
+struct ListOrderCopy {
+    const void *src;
+    int words;
+    void *dst;
+};
+int copy_in_list_order(const Index &ix, ListOrderCopy *copies, int n, cudaStream_t st);
 // Candidate refinement with partial scores (Algorithm 2): fprime[b][j] for every candidate.
 int64_t visit_list_nodes(const Index &ix, const Params &p);
 int launch_partial_scores(const Index &ix, const Params &p, const Layout &L, const int8_t *qdig,
@@ -306,7 +312,7 @@ int launch_graph_probes(const Index &ix, const float *queries, int64_t n_tokens,
                         uint32_t *visited, bool want_visited, int32_t *out_probes, int32_t *out_scores, int32_t *out_nvis,
                         cudaStream_t st);
 // rabitq.cu
-int attach_rabitq(Index &ix, const float *rotation, cudaStream_t st);
+int transpose_rotation(const Index &ix, const float *rotation, float **rot_t, cudaStream_t st);   // (allocates)
 int launch_rotate(const Index &ix, const Params &p, const float *queries, float *q_rot, cudaStream_t st);
 int launch_rabitq_partial(const Index &ix, const Params &p, const Layout &L, const int8_t *qdig_rot,
                           const int32_t *probes, const uint2 *ranks, const int32_t *n_cand, void *partial_m,

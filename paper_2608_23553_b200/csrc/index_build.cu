@@ -308,20 +308,41 @@ list_order_kernel(const uint32_t *__restrict__ src, const int32_t *__restrict__ 
     }
 }
 
-int copy_in_list_order(const Index &ix, const void *src, int words, void **out, cudaStream_t st)
+int copy_in_list_order(const Index &ix, ListOrderCopy *copies, int n, cudaStream_t st)
 {
-    const size_t bytes = (size_t)ix.T * words * 4;
-    size_t avail = 0, all = 0;
+    auto bytes_of = [&](const ListOrderCopy &c) { return ((size_t)ix.T * c.words * 4 + 255) & ~(size_t)255; };
+    size_t bytes = 0, avail = 0, all = 0;
+    for (int i = 0; i < n; ++i) {
+        copies[i].dst = nullptr;
+        bytes += bytes_of(copies[i]);
+    }
     CHIMERA_CUDA(cudaMemGetInfo(&avail, &all));
-    if (*out != nullptr || bytes > avail / 4) return CHIMERA_OK;
-    if (cudaMalloc(out, bytes) != cudaSuccess) {             // (an option: without it the searches gather)
+    if (bytes > avail / 4) return CHIMERA_OK;
+    char *mem = nullptr;
+    if (cudaMalloc(&mem, bytes) != cudaSuccess) {            // (an option: without it the searches gather)
         cudaGetLastError();
-        *out = nullptr;
         return CHIMERA_OK;
     }
-    list_order_kernel<<<(unsigned)(16 * ix.sm_count), 256, 0, st>>>(reinterpret_cast<const uint32_t *>(src), ix.tok_id, ix.T,
-                                                                    words, reinterpret_cast<uint32_t *>(*out));
-    CHIMERA_CUDA(cudaGetLastError());
+    cudaError_t e = cudaSuccess;
+    size_t at = 0;
+    for (int i = 0; i < n && e == cudaSuccess; ++i) {
+        list_order_kernel<<<(unsigned)(16 * ix.sm_count), 256, 0, st>>>(
+            reinterpret_cast<const uint32_t *>(copies[i].src), ix.tok_id, ix.T, copies[i].words,
+            reinterpret_cast<uint32_t *>(mem + at));
+        e = cudaGetLastError();
+        at += bytes_of(copies[i]);
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) {
+        cudaStreamSynchronize(st);
+        cudaFree(mem);
+        return fail(CHIMERA_CUDA_ERROR, "copy in list order: %s", cudaGetErrorString(e));
+    }
+    at = 0;
+    for (int i = 0; i < n; ++i) {
+        copies[i].dst = mem + at;
+        at += bytes_of(copies[i]);
+    }
     return CHIMERA_OK;
 }
 

@@ -24,12 +24,19 @@ __global__ void transpose_kernel(const float *__restrict__ in, int D, float *__r
     }
 }
 
-int attach_rabitq(Index &ix, const float *rotation, cudaStream_t st)
+int transpose_rotation(const Index &ix, const float *rotation, float **rot_t, cudaStream_t st)
 {
-    if (!ix.rot_t) CHIMERA_CUDA(cudaMalloc(&ix.rot_t, sizeof(float) * ix.D * ix.D));
-    transpose_kernel<<<(ix.D * ix.D + 255) / 256, 256, 0, st>>>(rotation, ix.D, ix.rot_t);
-    CHIMERA_CUDA(cudaGetLastError());
-    CHIMERA_CUDA(cudaStreamSynchronize(st));
+    *rot_t = nullptr;
+    float *out = nullptr;
+    CHIMERA_CUDA(cudaMalloc(&out, sizeof(float) * ix.D * ix.D));
+    transpose_kernel<<<(ix.D * ix.D + 255) / 256, 256, 0, st>>>(rotation, ix.D, out);
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) {
+        cudaFree(out);
+        return fail(CHIMERA_CUDA_ERROR, "rotation: %s", cudaGetErrorString(e));
+    }
+    *rot_t = out;
     return CHIMERA_OK;
 }
 
