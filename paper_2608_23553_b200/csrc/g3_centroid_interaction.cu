@@ -1133,8 +1133,12 @@ int launch_contenders(const Index &ix, const Params &p, const int32_t *cand, con
                       const int32_t *hi, int32_t *cont, int32_t *n_cont, int32_t *scratch, const int2 *rng,
                       int2 *cont_rng, cudaStream_t st)
 {
-    if (rng != nullptr && contenders_split(ix, p)) {
-        // few queries: CONT_SPLIT blocks each (the kernel that wrote the ranges has cleared the histograms)
+    if (contenders_split(ix, p)) {
+        // few queries: CONT_SPLIT blocks each.  The kernel that wrote the ranges has cleared the histograms; without ranges
+        // (2^31 tokens or more) nothing has.
+        if (rng == nullptr)
+            CHIMERA_CUDA(cudaMemset2DAsync(scratch, sizeof(int32_t) * (size_t)p.maxc, 0, sizeof(int32_t) * CONT_BINS,
+                                           (size_t)p.B, st));
         const dim3 grid(CONT_SPLIT, (unsigned)p.B);
         launch(contender_hist_kernel, grid, SEL_THREADS, 0, st, n_cand, lo, p.maxc, p.n_prune, p.nq, scratch);
         CHIMERA_CUDA(cudaGetLastError());
