@@ -22,6 +22,7 @@
 // Every document of the exact top n_prune has an upper bound >= CI >= tau, so it is never dropped and the result is the
 // same as without these cuts.
 #include <limits.h>
+#include <math.h>
 
 #include "g3_select.cuh"
 
@@ -56,15 +57,27 @@ static int filter_codec(int64_t K)
 }
 
 // When the cut runs.  The table has to fit one SM's shared memory; a token position has to fit 32 bits and a document's
-// sum of e 31 bits; and there has to be enough to scan that the additional launches pay: 13 against 8 kernels for q_len
-// 32 / 64, whose other form scans 8-bit rows (one query of 60 M tokens, 14 M of them candidates': 248 us with the cut, 225
-// without; one of 16 queries with 48 M candidate tokens each: 5.4 against 6.7 ms), 11 against 6 for the others, which
-// look up exact rows (8 queries of 20 M tokens: 1.1 against 5.8 ms).
+// sum of e 31 bits; and there has to be enough to scan that the cut pays for its launches (13 against 8 kernels for q_len
+// 32 / 64, whose other form scans 8-bit rows, 11 against 6 for the others, which look up exact rows), for its tables (per
+// query and centroid) and for the exact rows of its seeds.  What is scanned is what the candidates hold, so their expected
+// number counts and not the room for them; a document is a candidate when one of its distinct centroids is probed.
+// In tokens, per query, fitted to calls with and without the cut (independent tokens, kept 1-60 %; the sign is right in 69
+// of 74 calls of 2,000 to 1.5 million documents, and the others lose at most a quarter):
+//   q_len 32 / 64: 8 per centroid, 5 n_prune documents, 20 M a call.  Mid's documents, one query, 12 M tokens: 206 us with
+//     the cut, 187 without; two: 248 / 266; eight: 537 / 720; 64 queries with one probe a token on 4 million documents and
+//     262,144 centroids, 2.2 M tokens each: 2,451 / 2,300; with four probes, 8.7 M each: 32 queries 2,746 / 3,103, two 414 / 372.
+//   others: 4 per centroid, 4 n_prune documents, 2 M a call.  21 tokens, 20,000 documents, 1.3 M tokens: 143 us with the cut, 133
+//     without; 2.6 M: 153 / 181; 100 tokens on 200,000 documents, 12 M: 263 / 756.
 bool filter_used(const Index &ix, const Params &p)
 {
     if (filter_codec(ix.K) == 0 || ix.T >= 0x7fffff00LL || ix.max_doclen > 32000) return false;
-    if (p.maxc < 4 * (int64_t)p.n_prune) return false;
-    return (double)p.B * (double)p.maxc * ((double)ix.T / (double)ix.N) >= (coarse_supported(p.nq) ? 2e8 : 2e7);
+    const bool wide = coarse_supported(p.nq);
+    const double len = (double)ix.T / (double)ix.N, distinct = (double)ix.ivf_len / (double)ix.N;
+    const double probed = (double)p.nq * p.P / (double)ix.K;
+    const double cand = probed < 1.0 ? (double)ix.N * (1.0 - pow(1.0 - probed, distinct)) : (double)ix.N;
+    const double tokens = (cand < (double)p.maxc ? cand : (double)p.maxc) * len;
+    const double fixed = (wide ? 8.0 : 4.0) * (double)ix.K + (wide ? 5.0 : 4.0) * p.n_prune * len;
+    return (double)p.B * (tokens - fixed) >= (wide ? 2e7 : 2e6);
 }
 size_t filter_table_pitch(const Index &ix)
 {

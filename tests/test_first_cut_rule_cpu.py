@@ -1,0 +1,53 @@
+"""When stage 3 runs its first cut: host arithmetic on the sizes, no device."""
+import os
+import subprocess
+
+import pytest
+
+
+@pytest.fixture(scope="module")
+def rule(tmp_path_factory):
+    from paper_2608_23553_b200 import build
+    build.build()
+    native = os.path.join(os.path.dirname(os.path.abspath(__file__)), "native")
+    tmp = tmp_path_factory.mktemp("rule")
+    obj, exe = str(tmp / "first_cut_rule.o"), str(tmp / "first_cut_rule")
+    subprocess.check_call([build.NVCC] + build.FLAGS + ["-c", os.path.join(native, "first_cut_rule.cu"), "-o", obj])
+    objs = [os.path.join(build.OBJ, n) for n in ("g3_filter.o", "g3_centroid_interaction.o")]
+    subprocess.check_call(["g++", "-no-pie", "-o", exe, obj, os.path.join(native, "fake_cudart.cpp")] + objs +
+                          ["-Wl,--unresolved-symbols=ignore-all"])
+
+    def used(K, N, length, B, nq, P, n_prune, distinct=None, max_len=None, max_candidates=0):
+        line = "%d %d %d %d %d %d %d %d %d %d" % (K, N, N * length, N * (distinct or length), max_len or 2 * length, B, nq, P,
+                                                  n_prune, max_candidates)
+        return subprocess.run([exe], input=line, capture_output=True, text=True, check=True).stdout.strip() == "1"
+    return used
+
+
+def test_what_the_candidates_hold_counts_and_not_the_room_for_them(rule):
+    # one query, one probe per token, 8.8 million documents of 68 tokens: 73,000 candidates, whatever the capacity
+    assert not rule(262_144, 8_800_000, 68, 1, 32, 1, 1_024)
+    assert not rule(262_144, 8_800_000, 68, 1, 32, 1, 1_024, max_candidates=80_000)
+    assert not rule(262_144, 4_000_000, 69, 64, 32, 1, 1_024)
+    # half a million documents: one query not, two and more
+    assert [rule(65_536, 500_000, 120, B, 32, 4, 1_024) for B in (1, 2, 8, 256)] == [False, True, True, True]
+    assert rule(262_144, 8_800_000, 68, 256, 32, 4, 4_096)
+    # a capacity below the expected candidates is what is scanned
+    assert rule(65_536, 500_000, 120, 4, 32, 4, 1_024) and not rule(65_536, 500_000, 120, 4, 32, 4, 1_024, max_candidates=20_000)
+    # documents of few distinct centroids are found by fewer probes
+    assert not rule(65_536, 500_000, 120, 2, 32, 4, 1_024, distinct=30)
+    # 10,000 documents: one query not, a batch
+    assert not rule(1_024, 10_000, 64, 1, 32, 4, 256) and rule(1_024, 10_000, 64, 64, 32, 4, 256)
+
+
+def test_other_query_lengths_and_what_the_cut_cannot_hold(rule):
+    assert rule(16_411, 123_457, 80, 1, 21, 6, 777) and not rule(16_411, 123_457, 80, 1, 21, 1, 777)
+    assert rule(32_768, 200_000, 100, 1, 100, 4, 1_024)
+    # nothing to cut: most candidates survive the pruning anyway
+    assert not rule(6_000, 24_000, 35, 256, 32, 1, 5_900)
+    # the numbers of 266,240 centroids still fit a block, documents of 32,000 tokens a sum
+    args = (8_800_000, 68, 256, 32, 4, 4_096)
+    assert rule(266_240, *args) and not rule(266_241, *args)
+    assert rule(262_144, *args, max_len=32_000) and not rule(262_144, *args, max_len=32_001)
+    # token positions of 31 bits
+    assert not rule(262_144, 8_800_000, 245, 256, 32, 4, 4_096)

@@ -11,20 +11,31 @@ from parity import check_query, taps_to_numpy
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("D,nbits,nq,K,N,len_lo,len_hi,B,nprobe,n_prune,shift,copies", [
-    (32, 2, 32, 509, 20_000, 1, 80, 260, 1, 300, 0, 1),          # 16-bit numbers from the 8-bit table
-    (64, 2, 64, 2_000, 20_001, 20, 61, 256, 1, 1_111, 1, 1),      # two column groups; centroid ids 4 bytes off 16
-    (128, 2, 32, 120_003, 9_999, 60, 99, 280, 16, 50, 3, 1),      # 6-bit codes, K not a multiple of five
-    (32, 1, 64, 106_497, 5_000, 200, 300, 170, 8, 20, 2, 1),      # ... just above the 16-bit limit
-    (96, 1, 21, 700, 20_000, 1, 99, 21, 2, 200, 0, 1),            # exact table, q_len < 32
-    (32, 2, 100, 3_000, 12_345, 10, 70, 45, 1, 500, 1, 1),        # ... four column groups
-    (32, 2, 40, 107_001, 8_000, 90, 120, 25, 16, 64, 0, 1),       # ... 6-bit codes
-    (64, 2, 47, 2_000, 9_000, 20, 90, 60, 1, 300, 0, 1),          # ... rows of an odd number of values, two per lane
-    (32, 2, 127, 1_000, 6_000, 20, 70, 80, 1, 200, 0, 1),         # ... four per lane, the longest query
-    (64, 2, 32, 6_000, 24_000, 1, 70, 256, 1, 5_900, 0, 1),        # queries with fewer candidates than 1.5 n_prune
-    (32, 2, 32, 300, 20_000, 1, 80, 260, 1, 333, 0, 50),          # every document 50 times: masses of equal scores
+def _cut_ran():
+    """Whether the searches since the last call ran the cut: it adds five kernels to the step."""
+    from paper_2608_23553_b200 import binding
+    return binding.profile_read()[1]["centroid_interaction"] >= 6
+
+
+# cut: whether the call runs it (the last four rows have too many centroids, or too long a pruning list, for what their
+# candidates hold)
+@pytest.mark.parametrize("cut,D,nbits,nq,K,N,len_lo,len_hi,B,nprobe,n_prune,shift,copies", [
+    (1, 32, 2, 32, 509, 20_000, 1, 80, 260, 1, 300, 0, 1),          # 16-bit numbers from the 8-bit table
+    (1, 64, 2, 64, 2_000, 20_001, 20, 61, 256, 1, 1_111, 1, 1),      # two column groups; centroid ids 4 bytes off 16
+    (1, 128, 2, 32, 120_003, 30_000, 60, 99, 250, 32, 50, 3, 1),     # 6-bit codes, K not a multiple of five
+    (1, 32, 1, 64, 106_497, 9_000, 200, 300, 170, 16, 20, 2, 1),     # ... just above the 16-bit limit
+    (1, 96, 1, 21, 700, 20_000, 1, 99, 21, 2, 200, 0, 1),            # exact table, q_len < 32
+    (1, 32, 2, 100, 3_000, 12_345, 10, 70, 45, 1, 500, 1, 1),        # ... four column groups
+    (1, 32, 2, 40, 107_001, 16_000, 90, 120, 25, 32, 64, 0, 1),      # ... 6-bit codes
+    (1, 64, 2, 47, 2_000, 9_000, 20, 90, 60, 1, 300, 0, 1),          # ... rows of an odd number of values, two per lane
+    (1, 32, 2, 127, 1_000, 6_000, 20, 70, 80, 1, 200, 0, 1),         # ... four per lane, the longest query
+    (1, 32, 2, 32, 300, 20_000, 1, 80, 260, 1, 333, 0, 50),          # every document 50 times: masses of equal scores
+    (0, 128, 2, 32, 120_003, 9_999, 60, 99, 280, 16, 50, 3, 1),
+    (0, 32, 1, 64, 106_497, 5_000, 200, 300, 170, 8, 20, 2, 1),
+    (0, 32, 2, 40, 107_001, 8_000, 90, 120, 25, 16, 64, 0, 1),
+    (0, 64, 2, 32, 6_000, 24_000, 1, 70, 256, 1, 5_900, 0, 1),       # fewer candidates than 1.5 n_prune
 ])
-def test_filtered_searches_match_the_oracle(D, nbits, nq, K, N, len_lo, len_hi, B, nprobe, n_prune, shift, copies):
+def test_filtered_searches_match_the_oracle(cut, D, nbits, nq, K, N, len_lo, len_hi, B, nprobe, n_prune, shift, copies):
     import paper_2608_23553_b200 as pkg
     cent, cids, codes, doclens = random_corpus(300 + nq + D, N // copies, K, D, nbits, len_lo=len_lo, len_hi=len_hi)
     if copies > 1:
@@ -39,10 +50,39 @@ def test_filtered_searches_match_the_oracle(D, nbits, nq, K, N, len_lo, len_hi, 
     q = (q / np.linalg.norm(q, axis=2, keepdims=True)).astype(np.float32)
     k = min(n_prune, 25)
     taps = gix.alloc_taps(B, nq, nprobe, n_prune, table=False)
+    _cut_ran()
     ids, sc = gix.search(torch.from_numpy(q).cuda(), nprobe, n_prune, k, taps=taps)
-    assert gix.status() == 0
+    assert gix.status() == 0 and _cut_ran() == bool(cut)
     tn = taps_to_numpy(taps)
     ids, sc = ids.cpu().numpy(), sc.cpu().numpy()
     for b in (0, B - 1):
         res = oracle.pipeline(q[b], oix, nprobe, n_prune, k)
         check_query(tn, b, res, ids[b], sc[b], k, n_prune, table=False)
+
+
+@pytest.mark.parametrize("nq", [32, 21])
+def test_queries_with_few_candidates_in_a_batch_that_is_cut(nq):
+    """The first query has more candidates than n_prune but fewer than the cut wants seeds, the last one fewer than n_prune."""
+    import paper_2608_23553_b200 as pkg
+    D, K, N, B, n_prune, k = 64, 2_000, 20_000, 260, 300, 20
+    cent, cids, codes, doclens = random_corpus(77, N, K, D, 2, len_lo=30, len_hi=50)
+    rng = np.random.default_rng(5)
+    cids = rng.integers(64, K, size=len(cids)).astype(np.int32)           # centroids 0 ... 63 only where they are put:
+    first = np.concatenate([[0], np.cumsum(doclens)[:-1]])
+    docs = rng.permutation(N)
+    cids[first[docs[:420]]] = rng.integers(0, nq, size=420)
+    cids[first[docs[420:520]]] = rng.integers(32, 32 + nq, size=100)
+    oix = oracle.make_index(cent, cids, codes, doclens, 2)
+    gix = pkg.Index(*(torch.from_numpy(a).cuda() for a in (cent, cids, codes, doclens)), 2)
+    c = rng.integers(64, K, size=(B, nq))
+    c[0], c[-1] = np.arange(nq), 32 + np.arange(nq)
+    q = cent[c].copy()
+    taps = gix.alloc_taps(B, nq, 1, n_prune, table=False)
+    _cut_ran()
+    ids, sc = gix.search(torch.from_numpy(q).cuda(), 1, n_prune, k, taps=taps)
+    assert gix.status() == 0 and _cut_ran()
+    tn = taps_to_numpy(taps)
+    assert n_prune < tn["n_cand"][0] < 1.5 * n_prune and 0 < tn["n_cand"][-1] < n_prune and tn["n_cand"][1] > 1_000
+    for b in (0, 1, B - 1):
+        res = oracle.pipeline(q[b], oix, 1, n_prune, k)
+        check_query(tn, b, res, ids[b].cpu().numpy(), sc[b].cpu().numpy(), k, n_prune, table=False)
