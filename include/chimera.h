@@ -259,6 +259,14 @@ int chimera_search_rabitq_graph(const chimera_index *index, const float *queries
  * [-1, 1]), CHIMERA_TIMEOUT or (debug build) CHIMERA_DEBUG_CHECK_FAILED to *status (host pointer). */
 int chimera_workspace_status(const void *workspace, void *stream, int32_t *status);
 
+/* After a chimera_search with these parameters on `workspace`: how many candidates of each query the first cut of its
+ * centroid-interaction step left to the later ones (Sec. 3.2 step 2 scores every candidate; the cut drops, by a cheap upper
+ * bound, those that cannot be among the n_prune best).  Synchronises the stream and writes n_queries numbers to n_kept
+ * (host pointer): -1 where calls of these sizes do not cut; all candidates where a sample of them showed that the bound
+ * would not drop enough, as on documents that repeat their centroids. */
+int chimera_workspace_kept(const chimera_index *index, int32_t n_queries, int32_t q_len, int32_t nprobe, int32_t n_prune,
+                           int32_t k, int64_t max_candidates, const void *workspace, void *stream, int32_t *n_kept);
+
 /* How a search with these parameters finds its probes (Sec. 3.2 step 1, the top-n_probe centroids of each query
  * token).  Writes to *sample_stride (host pointer) 0 when stage 2a is a scan of the finished score table, or s > 1
  * when stages 1 and 2a run together in calls that cover both: every s-th tile of 128 centroids is scored first, a

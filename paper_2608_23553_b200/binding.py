@@ -313,6 +313,15 @@ class Index:
                                         ctypes.c_int32(nprobe), ctypes.byref(s)))
         return s.value
 
+    def kept(self, n_queries, q_len, nprobe, n_prune, k, max_candidates=0) -> list:
+        """After a search with these parameters (pruning by centroid interaction): the candidates of each query that the
+        first cut left, -1 where calls of these sizes do not cut (chimera_workspace_kept)."""
+        out = (ctypes.c_int32 * n_queries)()
+        _check(lib().chimera_workspace_kept(self._h, ctypes.c_int32(n_queries), ctypes.c_int32(q_len),
+                                            ctypes.c_int32(nprobe), ctypes.c_int32(n_prune), ctypes.c_int32(k),
+                                            ctypes.c_int64(max_candidates), _ptr(self._ws), _stream(), out))
+        return list(out)
+
     def workspace_check(self, n_queries, q_len, nprobe, n_prune, k, max_candidates=0) -> int:
         """Debug build only: index of the first damaged guard region of the workspace after a search with these
         parameters, -1 if all are intact (chimera_workspace_check)."""

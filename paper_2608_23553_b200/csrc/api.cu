@@ -140,8 +140,10 @@ Layout make_layout(const Index &ix, const Params &p)
     L.flt_tab = take(filter ? B * filter_table_pitch(ix) : 0);
     L.flt_hist = take(filter ? B * (size_t)filter_hist_bins() * sizeof(int32_t) : 0);
     L.flt_thr = take(filter ? B * sizeof(int32_t) : 0);
-    L.flt_slot = L.lo;                  // (the filtered pipeline has no lower bounds)
+    L.flt_slot = L.lo;                  // (a call that cuts has no lower bounds, one that does not has no seeds)
     L.flt_tau = take(filter ? B * sizeof(int32_t) : 0);
+    L.flt_smp = take(filter ? JUDGE_SAMPLES * sizeof(int2) : 0);
+    L.flt_vote = take(filter ? 64 * sizeof(int32_t) : 0);
     L.flt_parts = take(filter ? filter_parts_bytes(ix, p) : 0);
     L.flt_counts = take(filter ? B * (size_t)filter_count_slots() * sizeof(int32_t) : 0);
     L.kept = take(filter ? two_phase : 0);
@@ -400,17 +402,19 @@ static int run(const Index &ix, const Params &p, int first, int last, const floa
                 if ((rc = launch_filter_keep(ix, p, L, cand, n_cand, hi, ci, kept, kept_rng, n_kept, ws, st))) return rc;
                 prof_mark(SLOT_SELECT, st);
                 docs = kept; n_docs = n_kept; docs_rng = kept_rng;
-                // upper bounds of the kept ones from the 8-bit table
-                if ((rc = launch_coarse_bounds(ix, p, (uint8_t *)(ws + L.table8), docs, n_docs, nullptr, hi, docs_rng, st)))
+                // upper bounds of the kept ones from the 8-bit table (lower bounds too where the call turned out not to cut)
+                const FirstCut cut = first_cut(p, L, ws);
+                if ((rc = launch_coarse_bounds(ix, p, (uint8_t *)(ws + L.table8), docs, n_docs, two_phase ? lo : nullptr, hi,
+                                               docs_rng, &cut, st)))
                     return rc;
                 prof_mark(SLOT_CI, st);
-                if ((rc = launch_filter_contenders(ix, p, L, docs, docs_rng, n_docs, hi, cont, cont_rng, n_cont, ws, st)))
+                if ((rc = launch_filter_contenders(ix, p, L, docs, docs_rng, n_docs, lo, hi, cont, cont_rng, n_cont, ws, st)))
                     return rc;
                 prof_mark(SLOT_SELECT, st);
                 docs = cont; n_docs = n_cont; docs_rng = cont_rng;
             } else if (two_phase) {
                 // bounds for every candidate, contenders for the top n_prune, exact CI and selection among those
-                if ((rc = launch_coarse_bounds(ix, p, table8, docs, n_docs, lo, hi, docs_rng, st))) return rc;
+                if ((rc = launch_coarse_bounds(ix, p, table8, docs, n_docs, lo, hi, docs_rng, nullptr, st))) return rc;
                 prof_mark(SLOT_CI, st);
                 if ((rc = launch_contenders(ix, p, docs, n_docs, lo, hi, cont, n_cont, ci, docs_rng, cont_rng, st))) return rc;
                 prof_mark(SLOT_SELECT, st);
@@ -869,6 +873,25 @@ int chimera_probe_plan(const chimera_index *index, int32_t n_queries, int32_t q_
     if (rc) return rc;
     if (!sample_stride) return fail(CHIMERA_INVALID_ARG, "NULL argument");
     *sample_stride = probe_queue_stride(*ix, p);
+    return CHIMERA_OK;
+}
+
+int chimera_workspace_kept(const chimera_index *index, int32_t n_queries, int32_t q_len, int32_t nprobe, int32_t n_prune,
+                           int32_t k, int64_t max_candidates, const void *workspace, void *stream, int32_t *n_kept)
+{
+    const Index *ix = reinterpret_cast<const Index *>(index);
+    Params p;
+    int rc = check_params(ix, n_queries, q_len, nprobe, n_prune, k, max_candidates, &p);
+    if (rc) return rc;
+    if (!workspace || !n_kept) return fail(CHIMERA_INVALID_ARG, "NULL argument");
+    if (!filter_used(*ix, p)) {
+        for (int b = 0; b < p.B; ++b) n_kept[b] = -1;
+        return CHIMERA_OK;
+    }
+    const Layout L = make_layout(*ix, p);
+    CHIMERA_CUDA(cudaMemcpyAsync(n_kept, (const char *)workspace + L.n_kept, sizeof(int32_t) * (size_t)p.B,
+                                 cudaMemcpyDeviceToHost, (cudaStream_t)stream));
+    CHIMERA_CUDA(cudaStreamSynchronize((cudaStream_t)stream));
     return CHIMERA_OK;
 }
 

@@ -60,6 +60,15 @@ struct Params {
     int64_t maxc;                     // candidate capacity per query
 };
 
+// Whether a call cuts (on the device).  The load belongs beside a kernel's first ones, in front of the branch on it.
+struct FirstCut {
+    const int32_t *kept = nullptr;     // sampled candidates that would be kept; NULL: the call cuts
+    int32_t most = 0;                  // with more of them it does not
+#ifdef __CUDACC__
+    __device__ __forceinline__ bool on() const { return kept == nullptr || __ldg(kept) <= most; }
+#endif
+};
+
 constexpr int MAX_GUARDS = 64;
 struct Layout {
     // debug builds (CHIMERA_DEBUG) put a 256-byte guard region behind every region below; guards[i] is its offset
@@ -97,7 +106,9 @@ struct Layout {
     size_t flt_parts;     // int32  histograms and counters of the threshold kernel's blocks (few queries)
     size_t flt_thr;       // int32  [B]               hi0 from which a candidate is a seed,
     size_t flt_slot;      // int32  [B][maxc]         place of each seed in the seed list,
-    size_t flt_tau;       // int32  [B]               n_prune-th largest exact CI of the seeds,
+    size_t flt_tau;       // int32  [B]               n_prune-th largest exact CI of the seeds (lower bound, without the cut),
+    size_t flt_smp;       // int2   [JUDGE_SAMPLES]   CI and first bound of sampled candidates,
+    size_t flt_vote;      // int32  [64]              how many of those would be kept, counters of the kernel that finds out,
     size_t flt_counts;    // int32  [B][slots]        kept candidates per slice
     size_t kept;          // int32  [B][maxc]         candidates that pass it, ascending
     size_t kept_rng;      // int2   [B][maxc]         their token ranges
@@ -244,8 +255,8 @@ int launch_partial_scores(const Index &ix, const Params &p, const Layout &L, con
                           const int32_t *table, const int32_t *probes, const uint2 *ranks, const int32_t *n_cand,
                           void *partial_m, int32_t *fprime, cudaStream_t st);
 int launch_filter_contenders(const Index &ix, const Params &p, const Layout &L, const int32_t *kept, const int2 *kept_rng,
-                             const int32_t *n_kept, const int32_t *hi, int32_t *cont, int2 *cont_rng, int32_t *n_cont,
-                             char *ws, cudaStream_t st);
+                             const int32_t *n_kept, const int32_t *lo, const int32_t *hi, int32_t *cont, int2 *cont_rng,
+                             int32_t *n_cont, char *ws, cudaStream_t st);
 bool coarse_supported(int nq);
 int coarse_pitch(int nq);       // bytes of an 8-bit row
 int launch_coarse_table(const Index &ix, const Params &p, const int32_t *table, uint8_t *table8, cudaStream_t st);
@@ -254,13 +265,17 @@ int launch_coarse_table(const Index &ix, const Params &p, const int32_t *table, 
 int launch_cand_ranges(const Index &ix, const Params &p, const int32_t *cand, const int32_t *n_cand, int2 *rng,
                        int32_t *cont_scratch, cudaStream_t st);
 // rng: those ranges (may be NULL: per-document offset lookups instead; (CI, 0) stands for a document whose exact CI is
-// known).  lo may be NULL with ranges.
+// known).  lo may be NULL with ranges.  cut (may be NULL, else with ranges): a call that cuts wants no lower
+// bounds, one that does not knows no document's CI.
 int launch_coarse_bounds(const Index &ix, const Params &p, const uint8_t *table8, const int32_t *cand,
-                         const int32_t *n_cand, int32_t *lo, int32_t *hi, const int2 *rng, cudaStream_t st);
+                         const int32_t *n_cand, int32_t *lo, int32_t *hi, const int2 *rng, const FirstCut *cut, cudaStream_t st);
 // First cut of the candidates by an upper bound from one number per token (g3_filter.cu).  launch_filter_scan leaves the
 // bounds in hi0 and the best ~2 n_prune candidates in seed / seed_rng (their number in the workspace's n_seed);
 // launch_filter_keep takes the seeds' exact CI and writes the candidates that can still be in the top n_prune, ascending;
-// launch_filter_contenders narrows them down by the 8-bit upper bounds.
+// launch_filter_contenders narrows them down by the 8-bit upper bounds.  Where a sample shows that the cut would keep most
+// candidates, there are no seeds, all candidates are kept, and the contenders are found by the 8-bit lower bounds.
+constexpr int JUDGE_QUERIES = 16, JUDGE_SAMPLES = 4096;
+FirstCut first_cut(const Params &p, const Layout &L, char *ws);
 bool filter_used(const Index &ix, const Params &p);
 size_t filter_table_pitch(const Index &ix);
 int filter_hist_bins();

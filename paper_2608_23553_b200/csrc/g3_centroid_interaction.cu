@@ -291,15 +291,18 @@ __device__ __forceinline__ void coarse_accumulate2(uint32_t (&m)[8], const int4 
 }
 __device__ __forceinline__ int coarse_field_lo(uint32_t m) { return (int)((m >> 8) & 0xffu); }
 __device__ __forceinline__ int coarse_field_hi(uint32_t m) { return (int)(m >> 24); }
+// cut: of a call that may cut (kept not NULL): nothing is done when it does.
 // SMEM = true: the query's whole 8-bit table (K * q_len bytes) is first staged in shared memory and the row lookups
 // are shared-memory loads (small K only); blocks are then larger (THREADS) because only one fits an SM.
 template <int LPR, bool SMEM, int THREADS>
 __global__ void __launch_bounds__(THREADS)
 ci_coarse_kernel(const uint8_t *__restrict__ table8, int64_t K, const int32_t *__restrict__ cand,
                  const int32_t *__restrict__ n_cand, int64_t maxc, const int32_t *__restrict__ cids,
-                 const int64_t *__restrict__ doc_off, int32_t *__restrict__ lo, int32_t *__restrict__ hi)
+                 const int64_t *__restrict__ doc_off, int32_t *__restrict__ lo, int32_t *__restrict__ hi,
+                 FirstCut cut)
 {
     pdl_entry();
+    if (cut.kept && cut.on()) return;             // (the scan over ranges does it)
     extern __shared__ int4 smem_table[];
     constexpr int WARPS = THREADS / 32;
     constexpr int NQ = 16 * LPR;
@@ -574,6 +577,7 @@ ci_coarse_rng_body(const uint8_t *__restrict__ table8, int64_t K, int nq, const 
     }
 }
 
+// cut: of a call that may cut (kept not NULL): no lower bounds when it does; otherwise, with cut_only, nothing is done.
 // Two launch forms of the scan.  32-byte rows: no occupancy hint (the compiler's own 64 registers, four blocks per SM;
 // any hint measured slower).  64-byte rows: four blocks per SM instead of the three that the unhinted 75 registers
 // give (long-document corpus: 27.1 against 28.4 ms).
@@ -581,18 +585,26 @@ template <int LPR>
 __global__ void __launch_bounds__(CI_THREADS)
 ci_coarse_rng_kernel(const uint8_t *__restrict__ table8, int64_t K, const int2 *__restrict__ rng,
                      const int32_t *__restrict__ n_cand, int64_t maxc, const int32_t *__restrict__ cids,
-                     int32_t *__restrict__ lo, int32_t *__restrict__ hi)
+                     int32_t *__restrict__ lo, int32_t *__restrict__ hi, FirstCut cut, bool cut_only)
 {
     pdl_entry();
+    if (cut.kept) {
+        if (cut.on()) lo = nullptr;
+        else if (cut_only) return;
+    }
     ci_coarse_rng_body<LPR>(table8, K, 16 * LPR, rng, n_cand, maxc, cids, lo, hi);
 }
 template <int LPR>
 __global__ void __launch_bounds__(CI_THREADS, 4)
 ci_coarse_rng_kernel_b4(const uint8_t *__restrict__ table8, int64_t K, const int2 *__restrict__ rng,
                         const int32_t *__restrict__ n_cand, int64_t maxc, const int32_t *__restrict__ cids,
-                        int32_t *__restrict__ lo, int32_t *__restrict__ hi)
+                        int32_t *__restrict__ lo, int32_t *__restrict__ hi, FirstCut cut, bool cut_only)
 {
     pdl_entry();
+    if (cut.kept) {
+        if (cut.on()) lo = nullptr;
+        else if (cut_only) return;
+    }
     ci_coarse_rng_body<LPR>(table8, K, 16 * LPR, rng, n_cand, maxc, cids, lo, hi);
 }
 
@@ -631,11 +643,13 @@ int launch_cand_ranges(const Index &ix, const Params &p, const int32_t *cand, co
 }
 
 int launch_coarse_bounds(const Index &ix, const Params &p, const uint8_t *table8, const int32_t *cand,
-                         const int32_t *n_cand, int32_t *lo, int32_t *hi, const int2 *rng, cudaStream_t st)
+                         const int32_t *n_cand, int32_t *lo, int32_t *hi, const int2 *rng, const FirstCut *cut, cudaStream_t st)
 {
     const size_t table_bytes = (size_t)ix.K * coarse_pitch(p.nq);
     const bool use_rng = rng != nullptr;
-    if (table_bytes <= 160 * 1024 && lo != nullptr) {
+    const FirstCut call_cut = cut ? *cut : FirstCut();
+    const bool small = table_bytes <= 160 * 1024 && lo != nullptr;
+    if (small) {
         // the whole 8-bit table of a query fits in shared memory: stage it once per block and look rows up there
         constexpr int T = 512;
         int64_t gx = (4LL * ix.sm_count + p.B - 1) / p.B;       // every block re-reads the table: few, long blocks
@@ -650,16 +664,16 @@ int launch_coarse_bounds(const Index &ix, const Params &p, const uint8_t *table8
             CHIMERA_CUDA(cudaFuncSetAttribute(ci_coarse_kernel<2, true, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)table_bytes));
             launch(ci_coarse_kernel<2, true, T>, grid, T, table_bytes, st, table8, ix.K, cand, n_cand, p.maxc, ix.cids,
-                                                                       ix.doc_off, lo, hi);
+                                                                       ix.doc_off, lo, hi, call_cut);
         } else {
             CHIMERA_CUDA(cudaFuncSetAttribute(ci_coarse_kernel<4, true, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)table_bytes));
             launch(ci_coarse_kernel<4, true, T>, grid, T, table_bytes, st, table8, ix.K, cand, n_cand, p.maxc, ix.cids,
-                                                                       ix.doc_off, lo, hi);
+                                                                       ix.doc_off, lo, hi, call_cut);
         }
         CHIMERA_CUDA(cudaGetLastError());
         count_launch(SLOT_CI);
-        return CHIMERA_OK;
+        if (!cut) return CHIMERA_OK;             // (a cut leaves documents whose CI is known: they are passed over below)
     }
     // Blocks per query.  Four blocks are resident per SM and the blocks of a query are adjacent in the grid, so
     // (resident blocks) / (blocks per query) queries are scanned at the same time and their 8-bit tables compete for
@@ -682,19 +696,21 @@ int launch_coarse_bounds(const Index &ix, const Params &p, const uint8_t *table8
             auto kern = p.nq <= 32 ? ci_coarse_rng_kernel_pad<2> : p.nq <= 64 ? ci_coarse_rng_kernel_pad<4> : ci_coarse_rng_kernel_pad<8>;
             launch(kern, grid, CI_THREADS, 0, st, table8, ix.K, p.nq, rng, n_cand, p.maxc, ix.cids, hi);
         } else if (p.nq == 32)
-            launch(ci_coarse_rng_kernel<2>, grid, CI_THREADS, 0, st, table8, ix.K, rng, n_cand, p.maxc, ix.cids, lo, hi);
+            launch(ci_coarse_rng_kernel<2>, grid, CI_THREADS, 0, st, table8, ix.K, rng, n_cand, p.maxc, ix.cids, lo, hi, call_cut,
+                   small);
         else
-            launch(ci_coarse_rng_kernel_b4<4>, grid, CI_THREADS, 0, st, table8, ix.K, rng, n_cand, p.maxc, ix.cids, lo, hi);
+            launch(ci_coarse_rng_kernel_b4<4>, grid, CI_THREADS, 0, st, table8, ix.K, rng, n_cand, p.maxc, ix.cids, lo, hi, call_cut,
+                   small);
         CHIMERA_CUDA(cudaGetLastError());
         count_launch(SLOT_CI);
         return CHIMERA_OK;
     }
     if (p.nq == 32)
         launch(ci_coarse_kernel<2, false, CI_THREADS>, grid, CI_THREADS, 0, st, table8, ix.K, cand, n_cand, p.maxc, ix.cids,
-                                                                          ix.doc_off, lo, hi);
+                                                                          ix.doc_off, lo, hi, FirstCut());
     else
         launch(ci_coarse_kernel<4, false, CI_THREADS>, grid, CI_THREADS, 0, st, table8, ix.K, cand, n_cand, p.maxc, ix.cids,
-                                                                          ix.doc_off, lo, hi);
+                                                                          ix.doc_off, lo, hi, FirstCut());
     CHIMERA_CUDA(cudaGetLastError());
     count_launch(SLOT_CI);
     return CHIMERA_OK;
@@ -827,10 +843,6 @@ select_kernel(const int32_t *__restrict__ cand, const int32_t *__restrict__ n_ca
 
 // grid (B).  Contenders for the top n_prune: with tau = the n_prune-th largest lower bound, every document of the
 // true top n_prune has hi >= CI >= (n_prune-th largest CI) >= tau.  Writes their ids (ascending) and their number.
-// The lower bounds are lo = 2^16 sum - zeros (2^24 + 64) with sum = the sum of nq 8-bit maxima (coarse_lo), so
-// coarse_key(lo) = floor(lo / 2^16), clamped at 0, is a key of at most 14 bits and 2^16 key <= lo: one histogram sweep
-// over CONT_BINS bins (two neighbouring keys share a bin for q_len 64; tau is then the smaller of the two, still a
-// valid lower threshold) finds tau without radix passes.
 __global__ void __launch_bounds__(SEL_THREADS)
 contender_kernel(const int32_t *__restrict__ cand, const int32_t *__restrict__ n_cand, const int32_t *__restrict__ lo,
                  const int32_t *__restrict__ hi, int64_t maxc, int n_prune, int nq, int32_t *__restrict__ cont,
@@ -856,40 +868,7 @@ contender_kernel(const int32_t *__restrict__ cand, const int32_t *__restrict__ n
         if (threadIdx.x == 0) n_cont[b] = n;
         return;
     }
-    const int bin_shift = 255 * nq < CONT_BINS ? 0 : 1;            // q_len 32: one sum per bin; q_len 64: two
-    for (int i = threadIdx.x; i < CONT_BINS; i += SEL_THREADS) hist[i] = 0;
-    __syncthreads();
-    for (int base = 0; base < n; base += 16 * SEL_THREADS) {
-        int32_t v[16];
-#pragma unroll
-        for (int e = 0; e < 16; ++e) {
-            const int j = base + e * SEL_THREADS + threadIdx.x;
-            v[e] = j < n ? lb[j] : 0;
-        }
-#pragma unroll
-        for (int e = 0; e < 16; ++e) {
-            const int j = base + e * SEL_THREADS + threadIdx.x;
-            if (j < n) atomicAdd(&hist[coarse_key(v[e]) >> bin_shift], 1);
-        }
-    }
-    __syncthreads();
-    // descending bins, CONT_BINS / SEL_THREADS consecutive bins per thread
-    constexpr int PER = CONT_BINS / SEL_THREADS;
-    const int first_bin = CONT_BINS - 1 - PER * (int)threadIdx.x;  // this thread owns first_bin, first_bin - 1, ...
-    int h[PER], mine = 0;
-#pragma unroll
-    for (int e = 0; e < PER; ++e) { h[e] = hist[first_bin - e]; mine += h[e]; }
-    int total;
-    int before = sel_block_scan(mine, &total, warp_part);
-    if (before < n_prune && n_prune <= before + mine) {
-#pragma unroll
-        for (int e = 0; e < PER; ++e) {
-            if (before < n_prune && n_prune <= before + h[e]) s_bin = first_bin - e;
-            before += h[e];
-        }
-    }
-    __syncthreads();
-    const int32_t tau = (s_bin << bin_shift) << 16;                 // smallest lower bound of that bin
+    const int32_t tau = contender_threshold(lb, n, n_prune, nq, hist, warp_part, &s_bin);
     // ordered compaction, eight consecutive entries per thread and round (one block scan per 8192 entries); the ids
     // are only read for the few entries that are kept
     int run = 0;
@@ -1024,7 +1003,7 @@ contender_hist_kernel(const int32_t *__restrict__ n_cand, const int32_t *__restr
     int j0, j1;
     cont_slice(n, blockIdx.x, &j0, &j1);
     const int32_t *lb = lo + (int64_t)b * maxc;
-    const int bin_shift = 255 * nq < CONT_BINS ? 0 : 1;
+    const int bin_shift = contender_bin_shift(nq);
     for (int i = threadIdx.x; i < CONT_BINS; i += SEL_THREADS) hist[i] = 0;
     __syncthreads();
     for (int j = j0 + threadIdx.x; j < j1; j += SEL_THREADS)
@@ -1046,7 +1025,7 @@ contender_count_kernel(const int32_t *__restrict__ n_cand, const int32_t *__rest
     int32_t *gh = scratch + (int64_t)b * maxc;
     int32_t tau = INT_MIN;
     if (n > n_prune) {
-        const int bin_shift = 255 * nq < CONT_BINS ? 0 : 1;
+        const int bin_shift = contender_bin_shift(nq);
         constexpr int PER = CONT_BINS / SEL_THREADS;
         const int first_bin = CONT_BINS - 1 - PER * (int)threadIdx.x;
         int h[PER], mine = 0;

@@ -9,7 +9,12 @@
 // token per column of a long document the bound keeps 7-13 % of the candidates when 1 % are wanted (65,536 and 262,144
 // centroids, candidates of 85-512 tokens), with half or one and a half times as many up to twice that.
 //
+// With documents that repeat their centroids, or hold several near the same query token, the bound counts each of them where
+// CI counts one, and most candidates pass it; then the cut only costs (below, at filter_judge_kernel).
+//
 //   filter_theta_kernel    theta_i from a sample of the table's rows
+//   filter_judge_kernel    q_len 32 / 64: whether the cut would drop enough, from sampled candidates; if not, the kernels
+//                          down to the count return at once, all candidates are kept, and their 8-bit bounds decide
 //   filter_excess_kernel   e(c) of every centroid, rounded up (16 bits, or 6-bit codes five to a word for large K)
 //   filter_scan_kernel     hi0 of every candidate: the query's whole e table in shared memory, one lookup per token
 //   filter_seed_kernel     the ~2 n_prune candidates with the largest hi0 (their order does not matter)
@@ -32,6 +37,7 @@ constexpr double FILTER_LAMBDA = 1.0;     // wanted tokens of a document above t
 constexpr int FILTER_SAMPLE = 4096;       // table rows sampled per query for theta
 constexpr int KEEP_SPLIT = 32;            // most blocks per query of the selection kernels
 constexpr int FILTER_BINS = 2048;         // histogram bins of sum_t e(c_t), 2^17 (one 128th) each
+constexpr int JUDGE_KEPT_PERCENT = 58;        // of the sampled candidates: with more the call does without the cut
 constexpr int64_t FILTER_SMEM = 208 * 1024;   // shared memory of the scan's block that its e table may take
 
 // 6-bit codes of e in units of 2^16 (1/256): exact up to 20, then steps of about 7 % (the sums of a document's far
@@ -57,7 +63,7 @@ static int filter_codec(int64_t K)
 }
 
 // When the cut runs.  The table has to fit one SM's shared memory; a token position has to fit 32 bits and a document's
-// sum of e 31 bits; and there has to be enough to scan that the cut pays for its launches (13 against 8 kernels for q_len
+// sum of e 31 bits; and there has to be enough to scan that the cut pays for its launches (14 against 8 kernels for q_len
 // 32 / 64, whose other form scans 8-bit rows, 11 against 6 for the others, which look up exact rows), for its tables (per
 // query and centroid) and for the exact rows of its seeds.  What is scanned is what the candidates hold, so their expected
 // number counts and not the room for them; a document is a candidate when one of its distinct centroids is probed.
@@ -97,6 +103,17 @@ static int filter_split(const Index &ix, const Params &p)
     return (int)(g > KEEP_SPLIT ? KEEP_SPLIT : g < 1 ? 1 : g);
 }
 
+// Queries that the judge samples, candidates of each, and what the kernels behind it go by.
+static int judge_queries(const Params &p) { return p.B < JUDGE_QUERIES ? p.B : JUDGE_QUERIES; }
+static int judge_samples(const Params &p) { return JUDGE_SAMPLES / 32 / judge_queries(p) * 32; }
+FirstCut first_cut(const Params &p, const Layout &L, char *ws)
+{
+    FirstCut c;
+    c.kept = coarse_supported(p.nq) ? (const int32_t *)(ws + L.flt_vote) : nullptr;
+    c.most = judge_queries(p) * judge_samples(p) * JUDGE_KEPT_PERCENT / 100;
+    return c;
+}
+
 // Blocks per query and column group of the theta kernel, and the bytes they share.
 static int filter_parts(const Index &ix, const Params &p) { return 4 * p.B <= ix.sm_count ? 8 : 1; }
 size_t filter_parts_bytes(const Index &ix, const Params &p)
@@ -108,15 +125,17 @@ size_t filter_parts_bytes(const Index &ix, const Params &p)
 // grid (ceil(nq / 32), B, parts), lane = query token.  theta[b][i] = the smallest t (in units of 2^16) such that at most
 // `rank` of the m sampled rows (every step-th one) have S >= t 2^16.  With few queries the sample is split over several
 // blocks that add their histograms up in `parts_hist` ([B][groups][256 * 32], zero before and afterwards); the last one to
-// finish (`done`, likewise) reads the sum.  Also clears what the scan and the seed selection add to.
+// finish (`done`, likewise) reads the sum.  Also clears what the scan and the seed selection add to, and the judge's words (vote,
+// may be NULL).
 __global__ void __launch_bounds__(SEL_THREADS)
 filter_theta_kernel(const int32_t *__restrict__ table, int64_t K, int nq, int m, int step, int rank,
                     int32_t *__restrict__ theta, int32_t *__restrict__ hist_out, int32_t *__restrict__ n_seed,
-                    int32_t *__restrict__ parts_hist, int32_t *__restrict__ done)
+                    int32_t *__restrict__ parts_hist, int32_t *__restrict__ done, int32_t *__restrict__ vote)
 {
     pdl_entry();
     __shared__ int hist[256 * 32];
     __shared__ int s_last;
+    if (vote && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x < 64) vote[threadIdx.x] = 0;
     const int b = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int col = blockIdx.x * 32 + lane;
     for (int i = threadIdx.x; i < 256 * 32; i += SEL_THREADS) hist[i] = 0;
@@ -179,6 +198,119 @@ filter_theta_kernel(const int32_t *__restrict__ table, int64_t K, int nq, int m,
     if (lane == 0 && blockIdx.x * 32 + warp < nq) theta[(int64_t)b * nq + blockIdx.x * 32 + warp] = best;
 }
 
+// ------------------------------------------------------------------------------------------------ judge -----------
+// Does the cut pay?  JUDGE_SAMPLES candidates, spread over up to JUDGE_QUERIES queries of the call: CI from the 8-bit rows
+// and the bound hi0, then the share of them whose bound reaches the sample's own n_prune-th of n_cand.  A query with so few
+// candidates that all are kept counts as kept.  Queries of a batch search the same documents, so one answer per call is
+// enough, and results do not depend on it.
+// Where the line lies (batches of Mid's sizes unless said; the share that passes, with the cut / without it): documents that
+// draw a quarter as many centroids as they have tokens (100 %): 8.09 / 6.36 ms; of neighbouring centroids of four topics (63 %,
+// by the sample 57 %): 9.76 / 9.21, 16 queries (66 %, by the sample 60 %): 1,034 / 873 us; 512 tokens of such (35 %, sample 27 %):
+// 25.7 / 28.7 ms; independent centroids, 16 queries, n_prune 16,384 (55 %, sample 56 %): 2.96 / 3.04 ms.  As the judge has it: 6.46
+// ms, 9.73 ms, 915 us, 25.8 ms and 2.96 ms.  It costs 15 us where the cut stays (16 queries: 809 -> 825 us), most of it latency:
+// candidate, range, ids, rows, then the last block's histogram.
+// grid (blocks, queries), a document per warp, sixteen columns per lane, 64 tokens in flight.
+template <int NQ>
+__global__ void __launch_bounds__(SEL_THREADS)
+filter_judge_kernel(const uint8_t *__restrict__ table8, int64_t K, const int32_t *__restrict__ theta, int B,
+                    const int32_t *__restrict__ cand, const int32_t *__restrict__ n_cand, int64_t maxc,
+                    const int64_t *__restrict__ doc_off, const int32_t *__restrict__ cids, int n_prune, bool coded,
+                    int2 *__restrict__ smp, int32_t *__restrict__ vote)
+{
+    pdl_entry();
+    constexpr int LPR = NQ / 16;                             // lanes per row, 16 columns each
+    constexpr int TPL = 32 / LPR;                            // rows per load of the warp
+    constexpr int BINS = 2048;                               // of 8 units: CI <= 64 (255 + 1/2)
+    __shared__ int hist[BINS];
+    __shared__ int warp_part[32];
+    __shared__ int s_last, s_bin;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = lane % LPR, grp = lane / LPR;
+    const int b = (int)((int64_t)blockIdx.y * B / gridDim.y), m = (int)gridDim.x * 32;
+    const int n = n_cand[b];
+    int32_t *ticket = vote + 1 + blockIdx.y;
+    int2 *mine = smp + (int64_t)blockIdx.y * m;
+    const bool few = n <= 2 * n_prune + 32;
+    if (!few) {
+        const int s = blockIdx.x * 32 + warp;
+        const int2 r = doc_range(doc_off, cand[(int64_t)b * maxc + (int64_t)s * n / m]);
+        const uint4 *tb = reinterpret_cast<const uint4 *>(table8 + (int64_t)b * K * NQ) + sub;
+        uint2 tm1[4];                                        // thresholds minus one, as in filter_row_excess
+        int sum_tm1 = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int4 t = __ldg(reinterpret_cast<const int4 *>(theta + (int64_t)b * NQ + 16 * sub) + k);
+            tm1[k] = make_uint2((uint32_t)(t.x - 1) | (uint32_t)(t.z - 1) << 16, (uint32_t)(t.y - 1) | (uint32_t)(t.w - 1) << 16);
+            sum_tm1 += t.x + t.y + t.z + t.w - 4;
+        }
+        uint32_t best[4] = {0u, 0u, 0u, 0u};
+        int over = 0;
+        int32_t cid[2];                                      // 64 tokens at a time
+#pragma unroll
+        for (int h = 0; h < 2; ++h) cid[h] = 32 * h + lane < r.y ? cids[r.x + 32 * h + lane] : 0;
+        for (int t0 = 0; t0 < r.y; t0 += 64) {
+            uint4 v[2 * LPR];
+#pragma unroll
+            for (int u = 0; u < 2 * LPR; ++u) {
+                const int64_t c = DBG_CID(__shfl_sync(0xffffffffu, cid[u / LPR], u % LPR * TPL + grp));
+                v[u] = t0 + u * TPL + grp < r.y ? __ldg(tb + c * LPR) : make_uint4(0u, 0u, 0u, 0u);
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int t = t0 + 64 + 32 * h + lane;
+                cid[h] = t < r.y ? cids[r.x + t] : 0;
+            }
+#pragma unroll
+            for (int u = 0; u < 2 * LPR; ++u) {
+                const uint32_t w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+                uint32_t acc = 0;                            // 16-bit fields of at most 8 * 255
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    best[k] = __vmaxu4(best[k], w[k]);
+                    acc += __vmaxu2(w[k] & 0x00ff00ffu, tm1[k].x) + __vmaxu2((w[k] >> 8) & 0x00ff00ffu, tm1[k].y);
+                }
+                over += (int)(acc & 0xffffu) + (int)(acc >> 16) - sum_tm1;
+            }
+        }
+        int ci = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+#pragma unroll
+            for (int o = LPR; o < 32; o <<= 1) best[k] = __vmaxu4(best[k], __shfl_xor_sync(0xffffffffu, best[k], o));
+            ci += (int)__vsadu4(best[k], 0u);
+        }
+        ci = __reduce_add_sync(0xffffffffu, lane < LPR ? ci : 0) + NQ / 2;
+        over = __reduce_add_sync(0xffffffffu, over);
+        const int base = __reduce_add_sync(0xffffffffu, lane < LPR ? sum_tm1 : 0) + NQ;
+        if (coded) over += over / 28;                        // the 6-bit codes round up, by half a step of 7 % on average
+        if (lane == 0) mine[s] = make_int2(ci, base + over);
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(ticket, 1) == (int)gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;                                     // the query's last block goes on
+    __threadfence();
+    int kept = m;
+    if (!few) {
+        for (int i = threadIdx.x; i < BINS; i += SEL_THREADS) hist[i] = 0;
+        __syncthreads();
+        for (int i = threadIdx.x; i < m; i += SEL_THREADS) atomicAdd(&hist[min(__ldcg(&mine[i].x) >> 3, BINS - 1)], 1);
+        __syncthreads();
+        int want = (int)(((int64_t)m * n_prune + n / 2) / n);
+        if (want < 1) want = 1;
+        const int hi_bin = BINS - 1 - 2 * (int)threadIdx.x;
+        const int h_hi = hist[hi_bin], h_lo = hist[hi_bin - 1];
+        int total;
+        const int before = sel_block_scan(h_hi + h_lo, &total, warp_part);
+        if (before < want && want <= before + h_hi + h_lo) s_bin = want <= before + h_hi ? hi_bin : hi_bin - 1;
+        __syncthreads();
+        int pass = 0;
+        for (int i = threadIdx.x; i < m; i += SEL_THREADS) pass += __ldcg(&mine[i].y) >= s_bin << 3 ? 1 : 0;
+        sel_block_scan(pass, &kept, warp_part);
+    }
+    if (threadIdx.x == 0) atomicAdd(&vote[0], kept);
+}
+
 // ------------------------------------------------------------------------------------------------ excess table ----
 // Smallest code whose level is >= e.
 __device__ __forceinline__ int filter_encode(const uint8_t *enc, int e)
@@ -223,7 +355,7 @@ __device__ __forceinline__ int filter_row_excess(const uint4 *row, const uint2 *
 template <int WORDS, int CODEC>
 __global__ void __launch_bounds__(256)
 filter_excess_kernel(const uint8_t *__restrict__ table8, int64_t K, const int32_t *__restrict__ theta,
-                     uint8_t *__restrict__ out, size_t pitch)
+                     uint8_t *__restrict__ out, size_t pitch, FirstCut cut)
 {
     pdl_entry();
     __shared__ uint2 tm1[WORDS];
@@ -231,6 +363,7 @@ filter_excess_kernel(const uint8_t *__restrict__ table8, int64_t K, const int32_
     __shared__ uint8_t enc[512];
     const int b = blockIdx.y;
     const int32_t *th = theta + (int64_t)b * 4 * WORDS;
+    if (!cut.on()) return;
     if (threadIdx.x < WORDS) {
         const int32_t *t = th + 4 * threadIdx.x;
         tm1[threadIdx.x] = make_uint2((uint32_t)(t[0] - 1) | (uint32_t)(t[2] - 1) << 16,
@@ -345,7 +478,7 @@ __global__ void __launch_bounds__(SCAN_THREADS_F, 1)
 filter_scan_kernel(const uint8_t *__restrict__ tab, size_t pitch, const int32_t *__restrict__ theta, int nq, int us,
                    const int32_t *__restrict__ cand, const int64_t *__restrict__ doc_off,
                    const int32_t *__restrict__ n_cand, int64_t maxc, const int32_t *__restrict__ cids, int64_t T,
-                   int32_t *__restrict__ hi0, int32_t *__restrict__ hist)
+                   int32_t *__restrict__ hi0, int32_t *__restrict__ hist, FirstCut cut)
 {
     pdl_entry();
     extern __shared__ uint4 s_tab[];
@@ -356,10 +489,11 @@ filter_scan_kernel(const uint8_t *__restrict__ tab, size_t pitch, const int32_t 
     __shared__ uint16_t s_idx[SCAN_THREADS_F];
     __shared__ int s_theta;
     const int b = blockIdx.y, tid = threadIdx.x;
+    const bool on = cut.on();
     const int n = n_cand[b];
     const int per = (n + (int)gridDim.x - 1) / (int)gridDim.x;
     const int j0 = blockIdx.x * per, j1 = j0 + per < n ? j0 + per : n;
-    if (j0 >= n) return;
+    if (!on || j0 >= n) return;
     const int lane = tid & 31, warp = tid >> 5, grp = lane >> 3, sub = lane & 7;
     const int32_t *cb = cand + (int64_t)b * maxc;
     int32_t *out = hi0 + (int64_t)b * maxc;
@@ -509,12 +643,14 @@ filter_seed_kernel(const int32_t *__restrict__ cand, const int32_t *__restrict__
                    const int32_t *__restrict__ hi0, int64_t maxc, const int32_t *__restrict__ theta, int nq, bool wide, int us,
                    const int32_t *__restrict__ hist, int n_prune, int32_t *__restrict__ seed,
                    int2 *__restrict__ seed_rng, int32_t *__restrict__ n_seed, int32_t *__restrict__ seed_thr,
-                   int32_t *__restrict__ seed_slot)
+                   int32_t *__restrict__ seed_slot, FirstCut cut)
 {
     pdl_entry();
     __shared__ int warp_part[32];
     __shared__ int s_bin, s_theta;
+    const bool on = cut.on();
     const int b = blockIdx.y, n = n_cand[b];
+    if (!on) return;                                     // (no seeds: n_seed is 0)
     const int want = (wide ? 2 * n_prune : n_prune + n_prune / 2) + 32;
     if (n <= want) {
         if (blockIdx.x == 0 && threadIdx.x == 0) seed_thr[b] = INT_MAX;
@@ -650,19 +786,22 @@ __device__ __forceinline__ int block_count(const T *__restrict__ v, int j0, int 
 __global__ void __launch_bounds__(SEL_THREADS)
 filter_count_kernel(const int32_t *__restrict__ n_cand, const int32_t *__restrict__ hi0, int64_t maxc,
                     const int32_t *__restrict__ seed_ci, const int32_t *__restrict__ n_seed, int n_prune, int us,
-                    int32_t *__restrict__ tau_out, int32_t *__restrict__ counts)
+                    int32_t *__restrict__ tau_out, int32_t *__restrict__ counts, FirstCut cut)
 {
     pdl_entry();
     __shared__ int hist[2048];
     __shared__ int warp_part[32];
     __shared__ uint32_t s_prefix;
     __shared__ int s_want;
+    const bool on = cut.on();
     const int b = blockIdx.y;
     int32_t tau = INT_MIN + 1;
-    if (n_seed[b] >= n_prune) {
+    const int seeds = n_seed[b];
+    if (!on) return;
+    if (seeds >= n_prune) {
         const int32_t *sb = seed_ci + (int64_t)b * maxc;
         int need_eq;
-        const uint32_t u = radix_select([&](int j) { return sb[j]; }, n_seed[b], n_prune, hist, warp_part, &s_prefix,
+        const uint32_t u = radix_select([&](int j) { return sb[j]; }, seeds, n_prune, hist, warp_part, &s_prefix,
                                         &s_want, &need_eq);
         tau = (int32_t)(u ^ 0x80000000u);
     }
@@ -676,22 +815,34 @@ filter_count_kernel(const int32_t *__restrict__ n_cand, const int32_t *__restric
 }
 
 // Same grid: the kept candidates, ascending, behind those of the slices before, with their token ranges.  A seed's exact CI
-// is known already: its range is (CI, 0), which the later kernels pass through.
+// is known already: its range is (CI, 0), which the later kernels pass through.  Without the cut: all candidates.
 __global__ void __launch_bounds__(SEL_THREADS)
 filter_write_kernel(const int32_t *__restrict__ cand, const int32_t *__restrict__ n_cand,
                     const int64_t *__restrict__ doc_off, const int32_t *__restrict__ hi0, int64_t maxc,
                     const int32_t *__restrict__ seed_thr, const int32_t *__restrict__ seed_slot,
                     const int32_t *__restrict__ seed_ci, const int32_t *__restrict__ tau, int us,
                     const int32_t *__restrict__ counts, int32_t *__restrict__ kept, int2 *__restrict__ kept_rng,
-                    int32_t *__restrict__ n_kept)
+                    int32_t *__restrict__ n_kept, FirstCut cut)
 {
     pdl_entry();
     __shared__ int warp_part[32];
     const int b = blockIdx.y;
     const int64_t row = (int64_t)b * maxc;
-    const int32_t thr = seed_thr[b];
+    const bool on = cut.on();
+    const int n = n_cand[b];
     int j0, j1;
-    slice_of(n_cand[b], &j0, &j1);
+    slice_of(n, &j0, &j1);
+    if (!on) {
+#pragma unroll 4
+        for (int j = j0 + threadIdx.x; j < j1; j += SEL_THREADS) {
+            const int32_t d = cand[row + j];
+            kept[row + j] = d;
+            kept_rng[row + j] = doc_range(doc_off, d);
+        }
+        if (blockIdx.x == 0 && threadIdx.x == 0) n_kept[b] = n;
+        return;
+    }
+    const int32_t thr = seed_thr[b];
     const int run = block_compact(hi0 + row, j0, j1, units_up(tau[b], us), slices_before(counts + (int64_t)b * KEEP_SPLIT),
                                   warp_part, [&](int j, int32_t v, int pos) {
         const int32_t d = cand[row + j];
@@ -701,33 +852,56 @@ filter_write_kernel(const int32_t *__restrict__ cand, const int32_t *__restrict_
     if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) n_kept[b] = run;
 }
 
-// grid (split, B): contenders = kept candidates whose 8-bit upper bound reaches tau, with their ranges, ascending.  With
-// several slices the count kernel runs first.
+// What an upper bound has to reach: tau of the seeds, or without the cut the n_prune-th largest 8-bit lower bound.
+__device__ __forceinline__ int32_t contend_threshold(const int32_t *lo, int n, int n_prune, int nq, int32_t tau, bool cut,
+                                                     int *hist, int *warp_part, int *s_bin)
+{
+    if (cut) return tau;
+    return n > n_prune ? contender_threshold(lo, n, n_prune, nq, hist, warp_part, s_bin) : INT_MIN + 1;
+}
+
+// grid (split, B): contenders = kept candidates whose 8-bit upper bound reaches the threshold, with their ranges, ascending.
+// With several slices the count kernel runs first and leaves the threshold in tau.
 __global__ void __launch_bounds__(SEL_THREADS)
-filter_contend_count_kernel(const int32_t *__restrict__ n_kept, const int32_t *__restrict__ hi, int64_t maxc,
-                            const int32_t *__restrict__ tau, int32_t *__restrict__ counts)
+filter_contend_count_kernel(const int32_t *__restrict__ n_kept, const int32_t *__restrict__ lo, const int32_t *__restrict__ hi,
+                            int64_t maxc, int n_prune, int nq, const int32_t *tau_in, int32_t *tau_out,
+                            int32_t *__restrict__ counts, FirstCut cut)
 {
     pdl_entry();
+    __shared__ int hist[CONT_BINS];
     __shared__ int warp_part[32];
+    __shared__ int s_bin;
     const int b = blockIdx.y;
+    const int64_t row = (int64_t)b * maxc;
+    const bool on = cut.on();
+    const int n = n_kept[b];
+    const int32_t thr = contend_threshold(lo + row, n, n_prune, nq, tau_in[b], on, hist, warp_part, &s_bin);
     int j0, j1;
-    slice_of(n_kept[b], &j0, &j1);
-    const int total = block_count<int32_t>(hi + (int64_t)b * maxc, j0, j1, tau[b], warp_part);
-    if (threadIdx.x == 0) counts[(int64_t)b * KEEP_SPLIT + blockIdx.x] = total;
+    slice_of(n, &j0, &j1);
+    const int total = block_count<int32_t>(hi + row, j0, j1, thr, warp_part);
+    if (threadIdx.x == 0) {
+        counts[(int64_t)b * KEEP_SPLIT + blockIdx.x] = total;
+        if (blockIdx.x == 0 && !on) tau_out[b] = thr;
+    }
 }
 __global__ void __launch_bounds__(SEL_THREADS)
 filter_contend_kernel(const int32_t *__restrict__ kept, const int2 *__restrict__ kept_rng, const int32_t *__restrict__ n_kept,
-                      const int32_t *__restrict__ hi, int64_t maxc, const int32_t *__restrict__ tau,
-                      const int32_t *__restrict__ counts, int32_t *__restrict__ cont, int2 *__restrict__ cont_rng,
-                      int32_t *__restrict__ n_cont)
+                      const int32_t *__restrict__ lo, const int32_t *__restrict__ hi, int64_t maxc, int n_prune, int nq,
+                      const int32_t *__restrict__ tau, const int32_t *__restrict__ counts, int32_t *__restrict__ cont,
+                      int2 *__restrict__ cont_rng, int32_t *__restrict__ n_cont, FirstCut cut)
 {
     pdl_entry();
+    __shared__ int hist[CONT_BINS];
     __shared__ int warp_part[32];
+    __shared__ int s_bin;
     const int b = blockIdx.y;
     const int64_t row = (int64_t)b * maxc;
+    const bool known = cut.on() || gridDim.x > 1;       // (the threshold is in tau)
+    const int n = n_kept[b];
+    const int32_t thr = contend_threshold(lo + row, n, n_prune, nq, tau[b], known, hist, warp_part, &s_bin);
     int j0, j1;
-    slice_of(n_kept[b], &j0, &j1);
-    const int run = block_compact(hi + row, j0, j1, tau[b], slices_before(counts + (int64_t)b * KEEP_SPLIT), warp_part,
+    slice_of(n, &j0, &j1);
+    const int run = block_compact(hi + row, j0, j1, thr, slices_before(counts + (int64_t)b * KEEP_SPLIT), warp_part,
                                   [&](int j, int32_t, int pos) {
         cont[row + pos] = kept[row + j];
         cont_rng[row + pos] = kept_rng[row + j];
@@ -748,8 +922,10 @@ int launch_filter_scan(const Index &ix, const Params &p, const Layout &L, const 
                        int2 *seed_rng, char *ws, cudaStream_t st)
 {
     int32_t *theta = (int32_t *)(ws + L.flt_theta), *hist = (int32_t *)(ws + L.flt_hist);
-    int32_t *n_seed = (int32_t *)(ws + L.n_seed);
+    int32_t *n_seed = (int32_t *)(ws + L.n_seed), *vote = (int32_t *)(ws + L.flt_vote);
+    const FirstCut cut = first_cut(p, L, ws);
     uint8_t *tab = (uint8_t *)(ws + L.flt_tab);
+    const bool ready = coarse_supported(p.nq);           // stage 1 has written the 8-bit table
     const int codec = filter_codec(ix.K);
     const size_t pitch = filter_table_pitch(ix);
     const int step = (int)(ix.K / FILTER_SAMPLE > 1 ? ix.K / FILTER_SAMPLE : 1);
@@ -765,20 +941,28 @@ int launch_filter_scan(const Index &ix, const Params &p, const Layout &L, const 
     int32_t *parts_hist = (int32_t *)(ws + L.flt_parts), *done = parts_hist + (size_t)p.B * groups * 256 * 32;
     if (parts > 1)
         CHIMERA_CUDA(cudaMemsetAsync(parts_hist, 0, filter_parts_bytes(ix, p), st));
-    launch(filter_theta_kernel, dim3(groups, (unsigned)p.B, (unsigned)parts), SEL_THREADS, 0, st, table, ix.K, p.nq, m, step, rank, theta, hist, n_seed, parts_hist, done);
+    launch(filter_theta_kernel, dim3(groups, (unsigned)p.B, (unsigned)parts), SEL_THREADS, 0, st, table, ix.K, p.nq, m, step, rank, theta, hist, n_seed, parts_hist, done,
+           ready ? vote : nullptr);
     CHIMERA_CUDA(cudaGetLastError());
+    if (ready) {
+        const int jq = judge_queries(p);
+        const dim3 grid((unsigned)(judge_samples(p) / 32), (unsigned)jq);
+        launch(p.nq == 32 ? filter_judge_kernel<32> : filter_judge_kernel<64>, grid, SEL_THREADS, 0, st, table8, ix.K, theta, p.B,
+               cand, n_cand, p.maxc, ix.doc_off, ix.cids, p.n_prune, codec == 6, (int2 *)(ws + L.flt_smp), vote);
+        CHIMERA_CUDA(cudaGetLastError());
+        count_launch(SLOT_CI);
+    }
 
-    const bool ready = coarse_supported(p.nq);           // stage 1 has written the 8-bit table
     const int us = filter_unit(ix, p, ready);
     int64_t gx = (8LL * ix.sm_count + p.B - 1) / p.B;
     if (ready) {
         const int64_t want = ((codec == 16 ? ix.K : (ix.K + 4) / 5) + 255) / 256;
         if (gx > want) gx = want;
         const dim3 grid((unsigned)gx, (unsigned)p.B);
-        if (p.nq == 32 && codec == 16) launch(filter_excess_kernel<8, 16>, grid, 256, 0, st, table8, ix.K, theta, tab, pitch);
-        else if (p.nq == 32) launch(filter_excess_kernel<8, 6>, grid, 256, 0, st, table8, ix.K, theta, tab, pitch);
-        else if (codec == 16) launch(filter_excess_kernel<16, 16>, grid, 256, 0, st, table8, ix.K, theta, tab, pitch);
-        else launch(filter_excess_kernel<16, 6>, grid, 256, 0, st, table8, ix.K, theta, tab, pitch);
+        if (p.nq == 32 && codec == 16) launch(filter_excess_kernel<8, 16>, grid, 256, 0, st, table8, ix.K, theta, tab, pitch, cut);
+        else if (p.nq == 32) launch(filter_excess_kernel<8, 6>, grid, 256, 0, st, table8, ix.K, theta, tab, pitch, cut);
+        else if (codec == 16) launch(filter_excess_kernel<16, 16>, grid, 256, 0, st, table8, ix.K, theta, tab, pitch, cut);
+        else launch(filter_excess_kernel<16, 6>, grid, 256, 0, st, table8, ix.K, theta, tab, pitch, cut);
     } else {
         const int64_t want = (ix.K + 39) / 40;
         if (gx > want) gx = want;
@@ -803,15 +987,15 @@ int launch_filter_scan(const Index &ix, const Params &p, const Layout &L, const 
     if (codec == 16) {
         CHIMERA_CUDA(cudaFuncSetAttribute(filter_scan_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pitch));
         launch(filter_scan_kernel<16>, grid, SCAN_THREADS_F, pitch, st, tab, pitch, theta, p.nq, us, cand, ix.doc_off, n_cand, p.maxc,
-                                                                    ix.cids, ix.T, hi0, hist);
+                                                                    ix.cids, ix.T, hi0, hist, cut);
     } else {
         CHIMERA_CUDA(cudaFuncSetAttribute(filter_scan_kernel<6>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pitch));
         launch(filter_scan_kernel<6>, grid, SCAN_THREADS_F, pitch, st, tab, pitch, theta, p.nq, us, cand, ix.doc_off, n_cand, p.maxc,
-                                                                   ix.cids, ix.T, hi0, hist);
+                                                                   ix.cids, ix.T, hi0, hist, cut);
     }
     CHIMERA_CUDA(cudaGetLastError());
     launch(filter_seed_kernel, dim3((unsigned)filter_split(ix, p), (unsigned)p.B), SEL_THREADS, 0, st, cand, n_cand, ix.doc_off, hi0, p.maxc, theta, p.nq, ready, us, hist, p.n_prune, seed, seed_rng, n_seed,
-        (int32_t *)(ws + L.flt_thr), (int32_t *)(ws + L.flt_slot));
+        (int32_t *)(ws + L.flt_thr), (int32_t *)(ws + L.flt_slot), cut);
     CHIMERA_CUDA(cudaGetLastError());
     count_launch(SLOT_CI, 4);
     return CHIMERA_OK;
@@ -825,33 +1009,34 @@ int launch_filter_keep(const Index &ix, const Params &p, const Layout &L, const 
     int32_t *counts = (int32_t *)(ws + L.flt_counts);
     const int us = filter_unit(ix, p, coarse_supported(p.nq));
     int32_t *tau = (int32_t *)(ws + L.flt_tau);
+    const FirstCut cut = first_cut(p, L, ws);
     const int32_t *thr = (const int32_t *)(ws + L.flt_thr), *slot = (const int32_t *)(ws + L.flt_slot);
     const dim3 grid((unsigned)filter_split(ix, p), (unsigned)p.B);
-    launch(filter_count_kernel, grid, SEL_THREADS, 0, st, n_cand, hi0, p.maxc, seed_ci, n_seed, p.n_prune, us, tau, counts);
+    launch(filter_count_kernel, grid, SEL_THREADS, 0, st, n_cand, hi0, p.maxc, seed_ci, n_seed, p.n_prune, us, tau, counts, cut);
     CHIMERA_CUDA(cudaGetLastError());
     launch(filter_write_kernel, grid, SEL_THREADS, 0, st, cand, n_cand, ix.doc_off, hi0, p.maxc, thr, slot, seed_ci, tau, us,
-                                                      counts, kept, kept_rng, n_kept);
+                                                      counts, kept, kept_rng, n_kept, cut);
     CHIMERA_CUDA(cudaGetLastError());
     count_launch(SLOT_SELECT, 2);
     return CHIMERA_OK;
 }
 
 int launch_filter_contenders(const Index &ix, const Params &p, const Layout &L, const int32_t *kept, const int2 *kept_rng,
-                             const int32_t *n_kept, const int32_t *hi, int32_t *cont, int2 *cont_rng, int32_t *n_cont,
-                             char *ws, cudaStream_t st)
+                             const int32_t *n_kept, const int32_t *lo, const int32_t *hi, int32_t *cont, int2 *cont_rng,
+                             int32_t *n_cont, char *ws, cudaStream_t st)
 {
-    int32_t *counts = (int32_t *)(ws + L.flt_counts);
-    const int32_t *tau = (const int32_t *)(ws + L.flt_tau);
+    int32_t *counts = (int32_t *)(ws + L.flt_counts), *tau = (int32_t *)(ws + L.flt_tau);
+    const FirstCut cut = first_cut(p, L, ws);
     // one block per query keeps up in a large batch; a single query's list is spread
     const int split = 4 * p.B <= ix.sm_count ? filter_split(ix, p) : 1;
     const dim3 grid((unsigned)split, (unsigned)p.B);
     if (split > 1) {
-        launch(filter_contend_count_kernel, grid, SEL_THREADS, 0, st, n_kept, hi, p.maxc, tau, counts);
+        launch(filter_contend_count_kernel, grid, SEL_THREADS, 0, st, n_kept, lo, hi, p.maxc, p.n_prune, p.nq, tau, tau, counts, cut);
         CHIMERA_CUDA(cudaGetLastError());
         count_launch(SLOT_SELECT);
     }
-    launch(filter_contend_kernel, grid, SEL_THREADS, 0, st, kept, kept_rng, n_kept, hi, p.maxc, tau, counts, cont, cont_rng,
-                                                        n_cont);
+    launch(filter_contend_kernel, grid, SEL_THREADS, 0, st, kept, kept_rng, n_kept, lo, hi, p.maxc, p.n_prune, p.nq, tau, counts,
+           cont, cont_rng, n_cont, cut);
     CHIMERA_CUDA(cudaGetLastError());
     count_launch(SLOT_SELECT);
     return CHIMERA_OK;

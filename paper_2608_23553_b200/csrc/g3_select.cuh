@@ -36,6 +36,50 @@ __device__ __forceinline__ int sel_block_scan(int v, int *total, int *warp_part 
     return before + incl - v;
 }
 
+// tau of the contender step: the smallest lower bound in the histogram bin that holds the n_prune-th largest of lb[0..n)
+// (n > n_prune), so at most that one.  Whole block; hist: CONT_BINS entries, of any content.  The lower bounds are
+// lo = 2^16 sum - zeros (2^24 + 2^16) with sum = the sum of nq 8-bit maxima, so coarse_key(lo) is a key of at most 14 bits and
+// 2^16 key <= lo: one histogram sweep (two neighbouring keys share a bin for q_len 64) finds tau without radix passes.
+__device__ __forceinline__ int contender_bin_shift(int nq) { return 255 * nq < CONT_BINS ? 0 : 1; }
+__device__ __forceinline__ int32_t contender_threshold(const int32_t *__restrict__ lb, int n, int n_prune, int nq, int *hist,
+                                                       int *warp_part, int *s_bin)
+{
+    const int bin_shift = contender_bin_shift(nq);
+    for (int i = threadIdx.x; i < CONT_BINS; i += SEL_THREADS) hist[i] = 0;
+    __syncthreads();
+    for (int base = 0; base < n; base += 16 * SEL_THREADS) {
+        int32_t v[16];
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+            const int j = base + e * SEL_THREADS + threadIdx.x;
+            v[e] = j < n ? lb[j] : 0;
+        }
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+            const int j = base + e * SEL_THREADS + threadIdx.x;
+            if (j < n) atomicAdd(&hist[coarse_key(v[e]) >> bin_shift], 1);
+        }
+    }
+    __syncthreads();
+    // descending bins, CONT_BINS / SEL_THREADS consecutive bins per thread
+    constexpr int PER = CONT_BINS / SEL_THREADS;
+    const int first_bin = CONT_BINS - 1 - PER * (int)threadIdx.x;  // this thread owns first_bin, first_bin - 1, ...
+    int h[PER], mine = 0;
+#pragma unroll
+    for (int e = 0; e < PER; ++e) { h[e] = hist[first_bin - e]; mine += h[e]; }
+    int total;
+    int before = sel_block_scan(mine, &total, warp_part);
+    if (before < n_prune && n_prune <= before + mine) {
+#pragma unroll
+        for (int e = 0; e < PER; ++e) {
+            if (before < n_prune && n_prune <= before + h[e]) *s_bin = first_bin - e;
+            before += h[e];
+        }
+    }
+    __syncthreads();
+    return (*s_bin << bin_shift) << 16;
+}
+
 // Radix select (11 + 11 + 10 bits, most significant first) of the `want`-th largest value of sb[0..n) in the order of
 // u = value ^ 0x80000000.  Needs n >= want >= 1.  Returns that value's u; *need_eq = how many entries equal to it
 // belong to the top `want` (the rest of the top `want` are strictly greater).  Whole block, uniform.

@@ -11,12 +11,6 @@ from parity import check_query, taps_to_numpy
 pytestmark = pytest.mark.gpu
 
 
-def _cut_ran():
-    """Whether the searches since the last call ran the cut: it adds five kernels to the step."""
-    from paper_2608_23553_b200 import binding
-    return binding.profile_read()[1]["centroid_interaction"] >= 6
-
-
 # cut: whether the call runs it (the last four rows have too many centroids, or too long a pruning list, for what their
 # candidates hold)
 @pytest.mark.parametrize("cut,D,nbits,nq,K,N,len_lo,len_hi,B,nprobe,n_prune,shift,copies", [
@@ -50,10 +44,11 @@ def test_filtered_searches_match_the_oracle(cut, D, nbits, nq, K, N, len_lo, len
     q = (q / np.linalg.norm(q, axis=2, keepdims=True)).astype(np.float32)
     k = min(n_prune, 25)
     taps = gix.alloc_taps(B, nq, nprobe, n_prune, table=False)
-    _cut_ran()
     ids, sc = gix.search(torch.from_numpy(q).cuda(), nprobe, n_prune, k, taps=taps)
-    assert gix.status() == 0 and _cut_ran() == bool(cut)
+    assert gix.status() == 0
     tn = taps_to_numpy(taps)
+    kept = np.array(gix.kept(B, nq, nprobe, n_prune, k))
+    assert (kept.sum() < 0.7 * tn["n_cand"].sum() and (kept <= tn["n_cand"]).all()) if cut else (kept == -1).all()
     ids, sc = ids.cpu().numpy(), sc.cpu().numpy()
     for b in (0, B - 1):
         res = oracle.pipeline(q[b], oix, nprobe, n_prune, k)
@@ -78,11 +73,47 @@ def test_queries_with_few_candidates_in_a_batch_that_is_cut(nq):
     c[0], c[-1] = np.arange(nq), 32 + np.arange(nq)
     q = cent[c].copy()
     taps = gix.alloc_taps(B, nq, 1, n_prune, table=False)
-    _cut_ran()
     ids, sc = gix.search(torch.from_numpy(q).cuda(), 1, n_prune, k, taps=taps)
-    assert gix.status() == 0 and _cut_ran()
+    assert gix.status() == 0
     tn = taps_to_numpy(taps)
+    assert sum(gix.kept(B, nq, 1, n_prune, k)) < 0.7 * tn["n_cand"].sum()
     assert n_prune < tn["n_cand"][0] < 1.5 * n_prune and 0 < tn["n_cand"][-1] < n_prune and tn["n_cand"][1] > 1_000
     for b in (0, 1, B - 1):
         res = oracle.pipeline(q[b], oix, 1, n_prune, k)
+        check_query(tn, b, res, ids[b].cpu().numpy(), sc[b].cpu().numpy(), k, n_prune, table=False)
+
+
+@pytest.mark.parametrize("nq,K,N,B,nprobe", [
+    (32, 2_000, 20_000, 260, 2),       # 8-bit rows of a query in shared memory
+    (32, 8_000, 20_000, 260, 8),       # ... from L2
+    (64, 1_000, 20_000, 100, 1),
+    (64, 3_000, 20_000, 200, 2),
+    (32, 3_000, 40_000, 31, 8),        # few queries: their contenders over several blocks
+    (32, 8_000, 40_000, 37, 16),
+    (32, 120_003, 250_000, 100, 60),   # 6-bit codes
+])
+def test_documents_that_repeat_their_centroids_are_not_cut(nq, K, N, B, nprobe):
+    """Ten centroids for about forty tokens: nearly all candidates pass the bound, and the call has to notice."""
+    import paper_2608_23553_b200 as pkg
+    D, n_prune, k = 64, 100, 20
+    cent, cids, codes, doclens = random_corpus(K + B, N, K, D, 2, len_lo=30, len_hi=50)
+    rng = np.random.default_rng(K)
+    own = rng.integers(0, K, size=(N, 10)).astype(np.int32)
+    doc = np.repeat(np.arange(N), doclens)
+    cids = own[doc, rng.integers(0, 10, size=len(cids))]
+    oix = oracle.make_index(cent, cids, codes, doclens, 2)
+    gix = pkg.Index(*(torch.from_numpy(a).cuda() for a in (cent, cids, codes, doclens)), 2)
+    topic = own[rng.integers(0, N, size=(B, 1)), rng.integers(0, 10, size=(B, nq))]       # half of a query's tokens: one document's
+    q = cent[np.where(rng.random((B, nq)) < 0.5, topic, rng.integers(0, K, size=(B, nq)))]
+    q = q + 0.3 / np.sqrt(D) * rng.standard_normal(q.shape).astype(np.float32)
+    q = (q / np.linalg.norm(q, axis=2, keepdims=True)).astype(np.float32)
+    taps = gix.alloc_taps(B, nq, nprobe, n_prune, table=False)
+    ids, sc = gix.search(torch.from_numpy(q).cuda(), nprobe, n_prune, k, taps=taps)
+    assert gix.status() == 0
+    tn = taps_to_numpy(taps)
+    assert gix.kept(B, nq, nprobe, n_prune, k) == tn["n_cand"].tolist()
+    n_cont = taps.n_contenders.cpu().numpy()
+    assert (n_cont < 0.5 * tn["n_cand"]).all()           # the 8-bit bounds narrow them down
+    for b in (0, B - 1):
+        res = oracle.pipeline(q[b], oix, nprobe, n_prune, k)
         check_query(tn, b, res, ids[b].cpu().numpy(), sc[b].cpu().numpy(), k, n_prune, table=False)
