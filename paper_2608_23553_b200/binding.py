@@ -186,6 +186,12 @@ class Index:
             _check(lib().chimera_index_enable_partial(self._h, _stream()))
         self._ws = None
 
+    def list_copies(self) -> int:
+        """Which copies in list order the index holds: 1 = the codes, 2 = the 1-bit codes (chimera_index_list_copies)."""
+        out = ctypes.c_int32()
+        _check(lib().chimera_index_list_copies(self._h, ctypes.byref(out)))
+        return out.value
+
     def attach_rabitq(self, rotation: torch.Tensor, bits: torch.Tensor, inv_dot: torch.Tensor):
         """Attach RaBitQ 1-bit codes (kept referenced) for search(..., rabitq=True)."""
         rq = (rotation.contiguous().to(torch.float32), bits.contiguous().to(torch.uint8),

@@ -544,11 +544,18 @@ int chimera_index_enable_partial(chimera_index *index, void *stream)
 {
     Index *ix = reinterpret_cast<Index *>(index);
     if (!ix) return fail(CHIMERA_INVALID_ARG, "index is NULL");
-    int rc = build_token_lists(*ix, (cudaStream_t)stream);
-    if (rc || ix->list_codes) return rc;
+    if (ix->list_codes) return CHIMERA_OK;
     ListOrderCopy codes = {ix->codes, ix->CB / 4, nullptr};
-    if ((rc = copy_in_list_order(*ix, &codes, 1, (cudaStream_t)stream))) return rc;
+    const int rc = build_lists_and_copies(*ix, &codes, 1, ix->code_mem, (cudaStream_t)stream);
     ix->list_codes = (uint8_t *)codes.dst;
+    return rc;
+}
+
+int chimera_index_list_copies(const chimera_index *index, int32_t *copies)
+{
+    const Index *ix = reinterpret_cast<const Index *>(index);
+    if (!ix || !copies) return fail(CHIMERA_INVALID_ARG, "NULL argument");
+    *copies = (ix->list_codes ? 1 : 0) | (ix->list_bits ? 2 : 0);
     return CHIMERA_OK;
 }
 
@@ -571,20 +578,17 @@ int chimera_index_attach_rabitq(chimera_index *index, const float *rotation, con
     Index *ix = reinterpret_cast<Index *>(index);
     if (!ix || !rotation || !bits || !inv_dot) return fail(CHIMERA_INVALID_ARG, "NULL argument");
     if (((uintptr_t)bits & 15) || ((uintptr_t)inv_dot & 3)) return fail(CHIMERA_INVALID_ARG, "bits must be 16-byte aligned");
-    int rc = build_token_lists(*ix, (cudaStream_t)stream);
-    if (rc) return rc;
-    // Codes attached before, if any, are replaced: their copies go first, to make room.  Whatever fails below leaves the index
-    // with the codes and the rotation that it had (and no copies of them).
-    cudaFree(ix->list_bits);
+    // Codes attached before, if any, are replaced, their copies in place.  Whatever fails below leaves the index with the codes
+    // and the rotation that it had (and no copies of them).
+    const bool copied = ix->list_bits != nullptr;
     ix->list_bits = nullptr;
     ix->list_inv = nullptr;
+    if (copied) CHIMERA_CUDA(cudaDeviceSynchronize());       // (searches that still read them, on any stream)
     ListOrderCopy copies[2] = {{bits, ix->D / 32, nullptr}, {inv_dot, 1, nullptr}};
-    if ((rc = copy_in_list_order(*ix, copies, 2, (cudaStream_t)stream))) return rc;
+    int rc = build_lists_and_copies(*ix, copies, 2, ix->rq_mem, (cudaStream_t)stream);
+    if (rc) return rc;
     float *rot_t = nullptr;
-    if ((rc = transpose_rotation(*ix, rotation, &rot_t, (cudaStream_t)stream))) {
-        cudaFree(copies[0].dst);
-        return rc;
-    }
+    if ((rc = transpose_rotation(*ix, rotation, &rot_t, (cudaStream_t)stream))) return rc;
     cudaFree(ix->rot_t);
     ix->rot_t = rot_t;
     ix->rq_bits = bits;
@@ -749,10 +753,8 @@ int chimera_destroy_index(chimera_index *index)
     cudaFree(ix->xc);
     cudaFree(ix->rot_t);
     cudaFree(ix->tok_off);
-    cudaFree(ix->tok_id);
-    cudaFree(ix->tok_doc);
-    cudaFree(ix->list_codes);
-    cudaFree(ix->list_bits);
+    if (ix->code_mem.own) cudaFree(ix->code_mem.at);
+    if (ix->rq_mem.own) cudaFree(ix->rq_mem.at);
     cudaFree(ix->doc_off);
     cudaFree(ix->cdig);
     cudaFree(ix->ivf_off);

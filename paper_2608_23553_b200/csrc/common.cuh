@@ -11,6 +11,12 @@ namespace chimera {
 // ---------------------------------------------------------------------------------------------------------------
 // Index: everything resident on the device between searches.
 // ---------------------------------------------------------------------------------------------------------------
+// Memory of copies in list order: an allocation of their own, or room behind the token lists.  Kept once it is there (the
+// sizes of an index do not change).
+struct ListMemory {
+    void *at = nullptr;
+    bool own = false;
+};
 struct Index {
     int device = 0;
     int sm_count = 0;
@@ -26,13 +32,14 @@ struct Index {
     int64_t ivf_len = 0;
     int32_t max_doclen = 0;
     // token-level posting lists (only after chimera_index_enable_partial): per centroid its tokens and their documents
-    int64_t *tok_off = nullptr;       // [K+1]      owned
-    int32_t *tok_id = nullptr;        // [T]        owned: token ids per centroid, unordered
-    int32_t *tok_doc = nullptr;       // [T]        owned: document of each listed token
+    int64_t *tok_off = nullptr;       // [K+1]      owned, with the next two in the same allocation
+    int32_t *tok_id = nullptr;        // [T]        token ids per centroid, unordered
+    int32_t *tok_doc = nullptr;       // [T]        document of each listed token
     int64_t max_tok_list = 0;         // longest token list
-    uint8_t *list_codes = nullptr;    // [T, CB]    owned, optional: the codes in list order (see copy_in_list_order)
-    uint8_t *list_bits = nullptr;     // [T, D/8]   owned, optional: the RaBitQ codes in list order
-    float *list_inv = nullptr;        // [T]        their factors, in the same allocation: both or neither
+    ListMemory code_mem, rq_mem;      // owned: the next one, the two behind it
+    uint8_t *list_codes = nullptr;    // [T, CB]    optional: the codes in list order (see build_lists_and_copies)
+    uint8_t *list_bits = nullptr;     // [T, D/8]   optional: the RaBitQ codes in list order
+    float *list_inv = nullptr;        // [T]        their factors: both or neither
     // RaBitQ 1-bit codes (only after chimera_index_attach_rabitq)
     const uint8_t *rq_bits = nullptr; // [T, D/8]   borrowed: sign bits of the rotated tokens
     const float *rq_inv = nullptr;    // [T]        borrowed: 1 / <o_p, o_p-bar>
@@ -237,18 +244,16 @@ int launch_gather(const Index &ix, const Params &p, const Layout &L, const int32
                   int32_t *cont_scratch, uint32_t *status, cudaStream_t st);
 bool contenders_split(const Index &ix, const Params &p);
 int contender_hist_entries();
-// Token-level posting lists for the partial-score refinement (allocates; index_build.cu).
-int build_token_lists(Index &ix, cudaStream_t st);
-// Copies of `n` arrays ([T][words] 32-bit words each, document-major) in the order of the token lists, so that a list's
-// codes are one contiguous run instead of a scattered sector each.  One allocation (the first copy's address) holds all of
-// them; they are complete when the call returns.  Every dst stays NULL, with CHIMERA_OK, when they would take more than a
-// quarter of the free memory (the kernels then gather through the token ids), and on every error.
+// Token-level posting lists for the refinements, unless they are there, and copies of `n` arrays ([T][words] 32-bit words each,
+// document-major) in their order, so that a list's codes are one contiguous run instead of a scattered sector each
+// (index_build.cu).  The copies are complete when the call returns.  Every dst is NULL, with CHIMERA_OK, when they would take
+// more than a quarter of the free memory (the kernels then gather through the token ids), and on every error.
 struct ListOrderCopy {
     const void *src;
     int words;
     void *dst;
 };
-int copy_in_list_order(const Index &ix, ListOrderCopy *copies, int n, cudaStream_t st);
+int build_lists_and_copies(Index &ix, ListOrderCopy *copies, int n, ListMemory &mem, cudaStream_t st);
 // Candidate refinement with partial scores (Algorithm 2): fprime[b][j] for every candidate.
 int64_t visit_list_nodes(const Index &ix, const Params &p);
 int launch_partial_scores(const Index &ix, const Params &p, const Layout &L, const int8_t *qdig,

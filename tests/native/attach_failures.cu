@@ -40,9 +40,7 @@ int main()
             } else {
                 check(ix.rq_bits == bits[1] && ix.rq_inv == inv[1] && ix.rot_t != nullptr, "not attached", n, again);
             }
-            size_t held = (ix.rot_t != nullptr) + (ix.list_bits != nullptr);
-            if (ix.list_inv && fake_live.count(ix.list_inv)) ++held;            // (an allocation of its own)
-            check(fake_live.size() == held, "memory is lost", n, again);
+            check(fake_live.size() == (size_t)(ix.rot_t != nullptr) + ix.rq_mem.own, "memory is lost", n, again);
             while (!fake_live.empty()) cudaFree(*fake_live.begin());
             if (!injected) {
                 check(rc == 0 && ix.list_bits != nullptr, "no failure, yet no copies", n, again);

@@ -32,6 +32,7 @@ int cudaFree(void *p)
 }
 int cudaMemGetInfo(size_t *avail, size_t *all) { *avail = *all = (size_t)1 << 30; return step(); }
 int cudaStreamSynchronize(void *) { return step(); }
+int cudaDeviceSynchronize(void) { return step(); }
 int cudaLaunchKernel() { return step(); }                // (arguments are left where the caller put them)
 int cudaLaunchKernelExC() { return step(); }
 int cudaGetLastError(void) { const int e = fake_last_error; fake_last_error = 0; return e; }
