@@ -124,7 +124,7 @@ size_t filter_parts_bytes(const Index &ix, const Params &p)
 // ------------------------------------------------------------------------------------------------ thresholds ------
 // grid (ceil(nq / 32), B, parts), lane = query token.  theta[b][i] = the smallest t (in units of 2^16) such that at most
 // `rank` of the m sampled rows (every step-th one) have S >= t 2^16.  With few queries the sample is split over several
-// blocks that add their histograms up in `parts_hist` ([B][groups][256 * 32], zero before and afterwards); the last one to
+// blocks that add their histograms up in `parts_hist` ([B][groups][256 * 32], cleared before); the last one to
 // finish (`done`, likewise) reads the sum.  Also clears what the scan and the seed selection add to, and the judge's words (vote,
 // may be NULL).
 __global__ void __launch_bounds__(SEL_THREADS)
@@ -170,11 +170,7 @@ filter_theta_kernel(const int32_t *__restrict__ table, int64_t K, int nq, int m,
         __syncthreads();
         if (!s_last) return;
         __threadfence();
-        for (int i = threadIdx.x; i < 256 * 32; i += SEL_THREADS) {
-            hist[i] = __ldcg(&ph[i]);
-            ph[i] = 0;
-        }
-        if (threadIdx.x == 0) done[(int64_t)b * gridDim.x + blockIdx.x] = 0;
+        for (int i = threadIdx.x; i < 256 * 32; i += SEL_THREADS) hist[i] = __ldcg(&ph[i]);
         __syncthreads();
     }
     // warp w finds column w's threshold: lane l holds buckets 255 - 8 l ... 248 - 8 l, descending
