@@ -758,16 +758,16 @@ __device__ __forceinline__ int slices_before(const int32_t *counts)
     for (int s = 0; s < (int)blockIdx.x; ++s) run += counts[s];
     return run;
 }
-template <class T>
-__device__ __forceinline__ int block_count(const T *__restrict__ v, int j0, int j1, T thr, int *warp_part)
+// Elements of [j0, j1) with v >= thr (thr > INT_MIN).
+__device__ __forceinline__ int block_count(const int32_t *__restrict__ v, int j0, int j1, int32_t thr, int *warp_part)
 {
     int keep = 0;
     for (int base = j0; base < j1; base += 8 * SEL_THREADS) {
-        T x[8];
+        int32_t x[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
             const int j = base + u * SEL_THREADS + threadIdx.x;
-            x[u] = j < j1 ? v[j] : thr - 1;
+            x[u] = j < j1 ? v[j] : INT_MIN;
         }
 #pragma unroll
         for (int u = 0; u < 8; ++u) keep += x[u] >= thr ? 1 : 0;
@@ -803,7 +803,7 @@ filter_count_kernel(const int32_t *__restrict__ n_cand, const int32_t *__restric
     }
     int j0, j1;
     slice_of(n_cand[b], &j0, &j1);
-    const int total = block_count<int32_t>(hi0 + (int64_t)b * maxc, j0, j1, units_up(tau, us), warp_part);
+    const int total = block_count(hi0 + (int64_t)b * maxc, j0, j1, units_up(tau, us), warp_part);
     if (threadIdx.x == 0) {
         counts[(int64_t)b * KEEP_SPLIT + blockIdx.x] = total;
         if (blockIdx.x == 0) tau_out[b] = tau;
@@ -874,7 +874,7 @@ filter_contend_count_kernel(const int32_t *__restrict__ n_kept, const int32_t *_
     const int32_t thr = contend_threshold(lo + row, n, n_prune, nq, tau_in[b], on, hist, warp_part, &s_bin);
     int j0, j1;
     slice_of(n, &j0, &j1);
-    const int total = block_count<int32_t>(hi + row, j0, j1, thr, warp_part);
+    const int total = block_count(hi + row, j0, j1, thr, warp_part);
     if (threadIdx.x == 0) {
         counts[(int64_t)b * KEEP_SPLIT + blockIdx.x] = total;
         if (blockIdx.x == 0 && !on) tau_out[b] = thr;
