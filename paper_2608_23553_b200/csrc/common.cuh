@@ -127,7 +127,8 @@ struct Layout {
     size_t partial_m;     // int32  [B][maxc][nq]     per (candidate, query token) best retrieved-token score, or the visit
                           //                          lists in its place (g3_visits.cuh)
     int64_t visit_nodes;  // nodes per query of those lists; 0 = the table
-    size_t graph_vis;     // uint32 [B*nq][K/32]      visited centroids of the graph search (only with a centroid graph)
+    size_t graph_vis;     // uint32 [B*nq][K/32]      visited centroids of the graph search (only with a centroid graph, and
+                          //                          too many centroids for a bitmap in shared memory)
     size_t q_rot;         // float  [B, nq, D]        rotated queries (RaBitQ pipeline)
     size_t qdig_rot;      // int8   [3][B*residual_rows(nq)][128]  their digit planes for stage 4
     size_t n_pruned;      // int32  [B]
@@ -325,8 +326,10 @@ int launch_rabitq_scores_umma(const Index &ix, const Params &p, const float *q_r
 // g7_graph.cu
 int build_graph(Index &ix, const float *centroids, int degree, cudaStream_t st);
 size_t graph_scratch_bytes(const Index &ix, int64_t n_tokens);
+size_t graph_workspace_bytes(const Index &ix, int64_t n_tokens);     // of a search that does not want the visited sets
 int check_graph_params(const Index &ix, const GraphSearch &g, int nprobe);
 // visited: graph_scratch_bytes(ix, n_tokens) bytes of scratch, holding the visited sets afterwards if want_visited;
+// graph_workspace_bytes(ix, n_tokens) otherwise;
 // out_scores / out_nvis may be NULL.
 int launch_graph_probes(const Index &ix, const float *queries, int64_t n_tokens, int nprobe, const GraphSearch &g,
                         uint32_t *visited, bool want_visited, int32_t *out_probes, int32_t *out_scores, int32_t *out_nvis,

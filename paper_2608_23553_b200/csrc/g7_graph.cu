@@ -285,6 +285,13 @@ size_t graph_scratch_bytes(const Index &ix, int64_t n_tokens)
     return (size_t)n_tokens * (size_t)((ix.K + 31) / 32) * sizeof(uint32_t);
 }
 
+// The search keeps the visited set in shared memory up to a million centroids.
+static bool visited_in_shared(const Index &ix) { return (ix.K + 31) / 32 * (int64_t)sizeof(uint32_t) <= 128 * 1024; }
+size_t graph_workspace_bytes(const Index &ix, int64_t n_tokens)
+{
+    return visited_in_shared(ix) ? 0 : graph_scratch_bytes(ix, n_tokens);
+}
+
 int check_graph_params(const Index &ix, const GraphSearch &g, int nprobe)
 {
     if (!ix.graph) return fail(CHIMERA_INVALID_ARG, "the centroid graph is not built (chimera_index_build_graph)");
@@ -301,7 +308,7 @@ int launch_graph_probes(const Index &ix, const float *queries, int64_t n_tokens,
 {
     const int64_t vwords = (ix.K + 31) / 32;
     const size_t smem = sizeof(uint32_t) * (size_t)vwords;
-    const bool shared = smem <= 128 * 1024;              // a million centroids
+    const bool shared = visited_in_shared(ix);
     auto kern = shared ? graph_probe_kernel<true> : graph_probe_kernel<false>;
     if (shared) CHIMERA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     else CHIMERA_CUDA(cudaMemsetAsync(visited, 0, graph_scratch_bytes(ix, n_tokens), st));

@@ -51,7 +51,11 @@ def test_graph_search_at_the_largest_shared_bitmap(K):
     cids = rng.integers(0, K, size=200).astype(np.int32)
     codes = rng.integers(0, 256, size=(200, 8)).astype(np.uint8)
     gix = _index(cent, cids, codes, np.full(20, 10, dtype=np.int32))
+    sizes = (2, 8, 4, 10, 5)
+    before = gix.workspace_bytes(*sizes)
     gix.build_graph(3)
+    vis = 0 if K <= 1 << 20 else 2 * 8 * ((K + 31) // 32) * 4     # a search needs room for the visited sets where they are not shared
+    assert vis <= gix.workspace_bytes(*sizes) - before < vis + 256
     q = cent[rng.integers(0, K, size=8)][None] + 0.0
     q[0, -1] = cent[K - 1]
     pr, sc, nvis, bm = gix.graph_probes(torch.from_numpy(q).cuda(), 4, 40, 300, 1 << 30)
