@@ -15,6 +15,8 @@
 //
 // Batches on large corpora keep the visits as lists instead of the table (g3_visits.cuh); few queries per call keep the
 // table, whose update is one atomic and whose sum needs no second kernel.
+#include <math.h>
+
 #include "g3_visits.cuh"
 
 namespace chimera {
@@ -23,15 +25,21 @@ constexpr int PS_THREADS = 128;
 
 // Nodes per query of the visit lists, 0 when the table of maxima is used: no token lists, few queries per call (latency
 // counts), more nodes than their index holds, a table less than four times as large, or candidates with several visits
-// each, whose lists would be walked node by node (a mean of two: long documents under many probes stay with the table).
+// each, whose lists are chains of scattered reads: more than two as independent tokens would have them (long documents under
+// many probes, where the topics of real ones make it many more), or four by the distinct centroids of a document.
+// Whole searches, batch 256 on Mid's sizes, documents that draw 1/4 as many centroids as they have tokens (4.1 visits): lists
+// 2.98, table 2.93 ms, 1-bit codes 2.64 / 2.75; an eighth or less (10 visits): 2.96 / 2.68, 2.60 / 2.32; independent (1.1): 3.21 /
+// 4.27, 2.83 / 4.71; four topics of near centroids under 32 probes (64 queries): 3.37 / 2.52, 3.05 / 2.45.
 int64_t visit_list_nodes(const Index &ix, const Params &p)
 {
     if (!ix.tok_id || ix.max_tok_list <= 0 || 4 * p.B <= ix.sm_count) return 0;
     const int64_t nodes = (int64_t)p.nq * p.P * ix.max_tok_list;
     if (nodes > VISIT_MAX_NODES) return 0;
     if (4 * (nodes * 8 + p.maxc * 4) > (int64_t)p.maxc * p.nq * 4) return 0;
-    const double len = (double)ix.T / (double)ix.N, probed = (double)p.nq * p.P / (double)ix.K;
-    return len * probed <= 1.6 ? nodes : 0;              // (visits per candidate: x / (1 - exp(-x)) = 2 at x = 1.6)
+    const double len = (double)ix.T / (double)ix.N, distinct = (double)ix.ivf_len / (double)ix.N;
+    const double probed = (double)p.nq * p.P / (double)ix.K;
+    if (len * probed > 1.6) return 0;                    // (visits per candidate: x / (1 - exp(-x)) = 2 at x = 1.6)
+    return len * probed <= 4.0 * (1.0 - exp(-distinct * probed)) ? nodes : 0;
 }
 
 // Blocks per query token of the refinement kernels: one per probed list until the batch fills the GPU sixteen times over.
@@ -49,17 +57,43 @@ visit_clear_kernel(int32_t *__restrict__ head, const int32_t *__restrict__ n_can
     const int b = blockIdx.y, n = n_cand[b];
     for (int e = blockIdx.x * 256 + threadIdx.x; e < n; e += gridDim.x * 256) head[(int64_t)b * maxc + e] = 0;
 }
-// grid (blocks, B): fprime[b][j] of every candidate, one thread each.
+// grid (blocks, B): fprime[b][j] of every candidate, one thread each, the first nodes of two candidates in flight.  Long lists
+// take turns at the warp's rows of maxima: 8 for up to 32 query tokens, 4 for 64, 2 for 127 (1 KB a warp, which leaves the
+// scattered reads their L1; with 2 KB no list gains 1 %).
+constexpr int VISIT_ROW_WORDS = 264;                     // 8 x 33, 4 x 65 or 2 x 128
 template <bool FLOAT>
 __global__ void __launch_bounds__(256)
 visit_sum_kernel(const int32_t *__restrict__ head, const unsigned long long *__restrict__ node, int64_t cap,
-                 const int32_t *__restrict__ n_cand, int64_t maxc, int32_t *__restrict__ fprime)
+                 const int32_t *__restrict__ n_cand, int64_t maxc, int nq, int32_t *__restrict__ fprime)
 {
     pdl_entry();
-    const int b = blockIdx.y, n = n_cand[b];
+    __shared__ uint32_t s_rows[8][VISIT_ROW_WORDS];
+    const int b = blockIdx.y, n = n_cand[b], lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int rows = nq <= 32 ? 8 : nq <= 64 ? 4 : 2, pitch = nq <= 32 ? 33 : nq <= 64 ? 65 : 128;
     const unsigned long long *nodes = node + (int64_t)b * cap;
-    for (int j = blockIdx.x * 256 + threadIdx.x; j < n; j += gridDim.x * 256)
-        fprime[(int64_t)b * maxc + j] = visit_sum<FLOAT>(head[(int64_t)b * maxc + j], nodes);
+    const int32_t *hb = head + (int64_t)b * maxc;
+    const int step = gridDim.x * 256;
+    for (int j0 = blockIdx.x * 256 + warp * 32; j0 < n; j0 += 2 * step) {
+        int32_t first[2];
+        unsigned long long n0[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) first[u] = j0 + u * step + lane < n ? hb[j0 + u * step + lane] : 0;
+#pragma unroll
+        for (int u = 0; u < 2; ++u) n0[u] = first[u] != 0 ? nodes[first[u] - 1] : 0ull;
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int j = j0 + u * step + lane;
+            int32_t sum;
+            const bool done = visit_sum<FLOAT>(n0[u], nodes, sum);
+            for (unsigned left = __ballot_sync(0xffffffffu, !done); left;) {
+                const int place = __popc(left & ((1u << lane) - 1));
+                const bool mine = (left >> lane & 1u) && place < rows;
+                if (mine) sum = visit_sum_long<FLOAT>(first[u], nodes, s_rows[warp] + place * pitch, nq);
+                left &= ~__ballot_sync(0xffffffffu, mine);
+            }
+            if (j < n) fprime[(int64_t)b * maxc + j] = sum;
+        }
+    }
 }
 VisitLists visit_lists(const Params &p, const Layout &L, void *mem)
 {
@@ -80,8 +114,8 @@ int launch_visit_sum(const Index &ix, const Params &p, const VisitLists &v, bool
                      int32_t *fprime, cudaStream_t st)
 {
     const dim3 grid((unsigned)((16LL * ix.sm_count + p.B - 1) / p.B), (unsigned)p.B);
-    if (floats) launch(visit_sum_kernel<true>, grid, 256, 0, st, v.head, v.node, v.cap, n_cand, p.maxc, fprime);
-    else launch(visit_sum_kernel<false>, grid, 256, 0, st, v.head, v.node, v.cap, n_cand, p.maxc, fprime);
+    if (floats) launch(visit_sum_kernel<true>, grid, 256, 0, st, v.head, v.node, v.cap, n_cand, p.maxc, p.nq, fprime);
+    else launch(visit_sum_kernel<false>, grid, 256, 0, st, v.head, v.node, v.cap, n_cand, p.maxc, p.nq, fprime);
     CHIMERA_CUDA(cudaGetLastError());
     return CHIMERA_OK;
 }

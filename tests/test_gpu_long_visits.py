@@ -1,5 +1,5 @@
 """Candidates with many visits in a call that keeps visits as lists: documents that repeat a probed centroid, up to the visits
-that the sum holds in registers, one more, and hundreds."""
+that the sum holds in registers, one more, and hundreds; each size of the rows that long lists are summed in."""
 import numpy as np
 import pytest
 import torch
@@ -10,11 +10,12 @@ from helpers import random_corpus
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("mode,nbits", [("partial", 2), ("partial", 1), ("rabitq", 2)])
-def test_candidates_with_many_visits(mode, nbits):
+@pytest.mark.parametrize("mode,nbits,nq", [("partial", 2, 32), ("partial", 1, 51), ("partial", 2, 101), ("rabitq", 2, 32),
+                                           ("rabitq", 2, 64)])
+def test_candidates_with_many_visits(mode, nbits, nq):
     import paper_2608_23553_b200 as pkg
     from synth import CONFIGS, encode_rabitq_1bit, random_rotation
-    D, nq, K, N, nprobe, n_prune, k = 64, 32, 4096, 30_000, 2, 300, 20
+    D, K, N, nprobe, n_prune, k = 64, 4096, 30_000, 2, 300, 20
     cent, cids, codes, doclens = random_corpus(11 + nbits, N, K, D, nbits, len_lo=20, len_hi=40)
     rng = np.random.default_rng(1)
     first = np.concatenate([[0], np.cumsum(doclens)[:-1]])

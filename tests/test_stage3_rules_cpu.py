@@ -1,4 +1,4 @@
-"""When stage 3 runs its first cut: host arithmetic on the sizes, no device."""
+"""When stage 3 runs its first cut and keeps visits as lists: host arithmetic on the sizes, no device."""
 import os
 import subprocess
 
@@ -6,22 +6,33 @@ import pytest
 
 
 @pytest.fixture(scope="module")
-def rule(tmp_path_factory):
+def routes(tmp_path_factory):
     from paper_2608_23553_b200 import build
     build.build()
     native = os.path.join(os.path.dirname(os.path.abspath(__file__)), "native")
     tmp = tmp_path_factory.mktemp("rule")
-    obj, exe = str(tmp / "first_cut_rule.o"), str(tmp / "first_cut_rule")
-    subprocess.check_call([build.NVCC] + build.FLAGS + ["-c", os.path.join(native, "first_cut_rule.cu"), "-o", obj])
-    objs = [os.path.join(build.OBJ, n) for n in ("g3_filter.o", "g3_centroid_interaction.o")]
+    obj, exe = str(tmp / "stage3_rules.o"), str(tmp / "stage3_rules")
+    subprocess.check_call([build.NVCC] + build.FLAGS + ["-c", os.path.join(native, "stage3_rules.cu"), "-o", obj])
+    objs = [os.path.join(build.OBJ, n) for n in ("g3_filter.o", "g3_centroid_interaction.o", "g3_partial.o")]
     subprocess.check_call(["g++", "-no-pie", "-o", exe, obj, os.path.join(native, "fake_cudart.cpp")] + objs +
                           ["-Wl,--unresolved-symbols=ignore-all"])
 
-    def used(K, N, length, B, nq, P, n_prune, distinct=None, max_len=None, max_candidates=0):
-        line = "%d %d %d %d %d %d %d %d %d %d" % (K, N, N * length, N * (distinct or length), max_len or 2 * length, B, nq, P,
-                                                  n_prune, max_candidates)
-        return subprocess.run([exe], input=line, capture_output=True, text=True, check=True).stdout.strip() == "1"
-    return used
+    def routes(K, N, length, B, nq, P, n_prune, distinct=None, max_len=None, max_candidates=0, longest=0):
+        line = "%d %d %d %d %d %d %d %d %d %d %d" % (K, N, N * length, N * (distinct or length), max_len or 2 * length, B, nq,
+                                                     P, n_prune, max_candidates, longest or 2 * N * length // K)
+        out = subprocess.run([exe], input=line, capture_output=True, text=True, check=True).stdout.split()
+        return [x == "1" for x in out]
+    return routes
+
+
+@pytest.fixture(scope="module")
+def rule(routes):
+    return lambda *a, **kw: routes(*a, **kw)[0]
+
+
+@pytest.fixture(scope="module")
+def lists(routes):
+    return lambda *a, **kw: routes(*a, **kw)[1]
 
 
 def test_what_the_candidates_hold_counts_and_not_the_room_for_them(rule):
@@ -51,3 +62,12 @@ def test_other_query_lengths_and_what_the_cut_cannot_hold(rule):
     assert rule(262_144, *args, max_len=32_000) and not rule(262_144, *args, max_len=32_001)
     # token positions of 31 bits
     assert not rule(262_144, 8_800_000, 245, 256, 32, 4, 4_096)
+
+
+def test_visits_are_kept_as_lists_while_candidates_have_few(lists):
+    mid = (65_536, 500_000, 120, 256, 32)
+    assert lists(*mid, 4, 1_024) and lists(*mid, 16, 1_024) and not lists(*mid, 32, 1_024)
+    assert not lists(65_536, 500_000, 120, 16, 32, 4, 1_024)              # few queries
+    # documents that repeat their centroids: as few visits, but of fewer candidates
+    assert lists(*mid, 4, 1_024, distinct=40) and not lists(*mid, 4, 1_024, distinct=12)
+    assert not lists(*mid, 4, 1_024, longest=60_000)                     # as large as the table
