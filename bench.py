@@ -96,17 +96,17 @@ def isolated_int8_mma_tops():
 
 
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of one launch of the dominant kernel, from stored ncu
-# captures on small cases (a full-size launch is too large to capture; the profile named beside each figure gives the
-# command).  The stage-3 bound scan reads each query's 8-bit table once (batch x K x q_len bytes) and otherwise moves
+# captures on small cases (a full-size launch is too large to capture).  The stage-3 bound scan reads each query's 8-bit table once (batch x K x q_len bytes) and otherwise moves
 # a fixed number of bytes per algorithmic byte (centroid ids, ranges, ids, bounds), so a full-size launch is
 # ratio x algorithmic bytes + batch x K x q_len.
 NCU_CI_DRAM_PER_ALGORITHMIC_BYTE = {
-    "large": (1.243, "profiles/ncu_ci_coarse_large_slice.md (Large recipe, 1M documents, batch 16)"),
-    None: (0.939, "profiles/ncu_ci_coarse_mid.md (Mid corpus, batch 8)"),
+    "large": (1.243, "an ncu capture (Large recipe, 1M documents, batch 16)"),
+    None: (0.939, "an ncu capture (Mid corpus, batch 8)"),
 }
 # ... and the same of the launches that bound and seed stage 3 when its first cut runs.
-NCU_CUT_DRAM_PER_ALGORITHMIC_BYTE = (0.874, "profiles/ncu_first_cut_mid.md (Mid corpus, batch 64)")
-NCU_PARTIAL_DRAM_PER_QUERY = (1527e6 / 64.0, "profiles/ncu_partial_score_mid.md (Mid corpus, batch 64; bytes per query)")
+NCU_CUT_DRAM_PER_ALGORITHMIC_BYTE = (0.883, "an ncu capture (Mid corpus, batch 64)")
+NCU_PARTIAL_DRAM_PER_QUERY = (463.5e6 / 64.0, "an ncu capture of the visits and their sums (Mid corpus, batch 64; bytes "
+                                            "per query)")
 
 
 class ClockSampler:
@@ -530,6 +530,7 @@ def measure(pkg, cfg, corp, q, index, args, device, mode="ci", dist=None, local_
         toks4 = (doclens64[pr.clamp(min=0)] * (pr >= 0)).sum()
         work.append({"cand": int(taps.n_cand.sum()), "cand_tokens": int(toks), "pruned_tokens": int(toks4),
                      "contenders": int(taps.n_contenders.sum()),
+                     "kept": max(0, sum(index.kept(B, nq, P, n_prune, k, maxc))) if mode == "ci" else 0,
                      "retrieved": int(list_len[taps.probes.to(torch.int64)].sum())})
         del taps, mask
     del list_len
@@ -646,9 +647,9 @@ def measure(pkg, cfg, corp, q, index, args, device, mode="ci", dist=None, local_
     # algorithmic HBM bytes of one launch of the stage-3 bound scan: the centroid id of every candidate token (4 B) +
     # 8 B per candidate document (its token offsets); the kernel's own id / range / bound traffic is not the method's
     ci_bytes = 4.0 * mean("cand_tokens") + 8.0 * mean("cand")
-    # what binds it: one table-row lookup per candidate token; a lookup is one distinct 128-byte line for the SM's
-    # load pipe, which retires one line per cycle, so the roof is SMs x SM clock row lookups per second (derived from
-    # the device's SM count and the clock sampled during the timed region; not a measured peak)
+    # what binds it (without the first cut): one table-row lookup per candidate token; a lookup is one distinct 128-byte line
+    # for the SM's load pipe, which retires one line per cycle, so the roof is SMs x SM clock row lookups per second (derived
+    # from the device's SM count and the clock sampled during the timed region; not a measured peak)
     rows = mean("cand_tokens")
     sm_count = torch.cuda.get_device_properties(device).multi_processor_count
     sm_hz = 1e6 * (clocks["sm_mhz"] or clocks["sm_max_mhz"] or 1965.0)
@@ -662,10 +663,9 @@ def measure(pkg, cfg, corp, q, index, args, device, mode="ci", dist=None, local_
     g4_row_bytes = 0.0 if rq_mode else mean("pruned_tokens") * nq * 4.0
     stages = {name: round(v / n_prof, 4) for name, v in stage_ms.items()}
     if mode == "ci":
-        lookup_roof *= 32.0 / 3.5 if launches["centroid_interaction"] >= 3 * n_prof else 1.0
         ratio, src = NCU_CI_DRAM_PER_ALGORITHMIC_BYTE.get(cfg.name, NCU_CI_DRAM_PER_ALGORITHMIC_BYTE[None])
         frac = gbs(ci_bytes, ci_ms) / peak
-        # with the first cut stage 3's bounds are six launches instead of one
+        # with the first cut stage 3's bounds are seven launches instead of one
         first_cut = launches["centroid_interaction"] >= 3 * n_prof
         if first_cut:
             ratio, src = NCU_CUT_DRAM_PER_ALGORITHMIC_BYTE
@@ -685,10 +685,12 @@ def measure(pkg, cfg, corp, q, index, args, device, mode="ci", dist=None, local_
                                "costs a random lookup, in shared memory (about 3.5 bank conflicts each 32) or of a 32-byte "
                                "row through L1/L2, which binds the kernel" % ("met" if frac >= TARGET else "NOT met")},
             "contender_fraction": mean("contenders") / max(mean("cand"), 1.0),
-            "binding_roof": {"bound": ("shared-memory lookups (32 random banks in 3.5 cycles) of the scan alone, held against the "
-                                       "time of all six launches" if first_cut else
-                                       "table-row lookups (one 128-byte line per SM cycle)") +
-                                      "; derived from SM count x sampled SM clock, not a driver-measured peak",
+            # with the first cut no single rate binds the seven launches (the lookups of filter_scan_kernel alone run at 71 % of
+            # the shared-memory wavefront peak in an ncu capture)
+            "first_cut_kept_fraction": mean("kept") / max(mean("cand"), 1.0) if first_cut else None,
+            "binding_roof": None if first_cut else
+                            {"bound": "table-row lookups (one 128-byte line per SM cycle); derived from SM count x sampled SM "
+                                      "clock, not a measured peak",
                              "lookups_per_launch": rows, "achieved_glookups_s": rows / (ci_ms * 1e-3) / 1e9 if ci_ms > 0 else 0.0,
                              "peak_glookups_s": lookup_roof / 1e9, "sm_count": sm_count, "sm_mhz": sm_hz / 1e6,
                              "frac": rows / (ci_ms * 1e-3) / lookup_roof if ci_ms > 0 else 0.0},
@@ -697,8 +699,8 @@ def measure(pkg, cfg, corp, q, index, args, device, mode="ci", dist=None, local_
         # candidate refinement by partial scores replaces the scan: the dominant stage-3 kernel visits every token of
         # the nq * nprobe probed posting lists.  Algorithmic bytes per visit: the list entry (token id + document id,
         # 8 B) and the token's code (residual code, or 1-bit code + its 4-byte scale); per candidate document its
-        # partial score (4 B).  The table of running maxima is the implementation's, not the method's, and is not
-        # counted.  The slot times the clear, the scoring kernel and (RaBitQ) the summation together.
+        # partial score (4 B).  The visit lists (or the table of running maxima) are the implementation's, not the method's,
+        # and are not counted.  The slot times the clear, the scoring kernel and the summation together.
         code_b = (cfg.dim // 8 + 4.0) if rq_mode else float(cfg.code_bytes)
         ps_bytes = mean("retrieved") * (8.0 + code_b) + mean("cand") * 4.0
         frac = gbs(ps_bytes, ci_ms) / peak
@@ -708,7 +710,7 @@ def measure(pkg, cfg, corp, q, index, args, device, mode="ci", dist=None, local_
             traffic, tk = per_query * B, "stored ncu figure, not measured in this run: " + src + " x batch"
         roofline = {
             "kernel": ("rabitq_partial_kernel" if rq_mode else "partial_score_kernel")
-            + " (+ its clear kernel): partial scores of the retrieved tokens, Algorithm 2", "bound": "hbm",
+            + " (+ its clear and sum kernels): partial scores of the retrieved tokens, Algorithm 2", "bound": "hbm",
             "achieved": gbs(ps_bytes, ci_ms), "peak": peak, "peak_kind": peak_kind, "unit": "GB/s", "frac": frac,
             "traffic": traffic, "traffic_kind": tk, "ms_per_launch": ci_ms, "algorithmic_bytes_per_launch": ps_bytes,
             "target": {"frac": TARGET, "met": bool(frac >= TARGET)},

@@ -88,7 +88,7 @@ struct Layout {
     size_t qdig;          // int8   [3][B*nq][128]
     size_t qdig4;         // int8   [3][B*residual_rows(nq)][128]  the same for stage 4
     size_t table;         // int32  [B][K][nq]
-    size_t table8;        // uint8  [B][K][nq]        coarse copy: min((S + 2^24 + 64) >> 17, 255)
+    size_t table8;        // uint8  [B][K][coarse_pitch(nq)]  coarse copy: clamp(S >> 16, 0, 255), zeros past nq
     size_t part;          // uint64 [B][n_part][P][nq] partial top-P keys
     size_t probes;        // int32  [B][nq][P]
     size_t pq_gmax;       // int32  [B][pq_groups][nq] stages 1 + 2a together: largest score of each group of sample rows,

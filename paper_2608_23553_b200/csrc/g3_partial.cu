@@ -7,14 +7,13 @@
 // SQ_i = sum_x Xq_i[x], Xq = rint(q * 2^22): integers plus one correctly rounded double expression, so the result does
 // not depend on the order in which tokens are visited (integer max) nor on the machine.
 //
-// As in the paper's design a block serves one (query token, posting list) pair: the query token's integers sit in
-// shared memory, one thread scores one document token, and the maximum goes to the score table with atomicMax while the
-// thread moves on to its next token; every increase of a table entry is also added to the document's partial score, so
-// no separate summation pass is needed.  The table is indexed by candidate rank (bitmap word prefix + popcount), so it has
-// one 4*q_len-byte row per candidate rather than per document.
-//
-// Batches on large corpora keep the visits as lists instead of the table (g3_visits.cuh); few queries per call keep the
-// table, whose update is one atomic and whose sum needs no second kernel.
+// A block serves one query token: one of its posting lists when few queries are served, several or all of them in a batch
+// (refine_splits).  The query token's digits sit in shared memory and a thread scores two list entries at a time.  What becomes
+// of a score depends on the call:
+//   - Batches on large corpora push it onto its candidate's list of visits, which a second kernel sums (g3_visits.cuh).
+//   - Few queries per call, small corpora and candidates with many visits keep a table of maxima, one row of q_len per
+//     candidate rank (bitmap word prefix + popcount): atomicMax, and every increase is also added to the document's partial
+//     score, so that no second kernel is needed.
 #include <math.h>
 
 #include "g3_visits.cuh"

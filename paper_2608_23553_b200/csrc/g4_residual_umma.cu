@@ -8,7 +8,7 @@
 // int32; the three planes are recombined in fp32 (relative error 2^-24).
 //
 // A CTA owns one query and a run of its surviving documents, whose tokens form one stream cut into tiles of 128
-// (MMA M).  The kernel is bound by the instructions and latencies around the MMAs (tensor pipe 12 %), so:
+// (MMA M).  The kernel is bound by the instructions and latencies around the MMAs (tensor pipe 15 %), so:
 //   - codes expand with one shift and one mask per four dimensions (the query's digits are stored in the order in which
 //     codes expand, digit_dim()) and go into tensor memory as the A operand with one tcgen05.st per thread;
 //   - each warp takes 16 query tokens of a quarter's 32 token rows (two warps per quarter for q_len <= 32, four above) and

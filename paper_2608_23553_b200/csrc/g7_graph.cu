@@ -7,15 +7,15 @@
 // centroids take the place of query tokens in the stage-1 tensor-core kernel and stage 2a picks each row's best
 // degree + 1 entries, of which the centroid itself is dropped.
 //
-// Search (query time): one warp per query token runs a best-first search with a bounded result list:
+// Search (query time): a block of four warps per query token runs a best-first search with a bounded result list:
 //   - the entry points floor(j K / n_entries), j < n_entries, are visited (scored, marked, offered to the list);
 //   - repeatedly the first list member that has not been expanded is expanded: each of its graph neighbours that was
 //     never visited is visited; the search ends when every list member is expanded or after max_expansions expansions;
 //   - the list keeps the best `beam` visited centroids by (score descending, id ascending).
 // The score is the exact S_fx(q, c) = floor((sum_d Xq[d] Xc[d] + 2^19) / 2^20) in 64-bit integers, so the list after
 // each step is the best `beam` of everything offered so far whatever the order of evaluation, and the visited set, the
-// probes and their scores are reproducible bit for bit.  The list lives in registers (two 64-bit keys per lane, sorted
-// by slot = lane + 32 j), the visited set is a bitmap in global memory owned by the warp.
+// probes and their scores are reproducible bit for bit.  The list lives in the first warp's registers (two 64-bit keys per
+// lane, sorted by slot = lane + 32 j), the visited set is a bitmap in shared memory (in global memory above 2^20 centroids).
 #include "common.cuh"
 
 namespace chimera {

@@ -52,8 +52,8 @@ def test_partial_refinement_small_corpora(D, nbits, nq, K, N, nprobe, n_prune, k
 
 @pytest.mark.parametrize("nbits", [2, 1])
 def test_partial_refinement_hashed_table_equals_dense_and_oracle(nbits):
-    """With enough queries per call and a corpus large enough, the (candidate, query token) maxima live in an
-    open-addressing table instead of dense rows.  40 queries (on a B200) on 30,000 documents take that path; the same queries one
+    """With enough queries per call and a corpus large enough, the visits of each candidate are kept as a list instead of
+    dense rows of (candidate, query token) maxima.  40 queries (on a B200) on 30,000 documents take that path; the same queries one
     at a time take the dense path; both must agree bit for bit in F' of every candidate, pruned ids and final results,
     and sampled queries must match the oracle."""
     import paper_2608_23553_b200 as pkg
@@ -64,7 +64,7 @@ def test_partial_refinement_hashed_table_equals_dense_and_oracle(nbits):
     gix = pkg.Index(torch.from_numpy(cent).to(dev), torch.from_numpy(cids).to(dev), torch.from_numpy(codes).to(dev),
                     torch.from_numpy(doclens).to(dev), nbits)
     gix.enable_partial()
-    # calls of up to (SM count / 4) queries keep dense rows; three more queries and the table is hashed, which shows in
+    # calls of up to (SM count / 4) queries keep dense rows; three more queries and the visits are lists, which shows in
     # the workspace: more queries, yet fewer bytes
     small = torch.cuda.get_device_properties(0).multi_processor_count // 4
     B = small + 3
