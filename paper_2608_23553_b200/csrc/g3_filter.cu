@@ -6,8 +6,8 @@
 //     CI(d) = sum_i max_t S[c_t, i]  <=  sum_i theta_i + sum_t e(c_t) = hi0(d).
 // theta_i is set so that about FILTER_LAMBDA of a document's tokens exceed it: lower thresholds count a column's second
 // and third best tokens as well, higher ones replace the column's true maximum by theta.  Any choice is correct; with one
-// token per column of a long document the bound keeps 7-13 % of the candidates when 1 % are wanted (65,536 and 262,144
-// centroids, candidates of 85-512 tokens), with half or one and a half times as many up to twice that.
+// token per column of a long document of independent tokens the bound keeps 7-13 % of the candidates when 1 % are wanted
+// (65,536 and 262,144 centroids, candidates of 85-512 tokens), with half or one and a half times as many up to twice that.
 //
 // With documents that repeat their centroids, or hold several near the same query token, the bound counts each of them where
 // CI counts one, and most candidates pass it; then the cut only costs (below, at filter_judge_kernel).
@@ -67,8 +67,8 @@ static int filter_codec(int64_t K)
 // 32 / 64, whose other form scans 8-bit rows, 11 against 6 for the others, which look up exact rows), for its tables (per
 // query and centroid) and for the exact rows of its seeds.  What is scanned is what the candidates hold, so their expected
 // number counts and not the room for them; a document is a candidate when one of its distinct centroids is probed.
-// In tokens, per query, fitted to calls with and without the cut (independent tokens, kept 1-60 %; the sign is right in 69
-// of 74 calls of 2,000 to 1.5 million documents, and the others lose at most a quarter):
+// In tokens, per query, fitted to calls with and without the cut (independent tokens, kept 1-60 %; within 4 % of the better
+// form in 70 of 74 calls on 2,000 to 1.5 million documents, and the others lose at most a quarter):
 //   q_len 32 / 64: 8 per centroid, 5 n_prune documents, 20 M a call.  Mid's documents, one query, 12 M tokens: 206 us with
 //     the cut, 187 without; two: 248 / 266; eight: 537 / 720; 64 queries with one probe a token on 4 million documents and
 //     262,144 centroids, 2.2 M tokens each: 2,451 / 2,300; with four probes, 8.7 M each: 32 queries 2,746 / 3,103, two 414 / 372.
