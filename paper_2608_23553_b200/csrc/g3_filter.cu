@@ -203,8 +203,9 @@ filter_theta_kernel(const int32_t *__restrict__ table, int64_t K, int nq, int m,
 // draw a quarter as many centroids as they have tokens (100 %): 8.09 / 6.36 ms; of neighbouring centroids of four topics (63 %,
 // by the sample 57 %): 9.76 / 9.21, 16 queries (66 %, by the sample 60 %): 1,034 / 873 us; 512 tokens of such (35 %, sample 27 %):
 // 25.7 / 28.7 ms; independent centroids, 16 queries, n_prune 16,384 (55 %, sample 56 %): 2.96 / 3.04 ms.  As the judge has it: 6.46
-// ms, 9.73 ms, 915 us, 25.8 ms and 2.96 ms.  It costs 15 us where the cut stays (16 queries: 809 -> 825 us), most of it latency:
-// candidate, range, ids, rows, then the last block's histogram.
+// ms, 9.73 ms, 915 us, 25.8 ms and 2.96 ms.  It costs 15 us where the cut stays (16 queries: 809 -> 825 us; 64 of 64 tokens on
+// 512-token documents 30 of 12,740), most of it latency: candidate, range, ids, rows, then the last block's histogram (4 us).  Half as many
+// samples, eight rows in flight per lane, or four warps per document are no faster.
 // grid (blocks, queries), a document per warp, sixteen columns per lane, 64 tokens in flight.
 template <int NQ>
 __global__ void __launch_bounds__(SEL_THREADS)
