@@ -142,7 +142,7 @@ Layout make_layout(const Index &ix, const Params &p)
     L.flt_thr = take(filter ? B * sizeof(int32_t) : 0);
     L.flt_slot = L.lo;                  // (a call that cuts has no lower bounds, one that does not has no seeds)
     L.flt_tau = take(filter ? B * sizeof(int32_t) : 0);
-    L.flt_smp = take(filter ? JUDGE_SAMPLES * sizeof(int2) : 0);
+    L.flt_smp = take(filter ? CUT_SAMPLES * sizeof(int2) : 0);
     L.flt_vote = take(filter ? 64 * sizeof(int32_t) : 0);
     L.flt_parts = take(filter ? filter_parts_bytes(ix, p) : 0);
     L.flt_counts = take(filter ? B * (size_t)filter_count_slots() * sizeof(int32_t) : 0);

@@ -114,7 +114,7 @@ struct Layout {
     size_t flt_thr;       // int32  [B]               hi0 from which a candidate is a seed,
     size_t flt_slot;      // int32  [B][maxc]         place of each seed in the seed list,
     size_t flt_tau;       // int32  [B]               n_prune-th largest exact CI of the seeds (lower bound, without the cut),
-    size_t flt_smp;       // int2   [JUDGE_SAMPLES]   CI and first bound of sampled candidates,
+    size_t flt_smp;       // int2   [CUT_SAMPLES]   CI and first bound of sampled candidates,
     size_t flt_vote;      // int32  [64]              how many of those would be kept, counters of the kernel that finds out,
     size_t flt_counts;    // int32  [B][slots]        kept candidates per slice
     size_t kept;          // int32  [B][maxc]         candidates that pass it, ascending
@@ -280,7 +280,7 @@ int launch_coarse_bounds(const Index &ix, const Params &p, const uint8_t *table8
 // launch_filter_keep takes the seeds' exact CI and writes the candidates that can still be in the top n_prune, ascending;
 // launch_filter_contenders narrows them down by the 8-bit upper bounds.  Where a sample shows that the cut would keep most
 // candidates, there are no seeds, all candidates are kept, and the contenders are found by the 8-bit lower bounds.
-constexpr int JUDGE_QUERIES = 16, JUDGE_SAMPLES = 4096;
+constexpr int CUT_QUERIES = 16, CUT_SAMPLES = 4096;
 FirstCut first_cut(const Params &p, const Layout &L, char *ws);
 bool filter_used(const Index &ix, const Params &p);
 size_t filter_table_pitch(const Index &ix);

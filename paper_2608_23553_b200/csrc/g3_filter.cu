@@ -10,10 +10,10 @@
 // (65,536 and 262,144 centroids, candidates of 85-512 tokens), with half or one and a half times as many up to twice that.
 //
 // With documents that repeat their centroids, or hold several near the same query token, the bound counts each of them where
-// CI counts one, and most candidates pass it; then the cut only costs (below, at filter_judge_kernel).
+// CI counts one, and most candidates pass it; then the cut only costs (below, at filter_sample_kernel).
 //
 //   filter_theta_kernel    theta_i from a sample of the table's rows
-//   filter_judge_kernel    q_len 32 / 64: whether the cut would drop enough, from sampled candidates; if not, the kernels
+//   filter_sample_kernel    q_len 32 / 64: whether the cut would drop enough, from sampled candidates; if not, the kernels
 //                          down to the count return at once, all candidates are kept, and their 8-bit bounds decide
 //   filter_excess_kernel   e(c) of every centroid, rounded up (16 bits, or 6-bit codes five to a word for large K)
 //   filter_scan_kernel     hi0 of every candidate: the query's whole e table in shared memory, one lookup per token
@@ -37,7 +37,7 @@ constexpr double FILTER_LAMBDA = 1.0;     // wanted tokens of a document above t
 constexpr int FILTER_SAMPLE = 4096;       // table rows sampled per query for theta
 constexpr int KEEP_SPLIT = 32;            // most blocks per query of the selection kernels
 constexpr int FILTER_BINS = 2048;         // histogram bins of sum_t e(c_t), 2^17 (one 128th) each
-constexpr int JUDGE_KEPT_PERCENT = 58;        // of the sampled candidates: with more the call does without the cut
+constexpr int CUT_KEPT_PERCENT = 58;        // of the sampled candidates: with more the call does without the cut
 constexpr int64_t FILTER_SMEM = 208 * 1024;   // shared memory of the scan's block that its e table may take
 
 // 6-bit codes of e in units of 2^16 (1/256): exact up to 20, then steps of about 7 % (the sums of a document's far
@@ -103,14 +103,14 @@ static int filter_split(const Index &ix, const Params &p)
     return (int)(g > KEEP_SPLIT ? KEEP_SPLIT : g < 1 ? 1 : g);
 }
 
-// Queries that the judge samples, candidates of each, and what the kernels behind it go by.
-static int judge_queries(const Params &p) { return p.B < JUDGE_QUERIES ? p.B : JUDGE_QUERIES; }
-static int judge_samples(const Params &p) { return JUDGE_SAMPLES / 32 / judge_queries(p) * 32; }
+// Queries that are sampled, candidates of each, and what the kernels behind it go by.
+static int cut_queries(const Params &p) { return p.B < CUT_QUERIES ? p.B : CUT_QUERIES; }
+static int cut_samples(const Params &p) { return CUT_SAMPLES / 32 / cut_queries(p) * 32; }
 FirstCut first_cut(const Params &p, const Layout &L, char *ws)
 {
     FirstCut c;
     c.kept = coarse_supported(p.nq) ? (const int32_t *)(ws + L.flt_vote) : nullptr;
-    c.most = judge_queries(p) * judge_samples(p) * JUDGE_KEPT_PERCENT / 100;
+    c.most = cut_queries(p) * cut_samples(p) * CUT_KEPT_PERCENT / 100;
     return c;
 }
 
@@ -125,7 +125,7 @@ size_t filter_parts_bytes(const Index &ix, const Params &p)
 // grid (ceil(nq / 32), B, parts), lane = query token.  theta[b][i] = the smallest t (in units of 2^16) such that at most
 // `rank` of the m sampled rows (every step-th one) have S >= t 2^16.  With few queries the sample is split over several
 // blocks that add their histograms up in `parts_hist` ([B][groups][256 * 32], cleared before); the last one to
-// finish (`done`, likewise) reads the sum.  Also clears what the scan and the seed selection add to, and the judge's words (vote,
+// finish (`done`, likewise) reads the sum.  Also clears what the scan and the seed selection add to, and the sample's words (vote,
 // may be NULL).
 __global__ void __launch_bounds__(SEL_THREADS)
 filter_theta_kernel(const int32_t *__restrict__ table, int64_t K, int nq, int m, int step, int rank,
@@ -194,22 +194,22 @@ filter_theta_kernel(const int32_t *__restrict__ table, int64_t K, int nq, int m,
     if (lane == 0 && blockIdx.x * 32 + warp < nq) theta[(int64_t)b * nq + blockIdx.x * 32 + warp] = best;
 }
 
-// ------------------------------------------------------------------------------------------------ judge -----------
-// Does the cut pay?  JUDGE_SAMPLES candidates, spread over up to JUDGE_QUERIES queries of the call: CI from the 8-bit rows
+// ------------------------------------------------------------------------------------------------ sample ----------
+// Does the cut pay?  CUT_SAMPLES candidates, spread over up to CUT_QUERIES queries of the call: CI from the 8-bit rows
 // and the bound hi0, then the share of them whose bound reaches the sample's own n_prune-th of n_cand.  A query with so few
 // candidates that all are kept counts as kept.  Queries of a batch search the same documents, so one answer per call is
 // enough, and results do not depend on it.
 // Where the line lies (batches of Mid's sizes unless said; the share that passes, with the cut / without it): documents that
 // draw a quarter as many centroids as they have tokens (100 %): 8.09 / 6.36 ms; of neighbouring centroids of four topics (63 %,
 // by the sample 57 %): 9.76 / 9.21, 16 queries (66 %, by the sample 60 %): 1,034 / 873 us; 512 tokens of such (35 %, sample 27 %):
-// 25.7 / 28.7 ms; independent centroids, 16 queries, n_prune 16,384 (55 %, sample 56 %): 2.96 / 3.04 ms.  As the judge has it: 6.46
+// 25.7 / 28.7 ms; independent centroids, 16 queries, n_prune 16,384 (55 %, sample 56 %): 2.96 / 3.04 ms.  As the sample decides: 6.46
 // ms, 9.73 ms, 915 us, 25.8 ms and 2.96 ms.  It costs 15 us where the cut stays (16 queries: 809 -> 825 us; 64 of 64 tokens on
 // 512-token documents 30 of 12,740), most of it latency: candidate, range, ids, rows, then the last block's histogram (4 us).  Half as many
 // samples, eight rows in flight per lane, or four warps per document are no faster.
 // grid (blocks, queries), a document per warp, sixteen columns per lane, 64 tokens in flight.
 template <int NQ>
 __global__ void __launch_bounds__(SEL_THREADS)
-filter_judge_kernel(const uint8_t *__restrict__ table8, int64_t K, const int32_t *__restrict__ theta, int B,
+filter_sample_kernel(const uint8_t *__restrict__ table8, int64_t K, const int32_t *__restrict__ theta, int B,
                     const int32_t *__restrict__ cand, const int32_t *__restrict__ n_cand, int64_t maxc,
                     const int64_t *__restrict__ doc_off, const int32_t *__restrict__ cids, int n_prune, bool coded,
                     int2 *__restrict__ smp, int32_t *__restrict__ vote)
@@ -942,9 +942,9 @@ int launch_filter_scan(const Index &ix, const Params &p, const Layout &L, const 
            ready ? vote : nullptr);
     CHIMERA_CUDA(cudaGetLastError());
     if (ready) {
-        const int jq = judge_queries(p);
-        const dim3 grid((unsigned)(judge_samples(p) / 32), (unsigned)jq);
-        launch(p.nq == 32 ? filter_judge_kernel<32> : filter_judge_kernel<64>, grid, SEL_THREADS, 0, st, table8, ix.K, theta, p.B,
+        const int jq = cut_queries(p);
+        const dim3 grid((unsigned)(cut_samples(p) / 32), (unsigned)jq);
+        launch(p.nq == 32 ? filter_sample_kernel<32> : filter_sample_kernel<64>, grid, SEL_THREADS, 0, st, table8, ix.K, theta, p.B,
                cand, n_cand, p.maxc, ix.doc_off, ix.cids, p.n_prune, codec == 6, (int2 *)(ws + L.flt_smp), vote);
         CHIMERA_CUDA(cudaGetLastError());
         count_launch(SLOT_CI);
