@@ -137,7 +137,10 @@ Layout make_layout(const Index &ix, const Params &p)
     L.cont_rng = take(2 * two_phase);
     L.n_cont = take(B * sizeof(int32_t));
     L.flt_theta = take(filter ? B * nq * sizeof(int32_t) : 0);
-    L.flt_tab = take(filter ? B * filter_table_pitch(ix) : 0);
+    const bool batch = batch_scan_used(ix, p);
+    const size_t query_tab = filter ? B * filter_table_pitch(ix) : 0, batch_tab = batch ? batch_table_bytes(ix, p) : 0;
+    L.flt_tab = take(query_tab > batch_tab ? query_tab : batch_tab);   // (candidates from the caller are scanned by query)
+    L.flt_over = take(batch ? batch_over_bytes(p) : 0);
     L.flt_hist = take(filter ? B * (size_t)filter_hist_bins() * sizeof(int32_t) : 0);
     L.flt_thr = take(filter ? B * sizeof(int32_t) : 0);
     L.flt_slot = L.lo;                  // (a call that cuts has no lower bounds, one that does not has no seeds)
@@ -151,7 +154,7 @@ Layout make_layout(const Index &ix, const Params &p)
     L.n_kept = take(filter ? B * sizeof(int32_t) : 0);
     L.n_seed = take(filter ? B * sizeof(int32_t) : 0);
     L.pruned = take(B * p.n_prune * sizeof(int32_t));
-    L.ranks = take(ix.tok_id ? B * (size_t)L.words * sizeof(uint2) : 0);
+    L.ranks = take(ix.tok_id || batch ? B * (size_t)L.words * sizeof(uint2) : 0);
     // retrieved-token scores of the refinements: visit lists, or dense rows per candidate
     L.visit_nodes = visit_list_nodes(ix, p);
     L.partial_m = take(!ix.tok_id ? 0 : L.visit_nodes ? B * ((size_t)L.visit_nodes * 8 + (size_t)p.maxc * 4)
@@ -266,6 +269,7 @@ static int run(const Index &ix, const Params &p, int first, int last, const floa
     int32_t *ci = (int32_t *)(ws + L.ci);
     const bool two_phase = coarse_supported(p.nq) && !partial && !rabitq;
     const bool filter = filter_used(ix, p) && !partial && !rabitq;      // (stage 3's first cut)
+    const bool batch = filter && first <= 2 && batch_scan_used(ix, p);
     // the candidates' token ranges, where the 8-bit scan reads them for every candidate
     int2 *scan_rng = two_phase && !filter && ix.T < 0x7fffffffLL ? (int2 *)(ws + L.cand_rng) : nullptr;
     // blocks per query for the exact scores of a short list (two to three times n_prune documents): one per SM in a large
@@ -354,7 +358,7 @@ static int run(const Index &ix, const Params &p, int first, int last, const floa
             return rc;
         }
         prof_mark(SLOT_PROBE, st);
-        if ((rc = launch_gather(ix, p, L, probes, bitmap, clear_words > 0, chunk_cnt, cand, n_cand, partial || rabitq ? ranks : nullptr,
+        if ((rc = launch_gather(ix, p, L, probes, bitmap, clear_words > 0, chunk_cnt, cand, n_cand, partial || rabitq || batch ? ranks : nullptr,
                                 scan_rng, scan_rng && contenders_split(ix, p) ? ci : nullptr, status, st)))
             return rc;
         prof_mark(SLOT_GATHER, st);
@@ -391,7 +395,7 @@ static int run(const Index &ix, const Params &p, int first, int last, const floa
                 (rc = launch_cand_ranges(ix, p, cand, n_cand, scan_rng, ci, st)))
                 return rc;
             if (filter) {
-                if ((rc = launch_filter_scan(ix, p, L, table, (uint8_t *)(ws + L.table8), cand, n_cand, hi, cont, cont_rng, ws, st)))
+                if ((rc = launch_filter_scan(ix, p, L, batch, table, (uint8_t *)(ws + L.table8), cand, n_cand, hi, cont, cont_rng, ws, st)))
                     return rc;
                 if ((rc = launch_centroid_interaction(ix, p, table, cont, (const int32_t *)(ws + L.n_seed), ci, exact_blocks,
                                                       SLOT_CI, cont_rng, st)))

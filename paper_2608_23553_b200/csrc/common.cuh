@@ -108,7 +108,8 @@ struct Layout {
     size_t cont_rng;      // int2   [B][maxc]         the same for the contenders
     size_t n_cont;        // int32  [B]
     size_t flt_theta;     // int32  [B][nq]           first cut (g3_filter.cu): thresholds,
-    size_t flt_tab;       // uint8  [B][pitch]        one number per centroid,
+    size_t flt_tab;       // uint8  [B][pitch]        one number per centroid (a batch at a time: rows of codes, g3_batch_scan.cu),
+    size_t flt_over;      // that form's steps and listed centroids,
     size_t flt_hist;      // int32  [B][bins]         histogram of the bounds,
     size_t flt_parts;     // int32  histograms and counters of the threshold kernel's blocks (few queries)
     size_t flt_thr;       // int32  [B]               hi0 from which a candidate is a seed,
@@ -123,7 +124,7 @@ struct Layout {
     size_t n_seed;        // int32  [B]
     size_t pruned;        // int32  [B][n_prune]
     size_t ranks;         // uint2  [B][words]        bitmap word, candidates before it (document -> candidate index);
-                          //                          only with token lists
+                          //                          only with token lists, or where the first cut scans a batch at a time
     size_t partial_m;     // int32  [B][maxc][nq]     per (candidate, query token) best retrieved-token score, or the visit
                           //                          lists in its place (g3_visits.cuh)
     int64_t visit_nodes;  // nodes per query of those lists; 0 = the table
@@ -283,11 +284,15 @@ int launch_coarse_bounds(const Index &ix, const Params &p, const uint8_t *table8
 constexpr int CUT_QUERIES = 16, CUT_SAMPLES = 4096;
 FirstCut first_cut(const Params &p, const Layout &L, char *ws);
 bool filter_used(const Index &ix, const Params &p);
+bool batch_scan_used(const Index &ix, const Params &p);       // ... and scans for all queries at once (g3_batch_scan.cu)
+size_t batch_table_bytes(const Index &ix, const Params &p);
+size_t batch_over_bytes(const Params &p);
 size_t filter_table_pitch(const Index &ix);
 int filter_hist_bins();
 int filter_count_slots();
 size_t filter_parts_bytes(const Index &ix, const Params &p);
-int launch_filter_scan(const Index &ix, const Params &p, const Layout &L, const int32_t *table, uint8_t *table8,
+// batch: by the batch's form, which needs the workspace's ranks.
+int launch_filter_scan(const Index &ix, const Params &p, const Layout &L, bool batch, const int32_t *table, uint8_t *table8,
                        const int32_t *cand, const int32_t *n_cand, int32_t *hi0, int32_t *seed,
                        int2 *seed_rng, char *ws, cudaStream_t st);
 int launch_filter_keep(const Index &ix, const Params &p, const Layout &L, const int32_t *cand,

@@ -29,14 +29,13 @@
 #include <limits.h>
 #include <math.h>
 
-#include "g3_select.cuh"
+#include "g3_filter.cuh"
 
 namespace chimera {
 
 constexpr double FILTER_LAMBDA = 1.0;     // wanted tokens of a document above theta, per query token
 constexpr int FILTER_SAMPLE = 4096;       // table rows sampled per query for theta
 constexpr int KEEP_SPLIT = 32;            // most blocks per query of the selection kernels
-constexpr int FILTER_BINS = 2048;         // histogram bins of sum_t e(c_t), 2^17 (one 128th) each
 constexpr int CUT_KEPT_PERCENT = 58;        // of the sampled candidates: with more the call does without the cut
 constexpr int64_t FILTER_SMEM = 208 * 1024;   // shared memory of the scan's block that its e table may take
 
@@ -74,16 +73,20 @@ static int filter_codec(int64_t K)
 //     262,144 centroids, 2.2 M tokens each: 2,451 / 2,300; with four probes, 8.7 M each: 32 queries 2,746 / 3,103, two 414 / 372.
 //   others: 4 per centroid, 4 n_prune documents, 2 M a call.  21 tokens, 20,000 documents, 1.3 M tokens: 143 us with the cut, 133
 //     without; 2.6 M: 153 / 181; 100 tokens on 200,000 documents, 12 M: 263 / 756.
+double expected_tokens(const Index &ix, const Params &p)
+{
+    const double len = (double)ix.T / (double)ix.N, distinct = (double)ix.ivf_len / (double)ix.N;
+    const double probed = (double)p.nq * p.P / (double)ix.K;
+    const double cand = probed < 1.0 ? (double)ix.N * (1.0 - pow(1.0 - probed, distinct)) : (double)ix.N;
+    return (cand < (double)p.maxc ? cand : (double)p.maxc) * len;
+}
 bool filter_used(const Index &ix, const Params &p)
 {
     if (filter_codec(ix.K) == 0 || ix.T >= 0x7fffff00LL || ix.max_doclen > 32000) return false;
     const bool wide = coarse_supported(p.nq);
-    const double len = (double)ix.T / (double)ix.N, distinct = (double)ix.ivf_len / (double)ix.N;
-    const double probed = (double)p.nq * p.P / (double)ix.K;
-    const double cand = probed < 1.0 ? (double)ix.N * (1.0 - pow(1.0 - probed, distinct)) : (double)ix.N;
-    const double tokens = (cand < (double)p.maxc ? cand : (double)p.maxc) * len;
+    const double len = (double)ix.T / (double)ix.N;
     const double fixed = (wide ? 8.0 : 4.0) * (double)ix.K + (wide ? 5.0 : 4.0) * p.n_prune * len;
-    return (double)p.B * (tokens - fixed) >= (wide ? 2e7 : 2e6);
+    return (double)p.B * (expected_tokens(ix, p) - fixed) >= (wide ? 2e7 : 2e6);
 }
 size_t filter_table_pitch(const Index &ix)
 {
@@ -212,7 +215,7 @@ __global__ void __launch_bounds__(SEL_THREADS)
 filter_sample_kernel(const uint8_t *__restrict__ table8, int64_t K, const int32_t *__restrict__ theta, int B,
                     const int32_t *__restrict__ cand, const int32_t *__restrict__ n_cand, int64_t maxc,
                     const int64_t *__restrict__ doc_off, const int32_t *__restrict__ cids, int n_prune, bool coded,
-                    int2 *__restrict__ smp, int32_t *__restrict__ vote)
+                    const int2 *__restrict__ scale, int2 *__restrict__ smp, int32_t *__restrict__ vote)
 {
     pdl_entry();
     constexpr int LPR = NQ / 16;                             // lanes per row, 16 columns each
@@ -240,7 +243,7 @@ filter_sample_kernel(const uint8_t *__restrict__ table8, int64_t K, const int32_
             sum_tm1 += t.x + t.y + t.z + t.w - 4;
         }
         uint32_t best[4] = {0u, 0u, 0u, 0u};
-        int over = 0;
+        int over = 0, above = 0;                             // sum of e and tokens that have one
         int32_t cid[2];                                      // 64 tokens at a time
 #pragma unroll
         for (int h = 0; h < 2; ++h) cid[h] = 32 * h + lane < r.y ? cids[r.x + 32 * h + lane] : 0;
@@ -265,7 +268,9 @@ filter_sample_kernel(const uint8_t *__restrict__ table8, int64_t K, const int32_
                     best[k] = __vmaxu4(best[k], w[k]);
                     acc += __vmaxu2(w[k] & 0x00ff00ffu, tm1[k].x) + __vmaxu2((w[k] >> 8) & 0x00ff00ffu, tm1[k].y);
                 }
-                over += (int)(acc & 0xffffu) + (int)(acc >> 16) - sum_tm1;
+                const int e = (int)(acc & 0xffffu) + (int)(acc >> 16) - sum_tm1;
+                over += e;
+                above += e > 0 ? 1 : 0;
             }
         }
         int ci = 0;
@@ -278,7 +283,9 @@ filter_sample_kernel(const uint8_t *__restrict__ table8, int64_t K, const int32_
         ci = __reduce_add_sync(0xffffffffu, lane < LPR ? ci : 0) + NQ / 2;
         over = __reduce_add_sync(0xffffffffu, over);
         const int base = __reduce_add_sync(0xffffffffu, lane < LPR ? sum_tm1 : 0) + NQ;
-        if (coded) over += over / 28;                        // the 6-bit codes round up, by half a step of 7 % on average
+        // codes round up: 6-bit ones by half a step of 7 % on average, 4-bit ones by half a step of the query's
+        if (scale) over += __reduce_add_sync(0xffffffffu, above) * (scale[b].y - 1) / 2;
+        else if (coded) over += over / 28;
         if (lane == 0) mine[s] = make_int2(ci, base + over);
     }
     __threadfence();
@@ -322,29 +329,6 @@ __device__ __forceinline__ void filter_fill_encoder(uint8_t *enc)
         enc[e] = (uint8_t)j;
     }
     __syncthreads();
-}
-
-// e(c) in units of 2^16 from a row of the 8-bit table: S < 2^16 (u + 1), and for u = 255 S <= 2^16 * 257.  tm1[k]: the
-// thresholds minus one, the even bytes of word k in tm1[k].x and the odd ones in tm1[k].y (16-bit fields), so that
-// sum_i (u_i + 1 - t_i)+ = sum_i max(u_i, t_i - 1) - sum_i (t_i - 1).
-template <int WORDS>
-__device__ __forceinline__ int filter_row_excess(const uint4 *row, const uint2 *tm1, int sum_tm1)
-{
-    uint32_t acc = 0;
-    int full = 0;
-#pragma unroll
-    for (int q = 0; q < WORDS / 4; ++q) {
-        const uint4 v = __ldg(row + q);
-        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const uint2 t = tm1[4 * q + k];
-            acc += __vmaxu2(w[k] & 0x00ff00ffu, t.x);
-            acc += __vmaxu2((w[k] >> 8) & 0x00ff00ffu, t.y);
-            full += __popc((((w[k] & 0x7f7f7f7fu) + 0x01010101u) & w[k]) & 0x80808080u);
-        }
-    }
-    return (int)(acc & 0xffffu) + (int)(acc >> 16) - sum_tm1 + full;      // fields <= 32 * 256
 }
 
 // grid (blocks, B).  One thread per centroid (16-bit values) or per five centroids (6-bit codes): a stream of the 8-bit
@@ -914,43 +898,16 @@ static int filter_unit(const Index &ix, const Params &p, bool from_table8)
     return from_table8 || filter_codec(ix.K) != 16 ? 16 : p.nq <= 63 ? 14 : 15;
 }
 
-int launch_filter_scan(const Index &ix, const Params &p, const Layout &L, const int32_t *table, uint8_t *table8,
-                       const int32_t *cand, const int32_t *n_cand, int32_t *hi0, int32_t *seed,
-                       int2 *seed_rng, char *ws, cudaStream_t st)
+// The scan a query at a time.
+static int launch_query_scan(const Index &ix, const Params &p, const Layout &L, const int32_t *table, uint8_t *table8, int us,
+                             const int32_t *cand, const int32_t *n_cand, int32_t *hi0, char *ws, cudaStream_t st)
 {
     int32_t *theta = (int32_t *)(ws + L.flt_theta), *hist = (int32_t *)(ws + L.flt_hist);
-    int32_t *n_seed = (int32_t *)(ws + L.n_seed), *vote = (int32_t *)(ws + L.flt_vote);
     const FirstCut cut = first_cut(p, L, ws);
     uint8_t *tab = (uint8_t *)(ws + L.flt_tab);
     const bool ready = coarse_supported(p.nq);           // stage 1 has written the 8-bit table
     const int codec = filter_codec(ix.K);
     const size_t pitch = filter_table_pitch(ix);
-    const int step = (int)(ix.K / FILTER_SAMPLE > 1 ? ix.K / FILTER_SAMPLE : 1);
-    const int m = (int)((ix.K + step - 1) / step < 2 * FILTER_SAMPLE ? (ix.K + step - 1) / step : 2 * FILTER_SAMPLE);
-    // the length of the documents that compete for the top: about halfway between the candidates' mean (somewhat above
-    // the corpus's: long documents are probed more often) and the longest, outliers aside
-    const double mean = (double)ix.T / (double)ix.N, most = (double)ix.max_doclen;
-    const double len = 0.5 * ((1.2 * mean < most ? 1.2 * mean : most) + (2.4 * mean < most ? 2.4 * mean : most));
-    int rank = (int)(FILTER_LAMBDA / len * m + 0.5);
-    if (rank < 1) rank = 1;
-    const unsigned groups = (unsigned)((p.nq + 31) / 32);
-    const int parts = filter_parts(ix, p);
-    int32_t *parts_hist = (int32_t *)(ws + L.flt_parts), *done = parts_hist + (size_t)p.B * groups * 256 * 32;
-    if (parts > 1)
-        CHIMERA_CUDA(cudaMemsetAsync(parts_hist, 0, filter_parts_bytes(ix, p), st));
-    launch(filter_theta_kernel, dim3(groups, (unsigned)p.B, (unsigned)parts), SEL_THREADS, 0, st, table, ix.K, p.nq, m, step, rank, theta, hist, n_seed, parts_hist, done,
-           ready ? vote : nullptr);
-    CHIMERA_CUDA(cudaGetLastError());
-    if (ready) {
-        const int jq = cut_queries(p);
-        const dim3 grid((unsigned)(cut_samples(p) / 32), (unsigned)jq);
-        launch(p.nq == 32 ? filter_sample_kernel<32> : filter_sample_kernel<64>, grid, SEL_THREADS, 0, st, table8, ix.K, theta, p.B,
-               cand, n_cand, p.maxc, ix.doc_off, ix.cids, p.n_prune, codec == 6, (int2 *)(ws + L.flt_smp), vote);
-        CHIMERA_CUDA(cudaGetLastError());
-        count_launch(SLOT_CI);
-    }
-
-    const int us = filter_unit(ix, p, ready);
     int64_t gx = (8LL * ix.sm_count + p.B - 1) / p.B;
     if (ready) {
         const int64_t want = ((codec == 16 ? ix.K : (ix.K + 4) / 5) + 255) / 256;
@@ -991,10 +948,57 @@ int launch_filter_scan(const Index &ix, const Params &p, const Layout &L, const 
                                                                    ix.cids, ix.T, hi0, hist, cut);
     }
     CHIMERA_CUDA(cudaGetLastError());
+    count_launch(SLOT_CI, 2);
+    return CHIMERA_OK;
+}
+
+int launch_filter_scan(const Index &ix, const Params &p, const Layout &L, bool batch, const int32_t *table, uint8_t *table8,
+                       const int32_t *cand, const int32_t *n_cand, int32_t *hi0, int32_t *seed,
+                       int2 *seed_rng, char *ws, cudaStream_t st)
+{
+    int32_t *theta = (int32_t *)(ws + L.flt_theta), *hist = (int32_t *)(ws + L.flt_hist);
+    int32_t *n_seed = (int32_t *)(ws + L.n_seed), *vote = (int32_t *)(ws + L.flt_vote);
+    const FirstCut cut = first_cut(p, L, ws);
+    const bool ready = coarse_supported(p.nq);           // stage 1 has written the 8-bit table
+    const int codec = filter_codec(ix.K);
+    const int step = (int)(ix.K / FILTER_SAMPLE > 1 ? ix.K / FILTER_SAMPLE : 1);
+    const int m = (int)((ix.K + step - 1) / step < 2 * FILTER_SAMPLE ? (ix.K + step - 1) / step : 2 * FILTER_SAMPLE);
+    // the length of the documents that compete for the top: about halfway between the candidates' mean (somewhat above
+    // the corpus's: long documents are probed more often) and the longest, outliers aside
+    const double mean = (double)ix.T / (double)ix.N, most = (double)ix.max_doclen;
+    const double len = 0.5 * ((1.2 * mean < most ? 1.2 * mean : most) + (2.4 * mean < most ? 2.4 * mean : most));
+    int rank = (int)(FILTER_LAMBDA / len * m + 0.5);
+    if (rank < 1) rank = 1;
+    const unsigned groups = (unsigned)((p.nq + 31) / 32);
+    const int parts = filter_parts(ix, p);
+    int32_t *parts_hist = (int32_t *)(ws + L.flt_parts), *done = parts_hist + (size_t)p.B * groups * 256 * 32;
+    if (parts > 1)
+        CHIMERA_CUDA(cudaMemsetAsync(parts_hist, 0, filter_parts_bytes(ix, p), st));
+    launch(filter_theta_kernel, dim3(groups, (unsigned)p.B, (unsigned)parts), SEL_THREADS, 0, st, table, ix.K, p.nq, m, step, rank, theta, hist, n_seed, parts_hist, done,
+           ready ? vote : nullptr);
+    CHIMERA_CUDA(cudaGetLastError());
+    const int us = filter_unit(ix, p, ready);
+    int rc;
+    if (batch && (rc = launch_batch_quantum(ix, p, L, table, table8, us, ws, st))) return rc;
+    if (ready) {
+        const int jq = cut_queries(p);
+        const dim3 grid((unsigned)(cut_samples(p) / 32), (unsigned)jq);
+        launch(p.nq == 32 ? filter_sample_kernel<32> : filter_sample_kernel<64>, grid, SEL_THREADS, 0, st, table8, ix.K, theta, p.B,
+               cand, n_cand, p.maxc, ix.doc_off, ix.cids, p.n_prune, codec == 6, batch ? (const int2 *)(ws + L.flt_over) : nullptr,
+               (int2 *)(ws + L.flt_smp), vote);
+        CHIMERA_CUDA(cudaGetLastError());
+        count_launch(SLOT_CI);
+    }
+
+    if (batch) {
+        if ((rc = launch_batch_scan(ix, p, L, table, table8, us, n_cand, hi0, ws, st))) return rc;
+    } else if ((rc = launch_query_scan(ix, p, L, table, table8, us, cand, n_cand, hi0, ws, st))) {
+        return rc;
+    }
     launch(filter_seed_kernel, dim3((unsigned)filter_split(ix, p), (unsigned)p.B), SEL_THREADS, 0, st, cand, n_cand, ix.doc_off, hi0, p.maxc, theta, p.nq, ready, us, hist, p.n_prune, seed, seed_rng, n_seed,
         (int32_t *)(ws + L.flt_thr), (int32_t *)(ws + L.flt_slot), cut);
     CHIMERA_CUDA(cudaGetLastError());
-    count_launch(SLOT_CI, 4);
+    count_launch(SLOT_CI, 2);                            // (with the thresholds)
     return CHIMERA_OK;
 }
 
