@@ -141,6 +141,7 @@ Layout make_layout(const Index &ix, const Params &p)
     const size_t query_tab = filter ? B * filter_table_pitch(ix) : 0, batch_tab = batch ? batch_table_bytes(ix, p) : 0;
     L.flt_tab = take(query_tab > batch_tab ? query_tab : batch_tab);   // (candidates from the caller are scanned by query)
     L.flt_over = take(batch ? batch_over_bytes(p) : 0);
+    L.flt_mask = take(filter ? B * (size_t)((ix.K + 31) / 32) * sizeof(uint32_t) : 0);
     L.flt_hist = take(filter ? B * (size_t)filter_hist_bins() * sizeof(int32_t) : 0);
     L.flt_thr = take(filter ? B * sizeof(int32_t) : 0);
     L.flt_slot = L.lo;                  // (a call that cuts has no lower bounds, one that does not has no seeds)
@@ -153,6 +154,7 @@ Layout make_layout(const Index &ix, const Params &p)
     L.kept_rng = take(filter ? 2 * two_phase : 0);
     L.n_kept = take(filter ? B * sizeof(int32_t) : 0);
     L.n_seed = take(filter ? B * sizeof(int32_t) : 0);
+    L.n_rest = take(filter ? B * sizeof(int32_t) : 0);
     L.pruned = take(B * p.n_prune * sizeof(int32_t));
     L.ranks = take(ix.tok_id || batch ? B * (size_t)L.words * sizeof(uint2) : 0);
     // retrieved-token scores of the refinements: visit lists, or dense rows per candidate
@@ -406,11 +408,14 @@ static int run(const Index &ix, const Params &p, int first, int last, const floa
                 if ((rc = launch_filter_keep(ix, p, L, cand, n_cand, hi, ci, kept, kept_rng, n_kept, ws, st))) return rc;
                 prof_mark(SLOT_SELECT, st);
                 docs = kept; n_docs = n_kept; docs_rng = kept_rng;
-                // upper bounds of the kept ones from the 8-bit table (lower bounds too where the call turned out not to cut)
+                // upper bounds of the kept ones; where the call turned out not to cut, both bounds of all candidates
                 const FirstCut cut = first_cut(p, L, ws);
-                if ((rc = launch_coarse_bounds(ix, p, (uint8_t *)(ws + L.table8), docs, n_docs, two_phase ? lo : nullptr, hi,
-                                               docs_rng, &cut, st)))
+                const uint8_t *rows8 = (const uint8_t *)(ws + L.table8);
+                if ((rc = launch_kept_bounds(ix, p, rows8, filter_mask_used(ix, p, batch) ? (const uint32_t *)(ws + L.flt_mask) : nullptr,
+                                             (const int32_t *)(ws + L.flt_theta), (const int32_t *)(ws + L.flt_tau), docs_rng, n_docs,
+                                             hi, lo, (int32_t *)(ws + L.n_rest), cut, st)))
                     return rc;
+                if (two_phase && (rc = launch_coarse_bounds(ix, p, rows8, docs, n_docs, lo, hi, docs_rng, &cut, st))) return rc;
                 prof_mark(SLOT_CI, st);
                 if ((rc = launch_filter_contenders(ix, p, L, docs, docs_rng, n_docs, lo, hi, cont, cont_rng, n_cont, ws, st)))
                     return rc;

@@ -110,6 +110,7 @@ struct Layout {
     size_t flt_theta;     // int32  [B][nq]           first cut (g3_filter.cu): thresholds,
     size_t flt_tab;       // uint8  [B][pitch]        one number per centroid (a batch at a time: rows of codes, g3_batch_scan.cu),
     size_t flt_over;      // that form's steps and listed centroids,
+    size_t flt_mask;      // uint32 [B][ceil(K / 32)] centroids with a number above zero,
     size_t flt_hist;      // int32  [B][bins]         histogram of the bounds,
     size_t flt_parts;     // int32  histograms and counters of the threshold kernel's blocks (few queries)
     size_t flt_thr;       // int32  [B]               hi0 from which a candidate is a seed,
@@ -122,6 +123,7 @@ struct Layout {
     size_t kept_rng;      // int2   [B][maxc]         their token ranges
     size_t n_kept;        // int32  [B]
     size_t n_seed;        // int32  [B]
+    size_t n_rest;        // int32  [B]               kept candidates whose first upper bound does not decide
     size_t pruned;        // int32  [B][n_prune]
     size_t ranks;         // uint2  [B][words]        bitmap word, candidates before it (document -> candidate index);
                           //                          only with token lists, or where the first cut scans a batch at a time
@@ -271,11 +273,16 @@ int launch_coarse_table(const Index &ix, const Params &p, const int32_t *table, 
 // head of its scratch rows (int32 [B][maxc]) where launch_contenders will use them.
 int launch_cand_ranges(const Index &ix, const Params &p, const int32_t *cand, const int32_t *n_cand, int2 *rng,
                        int32_t *cont_scratch, cudaStream_t st);
-// rng: those ranges (may be NULL: per-document offset lookups instead; (CI, 0) stands for a document whose exact CI is
-// known).  lo may be NULL with ranges.  cut (may be NULL, else with ranges): a call that cuts wants no lower
-// bounds, one that does not knows no document's CI.
+// rng: those ranges (may be NULL: per-document offset lookups instead).  cut (may be NULL, else with ranges): a call that cuts
+// does nothing here.
 int launch_coarse_bounds(const Index &ix, const Params &p, const uint8_t *table8, const int32_t *cand,
                          const int32_t *n_cand, int32_t *lo, int32_t *hi, const int2 *rng, const FirstCut *cut, cudaStream_t st);
+// Upper bounds of what a call that cuts has kept.  mask: [B][ceil(K / 32)] bits of the centroids near a query token, or NULL;
+// theta, tau: the cut's.  rng: token ranges; (CI, 0) stands for a document whose exact CI is known.  rest: int32 [B][maxc] scratch,
+// n_rest: int32 [B], zero before.
+int launch_kept_bounds(const Index &ix, const Params &p, const uint8_t *table8, const uint32_t *mask, const int32_t *theta,
+                       const int32_t *tau, const int2 *rng, const int32_t *n_docs, int32_t *hi, int32_t *rest, int32_t *n_rest,
+                       const FirstCut &cut, cudaStream_t st);
 // First cut of the candidates by an upper bound from one number per token (g3_filter.cu).  launch_filter_scan leaves the
 // bounds in hi0 and the best ~2 n_prune candidates in seed / seed_rng (their number in the workspace's n_seed);
 // launch_filter_keep takes the seeds' exact CI and writes the candidates that can still be in the top n_prune, ascending;
@@ -284,6 +291,7 @@ int launch_coarse_bounds(const Index &ix, const Params &p, const uint8_t *table8
 constexpr int CUT_QUERIES = 16, CUT_SAMPLES = 4096;
 FirstCut first_cut(const Params &p, const Layout &L, char *ws);
 bool filter_used(const Index &ix, const Params &p);
+bool filter_mask_used(const Index &ix, const Params &p, bool batch);      // the masks are written
 bool batch_scan_used(const Index &ix, const Params &p);       // ... and scans for all queries at once (g3_batch_scan.cu)
 size_t batch_table_bytes(const Index &ix, const Params &p);
 size_t batch_over_bytes(const Params &p);

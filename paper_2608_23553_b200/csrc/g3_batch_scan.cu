@@ -79,11 +79,12 @@ __device__ __forceinline__ void list_over(int32_t *n_over, int2 *over, int b, in
     if (at < BS_OVER) over[(int64_t)b * BS_OVER + at] = make_int2((int)c, (int)rest);
 }
 
-// e(c) of a row of the exact table, on all lanes of a warp (lane = column), in units of 2^us, rounded up.
+// e(c) of a row of the exact table, on all lanes of a warp (lane = column), in units of 2^us, rounded up.  (A score that reaches
+// theta counts, so that zero means a centroid with none.)
 __device__ __forceinline__ uint32_t exact_row_excess(const int32_t *row, int nq, const int32_t *th, int us, int lane)
 {
     int e = 0;
-    for (int w = lane; w < nq; w += 32) e += max(__ldg(row + w) - (th[w] << 16), 0);
+    for (int w = lane; w < nq; w += 32) e += max(__ldg(row + w) - ((th[w] << 16) - 1), 0);
     return ((uint32_t)__reduce_add_sync(0xffffffffu, e) + ((1u << us) - 1)) >> us;       // (127 columns: below 2^31)
 }
 
@@ -140,7 +141,7 @@ batch_quantum_kernel(const int32_t *__restrict__ table, const uint8_t *__restric
             for (int u = 0; u < 8; ++u) {
                 e[u] = 0;
 #pragma unroll
-                for (int w = 0; w < 4; ++w) e[u] += max(v[u][w] - (lane + 32 * w < nq ? s_th[lane + 32 * w] << 16 : 0), 0);
+                for (int w = 0; w < 4; ++w) e[u] += max(v[u][w] - (lane + 32 * w < nq ? (s_th[lane + 32 * w] << 16) - 1 : 0), 0);
                 e[u] = __reduce_add_sync(0xffffffffu, e[u]) >> 16;
                 if (lane == 0 && r0 + 32 * u < m) atomicAdd(&hist[e[u] < SEL_THREADS ? e[u] : SEL_THREADS - 1], 1);
             }
@@ -167,7 +168,7 @@ template <int WORDS, int CW>
 __global__ void __launch_bounds__(BS_THREADS)
 batch_excess_kernel(const uint8_t *__restrict__ table8, int64_t K, int B, int group, const int32_t *__restrict__ theta,
                     const int2 *__restrict__ scale, uint32_t *__restrict__ out, int32_t *__restrict__ n_over,
-                    int2 *__restrict__ over, FirstCut cut)
+                    int2 *__restrict__ over, uint32_t *__restrict__ mask, FirstCut cut)
 {
     pdl_entry();
     constexpr int NQ = 4 * WORDS, ROWS = BS_THREADS / CW, QB = 4 * CW;
@@ -201,21 +202,24 @@ batch_excess_kernel(const uint8_t *__restrict__ table8, int64_t K, int B, int gr
     for (int64_t c0 = (int64_t)blockIdx.x * ROWS; c0 <= K; c0 += (int64_t)gridDim.x * ROWS, buf ^= 1) {
         const int64_t c = c0 + row;
         uint32_t packed = 0;
-        if (c < K) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int b = first + k;
-                if (b >= B) break;
+        for (int k = 0; k < 4; ++k) {
+            const int b = first + k;
+            if (b >= B) break;                               // (the same for all lanes)
+            uint32_t e = 0;
+            if (c < K) {
                 const uint4 *src = reinterpret_cast<const uint4 *>(table8 + ((int64_t)b * K + c) * NQ);
-                const uint32_t e = (uint32_t)filter_row_excess<WORDS>(src, tm1[q0 + k], s_sum[q0 + k]);
-                const uint32_t step = s_step[q0 + k];
-                uint32_t code = code_of(e, step, s_inv[q0 + k]);
-                if (code > BS_TOP) {
-                    code = BS_TOP;
-                    list_over(n_over, over, b, c, e - BS_TOP * step);
-                }
-                packed |= code << code_shift(k);
+                e = (uint32_t)filter_row_excess<WORDS>(src, tm1[q0 + k], s_sum[q0 + k]);
             }
+            const uint32_t near = __ballot_sync(0xffffffffu, e > 0);
+            if ((threadIdx.x & 31) == 0 && c < K) mask[(int64_t)b * ((K + 31) / 32) + (c >> 5)] = near;
+            const uint32_t step = s_step[q0 + k];
+            uint32_t code = code_of(e, step, s_inv[q0 + k]);
+            if (code > BS_TOP) {
+                code = BS_TOP;
+                list_over(n_over, over, b, c, e - BS_TOP * step);
+            }
+            packed |= code << code_shift(k);
         }
         s_word[buf][row][word] = packed;
         __syncthreads();                                     // (the other buffer's readers are past the barrier before)
@@ -230,7 +234,7 @@ template <int NQW>
 __global__ void __launch_bounds__(BS_THREADS)
 batch_excess_exact_kernel(const int32_t *__restrict__ table, int64_t K, int nq, int B, int group, const int32_t *__restrict__ theta,
                           int us, const int2 *__restrict__ scale, uint8_t *__restrict__ table8, uint32_t *__restrict__ out,
-                          int32_t *__restrict__ n_over, int2 *__restrict__ over)
+                          int32_t *__restrict__ n_over, int2 *__restrict__ over, uint8_t *__restrict__ mask)
 {
     pdl_entry();
     constexpr int PER = 8, pitch8 = 32 * NQW;
@@ -244,7 +248,7 @@ batch_excess_exact_kernel(const int32_t *__restrict__ table, int64_t K, int nq, 
     uint8_t *t8 = table8 + row0 * pitch8;
     int th[NQW];
 #pragma unroll
-    for (int w = 0; w < NQW; ++w) th[w] = live && lane + 32 * w < nq ? theta[(int64_t)b * nq + lane + 32 * w] << 16 : 0;
+    for (int w = 0; w < NQW; ++w) th[w] = live && lane + 32 * w < nq ? (theta[(int64_t)b * nq + lane + 32 * w] << 16) - 1 : 0;
     const uint32_t step = live ? (uint32_t)scale[b].y : 1u, inv = step_inverse(step);
     const int64_t groups = (K + 1 + PER - 1) / PER;
     int buf = 0;
@@ -274,13 +278,15 @@ batch_excess_exact_kernel(const int32_t *__restrict__ table, int64_t K, int nq, 
                 else if constexpr (NQW == 2) reinterpret_cast<uint16_t *>(row)[lane] = (uint16_t)coarse[r];
                 else reinterpret_cast<uint32_t *>(row)[lane] = coarse[r];
             }
-        uint32_t mine = 0;
+        uint32_t mine = 0, near = 0;
 #pragma unroll
         for (int r = 0; r < PER; ++r) {
             // the sum of 127 columns stays below 2^31; + the rounding, so add in unsigned
             const uint32_t s = ((uint32_t)__reduce_add_sync(0xffffffffu, e[r]) + ((1u << us) - 1)) >> us;
+            near |= (uint32_t)(s > 0) << r;
             if (lane == r) mine = s;
         }
+        if (live && lane == 0 && gr * PER < K) mask[(int64_t)b * ((K + 31) / 32) * 4 + gr] = (uint8_t)near;
         if (lane < PER) {
             uint32_t code = code_of(mine, step, inv);
             if (code > BS_TOP) {
@@ -616,22 +622,22 @@ static void launch_scan(const Index &ix, const Params &p, const uint32_t *tab, c
 }
 template <int WORDS, int CW>
 static void launch_excess(const Index &ix, const Params &p, const uint8_t *table8, const int32_t *theta, const BatchScratch &s,
-                          uint32_t *tab, FirstCut cut, cudaStream_t st)
+                          uint32_t *tab, uint32_t *mask, FirstCut cut, cudaStream_t st)
 {
     const int gy = batch_groups(p) * batch_group(p) / 4 / CW, rows = BS_THREADS / CW;
     int64_t gx = (8LL * ix.sm_count + gy - 1) / gy;
     if (gx > (ix.K + rows) / rows) gx = (ix.K + rows) / rows;
     launch(batch_excess_kernel<WORDS, CW>, dim3((unsigned)gx, (unsigned)gy), BS_THREADS, 0, st, table8, ix.K, p.B, batch_group(p), theta,
-           s.scale, tab, s.n_over, s.over, cut);
+           s.scale, tab, s.n_over, s.over, mask, cut);
 }
 template <int WORDS>
 static void launch_excess(const Index &ix, const Params &p, const uint8_t *table8, const int32_t *theta, const BatchScratch &s,
-                          uint32_t *tab, FirstCut cut, cudaStream_t st)
+                          uint32_t *tab, uint32_t *mask, FirstCut cut, cudaStream_t st)
 {
     const int group = batch_group(p);
-    if (group == 8) launch_excess<WORDS, 2>(ix, p, table8, theta, s, tab, cut, st);
-    else if (group == 16) launch_excess<WORDS, 4>(ix, p, table8, theta, s, tab, cut, st);
-    else launch_excess<WORDS, 8>(ix, p, table8, theta, s, tab, cut, st);
+    if (group == 8) launch_excess<WORDS, 2>(ix, p, table8, theta, s, tab, mask, cut, st);
+    else if (group == 16) launch_excess<WORDS, 4>(ix, p, table8, theta, s, tab, mask, cut, st);
+    else launch_excess<WORDS, 8>(ix, p, table8, theta, s, tab, mask, cut, st);
 }
 
 int launch_batch_scan(const Index &ix, const Params &p, const Layout &L, const int32_t *table, uint8_t *table8, int us,
@@ -641,20 +647,20 @@ int launch_batch_scan(const Index &ix, const Params &p, const Layout &L, const i
     const int32_t *theta = (const int32_t *)(ws + L.flt_theta);
     const FirstCut cut = first_cut(p, L, ws);
     const uint2 *ranks = (const uint2 *)(ws + L.ranks);
-    uint32_t *tab = (uint32_t *)(ws + L.flt_tab);
+    uint32_t *tab = (uint32_t *)(ws + L.flt_tab), *mask = (uint32_t *)(ws + L.flt_mask);
     const int group = batch_group(p);
     const bool wide = coarse_supported(p.nq);
     if (p.nq == 32) {
-        launch_excess<8>(ix, p, table8, theta, s, tab, cut, st);
+        launch_excess<8>(ix, p, table8, theta, s, tab, mask, cut, st);
     } else if (p.nq == 64) {
-        launch_excess<16>(ix, p, table8, theta, s, tab, cut, st);
+        launch_excess<16>(ix, p, table8, theta, s, tab, mask, cut, st);
     } else {
         const int gy = batch_groups(p) * group / 8;
         int64_t gx = (8LL * ix.sm_count + gy - 1) / gy;
         if (gx > (ix.K + 8) / 8) gx = (ix.K + 8) / 8;
         launch(p.nq <= 32 ? batch_excess_exact_kernel<1> : p.nq <= 64 ? batch_excess_exact_kernel<2> : batch_excess_exact_kernel<4>,
                dim3((unsigned)gx, (unsigned)gy), BS_THREADS, 0, st, table, ix.K, p.nq, p.B, group, theta, us, s.scale, table8, tab,
-               s.n_over, s.over);
+               s.n_over, s.over, (uint8_t *)mask);
     }
     CHIMERA_CUDA(cudaGetLastError());
     auto scan = group == 8     ? launch_scan<1, 2, 1, 4>

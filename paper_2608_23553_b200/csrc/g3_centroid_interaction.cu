@@ -438,11 +438,12 @@ cand_range_kernel(const int32_t *__restrict__ cand, const int32_t *__restrict__ 
 // load), the ranges are handed out by shuffle, and while document i is scanned the first centroid ids of document
 // i + 1 are already being fetched -- a one-level prefetch where the per-document chain used to have three levels.
 // The 32 results of a group are written back coalesced.
-// nq: the columns that count; those up to 16 LPR are zero in every row (lower bounds are for nq == 16 LPR only).
+// nq: the columns that count; those up to 16 LPR are zero in every row.  list (may be NULL): the places of the ranges to take.
+// lo may be NULL (and has to be where nq < 16 LPR).
 template <int LPR>
 __device__ __forceinline__ void
 ci_coarse_rng_body(const uint8_t *__restrict__ table8, int64_t K, int nq, const int2 *__restrict__ rng,
-                     const int32_t *__restrict__ n_cand, int64_t maxc, const int32_t *__restrict__ cids,
+                     const int32_t *__restrict__ list, const int32_t *__restrict__ n_cand, int64_t maxc, const int32_t *__restrict__ cids,
                      int32_t *__restrict__ lo, int32_t *__restrict__ hi)
 {
     constexpr int NQ = 16 * LPR;
@@ -468,7 +469,8 @@ ci_coarse_rng_body(const uint8_t *__restrict__ table8, int64_t K, int nq, const 
 
     for (int jb = j_begin; jb < j_end; jb += 32) {
         const int cnt = j_end - jb < 32 ? j_end - jb : 32;
-        int2 mine = lane < cnt ? rb[jb + lane] : make_int2(0, 1);
+        const int place = lane >= cnt ? 0 : list ? list[(int64_t)b * maxc + jb + lane] : jb + lane;
+        int2 mine = lane < cnt ? rb[place] : make_int2(0, 1);
         int my_lo = 0, my_hi = 0;
         if (mine.y == 0) {                             // its exact CI is known: both bounds
             my_lo = my_hi = mine.x;
@@ -571,53 +573,211 @@ ci_coarse_rng_body(const uint8_t *__restrict__ table8, int64_t K, int nq, const 
             }
         }
         if (lane < cnt) {
-            if (lo) lo[(int64_t)b * maxc + jb + lane] = my_lo;
-            hi[(int64_t)b * maxc + jb + lane] = my_hi;
+            if (lo) lo[(int64_t)b * maxc + place] = my_lo;
+            hi[(int64_t)b * maxc + place] = my_hi;
         }
     }
 }
 
-// cut: of a call that may cut (kept not NULL): no lower bounds when it does; otherwise, with cut_only, nothing is done.
-// Two launch forms of the scan.  32-byte rows: no occupancy hint (the compiler's own 64 registers, four blocks per SM;
-// any hint measured slower).  64-byte rows: four blocks per SM instead of the three that the unhinted 75 registers
-// give (long-document corpus: 27.1 against 28.4 ms).
-template <int LPR>
-__global__ void __launch_bounds__(CI_THREADS)
-ci_coarse_rng_kernel(const uint8_t *__restrict__ table8, int64_t K, const int2 *__restrict__ rng,
-                     const int32_t *__restrict__ n_cand, int64_t maxc, const int32_t *__restrict__ cids,
-                     int32_t *__restrict__ lo, int32_t *__restrict__ hi, FirstCut cut, bool cut_only)
-{
-    pdl_entry();
-    if (cut.kept) {
-        if (cut.on()) lo = nullptr;
-        else if (cut_only) return;
-    }
-    ci_coarse_rng_body<LPR>(table8, K, 16 * LPR, rng, n_cand, maxc, cids, lo, hi);
-}
+// cut: of a call that may cut (kept not NULL): nothing is done when it does (ci_bound_kernel has the bounds then).
+// Four blocks per SM, that is 64 registers: 64-byte rows would take 75 (long-document corpus: 27.1 against 28.4 ms), 32-byte rows
+// 48, with fewer loads in flight (one query, 190,000 documents: 219 against 245 us).
 template <int LPR>
 __global__ void __launch_bounds__(CI_THREADS, 4)
-ci_coarse_rng_kernel_b4(const uint8_t *__restrict__ table8, int64_t K, const int2 *__restrict__ rng,
-                        const int32_t *__restrict__ n_cand, int64_t maxc, const int32_t *__restrict__ cids,
-                        int32_t *__restrict__ lo, int32_t *__restrict__ hi, FirstCut cut, bool cut_only)
+ci_coarse_rng_kernel(const uint8_t *__restrict__ table8, int64_t K, const int2 *__restrict__ rng,
+                     const int32_t *__restrict__ n_cand, int64_t maxc, const int32_t *__restrict__ cids,
+                     int32_t *__restrict__ lo, int32_t *__restrict__ hi, FirstCut cut)
 {
     pdl_entry();
-    if (cut.kept) {
-        if (cut.on()) lo = nullptr;
-        else if (cut_only) return;
+    if (cut.kept && cut.on()) return;
+    ci_coarse_rng_body<LPR>(table8, K, 16 * LPR, rng, nullptr, n_cand, maxc, cids, lo, hi);
+}
+// Upper bounds of what the first cut keeps, from the rows of few tokens.  A centroid counts as near when its score reaches
+// theta_i for some query token i (mask: a bit per centroid).  The others cannot raise a column's maximum above theta_i, so
+//     CI(d) <= sum_i max(theta_i, max over the near tokens of S[c_t, i]),
+// and a fifth of the tokens are near (120 tokens, 32 columns, about one token above each threshold).  Documents whose bound
+// reaches tau, one in six, go on to ci_rest_kernel.
+// Measured (all kept documents at once / both kernels): Mid, batch 256, 1,717 us / 988 + 385; 512-token documents, 64 queries of
+// 64 tokens, 1,795 / 856 + 223; 262,144 centroids, batch 256, 4,458 / 2,724 + 1,034.
+// With few rows left to look up the instructions around them count (a document per warp: 1,890 us, 570 instructions each), so four documents share a warp, eight lanes each, those of
+// a group of 32 taken by length: a bit per token from shared memory says whether it is near, near ids are collected in
+// shared memory and their rows looked up 8 / LPR at a time and document.  nq: the columns that count; those up to 16 LPR are
+// zero in every row.  rng: token ranges; (CI, 0) stands for a document whose CI is known.
+constexpr int BOUND_THREADS = 512;
+constexpr int BOUND_LIST = 64, BOUND_PITCH = BOUND_LIST + 8;
+template <int LPR>
+__global__ void __launch_bounds__(BOUND_THREADS, 2)
+ci_bound_kernel(const uint8_t *__restrict__ table8, int64_t K, int nq, const uint32_t *__restrict__ mask, int mask_words,
+                const int32_t *__restrict__ theta, const int32_t *__restrict__ tau, const int2 *__restrict__ rng,
+                const int32_t *__restrict__ n_docs, int64_t maxc, const int32_t *__restrict__ cids, int32_t *__restrict__ hi,
+                int32_t *__restrict__ rest, int32_t *__restrict__ n_rest, FirstCut cut)
+{
+    pdl_entry();
+    constexpr int NQ = 16 * LPR, RPS = 8 / LPR;              // columns of a row, rows per step and document
+    constexpr int NF = LPR;                                  // registers (two columns each) of a lane after the folding
+    constexpr int U = 4;                                     // steps in flight
+    extern __shared__ uint32_t s_mask[];                     // and a zero word for positions past a document's end
+    __shared__ int32_t s_ids[BOUND_THREADS / 32][4][BOUND_PITCH];
+    __shared__ int32_t s_res[BOUND_THREADS / 32][32];
+    __shared__ uint8_t s_ord[BOUND_THREADS / 32][32];
+    const bool on = cut.on();
+    const int b = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int dg = lane >> 3, l8 = lane & 7, grp = l8 / LPR, sub = l8 % LPR;
+    const int n = n_docs[b];
+    const int warps_per_query = gridDim.x * (BOUND_THREADS / 32);
+    const int per_warp = (n + warps_per_query - 1) / warps_per_query;
+    if (!on || (int)blockIdx.x * (BOUND_THREADS / 32) * per_warp >= n) return;
+    for (int i = threadIdx.x; i <= mask_words; i += BOUND_THREADS)
+        s_mask[i] = i == mask_words ? 0u : __ldg(mask + (int64_t)b * mask_words + i);
+    const int32_t nobody = 32 * mask_words, limit = tau[b];
+    const int4 *tb = reinterpret_cast<const int4 *>(table8 + (int64_t)b * K * NQ) + sub;
+    // the fields (see coarse_accumulate2) that this lane holds after the folding, with theta - 1 in the columns
+    uint32_t floor_f[8];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        uint32_t w = 0;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int col = 16 * sub + 4 * k + e;
+            if (col < nq) w |= (uint32_t)(theta[(int64_t)b * nq + col] - 1) << (8 * e);
+        }
+        floor_f[k] = w << 8;
+        floor_f[4 + k] = w;
     }
-    ci_coarse_rng_body<LPR>(table8, K, 16 * LPR, rng, n_cand, maxc, cids, lo, hi);
+    {
+        int nreg = 8;
+#pragma unroll
+        for (int o = 4; o >= LPR; o >>= 1) {
+            nreg >>= 1;
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+                if (r < nreg && (l8 & o)) floor_f[r] = floor_f[r + nreg];
+        }
+    }
+    __syncthreads();
+    int32_t *ids = s_ids[warp][dg];
+    const int2 *rb = rng + (int64_t)b * maxc;
+    const int wq = blockIdx.x * (BOUND_THREADS / 32) + warp;
+    const int j_begin = wq * per_warp < n ? wq * per_warp : n;
+    const int j_end = j_begin + per_warp < n ? j_begin + per_warp : n;
+    for (int jb = j_begin; jb < j_end; jb += 32) {
+        const int cnt_docs = j_end - jb < 32 ? j_end - jb : 32;
+        const int2 mine = lane < cnt_docs ? rb[jb + lane] : make_int2(0, 0);
+        // longest first; documents whose CI is known (no tokens) come last and are not looked at
+        const int key = mine.y << 5 | lane;
+        int rank = 0;
+#pragma unroll
+        for (int i = 0; i < 32; ++i) rank += __shfl_sync(0xffffffffu, key, i) > key ? 1 : 0;
+        __syncwarp();
+        s_ord[warp][rank] = (uint8_t)lane;
+        s_res[warp][lane] = mine.x;
+        __syncwarp();
+        const int todo = __popc(__ballot_sync(0xffffffffu, mine.y > 0));
+        // ids of positions from ... from + 31 of the group's document, `nobody` past its end
+        int32_t id[4];
+        auto load_ids = [&](int t0, int from, int len) {
+            const int32_t *src = cids + DBG_TOK((int64_t)(len > 0 ? t0 : 0)) + from + l8;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) id[k] = from + l8 + 8 * k < len ? DBG_CID(__ldg(src + 8 * k)) : nobody;
+        };
+        int own = s_ord[warp][dg];
+        int t0 = __shfl_sync(0xffffffffu, mine.x, own), len = __shfl_sync(0xffffffffu, mine.y, own);
+        load_ids(t0, 0, len);
+        for (int r = 0; r < todo; r += 4) {
+            const int ownn = s_ord[warp][(r + 4 + dg) & 31];
+            const int t0n = __shfl_sync(0xffffffffu, mine.x, ownn);
+            int lenn = __shfl_sync(0xffffffffu, mine.y, ownn);
+            if (r + 4 >= todo) lenn = 0;
+            const int most = __shfl_sync(0xffffffffu, len, 0);               // (the longest of the four)
+            uint32_t m[8];
+#pragma unroll
+            for (int x = 0; x < 8; ++x) m[x] = 0u;
+            int have = 0;
+            auto rows = [&](int many) {                      // of the collected ids, `many` of the fullest document
+                __syncwarp();
+                for (int s0 = 0; s0 < many; s0 += U * RPS) {
+                    int4 v[U];
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const int k = s0 + u * RPS + grp;
+                        v[u] = make_int4(0, 0, 0, 0);
+                        if (k < have) v[u] = __ldg(tb + (int64_t)ids[k] * LPR);
+                    }
+#pragma unroll
+                    for (int u = 0; u < U; u += 2) coarse_accumulate2(m, v[u], v[u + 1]);
+                }
+                __syncwarp();
+            };
+            int base = 0;
+            do {
+                int32_t cur[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) cur[k] = id[k];
+                base += 32;
+                const bool more = base < most;
+                load_ids(more ? t0 : t0n, more ? base : 0, more ? len : lenn);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const bool near = s_mask[cur[k] >> 5] >> (cur[k] & 31) & 1u;
+                    const uint32_t which = __ballot_sync(0xffffffffu, near) >> (8 * dg) & 0xffu;
+                    if (near) ids[have + __popc(which & ((1u << l8) - 1u))] = cur[k];
+                    have += __popc(which);
+                }
+                const int many = __reduce_max_sync(0xffffffffu, have);
+                if (!more || many > BOUND_LIST - 32) {
+                    rows(many);
+                    have = 0;
+                }
+            } while (base < most);
+            // merge the lanes of a document (same columns, different tokens): each exchange keeps one half of the registers
+            int nreg = 8;
+#pragma unroll
+            for (int o = 4; o >= LPR; o >>= 1) {
+                const int half = nreg >> 1;
+                const bool up = (l8 & o) != 0;
+#pragma unroll
+                for (int x = 0; x < 4; ++x)
+                    if (x < half) {
+                        const uint32_t send = up ? m[x] : m[x + half], keep = up ? m[x + half] : m[x];
+                        m[x] = __vmaxu2(keep, __shfl_xor_sync(0xffffffffu, send, o));
+                    }
+                nreg = half;
+            }
+            int packed = 0;                                  // sum of maxima | saturated << 16
+#pragma unroll
+            for (int x = 0; x < NF; ++x) {
+                const uint32_t f = __vmaxu2(m[x], floor_f[x]);
+                const int u_lo = coarse_field_lo(f), u_hi = coarse_field_hi(f);
+                packed += (u_lo + u_hi) + (((u_lo >= 255) + (u_hi >= 255)) << 16);
+            }
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) packed += __shfl_xor_sync(0xffffffffu, packed, o);      // (127 * 255 < 2^16)
+            if (l8 == 0 && r + dg < todo) s_res[warp][own] = coarse_hi(packed, nq);
+            own = ownn; t0 = t0n; len = lenn;
+        }
+        __syncwarp();
+        const int32_t res = s_res[warp][lane];
+        if (lane < cnt_docs) hi[(int64_t)b * maxc + jb + lane] = res;
+        const bool goes_on = mine.y > 0 && res >= limit;
+        const unsigned which = __ballot_sync(0xffffffffu, goes_on);
+        if (which) {
+            int at = 0;
+            if (lane == 0) at = atomicAdd(&n_rest[b], __popc(which));
+            at = __shfl_sync(0xffffffffu, at, 0);
+            if (goes_on) rest[(int64_t)b * maxc + at + __popc(which & ((1u << lane) - 1u))] = jb + lane;
+        }
+    }
 }
 
-// Other query lengths, rows padded to 32, 64 or 128 bytes (made beside the first cut's excess table): 28 M lookups for 8
-// queries of 100 tokens in 213 us, where the exact rows took 860.
+// The bounds of those documents (places in the list of ranges, in no order; rest NULL: of all) from the rows of all their tokens.
 template <int LPR>
 __global__ void __launch_bounds__(CI_THREADS, LPR == 2 ? 4 : 3)
-ci_coarse_rng_kernel_pad(const uint8_t *__restrict__ table8, int64_t K, int nq, const int2 *__restrict__ rng,
-                         const int32_t *__restrict__ n_cand, int64_t maxc, const int32_t *__restrict__ cids,
-                         int32_t *__restrict__ hi)
+ci_rest_kernel(const uint8_t *__restrict__ table8, int64_t K, int nq, const int2 *__restrict__ rng, const int32_t *__restrict__ rest,
+               const int32_t *__restrict__ n_rest, int64_t maxc, const int32_t *__restrict__ cids, int32_t *__restrict__ hi, FirstCut cut)
 {
     pdl_entry();
-    ci_coarse_rng_body<LPR>(table8, K, nq, rng, n_cand, maxc, cids, nullptr, hi);
+    if (!cut.on()) return;
+    ci_coarse_rng_body<LPR>(table8, K, nq, rng, rest, n_rest, maxc, cids, nullptr, hi);
 }
 
 bool coarse_supported(int nq) { return nq == 32 || nq == 64; }
@@ -648,7 +808,7 @@ int launch_coarse_bounds(const Index &ix, const Params &p, const uint8_t *table8
     const size_t table_bytes = (size_t)ix.K * coarse_pitch(p.nq);
     const bool use_rng = rng != nullptr;
     const FirstCut call_cut = cut ? *cut : FirstCut();
-    const bool small = table_bytes <= 160 * 1024 && lo != nullptr;
+    const bool small = table_bytes <= 160 * 1024;
     if (small) {
         // the whole 8-bit table of a query fits in shared memory: stage it once per block and look rows up there
         constexpr int T = 512;
@@ -673,7 +833,7 @@ int launch_coarse_bounds(const Index &ix, const Params &p, const uint8_t *table8
         }
         CHIMERA_CUDA(cudaGetLastError());
         count_launch(SLOT_CI);
-        if (!cut) return CHIMERA_OK;             // (a cut leaves documents whose CI is known: they are passed over below)
+        return CHIMERA_OK;
     }
     // Blocks per query.  Four blocks are resident per SM and the blocks of a query are adjacent in the grid, so
     // (resident blocks) / (blocks per query) queries are scanned at the same time and their 8-bit tables compete for
@@ -692,15 +852,10 @@ int launch_coarse_bounds(const Index &ix, const Params &p, const uint8_t *table8
     const unsigned gx = (unsigned)per_query;
     dim3 grid(gx, (unsigned)p.B);
     if (use_rng) {
-        if (!coarse_supported(p.nq)) {
-            auto kern = p.nq <= 32 ? ci_coarse_rng_kernel_pad<2> : p.nq <= 64 ? ci_coarse_rng_kernel_pad<4> : ci_coarse_rng_kernel_pad<8>;
-            launch(kern, grid, CI_THREADS, 0, st, table8, ix.K, p.nq, rng, n_cand, p.maxc, ix.cids, hi);
-        } else if (p.nq == 32)
-            launch(ci_coarse_rng_kernel<2>, grid, CI_THREADS, 0, st, table8, ix.K, rng, n_cand, p.maxc, ix.cids, lo, hi, call_cut,
-                   small);
+        if (p.nq == 32)
+            launch(ci_coarse_rng_kernel<2>, grid, CI_THREADS, 0, st, table8, ix.K, rng, n_cand, p.maxc, ix.cids, lo, hi, call_cut);
         else
-            launch(ci_coarse_rng_kernel_b4<4>, grid, CI_THREADS, 0, st, table8, ix.K, rng, n_cand, p.maxc, ix.cids, lo, hi, call_cut,
-                   small);
+            launch(ci_coarse_rng_kernel<4>, grid, CI_THREADS, 0, st, table8, ix.K, rng, n_cand, p.maxc, ix.cids, lo, hi, call_cut);
         CHIMERA_CUDA(cudaGetLastError());
         count_launch(SLOT_CI);
         return CHIMERA_OK;
@@ -711,6 +866,44 @@ int launch_coarse_bounds(const Index &ix, const Params &p, const uint8_t *table8
     else
         launch(ci_coarse_kernel<4, false, CI_THREADS>, grid, CI_THREADS, 0, st, table8, ix.K, cand, n_cand, p.maxc, ix.cids,
                                                                           ix.doc_off, lo, hi, FirstCut());
+    CHIMERA_CUDA(cudaGetLastError());
+    count_launch(SLOT_CI);
+    return CHIMERA_OK;
+}
+
+// Upper bounds of the documents that the first cut keeps (ci_bound_kernel, ci_rest_kernel).  rest: int32 [B][maxc] scratch.
+int launch_kept_bounds(const Index &ix, const Params &p, const uint8_t *table8, const uint32_t *mask, const int32_t *theta,
+                       const int32_t *tau, const int2 *rng, const int32_t *n_docs, int32_t *hi, int32_t *rest, int32_t *n_rest,
+                       const FirstCut &cut, cudaStream_t st)
+{
+    const int64_t want = (p.maxc + CI_WARPS - 1) / CI_WARPS;
+    int64_t gx;
+    if (mask) {
+        // Two blocks are resident per SM, those of a query adjacent in the grid; few blocks per query keep the copies of its mask
+        // few, and sixteen documents or more to a warp, of some six n_prune, find their like in length.
+        const int64_t words = (ix.K + 31) / 32;
+        const size_t smem = (size_t)(words + 1) * 4;
+        gx = (8LL * ix.sm_count + p.B - 1) / p.B;
+        if (gx < ix.sm_count / 4) gx = ix.sm_count / 4;
+        if (gx > 6 * p.n_prune / (BOUND_THREADS / 2)) gx = 6 * p.n_prune / (BOUND_THREADS / 2);
+        if (gx < (2LL * ix.sm_count + p.B - 1) / p.B) gx = (2LL * ix.sm_count + p.B - 1) / p.B;
+        if (gx > (want + 1) / 2) gx = (want + 1) / 2;
+        auto kern = p.nq <= 32 ? ci_bound_kernel<2> : p.nq <= 64 ? ci_bound_kernel<4> : ci_bound_kernel<8>;
+        CHIMERA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        launch(kern, dim3((unsigned)gx, (unsigned)p.B), BOUND_THREADS, smem, st, table8, ix.K, p.nq, mask, (int)words, theta, tau, rng,
+               n_docs, p.maxc, ix.cids, hi, rest, n_rest, cut);
+        CHIMERA_CUDA(cudaGetLastError());
+        count_launch(SLOT_CI);
+        gx = (8LL * ix.sm_count + p.B - 1) / p.B;            // of one or two n_prune documents a query
+        if (gx < p.n_prune / 32) gx = p.n_prune / 32;
+    } else {
+        gx = (8LL * ix.sm_count + p.B - 1) / p.B;
+        if (gx < ix.sm_count / 2) gx = ix.sm_count / 2;
+    }
+    if (gx > want) gx = want;
+    auto rest_kern = p.nq <= 32 ? ci_rest_kernel<2> : p.nq <= 64 ? ci_rest_kernel<4> : ci_rest_kernel<8>;
+    launch(rest_kern, dim3((unsigned)gx, (unsigned)p.B), CI_THREADS, 0, st, table8, ix.K, p.nq, rng, mask ? rest : nullptr,
+           mask ? n_rest : n_docs, p.maxc, ix.cids, hi, cut);
     CHIMERA_CUDA(cudaGetLastError());
     count_launch(SLOT_CI);
     return CHIMERA_OK;

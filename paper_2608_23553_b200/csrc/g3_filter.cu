@@ -15,13 +15,15 @@
 //   filter_theta_kernel    theta_i from a sample of the table's rows
 //   filter_sample_kernel    q_len 32 / 64: whether the cut would drop enough, from sampled candidates; if not, the kernels
 //                          down to the count return at once, all candidates are kept, and their 8-bit bounds decide
-//   filter_excess_kernel   e(c) of every centroid, rounded up (16 bits, or 6-bit codes five to a word for large K)
+//   filter_excess_kernel   e(c) of every centroid, rounded up (16 bits, or 6-bit codes five to a word for large K), and a mask
+//                          of those where it is not zero
 //   filter_scan_kernel     hi0 of every candidate: the query's whole e table in shared memory, one lookup per token
+//                          (batches whose candidates are a good part of the corpus: all queries at once, g3_batch_scan.cu)
 //   filter_seed_kernel     the ~2 n_prune candidates with the largest hi0 (their order does not matter)
 //   (their exact CI: g3_centroid_interaction.cu)
 //   filter_count_kernel,   tau = the n_prune-th largest of those, a lower bound on the n_prune-th largest CI; keeps every
 //   filter_write_kernel    candidate with hi0 >= tau, ascending, with its token range
-//   (upper bounds of the kept ones from the 8-bit table: g3_centroid_interaction.cu)
+//   (upper bounds of the kept ones from the 8-bit table, of few tokens first: g3_centroid_interaction.cu)
 //   filter_contend_kernel  and of those the ones whose bound reaches tau
 //   (exact CI of what is left, except for the seeds, and the exact selection: g3_centroid_interaction.cu)
 // Every document of the exact top n_prune has an upper bound >= CI >= tau, so it is never dropped and the result is the
@@ -79,6 +81,25 @@ double expected_tokens(const Index &ix, const Params &p)
     const double probed = (double)p.nq * p.P / (double)ix.K;
     const double cand = probed < 1.0 ? (double)ix.N * (1.0 - pow(1.0 - probed, distinct)) : (double)ix.N;
     return (cand < (double)p.maxc ? cand : (double)p.maxc) * len;
+}
+// Share of the centroids above each threshold: FILTER_LAMBDA tokens of a document.  Its length is that of the documents that
+// compete for the top: about halfway between the candidates' mean (somewhat above the corpus's: long documents are probed more
+// often) and the longest, outliers aside.
+static double filter_share(const Index &ix)
+{
+    const double mean = (double)ix.T / (double)ix.N, most = (double)ix.max_doclen;
+    const double len = 0.5 * ((1.2 * mean < most ? 1.2 * mean : most) + (2.4 * mean < most ? 2.4 * mean : most));
+    return FILTER_LAMBDA / len;
+}
+// Whether the bounds of what is kept start with the tokens near the query (ci_bound_kernel).  With more than a third of the tokens
+// near, the other columns are too many for a bound that decides: 100 tokens on 100-token documents (half of them near) 405 us,
+// all rows at once 224.  And a document is a chain of lookups whose length does not shrink with the rows: too few of them to
+// hide it, and a second kernel, cost more (one query, 603 survivors: 219 -> 245 us for the call; 37 queries, 777: 55 -> 68 us for the
+// step; 64 queries, 2,048: 1,795 -> 1,079).  (6-bit codes from the exact table come five centroids to a warp: no words of a mask.)
+bool filter_mask_used(const Index &ix, const Params &p, bool batch)
+{
+    return filter_share(ix) * p.nq < 0.4 && (int64_t)p.B * p.n_prune >= 65536 &&
+           (batch || coarse_supported(p.nq) || filter_codec(ix.K) == 16);
 }
 bool filter_used(const Index &ix, const Params &p)
 {
@@ -336,10 +357,11 @@ __device__ __forceinline__ void filter_fill_encoder(uint8_t *enc)
 template <int WORDS, int CODEC>
 __global__ void __launch_bounds__(256)
 filter_excess_kernel(const uint8_t *__restrict__ table8, int64_t K, const int32_t *__restrict__ theta,
-                     uint8_t *__restrict__ out, size_t pitch, FirstCut cut)
+                     uint8_t *__restrict__ out, size_t pitch, uint32_t *__restrict__ mask, FirstCut cut)
 {
     pdl_entry();
     __shared__ uint2 tm1[WORDS];
+    __shared__ uint32_t s_bits[2][CODEC == 6 ? 40 : 1];      // of 256 words of five codes
     __shared__ int s_sum;
     __shared__ uint8_t enc[512];
     const int b = blockIdx.y;
@@ -360,30 +382,52 @@ filter_excess_kernel(const uint8_t *__restrict__ table8, int64_t K, const int32_
     const uint4 *tb = reinterpret_cast<const uint4 *>(table8 + (int64_t)b * K * 4 * WORDS);
     uint8_t *ob = out + (size_t)b * pitch;
     const int sum = s_sum;
+    uint32_t *mb = mask + (int64_t)b * ((K + 31) / 32);
     if (CODEC == 16) {
-        for (int64_t c = (int64_t)blockIdx.x * 256 + threadIdx.x; c < K; c += (int64_t)gridDim.x * 256)
-            reinterpret_cast<uint16_t *>(ob)[c] = (uint16_t)filter_row_excess<WORDS>(tb + c * (WORDS / 4), tm1, sum);
+        for (int64_t c0 = (int64_t)blockIdx.x * 256; c0 < K; c0 += (int64_t)gridDim.x * 256) {
+            const int64_t c = c0 + threadIdx.x;
+            const int e = c < K ? filter_row_excess<WORDS>(tb + c * (WORDS / 4), tm1, sum) : 0;
+            if (c < K) reinterpret_cast<uint16_t *>(ob)[c] = (uint16_t)e;
+            const uint32_t bits = __ballot_sync(0xffffffffu, e > 0);
+            if ((threadIdx.x & 31) == 0 && c < K) mb[c >> 5] = bits;
+        }
     } else {
         const int64_t words = (K + 4) / 5;
-        for (int64_t w = (int64_t)blockIdx.x * 256 + threadIdx.x; w < words; w += (int64_t)gridDim.x * 256) {
-            uint32_t packed = 0;
+        if (threadIdx.x < 40) s_bits[0][threadIdx.x] = 0u;
+        __syncthreads();
+        int buf = 0;
+        for (int64_t w0 = (int64_t)blockIdx.x * 256; w0 < words; w0 += (int64_t)gridDim.x * 256, buf ^= 1) {
+            const int64_t w = w0 + threadIdx.x;
+            if (threadIdx.x < 40) s_bits[buf ^ 1][threadIdx.x] = 0u;
+            if (w < words) {
+                uint32_t packed = 0, bits = 0;
 #pragma unroll
-            for (int r = 0; r < 5; ++r) {
-                const int64_t c = w * 5 + r < K ? w * 5 + r : K - 1;
-                packed |= (uint32_t)filter_encode(enc, filter_row_excess<WORDS>(tb + c * (WORDS / 4), tm1, sum)) << (6 * r + (r > 2));
+                for (int r = 0; r < 5; ++r) {
+                    const int64_t c = w * 5 + r < K ? w * 5 + r : K - 1;
+                    const int e = filter_row_excess<WORDS>(tb + c * (WORDS / 4), tm1, sum);
+                    packed |= (uint32_t)filter_encode(enc, e) << (6 * r + (r > 2));
+                    bits |= (uint32_t)(e > 0) << r;
+                }
+                reinterpret_cast<uint32_t *>(ob)[w] = packed;
+                const int at = 5 * threadIdx.x;
+                atomicOr(&s_bits[buf][at >> 5], bits << (at & 31));
+                if ((at & 31) > 27) atomicOr(&s_bits[buf][(at >> 5) + 1], bits >> (32 - (at & 31)));
             }
-            reinterpret_cast<uint32_t *>(ob)[w] = packed;
+            __syncthreads();                             // (the next round clears and fills the other half)
+            const int64_t mw = w0 * 5 / 32 + threadIdx.x;
+            if (threadIdx.x < 40 && mw < (K + 31) / 32) mb[mw] = s_bits[buf][threadIdx.x];
         }
     }
 }
 
-// The same from the exact table, for any q_len: one warp per row, values rounded up to units of 2^us.  The 8-bit rows that
+// The same from the exact table, for any q_len: one warp per row, values rounded up to units of 2^us (a score that reaches theta
+// counts, so that zero means a centroid with none).  The 8-bit rows that
 // the second bound looks up are made on the way (table8: [B][K][pitch8], a lane's columns side by side, zeros for those
 // past nq: the bound is a sum over columns, whatever their order).
 template <int CODEC, int NQW>      // NQW = pitch8 / 32
 __global__ void __launch_bounds__(256)
 filter_excess_exact_kernel(const int32_t *__restrict__ table, int64_t K, int nq, const int32_t *__restrict__ theta, int us,
-                           uint8_t *__restrict__ table8, uint8_t *__restrict__ out, size_t pitch)
+                           uint8_t *__restrict__ table8, uint8_t *__restrict__ out, size_t pitch, uint8_t *__restrict__ mask)
 {
     pdl_entry();
     __shared__ uint8_t enc[512];
@@ -393,7 +437,7 @@ filter_excess_exact_kernel(const int32_t *__restrict__ table, int64_t K, int nq,
     uint8_t *t8 = table8 + (int64_t)b * K * pitch8;
     int th[NQW];
 #pragma unroll
-    for (int w = 0; w < NQW; ++w) th[w] = lane + 32 * w < nq ? theta[(int64_t)b * nq + lane + 32 * w] << 16 : 0;
+    for (int w = 0; w < NQW; ++w) th[w] = lane + 32 * w < nq ? (theta[(int64_t)b * nq + lane + 32 * w] << 16) - 1 : 0;
     const int32_t *tb = table + (int64_t)b * K * nq;
     uint8_t *ob = out + (size_t)b * pitch;
     constexpr int PER = CODEC == 16 ? 8 : 5;                          // rows per warp and iteration
@@ -423,17 +467,19 @@ filter_excess_exact_kernel(const int32_t *__restrict__ table, int64_t K, int nq,
             else if constexpr (NQW == 2) reinterpret_cast<uint16_t *>(row)[lane] = (uint16_t)coarse[r];
             else reinterpret_cast<uint32_t *>(row)[lane] = coarse[r];
         }
-        uint32_t packed = 0;
+        uint32_t packed = 0, near = 0;
         int val = 0;
 #pragma unroll
         for (int r = 0; r < PER; ++r) {
             // the sum of 127 columns stays below 2^31; + the rounding, so add in unsigned
             const uint32_t s = ((uint32_t)__reduce_add_sync(0xffffffffu, e[r]) + ((1u << us) - 1)) >> us;
+            near |= (uint32_t)(s > 0) << r;
             if (CODEC == 16) { if (lane == r) val = (int)s; }
             else packed |= (uint32_t)filter_encode(enc, (int)s) << (6 * r + (r > 2));
         }
         if (CODEC == 16) {
             if (lane < PER && g * PER + lane < K) reinterpret_cast<uint16_t *>(ob)[g * PER + lane] = (uint16_t)val;
+            if (lane == 0) mask[(int64_t)b * ((K + 31) / 32) * 4 + g] = (uint8_t)near;
         } else if (lane == 0) {
             reinterpret_cast<uint32_t *>(ob)[g] = packed;
         }
@@ -613,16 +659,13 @@ filter_scan_kernel(const uint8_t *__restrict__ tab, size_t pitch, const int32_t 
 // A Q.24 threshold in units of 2^us, rounded up (hi0 is a whole number of them).
 __device__ __forceinline__ int32_t units_up(int32_t tau, int us) { return (int32_t)(((long long)tau + (1 << us) - 1) >> us); }
 
-// grid (split, B): candidates with the largest hi0, 2 n_prune of them (wide: q_len 32 or 64, whose exact rows are read in
-// 16-byte pieces) or 1.5 n_prune (other lengths, where an exact row costs three to four times its 8-bit copy: 37 queries of
-// 21 tokens 1,255 against 1,309 us; on the wide ones 1.5 costs more in the later cuts than it saves) and the rest of the
-// last histogram bin, with their token ranges, in no particular order; seed_thr[b] = the hi0 they
-// start at, seed_slot[candidate] = where each one went.  n_seed (cleared before) stays 0 when a query has so few
-// candidates that all are kept.
+// grid (split, B): candidates with the largest hi0, `want` of them and the rest of the last histogram bin, with their token
+// ranges, in no particular order; seed_thr[b] = the hi0 they start at, seed_slot[candidate] = where each one went.  n_seed
+// (cleared before) stays 0 when a query has so few candidates that all are kept.
 __global__ void __launch_bounds__(SEL_THREADS)
 filter_seed_kernel(const int32_t *__restrict__ cand, const int32_t *__restrict__ n_cand, const int64_t *__restrict__ doc_off,
-                   const int32_t *__restrict__ hi0, int64_t maxc, const int32_t *__restrict__ theta, int nq, bool wide, int us,
-                   const int32_t *__restrict__ hist, int n_prune, int32_t *__restrict__ seed,
+                   const int32_t *__restrict__ hi0, int64_t maxc, const int32_t *__restrict__ theta, int nq, int us,
+                   const int32_t *__restrict__ hist, int want, int32_t *__restrict__ seed,
                    int2 *__restrict__ seed_rng, int32_t *__restrict__ n_seed, int32_t *__restrict__ seed_thr,
                    int32_t *__restrict__ seed_slot, FirstCut cut)
 {
@@ -632,7 +675,6 @@ filter_seed_kernel(const int32_t *__restrict__ cand, const int32_t *__restrict__
     const bool on = cut.on();
     const int b = blockIdx.y, n = n_cand[b];
     if (!on) return;                                     // (no seeds: n_seed is 0)
-    const int want = (wide ? 2 * n_prune : n_prune + n_prune / 2) + 32;
     if (n <= want) {
         if (blockIdx.x == 0 && threadIdx.x == 0) seed_thr[b] = INT_MAX;
         return;
@@ -767,7 +809,7 @@ __device__ __forceinline__ int block_count(const int32_t *__restrict__ v, int j0
 __global__ void __launch_bounds__(SEL_THREADS)
 filter_count_kernel(const int32_t *__restrict__ n_cand, const int32_t *__restrict__ hi0, int64_t maxc,
                     const int32_t *__restrict__ seed_ci, const int32_t *__restrict__ n_seed, int n_prune, int us,
-                    int32_t *__restrict__ tau_out, int32_t *__restrict__ counts, FirstCut cut)
+                    int32_t *__restrict__ tau_out, int32_t *__restrict__ counts, int32_t *__restrict__ n_rest, FirstCut cut)
 {
     pdl_entry();
     __shared__ int hist[2048];
@@ -791,7 +833,10 @@ filter_count_kernel(const int32_t *__restrict__ n_cand, const int32_t *__restric
     const int total = block_count(hi0 + (int64_t)b * maxc, j0, j1, units_up(tau, us), warp_part);
     if (threadIdx.x == 0) {
         counts[(int64_t)b * KEEP_SPLIT + blockIdx.x] = total;
-        if (blockIdx.x == 0) tau_out[b] = tau;
+        if (blockIdx.x == 0) {
+            tau_out[b] = tau;
+            n_rest[b] = 0;                               // (counted up by the bounds of what is kept)
+        }
     }
 }
 
@@ -905,6 +950,7 @@ static int launch_query_scan(const Index &ix, const Params &p, const Layout &L, 
     int32_t *theta = (int32_t *)(ws + L.flt_theta), *hist = (int32_t *)(ws + L.flt_hist);
     const FirstCut cut = first_cut(p, L, ws);
     uint8_t *tab = (uint8_t *)(ws + L.flt_tab);
+    uint32_t *mask = (uint32_t *)(ws + L.flt_mask);
     const bool ready = coarse_supported(p.nq);           // stage 1 has written the 8-bit table
     const int codec = filter_codec(ix.K);
     const size_t pitch = filter_table_pitch(ix);
@@ -913,10 +959,10 @@ static int launch_query_scan(const Index &ix, const Params &p, const Layout &L, 
         const int64_t want = ((codec == 16 ? ix.K : (ix.K + 4) / 5) + 255) / 256;
         if (gx > want) gx = want;
         const dim3 grid((unsigned)gx, (unsigned)p.B);
-        if (p.nq == 32 && codec == 16) launch(filter_excess_kernel<8, 16>, grid, 256, 0, st, table8, ix.K, theta, tab, pitch, cut);
-        else if (p.nq == 32) launch(filter_excess_kernel<8, 6>, grid, 256, 0, st, table8, ix.K, theta, tab, pitch, cut);
-        else if (codec == 16) launch(filter_excess_kernel<16, 16>, grid, 256, 0, st, table8, ix.K, theta, tab, pitch, cut);
-        else launch(filter_excess_kernel<16, 6>, grid, 256, 0, st, table8, ix.K, theta, tab, pitch, cut);
+        if (p.nq == 32 && codec == 16) launch(filter_excess_kernel<8, 16>, grid, 256, 0, st, table8, ix.K, theta, tab, pitch, mask, cut);
+        else if (p.nq == 32) launch(filter_excess_kernel<8, 6>, grid, 256, 0, st, table8, ix.K, theta, tab, pitch, mask, cut);
+        else if (codec == 16) launch(filter_excess_kernel<16, 16>, grid, 256, 0, st, table8, ix.K, theta, tab, pitch, mask, cut);
+        else launch(filter_excess_kernel<16, 6>, grid, 256, 0, st, table8, ix.K, theta, tab, pitch, mask, cut);
     } else {
         const int64_t want = (ix.K + 39) / 40;
         if (gx > want) gx = want;
@@ -927,7 +973,7 @@ static int launch_query_scan(const Index &ix, const Params &p, const Layout &L, 
                                 : (p.nq <= 32   ? filter_excess_exact_kernel<6, 1>
                                    : p.nq <= 64 ? filter_excess_exact_kernel<6, 2>
                                                 : filter_excess_exact_kernel<6, 4>);
-        launch(kern, grid, 256, 0, st, table, ix.K, p.nq, theta, us, table8, tab, pitch);
+        launch(kern, grid, 256, 0, st, table, ix.K, p.nq, theta, us, table8, tab, pitch, (uint8_t *)mask);
     }
     CHIMERA_CUDA(cudaGetLastError());
 
@@ -963,11 +1009,7 @@ int launch_filter_scan(const Index &ix, const Params &p, const Layout &L, bool b
     const int codec = filter_codec(ix.K);
     const int step = (int)(ix.K / FILTER_SAMPLE > 1 ? ix.K / FILTER_SAMPLE : 1);
     const int m = (int)((ix.K + step - 1) / step < 2 * FILTER_SAMPLE ? (ix.K + step - 1) / step : 2 * FILTER_SAMPLE);
-    // the length of the documents that compete for the top: about halfway between the candidates' mean (somewhat above
-    // the corpus's: long documents are probed more often) and the longest, outliers aside
-    const double mean = (double)ix.T / (double)ix.N, most = (double)ix.max_doclen;
-    const double len = 0.5 * ((1.2 * mean < most ? 1.2 * mean : most) + (2.4 * mean < most ? 2.4 * mean : most));
-    int rank = (int)(FILTER_LAMBDA / len * m + 0.5);
+    int rank = (int)(filter_share(ix) * m + 0.5);
     if (rank < 1) rank = 1;
     const unsigned groups = (unsigned)((p.nq + 31) / 32);
     const int parts = filter_parts(ix, p);
@@ -995,7 +1037,10 @@ int launch_filter_scan(const Index &ix, const Params &p, const Layout &L, bool b
     } else if ((rc = launch_query_scan(ix, p, L, table, table8, us, cand, n_cand, hi0, ws, st))) {
         return rc;
     }
-    launch(filter_seed_kernel, dim3((unsigned)filter_split(ix, p), (unsigned)p.B), SEL_THREADS, 0, st, cand, n_cand, ix.doc_off, hi0, p.maxc, theta, p.nq, ready, us, hist, p.n_prune, seed, seed_rng, n_seed,
+    // 2 n_prune for q_len 32 / 64, whose exact rows are read in 16-byte pieces (Mid, batch 256: 1.5 n_prune 6,641 us, 2 6,419, 2.5
+    // 6,437), 1.5 n_prune for others, where an exact row costs three to four times its 8-bit copy (37 queries of 21 tokens: 1.5
+    // 1,047 us, 2.5 1,148)
+    launch(filter_seed_kernel, dim3((unsigned)filter_split(ix, p), (unsigned)p.B), SEL_THREADS, 0, st, cand, n_cand, ix.doc_off, hi0, p.maxc, theta, p.nq, us, hist, (ready ? 2 * p.n_prune : p.n_prune + p.n_prune / 2) + 32, seed, seed_rng, n_seed,
         (int32_t *)(ws + L.flt_thr), (int32_t *)(ws + L.flt_slot), cut);
     CHIMERA_CUDA(cudaGetLastError());
     count_launch(SLOT_CI, 2);                            // (with the thresholds)
@@ -1013,7 +1058,8 @@ int launch_filter_keep(const Index &ix, const Params &p, const Layout &L, const 
     const FirstCut cut = first_cut(p, L, ws);
     const int32_t *thr = (const int32_t *)(ws + L.flt_thr), *slot = (const int32_t *)(ws + L.flt_slot);
     const dim3 grid((unsigned)filter_split(ix, p), (unsigned)p.B);
-    launch(filter_count_kernel, grid, SEL_THREADS, 0, st, n_cand, hi0, p.maxc, seed_ci, n_seed, p.n_prune, us, tau, counts, cut);
+    launch(filter_count_kernel, grid, SEL_THREADS, 0, st, n_cand, hi0, p.maxc, seed_ci, n_seed, p.n_prune, us, tau, counts,
+           (int32_t *)(ws + L.n_rest), cut);
     CHIMERA_CUDA(cudaGetLastError());
     launch(filter_write_kernel, grid, SEL_THREADS, 0, st, cand, n_cand, ix.doc_off, hi0, p.maxc, thr, slot, seed_ci, tau, us,
                                                       counts, kept, kept_rng, n_kept, cut);

@@ -54,7 +54,7 @@ def check(arrays, q, nprobe, n_prune, cut=True):
         kept = np.array(gix.kept(B, nq, nprobe, n_prune, k))
         assert kept.sum() < 0.8 * tn["n_cand"].sum() and (kept <= tn["n_cand"]).all()
     ids, sc = ids.cpu().numpy(), sc.cpu().numpy()
-    for b in sorted({0, 1, 7, B // 2, B - 1}):
+    for b in sorted({0, 1, B // 3, B // 2, B - 1}):
         res = oracle.pipeline(q[b], oix, nprobe, n_prune, k)
         check_query(tn, b, res, ids[b], sc[b], k, n_prune, table=False)
     return gix, tn
