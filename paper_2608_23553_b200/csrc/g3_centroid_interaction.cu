@@ -31,8 +31,9 @@ constexpr int CI_THREADS = 256;
 constexpr int CI_WARPS = CI_THREADS / 32;
 
 // Any q_len.  rng: NULL, or the documents' token ranges (first token, length); (CI, 0) stands for a document whose CI is
-// known.  L2 is the limit (rows of 84 bytes, 59,000 documents of 173 tokens: 1.1 GB of sectors in 332 us); the next 32
-// centroid ids are loaded ahead of the rows.
+// known.  Instructions are the limit (21 a row, with a 64-bit product and a predicate for each, took 271 us for 8.3 million rows of 84
+// bytes at 65 % of the issue rate), so a row's address is one 32 x 32-bit multiply-add and lanes past the last column read that one
+// again instead of nothing.  The next 32 centroid ids are loaded ahead of the rows.
 template <int NQW>   // 32-column groups handled per lane
 __global__ void __launch_bounds__(CI_THREADS)
 ci_kernel(const int32_t *__restrict__ table, int64_t K, int nq, const int32_t *__restrict__ cand,
@@ -44,7 +45,11 @@ ci_kernel(const int32_t *__restrict__ table, int64_t K, int nq, const int32_t *_
     const int b = blockIdx.y;
     const int lane = threadIdx.x & 31;
     const int n = n_cand[b];
-    const int32_t *tb = table + (int64_t)b * K * nq;
+    const char *col[NQW];                                    // this lane's columns of row 0
+    const uint32_t row_bytes = 4u * (uint32_t)nq;
+#pragma unroll
+    for (int w = 0; w < NQW; ++w)
+        col[w] = reinterpret_cast<const char *>(table + (int64_t)b * K * nq + (lane + 32 * w < nq ? lane + 32 * w : nq - 1));
     const int32_t *cb = cand + (int64_t)b * maxc;
     int32_t *out = ci + (int64_t)b * maxc;
     const int warps_per_query = gridDim.x * CI_WARPS;
@@ -76,18 +81,15 @@ ci_kernel(const int32_t *__restrict__ table, int64_t K, int nq, const int32_t *_
                 int32_t v[U][NQW];
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
-                    const int32_t c = __shfl_sync(0xffffffffu, cidv, t + u);                // t + u <= 31
-                    const int32_t *row = tb + (int64_t)DBG_CID(c) * nq;
+                    const uint32_t c = (uint32_t)DBG_CID(__shfl_sync(0xffffffffu, cidv, t + u));       // t + u <= 31
 #pragma unroll
-                    for (int w = 0; w < NQW; ++w) {
-                        int col = lane + 32 * w;
-                        v[u][w] = (col < nq) ? __ldg(row + col) : INT_MIN;
-                    }
+                    for (int w = 0; w < NQW; ++w)
+                        v[u][w] = __ldg(reinterpret_cast<const int32_t *>(col[w] + (uint64_t)c * row_bytes));
                 }
 #pragma unroll
-                for (int u = 0; u < U; ++u)
+                for (int u = 0; u < U; u += 2)
 #pragma unroll
-                    for (int w = 0; w < NQW; ++w) m[w] = max(m[w], v[u][w]);
+                    for (int w = 0; w < NQW; ++w) m[w] = __vimax3_s32(m[w], v[u][w], v[u + 1][w]);
             }
         }
         int s = 0;
