@@ -217,8 +217,12 @@ compact_kernel(const uint32_t *__restrict__ bitmap, int64_t words, int n_chunks,
     }
     int32_t *out = cand + (int64_t)b * maxc;
     // A thread's ids are consecutive in the output but the threads' runs are ~30 ids apart, so direct stores are
-    // scattered 4-byte writes: when the chunk's ids fit, they are staged in shared memory and copied out coalesced.
-    __shared__ int32_t staged[COMPACT_STAGE];
+    // scattered 4-byte writes: when the chunk's ids fit, they are staged in shared memory and copied out coalesced.  A fuller chunk
+    // (a quarter of its documents) is written a bitmap word per warp, from the words and the positions that they start at (64
+    // queries with all of 200,000 documents: 117 -> 24 us).
+    __shared__ __align__(8) int32_t staged[COMPACT_STAGE];
+    uint2 *starts = reinterpret_cast<uint2 *>(staged);
+    static_assert(sizeof(uint2) * BITMAP_CHUNK_WORDS <= sizeof(staged), "words and positions of a chunk");
     const bool use_stage = total <= COMPACT_STAGE;
     int64_t pos = use_stage ? local : base + local;
 #pragma unroll
@@ -226,27 +230,37 @@ compact_kernel(const uint32_t *__restrict__ bitmap, int64_t words, int n_chunks,
         uint32_t bits = w[j];
         if (ranks && j < mine && w0 + j < words)          // the word and the candidates before it: document -> candidate index
             ranks[(int64_t)b * words + w0 + j] = make_uint2(w[j], (uint32_t)(use_stage ? base + pos : pos));
+        if (!use_stage) {
+            if (j < mine) starts[threadIdx.x * wpt + j] = make_uint2(w[j], (uint32_t)pos);
+            pos += __popc(bits);
+            continue;
+        }
         while (bits) {
             int t = __ffs(bits) - 1;
             bits &= bits - 1;
-            const int32_t id = (int32_t)(((w0 + j) << 5) + t);
-            if (use_stage) {
-                staged[pos] = id;
-            } else if (pos < maxc) {
-                out[pos] = id;
-                if (rng) rng[(int64_t)b * maxc + pos] = doc_range(doc_off, id);
-            }
-            ++pos;
+            staged[pos++] = (int32_t)(((w0 + j) << 5) + t);
         }
     }
-    if (use_stage) {
+    if (!use_stage) {
         __syncthreads();
-        for (int e = threadIdx.x; e < total; e += CHUNK_THREADS)
-            if (base + e < maxc) {
-                out[base + e] = staged[e];
-                if (rng) rng[(int64_t)b * maxc + base + e] = doc_range(doc_off, staged[e]);
+        const int lane = threadIdx.x & 31;
+        for (int i = threadIdx.x >> 5; i < chunk_words; i += CHUNK_THREADS / 32) {
+            const uint2 s = starts[i];
+            const int64_t at = (int64_t)s.y + __popc(s.x & ((1u << lane) - 1u));
+            if ((s.x >> lane & 1u) && at < maxc) {
+                const int32_t id = (int32_t)((((int64_t)blockIdx.x * chunk_words + i) << 5) + lane);
+                out[at] = id;
+                if (rng) rng[(int64_t)b * maxc + at] = doc_range(doc_off, id);
             }
+        }
+        return;
     }
+    __syncthreads();
+    for (int e = threadIdx.x; e < total; e += CHUNK_THREADS)
+        if (base + e < maxc) {
+            out[base + e] = staged[e];
+            if (rng) rng[(int64_t)b * maxc + base + e] = doc_range(doc_off, staged[e]);
+        }
 }
 
 int launch_gather(const Index &ix, const Params &p, const Layout &L, const int32_t *probes, uint32_t *bitmap,
@@ -256,7 +270,12 @@ int launch_gather(const Index &ix, const Params &p, const Layout &L, const int32
     const int n_lists = p.nq * p.P;
     const bool few = 4 * p.B <= ix.sm_count;
     const int ranges = (int)((L.words + MARK_RANGE_WORDS - 1) / MARK_RANGE_WORDS);
-    const bool by_range = !few && ranges <= 8;           // (every range reads all lists: up to 14 million documents)
+    // Bitmaps of up to 96 KB whose words are set a dozen times or more on average: in shared memory, sixteen blocks a query (16
+    // queries of 1,024 lists, 61 entries a word: 158 us in L2, 29 so; 37 queries, 19: 32 and 28; one query, 8: 5.7 and 8.3).
+    const bool shared = L.words <= 24 * 1024 && (double)n_lists * ((double)ix.ivf_len / (double)ix.K) >= 12.0 * (double)L.words;
+    // A block per query and range (every range reads all lists: up to 14 million documents), unless that leaves SMs idle (64 queries
+    // on one range of 25 KB: 198 us, sixteen blocks a query 100).
+    const bool by_range = !few && ranges <= 8 && (!shared || (int64_t)ranges * p.B >= ix.sm_count);
     if (!by_range && !bitmap_clear) CHIMERA_CUDA(cudaMemsetAsync(bitmap, 0, sizeof(uint32_t) * (size_t)L.words * p.B, st));
     if (by_range) {
         int range_words = (int)((L.words + ranges - 1) / ranges);
@@ -265,8 +284,9 @@ int launch_gather(const Index &ix, const Params &p, const Layout &L, const int32
         CHIMERA_CUDA(cudaFuncSetAttribute(mark_range_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         launch(mark_range_kernel, dim3((unsigned)((L.words + range_words - 1) / range_words), (unsigned)p.B), 1024, smem, st, probes,
                n_lists, ix.ivf_off, ix.ivf_doc, bitmap, L.words, range_words, L.n_chunks, chunk_cnt);
-    } else if (L.words <= 12 * 1024 && (double)n_lists * ((double)ix.ivf_len / (double)ix.K) >= 32.0 * (double)L.words) {
-        // bitmaps of up to 48 KB whose words are set 32 times or more on average
+    } else if (shared) {
+        CHIMERA_CUDA(cudaFuncSetAttribute(mark_shared_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)(sizeof(uint32_t) * (size_t)L.words)));
         launch(mark_shared_kernel, dim3((unsigned)(n_lists < 16 ? n_lists : 16), (unsigned)p.B), 512,
                sizeof(uint32_t) * (size_t)L.words, st, probes, n_lists, ix.ivf_off, ix.ivf_doc, bitmap, (int)L.words);
     } else {
