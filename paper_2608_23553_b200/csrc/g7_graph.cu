@@ -20,10 +20,6 @@
 
 namespace chimera {
 
-constexpr int GP_WARPS = 4;              // warps per query token
-constexpr int GP_PIPE = 4;               // centroid rows in flight per warp while scoring
-constexpr int GP_BATCH = GP_WARPS * 32;  // centroids per step
-
 // Xc[c][d] = rint(centroid * 2^22), recombined from the three balanced base-256 digit planes of the index.
 __global__ void xc_kernel(const int8_t *__restrict__ cdig, int64_t K, int D, int nbits, int32_t *__restrict__ xc)
 {
@@ -129,95 +125,108 @@ __device__ __forceinline__ unsigned long long gp_key(int32_t score, int32_t id)
 __device__ __forceinline__ int32_t gp_id(unsigned long long key) { return 0x7FFFFFFF - (int32_t)((uint32_t)key >> 1); }
 __device__ __forceinline__ int32_t gp_score(unsigned long long key) { return (int32_t)((uint32_t)(key >> 32) ^ 0x80000000u); }
 
-// grid (tokens), one block of four warps per query token.  The search is a chain -- best unexpanded member -> its neighbours ->
+// grid (tokens), one block of WARPS warps per query token.  The search is a chain -- best unexpanded member -> its neighbours ->
 // which are new -> their rows -> their scores -> the list -- so it is latency that counts: the visited set is a bitmap in
 // shared memory (SHARED; written out at the end when wanted), all warps fetch and score the new centroids of a step
-// together, and warp 0 keeps the list in registers and looks only at scores that rank inside it.  With one warp per token,
-// a bitmap in global memory and every score offered in turn, Mid's 2,048 tokens of a batch of 64 took 860 us; now 469.
+// together, and warp 0 keeps the list in registers and looks only at scores that rank inside it.  Many tokens hide that chain,
+// and then the instructions count: eight lanes score a centroid (a warp per centroid, its sum by two hardware reductions, took 94
+// instructions each over all warps), a row's address is one 32 x 32-bit multiply-add, places in s_ids come from votes, keys
+// are compared as they are, and only lists of more than 32 members (WIDE) have a second key per lane.
+// Mid, beam 32, 256 entries: 2,048 tokens 470 -> 244 us with two warps (all blocks resident at once; four: 268), 32 tokens 192 -> 116
+// with four (two: 155), 8,192 tokens 1,492 -> 718.  Two rows in flight per eight lanes: 300.
 // visited (NULL: not wanted; !SHARED: [tokens][vwords] zeroed by the caller).
-template <bool SHARED>
-__global__ void __launch_bounds__(GP_WARPS * 32, 8)
+template <bool SHARED, bool WIDE, int WARPS>
+__global__ void __launch_bounds__(WARPS * 32, 32 / WARPS)
 graph_probe_kernel(const float *__restrict__ queries, int D, const int32_t *__restrict__ xc,
                    const int32_t *__restrict__ graph, int R, int64_t K, int n_entries, int beam, int max_exp,
                    int nprobe, uint32_t *__restrict__ visited, int64_t vwords, int32_t *__restrict__ out_probes,
                    int32_t *__restrict__ out_scores, int32_t *__restrict__ out_nvis)
 {
     pdl_entry();
+    constexpr int BATCH = WARPS * 32;                    // centroids of a step, at most
     extern __shared__ uint32_t s_vis[];
-    __shared__ int32_t s_ids[GP_BATCH], s_sc[GP_BATCH];
+    __shared__ int32_t s_ids[BATCH], s_sc[BATCH];
     __shared__ int s_n, s_next;                          // centroids of the step; the member to expand (-1: none)
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t token = blockIdx.x;
-    const bool has_dims = 4 * lane < D;                  // lane owns dimensions 4 lane .. 4 lane + 3
-    int xq[4] = {0, 0, 0, 0};
-    if (has_dims) {
-        const float4 v = __ldg(reinterpret_cast<const float4 *>(queries + token * D) + lane);
-        xq[0] = __float2int_rn(fminf(fmaxf(v.x, -1.0f), 1.0f) * 4194304.0f);
-        xq[1] = __float2int_rn(fminf(fmaxf(v.y, -1.0f), 1.0f) * 4194304.0f);
-        xq[2] = __float2int_rn(fminf(fmaxf(v.z, -1.0f), 1.0f) * 4194304.0f);
-        xq[3] = __float2int_rn(fminf(fmaxf(v.w, -1.0f), 1.0f) * 4194304.0f);
+    // eight lanes score a centroid: lane l8 has dimensions 32 q + 4 l8 ... + 3 of it, q < D / 32
+    const int l8 = lane & 7, quads = D >> 5;
+    int xq[4][4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const float4 v = q < quads ? __ldg(reinterpret_cast<const float4 *>(queries + token * D) + 8 * q + l8) : make_float4(0.f, 0.f, 0.f, 0.f);
+        xq[q][0] = __float2int_rn(fminf(fmaxf(v.x, -1.0f), 1.0f) * 4194304.0f);
+        xq[q][1] = __float2int_rn(fminf(fmaxf(v.y, -1.0f), 1.0f) * 4194304.0f);
+        xq[q][2] = __float2int_rn(fminf(fmaxf(v.z, -1.0f), 1.0f) * 4194304.0f);
+        xq[q][3] = __float2int_rn(fminf(fmaxf(v.w, -1.0f), 1.0f) * 4194304.0f);
     }
     uint32_t *vis = SHARED ? s_vis : visited + token * vwords;
     if (SHARED)
-        for (int w = tid; w < (int)vwords; w += GP_WARPS * 32) s_vis[w] = 0u;
+        for (int w = tid; w < (int)vwords; w += BATCH) s_vis[w] = 0u;
     if (tid == 0) s_n = 0;
     __syncthreads();
 
-    unsigned long long key0 = 0ull, key1 = 0ull;         // warp 0: list slots lane and 32 + lane, best first
+    const char *const xc_lane = reinterpret_cast<const char *>(xc) + 16 * l8;
+    const uint32_t row_bytes = 4u * (uint32_t)D;
+    unsigned long long key0 = 0ull, key1 = 0ull;         // warp 0: list slots lane and (WIDE) 32 + lane, best first
     int n_vis = 0;
 
     // offer a scored centroid (warp-uniform argument) to the list
     auto offer = [&](unsigned long long x) {
-        const int pos = __popc(__ballot_sync(0xffffffffu, (key0 >> 1) > (x >> 1))) +
-                        __popc(__ballot_sync(0xffffffffu, (key1 >> 1) > (x >> 1)));
+        // (x is no member: where the flags differ the ids do)
+        int pos = __popc(__ballot_sync(0xffffffffu, key0 > x));
+        if (WIDE) pos += __popc(__ballot_sync(0xffffffffu, key1 > x));
         if (pos >= beam) return;                          // ranks behind a full list
-        const unsigned long long up0 = __shfl_up_sync(0xffffffffu, key0, 1), up1 = __shfl_up_sync(0xffffffffu, key1, 1);
-        const unsigned long long last0 = __shfl_sync(0xffffffffu, key0, 31);
-        const int s0 = lane, s1 = 32 + lane;
-        if (s1 > pos) key1 = lane == 0 ? last0 : up1;
-        else if (s1 == pos) key1 = x;
-        if (s0 > pos) key0 = up0;
-        else if (s0 == pos) key0 = x;
-        if (s0 >= beam) key0 = 0ull;                      // the member pushed past the end falls off
-        if (s1 >= beam) key1 = 0ull;
+        const unsigned long long up0 = __shfl_up_sync(0xffffffffu, key0, 1);
+        if (WIDE) {
+            const unsigned long long up1 = __shfl_up_sync(0xffffffffu, key1, 1);
+            const unsigned long long last0 = __shfl_sync(0xffffffffu, key0, 31);
+            const int s1 = 32 + lane;
+            if (s1 > pos) key1 = lane == 0 ? last0 : up1;
+            else if (s1 == pos) key1 = x;
+            if (s1 >= beam) key1 = 0ull;
+        }
+        if (lane > pos) key0 = up0;
+        else if (lane == pos) key0 = x;
+        if (lane >= beam) key0 = 0ull;                    // the member pushed past the end falls off
     };
-    // exact S_fx(q, c) from a lane's four products
-    auto finish_score = [&](const int4 &c) -> int32_t {
-        long long s = 0;
-        if (has_dims) s = (long long)xq[0] * c.x + (long long)xq[1] * c.y + (long long)xq[2] * c.z + (long long)xq[3] * c.w;
-        // |s| < 2^46: the low 24 bits and the rest are summed over the warp separately (both fit 32 bits)
-        const uint32_t lo = __reduce_add_sync(0xffffffffu, (uint32_t)(s & 0xffffff));
-        const int32_t hi = __reduce_add_sync(0xffffffffu, (int32_t)(s >> 24));
-        const long long t = ((long long)hi << 24) + (long long)lo;
-        return (int32_t)((t + (1LL << 19)) >> 20);
-    };
-    // this thread's centroid of the step: into s_ids when it was never visited (order does not matter: the list is the best
-    // `beam` of everything offered)
+    // this thread's centroid of the step (-1: none; whole warps): into s_ids when it was never visited (order does not matter:
+    // the list is the best `beam` of everything offered)
     auto collect = [&](int32_t n) {
-        n = DBG_CID(n);
-        const uint32_t bit = 1u << (n & 31);
-        if ((atomicOr(&vis[n >> 5], bit) & bit) == 0u) s_ids[atomicAdd(&s_n, 1)] = n;
+        bool fresh = false;
+        if (n >= 0) {
+            n = DBG_CID(n);
+            const uint32_t bit = 1u << (n & 31);
+            fresh = (atomicOr(&vis[n >> 5], bit) & bit) == 0u;
+        }
+        const unsigned who = __ballot_sync(0xffffffffu, fresh);
+        if (who == 0u) return;
+        int at = 0;
+        if (lane == 0) at = atomicAdd(&s_n, __popc(who));
+        at = __shfl_sync(0xffffffffu, at, 0);
+        if (fresh) s_ids[at + __popc(who & ((1u << lane) - 1u))] = n;
     };
-    // the step's centroids (at most GP_BATCH): scored by all warps, offered by warp 0.  Two barriers; s_n is 0 afterwards.
+    // the step's centroids (at most BATCH): scored by all warps, offered by warp 0.  Two barriers; s_n is 0 afterwards.
     auto score_and_offer = [&]() {
         __syncthreads();
         const int cnt = s_n;
-        for (int k0 = warp; k0 < cnt; k0 += GP_WARPS * GP_PIPE) {
-            int4 rows[GP_PIPE];
+        for (int k0 = 4 * warp; k0 < cnt; k0 += 4 * WARPS) {
+            const int k = k0 + (lane >> 3);                  // (past the end: the last one again)
+            const char *row = xc_lane + (uint64_t)(uint32_t)s_ids[k < cnt ? k : cnt - 1] * row_bytes;
+            int4 v[4];
 #pragma unroll
-            for (int u = 0; u < GP_PIPE; ++u) {
-                const int k = k0 + GP_WARPS * u;
-                rows[u] = make_int4(0, 0, 0, 0);
-                if (k < cnt && has_dims) rows[u] = __ldg(reinterpret_cast<const int4 *>(xc + (int64_t)s_ids[k] * D) + lane);
-            }
+            for (int q = 0; q < 4; ++q)
+                if (q < quads) v[q] = __ldg(reinterpret_cast<const int4 *>(row + 128 * q));
+            // exact S_fx(q, c): |s| < 2^46
+            long long s = 0;
 #pragma unroll
-            for (int u = 0; u < GP_PIPE; ++u) {
-                const int k = k0 + GP_WARPS * u;
-                if (k < cnt) {
-                    const int32_t sc = finish_score(rows[u]);
-                    if (lane == 0) s_sc[k] = sc;
-                }
-            }
+            for (int q = 0; q < 4; ++q)
+                if (q < quads)
+                    s += (long long)xq[q][0] * v[q].x + (long long)xq[q][1] * v[q].y + (long long)xq[q][2] * v[q].z +
+                         (long long)xq[q][3] * v[q].w;
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (l8 == 0 && k < cnt) s_sc[k] = (int32_t)((s + (1LL << 19)) >> 20);
         }
         __syncthreads();
         if (warp == 0) {
@@ -227,9 +236,9 @@ graph_probe_kernel(const float *__restrict__ queries, int D, const int32_t *__re
                 const unsigned long long mine = k < cnt ? gp_key(s_sc[k], s_ids[k]) : 0ull;
                 for (uint32_t left = __ballot_sync(0xffffffffu, k < cnt); left;) {
                     // the keys that rank inside the list as it is now (it only gets better)
-                    const unsigned long long last = beam <= 32 ? __shfl_sync(0xffffffffu, key0, beam - 1)
-                                                               : __shfl_sync(0xffffffffu, key1, beam - 33);
-                    left &= __ballot_sync(0xffffffffu, (mine >> 1) > (last >> 1));
+                    const unsigned long long last = WIDE && beam > 32 ? __shfl_sync(0xffffffffu, key1, beam - 33)
+                                                                     : __shfl_sync(0xffffffffu, key0, beam - 1);
+                    left &= __ballot_sync(0xffffffffu, mine > last);
                     if (!left) break;
                     const int src = __ffs(left) - 1;
                     left &= left - 1;
@@ -240,16 +249,16 @@ graph_probe_kernel(const float *__restrict__ queries, int D, const int32_t *__re
         }
     };
 
-    for (int j0 = 0; j0 < n_entries; j0 += GP_WARPS * 32) {
+    for (int j0 = 0; j0 < n_entries; j0 += BATCH) {
         const int j = j0 + tid;
-        if (j < n_entries) collect((int32_t)(((long long)j * K) / n_entries));
+        collect(j < n_entries ? (int32_t)(((long long)j * K) / n_entries) : -1);
         score_and_offer();
         __syncthreads();
     }
     for (int done = 0; done < max_exp; ++done) {
         if (warp == 0) {
             const uint32_t u0 = __ballot_sync(0xffffffffu, (key0 & 1ull) != 0ull);
-            const uint32_t u1 = __ballot_sync(0xffffffffu, (key1 & 1ull) != 0ull);
+            const uint32_t u1 = WIDE ? __ballot_sync(0xffffffffu, (key1 & 1ull) != 0ull) : 0u;
             int32_t p = -1;                              // every member expanded
             if (u0) {
                 const int src = __ffs(u0) - 1;
@@ -265,7 +274,7 @@ graph_probe_kernel(const float *__restrict__ queries, int D, const int32_t *__re
         __syncthreads();
         const int32_t p = s_next;
         if (p < 0) break;
-        if (tid < R) collect(__ldg(graph + (int64_t)p * R + tid));          // (R <= 63)
+        if (warp * 32 < R) collect(tid < R ? __ldg(graph + (int64_t)p * R + tid) : -1);          // (R <= 63)
         score_and_offer();
     }
     if (warp == 0) {
@@ -277,7 +286,7 @@ graph_probe_kernel(const float *__restrict__ queries, int D, const int32_t *__re
         if (out_nvis && lane == 0) out_nvis[token] = n_vis;
     }
     if (SHARED && visited)
-        for (int w = tid; w < (int)vwords; w += GP_WARPS * 32) visited[token * vwords + w] = s_vis[w];
+        for (int w = tid; w < (int)vwords; w += BATCH) visited[token * vwords + w] = s_vis[w];
 }
 
 size_t graph_scratch_bytes(const Index &ix, int64_t n_tokens)
@@ -309,10 +318,14 @@ int launch_graph_probes(const Index &ix, const float *queries, int64_t n_tokens,
     const int64_t vwords = (ix.K + 31) / 32;
     const size_t smem = sizeof(uint32_t) * (size_t)vwords;
     const bool shared = visited_in_shared(ix);
-    auto kern = shared ? graph_probe_kernel<true> : graph_probe_kernel<false>;
+    const bool wide = g.beam > 32, four = n_tokens <= 8LL * ix.sm_count;      // (blocks that are resident at once)
+    auto kern = four ? (wide ? (shared ? graph_probe_kernel<true, true, 4> : graph_probe_kernel<false, true, 4>)
+                             : (shared ? graph_probe_kernel<true, false, 4> : graph_probe_kernel<false, false, 4>))
+                     : (wide ? (shared ? graph_probe_kernel<true, true, 2> : graph_probe_kernel<false, true, 2>)
+                             : (shared ? graph_probe_kernel<true, false, 2> : graph_probe_kernel<false, false, 2>));
     if (shared) CHIMERA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     else CHIMERA_CUDA(cudaMemsetAsync(visited, 0, graph_scratch_bytes(ix, n_tokens), st));
-    launch(kern, (unsigned)n_tokens, GP_WARPS * 32, shared ? smem : 0, st, queries, ix.D, ix.xc, ix.graph, ix.graph_deg, ix.K,
+    launch(kern, (unsigned)n_tokens, four ? 128 : 64, shared ? smem : 0, st, queries, ix.D, ix.xc, ix.graph, ix.graph_deg, ix.K,
            g.n_entries, g.beam, g.max_expansions, nprobe, shared && !want_visited ? nullptr : visited, vwords, out_probes,
            out_scores, out_nvis);
     CHIMERA_CUDA(cudaGetLastError());
