@@ -119,7 +119,7 @@ Layout make_layout(const Index &ix, const Params &p)
     L.probes = take(B * nq * p.P * sizeof(int32_t));
     L.pq_cap = L.pq_stride ? probe_queue_cap() : 0;
     L.pq_gmax = take(L.pq_stride ? B * (size_t)L.pq_groups * nq * sizeof(int32_t) : 0);
-    L.pq_thr = take(L.pq_stride ? B * nq * sizeof(int32_t) : 0);
+    L.pq_thr = take(L.pq_stride ? (B * nq + 31) / 32 * 32 * sizeof(int32_t) : 0);
     L.pq_cnt = take(L.pq_stride ? B * nq * sizeof(int32_t) : 0);
     L.pq_keys = take(L.pq_stride ? B * nq * (size_t)L.pq_cap * sizeof(unsigned long long) : 0);
     L.pq_ovf = take(L.pq_stride ? B * sizeof(int32_t) : 0);

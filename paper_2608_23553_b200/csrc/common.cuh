@@ -92,7 +92,7 @@ struct Layout {
     size_t part;          // uint64 [B][n_part][P][nq] partial top-P keys
     size_t probes;        // int32  [B][nq][P]
     size_t pq_gmax;       // int32  [B][pq_groups][nq] stages 1 + 2a together: largest score of each group of sample rows,
-    size_t pq_thr;        // int32  [B*nq]            score bound per query-token row,
+    size_t pq_thr;        // int32  [B*nq]            score bound per query-token row, padded to 32 rows,
     size_t pq_cnt;        // int32  [B*nq]            keys queued for the row,
     size_t pq_keys;       // uint64 [B*nq][pq_cap]    the keys,
     size_t pq_ovf;        // int32  [B]               1 = a queue of this query overflowed (redo by the table scan)

@@ -68,7 +68,7 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar)
 //   tile_stride  > 1, sample != 0: the sample tiles 0, s, 2s, ... (tile = blockIdx.x * s).
 //   tile_stride  > 1, sample == 0: all the others (the j-th tile that is not a multiple of s).
 // FILTER (only with the "others"): thr[row] holds, for every query-token row, a lower bound on the score of the row's
-// nprobe-th best centroid (found on the sample); every score >= thr[row] goes, as a (score, centroid) key, into that
+// nprobe-th best centroid (found on the sample; padded to whole tiles of rows); every score >= thr[row] goes, as a (score, centroid) key, into that
 // row's queue (keys[row][cap], counted in cnt[row]; entries past cap are dropped and the count tells).  The top nprobe
 // of a row are then in its queue, so the probe stage never reads the table again, and a search that needs only the
 // probes passes no table (the RaBitQ pipeline: 2.1 GB less to write at Mid, batch 256).
@@ -264,8 +264,8 @@ score_table_umma(const int8_t *__restrict__ cdig, const __grid_constant__ CUtens
             if (FILTER) {
 #pragma unroll
                 for (int g = 0; g < 4; ++g) {
-                    int4 v = make_int4(0x7fffffff, 0x7fffffff, 0x7fffffff, 0x7fffffff);     // rows past the end
-                    if (r0 + 4 * g < rows32) v = __ldg(reinterpret_cast<const int4 *>(tiles.thr + r0) + g);
+                    // (rows past the end: 0x7fffffff, in the padding behind the bounds)
+                    const int4 v = __ldg(reinterpret_cast<const int4 *>(tiles.thr + r0) + g);
                     thr_v[4 * g] = v.x; thr_v[4 * g + 1] = v.y; thr_v[4 * g + 2] = v.z; thr_v[4 * g + 3] = v.w;
                 }
             }
@@ -302,22 +302,35 @@ score_table_umma(const int8_t *__restrict__ cdig, const __grid_constant__ CUtens
                     for (int e = 0; e < 8; ++e) any |= out[e] >= thr_v[ch * 8 + e];
                     if (any) {                  // about nprobe x tile_stride keys per row in all: one lane of a warp every
                                                 // few chunks, and then hardly ever two values of the lane
-                        uint32_t pass = 0u;
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) pass |= out[e] >= thr_v[ch * 8 + e] ? 1u << e : 0u;
-                        while (pass) {          // (rows past the end have the largest threshold: they never pass)
-                            const int e = __ffs(pass) - 1;
-                            pass &= pass - 1;
-                            int32_t v = out[0];
-#pragma unroll
-                            for (int x = 1; x < 8; ++x) v = e == x ? out[x] : v;
-                            // The slot comes back from the atomic hundreds of cycles later; the key is stored only when
-                            // this thread's next key turns up (or at the end), so nobody waits for it.
+                        // The slot comes back from the atomic hundreds of cycles later; the key is stored only when
+                        // this thread's next key turns up (or at the end), so nobody waits for it.
+                        auto push = [&](int e, int32_t v) {
                             if (pend_key && pend_slot < tiles.cap) pend_dst[pend_slot] = pend_key;
                             const uint32_t row = rc + e;
                             pend_key = key_int(v, (int32_t)c);
                             pend_dst = tiles.keys + (int64_t)row * tiles.cap;
                             pend_slot = atomicAdd(tiles.cnt + row, 1);
+                        };
+                        // (Rows past the end have the largest threshold: they never pass.)  Issue binds the tiles that
+                        // are not stored (357 instructions per warp and tile): eight copies of the push take fewer than the
+                        // mask and the selects (Mid, batch 256: 617 -> 562 us).  Where the stores of the scores bind, the
+                        // copies cost more than they save (768 -> 796 us): there a loop over the few that pass.
+                        if (!TABLE) {
+#pragma unroll
+                            for (int e = 0; e < 8; ++e)
+                                if (out[e] >= thr_v[ch * 8 + e]) push(e, out[e]);
+                        } else {
+                            uint32_t pass = 0u;
+#pragma unroll
+                            for (int e = 0; e < 8; ++e) pass |= out[e] >= thr_v[ch * 8 + e] ? 1u << e : 0u;
+                            while (pass) {
+                                const int e = __ffs(pass) - 1;
+                                pass &= pass - 1;
+                                int32_t v = out[0];
+#pragma unroll
+                                for (int x = 1; x < 8; ++x) v = e == x ? out[x] : v;
+                                push(e, v);
+                            }
                         }
                     }
                 }

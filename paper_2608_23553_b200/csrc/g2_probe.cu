@@ -369,6 +369,7 @@ sample_bound_kernel(const int32_t *__restrict__ gmax, int G, int nq, int P, int6
         }
         prev = best;
     }
+    if (row == rows - 1 && lane < (int)(-rows & 31)) thr[rows + lane] = INT32_MAX;       // the padding that no score reaches
     if (lane == 0) {
         thr[row] = (int32_t)((uint32_t)(prev >> 32) ^ 0x80000000u);
         cnt[row] = 0;
