@@ -15,7 +15,7 @@
 // loads (lane = token), each is broadcast with a shuffle, and the warp gathers the table row S[cid, :] with
 // lane = query token (one 128-byte line for 32 query tokens), keeping a running maximum per lane.
 //
-// select_kernel: one block per query.  Radix select (11 + 11 + 10 bits) of the n_prune-th largest score, then an
+// select_kernel: one block per query.  Few of many: select_few.  Else radix select (11 + 11 + 10 bits) of the n_prune-th largest score, then an
 // ordered compaction of the candidate list (which is ascending in id), so equal scores are resolved towards smaller
 // ids and the survivors come out ascending.  With few queries per call the contender and selection steps run over 32
 // blocks per query instead (contender_hist/count/write kernels, sels_* kernels), and shard_select_kernel merges the
@@ -965,6 +965,135 @@ int launch_centroid_interaction(const Index &ix, const Params &p, const int32_t 
 }
 
 // ------------------------------------------------------------------------------------------------ selection ------
+// The selection of few from many in one pass over the scores.  A block waits for its loads most of the time, and the radix
+// select with the compaction behind it passes over the scores four times and over the ids once.  Here a sample of SEL_SAMPLE
+// scores gives a bound that somewhat more than n_prune scores reach (the wanted rank of the sample and four standard deviations
+// more), one pass collects those in shared memory, and the selection and the order of the survivors are found there.  False,
+// with nothing written: the bound let too few through or more than there is room for; the caller selects among all then.
+// Measured (1,024 wanted of Mid's candidates, 1-bit refinement): 256 queries 122 -> 50 us, 64 queries 69 -> 30 us.
+constexpr int SEL_SAMPLE = 8192, SEL_FEW = 3584, SEL_BINS = 2048;
+struct SelFew {
+    union {
+        uint32_t sample[SEL_SAMPLE];
+        struct {
+            uint32_t u[SEL_FEW];                             // scores in the order of radix_select, in any order
+            int pos[SEL_FEW];                                // their places in the candidate list
+            uint16_t ord[SEL_FEW];                           // the survivors by bucket of places
+        };
+    };
+    int n;
+};
+// The wanted rank of the sample.  Taken from 16,384 scores on (shorter lists cost a pass of the block's loads or two, no more
+// than the sample) while the documents to be expected fill no more than 6/7 of the list.
+__device__ __forceinline__ bool select_few_applies(int n, int n_prune, int *want)
+{
+    const float r = (float)n_prune * ((float)SEL_SAMPLE / (float)n);
+    const float w = r + 4.f * sqrtf(r) + 8.f;
+    *want = (int)w;
+    return n >= 2 * SEL_SAMPLE && w * (float)n <= 3072.f * SEL_SAMPLE;
+}
+__device__ __forceinline__ bool select_few(const int32_t *__restrict__ cb, const int32_t *__restrict__ sb, int n, int n_prune,
+                                           int want, int32_t *__restrict__ out, int32_t *__restrict__ out_ci, SelFew &few,
+                                           int *hist /* [SEL_BINS] */, int *warp_part, uint32_t *s_prefix, int *s_want)
+{
+    const int tid = threadIdx.x;
+    // groups of four neighbours at equal distances (a 32-byte sector costs the same for one)
+    {
+        const int step = n / (SEL_SAMPLE / 4);
+        uint32_t v[SEL_SAMPLE / SEL_THREADS];
+#pragma unroll
+        for (int e = 0; e < SEL_SAMPLE / SEL_THREADS; ++e) {
+            const int i = e * SEL_THREADS + tid;
+            v[e] = (uint32_t)sb[(i >> 2) * step + (i & 3)];
+        }
+#pragma unroll
+        for (int e = 0; e < SEL_SAMPLE / SEL_THREADS; ++e) few.sample[e * SEL_THREADS + tid] = v[e];
+    }
+    if (tid == 0) few.n = 0;
+    __syncthreads();
+    int need_eq;
+    const uint32_t bound = radix_select([&](int j) { return (int32_t)few.sample[j]; }, SEL_SAMPLE, want, hist, warp_part, s_prefix,
+                                        s_want, &need_eq);
+    __syncthreads();                                         // the sample's place is used again
+    for (int base = 0; base < n; base += 8 * SEL_THREADS) {
+        uint32_t u[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const int j = base + e * SEL_THREADS + tid;
+            u[e] = j < n ? (uint32_t)sb[j] ^ 0x80000000u : 0u;
+        }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const int j = base + e * SEL_THREADS + tid;
+            if (u[e] >= bound && j < n) {
+                const int slot = atomicAdd(&few.n, 1);
+                if (slot < SEL_FEW) { few.u[slot] = u[e]; few.pos[slot] = j; }
+            }
+        }
+    }
+    __syncthreads();
+    const int c = few.n;
+    if (c < n_prune || c > SEL_FEW) return false;
+    const uint32_t thr = radix_select([&](int j) { return (int32_t)(few.u[j] ^ 0x80000000u); }, c, n_prune, hist, warp_part,
+                                      s_prefix, s_want, &need_eq);
+    int mine = 0, n_eq;
+    for (int i = tid; i < c; i += SEL_THREADS) mine += few.u[i] == thr ? 1 : 0;
+    int at = sel_block_scan(mine, &n_eq, warp_part);
+    const bool tied = n_eq > need_eq;                        // ties at the edge go to the smaller ids
+    if (tied) {
+        if (n_eq > SEL_BINS) return false;
+        for (int i = tid; i < c; i += SEL_THREADS)
+            if (few.u[i] == thr) hist[at++] = few.pos[i];
+        __syncthreads();
+    }
+    bool keep[(SEL_FEW + SEL_THREADS - 1) / SEL_THREADS];
+#pragma unroll
+    for (int e = 0; e < (SEL_FEW + SEL_THREADS - 1) / SEL_THREADS; ++e) {
+        const int i = e * SEL_THREADS + tid;
+        keep[e] = i < c && few.u[i] >= thr;
+        if (keep[e] && tied && few.u[i] == thr) {
+            int before = 0;
+            for (int k = 0; k < n_eq; ++k) before += hist[k] < few.pos[i] ? 1 : 0;
+            keep[e] = before < need_eq;
+        }
+    }
+    __syncthreads();
+    // the survivors' order: buckets of neighbouring places (half a survivor each at 1,024), then the place within the bucket
+    int shift = 0;
+    while (((n - 1) >> shift) >= SEL_BINS) ++shift;
+    for (int i = tid; i < SEL_BINS; i += SEL_THREADS) hist[i] = 0;
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < (SEL_FEW + SEL_THREADS - 1) / SEL_THREADS; ++e)
+        if (keep[e]) atomicAdd(&hist[few.pos[e * SEL_THREADS + tid] >> shift], 1);
+    __syncthreads();
+    const int h0 = hist[2 * tid], h1 = hist[2 * tid + 1];
+    int total;
+    const int first = sel_block_scan(h0 + h1, &total, warp_part);
+    hist[2 * tid] = first;
+    hist[2 * tid + 1] = first + h0;
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < (SEL_FEW + SEL_THREADS - 1) / SEL_THREADS; ++e) {
+        const int i = e * SEL_THREADS + tid;
+        if (keep[e]) few.ord[atomicAdd(&hist[few.pos[i] >> shift], 1)] = (uint16_t)i;
+    }
+    __syncthreads();                                         // hist[x]: where bucket x ends
+#pragma unroll
+    for (int e = 0; e < (SEL_FEW + SEL_THREADS - 1) / SEL_THREADS; ++e) {
+        const int i = e * SEL_THREADS + tid;
+        if (keep[e]) {
+            const int pos = few.pos[i], x = pos >> shift;
+            const int begin = x ? hist[x - 1] : 0, end = hist[x];
+            int rank = begin;
+            for (int k = begin; k < end; ++k) rank += few.pos[few.ord[k]] < pos ? 1 : 0;
+            out[rank] = cb[pos];
+            if (out_ci) out_ci[rank] = (int32_t)(few.u[i] ^ 0x80000000u);
+        }
+    }
+    return true;
+}
+
 // grid (B).  pruned[b][0..n_prune) ascending ids, -1 padded; n_pruned[b]; pruned_ci (optional): the score of each
 // kept document, INT_MIN beside every -1.
 __global__ void __launch_bounds__(SEL_THREADS)
@@ -973,7 +1102,8 @@ select_kernel(const int32_t *__restrict__ cand, const int32_t *__restrict__ n_ca
               int32_t *__restrict__ pruned_ci)
 {
     pdl_entry();
-    __shared__ int hist[2048];
+    __shared__ SelFew few;
+    __shared__ int hist[SEL_BINS];
     __shared__ int warp_part[32];
     __shared__ uint32_t s_prefix;
     __shared__ int s_want;
@@ -992,7 +1122,13 @@ select_kernel(const int32_t *__restrict__ cand, const int32_t *__restrict__ n_ca
         if (threadIdx.x == 0) n_pruned[b] = n;
         return;
     }
-    int need_eq;
+    int need_eq, want;
+    if (select_few_applies(n, n_prune, &want) &&
+        select_few(cb, sb, n, n_prune, want, out, out_ci, few, hist, warp_part, &s_prefix, &s_want)) {
+        if (threadIdx.x == 0) n_pruned[b] = n_prune;
+        return;
+    }
+    __syncthreads();
     const uint32_t thr = radix_select([&](int j) { return sb[j]; }, n, n_prune, hist, warp_part, &s_prefix, &s_want,
                                       &need_eq);
 
