@@ -159,7 +159,7 @@ Layout make_layout(const Index &ix, const Params &p)
     L.ranks = take(ix.tok_id || batch ? B * (size_t)L.words * sizeof(uint2) : 0);
     // retrieved-token scores of the refinements: visit lists, or dense rows per candidate
     L.visit_nodes = visit_list_nodes(ix, p);
-    L.partial_m = take(!ix.tok_id ? 0 : L.visit_nodes ? B * ((size_t)L.visit_nodes * 8 + (size_t)p.maxc * 4)
+    L.partial_m = take(!ix.tok_id ? 0 : L.visit_nodes ? B * ((size_t)L.visit_nodes + (size_t)p.maxc) * 8
                                                       : B * (size_t)p.maxc * nq * sizeof(int32_t));
     L.graph_vis = take(ix.graph ? graph_workspace_bytes(ix, (int64_t)p.B * p.nq) : 0);
     L.q_rot = take(ix.rot_t ? B * nq * ix.D * sizeof(float) : 0);

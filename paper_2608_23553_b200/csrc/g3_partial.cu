@@ -23,7 +23,7 @@ namespace chimera {
 constexpr int PS_THREADS = 128;
 
 // Nodes per query of the visit lists, 0 when the table of maxima is used: no token lists, few queries per call (latency
-// counts), more nodes than their index holds, a table less than four times as large, or candidates with several visits
+// counts), more nodes than their index holds, a table less than about four times as large, or candidates with several visits
 // each, whose lists are chains of scattered reads: more than two as independent tokens would have them (long documents under
 // many probes, where the topics of real ones make it many more), or four by the distinct centroids of a document.
 // Whole searches, batch 256 on Mid's sizes, documents that draw 1/4 as many centroids as they have tokens (4.1 visits): lists
@@ -50,56 +50,79 @@ int refine_splits(const Index &ix, const Params &p)
 
 // grid (blocks, B): empty lists for the first n_cand[b] candidates.
 __global__ void __launch_bounds__(256)
-visit_clear_kernel(int32_t *__restrict__ head, const int32_t *__restrict__ n_cand, int64_t maxc)
+visit_clear_kernel(unsigned long long *__restrict__ head, const int32_t *__restrict__ n_cand, int64_t maxc)
 {
     pdl_entry();
     const int b = blockIdx.y, n = n_cand[b];
-    for (int e = blockIdx.x * 256 + threadIdx.x; e < n; e += gridDim.x * 256) head[(int64_t)b * maxc + e] = 0;
+    for (int e = blockIdx.x * 256 + threadIdx.x; e < n; e += gridDim.x * 256) head[(int64_t)b * maxc + e] = 0ull;
 }
-// grid (blocks, B): fprime[b][j] of every candidate, one thread each, the first nodes of two candidates in flight.  Long lists
+// grid (blocks, B): fprime[b][j] of every candidate.  Walking a list takes some 50 instructions a visit, and nearly every warp
+// of 32 candidates has one of several visits: the candidates of one visit or none are written at once, the others collected and
+// walked 32 at a time (Mid, batch 256: 226 us with each warp walking its own lists, 134 so).  Long lists
 // take turns at the warp's rows of maxima: 8 for up to 32 query tokens, 4 for 64, 2 for 127 (1 KB a warp, which leaves the
 // scattered reads their L1; with 2 KB no list gains 1 %).
 constexpr int VISIT_ROW_WORDS = 264;                     // 8 x 33, 4 x 65 or 2 x 128
+constexpr int VISIT_AHEAD = 4;                           // heads in flight per lane
 template <bool FLOAT>
 __global__ void __launch_bounds__(256)
-visit_sum_kernel(const int32_t *__restrict__ head, const unsigned long long *__restrict__ node, int64_t cap,
+visit_sum_kernel(const unsigned long long *__restrict__ head, const unsigned long long *__restrict__ node, int64_t cap,
                  const int32_t *__restrict__ n_cand, int64_t maxc, int nq, int32_t *__restrict__ fprime)
 {
     pdl_entry();
     __shared__ uint32_t s_rows[8][VISIT_ROW_WORDS];
+    __shared__ unsigned long long s_head[8][64];
+    __shared__ int s_place[8][64];
     const int b = blockIdx.y, n = n_cand[b], lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int rows = nq <= 32 ? 8 : nq <= 64 ? 4 : 2, pitch = nq <= 32 ? 33 : nq <= 64 ? 65 : 128;
     const unsigned long long *nodes = node + (int64_t)b * cap;
-    const int32_t *hb = head + (int64_t)b * maxc;
+    const unsigned long long *hb = head + (int64_t)b * maxc;
+    int32_t *out = fprime + (int64_t)b * maxc;
+    int waiting = 0;                                     // lists collected (uniform)
+    auto walk = [&](int m) {                             // the last m of them
+        __syncwarp();
+        const bool on = lane < m;
+        const unsigned long long h = on ? s_head[warp][waiting - m + lane] : 0ull;
+        const int place = on ? s_place[warp][waiting - m + lane] : 0;
+        waiting -= m;
+        int32_t sum;
+        const bool done = visit_sum<FLOAT>(h, nodes, sum);
+        for (unsigned left = __ballot_sync(0xffffffffu, !done); left;) {
+            const int turn = __popc(left & ((1u << lane) - 1));
+            const bool mine = (left >> lane & 1u) && turn < rows;
+            if (mine) sum = visit_sum_long<FLOAT>(h, nodes, s_rows[warp] + turn * pitch, nq);
+            left &= ~__ballot_sync(0xffffffffu, mine);
+        }
+        if (on) out[place] = sum;
+        __syncwarp();
+    };
     const int step = gridDim.x * 256;
-    for (int j0 = blockIdx.x * 256 + warp * 32; j0 < n; j0 += 2 * step) {
-        int32_t first[2];
-        unsigned long long n0[2];
+    for (int j0 = blockIdx.x * 256 + warp * 32; j0 < n; j0 += VISIT_AHEAD * step) {
+        unsigned long long h[VISIT_AHEAD];
 #pragma unroll
-        for (int u = 0; u < 2; ++u) first[u] = j0 + u * step + lane < n ? hb[j0 + u * step + lane] : 0;
+        for (int u = 0; u < VISIT_AHEAD; ++u) h[u] = (int64_t)j0 + u * step + lane < n ? hb[j0 + u * step + lane] : 0ull;
 #pragma unroll
-        for (int u = 0; u < 2; ++u) n0[u] = first[u] != 0 ? nodes[first[u] - 1] : 0ull;
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const int j = j0 + u * step + lane;
-            int32_t sum;
-            const bool done = visit_sum<FLOAT>(n0[u], nodes, sum);
-            for (unsigned left = __ballot_sync(0xffffffffu, !done); left;) {
-                const int place = __popc(left & ((1u << lane) - 1));
-                const bool mine = (left >> lane & 1u) && place < rows;
-                if (mine) sum = visit_sum_long<FLOAT>(first[u], nodes, s_rows[warp] + place * pitch, nq);
-                left &= ~__ballot_sync(0xffffffffu, mine);
+        for (int u = 0; u < VISIT_AHEAD; ++u) {
+            const int64_t j = (int64_t)j0 + u * step + lane;
+            const bool more = (h[u] & VISIT_MORE) != 0;
+            if (!more && j < n) out[j] = (int32_t)(h[u] >> 32);
+            const unsigned votes = __ballot_sync(0xffffffffu, more);
+            if (more) {
+                const int at = waiting + __popc(votes & ((1u << lane) - 1));
+                s_head[warp][at] = h[u];
+                s_place[warp][at] = (int)j;
             }
-            if (j < n) fprime[(int64_t)b * maxc + j] = sum;
+            waiting += __popc(votes);
+            if (waiting >= 32) walk(32);
         }
     }
+    if (waiting > 0) walk(waiting);
 }
 VisitLists visit_lists(const Params &p, const Layout &L, void *mem)
 {
     VisitLists v;
     v.cap = L.visit_nodes;
     v.node = (unsigned long long *)mem;
-    v.head = (int32_t *)(v.node + (int64_t)p.B * v.cap);
+    v.head = v.node + (int64_t)p.B * v.cap;
     return v;
 }
 int launch_visit_clear(const Index &ix, const Params &p, const VisitLists &v, const int32_t *n_cand, cudaStream_t st)
@@ -160,7 +183,7 @@ partial_score_kernel(const int8_t *__restrict__ qdig, const int32_t *__restrict_
     const double kterm = __dmul_rn(__dmul_rn((double)kappa, 4.0), (double)query_sum(dig));
     const uint2 *rk = ranks + (int64_t)b * words;
     int32_t *Mb = LISTS ? nullptr : M + (int64_t)b * maxc * nq;
-    int32_t *heads = LISTS ? lists.head + (int64_t)b * maxc : nullptr;
+    unsigned long long *heads = LISTS ? lists.head + (int64_t)b * maxc : nullptr;
     unsigned long long *nodes = LISTS ? lists.node + (int64_t)b * lists.cap : nullptr;
     int32_t s_c;
     uint32_t v0;                                       // node of the list's first entry

@@ -4,7 +4,10 @@
 // score, of which the largest per (candidate, i) counts.  A candidate has about one visit, so a row of q_len maxima per
 // candidate is nearly empty: clearing, updating and summing such rows was most of the refinement's traffic (Mid, batch
 // 256: 3.4 GB cleared, 3.4 GB read back).  Here every visit is a node of its candidate's list: one exchange of the list's
-// head and one 8-byte store; the visits of a candidate are put together afterwards (visit_sum_kernel).  Nearly every list has
+// head and one 8-byte store; the visits of a candidate are put together afterwards (visit_sum_kernel).  The head holds the last
+// visit itself and the place where that visit left the one before, so a list of one node is known from its head alone, without a scattered
+// read (the wider heads cost the pushes 587 -> 623 us and their clearing 20 -> 36, Mid's partial scores, batch 256; the sum gains
+// more than that, visit_sum_kernel).  Nearly every list has
 // one node on documents of independent tokens, several where documents repeat probed centroids or hold neighbours of one:
 // lists of up to six are sorted in registers, longer ones walked once over a row of maxima in shared memory (one walk per
 // query token before: batch 256, ten visits each, 2.16 ms of refinement, 0.92 so).  The order of a list does not matter: maxima
@@ -14,12 +17,15 @@
 
 namespace chimera {
 
-// node = score bits << 32 | (index of the next node + 1) << 7 | query token
+// visit = score bits << 32 | (its own index + 1) << 7 | query token, scores > 0; node[index] holds the visit before it in the
+// list (0: none), and a head with VISIT_MORE has one.  The flag is set by whoever finds a visit in the head, after the exchange:
+// whichever visit is the head by then, it has a predecessor too.
 constexpr int VISIT_I_BITS = 7;                          // q_len <= 127
 constexpr int64_t VISIT_MAX_NODES = (1LL << 25) - 1;     // per query
+constexpr unsigned long long VISIT_MORE = 1ull << 63;
 
 struct VisitLists {
-    int32_t *head;                 // [B][maxc]: index of the first node + 1, 0 = empty
+    unsigned long long *head;      // [B][maxc]: the last visit, 0 = none
     unsigned long long *node;      // [B][cap]
     int64_t cap;                   // q_len * nprobe * longest list
 };
@@ -30,11 +36,17 @@ int launch_visit_clear(const Index &ix, const Params &p, const VisitLists &v, co
 int launch_visit_sum(const Index &ix, const Params &p, const VisitLists &v, bool floats, const int32_t *n_cand,
                      int32_t *fprime, cudaStream_t st);
 
-__device__ __forceinline__ void visit_push(int32_t *head /* of the candidate */, unsigned long long *nodes, uint32_t v, int i,
-                                           uint32_t score)
+__device__ __forceinline__ void visit_push(unsigned long long *head /* of the candidate */, unsigned long long *nodes, uint32_t v,
+                                           int i, uint32_t score)
 {
-    const uint32_t next = (uint32_t)atomicExch(head, (int)v + 1);
-    nodes[v] = (unsigned long long)score << 32 | next << VISIT_I_BITS | (uint32_t)i;
+    const unsigned long long before = atomicExch(head, (unsigned long long)score << 32 | (v + 1) << VISIT_I_BITS | (uint32_t)i);
+    nodes[v] = before & ~VISIT_MORE;
+    if (before) atomicOr(head, VISIT_MORE);
+}
+// The visit before this one, 0 = none.
+__device__ __forceinline__ unsigned long long visit_before(unsigned long long visit, const unsigned long long *nodes)
+{
+    return nodes[((uint32_t)visit >> VISIT_I_BITS) - 1];
 }
 
 // ---- products of packed codes with a query token --------------------------------------------------------------------------
@@ -123,28 +135,25 @@ __device__ __forceinline__ void code_dots(int (&T)[N], const uint32_t (&w)[N][CO
 }
 
 // Largest score per query token, summed in increasing query token.  FLOAT: the scores are float bits > 0 (whose order is
-// that of the integers) and the sum is a chain of fp32 additions from 0.  n0: the first node (0: an empty list).  Lists of up
-// to six visits; false: a longer one.
+// that of the integers) and the sum is a chain of fp32 additions from 0.  Lists of up to six visits; false: a longer one.
 template <bool FLOAT>
-__device__ __forceinline__ bool visit_sum(unsigned long long n0, const unsigned long long *nodes, int32_t &sum)
+__device__ __forceinline__ bool visit_sum(unsigned long long head, const unsigned long long *nodes, int32_t &sum)
 {
-    sum = 0;                                             // (0 is 0.0f as well)
-    if (n0 == 0) return true;
-    uint32_t next = (uint32_t)n0 >> VISIT_I_BITS;
-    if (next == 0) {                                     // one visit; 0.0f + x = x
-        sum = (int32_t)(n0 >> 32);
+    if (!(head & VISIT_MORE)) {                          // no visit or one; 0.0f + x = x
+        sum = (int32_t)(head >> 32);
         return true;
     }
+    head &= ~VISIT_MORE;
     constexpr int KEPT = 6;
-    // a node as (query token, score): sorting descending puts the largest score of a query token first
+    // a visit as (query token, score): sorting descending puts the largest score of a query token first
     unsigned long long key[KEPT];
 #pragma unroll
     for (int k = 0; k < KEPT; ++k) key[k] = ~0ull;
     auto key_of = [](unsigned long long n) { return (n & ((1ull << VISIT_I_BITS) - 1)) << 32 | (uint32_t)~(uint32_t)(n >> 32); };
-    key[0] = key_of(n0);
+    key[0] = key_of(head);
     int cnt = 1;
-    while (next != 0 && cnt < KEPT) {
-        const unsigned long long n = nodes[next - 1];
+    unsigned long long n = visit_before(head, nodes);
+    while (n != 0 && cnt < KEPT) {
         unsigned long long x = key_of(n);                // ascending (query token, inverted score)
 #pragma unroll
         for (int k = 0; k < KEPT; ++k) {
@@ -153,9 +162,10 @@ __device__ __forceinline__ bool visit_sum(unsigned long long n0, const unsigned 
             key[k] = lo;
         }
         ++cnt;
-        next = (uint32_t)n >> VISIT_I_BITS;
+        n = visit_before(n, nodes);
     }
-    if (next != 0) return false;
+    if (n != 0) return false;
+    sum = 0;
     float fs = 0.0f;
     uint32_t last = ~0u;
 #pragma unroll
@@ -172,14 +182,12 @@ __device__ __forceinline__ bool visit_sum(unsigned long long n0, const unsigned 
 
 // The same of a list of any length, walked once: row = q_len words of shared memory (a query token without a visit adds 0).
 template <bool FLOAT>
-__device__ __forceinline__ int32_t visit_sum_long(int32_t first, const unsigned long long *nodes, uint32_t *row, int nq)
+__device__ __forceinline__ int32_t visit_sum_long(unsigned long long head, const unsigned long long *nodes, uint32_t *row, int nq)
 {
     for (int i = 0; i < nq; ++i) row[i] = 0u;
-    for (uint32_t v = (uint32_t)first; v != 0;) {
-        const unsigned long long n = nodes[v - 1];
+    for (unsigned long long n = head & ~VISIT_MORE; n != 0; n = visit_before(n, nodes)) {
         const int i = (int)(n & ((1u << VISIT_I_BITS) - 1));
         row[i] = max(row[i], (uint32_t)(n >> 32));
-        v = (uint32_t)n >> VISIT_I_BITS;
     }
     float fs = 0.0f;
     int32_t is = 0;

@@ -104,7 +104,7 @@ rabitq_partial_kernel(const int8_t *__restrict__ qdig, int nq, int B, int CW, in
     const int sq = query_sum(dig);
     const uint2 *rk = ranks + (int64_t)b * words;
     int32_t *Mb = LISTS ? nullptr : M + (int64_t)b * maxc * nq;
-    int32_t *heads = LISTS ? lists.head + (int64_t)b * maxc : nullptr;
+    unsigned long long *heads = LISTS ? lists.head + (int64_t)b * maxc : nullptr;
     unsigned long long *nodes = LISTS ? lists.node + (int64_t)b * lists.cap : nullptr;
     uint32_t v0;                                       // node of the list's first entry
     int64_t e0;
