@@ -108,7 +108,7 @@ Layout make_layout(const Index &ix, const Params &p)
     L.q_stage = take(B * nq * ix.D * sizeof(float));
     L.out_ids = take(B * p.k * sizeof(int32_t));
     L.out_scores = take(B * p.k * sizeof(float));
-    L.qdig = take(3 * B * nq * 128);
+    L.qdig = take(3 * (size_t)table_rows((int64_t)(B * nq)) * 128);
     const size_t rows4 = B * (size_t)residual_rows(p.nq);
     L.qdig4 = take(3 * rows4 * 128);
     L.table = take(B * (size_t)ix.K * nq * sizeof(int32_t));
@@ -369,7 +369,7 @@ static int run(const Index &ix, const Params &p, int first, int last, const floa
         if (rabitq) {
             // the paper's pipeline on its own codec: rotate the queries, refine by partial 1-bit scores
             if ((rc = launch_rotate(ix, p, queries, q_rot, st))) return rc;
-            if ((rc = launch_digits(q_rot, (int64_t)p.B * p.nq, ix.D, 1, nullptr, qdig_rot, p.nq, status, st))) return rc;
+            if ((rc = launch_digits(q_rot, (int64_t)p.B * p.nq, ix.D, 1, nullptr, false, qdig_rot, p.nq, status, st))) return rc;
             count_launch(SLOT_G1);
             prof_mark(SLOT_G1, st);
             if ((rc = launch_rabitq_partial(ix, p, L, qdig_rot, probes, ranks, n_cand, partial_m, ci, st)))
@@ -445,7 +445,7 @@ static int run(const Index &ix, const Params &p, int first, int last, const floa
             if ((rc = launch_rabitq_scores_umma(ix, p, q_rot, qdig_rot, pruned, score4, status, st))) return rc;
         } else {
             if (first > 1) {                       // stage 1 did not run in this call: build the query digit planes
-                if ((rc = launch_digits(queries, (int64_t)p.B * p.nq, ix.D, ix.nbits, nullptr, qdig4, p.nq, status, st))) return rc;
+                if ((rc = launch_digits(queries, (int64_t)p.B * p.nq, ix.D, ix.nbits, nullptr, false, qdig4, p.nq, status, st))) return rc;
                 count_launch(SLOT_G4);
             }
             if ((rc = launch_residual_scores_umma(ix, p, queries, qdig4, table, pruned, score4, status, st))) return rc;

@@ -85,7 +85,7 @@ struct Layout {
     size_t q_stage;       // float  [B, nq, D]        (host-entry staging of the queries)
     size_t out_ids;       // int32  [B, k]            (host-entry staging)
     size_t out_scores;    // float  [B, k]
-    size_t qdig;          // int8   [3][B*nq][128]
+    size_t qdig;          // int8   [3][table_rows(B*nq)][128], rows in table_row() order
     size_t qdig4;         // int8   [3][B*residual_rows(nq)][128]  the same for stage 4
     size_t table;         // int32  [B][K][nq]
     size_t table8;        // uint8  [B][K][coarse_pitch(nq)]  coarse copy: clamp(S >> 16, 0, 255), zeros past nq
@@ -209,12 +209,12 @@ __device__ __forceinline__ void pdl_entry() { asm volatile("griddepcontrol.wait;
 // ---------------------------------------------------------------------------------------------------------------
 int build_index_device(Index &ix, const float *centroids, const int32_t *doclens, cudaStream_t st);
 // rows x D float32 in [-1, 1] -> three int8 digit planes [3][rows][128] (zero padded, dimensions in digit_dim() order);
-// out-of-range elements set ST_BAD_QUERY.
+// out-of-range elements set ST_BAD_QUERY.  tiles: planes of table_rows(rows) rows in table_row() order, the padding not written.
 // dig4 (may be NULL): the same planes for stage 4, rows = query tokens (q_len of them per query) in score_row() order,
 // padded to residual_rows(q_len) per query; the padding is not written.  dig may be NULL then.
 // clear / clear_n (may be NULL / 0): 32-bit words set to zero on the side, for a later kernel of the same call.
-int launch_digits(const float *x, int64_t rows, int D, int nbits, int8_t *dig, int8_t *dig4, int q_len, uint32_t *status,
-                  cudaStream_t st, uint32_t *clear = nullptr, int64_t clear_n = 0);
+int launch_digits(const float *x, int64_t rows, int D, int nbits, int8_t *dig, bool tiles, int8_t *dig4, int q_len,
+                  uint32_t *status, cudaStream_t st, uint32_t *clear = nullptr, int64_t clear_n = 0);
 
 // table8 may be NULL (no coarse copy wanted).
 int launch_score_table(const Index &ix, const Params &p, const float *queries, int8_t *qdig, int8_t *qdig4, int32_t *table,
@@ -396,6 +396,12 @@ __host__ __device__ __forceinline__ int digit_dim(int pos, int nbits)
 {
     return nbits == 2 ? (pos & ~15) | (pos & 3) << 2 | (pos >> 2 & 3) : (pos & ~31) | (pos & 3) << 3 | (pos >> 2 & 7);
 }
+
+// Stage 1 on the tensor cores: rows of the query digit planes (whole tiles of 32), and the row of query token i of a batch.
+// Within a tile, tokens 8 g ... 8 g + 7 sit in rows 2 g, 2 g + 1, 8 + 2 g, 8 + 2 g + 1, ...: the accumulator columns that the
+// same thread reads back, so that it stores eight neighbouring scores of a centroid and four threads a whole row of 32.
+__host__ __device__ __forceinline__ int64_t table_rows(int64_t rows) { return (rows + 31) & ~(int64_t)31; }
+__host__ __device__ __forceinline__ int64_t table_row(int64_t i) { return (i & ~(int64_t)31) | (i << 2 & 24) | (i >> 2 & 6) | (i & 1); }
 
 // Stage 4 on the tensor cores: rows per query of its digit planes, and the row of query token i.  Within 16 tokens, tokens
 // 4 g ... 4 g + 3 sit in rows 2 g, 2 g + 1, 8 + 2 g, 8 + 2 g + 1: the accumulator columns that the same thread reads back,

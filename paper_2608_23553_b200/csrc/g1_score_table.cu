@@ -16,8 +16,8 @@
 // that one instruction with N = 96 multiplies a centroid digit plane with all three query planes (see the schedule at
 // the MMA loop).  Tensor memory per CTA: 5 accumulators x 32 columns + 96 columns of centroid digits = 256 columns, so
 // two CTAs share an SM.  A producer warp issues the loads and the MMAs; eight warps drain the accumulators (two per
-// tensor-memory lane quarter, a pair of eight-column chunks each).  A draining warp hands the accumulators back as soon
-// as its tcgen05.ld's have landed in registers, so the next tile's MMAs run while it recombines and stores.  An
+// tensor-memory lane quarter; how they share it depends on whether the scores are stored).  A draining warp hands the accumulators
+// back as soon as its tcgen05.ld's have landed in registers, so the next tile's MMAs run while it recombines and stores.  An
 // isolated loop of these instructions runs at half a cycle per column of N (8,192 multiply-adds per SM cycle) but
 // never faster than ~45 cycles per instruction, which is why the instructions here are N = 96 wide (48 cycles).
 // Every wait on an mbarrier is bounded; a wait that gives up sets the workspace's TIMEOUT status bit, and the CTA
@@ -68,8 +68,8 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar)
 //   tile_stride  > 1, sample != 0: the sample tiles 0, s, 2s, ... (tile = blockIdx.x * s).
 //   tile_stride  > 1, sample == 0: all the others (the j-th tile that is not a multiple of s).
 // FILTER (only with the "others"): thr[row] holds, for every query-token row, a lower bound on the score of the row's
-// nprobe-th best centroid (found on the sample; padded to whole tiles of rows); every score >= thr[row] goes, as a (score, centroid) key, into that
-// row's queue (keys[row][cap], counted in cnt[row]; entries past cap are dropped and the count tells).  The top nprobe
+// nprobe-th best centroid (found on the sample; padded to whole tiles of rows); every score >= thr[row] goes, as a (score,
+// centroid) key, into that row's queue (keys[row][cap], counted in cnt[row]; entries past cap are dropped and the count tells).  The top nprobe
 // of a row are then in its queue, so the probe stage never reads the table again, and a search that needs only the
 // probes passes no table (the RaBitQ pipeline: 2.1 GB less to write at Mid, batch 256).
 // redo: a flag per query (nonzero: its rows of these tiles are wanted after all); a CTA without such a query returns.
@@ -247,132 +247,170 @@ score_table_umma(const int8_t *__restrict__ cdig, const __grid_constant__ CUtens
         }
     } else {
         // ============================================================================================ draining warps ===
-        // warp w reads tensor-memory lanes 32 (w % 4) ... + 31 (its centroids); the G1_WPQ warps of a lane quarter
-        // take one pair of adjacent eight-column chunks each
-        const int quad = warp & 3;
-        const int64_t c = c0 + quad * 32 + lane;
-        const uint32_t lane_addr = tmem + ((uint32_t)(quad * 32) << 16);
-        const uint32_t unq = (uint32_t)nq, rows32 = (uint32_t)q_rows;
-        const int first_chunk = 2 * (warp >> 2);
-        const uint32_t col0 = (uint32_t)first_chunk * 8;
+        const uint32_t unq = (uint32_t)nq, n_rows = (uint32_t)q_rows, n_cent = (uint32_t)K;
         unsigned long long pend_key = 0ull, *pend_dst = nullptr;   // FILTER: this thread's last key, not stored yet
         int pend_slot = 0;
-        for (int it = 0; it < my_tiles; ++it) {
-            const uint32_t r0 = (uint32_t)(t_begin + it) * G1_N + col0;      // this warp's first query-token row
-            // FILTER: the thresholds of this warp's 16 query-token rows (the same for every lane), asked for before the wait
-            int32_t thr_v[16];
-            if (FILTER) {
-#pragma unroll
-                for (int g = 0; g < 4; ++g) {
-                    // (rows past the end: 0x7fffffff, in the padding behind the bounds)
-                    const int4 v = __ldg(reinterpret_cast<const int4 *>(tiles.thr + r0) + g);
-                    thr_v[4 * g] = v.x; thr_v[4 * g + 1] = v.y; thr_v[4 * g + 2] = v.z; thr_v[4 * g + 3] = v.w;
-                }
-            }
-            // (the vote makes the decision uniform: the tensor-memory loads below need the whole warp)
-            if (!__all_sync(0xffffffffu, mbar_wait(bar_mma, it & 1, wait_limit))) {
-                if (lane == 0) atomicOr(status, ST_TIMEOUT);
-                break;
-            }
-            tc_fence_after();
-            int32_t accs[2][5][8];
-#pragma unroll
-            for (int w = 0; w < 5; ++w) {
-                tmem_ld8(lane_addr + w * G1_N + col0, accs[0][w]);
-                tmem_ld8(lane_addr + w * G1_N + col0 + 8, accs[1][w]);
-            }
-            tmem_ld_wait();
+        // The slot comes back from the atomic hundreds of cycles later; the key is stored only when this thread's next key
+        // turns up (or at the end), so nobody waits for it.
+        auto push = [&](uint32_t row, uint32_t c, int32_t v) {
+            if (pend_key && pend_slot < tiles.cap) pend_dst[pend_slot] = pend_key;
+            pend_key = key_int(v, (int32_t)c);
+            pend_dst = tiles.keys + (int64_t)row * tiles.cap;
+            pend_slot = atomicAdd(tiles.cnt + row, 1);
+        };
+        // (the vote makes the decision uniform: the tensor-memory loads below need the whole warp)
+        auto wait_tile = [&](int it) {
+            const bool ok = __all_sync(0xffffffffu, mbar_wait(bar_mma, it & 1, wait_limit));
+            if (ok) tc_fence_after();
+            else if (lane == 0) atomicOr(status, ST_TIMEOUT);
+            return ok;
+        };
+        auto hand_back = [&]() {                               // the accumulators may be overwritten from here on
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(bar_empty);             // the accumulators may be overwritten from here on
-
-            // (query, token) coordinates of that row (rows fit 32 bits: n_queries * q_len < 2^23)
-            uint32_t qb = TABLE ? r0 / unq : 0u, qi = TABLE ? r0 - qb * unq : 0u;
-            uint32_t w8[4];                                    // their 8-bit copies
+            if (lane == 0) mbar_arrive(bar_empty);
+        };
+        if (!TABLE) {
+            // Only the keys are wanted, and issue binds.  Warp w reads tensor-memory lanes 32 (w % 4) ... + 31 (a centroid a
+            // thread) and the 16 columns from 16 (w / 4) on: column 8 o + 2 g + b is row 8 g + 2 o + b of the tile (table_row()).
+            // Eight copies of the push take fewer instructions than a mask of the passing rows and the selects of their values (357
+            // per warp and tile with those; Mid, batch 256: 617 -> 541 us).  Rows past the end have the largest threshold.
+            const uint32_t c = (uint32_t)c0 + (warp & 3) * 32 + lane;
+            const int group = warp >> 2;
+            const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + 16 * group;
+            for (int it = 0; it < my_tiles; ++it) {
+                const uint32_t r0 = (uint32_t)(t_begin + it) * G1_N + 4 * group;
+                int32_t thr_v[16];                             // by column; the same for every lane, asked for before the wait
 #pragma unroll
-            for (int ch = 0; ch < 2; ++ch) {
-                int32_t out[8];
+                for (int g = 0; g < 4; ++g) {
+                    const int4 v = __ldg(reinterpret_cast<const int4 *>(tiles.thr + r0 + 8 * g));
+                    thr_v[2 * g] = v.x; thr_v[2 * g + 1] = v.y; thr_v[8 + 2 * g] = v.z; thr_v[8 + 2 * g + 1] = v.w;
+                }
+                if (!wait_tile(it)) break;
+                int32_t accs[2][5][8];
 #pragma unroll
-                for (int e = 0; e < 8; ++e)
-                    out[e] = combine_digits(accs[ch][0][e], accs[ch][1][e], accs[ch][2][e], accs[ch][3][e], accs[ch][4][e]);
-                const uint32_t rc = r0 + 8 * ch;               // first query-token row of this chunk
-                if (FILTER && c < K) {
-                    bool any = false;
+                for (int w = 0; w < 5; ++w) {
+                    tmem_ld8(lane_addr + w * G1_N, accs[0][w]);
+                    tmem_ld8(lane_addr + w * G1_N + 8, accs[1][w]);
+                }
+                tmem_ld_wait();
+                hand_back();
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) any |= out[e] >= thr_v[ch * 8 + e];
-                    if (any) {                  // about nprobe x tile_stride keys per row in all: one lane of a warp every
+                for (int o = 0; o < 2; ++o) {
+                    int32_t out[8];
+#pragma unroll
+                    for (int x = 0; x < 8; ++x)
+                        out[x] = combine_digits(accs[o][0][x], accs[o][1][x], accs[o][2][x], accs[o][3][x], accs[o][4][x]);
+                    if (c < n_cent) {
+                        bool any = false;
+#pragma unroll
+                        for (int x = 0; x < 8; ++x) any |= out[x] >= thr_v[8 * o + x];
+                        if (any) {              // about nprobe x tile_stride keys per row in all: one lane of a warp every
                                                 // few chunks, and then hardly ever two values of the lane
-                        // The slot comes back from the atomic hundreds of cycles later; the key is stored only when
-                        // this thread's next key turns up (or at the end), so nobody waits for it.
-                        auto push = [&](int e, int32_t v) {
-                            if (pend_key && pend_slot < tiles.cap) pend_dst[pend_slot] = pend_key;
-                            const uint32_t row = rc + e;
-                            pend_key = key_int(v, (int32_t)c);
-                            pend_dst = tiles.keys + (int64_t)row * tiles.cap;
-                            pend_slot = atomicAdd(tiles.cnt + row, 1);
-                        };
-                        // (Rows past the end have the largest threshold: they never pass.)  Issue binds the tiles that
-                        // are not stored (357 instructions per warp and tile): eight copies of the push take fewer than the
-                        // mask and the selects (Mid, batch 256: 617 -> 562 us).  Where the stores of the scores bind, the
-                        // copies cost more than they save (768 -> 796 us): there a loop over the few that pass.
-                        if (!TABLE) {
 #pragma unroll
-                            for (int e = 0; e < 8; ++e)
-                                if (out[e] >= thr_v[ch * 8 + e]) push(e, out[e]);
-                        } else {
+                            for (int x = 0; x < 8; ++x)
+                                if (out[x] >= thr_v[8 * o + x]) push(r0 + 8 * (x >> 1) + 2 * o + (x & 1), c, out[x]);
+                        }
+                    }
+                }
+            }
+        } else {
+            // Warp w reads tensor-memory lanes 32 (w % 4) + 16 (w / 4) ... + 15 and all 32 columns: a thread gets eight
+            // neighbouring query-token rows (table_row()) of two centroids, and a warp's store is a kilobyte in a row at 32 tokens.
+            // With a thread per centroid and 16 rows a store was 32 pieces of 32 lines, and the stores' wavefronts (65 % of the
+            // unit's) were what bound the kernel.  Mid, batch 256: 772 -> 685 us; 262,144 centroids 2,857 -> 2,533.
+            // 16 columns at a time: all 32 at once need the thresholds loaded late for want of registers (702 us).
+            const uint32_t c_first = (uint32_t)c0 + (warp & 3) * 32 + (warp >> 2) * 16 + (lane >> 2);      // and c_first + 8
+            const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32 + (warp >> 2) * 16) << 16);
+            for (int it = 0; it < my_tiles; ++it) {
+                const uint32_t rc = (uint32_t)(t_begin + it) * G1_N + 8 * (lane & 3);          // this thread's first query-token row
+                // FILTER: the thresholds of its eight rows, asked for before the wait
+                int32_t thr_v[8];
+                if (FILTER) {
+#pragma unroll
+                    for (int g = 0; g < 2; ++g) {
+                        // (rows past the end: 0x7fffffff, in the padding behind the bounds)
+                        const int4 v = __ldg(reinterpret_cast<const int4 *>(tiles.thr + rc) + g);
+                        thr_v[4 * g] = v.x; thr_v[4 * g + 1] = v.y; thr_v[4 * g + 2] = v.z; thr_v[4 * g + 3] = v.w;
+                    }
+                }
+                if (!wait_tile(it)) break;
+                int32_t scores[2][8];                              // of the two centroids
+#pragma unroll
+                for (int o = 0; o < 2; ++o) {
+                    int32_t accs[5][8];
+#pragma unroll
+                    for (int w = 0; w < 5; ++w) tmem_ld_16x16(lane_addr + w * G1_N + 16 * o, accs[w]);
+                    tmem_ld_wait();
+                    if (o == 1) hand_back();
+#pragma unroll
+                    for (int x = 0; x < 8; ++x)
+                        scores[x >> 1 & 1][4 * o + (x >> 2) * 2 + (x & 1)] =
+                            combine_digits(accs[0][x], accs[1][x], accs[2][x], accs[3][x], accs[4][x]);
+                }
+
+                // (query, token) coordinates of the first row (rows fit 32 bits: n_queries * q_len < 2^23)
+                const uint32_t qb0 = rc / unq, qi0 = rc - qb0 * unq;
+#pragma unroll
+                for (int half = 0; half < 2; ++half) {
+                    const uint32_t c = c_first + 8 * half;
+                    const int32_t (&out)[8] = scores[half];
+                    if (FILTER && c < n_cent) {
+                        bool any = false;
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) any |= out[e] >= thr_v[e];
+                        if (any) {                  // about nprobe x tile_stride keys per row in all: one lane of a warp every
+                                                    // few chunks, and then hardly ever two values of the lane
                             uint32_t pass = 0u;
 #pragma unroll
-                            for (int e = 0; e < 8; ++e) pass |= out[e] >= thr_v[ch * 8 + e] ? 1u << e : 0u;
-                            while (pass) {
+                            for (int e = 0; e < 8; ++e) pass |= out[e] >= thr_v[e] ? 1u << e : 0u;
+                            while (pass) {          // (eight copies of the push, as above, are slower here: 768 -> 796 us)
                                 const int e = __ffs(pass) - 1;
                                 pass &= pass - 1;
                                 int32_t v = out[0];
 #pragma unroll
                                 for (int x = 1; x < 8; ++x) v = e == x ? out[x] : v;
-                                push(e, v);
+                                push(rc + e, c, v);
                             }
                         }
                     }
-                }
-                if (TABLE && c < K && rc < rows32) {
-                    if (table8 != nullptr) {
-                        // coarse copy for the bound phase of stage 3: clamp(S >> 16, 0, 255); q_len is a multiple of 16 here,
-                        // so the 16 rows of a warp belong to one query: one 16-byte store for both chunks
+                    if (c < n_cent && rc < n_rows) {
+                        uint32_t qb = qb0, qi = qi0;
+                        const int64_t at = ((int64_t)qb * K + c) * nq + qi;
+                        if (table8 != nullptr) {
+                            // coarse copy for the bound phase of stage 3: clamp(S >> 16, 0, 255); q_len is a multiple of 16 here,
+                            // so the eight rows belong to one query
+                            uint32_t w8[2];
 #pragma unroll
-                        for (int g = 0; g < 2; ++g) {
-                            uint32_t v[4];
+                            for (int g = 0; g < 2; ++g) {
+                                uint32_t v[4];
 #pragma unroll
-                            for (int e = 0; e < 4; ++e) v[e] = (uint32_t)__vimin_s32_relu(out[4 * g + e] >> 16, 255);
-                            w8[2 * ch + g] =
-                                __byte_perm(__byte_perm(v[0], v[1], 0x0040), __byte_perm(v[2], v[3], 0x0040), 0x5410);
+                                for (int e = 0; e < 4; ++e) v[e] = (uint32_t)__vimin_s32_relu(out[4 * g + e] >> 16, 255);
+                                w8[g] = __byte_perm(__byte_perm(v[0], v[1], 0x0040), __byte_perm(v[2], v[3], 0x0040), 0x5410);
+                            }
+                            *reinterpret_cast<uint2 *>(table8 + at) = make_uint2(w8[0], w8[1]);
                         }
-                        if (ch == 1)
-                            *reinterpret_cast<uint4 *>(table8 + ((int64_t)qb * K + c) * nq + qi - 8) =
-                                make_uint4(w8[0], w8[1], w8[2], w8[3]);
-                    }
-                    if ((nq & 7) == 0) {
-                        // the chunk's eight values are consecutive tokens of one query, 32-byte aligned: one store
-                        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(
-                                         table + ((int64_t)qb * K + c) * nq + qi),
-                                     "r"(out[0]), "r"(out[1]), "r"(out[2]), "r"(out[3]), "r"(out[4]), "r"(out[5]),
-                                     "r"(out[6]), "r"(out[7])
-                                     : "memory");
-                        qi += 8;
-                        if (qi >= unq) { qi -= unq; ++qb; }
-                    } else if ((nq & 3) == 0) {
+                        if ((nq & 7) == 0) {
+                            // eight consecutive tokens of one query, 32-byte aligned: one store
+                            asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(table + at),
+                                         "r"(out[0]), "r"(out[1]), "r"(out[2]), "r"(out[3]), "r"(out[4]), "r"(out[5]),
+                                         "r"(out[6]), "r"(out[7])
+                                         : "memory");
+                        } else if ((nq & 3) == 0) {
 #pragma unroll
-                        for (int e = 0; e < 8; e += 4) {
-                            if (rc + e < rows32)                          // q_rows is a multiple of 4 here
-                                *reinterpret_cast<int4 *>(table + ((int64_t)qb * K + c) * nq + qi) =
-                                    make_int4(out[e], out[e + 1], out[e + 2], out[e + 3]);
-                            qi += 4;
-                            if (qi >= unq) { qi -= unq; ++qb; }           // groups of four never straddle two queries
-                        }
-                    } else {
+                            for (int e = 0; e < 8; e += 4) {
+                                if (rc + e < n_rows)                          // q_rows is a multiple of 4 here
+                                    *reinterpret_cast<int4 *>(table + ((int64_t)qb * K + c) * nq + qi) =
+                                        make_int4(out[e], out[e + 1], out[e + 2], out[e + 3]);
+                                qi += 4;
+                                if (qi >= unq) { qi -= unq; ++qb; }           // groups of four never straddle two queries
+                            }
+                        } else {
 #pragma unroll
-                        for (int e = 0; e < 8; ++e) {
-                            if (rc + e < rows32) table[((int64_t)qb * K + c) * nq + qi] = out[e];
-                            if (++qi == unq) { qi = 0; ++qb; }
+                            for (int e = 0; e < 8; ++e) {
+                                if (rc + e < n_rows) table[((int64_t)qb * K + c) * nq + qi] = out[e];
+                                if (++qi == unq) { qi = 0; ++qb; }
+                            }
                         }
                     }
                 }
@@ -464,10 +502,10 @@ int launch_score_table(const Index &ix, const Params &p, const float *queries, i
                        uint8_t *table8, uint32_t *status, cudaStream_t st, uint32_t *clear, int64_t clear_n)
 {
     const int64_t rows = (int64_t)p.B * p.nq;
-    int rc = launch_digits(queries, rows, ix.D, ix.nbits, qdig, qdig4, p.nq, status, st, clear, clear_n);
+    int rc = launch_digits(queries, rows, ix.D, ix.nbits, qdig, true, qdig4, p.nq, status, st, clear, clear_n);
     if (rc) return rc;
     CUtensorMap map_q;
-    if ((rc = make_plane_map(&map_q, qdig, rows, G1_N, 3))) return rc;        // one load brings a tile's three planes
+    if ((rc = make_plane_map(&map_q, qdig, table_rows(rows), G1_N, 3))) return rc;        // one load brings a tile's three planes
     const G1Tiles all = {0, 0, nullptr, nullptr, nullptr, 0, nullptr};
     if ((rc = launch_g1_tiles<false, true>(ix, p, map_q, (int)((ix.K + G1_M - 1) / G1_M), table, table8, status, all, st)))
         return rc;
@@ -486,10 +524,10 @@ int launch_score_table_probes(const Index &ix, const Params &p, const Layout &L,
                               uint32_t *clear, int64_t clear_n)
 {
     const int64_t rows = (int64_t)p.B * p.nq;
-    int rc = launch_digits(queries, rows, ix.D, ix.nbits, qdig, qdig4, p.nq, status, st, clear, clear_n);
+    int rc = launch_digits(queries, rows, ix.D, ix.nbits, qdig, true, qdig4, p.nq, status, st, clear, clear_n);
     if (rc) return rc;
     CUtensorMap map_q;
-    if ((rc = make_plane_map(&map_q, qdig, rows, G1_N, 3))) return rc;
+    if ((rc = make_plane_map(&map_q, qdig, table_rows(rows), G1_N, 3))) return rc;
     const int c_tiles = (int)((ix.K + G1_M - 1) / G1_M);
     const int stride = L.pq_stride;
     const int n_sample = (c_tiles + stride - 1) / stride;
@@ -512,7 +550,7 @@ int launch_score_table_redo(const Index &ix, const Params &p, const Layout &L, c
                             const int32_t *redo, uint32_t *status, cudaStream_t st)
 {
     CUtensorMap map_q;
-    const int rc = make_plane_map(&map_q, qdig, (int64_t)p.B * p.nq, G1_N, 3);
+    const int rc = make_plane_map(&map_q, qdig, table_rows((int64_t)p.B * p.nq), G1_N, 3);
     if (rc) return rc;
     const int c_tiles = (int)((ix.K + G1_M - 1) / G1_M);
     const int n_sample = (c_tiles + L.pq_stride - 1) / L.pq_stride;

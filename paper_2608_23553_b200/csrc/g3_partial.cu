@@ -177,7 +177,7 @@ partial_score_kernel(const int8_t *__restrict__ qdig, const int32_t *__restrict_
     __shared__ __align__(16) QueryDigits dig;
     const int b = blockIdx.y;
     const int i = blockIdx.x / splits;
-    load_query_digits(dig, qdig, (int64_t)B * nq, (int64_t)b * nq + i);
+    load_query_digits(dig, qdig, table_rows((int64_t)B * nq), table_row((int64_t)b * nq + i));
     __syncthreads();
     const double d4 = __dmul_rn((double)delta, 4.0);
     const double kterm = __dmul_rn(__dmul_rn((double)kappa, 4.0), (double)query_sum(dig));

@@ -117,7 +117,7 @@ static int exclusive_scan(const int32_t *in, int64_t n, int64_t *out, int64_t *t
 constexpr int DIGIT_PITCH = 128;
 constexpr long long MAX_ROW_SQUARE_SUM = (1LL << 44) + (1LL << 35);
 
-__global__ void digits_kernel(const float *__restrict__ x, int64_t rows, int D, int nbits, int8_t *__restrict__ dig,
+__global__ void digits_kernel(const float *__restrict__ x, int64_t rows, int D, int nbits, int8_t *__restrict__ dig, bool tiles,
                               int8_t *__restrict__ dig4, int q_len, uint32_t *status, uint32_t *__restrict__ clear,
                               int64_t clear_n)
 {
@@ -147,9 +147,11 @@ __global__ void digits_kernel(const float *__restrict__ x, int64_t rows, int D, 
         d2 = (X1 - d1) >> 8;
     }
     if (i < n && dig) {
-        dig[i] = (int8_t)d0;
-        dig[n + i] = (int8_t)d1;
-        dig[2 * n + i] = (int8_t)d2;
+        const int64_t plane = (tiles ? table_rows(rows) : rows) * DIGIT_PITCH;
+        int8_t *at = dig + (tiles ? table_row(r) : r) * DIGIT_PITCH + i % DIGIT_PITCH;
+        at[0] = (int8_t)d0;
+        at[plane] = (int8_t)d1;
+        at[2 * plane] = (int8_t)d2;
     }
     if (i < n && dig4) {
         const int per = residual_rows(q_len);
@@ -167,11 +169,11 @@ __global__ void digits_kernel(const float *__restrict__ x, int64_t rows, int D, 
         atomicOr(status, ST_BAD_QUERY);
 }
 
-int launch_digits(const float *x, int64_t rows, int D, int nbits, int8_t *dig, int8_t *dig4, int q_len, uint32_t *status,
-                  cudaStream_t st, uint32_t *clear, int64_t clear_n)
+int launch_digits(const float *x, int64_t rows, int D, int nbits, int8_t *dig, bool tiles, int8_t *dig4, int q_len,
+                  uint32_t *status, cudaStream_t st, uint32_t *clear, int64_t clear_n)
 {
     const int64_t n = rows * DIGIT_PITCH;
-    launch(digits_kernel, (unsigned)((n + 255) / 256), 256, 0, st, x, rows, D, nbits, dig, dig4, q_len, status, clear,
+    launch(digits_kernel, (unsigned)((n + 255) / 256), 256, 0, st, x, rows, D, nbits, dig, tiles, dig4, q_len, status, clear,
            clear_n);
     CHIMERA_CUDA(cudaGetLastError());
     return CHIMERA_OK;
@@ -413,7 +415,7 @@ int build_index_device(Index &ix, const float *centroids, const int32_t *doclens
     // centroid digit planes
     BUILD_CUDA(cudaMalloc(&ix.cdig, (size_t)3 * ix.K * DIGIT_PITCH));
     BUILD_CUDA(cudaMemsetAsync(flags, 0, sizeof(int32_t), st));
-    rc = launch_digits(centroids, ix.K, ix.D, ix.nbits, ix.cdig, nullptr, 1, (uint32_t *)flags, st);
+    rc = launch_digits(centroids, ix.K, ix.D, ix.nbits, ix.cdig, false, nullptr, 1, (uint32_t *)flags, st);
     if (rc) { cleanup(); return rc; }
 
     // inverted file
