@@ -165,9 +165,11 @@ ci_wide_kernel(const int32_t *__restrict__ table, int64_t K, const int32_t *__re
 }
 
 // The wide variant over precomputed token ranges (first token, length) of the documents to score: a warp owns a
-// contiguous run of them and takes them 32 at a time -- one coalesced load of the ranges, handed out by shuffle, and the
-// first centroid ids of the next document fetched while the current one is scored -- instead of the dependent chain
-// id -> offsets -> centroid ids per document.
+// contiguous run of them and takes them 32 at a time -- one coalesced load of the ranges, handed out by shuffle -- instead of the
+// dependent chain id -> offsets -> centroid ids per document.  Latency is the limit (79 % of the stalls; a third of the rows come
+// from DRAM), so the next 32 centroid ids, of this document or the next, are always on their way while rows are looked up: Mid,
+// batch 256, 1,077 -> 1,041 us; 512-token documents, 64 queries of 64 tokens, 1,951 -> 1,792.  32 bytes a lane instead of 16 are
+// no faster (1,097, 1,834), and rows that L1 does not keep much slower (1,440).
 template <int LPR>
 __global__ void __launch_bounds__(CI_THREADS)
 ci_wide_rng_kernel(const int32_t *__restrict__ table, int64_t K, const int2 *__restrict__ rng,
@@ -205,17 +207,20 @@ ci_wide_rng_kernel(const int32_t *__restrict__ table, int64_t K, const int2 *__r
         }
         for (int di = 0; di < cnt_docs; ++di) {
             const int t0 = __shfl_sync(0xffffffffu, mine.x, di), len = __shfl_sync(0xffffffffu, mine.y, di);
-            int32_t cidv = nx_cid;
-            if (di + 1 < cnt_docs) {
-                const int n0 = __shfl_sync(0xffffffffu, mine.x, di + 1), nl = __shfl_sync(0xffffffffu, mine.y, di + 1);
-                nx_cid = cids[DBG_TOK((int64_t)n0 + (lane < nl - 1 ? lane : nl > 0 ? nl - 1 : 0))];
-            }
-            if (len == 0) continue;
+            const int n0 = __shfl_sync(0xffffffffu, mine.x, di + 1 < cnt_docs ? di + 1 : di);
+            const int nl = __shfl_sync(0xffffffffu, mine.y, di + 1 < cnt_docs ? di + 1 : di);
             int4 m = make_int4(INT_MIN, INT_MIN, INT_MIN, INT_MIN);
-            for (int base = 0; base < len; base += 32) {
+            for (int base = 0; base < len || base == 0; base += 32) {
                 const int cnt = len - base < 32 ? len - base : 32;
-                // lanes past the end repeat the last token: a duplicate cannot change a maximum
-                if (base != 0) cidv = cids[DBG_TOK((int64_t)t0 + base + (lane < cnt ? lane : cnt - 1))];
+                // the next 32 ids, of this document or the next one, travel with the rows of these; lanes past the end repeat the
+                // last token: a duplicate cannot change a maximum
+                const int32_t cidv = nx_cid;
+                {
+                    const bool more = base + 32 < len;
+                    const int64_t f0 = more ? (int64_t)t0 + base + 32 : n0;
+                    const int fl = more ? len - base - 32 : nl;
+                    nx_cid = cids[DBG_TOK(f0 + (lane < fl - 1 ? lane : fl > 0 ? fl - 1 : 0))];
+                }
                 for (int s = 0; s * TPL < cnt; s += UNROLL) {
                     int4 v[UNROLL];
 #pragma unroll
@@ -234,6 +239,7 @@ ci_wide_rng_kernel(const int32_t *__restrict__ table, int64_t K, const int2 *__r
                     }
                 }
             }
+            if (len == 0) continue;
 #pragma unroll
             for (int o = LPR; o < 32; o <<= 1) {           // merge the TPL lane groups
                 m.x = max(m.x, __shfl_xor_sync(0xffffffffu, m.x, o));
