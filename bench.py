@@ -104,7 +104,7 @@ NCU_CI_DRAM_PER_ALGORITHMIC_BYTE = {
     None: (0.939, "an ncu capture (Mid corpus, batch 8)"),
 }
 # ... and the same of the launches that bound and seed stage 3 when its first cut runs.
-NCU_CUT_DRAM_PER_ALGORITHMIC_BYTE = (0.883, "an ncu capture (Mid corpus, batch 64)")
+NCU_CUT_DRAM_PER_ALGORITHMIC_BYTE = (0.883, "an ncu capture of the form that scans by query (Mid corpus, batch 64)")
 NCU_PARTIAL_DRAM_PER_QUERY = (463.5e6 / 64.0, "an ncu capture of the visits and their sums (Mid corpus, batch 64; bytes "
                                             "per query)")
 
@@ -665,13 +665,13 @@ def measure(pkg, cfg, corp, q, index, args, device, mode="ci", dist=None, local_
     if mode == "ci":
         ratio, src = NCU_CI_DRAM_PER_ALGORITHMIC_BYTE.get(cfg.name, NCU_CI_DRAM_PER_ALGORITHMIC_BYTE[None])
         frac = gbs(ci_bytes, ci_ms) / peak
-        # with the first cut stage 3's bounds are seven launches instead of one
+        # with the first cut stage 3's bounds are many launches instead of one
         first_cut = launches["centroid_interaction"] >= 3 * n_prof
         if first_cut:
             ratio, src = NCU_CUT_DRAM_PER_ALGORITHMIC_BYTE
         roofline = {
-            "kernel": ("filter_scan_kernel + ci_coarse_rng_kernel + ci_wide_rng_kernel (stage 3: one number per candidate token "
-                       "from shared memory, 8-bit rows of the documents that keeps, exact rows of the seeds)" if first_cut else
+            "kernel": ("filter_scan_kernel or batch_scan_kernel + ci_bound_kernel + ci_rest_kernel + ci_wide_rng_kernel (stage 3: one "
+                       "number per candidate token, 8-bit rows of the documents that keeps, exact rows of the seeds)" if first_cut else
                        "ci_coarse_rng_kernel (stage 3 bound scan over every candidate token)"), "bound": "hbm",
             "achieved": gbs(ci_bytes, ci_ms), "peak": peak, "peak_kind": peak_kind, "unit": "GB/s", "frac": frac,
             "frac_of_nominal_8_tb_s": gbs(ci_bytes, ci_ms) / 8000.0,       # the task quotes ~8 TB/s; context only
@@ -685,7 +685,7 @@ def measure(pkg, cfg, corp, q, index, args, device, mode="ci", dist=None, local_
                                "costs a random lookup, in shared memory (about 3.5 bank conflicts each 32) or of a 32-byte "
                                "row through L1/L2, which binds the kernel" % ("met" if frac >= TARGET else "NOT met")},
             "contender_fraction": mean("contenders") / max(mean("cand"), 1.0),
-            # with the first cut no single rate binds the seven launches (the lookups of filter_scan_kernel alone run at 71 % of
+            # with the first cut no single rate binds its launches (the lookups of filter_scan_kernel alone run at 71 % of
             # the shared-memory wavefront peak in an ncu capture)
             "first_cut_kept_fraction": mean("kept") / max(mean("cand"), 1.0) if first_cut else None,
             "binding_roof": None if first_cut else
