@@ -15,9 +15,9 @@
 // loads (lane = token), each is broadcast with a shuffle, and the warp gathers the table row S[cid, :] with
 // lane = query token (one 128-byte line for 32 query tokens), keeping a running maximum per lane.
 //
-// select_kernel: one block per query.  Few of many: select_few.  Else radix select (11 + 11 + 10 bits) of the n_prune-th largest score, then an
-// ordered compaction of the candidate list (which is ascending in id), so equal scores are resolved towards smaller
-// ids and the survivors come out ascending.  With few queries per call the contender and selection steps run over 32
+// select_kernel: one block per query.  Few of many: select_few.  Else radix select (11 + 11 + 10 bits) of the n_prune-th
+// largest score, then an ordered compaction of the candidate list (which is ascending in id), so equal scores are resolved
+// towards smaller ids and the survivors come out ascending.  With few queries per call the contender and selection steps run over 32
 // blocks per query instead (contender_hist/count/write kernels, sels_* kernels), and shard_select_kernel merges the
 // lists of a document-sharded search.
 #include <limits.h>
@@ -607,9 +607,9 @@ ci_coarse_rng_kernel(const uint8_t *__restrict__ table8, int64_t K, const int2 *
 // reaches tau, one in six, go on to ci_rest_kernel.
 // Measured (all kept documents at once / both kernels): Mid, batch 256, 1,717 us / 988 + 385; 512-token documents, 64 queries of
 // 64 tokens, 1,795 / 856 + 223; 262,144 centroids, batch 256, 4,458 / 2,724 + 1,034.
-// With few rows left to look up the instructions around them count (a document per warp: 1,890 us, 570 instructions each), so four documents share a warp, eight lanes each, those of
-// a group of 32 taken by length: a bit per token from shared memory says whether it is near, near ids are collected in
-// shared memory and their rows looked up 8 / LPR at a time and document.  nq: the columns that count; those up to 16 LPR are
+// With few rows left to look up the instructions around them count (a document per warp: 1,890 us, 570 instructions each), so four
+// documents share a warp, eight lanes each, those of a group of 32 taken by length: a bit per token from shared memory says
+// whether it is near, near ids are collected in shared memory and their rows looked up 8 / LPR at a time and document.  nq: the columns that count; those up to 16 LPR are
 // zero in every row.  rng: token ranges; (CI, 0) stands for a document whose CI is known.
 constexpr int BOUND_THREADS = 512;
 constexpr int BOUND_LIST = 64, BOUND_PITCH = BOUND_LIST + 8;

@@ -190,14 +190,15 @@ partial_score_kernel(const int8_t *__restrict__ qdig, const int32_t *__restrict_
     int64_t e0;
     // (the document's bitmap word and rank come as an argument: they depend on the list entry alone, so their load is
     // issued with the code loads instead of after the score is known -- one memory latency less per visit)
-    auto update = [&](int64_t e, uint32_t d, int T, uint2 r) {
+    VisitPush push[2];
+    auto update = [&](int n, int64_t e, uint32_t d, int T, uint2 r) {
         const double x = __dadd_rn(__dmul_rn(d4, (double)T), kterm);
         const long long dist = (long long)s_c + __double2ll_rn(x);
         if (dist > 0) {                                // the table starts at 0 (Algorithm 2)
             const int64_t rank = (int64_t)r.y + __popc(r.x & ((1u << (d & 31)) - 1u));
             if (rank < maxc && DBG_RANK_OK(rank)) {
                 if (LISTS) {
-                    visit_push(heads + rank, nodes, v0 + (uint32_t)(e - e0), i, (uint32_t)dist);
+                    visit_begin(push[n], heads + rank, v0 + (uint32_t)(e - e0), i, (uint32_t)dist);
                 } else {
                     // F' = sum_i M[., i] is kept up to date with the increments: M only grows, integer adds commute
                     const int32_t old = atomicMax(&Mb[rank * nq + i], (int32_t)dist);
@@ -223,12 +224,14 @@ partial_score_kernel(const int8_t *__restrict__ qdig, const int32_t *__restrict_
                 d[n] = (uint32_t)DBG_DOC(tok_doc[at[n]]);
                 r[n] = __ldg(rk + (d[n] >> 5));
             }
+            if (LISTS) { visit_end(push[0], nodes); visit_end(push[1], nodes); }
             int T[2];
             code_dots<NBITS, 2>(T, w, CW, dig);
-            update(at[0], d[0], T[0], r[0]);
-            if (at[1] != e) update(at[1], d[1], T[1], r[1]);
+            update(0, at[0], d[0], T[0], r[0]);
+            if (at[1] != e) update(1, at[1], d[1], T[1], r[1]);
         }
     }
+    if (LISTS) { visit_end(push[0], nodes); visit_end(push[1], nodes); }
 }
 
 int launch_partial_scores(const Index &ix, const Params &p, const Layout &L, const int8_t *qdig,

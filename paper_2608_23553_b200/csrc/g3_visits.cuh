@@ -36,12 +36,27 @@ int launch_visit_clear(const Index &ix, const Params &p, const VisitLists &v, co
 int launch_visit_sum(const Index &ix, const Params &p, const VisitLists &v, bool floats, const int32_t *n_cand,
                      int32_t *fprime, cudaStream_t st);
 
-__device__ __forceinline__ void visit_push(unsigned long long *head /* of the candidate */, unsigned long long *nodes, uint32_t v,
-                                           int i, uint32_t score)
+// In two halves: the exchange's answer comes back hundreds of cycles later, so it is put away behind the loads of the next visits.
+// (Put away at once, with the branch on it, every visit of a thread
+// waited for the one before: 1-bit codes, Mid, batch 256, 503 us, so 488; residual codes 623 either way.)
+struct VisitPush {
+    unsigned long long *head = nullptr;                  // of the candidate; NULL: nothing pending
+    unsigned long long before;
+    uint32_t v;
+};
+__device__ __forceinline__ void visit_begin(VisitPush &push, unsigned long long *head, uint32_t v, int i, uint32_t score)
 {
-    const unsigned long long before = atomicExch(head, (unsigned long long)score << 32 | (v + 1) << VISIT_I_BITS | (uint32_t)i);
-    nodes[v] = before & ~VISIT_MORE;
-    if (before) atomicOr(head, VISIT_MORE);
+    push.head = head;
+    push.v = v;
+    push.before = atomicExch(head, (unsigned long long)score << 32 | (v + 1) << VISIT_I_BITS | (uint32_t)i);
+}
+__device__ __forceinline__ void visit_end(VisitPush &push, unsigned long long *nodes)
+{
+    if (push.head) {
+        nodes[push.v] = push.before & ~VISIT_MORE;
+        if (push.before) atomicOr(push.head, VISIT_MORE);
+        push.head = nullptr;
+    }
 }
 // The visit before this one, 0 = none.
 __device__ __forceinline__ unsigned long long visit_before(unsigned long long visit, const unsigned long long *nodes)

@@ -110,12 +110,13 @@ rabitq_partial_kernel(const int8_t *__restrict__ qdig, int nq, int B, int CW, in
     int64_t e0;
     // (the token's factor, the document's bitmap word and its rank come as arguments: they depend on the list entry
     // alone, so their loads are issued with the code loads instead of one after the other behind the score)
-    auto update = [&](int64_t e, uint32_t d, float factor, int T, uint2 r) {
+    VisitPush push[2];
+    auto update = [&](int n, int64_t e, uint32_t d, float factor, int T, uint2 r) {
         const float est = __fmul_rn(factor, __fmul_rn(c, (float)(2 * T - sq)));
         if (est > 0.0f) {                              // the table starts at 0 (Algorithm 2)
             const int64_t rank = (int64_t)r.y + __popc(r.x & ((1u << (d & 31)) - 1u));
             if (rank < maxc && DBG_RANK_OK(rank)) {
-                if (LISTS) visit_push(heads + rank, nodes, v0 + (uint32_t)(e - e0), i, __float_as_uint(est));
+                if (LISTS) visit_begin(push[n], heads + rank, v0 + (uint32_t)(e - e0), i, __float_as_uint(est));
                 else atomicMax(&Mb[rank * nq + i], __float_as_int(est));
             }
         }
@@ -139,12 +140,14 @@ rabitq_partial_kernel(const int8_t *__restrict__ qdig, int nq, int B, int CW, in
                 d[n] = (uint32_t)DBG_DOC(tok_doc[at[n]]);
                 r[n] = __ldg(rk + (d[n] >> 5));
             }
+            if (LISTS) { visit_end(push[0], nodes); visit_end(push[1], nodes); }
             int T[2];
             code_dots<1, 2>(T, w, CW, dig);
-            update(at[0], d[0], f[0], T[0], r[0]);
-            if (at[1] != e) update(at[1], d[1], f[1], T[1], r[1]);
+            update(0, at[0], d[0], f[0], T[0], r[0]);
+            if (at[1] != e) update(1, at[1], d[1], f[1], T[1], r[1]);
         }
     }
+    if (LISTS) { visit_end(push[0], nodes); visit_end(push[1], nodes); }
 }
 
 // grid (blocks, B): F'[b][j] = M[b][j][0] + M[b][j][1] + ... in that order (fp32), one thread per candidate.
