@@ -375,14 +375,14 @@ static int run(const Index &ix, const Params &p, int first, int last, const floa
             if ((rc = launch_rabitq_partial(ix, p, L, qdig_rot, probes, ranks, n_cand, partial_m, ci, st)))
                 return rc;
             prof_mark(SLOT_CI, st);
-            if ((rc = launch_select(ix, p, cand, n_cand, ci, pruned, n_pruned, pruned_ci, sel_scratch, st))) return rc;
+            if ((rc = launch_select(ix, p, cand, n_cand, ci, pruned, n_pruned, pruned_ci, sel_scratch, true, st))) return rc;
             prof_mark(SLOT_SELECT, st);
         } else if (partial) {
             // the paper's candidate refinement: partial scores from the retrieved tokens only, then the same selection
             if ((rc = launch_partial_scores(ix, p, L, qdig, table, probes, ranks, n_cand, partial_m, ci, st)))
                 return rc;
             prof_mark(SLOT_CI, st);
-            if ((rc = launch_select(ix, p, cand, n_cand, ci, pruned, n_pruned, pruned_ci, sel_scratch, st))) return rc;
+            if ((rc = launch_select(ix, p, cand, n_cand, ci, pruned, n_pruned, pruned_ci, sel_scratch, true, st))) return rc;
             prof_mark(SLOT_SELECT, st);
         } else {
             if (two_phase && first > 1) {          // the table came from the caller: derive its coarse copy
@@ -435,7 +435,7 @@ static int run(const Index &ix, const Params &p, int first, int last, const floa
                 return rc;
             prof_mark(short_list ? SLOT_CI_EXACT : SLOT_CI, st);
             if ((rc = launch_select(ix, p, docs, n_docs, ci, pruned, n_pruned, pruned_ci, short_list ? nullptr : sel_scratch,
-                                    st)))
+                                    !short_list, st)))
                 return rc;
             prof_mark(SLOT_SELECT, st);
         }

@@ -321,7 +321,7 @@ int launch_centroid_interaction(const Index &ix, const Params &p, const int32_t 
 bool select_split_used(const Index &ix, const Params &p);
 size_t select_split_scratch_bytes(const Index &ix, const Params &p);
 int launch_select(const Index &ix, const Params &p, const int32_t *cand, const int32_t *n_cand, const int32_t *ci,
-                  int32_t *pruned, int32_t *n_pruned, int32_t *pruned_ci, int32_t *scratch, cudaStream_t st);
+                  int32_t *pruned, int32_t *n_pruned, int32_t *pruned_ci, int32_t *scratch, bool many, cudaStream_t st);
 // Document-sharded search: the global top-n_prune of the shards' lists and the final top-k merge.
 int launch_shard_export(const Params &p, const int32_t *pruned, const int32_t *pruned_ci, int64_t doc_base,
                         int32_t *out_ids, int32_t *out_ci, cudaStream_t st);

@@ -977,7 +977,8 @@ int launch_centroid_interaction(const Index &ix, const Params &p, const int32_t 
 // more), one pass collects those in shared memory, and the selection and the order of the survivors are found there.  False,
 // with nothing written: the bound let too few through or more than there is room for; the caller selects among all then.
 // Measured (1,024 wanted of Mid's candidates, 1-bit refinement): 256 queries 122 -> 50 us, 64 queries 69 -> 30 us.
-constexpr int SEL_SAMPLE = 8192, SEL_FEW = 3584, SEL_BINS = 2048;
+// Room for 7,168 serves 4,096 wanted too (4 million documents, 64 queries, 1-bit codes: 1,798 -> 1,742 us a call; 3,584 did not).
+constexpr int SEL_SAMPLE = 8192, SEL_FEW = 7168, SEL_BINS = 2048;
 struct SelFew {
     union {
         uint32_t sample[SEL_SAMPLE];
@@ -996,7 +997,7 @@ __device__ __forceinline__ bool select_few_applies(int n, int n_prune, int *want
     const float r = (float)n_prune * ((float)SEL_SAMPLE / (float)n);
     const float w = r + 4.f * sqrtf(r) + 8.f;
     *want = (int)w;
-    return n >= 2 * SEL_SAMPLE && w * (float)n <= 3072.f * SEL_SAMPLE;
+    return n >= 2 * SEL_SAMPLE && w * (float)n <= (float)(SEL_FEW / 7 * 6) * SEL_SAMPLE;
 }
 __device__ __forceinline__ bool select_few(const int32_t *__restrict__ cb, const int32_t *__restrict__ sb, int n, int n_prune,
                                            int want, int32_t *__restrict__ out, int32_t *__restrict__ out_ci, SelFew &few,
@@ -1102,13 +1103,15 @@ __device__ __forceinline__ bool select_few(const int32_t *__restrict__ cb, const
 
 // grid (B).  pruned[b][0..n_prune) ascending ids, -1 padded; n_pruned[b]; pruned_ci (optional): the score of each
 // kept document, INT_MIN beside every -1.
+template <bool MANY>      // the list may be long (the shared memory of select_few is there)
 __global__ void __launch_bounds__(SEL_THREADS)
 select_kernel(const int32_t *__restrict__ cand, const int32_t *__restrict__ n_cand, const int32_t *__restrict__ ci,
               int64_t maxc, int n_prune, int32_t *__restrict__ pruned, int32_t *__restrict__ n_pruned,
               int32_t *__restrict__ pruned_ci)
 {
     pdl_entry();
-    __shared__ SelFew few;
+    extern __shared__ uint4 s_few[];                         // (two blocks per SM: 72 KB each)
+    SelFew &few = *reinterpret_cast<SelFew *>(s_few);
     __shared__ int hist[SEL_BINS];
     __shared__ int warp_part[32];
     __shared__ uint32_t s_prefix;
@@ -1129,7 +1132,7 @@ select_kernel(const int32_t *__restrict__ cand, const int32_t *__restrict__ n_ca
         return;
     }
     int need_eq, want;
-    if (select_few_applies(n, n_prune, &want) &&
+    if (MANY && select_few_applies(n, n_prune, &want) &&
         select_few(cb, sb, n, n_prune, want, out, out_ci, few, hist, warp_part, &s_prefix, &s_want)) {
         if (threadIdx.x == 0) n_pruned[b] = n_prune;
         return;
@@ -1674,9 +1677,10 @@ size_t select_split_scratch_bytes(const Index &ix, const Params &p)
     return select_split_used(ix, p) ? sizeof(int32_t) * (size_t)p.B * SELS_SCRATCH : 0;
 }
 
-// scratch: select_split_scratch_bytes() bytes, or NULL (one block per query then).
+// scratch: select_split_scratch_bytes() bytes, or NULL (one block per query then).  many: the lists are all the candidates, not
+// a few contenders.
 int launch_select(const Index &ix, const Params &p, const int32_t *cand, const int32_t *n_cand, const int32_t *ci,
-                  int32_t *pruned, int32_t *n_pruned, int32_t *pruned_ci, int32_t *scratch, cudaStream_t st)
+                  int32_t *pruned, int32_t *n_pruned, int32_t *pruned_ci, int32_t *scratch, bool many, cudaStream_t st)
 {
     // the slices must stay below 2^15 entries (two counters packed in an int) and be worth five launches
     if (scratch != nullptr && select_split_used(ix, p) && p.maxc >= 16384 && p.maxc < (int64_t)SELS_SPLIT * 32767) {
@@ -1692,8 +1696,14 @@ int launch_select(const Index &ix, const Params &p, const int32_t *cand, const i
         count_launch(SLOT_SELECT, 5);
         return CHIMERA_OK;
     }
-    launch(select_kernel, (unsigned)p.B, SEL_THREADS, 0, st, cand, n_cand, ci, p.maxc, p.n_prune, pruned, n_pruned,
-                                                         pruned_ci);
+    // (shared memory that a short list does not need makes the SM change its split between kernels: one query 167.7 -> 168.9 us)
+    if (many) {
+        CHIMERA_CUDA(cudaFuncSetAttribute(select_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SelFew)));
+        launch(select_kernel<true>, (unsigned)p.B, SEL_THREADS, sizeof(SelFew), st, cand, n_cand, ci, p.maxc, p.n_prune, pruned,
+               n_pruned, pruned_ci);
+    } else {
+        launch(select_kernel<false>, (unsigned)p.B, SEL_THREADS, 0, st, cand, n_cand, ci, p.maxc, p.n_prune, pruned, n_pruned, pruned_ci);
+    }
     CHIMERA_CUDA(cudaGetLastError());
     count_launch(SLOT_SELECT);
     return CHIMERA_OK;

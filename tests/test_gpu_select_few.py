@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("N,n_prune,distinct", [
-    (16383, 100, 0), (16384, 100, 0), (16384, 1, 0), (40001, 1024, 0), (40001, 2000, 0), (60000, 4000, 0),
+    (16383, 100, 0), (16384, 100, 0), (16384, 1, 0), (40001, 1024, 0), (40001, 2000, 0), (60000, 4000, 0), (60000, 3000, 0), (60000, 5000, 0),
     (40001, 700, 20000),          # pairs of equal documents, half a pair at the edge now and then
     (40001, 700, 60),             # 667 documents with each score: ties at the edge
     (40001, 700, 5),              # 8,000 with the best score: more than the list holds
