@@ -680,10 +680,15 @@ def measure(pkg, cfg, corp, q, index, args, device, mode="ci", dist=None, local_
                             "x this launch's algorithmic bytes%s" % (ratio, src, "" if first_cut else
                                                                      ", + each query's 8-bit table once"),
             "ms_per_launch": ci_ms, "algorithmic_bytes_per_launch": ci_bytes,
-            "target": {"frac": TARGET, "met": bool(frac >= TARGET),
+            # (bytes are counted per query; a scan of the whole batch reads the ids once for all of its queries, so with the first
+            # cut the fraction can pass the target without the memory doing so: never claimed as met there)
+            "target": {"frac": TARGET, "met": bool(frac >= TARGET and not first_cut),
                        "note": "the task's 60 %% of HBM peak for the code-scan stages is %s: every 4-byte centroid id "
-                               "costs a random lookup, in shared memory (about 3.5 bank conflicts each 32) or of a 32-byte "
-                               "row through L1/L2, which binds the kernel" % ("met" if frac >= TARGET else "NOT met")},
+                               "costs a random lookup, in shared memory (about 3.5 bank conflicts each 32) or of a row "
+                               "through L1/L2, which binds the kernel%s" %
+                               ("met" if frac >= TARGET and not first_cut else "NOT met",
+                                "; bytes are per query, and a scan of the whole batch reads the ids once for all queries"
+                                if first_cut else "")},
             "contender_fraction": mean("contenders") / max(mean("cand"), 1.0),
             # with the first cut no single rate binds its launches (the lookups of filter_scan_kernel alone run at 71 % of
             # the shared-memory wavefront peak in an ncu capture)
@@ -737,7 +742,7 @@ def measure(pkg, cfg, corp, q, index, args, device, mode="ci", dist=None, local_
                                   table_write_gbs=gbs(B * nq * cfg.n_centroids * 5.0, g1_ms)),
         "probes": frac_entry("hbm", B * nq * cfg.n_centroids * 4.0 / 1e9, pr_ms, peak, "GB/s"),
         ("partial_scores" if mode != "ci" else "centroid_interaction_bounds"):
-            frac_entry("hbm", ci_bytes / 1e9, ci_ms, peak, "GB/s", target_frac=TARGET, target_met=bool(frac >= TARGET)),
+            frac_entry("hbm", ci_bytes / 1e9, ci_ms, peak, "GB/s", target_frac=TARGET, target_met=roofline["target"]["met"]),
         "residual_scores": frac_entry("hbm (code + centroid-id bytes)", g4_bytes / 1e9, g4_ms, peak, "GB/s",
                                       target_frac=TARGET, target_met=bool(g4_frac >= TARGET),
                                       with_table_row_gathers_gbs=gbs(g4_bytes + g4_row_bytes, g4_ms),
