@@ -609,13 +609,13 @@ ci_coarse_rng_kernel(const uint8_t *__restrict__ table8, int64_t K, const int2 *
 // 64 tokens, 1,795 / 856 + 223; 262,144 centroids, batch 256, 4,458 / 2,724 + 1,034.
 // With few rows left to look up the instructions around them count (a document per warp: 1,890 us, 570 instructions each), so four
 // documents share a warp, eight lanes each, those of a group of 32 taken by length: a bit per token from shared memory says
-// whether it is near, near ids are collected in shared memory and their rows looked up 8 / LPR at a time and document.  nq: the columns that count; those up to 16 LPR are
-// zero in every row.  rng: token ranges; (CI, 0) stands for a document whose CI is known.
+// whether it is near, near ids are collected in shared memory and their rows looked up 8 / LPR at a time and document.  nq: the columns that count; the rest of
+// the 16 LPR are zero in every row.  runs: byte x of a row is column x / runs + 32 (x % runs).  rng: token ranges; (CI, 0) stands for a document whose CI is known.
 constexpr int BOUND_THREADS = 512;
 constexpr int BOUND_LIST = 64, BOUND_PITCH = BOUND_LIST + 8;
 template <int LPR>
 __global__ void __launch_bounds__(BOUND_THREADS, 2)
-ci_bound_kernel(const uint8_t *__restrict__ table8, int64_t K, int nq, const uint32_t *__restrict__ mask, int mask_words,
+ci_bound_kernel(const uint8_t *__restrict__ table8, int64_t K, int nq, int runs, const uint32_t *__restrict__ mask, int mask_words,
                 const int32_t *__restrict__ theta, const int32_t *__restrict__ tau, const int2 *__restrict__ rng,
                 const int32_t *__restrict__ n_docs, int64_t maxc, const int32_t *__restrict__ cids, int32_t *__restrict__ hi,
                 int32_t *__restrict__ rest, int32_t *__restrict__ n_rest, FirstCut cut)
@@ -646,7 +646,7 @@ ci_bound_kernel(const uint8_t *__restrict__ table8, int64_t K, int nq, const uin
         uint32_t w = 0;
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-            const int col = 16 * sub + 4 * k + e;
+            const int at = 16 * sub + 4 * k + e, col = at / runs + 32 * (at % runs);
             if (col < nq) w |= (uint32_t)(theta[(int64_t)b * nq + col] - 1) << (8 * e);
         }
         floor_f[k] = w << 8;
@@ -898,7 +898,8 @@ int launch_kept_bounds(const Index &ix, const Params &p, const uint8_t *table8, 
         if (gx > (want + 1) / 2) gx = (want + 1) / 2;
         auto kern = p.nq <= 32 ? ci_bound_kernel<2> : p.nq <= 64 ? ci_bound_kernel<4> : ci_bound_kernel<8>;
         CHIMERA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        launch(kern, dim3((unsigned)gx, (unsigned)p.B), BOUND_THREADS, smem, st, table8, ix.K, p.nq, mask, (int)words, theta, tau, rng,
+        const int runs = coarse_supported(p.nq) ? 1 : coarse_pitch(p.nq) / 32;        // (rows from stage 1, or from the first cut)
+        launch(kern, dim3((unsigned)gx, (unsigned)p.B), BOUND_THREADS, smem, st, table8, ix.K, p.nq, runs, mask, (int)words, theta, tau, rng,
                n_docs, p.maxc, ix.cids, hi, rest, n_rest, cut);
         CHIMERA_CUDA(cudaGetLastError());
         count_launch(SLOT_CI);
