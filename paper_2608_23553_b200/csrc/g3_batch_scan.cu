@@ -286,7 +286,7 @@ batch_excess_exact_kernel(const int32_t *__restrict__ table, int64_t K, int nq, 
             near |= (uint32_t)(s > 0) << r;
             if (lane == r) mine = s;
         }
-        if (live && lane == 0 && gr * PER < K) mask[(int64_t)b * ((K + 31) / 32) * 4 + gr] = (uint8_t)near;
+        if (NQW > 1 && live && lane == 0 && gr * PER < K) mask[(int64_t)b * ((K + 31) / 32) * 4 + gr] = (uint8_t)near;
         if (lane < PER) {
             uint32_t code = code_of(mine, step, inv);
             if (code > BS_TOP) {

@@ -91,14 +91,23 @@ static double filter_share(const Index &ix)
     const double len = 0.5 * ((1.2 * mean < most ? 1.2 * mean : most) + (2.4 * mean < most ? 2.4 * mean : most));
     return FILTER_LAMBDA / len;
 }
-// Whether the bounds of what is kept start with the tokens near the query (ci_bound_kernel).  With more than a third of the tokens
-// near, the other columns are too many for a bound that decides: 100 tokens on 100-token documents (half of them near) 405 us,
-// all rows at once 224.  And a document is a chain of lookups whose length does not shrink with the rows: too few of them to
-// hide it, and a second kernel, cost more (one query, 603 survivors: 219 -> 245 us for the call; 37 queries, 777: 55 -> 68 us for the
-// step; 64 queries, 2,048: 1,795 -> 1,079).  (6-bit codes from the exact table come five centroids to a warp: no words of a mask.)
+// Whether the bounds of what is kept start with the tokens near the query (ci_bound_kernel).  Measured as the time of the step, all
+// rows at once / near tokens first (independent tokens unless said):
+//   Tokens near, as the thresholds are set: with more than four tenths of them the other columns are too many for a bound that
+//     decides.  64 queries, n_prune 2,048, by the share: 32 query tokens 0.30 301 / 283 us, 0.39 264 / 249, 0.44 255 / 267, 0.66 212 / 219; 64:
+//     0.47 783 / 748, 0.59 669 / 682; 100: 0.31 2,130 / 1,850, 0.41 1,865 / 1,833, 0.53 1,535 / 1,646, 0.74 1,342 / 1,589.
+//   Documents looked at: each is a chain of lookups whose length does not shrink with the rows, and there is a second kernel.
+//     B n_prune from 65,536 on nothing of 32 tokens or more lost more than 10 % (topics, most of them kept), and most gained 5 to 35 %:
+//     Mid, 64 queries, n_prune 1,024, 308 / 263; 64 tokens on 512-token documents, 64 queries, n_prune 1,024, 890 / 576; 100 tokens on
+//     those, 64 queries, 2,048, 3,886 / 2,608.  Below, it goes by the documents: 32,768: 200 / 203, 165 / 150 (Mid, n_prune 256 and 512),
+//     475 / 336 (64 tokens); 16,384: 101 / 118, 89 / 74, 322 / 294, and 302 / 458 with 60 tokens, 1,151 / 2,040 with 110.
+//   Fewer than 32 query tokens: the bound of a document is a sum of few columns, and those that pass cost both kernels.  Mid, 64
+//     queries, n_prune 2,048: 8 tokens 124 / 159, 16: 258 / 291, 21: 356 / 376, 28: 452 / 449; documents of four topics 461 / 595, 1,088 /
+//     1,472, 1,174 / 1,601, 1,657 / 2,123.  (32 tokens: 504 / 435; topics that keep most of them do without the cut.)
+// (6-bit codes from the exact table come five centroids to a warp: no words of a mask.)
 bool filter_mask_used(const Index &ix, const Params &p, bool batch)
 {
-    return filter_share(ix) * p.nq < 0.4 && (int64_t)p.B * p.n_prune >= 65536 &&
+    return p.nq >= 32 && filter_share(ix) * p.nq < 0.4 && (int64_t)p.B * p.n_prune >= 65536 &&
            (batch || coarse_supported(p.nq) || filter_codec(ix.K) == 16);
 }
 bool filter_used(const Index &ix, const Params &p)
@@ -478,7 +487,7 @@ filter_excess_exact_kernel(const int32_t *__restrict__ table, int64_t K, int nq,
         }
         if (CODEC == 16) {
             if (lane < PER && g * PER + lane < K) reinterpret_cast<uint16_t *>(ob)[g * PER + lane] = (uint16_t)val;
-            if (lane == 0) mask[(int64_t)b * ((K + 31) / 32) * 4 + g] = (uint8_t)near;
+            if (NQW > 1 && lane == 0) mask[(int64_t)b * ((K + 31) / 32) * 4 + g] = (uint8_t)near;    // (filter_mask_used)
         } else if (lane == 0) {
             reinterpret_cast<uint32_t *>(ob)[g] = packed;
         }

@@ -1,4 +1,5 @@
-"""When stage 3 runs its first cut and keeps visits as lists: host arithmetic on the sizes, no device."""
+"""When stage 3 runs its first cut, starts its bounds from near tokens and keeps visits as lists: host arithmetic on the sizes, no
+device."""
 import os
 import subprocess
 
@@ -13,7 +14,7 @@ def routes(tmp_path_factory):
     tmp = tmp_path_factory.mktemp("rule")
     obj, exe = str(tmp / "stage3_rules.o"), str(tmp / "stage3_rules")
     subprocess.check_call([build.NVCC] + build.FLAGS + ["-c", os.path.join(native, "stage3_rules.cu"), "-o", obj])
-    objs = [os.path.join(build.OBJ, n) for n in ("g3_filter.o", "g3_centroid_interaction.o", "g3_partial.o")]
+    objs = [os.path.join(build.OBJ, n) for n in ("g3_filter.o", "g3_batch_scan.o", "g3_centroid_interaction.o", "g3_partial.o")]
     subprocess.check_call(["g++", "-no-pie", "-o", exe, obj, os.path.join(native, "fake_cudart.cpp")] + objs +
                           ["-Wl,--unresolved-symbols=ignore-all"])
 
@@ -33,6 +34,11 @@ def rule(routes):
 @pytest.fixture(scope="module")
 def lists(routes):
     return lambda *a, **kw: routes(*a, **kw)[1]
+
+
+@pytest.fixture(scope="module")
+def near_first(routes):
+    return lambda *a, **kw: routes(*a, **kw)[2]
 
 
 def test_what_the_candidates_hold_counts_and_not_the_room_for_them(rule):
@@ -71,3 +77,15 @@ def test_visits_are_kept_as_lists_while_candidates_have_few(lists):
     # documents that repeat their centroids: as few visits, but of fewer candidates
     assert lists(*mid, 4, 1_024, distinct=40) and not lists(*mid, 4, 1_024, distinct=12)
     assert not lists(*mid, 4, 1_024, longest=60_000)                     # as large as the table
+
+
+def test_bounds_start_with_near_tokens_where_that_decides(near_first):
+    mid = (65_536, 500_000, 120)
+    assert near_first(*mid, 64, 32, 4, 1_024) and near_first(*mid, 64, 40, 4, 1_024) and near_first(*mid, 64, 64, 4, 1_024)
+    assert not near_first(*mid, 64, 32, 4, 1_023)                        # few documents
+    # short queries: every length below 32, in a batch scanned together and by query
+    assert not any(near_first(*mid, B, nq, 8, 2_048) for nq in (8, 16, 21, 28, 31) for B in (64, 256))
+    # documents too short for the query (1.6 x 50 = 80 tokens of weight: 0.4)
+    assert not near_first(65_536, 500_000, 50, 64, 32, 8, 2_048) and near_first(65_536, 500_000, 51, 64, 32, 8, 2_048)
+    # 6-bit codes from the exact table, a query at a time
+    assert not near_first(262_144, 8_800_000, 68, 256, 40, 4, 4_096) and near_first(262_144, 8_800_000, 68, 256, 32, 4, 4_096)
