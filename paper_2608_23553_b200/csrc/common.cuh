@@ -175,6 +175,15 @@ int fault_skip_tma_loads();
 enum Slot { SLOT_G1 = 0, SLOT_PROBE, SLOT_GATHER, SLOT_CI, SLOT_SELECT, SLOT_G4, SLOT_TOPK, SLOT_MISC, SLOT_CI_EXACT };
 void count_launch(int slot, int n = 1);
 
+// Dynamic shared memory above the default 48 KB.  The limit belongs to the kernel and not to a call, so every call sets the most that
+// any call of the kernel takes: with its own size a search on another thread, of another index or other parameters, could lower
+// the limit between this call's setting and its launch.
+template <class... P>
+cudaError_t allow_shared(void (*kernel)(P...), size_t most)
+{
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+
 // ---------------------------------------------------------------------------------------------------------------
 // Launches of a search.  A search is a chain of up to two dozen short kernels on one stream, so the gaps between them are a
 // good part of a small call.  Every kernel is launched as a programmatic dependent of the one before it: its blocks are

@@ -481,8 +481,7 @@ static int launch_g1_tiles(const Index &ix, const Params &p, const CUtensorMap &
     const int skip = fault_skip_tma_loads();
 #define CHIMERA_G1_LAUNCH(KS)                                                                                          \
     do {                                                                                                               \
-        CHIMERA_CUDA(cudaFuncSetAttribute(score_table_umma<KS, FILTER, TABLE>, cudaFuncAttributeMaxDynamicSharedMemorySize,   \
-                                          (int)G1_SMEM));                                                              \
+        CHIMERA_CUDA(allow_shared(score_table_umma<KS, FILTER, TABLE>, G1_SMEM));                                      \
         launch(score_table_umma<KS, FILTER, TABLE>, grid, G1_THREADS, G1_SMEM, st, ix.cdig, map_q, ix.K, p.nq, rows, n_tiles,     \
                                                                         tiles_per_split, table, table8, status, limit, \
                                                                         skip, tiles);                                  \

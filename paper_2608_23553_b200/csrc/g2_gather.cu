@@ -41,6 +41,7 @@ mark_kernel(const int32_t *__restrict__ probes, int n_lists, const int64_t *__re
 // The same with the bitmap in shared memory, for small corpora: their lists set the same few words over and over, and
 // atomics on one L2 line come one after the other (10,000 documents, 128 lists of 625: 17 us, here 6.5).  grid (blocks, B): a
 // block takes every gridDim.x-th list and adds its bits to the query's bitmap at the end.
+constexpr int MARK_SHARED_WORDS = 24 * 1024;
 __global__ void __launch_bounds__(512)
 mark_shared_kernel(const int32_t *__restrict__ probes, int n_lists, const int64_t *__restrict__ ivf_off,
                    const int32_t *__restrict__ ivf_doc, uint32_t *__restrict__ bitmap, int words)
@@ -272,7 +273,7 @@ int launch_gather(const Index &ix, const Params &p, const Layout &L, const int32
     const int ranges = (int)((L.words + MARK_RANGE_WORDS - 1) / MARK_RANGE_WORDS);
     // Bitmaps of up to 96 KB whose words are set a dozen times or more on average: in shared memory, sixteen blocks a query (16
     // queries of 1,024 lists, 61 entries a word: 158 us in L2, 29 so; 37 queries, 19: 32 and 28; one query, 8: 5.7 and 8.3).
-    const bool shared = L.words <= 24 * 1024 && (double)n_lists * ((double)ix.ivf_len / (double)ix.K) >= 12.0 * (double)L.words;
+    const bool shared = L.words <= MARK_SHARED_WORDS && (double)n_lists * ((double)ix.ivf_len / (double)ix.K) >= 12.0 * (double)L.words;
     // A block per query and range (every range reads all lists: up to 14 million documents), unless that leaves SMs idle (64 queries
     // on one range of 25 KB: 198 us, sixteen blocks a query 100).
     const bool by_range = !few && ranges <= 8 && (!shared || (int64_t)ranges * p.B >= ix.sm_count);
@@ -281,12 +282,11 @@ int launch_gather(const Index &ix, const Params &p, const Layout &L, const int32
         int range_words = (int)((L.words + ranges - 1) / ranges);
         range_words = (range_words + BITMAP_CHUNK_WORDS - 1) / BITMAP_CHUNK_WORDS * BITMAP_CHUNK_WORDS;
         const size_t smem = sizeof(uint32_t) * (size_t)range_words;
-        CHIMERA_CUDA(cudaFuncSetAttribute(mark_range_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        CHIMERA_CUDA(allow_shared(mark_range_kernel, sizeof(uint32_t) * MARK_RANGE_WORDS));
         launch(mark_range_kernel, dim3((unsigned)((L.words + range_words - 1) / range_words), (unsigned)p.B), 1024, smem, st, probes,
                n_lists, ix.ivf_off, ix.ivf_doc, bitmap, L.words, range_words, L.n_chunks, chunk_cnt);
     } else if (shared) {
-        CHIMERA_CUDA(cudaFuncSetAttribute(mark_shared_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)(sizeof(uint32_t) * (size_t)L.words)));
+        CHIMERA_CUDA(allow_shared(mark_shared_kernel, sizeof(uint32_t) * MARK_SHARED_WORDS));
         launch(mark_shared_kernel, dim3((unsigned)(n_lists < 16 ? n_lists : 16), (unsigned)p.B), 512,
                sizeof(uint32_t) * (size_t)L.words, st, probes, n_lists, ix.ivf_off, ix.ivf_doc, bitmap, (int)L.words);
     } else {

@@ -13,6 +13,7 @@
 namespace chimera {
 
 constexpr int PROBE_THREADS = PROBE_WARPS * 32;
+constexpr size_t PROBE_LISTS_MOST = sizeof(unsigned long long) * CHIMERA_MAX_NPROBE * PROBE_THREADS;     // shared memory of a block
 
 template <int STRIDE = PROBE_THREADS>
 __device__ __forceinline__ void list_insert(unsigned long long *list, int P, unsigned long long key)
@@ -186,8 +187,7 @@ static int launch_probe_final(const unsigned long long *part, int B, int nq, int
     } else {
         const size_t smem = per_thread * PROBE_THREADS;
         if (smem > 48 * 1024)
-            CHIMERA_CUDA(cudaFuncSetAttribute(probe_final<PROBE_THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)smem));
+            CHIMERA_CUDA(allow_shared(probe_final<PROBE_THREADS>, PROBE_LISTS_MOST));
         launch(probe_final<PROBE_THREADS>, grid, PROBE_THREADS, smem, st, part, nq, P, n_part, probes, only_flagged);
     }
     CHIMERA_CUDA(cudaGetLastError());
@@ -252,7 +252,7 @@ int launch_probes(const Index &ix, const Params &p, const Layout &L, const int32
     }
     const size_t smem = sizeof(unsigned long long) * (size_t)p.P * PROBE_THREADS;
     if (smem > 48 * 1024)
-        CHIMERA_CUDA(cudaFuncSetAttribute(probe_partial, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        CHIMERA_CUDA(allow_shared(probe_partial, PROBE_LISTS_MOST));
     const int rows_per_block = (int)((ix.K + L.probe_blocks - 1) / L.probe_blocks);
     const unsigned col_groups = (unsigned)((p.nq + 31) / 32);
     dim3 g1((unsigned)L.probe_blocks, (unsigned)p.B, col_groups);
@@ -495,7 +495,7 @@ int launch_probe_merge(const Index &ix, const Params &p, const Layout &L, int32_
     }
     const size_t smem = sizeof(unsigned long long) * (size_t)p.P * PROBE_THREADS;
     if (smem > 48 * 1024)
-        CHIMERA_CUDA(cudaFuncSetAttribute(probe_partial, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        CHIMERA_CUDA(allow_shared(probe_partial, PROBE_LISTS_MOST));
     const int rows_per_block = (int)((ix.K + L.probe_blocks - 1) / L.probe_blocks);
     const unsigned col_groups = (unsigned)((p.nq + 31) / 32);
     launch(probe_partial, dim3((unsigned)L.probe_blocks, (unsigned)p.B, col_groups), PROBE_THREADS, smem, st, table, ix.K, p.nq, p.P, rows_per_block, L.n_part, part, ovf, nullptr, probes);
@@ -577,7 +577,7 @@ extern "C" int chimera_probes_static(const int32_t *score_table, int64_t n_centr
     cudaStream_t st = (cudaStream_t)stream;
     const size_t smem = sizeof(unsigned long long) * (size_t)nprobe * PROBE_THREADS;
     if (smem > 48 * 1024)
-        CHIMERA_CUDA(cudaFuncSetAttribute(probe_partial, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        CHIMERA_CUDA(allow_shared(probe_partial, PROBE_LISTS_MOST));
     const int rows_per_block = (int)((n_centroids + blocks - 1) / blocks);
     const unsigned col_groups = (unsigned)((q_len + 31) / 32);
     // probe_partial writes every entry probe_final reads (all n_part lists x nprobe keys x q_len columns), so nothing

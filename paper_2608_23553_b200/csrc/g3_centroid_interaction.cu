@@ -816,7 +816,8 @@ int launch_coarse_bounds(const Index &ix, const Params &p, const uint8_t *table8
     const size_t table_bytes = (size_t)ix.K * coarse_pitch(p.nq);
     const bool use_rng = rng != nullptr;
     const FirstCut call_cut = cut ? *cut : FirstCut();
-    const bool small = table_bytes <= 160 * 1024;
+    constexpr size_t COARSE_SMEM = 160 * 1024;
+    const bool small = table_bytes <= COARSE_SMEM;
     if (small) {
         // the whole 8-bit table of a query fits in shared memory: stage it once per block and look rows up there
         constexpr int T = 512;
@@ -829,13 +830,11 @@ int launch_coarse_bounds(const Index &ix, const Params &p, const uint8_t *table8
         if (gx < 1) gx = 1;
         dim3 grid((unsigned)gx, (unsigned)p.B);
         if (p.nq == 32) {
-            CHIMERA_CUDA(cudaFuncSetAttribute(ci_coarse_kernel<2, true, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)table_bytes));
+            CHIMERA_CUDA(allow_shared(ci_coarse_kernel<2, true, T>, COARSE_SMEM));
             launch(ci_coarse_kernel<2, true, T>, grid, T, table_bytes, st, table8, ix.K, cand, n_cand, p.maxc, ix.cids,
                                                                        ix.doc_off, lo, hi, call_cut);
         } else {
-            CHIMERA_CUDA(cudaFuncSetAttribute(ci_coarse_kernel<4, true, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)table_bytes));
+            CHIMERA_CUDA(allow_shared(ci_coarse_kernel<4, true, T>, COARSE_SMEM));
             launch(ci_coarse_kernel<4, true, T>, grid, T, table_bytes, st, table8, ix.K, cand, n_cand, p.maxc, ix.cids,
                                                                        ix.doc_off, lo, hi, call_cut);
         }
@@ -897,7 +896,8 @@ int launch_kept_bounds(const Index &ix, const Params &p, const uint8_t *table8, 
         if (gx < (2LL * ix.sm_count + p.B - 1) / p.B) gx = (2LL * ix.sm_count + p.B - 1) / p.B;
         if (gx > (want + 1) / 2) gx = (want + 1) / 2;
         auto kern = p.nq <= 32 ? ci_bound_kernel<2> : p.nq <= 64 ? ci_bound_kernel<4> : ci_bound_kernel<8>;
-        CHIMERA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        constexpr size_t MASK_MOST = 40 * 1024;             // more than 266,240 centroids are not cut (filter_used)
+        CHIMERA_CUDA(allow_shared(kern, MASK_MOST));
         const int runs = coarse_supported(p.nq) ? 1 : coarse_pitch(p.nq) / 32;        // (rows from stage 1, or from the first cut)
         launch(kern, dim3((unsigned)gx, (unsigned)p.B), BOUND_THREADS, smem, st, table8, ix.K, p.nq, runs, mask, (int)words, theta, tau, rng,
                n_docs, p.maxc, ix.cids, hi, rest, n_rest, cut);
@@ -1699,7 +1699,7 @@ int launch_select(const Index &ix, const Params &p, const int32_t *cand, const i
     }
     // (shared memory that a short list does not need makes the SM change its split between kernels: one query 167.7 -> 168.9 us)
     if (many) {
-        CHIMERA_CUDA(cudaFuncSetAttribute(select_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SelFew)));
+        CHIMERA_CUDA(allow_shared(select_kernel<true>, sizeof(SelFew)));
         launch(select_kernel<true>, (unsigned)p.B, SEL_THREADS, sizeof(SelFew), st, cand, n_cand, ci, p.maxc, p.n_prune, pruned,
                n_pruned, pruned_ci);
     } else {

@@ -1013,11 +1013,11 @@ static int launch_query_scan(const Index &ix, const Params &p, const Layout &L, 
     if (gx > want) gx = want;
     const dim3 grid((unsigned)gx, (unsigned)p.B);
     if (codec == 16) {
-        CHIMERA_CUDA(cudaFuncSetAttribute(filter_scan_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pitch));
+        CHIMERA_CUDA(allow_shared(filter_scan_kernel<16>, FILTER_SMEM));
         launch(filter_scan_kernel<16>, grid, SCAN_THREADS_F, pitch, st, tab, pitch, theta, p.nq, us, cand, ix.doc_off, n_cand, p.maxc,
                                                                     ix.cids, ix.T, hi0, hist, cut);
     } else {
-        CHIMERA_CUDA(cudaFuncSetAttribute(filter_scan_kernel<6>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pitch));
+        CHIMERA_CUDA(allow_shared(filter_scan_kernel<6>, FILTER_SMEM));
         launch(filter_scan_kernel<6>, grid, SCAN_THREADS_F, pitch, st, tab, pitch, theta, p.nq, us, cand, ix.doc_off, n_cand, p.maxc,
                                                                    ix.cids, ix.T, hi0, hist, cut);
     }

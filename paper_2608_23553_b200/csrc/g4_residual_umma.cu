@@ -432,7 +432,7 @@ static int launch_g4_umma(const Index &ix, const Params &p, int q_base, int nq, 
     case 64: kern = full ? residual_maxsim_umma<NQP, NBITS, RQ, 64, true> : residual_maxsim_umma<NQP, NBITS, RQ, 64, false>; break;
     case 96: kern = full ? residual_maxsim_umma<NQP, NBITS, RQ, 96, true> : residual_maxsim_umma<NQP, NBITS, RQ, 96, false>; break;
     }
-    CHIMERA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    CHIMERA_CUDA(allow_shared(kern, smem));                  // (the same in every call of this kernel)
     // documents per CTA: whole waves of resident CTAs, as few as documents-per-CTA limit allows (a second wave of a few CTAs
     // costs as much as a full one: 37 queries of 777 survivors in 2.1 waves of 32 documents, or in three of 22)
     const int64_t slots = (int64_t)(NQP == 32 ? (RQ ? 4 : 3) : 2) * ix.sm_count, docs = (int64_t)p.n_prune * p.B;

@@ -188,14 +188,15 @@ static int launch_topk_entries(const int32_t *ids, const float *scores, int B, i
     int n_pow2 = 2;
     while (n_pow2 < n) n_pow2 <<= 1;
     const size_t smem = sizeof(unsigned long long) * (size_t)n_pow2;
-    if (smem > 128 * 1024) return fail(CHIMERA_UNSUPPORTED, "top-k over %d entries per query does not fit shared memory", n);
+    constexpr size_t TOPK_SMEM = 128 * 1024;
+    if (smem > TOPK_SMEM) return fail(CHIMERA_UNSUPPORTED, "top-k over %d entries per query does not fit shared memory", n);
     int cap = 4;
     while (cap < 2 * k) cap <<= 1;
     const bool select = n >= 4 * k && n >= 256;
     const size_t bytes = smem + (select ? sizeof(unsigned long long) * (size_t)cap : 0);
     auto kern = select ? topk_kernel<true> : topk_kernel<false>;
     if (bytes > 48 * 1024 - 16 * 1024)                    // (the selection has 8 KB of its own)
-        CHIMERA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+        CHIMERA_CUDA(allow_shared(kern, TOPK_SMEM + (select ? TOPK_SMEM / 2 : 0)));     // (k <= n / 4, so cap <= n_pow2 / 2)
     launch(kern, (unsigned)B, TOPK_THREADS, bytes, st, ids, scores, n, n_pow2, cap, k, seg_len, seg_stride, out_ids, out_scores);
     CHIMERA_CUDA(cudaGetLastError());
     return CHIMERA_OK;

@@ -295,7 +295,8 @@ size_t graph_scratch_bytes(const Index &ix, int64_t n_tokens)
 }
 
 // The search keeps the visited set in shared memory up to a million centroids.
-static bool visited_in_shared(const Index &ix) { return (ix.K + 31) / 32 * (int64_t)sizeof(uint32_t) <= 128 * 1024; }
+constexpr size_t VISITED_SMEM = 128 * 1024;
+static bool visited_in_shared(const Index &ix) { return (size_t)((ix.K + 31) / 32) * sizeof(uint32_t) <= VISITED_SMEM; }
 size_t graph_workspace_bytes(const Index &ix, int64_t n_tokens)
 {
     return visited_in_shared(ix) ? 0 : graph_scratch_bytes(ix, n_tokens);
@@ -323,7 +324,7 @@ int launch_graph_probes(const Index &ix, const float *queries, int64_t n_tokens,
                              : (shared ? graph_probe_kernel<true, false, 4> : graph_probe_kernel<false, false, 4>))
                      : (wide ? (shared ? graph_probe_kernel<true, true, 2> : graph_probe_kernel<false, true, 2>)
                              : (shared ? graph_probe_kernel<true, false, 2> : graph_probe_kernel<false, false, 2>));
-    if (shared) CHIMERA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (shared) CHIMERA_CUDA(allow_shared(kern, VISITED_SMEM));
     else CHIMERA_CUDA(cudaMemsetAsync(visited, 0, graph_scratch_bytes(ix, n_tokens), st));
     launch(kern, (unsigned)n_tokens, four ? 128 : 64, shared ? smem : 0, st, queries, ix.D, ix.xc, ix.graph, ix.graph_deg, ix.K,
            g.n_entries, g.beam, g.max_expansions, nprobe, shared && !want_visited ? nullptr : visited, vwords, out_probes,

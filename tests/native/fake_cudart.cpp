@@ -1,11 +1,15 @@
 // The CUDA runtime calls of the library's host code, without a device: memory comes from the host's heap, launches do
-// nothing, and the call that a test chooses returns an error.  (No CUDA header: its inline wrappers would be defined twice.)
+// nothing, the call that a test chooses returns an error, and limits on shared memory are noted beside what launches ask for.
+// (No CUDA header: its inline wrappers would be defined twice.)
 #include <stdio.h>
 #include <stdlib.h>
 
+#include <map>
 #include <set>
 
 std::set<void *> fake_live;
+std::map<const void *, std::set<int>> fake_limits;       // dynamic shared memory allowed, of each kernel
+std::map<const void *, std::set<size_t>> fake_shared;    // ... and asked for
 int fake_calls = 0, fake_fail_at = 0, fake_last_error = 0;
 
 static int step()
@@ -34,7 +38,18 @@ int cudaMemGetInfo(size_t *avail, size_t *all) { *avail = *all = (size_t)1 << 30
 int cudaStreamSynchronize(void *) { return step(); }
 int cudaDeviceSynchronize(void) { return step(); }
 int cudaLaunchKernel() { return step(); }                // (arguments are left where the caller put them)
-int cudaLaunchKernelExC() { return step(); }
+struct fake_config { unsigned grid[3], block[3]; size_t shared; };
+int cudaLaunchKernelExC(const fake_config *c, const void *kernel, void **)
+{
+    fake_shared[kernel].insert(c->shared);
+    return step();
+}
+int cudaFuncSetAttribute(const void *kernel, int, int bytes)
+{
+    fake_limits[kernel].insert(bytes);
+    return step();
+}
+int cudaMemsetAsync(void *, int, size_t, void *) { return step(); }
 int cudaGetLastError(void) { const int e = fake_last_error; fake_last_error = 0; return e; }
 const char *cudaGetErrorString(int) { return "injected"; }
 unsigned __cudaPushCallConfiguration() { return 0; }
