@@ -168,7 +168,7 @@ int chimera_run_stages(const chimera_index *index, int32_t first_stage, int32_t 
  * lists at token level) that chimera_search_partial needs.  Allocates 8 bytes per token plus 12 per centroid inside the
  * index (cudaMalloc) and, where that takes no more than a quarter of the free device memory, room for a copy of the codes in
  * the order of the lists (chimera_index_list_copies tells); synchronises the stream.  Idempotent, but a call that finds
- * the memory for a copy that an earlier one did not find makes it.  Workspace sizes grow afterwards (visit lists, or a score
+ * the memory for a copy that an earlier one did not find makes it.  Workspace sizes may grow afterwards (visit lists, or a score
  * table of n_queries x max_candidates x q_len int32), so query chimera_workspace_bytes again.
  * Errors: INVALID_ARG, UNSUPPORTED (more than 2^31 - 1 tokens), CUDA_ERROR (the index can be used as before the call). */
 int chimera_index_enable_partial(chimera_index *index, void *stream);

@@ -130,6 +130,7 @@ Layout make_layout(const Index &ix, const Params &p)
     L.ci = take(B * (size_t)p.maxc * sizeof(int32_t));
     const bool filter = filter_used(ix, p);
     const size_t two_phase = (coarse_supported(p.nq) || filter) ? B * (size_t)p.maxc * sizeof(int32_t) : 0;
+    const size_t ci_only = o;
     L.lo = take(two_phase);
     L.hi = take(two_phase);
     L.cont = take(two_phase);
@@ -155,12 +156,20 @@ Layout make_layout(const Index &ix, const Params &p)
     L.n_kept = take(filter ? B * sizeof(int32_t) : 0);
     L.n_seed = take(filter ? B * sizeof(int32_t) : 0);
     L.n_rest = take(filter ? B * sizeof(int32_t) : 0);
+    // Retrieved-token scores of the refinements: visit lists, or dense rows per candidate.  They take the place of what only the
+    // pruning by centroid interaction uses (from L.lo to here; no call does both), so an index with token lists needs no more room
+    // unless they are larger.  (Debug builds have guards in between, and a place of its own.)
+    L.visit_nodes = visit_list_nodes(ix, p);
+    const size_t scores = !ix.tok_id ? 0 : L.visit_nodes ? B * ((size_t)L.visit_nodes + (size_t)p.maxc) * 8 : B * (size_t)p.maxc * nq * sizeof(int32_t);
+#ifdef CHIMERA_DEBUG
+    (void)ci_only;
+    L.partial_m = take(scores);
+#else
+    L.partial_m = ci_only;
+    if (o < align_up(ci_only + scores)) o = align_up(ci_only + scores);
+#endif
     L.pruned = take(B * p.n_prune * sizeof(int32_t));
     L.ranks = take(ix.tok_id || batch ? B * (size_t)L.words * sizeof(uint2) : 0);
-    // retrieved-token scores of the refinements: visit lists, or dense rows per candidate
-    L.visit_nodes = visit_list_nodes(ix, p);
-    L.partial_m = take(!ix.tok_id ? 0 : L.visit_nodes ? B * ((size_t)L.visit_nodes + (size_t)p.maxc) * 8
-                                                      : B * (size_t)p.maxc * nq * sizeof(int32_t));
     L.graph_vis = take(ix.graph ? graph_workspace_bytes(ix, (int64_t)p.B * p.nq) : 0);
     L.q_rot = take(ix.rot_t ? B * nq * ix.D * sizeof(float) : 0);
     L.qdig_rot = take(ix.rot_t ? 3 * rows4 * 128 : 0);

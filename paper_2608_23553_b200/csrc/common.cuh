@@ -128,7 +128,7 @@ struct Layout {
     size_t ranks;         // uint2  [B][words]        bitmap word, candidates before it (document -> candidate index);
                           //                          only with token lists, or where the first cut scans a batch at a time
     size_t partial_m;     // int32  [B][maxc][nq]     per (candidate, query token) best retrieved-token score, or the visit
-                          //                          lists in its place (g3_visits.cuh)
+                          //                          lists in its place (g3_visits.cuh); in the place of lo ... n_rest
     int64_t visit_nodes;  // nodes per query of those lists; 0 = the table
     size_t graph_vis;     // uint32 [B*nq][K/32]      visited centroids of the graph search (only with a centroid graph, and
                           //                          too many centroids for a bitmap in shared memory)
