@@ -23,18 +23,22 @@ namespace chimera {
 constexpr int PS_THREADS = 128;
 
 // Nodes per query of the visit lists, 0 when the table of maxima is used: no token lists, few queries per call (latency
-// counts), more nodes than their index holds, a table less than about four times as large, or candidates with several visits
+// counts), more nodes than their index holds, a table less than three times as large, or candidates with several visits
 // each, whose lists are chains of scattered reads: more than two as independent tokens would have them (long documents under
 // many probes, where the topics of real ones make it many more), or four by the distinct centroids of a document.
 // Whole searches, batch 256 on Mid's sizes, documents that draw 1/4 as many centroids as they have tokens (4.1 visits): lists
 // 2.98, table 2.93 ms, 1-bit codes 2.64 / 2.75; an eighth or less (10 visits): 2.96 / 2.68, 2.60 / 2.32; independent (1.1): 3.21 /
 // 4.27, 2.83 / 4.71; four topics of near centroids under 32 probes (64 queries): 3.37 / 2.52, 3.05 / 2.45.
+// By the ratio of the sizes (batch 256, room for 1.15 times the candidates, residual / 1-bit codes, in us): documents of four topics, 1.9
+// lists 2,003 / 1,735, table 1,955 / 1,726; 3.2 2,486 / 2,334 and 2,463 / 2,412; 3.3 (short documents) 1,318 / 1,063 and 1,407 / 1,207;
+// independent tokens, where a visit is nearly always a candidate's only one, gain earlier: 1.25 1,796 / 1,450 and 1,816 / 1,450, 2.5 2,419 /
+// 2,006 and 2,508 / 2,081, 3.9 1,830 / 1,395 and 2,093 / 1,670.
 int64_t visit_list_nodes(const Index &ix, const Params &p)
 {
     if (!ix.tok_id || ix.max_tok_list <= 0 || 4 * p.B <= ix.sm_count) return 0;
     const int64_t nodes = (int64_t)p.nq * p.P * ix.max_tok_list;
     if (nodes > VISIT_MAX_NODES) return 0;
-    if (4 * (nodes * 8 + p.maxc * 4) > (int64_t)p.maxc * p.nq * 4) return 0;
+    if (3 * 8 * (nodes + p.maxc) > (int64_t)p.maxc * p.nq * 4) return 0;      // (8 bytes a node and a head, 4 an entry of the table)
     const double len = (double)ix.T / (double)ix.N, distinct = (double)ix.ivf_len / (double)ix.N;
     const double probed = (double)p.nq * p.P / (double)ix.K;
     if (len * probed > 1.6) return 0;                    // (visits per candidate: x / (1 - exp(-x)) = 2 at x = 1.6)

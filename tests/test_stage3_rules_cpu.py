@@ -77,6 +77,9 @@ def test_visits_are_kept_as_lists_while_candidates_have_few(lists):
     # documents that repeat their centroids: as few visits, but of fewer candidates
     assert lists(*mid, 4, 1_024, distinct=40) and not lists(*mid, 4, 1_024, distinct=12)
     assert not lists(*mid, 4, 1_024, longest=60_000)                     # as large as the table
+    # a third of the table, 8 bytes a node and a head: 24 (128 x 1,000 + m) <= 128 m, and 24 (32 x 500 + m) <= 32 m
+    assert [lists(*mid, 4, 1_024, longest=1_000, max_candidates=m) for m in (29_538, 29_539)] == [False, True]
+    assert [lists(*mid[:4], 8, 4, 1_024, longest=500, max_candidates=m) for m in (47_999, 48_000)] == [False, True]
 
 
 def test_bounds_start_with_near_tokens_where_that_decides(near_first):
