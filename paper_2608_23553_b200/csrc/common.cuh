@@ -349,6 +349,7 @@ int launch_rabitq_scores_umma(const Index &ix, const Params &p, const float *q_r
 int build_graph(Index &ix, const float *centroids, int degree, cudaStream_t st);
 size_t graph_scratch_bytes(const Index &ix, int64_t n_tokens);
 size_t graph_workspace_bytes(const Index &ix, int64_t n_tokens);     // of a search that does not want the visited sets
+int graph_search_warps(const Index &ix, int64_t n_tokens);           // warps of a search's block: 2 or 4
 int check_graph_params(const Index &ix, const GraphSearch &g, int nprobe);
 // visited: graph_scratch_bytes(ix, n_tokens) bytes of scratch, holding the visited sets afterwards if want_visited;
 // graph_workspace_bytes(ix, n_tokens) otherwise;

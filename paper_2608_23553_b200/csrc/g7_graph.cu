@@ -7,7 +7,7 @@
 // centroids take the place of query tokens in the stage-1 tensor-core kernel and stage 2a picks each row's best
 // degree + 1 entries, of which the centroid itself is dropped.
 //
-// Search (query time): a block of four warps per query token runs a best-first search with a bounded result list:
+// Search (query time): a block of two or four warps per query token runs a best-first search with a bounded result list:
 //   - the entry points floor(j K / n_entries), j < n_entries, are visited (scored, marked, offered to the list);
 //   - repeatedly the first list member that has not been expanded is expanded: each of its graph neighbours that was
 //     never visited is visited; the search ends when every list member is expanded or after max_expansions expansions;
@@ -133,7 +133,7 @@ __device__ __forceinline__ int32_t gp_score(unsigned long long key) { return (in
 // instructions each over all warps), a row's address is one 32 x 32-bit multiply-add, places in s_ids come from votes, keys
 // are compared as they are, and only lists of more than 32 members (WIDE) have a second key per lane.
 // Mid, beam 32, 256 entries: 2,048 tokens 470 -> 244 us with two warps (all blocks resident at once; four: 268), 32 tokens 192 -> 116
-// with four (two: 155), 8,192 tokens 1,492 -> 718.  Two rows in flight per eight lanes: 300.
+// with four (two: 155), 8,192 tokens 1,492 -> 718.  Two rows in flight per eight lanes: 300.  (Which of the two: graph_search_warps.)
 // visited (NULL: not wanted; !SHARED: [tokens][vwords] zeroed by the caller).
 template <bool SHARED, bool WIDE, int WARPS>
 __global__ void __launch_bounds__(WARPS * 32, 32 / WARPS)
@@ -302,6 +302,27 @@ size_t graph_workspace_bytes(const Index &ix, int64_t n_tokens)
     return visited_in_shared(ix) ? 0 : graph_scratch_bytes(ix, n_tokens);
 }
 
+// Warps per token: two where they make the search end in fewer rounds of resident blocks.  Registers hold 8 blocks of four warps or 16
+// of two on an SM, its shared memory as many as have room for the visited set: up to 65,536 centroids (8 KB) all of them, at 131,072 13
+// blocks of two, from 262,144 on (32 KB) no more of two than of four, and then two warps leave an SM half as many to hide its
+// latencies with.  A round of two-warp blocks takes about a third longer than one of four-warp blocks, which are fewer tokens.
+// Measured (beam 32, 256 entries, four / two warps, us): 65,536 centroids: 1,184 tokens 164 / 212, 1,536 241 / 221, 8,192 834 / 718;
+// 131,072: 1,536 290 / 278, 2,048 331 / 400, 4,096 562 / 579, 8,192 994 / 948; 262,144: 1,536 384 / 526, 8,192 1,550 / 2,091; a million:
+// 8,192 6,574 / 9,556.  With 64 members and 512 entries the same sides win.
+int graph_search_warps(const Index &ix, int64_t n_tokens)
+{
+    constexpr int64_t SM_SHARED = 228 * 1024, RESERVED = 1024;
+    auto rounds = [&](int warps) {
+        int64_t resident = 32 / warps;                       // __launch_bounds__
+        if (visited_in_shared(ix)) {
+            const int64_t room = SM_SHARED / ((ix.K + 31) / 32 * 4 + 2 * 4 * 32 * warps + 8 + RESERVED);
+            if (resident > room) resident = room;
+        }
+        return (n_tokens + resident * ix.sm_count - 1) / (resident * ix.sm_count);
+    };
+    return 4 * rounds(2) < 3 * rounds(4) ? 2 : 4;
+}
+
 int check_graph_params(const Index &ix, const GraphSearch &g, int nprobe)
 {
     if (!ix.graph) return fail(CHIMERA_INVALID_ARG, "the centroid graph is not built (chimera_index_build_graph)");
@@ -319,7 +340,7 @@ int launch_graph_probes(const Index &ix, const float *queries, int64_t n_tokens,
     const int64_t vwords = (ix.K + 31) / 32;
     const size_t smem = sizeof(uint32_t) * (size_t)vwords;
     const bool shared = visited_in_shared(ix);
-    const bool wide = g.beam > 32, four = n_tokens <= 8LL * ix.sm_count;      // (blocks that are resident at once)
+    const bool wide = g.beam > 32, four = graph_search_warps(ix, n_tokens) == 4;
     auto kern = four ? (wide ? (shared ? graph_probe_kernel<true, true, 4> : graph_probe_kernel<false, true, 4>)
                              : (shared ? graph_probe_kernel<true, false, 4> : graph_probe_kernel<false, false, 4>))
                      : (wide ? (shared ? graph_probe_kernel<true, true, 2> : graph_probe_kernel<false, true, 2>)

@@ -1,5 +1,5 @@
-"""Graph search for more query tokens than four-warp blocks are resident (two warps per token then), every dimension, short and long
-lists: probes, scores and visited sets equal the oracle's."""
+"""Graph search for more query tokens than four-warp blocks are resident (two warps per token then, unless shared memory holds as few
+of their blocks), every dimension, short and long lists: probes, scores and visited sets equal the oracle's."""
 import numpy as np
 import pytest
 import torch
@@ -35,3 +35,21 @@ def test_many_tokens(K, D, R, B, nq, nprobe, beam, E, max_exp):
         o_pr, o_sc, o_vis = oracle.graph_probes(q[b], cent, g, nprobe, beam, E, max_exp)
         assert np.array_equal(pr[b], o_pr) and np.array_equal(sc[b], o_sc)
         assert np.array_equal(vis[b], o_vis) and np.array_equal(nvis[b], o_vis.sum(1))
+
+
+@pytest.mark.parametrize("beam,E", [(32, 64), (48, 300)])
+def test_the_number_of_warps_does_not_change_a_search(beam, E):
+    """So many centroids that shared memory bounds the resident blocks: two warps per token for 1,500 tokens, four for 2,100 and for few."""
+    import paper_2608_23553_b200 as pkg
+    K, D, nq = 140_001, 32, 30
+    cent, cids, codes, doclens = random_corpus(3, 50, K, D, 2)
+    gix = pkg.Index(*(torch.from_numpy(a).cuda() for a in (cent, cids, codes, doclens)), 2)
+    gix.build_graph(32)
+    rng = np.random.default_rng(beam)
+    q = cent[rng.integers(0, K, 2_100)] + 0.2 * rng.standard_normal((2_100, D)).astype(np.float32)
+    q = torch.from_numpy((q / np.linalg.norm(q, axis=1, keepdims=True)).reshape(-1, nq, D).astype(np.float32)).cuda()
+    few = [gix.graph_probes(q[b:b + 10].contiguous(), 8, beam, E, 1 << 30) for b in range(0, len(q), 10)]
+    few = [torch.cat(x) for x in zip(*few)]
+    for b in (50, 70):
+        for got, want in zip(gix.graph_probes(q[:b].contiguous(), 8, beam, E, 1 << 30), few):
+            assert torch.equal(got, want[:len(got)])
