@@ -975,10 +975,15 @@ int launch_centroid_interaction(const Index &ix, const Params &p, const int32_t 
 // The selection of few from many in one pass over the scores.  A block waits for its loads most of the time, and the radix
 // select with the compaction behind it passes over the scores four times and over the ids once.  Here a sample of SEL_SAMPLE
 // scores gives a bound that somewhat more than n_prune scores reach (the wanted rank of the sample and four standard deviations
-// more), one pass collects those in shared memory, and the selection and the order of the survivors are found there.  False,
-// with nothing written: the bound let too few through or more than there is room for; the caller selects among all then.
+// more), one pass collects those in shared memory, and the selection and the order of the survivors are found there.  Scores in
+// masses (documents that repeat) can put more at the bound than there is room for, as the sample shows: they are counted then, and
+// where some of them are needed the bound is the threshold itself, else the ones above it are collected.
 // Measured (1,024 wanted of Mid's candidates, 1-bit refinement): 256 queries 122 -> 50 us, 64 queries 69 -> 30 us.
 // Room for 7,168 serves 4,096 wanted too (4 million documents, 64 queries, 1-bit codes: 1,798 -> 1,742 us a call; 3,584 did not).
+// Masses of equal scores, 256 queries, selected among all / with every mass collected and ties at the edge counted against one
+// another / so: 40,000 candidates, 4,096 wanted, 400 of each score 53 / 120 / 52 us, 2,000 54 / 483 / 54; 200,000, 2,000 of each 244 /
+// 526 / 225; 1,024 wanted, 10,000 of each 239 / 314 / 177.  (Collecting by votes, without an atomic each: 35 -> 50, 71 -> 115 us where all
+// scores differ: the instructions count.)
 constexpr int SEL_SAMPLE = 8192, SEL_FEW = 7168, SEL_BINS = 2048;
 struct SelFew {
     union {
@@ -1000,9 +1005,11 @@ __device__ __forceinline__ bool select_few_applies(int n, int n_prune, int *want
     *want = (int)w;
     return n >= 2 * SEL_SAMPLE && w * (float)n <= (float)(SEL_FEW / 7 * 6) * SEL_SAMPLE;
 }
-__device__ __forceinline__ bool select_few(const int32_t *__restrict__ cb, const int32_t *__restrict__ sb, int n, int n_prune,
-                                           int want, int32_t *__restrict__ out, int32_t *__restrict__ out_ci, SelFew &few,
-                                           int *hist /* [SEL_BINS] */, int *warp_part, uint32_t *s_prefix, int *s_want)
+enum { FEW_DONE, FEW_THRESHOLD, FEW_NOT };                   // selected; nothing written, *thr and *need_eq known; nothing known
+__device__ __forceinline__ int select_few(const int32_t *__restrict__ cb, const int32_t *__restrict__ sb, int n, int n_prune,
+                                          int want, int32_t *__restrict__ out, int32_t *__restrict__ out_ci, SelFew &few,
+                                          int *hist /* [SEL_BINS] */, int *warp_part, uint32_t *s_prefix, int *s_want,
+                                          uint32_t *thr_out, int *need_eq_out)
 {
     const int tid = threadIdx.x;
     // groups of four neighbours at equal distances (a 32-byte sector costs the same for one)
@@ -1020,9 +1027,36 @@ __device__ __forceinline__ bool select_few(const int32_t *__restrict__ cb, const
     if (tid == 0) few.n = 0;
     __syncthreads();
     int need_eq;
-    const uint32_t bound = radix_select([&](int j) { return (int32_t)few.sample[j]; }, SEL_SAMPLE, want, hist, warp_part, s_prefix,
-                                        s_want, &need_eq);
-    __syncthreads();                                         // the sample's place is used again
+    uint32_t bound = radix_select([&](int j) { return (int32_t)few.sample[j]; }, SEL_SAMPLE, want, hist, warp_part, s_prefix,
+                                  s_want, &need_eq);
+    // (the last digit's histogram has how many scores of the sample equal the bound)
+    const bool masses = (float)(want - need_eq + hist[bound & 1023u]) * (float)n > (float)SEL_FEW * SEL_SAMPLE;
+    __syncthreads();                                         // the sample's place and the histogram are used again
+    if (masses) {
+        int above = 0, equal = 0, n_above, n_equal;          // (of this thread's scores, of all)
+        for (int base = 0; base < n; base += 8 * SEL_THREADS) {
+            uint32_t u[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const int j = base + e * SEL_THREADS + tid;
+                u[e] = j < n ? (uint32_t)sb[j] ^ 0x80000000u : 0u;
+            }
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                above += u[e] > bound ? 1 : 0;
+                equal += u[e] == bound && base + e * SEL_THREADS + tid < n ? 1 : 0;
+            }
+        }
+        sel_block_scan(above, &n_above, warp_part);
+        sel_block_scan(equal, &n_equal, warp_part);
+        if (n_above < n_prune) {
+            *thr_out = bound;
+            *need_eq_out = n_prune - n_above;
+            return n_prune - n_above <= n_equal ? FEW_THRESHOLD : FEW_NOT;
+        }
+        if (n_above > SEL_FEW) return FEW_NOT;
+        ++bound;                                             // (there are scores above it)
+    }
     for (int base = 0; base < n; base += 8 * SEL_THREADS) {
         uint32_t u[8];
 #pragma unroll
@@ -1041,29 +1075,36 @@ __device__ __forceinline__ bool select_few(const int32_t *__restrict__ cb, const
     }
     __syncthreads();
     const int c = few.n;
-    if (c < n_prune || c > SEL_FEW) return false;
+    if (c < n_prune || c > SEL_FEW) return FEW_NOT;
     const uint32_t thr = radix_select([&](int j) { return (int32_t)(few.u[j] ^ 0x80000000u); }, c, n_prune, hist, warp_part,
                                       s_prefix, s_want, &need_eq);
-    int mine = 0, n_eq;
-    for (int i = tid; i < c; i += SEL_THREADS) mine += few.u[i] == thr ? 1 : 0;
-    int at = sel_block_scan(mine, &n_eq, warp_part);
-    const bool tied = n_eq > need_eq;                        // ties at the edge go to the smaller ids
-    if (tied) {
-        if (n_eq > SEL_BINS) return false;
-        for (int i = tid; i < c; i += SEL_THREADS)
-            if (few.u[i] == thr) hist[at++] = few.pos[i];
+    const int n_eq = hist[thr & 1023u];
+    int last = n;                                            // ties at the edge go to the smaller ids: places up to this one
+    __syncthreads();
+    if (n_eq > need_eq && n_eq <= 256) {
+        if (tid == 0) few.n = 0;
         __syncthreads();
+        for (int i = tid; i < c; i += SEL_THREADS)
+            if (few.u[i] == thr) hist[atomicAdd(&few.n, 1)] = few.pos[i];
+        __syncthreads();
+        if (tid < n_eq) {
+            const int pos = hist[tid];
+            int before = 0;
+            for (int k = 0; k < n_eq; ++k) before += hist[k] < pos ? 1 : 0;
+            if (before == need_eq - 1) *s_want = pos;
+        }
+        __syncthreads();
+        last = *s_want;
+    } else if (n_eq > need_eq) {
+        int one;                                             // (places are distinct)
+        last = -(int)(radix_select([&](int j) { return few.u[j] == thr ? -few.pos[j] : INT_MIN; }, c, need_eq, hist, warp_part,
+                                   s_prefix, s_want, &one) ^ 0x80000000u);
     }
     bool keep[(SEL_FEW + SEL_THREADS - 1) / SEL_THREADS];
 #pragma unroll
     for (int e = 0; e < (SEL_FEW + SEL_THREADS - 1) / SEL_THREADS; ++e) {
         const int i = e * SEL_THREADS + tid;
-        keep[e] = i < c && few.u[i] >= thr;
-        if (keep[e] && tied && few.u[i] == thr) {
-            int before = 0;
-            for (int k = 0; k < n_eq; ++k) before += hist[k] < few.pos[i] ? 1 : 0;
-            keep[e] = before < need_eq;
-        }
+        keep[e] = i < c && (few.u[i] > thr || (few.u[i] == thr && few.pos[i] <= last));
     }
     __syncthreads();
     // the survivors' order: buckets of neighbouring places (half a survivor each at 1,024), then the place within the bucket
@@ -1099,7 +1140,7 @@ __device__ __forceinline__ bool select_few(const int32_t *__restrict__ cb, const
             if (out_ci) out_ci[rank] = (int32_t)(few.u[i] ^ 0x80000000u);
         }
     }
-    return true;
+    return FEW_DONE;
 }
 
 // grid (B).  pruned[b][0..n_prune) ascending ids, -1 padded; n_pruned[b]; pruned_ci (optional): the score of each
@@ -1132,15 +1173,18 @@ select_kernel(const int32_t *__restrict__ cand, const int32_t *__restrict__ n_ca
         if (threadIdx.x == 0) n_pruned[b] = n;
         return;
     }
-    int need_eq, want;
-    if (MANY && select_few_applies(n, n_prune, &want) &&
-        select_few(cb, sb, n, n_prune, want, out, out_ci, few, hist, warp_part, &s_prefix, &s_want)) {
+    int need_eq, want, how = FEW_NOT;
+    uint32_t thr;
+    if (MANY && select_few_applies(n, n_prune, &want))
+        how = select_few(cb, sb, n, n_prune, want, out, out_ci, few, hist, warp_part, &s_prefix, &s_want, &thr, &need_eq);
+    if (how == FEW_DONE) {
         if (threadIdx.x == 0) n_pruned[b] = n_prune;
         return;
     }
-    __syncthreads();
-    const uint32_t thr = radix_select([&](int j) { return sb[j]; }, n, n_prune, hist, warp_part, &s_prefix, &s_want,
-                                      &need_eq);
+    if (how == FEW_NOT) {
+        __syncthreads();
+        thr = radix_select([&](int j) { return sb[j]; }, n, n_prune, hist, warp_part, &s_prefix, &s_want, &need_eq);
+    }
 
     // Ordered compaction: keep u > thr, and the first need_eq entries with u == thr.  Each thread owns four
     // consecutive entries per round, so one block scan covers 4096 entries.
