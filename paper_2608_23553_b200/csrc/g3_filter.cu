@@ -751,10 +751,10 @@ filter_seed_kernel(const int32_t *__restrict__ cand, const int32_t *__restrict__
         if (have >= 32) {
             int from = 0;
             for (; have - from >= 32; from += 32) flush(from, 32);
-            const int32_t rest = lane < have - from ? list[from + lane] : 0;
-            __syncwarp();
-            list[lane] = rest;
             have -= from;
+            const int32_t rest = lane < have ? list[from + lane] : 0;
+            __syncwarp();
+            if (lane < have) list[lane] = rest;              // (the places behind are written next, by other lanes)
         }
     }
     __syncwarp();

@@ -5,6 +5,7 @@ import subprocess
 import pytest
 
 from test_gpu_batch_scan import CALLS, tokens_and_entries
+from test_gpu_filter import REPEATED
 
 
 @pytest.fixture(scope="module")
@@ -30,6 +31,11 @@ def test_the_calls_of_the_gpu_test_take_it(rule, call):
     D, nq, K, N, lo, hi, B, nprobe, n_prune = call
     T, entries, longest = tokens_and_entries(*call)
     assert rule(K, N, T, entries, longest, B, nq, nprobe, n_prune)
+
+
+@pytest.mark.parametrize("together,nq,K,N,B,nprobe", REPEATED)
+def test_the_calls_that_turn_out_not_to_cut_are_of_both_forms(rule, together, nq, K, N, B, nprobe):
+    assert rule(K, N, 40 * N, int(9.8 * N), 50, B, nq, nprobe, 100) == bool(together)
 
 
 def test_where_it_stops(rule):

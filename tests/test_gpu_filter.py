@@ -83,17 +83,24 @@ def test_queries_with_few_candidates_in_a_batch_that_is_cut(nq):
         check_query(tn, b, res, ids[b].cpu().numpy(), sc[b].cpu().numpy(), k, n_prune, table=False)
 
 
-@pytest.mark.parametrize("nq,K,N,B,nprobe", [
-    (32, 2_000, 20_000, 260, 2),       # 8-bit rows of a query in shared memory
-    (32, 8_000, 20_000, 260, 8),       # ... from L2
-    (64, 1_000, 20_000, 100, 1),
-    (64, 3_000, 20_000, 200, 2),
-    (32, 3_000, 40_000, 31, 8),        # few queries: their contenders over several blocks
-    (32, 8_000, 40_000, 37, 16),
-    (32, 120_003, 250_000, 100, 60),   # 6-bit codes
-])
-def test_documents_that_repeat_their_centroids_are_not_cut(nq, K, N, B, nprobe):
-    """Ten centroids for about forty tokens: nearly all candidates pass the bound, and the call has to notice."""
+# scanned together, q_len, centroids, documents, queries, nprobe
+REPEATED = [
+    (1, 32, 2_000, 20_000, 260, 2),       # 8-bit rows of a query in shared memory
+    (1, 32, 8_000, 20_000, 260, 8),       # ... from L2
+    (1, 64, 1_000, 20_000, 100, 1),
+    (1, 64, 3_000, 20_000, 200, 2),
+    (1, 32, 3_000, 40_000, 31, 8),        # few queries: their contenders over several blocks
+    (1, 32, 8_000, 40_000, 37, 16),
+    (1, 32, 120_003, 250_000, 100, 60),   # 6-bit codes
+    (0, 32, 8_000, 60_000, 260, 3),
+    (0, 64, 12_000, 80_000, 130, 2),
+]
+
+
+@pytest.mark.parametrize("together,nq,K,N,B,nprobe", REPEATED)
+def test_documents_that_repeat_their_centroids_are_not_cut(together, nq, K, N, B, nprobe):
+    """Ten centroids for about forty tokens: nearly all candidates pass the bound, and the call has to notice, whether it would scan all
+    queries together or one at a time."""
     import paper_2608_23553_b200 as pkg
     D, n_prune, k = 64, 100, 20
     cent, cids, codes, doclens = random_corpus(K + B, N, K, D, 2, len_lo=30, len_hi=50)
