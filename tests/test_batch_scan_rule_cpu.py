@@ -5,7 +5,7 @@ import subprocess
 import pytest
 
 from test_gpu_batch_scan import CALLS, tokens_and_entries
-from test_gpu_filter import REPEATED
+from test_gpu_filter import CALLS as CUT_CALLS, REPEATED
 
 
 @pytest.fixture(scope="module")
@@ -36,6 +36,14 @@ def test_the_calls_of_the_gpu_test_take_it(rule, call):
 @pytest.mark.parametrize("together,nq,K,N,B,nprobe", REPEATED)
 def test_the_calls_that_turn_out_not_to_cut_are_of_both_forms(rule, together, nq, K, N, B, nprobe):
     assert rule(K, N, 40 * N, int(9.8 * N), 50, B, nq, nprobe, 100) == bool(together)
+
+
+def test_two_calls_of_the_cut_go_by_query(rule):
+    forms = []
+    for cut, _, _, nq, K, N, lo, hi, B, nprobe, n_prune, _, _ in CUT_CALLS:
+        length = (lo + hi) / 2
+        forms.append(rule(K, N, N * length, N * K * (1 - (1 - 1 / K) ** length), hi, B, nq, nprobe, n_prune))
+    assert forms == 10 * [True] + 2 * [False] + 4 * [False]
 
 
 def test_where_it_stops(rule):

@@ -12,8 +12,8 @@ pytestmark = pytest.mark.gpu
 
 
 # cut: whether the call runs it (the last four rows have too many centroids, or too long a pruning list, for what their
-# candidates hold)
-@pytest.mark.parametrize("cut,D,nbits,nq,K,N,len_lo,len_hi,B,nprobe,n_prune,shift,copies", [
+# candidates hold).  The two before those scan one query at a time, the others all queries together.
+CALLS = [
     (1, 32, 2, 32, 509, 20_000, 1, 80, 260, 1, 300, 0, 1),          # 16-bit numbers from the 8-bit table
     (1, 64, 2, 64, 2_000, 20_001, 20, 61, 256, 1, 1_111, 1, 1),      # two column groups; centroid ids 4 bytes off 16
     (1, 128, 2, 32, 120_003, 30_000, 60, 99, 250, 32, 50, 3, 1),     # 6-bit codes, K not a multiple of five
@@ -24,24 +24,41 @@ pytestmark = pytest.mark.gpu
     (1, 64, 2, 47, 2_000, 9_000, 20, 90, 60, 1, 300, 0, 1),          # ... rows of an odd number of values, two per lane
     (1, 32, 2, 127, 1_000, 6_000, 20, 70, 80, 1, 200, 0, 1),         # ... four per lane, the longest query
     (1, 32, 2, 32, 300, 20_000, 1, 80, 260, 1, 333, 0, 50),          # every document 50 times: masses of equal scores
+    (1, 64, 2, 32, 12_000, 60_000, 30, 50, 260, 1, 100, 1, 1),
+    (1, 96, 1, 21, 8_000, 40_000, 1, 99, 260, 1, 100, 3, 1),
     (0, 128, 2, 32, 120_003, 9_999, 60, 99, 280, 16, 50, 3, 1),
     (0, 32, 1, 64, 106_497, 5_000, 200, 300, 170, 8, 20, 2, 1),
     (0, 32, 2, 40, 107_001, 8_000, 90, 120, 25, 16, 64, 0, 1),
     (0, 64, 2, 32, 6_000, 24_000, 1, 70, 256, 1, 5_900, 0, 1),       # fewer candidates than 1.5 n_prune
-])
-def test_filtered_searches_match_the_oracle(cut, D, nbits, nq, K, N, len_lo, len_hi, B, nprobe, n_prune, shift, copies):
+]
+PARAMETERS = "cut,D,nbits,nq,K,N,len_lo,len_hi,B,nprobe,n_prune,shift,copies"
+
+
+def corpus(D, nbits, nq, K, N, len_lo, len_hi, shift, copies):
+    """Arrays on the host and an index of them whose centroid ids start `shift` places behind a 16-byte boundary."""
     import paper_2608_23553_b200 as pkg
     cent, cids, codes, doclens = random_corpus(300 + nq + D, N // copies, K, D, nbits, len_lo=len_lo, len_hi=len_hi)
     if copies > 1:
         cids, codes, doclens = (np.concatenate([a] * copies) for a in (cids, codes, doclens))
-    oix = oracle.make_index(cent, cids, codes, doclens, nbits)
     padded = torch.zeros(shift + len(cids), dtype=torch.int32, device="cuda")
     padded[shift:] = torch.from_numpy(cids).cuda()
     gix = pkg.Index(torch.from_numpy(cent).cuda(), padded[shift:], torch.from_numpy(codes).cuda(),
                     torch.from_numpy(doclens).cuda(), nbits)
+    return cent, cids, codes, doclens, gix
+
+
+def queries(cent, B, nq):
     rng = np.random.default_rng(nq)
+    K, D = cent.shape
     q = cent[rng.integers(0, K, size=(B, nq))] + 0.3 / np.sqrt(D) * rng.standard_normal((B, nq, D)).astype(np.float32)
-    q = (q / np.linalg.norm(q, axis=2, keepdims=True)).astype(np.float32)
+    return (q / np.linalg.norm(q, axis=2, keepdims=True)).astype(np.float32)
+
+
+@pytest.mark.parametrize(PARAMETERS, CALLS)
+def test_filtered_searches_match_the_oracle(cut, D, nbits, nq, K, N, len_lo, len_hi, B, nprobe, n_prune, shift, copies):
+    cent, cids, codes, doclens, gix = corpus(D, nbits, nq, K, N, len_lo, len_hi, shift, copies)
+    oix = oracle.make_index(cent, cids, codes, doclens, nbits)
+    q = queries(cent, B, nq)
     k = min(n_prune, 25)
     taps = gix.alloc_taps(B, nq, nprobe, n_prune, table=False)
     ids, sc = gix.search(torch.from_numpy(q).cuda(), nprobe, n_prune, k, taps=taps)
@@ -53,6 +70,25 @@ def test_filtered_searches_match_the_oracle(cut, D, nbits, nq, K, N, len_lo, len
     for b in (0, B - 1):
         res = oracle.pipeline(q[b], oix, nprobe, n_prune, k)
         check_query(tn, b, res, ids[b], sc[b], k, n_prune, table=False)
+
+
+@pytest.mark.parametrize(PARAMETERS, [c for c in CALLS if c[0]])
+def test_candidates_from_the_caller_are_cut_one_query_at_a_time(cut, D, nbits, nq, K, N, len_lo, len_hi, B, nprobe, n_prune, shift, copies):
+    """Stages 3 to 5 on the table and the candidates of a search (whose results the test above checks): the scan by query in all its
+    forms, where the search scanned all queries together."""
+    cent, _, _, _, gix = corpus(D, nbits, nq, K, N, len_lo, len_hi, shift, copies)
+    q = torch.from_numpy(queries(cent, B, nq)).cuda()
+    k = min(n_prune, 25)
+    taps = gix.alloc_taps(B, nq, nprobe, n_prune, ci=False)
+    whole = [t.clone() for t in gix.search(q, nprobe, n_prune, k, taps=taps)]
+    pruned, n_pruned, n_cand = taps.pruned.clone(), taps.n_pruned.clone(), taps.n_cand.clone()
+    taps.pruned.fill_(-2)
+    got = gix.run_stages(3, 5, q, B, nq, nprobe, n_prune, k, taps)
+    assert gix.status() == 0
+    kept = np.array(gix.kept(B, nq, nprobe, n_prune, k))
+    assert kept.sum() < 0.7 * int(n_cand.sum()) and (kept <= n_cand.cpu().numpy()).all()
+    assert torch.equal(taps.pruned, pruned) and torch.equal(taps.n_pruned, n_pruned)
+    assert torch.equal(got[0], whole[0]) and torch.equal(got[1], whole[1])
 
 
 @pytest.mark.parametrize("nq", [32, 21])

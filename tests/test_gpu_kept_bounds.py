@@ -10,7 +10,7 @@ pytestmark = pytest.mark.gpu
 
 
 # D, q_len, centroids, documents, shortest, longest, queries, nprobe, n_prune
-@pytest.mark.parametrize("call", [
+CALLS = [
     (32, 32, 1_029, 9_000, 1, 400, 257, 4, 260),         # 32-byte rows
     (32, 64, 2_047, 3_000, 500, 1_500, 220, 1, 300),     # 64-byte rows, hundreds of near tokens
     (64, 90, 999, 3_000, 300, 900, 220, 1, 300),         # 128-byte rows
@@ -19,10 +19,30 @@ pytestmark = pytest.mark.gpu
     (32, 32, 1_029, 9_000, 1, 400, 41, 4, 60),           # too few documents: the same
     (128, 32, 120_003, 20_000, 90, 160, 250, 32, 263),   # 6-bit codes
     (32, 40, 107_001, 9_000, 150, 250, 220, 16, 300),    # ... without a mask
-])
+]
+
+
+@pytest.mark.parametrize("call", CALLS)
 def test_kept_candidates_are_bounded_like_the_oracle_orders_them(call):
     arrays = corpus(*call)
     check(arrays, queries(np.random.default_rng(call[1]), arrays[0], call[6], call[1]), call[7], call[8])
+
+
+@pytest.mark.parametrize("call", CALLS)
+def test_the_masks_of_a_scan_by_query_lead_to_the_same_documents(call):
+    """Stages 3 to 5 on the table and candidates of the search that the test above checks: the other kernels that write the masks."""
+    import torch
+    import paper_2608_23553_b200 as pkg
+    B, nq, nprobe, n_prune = call[6], call[1], call[7], call[8]
+    arrays = corpus(*call)
+    gix = pkg.Index(*(torch.from_numpy(a).cuda() for a in arrays), 2)
+    q = torch.from_numpy(queries(np.random.default_rng(nq), arrays[0], B, nq)).cuda()
+    taps = gix.alloc_taps(B, nq, nprobe, n_prune, ci=False)
+    ids, scores = (t.clone() for t in gix.search(q, nprobe, n_prune, 10, taps=taps))
+    pruned = taps.pruned.clone()
+    got = gix.run_stages(3, 5, q, B, nq, nprobe, n_prune, 10, taps)
+    assert gix.status() == 0
+    assert torch.equal(taps.pruned, pruned) and torch.equal(got[0], ids) and torch.equal(got[1], scores)
 
 
 # q_len, query tokens near one direction
