@@ -272,6 +272,19 @@ int chimera_workspace_status(const void *workspace, void *stream, int32_t *statu
 int chimera_workspace_kept(const chimera_index *index, int32_t n_queries, int32_t q_len, int32_t nprobe, int32_t n_prune,
                            int32_t k, int64_t max_candidates, const void *workspace, void *stream, int32_t *n_kept);
 
+/* How the first cut of a chimera_search with these parameters scans its candidates (host arithmetic on the sizes): writes to
+ * *together (host pointer) 0 where calls of these sizes do not cut, 1 where each query's candidates are scanned by themselves, or
+ * the number of queries (8 to 256) that one pass over the corpus serves side by side. */
+int chimera_cut_plan(const chimera_index *index, int32_t n_queries, int32_t q_len, int32_t nprobe, int32_t n_prune, int32_t k,
+                     int64_t max_candidates, int32_t *together);
+/* After a chimera_search with these parameters on `workspace` that scanned queries side by side (chimera_cut_plan > 1): how many
+ * centroids of each query reached past the largest code of that pass and were added to their documents afterwards; beyond
+ * CHIMERA_LISTED_ROOM all of the query's centroids are looked at again for it.  Synchronises the stream and writes n_queries
+ * numbers to n_listed (host pointer), -1 where the search had no such pass. */
+#define CHIMERA_LISTED_ROOM 1024
+int chimera_workspace_listed(const chimera_index *index, int32_t n_queries, int32_t q_len, int32_t nprobe, int32_t n_prune,
+                             int32_t k, int64_t max_candidates, const void *workspace, void *stream, int32_t *n_listed);
+
 /* How a search with these parameters finds its probes (Sec. 3.2 step 1, the top-n_probe centroids of each query
  * token).  Writes to *sample_stride (host pointer) 0 when stage 2a is a scan of the finished score table, or s > 1
  * when stages 1 and 2a run together in calls that cover both: every s-th tile of 128 centroids is scored first, a

@@ -328,6 +328,24 @@ class Index:
                                             ctypes.c_int64(max_candidates), _ptr(self._ws), _stream(), out))
         return list(out)
 
+    def cut_plan(self, n_queries, q_len, nprobe, n_prune, k, max_candidates=0) -> int:
+        """0 where searches with these parameters have no first cut, 1 where it scans a query at a time, else how many
+        queries one pass over the corpus serves (chimera_cut_plan)."""
+        n = ctypes.c_int32()
+        _check(lib().chimera_cut_plan(self._h, ctypes.c_int32(n_queries), ctypes.c_int32(q_len), ctypes.c_int32(nprobe),
+                                      ctypes.c_int32(n_prune), ctypes.c_int32(k), ctypes.c_int64(max_candidates),
+                                      ctypes.byref(n)))
+        return n.value
+
+    def listed(self, n_queries, q_len, nprobe, n_prune, k, max_candidates=0) -> list:
+        """After a search with these parameters: the centroids of each query past the largest code of such a pass, -1
+        where there was none (chimera_workspace_listed)."""
+        out = (ctypes.c_int32 * n_queries)()
+        _check(lib().chimera_workspace_listed(self._h, ctypes.c_int32(n_queries), ctypes.c_int32(q_len),
+                                              ctypes.c_int32(nprobe), ctypes.c_int32(n_prune), ctypes.c_int32(k),
+                                              ctypes.c_int64(max_candidates), _ptr(self._ws), _stream(), out))
+        return list(out)
+
     def workspace_check(self, n_queries, q_len, nprobe, n_prune, k, max_candidates=0) -> int:
         """Debug build only: index of the first damaged guard region of the workspace after a search with these
         parameters, -1 if all are intact (chimera_workspace_check)."""

@@ -915,6 +915,37 @@ int chimera_workspace_kept(const chimera_index *index, int32_t n_queries, int32_
     return CHIMERA_OK;
 }
 
+int chimera_cut_plan(const chimera_index *index, int32_t n_queries, int32_t q_len, int32_t nprobe, int32_t n_prune, int32_t k,
+                     int64_t max_candidates, int32_t *together)
+{
+    const Index *ix = reinterpret_cast<const Index *>(index);
+    Params p;
+    int rc = check_params(ix, n_queries, q_len, nprobe, n_prune, k, max_candidates, &p);
+    if (rc) return rc;
+    if (!together) return fail(CHIMERA_INVALID_ARG, "NULL argument");
+    *together = batch_scan_used(*ix, p) ? batch_group(p) : filter_used(*ix, p) ? 1 : 0;
+    return CHIMERA_OK;
+}
+
+int chimera_workspace_listed(const chimera_index *index, int32_t n_queries, int32_t q_len, int32_t nprobe, int32_t n_prune,
+                             int32_t k, int64_t max_candidates, const void *workspace, void *stream, int32_t *n_listed)
+{
+    const Index *ix = reinterpret_cast<const Index *>(index);
+    Params p;
+    int rc = check_params(ix, n_queries, q_len, nprobe, n_prune, k, max_candidates, &p);
+    if (rc) return rc;
+    if (!workspace || !n_listed) return fail(CHIMERA_INVALID_ARG, "NULL argument");
+    if (!batch_scan_used(*ix, p)) {
+        for (int b = 0; b < p.B; ++b) n_listed[b] = -1;
+        return CHIMERA_OK;
+    }
+    const Layout L = make_layout(*ix, p);
+    CHIMERA_CUDA(cudaMemcpyAsync(n_listed, (const char *)workspace + L.flt_over + batch_over_bytes(p) - sizeof(int32_t) * (size_t)p.B,
+                                 sizeof(int32_t) * (size_t)p.B, cudaMemcpyDeviceToHost, (cudaStream_t)stream));
+    CHIMERA_CUDA(cudaStreamSynchronize((cudaStream_t)stream));
+    return CHIMERA_OK;
+}
+
 int chimera_is_debug_build(void)
 {
 #ifdef CHIMERA_DEBUG

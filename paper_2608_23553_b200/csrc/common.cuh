@@ -302,7 +302,9 @@ FirstCut first_cut(const Params &p, const Layout &L, char *ws);
 bool filter_used(const Index &ix, const Params &p);
 bool filter_mask_used(const Index &ix, const Params &p, bool batch);      // the masks are written
 bool batch_scan_used(const Index &ix, const Params &p);       // ... and scans for all queries at once (g3_batch_scan.cu)
+int batch_group(const Params &p);                             // that many side by side
 size_t batch_table_bytes(const Index &ix, const Params &p);
+// ... with the numbers of listed centroids, int32 [B], at its end.
 size_t batch_over_bytes(const Params &p);
 size_t filter_table_pitch(const Index &ix);
 int filter_hist_bins();

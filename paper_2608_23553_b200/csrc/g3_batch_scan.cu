@@ -24,13 +24,13 @@ namespace chimera {
 
 constexpr int BS_TILE = 64;               // documents per tile
 constexpr int BS_THREADS = 256;
-constexpr int BS_OVER = 1024;             // listed centroids per query; with more of them all rows are looked at again
+constexpr int BS_OVER = CHIMERA_LISTED_ROOM;             // listed centroids per query; with more of them all rows are looked at again
 
 constexpr int BS_TOP = 63;                // the largest code
 constexpr int BS_MAX_LEN = 65535 / BS_TOP;              // tokens of a document: sums are 16-bit fields
 
 // Queries side by side in a row, a byte each.
-static int batch_group(const Params &p)
+int batch_group(const Params &p)
 {
     return p.B <= 8 ? 8 : p.B <= 16 ? 16 : p.B <= 32 ? 32 : p.B <= 64 ? 64 : p.B <= 128 ? 128 : 256;
 }

@@ -4,7 +4,7 @@ import subprocess
 
 import pytest
 
-from test_gpu_batch_scan import CALLS, tokens_and_entries
+from test_gpu_batch_scan import CALLS, CROWDED, tokens_and_entries
 from test_gpu_filter import CALLS as CUT_CALLS, REPEATED
 
 
@@ -31,6 +31,12 @@ def test_the_calls_of_the_gpu_test_take_it(rule, call):
     D, nq, K, N, lo, hi, B, nprobe, n_prune = call
     T, entries, longest = tokens_and_entries(*call)
     assert rule(K, N, T, entries, longest, B, nq, nprobe, n_prune)
+
+
+@pytest.mark.parametrize("nq", [20, 32, 64])
+def test_so_does_the_call_with_too_many_listed_centroids(rule, nq):
+    D, K, N, lo, hi, B, nprobe, n_prune = CROWDED
+    assert rule(K, N, 100 * N, 99 * N, hi, B, nq, nprobe, n_prune)
 
 
 @pytest.mark.parametrize("together,nq,K,N,B,nprobe", REPEATED)

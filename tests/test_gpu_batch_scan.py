@@ -67,21 +67,27 @@ def test_batches_scanned_together_match_the_oracle(call):
     check(arrays, queries(np.random.default_rng(call[1]), arrays[0], call[6], call[1]), call[7], call[8])
 
 
+CROWDED = (32, 8_192, 6_000, 60, 140, 60, 16, 50)        # D, centroids, documents, shortest, longest, queries, nprobe, n_prune
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("nq", [20, 32, 64])
 def test_more_listed_centroids_than_there_is_room_for(nq):
-    """Six thousand centroids near one direction, at places that no sample looks at; every query has tokens there."""
+    """Four thousand centroids near one direction, at odd places, which neither sample looks at (every second centroid for the
+    thresholds, every fourth for the step); every query has tokens there, and a fiftieth of the documents' tokens."""
     rng = np.random.default_rng(nq)
-    D, K, N, B = 32, 8_192, 6_000, 60
-    cent, cids, codes, doclens = random_corpus(9, N, K, D, 2, len_lo=60, len_hi=140)
-    near = np.arange(K) % 4 != 0
+    D, K, N, lo, hi, B, nprobe, n_prune = CROWDED
+    cent, cids, codes, doclens = random_corpus(9, N, K, D, 2, len_lo=lo, len_hi=hi)
+    near = np.arange(K) % 2 == 1
     cent[near] = cent[4] + 0.9 / np.sqrt(D) * rng.standard_normal((int(near.sum()), D)).astype(np.float32)
     cent[near] /= np.linalg.norm(cent[near], axis=1, keepdims=True)
     far = np.flatnonzero(~near)
     cids = np.where(rng.random(len(cids)) < 0.02, cids, rng.choice(far, len(cids))).astype(np.int32)
     q = queries(rng, cent[far], B, nq)
     q[:, :nq // 2] = queries(rng, cent[near], B, nq // 2)
-    check((cent, cids, codes, doclens), q, 16, 50, cut=False)
+    gix, _ = check((cent, cids, codes, doclens), q, nprobe, n_prune)
+    assert gix.cut_plan(B, nq, nprobe, n_prune, 25) == 64
+    assert min(gix.listed(B, nq, nprobe, n_prune, 25)) > 1_024
 
 
 @pytest.mark.gpu
