@@ -13,8 +13,8 @@
 // scan of Mid's batch of 256, but four times the step: a third more candidates kept, or long lists to add.)
 //
 //   batch_quantum_kernel   step and sum of theta of each query
-//   batch_excess_kernel    the codes, and the list of centroids with more than 15 steps (from the 8-bit table;
-//                          batch_excess_exact_kernel for other query lengths)
+//   batch_excess_kernel    the codes, and the list of centroids with more than BS_TOP steps (from the 8-bit
+//                          table; batch_excess_exact_kernel for other query lengths)
 //   batch_scan_kernel      hi0 of every candidate
 //   batch_over_kernel      the rest of the listed centroids
 //   batch_hist_kernel      histogram of the bounds, for the choice of the seeds
@@ -24,7 +24,7 @@ namespace chimera {
 
 constexpr int BS_TILE = 64;               // documents per tile
 constexpr int BS_THREADS = 256;
-constexpr int BS_OVER = CHIMERA_LISTED_ROOM;             // listed centroids per query; with more of them all rows are looked at again
+constexpr int BS_OVER = CHIMERA_LISTED_ROOM;     // listed centroids per query; with more of them all rows are looked at again
 
 constexpr int BS_TOP = 63;                // the largest code
 constexpr int BS_MAX_LEN = 65535 / BS_TOP;              // tokens of a document: sums are 16-bit fields

@@ -312,7 +312,7 @@ filter_sample_kernel(const uint8_t *__restrict__ table8, int64_t K, const int32_
         ci = __reduce_add_sync(0xffffffffu, lane < LPR ? ci : 0) + NQ / 2;
         over = __reduce_add_sync(0xffffffffu, over);
         const int base = __reduce_add_sync(0xffffffffu, lane < LPR ? sum_tm1 : 0) + NQ;
-        // codes round up: 6-bit ones by half a step of 7 % on average, 4-bit ones by half a step of the query's
+        // codes round up: the scan by query's by half a step of 7 % on average, the batch's by half a step of the query's
         if (scale) over += __reduce_add_sync(0xffffffffu, above) * (scale[b].y - 1) / 2;
         else if (coded) over += over / 28;
         if (lane == 0) mine[s] = make_int2(ci, base + over);
