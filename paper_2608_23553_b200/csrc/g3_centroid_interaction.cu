@@ -610,18 +610,20 @@ ci_coarse_rng_kernel(const uint8_t *__restrict__ table8, int64_t K, const int2 *
 // With few rows left to look up the instructions around them count (a document per warp: 1,890 us, 570 instructions each), so four
 // documents share a warp, eight lanes each, those of a group of 32 taken by length: a bit per token from shared memory says
 // whether it is near, near ids are collected in shared memory and their rows looked up 8 / LPR at a time and document.  nq: the columns that count; the rest of
-// the 16 LPR are zero in every row.  runs: byte x of a row is column x / runs + 32 (x % runs).  rng: token ranges; (CI, 0) stands for a document whose CI is known.
+// the 16 LPR are zero in every row.  Byte x of a row is column x / RUNS + 32 (x % RUNS), or x where stage 1 wrote the rows (RUNS as an
+// argument: 1,013 us where constants take 981, Mid, batch 256).  rng: token ranges; (CI, 0) stands for a document whose CI is known.
 constexpr int BOUND_THREADS = 512;
 constexpr int BOUND_LIST = 64, BOUND_PITCH = BOUND_LIST + 8;
 template <int LPR>
 __global__ void __launch_bounds__(BOUND_THREADS, 2)
-ci_bound_kernel(const uint8_t *__restrict__ table8, int64_t K, int nq, int runs, const uint32_t *__restrict__ mask, int mask_words,
+ci_bound_kernel(const uint8_t *__restrict__ table8, int64_t K, int nq, const uint32_t *__restrict__ mask, int mask_words,
                 const int32_t *__restrict__ theta, const int32_t *__restrict__ tau, const int2 *__restrict__ rng,
                 const int32_t *__restrict__ n_docs, int64_t maxc, const int32_t *__restrict__ cids, int32_t *__restrict__ hi,
                 int32_t *__restrict__ rest, int32_t *__restrict__ n_rest, FirstCut cut)
 {
     pdl_entry();
     constexpr int NQ = 16 * LPR, RPS = 8 / LPR;              // columns of a row, rows per step and document
+    constexpr int RUNS = NQ / 32;                            // of a row that the first cut made (stage 1: nq == NQ, in order)
     constexpr int NF = LPR;                                  // registers (two columns each) of a lane after the folding
     constexpr int U = 4;                                     // steps in flight
     extern __shared__ uint32_t s_mask[];                     // and a zero word for positions past a document's end
@@ -646,7 +648,7 @@ ci_bound_kernel(const uint8_t *__restrict__ table8, int64_t K, int nq, int runs,
         uint32_t w = 0;
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-            const int at = 16 * sub + 4 * k + e, col = at / runs + 32 * (at % runs);
+            const int at = 16 * sub + 4 * k + e, col = nq == NQ ? at : at / RUNS + 32 * (at % RUNS);
             if (col < nq) w |= (uint32_t)(theta[(int64_t)b * nq + col] - 1) << (8 * e);
         }
         floor_f[k] = w << 8;
@@ -898,8 +900,7 @@ int launch_kept_bounds(const Index &ix, const Params &p, const uint8_t *table8, 
         auto kern = p.nq <= 32 ? ci_bound_kernel<2> : p.nq <= 64 ? ci_bound_kernel<4> : ci_bound_kernel<8>;
         constexpr size_t MASK_MOST = 40 * 1024;             // more than 266,240 centroids are not cut (filter_used)
         CHIMERA_CUDA(allow_shared(kern, MASK_MOST));
-        const int runs = coarse_supported(p.nq) ? 1 : coarse_pitch(p.nq) / 32;        // (rows from stage 1, or from the first cut)
-        launch(kern, dim3((unsigned)gx, (unsigned)p.B), BOUND_THREADS, smem, st, table8, ix.K, p.nq, runs, mask, (int)words, theta, tau, rng,
+        launch(kern, dim3((unsigned)gx, (unsigned)p.B), BOUND_THREADS, smem, st, table8, ix.K, p.nq, mask, (int)words, theta, tau, rng,
                n_docs, p.maxc, ix.cids, hi, rest, n_rest, cut);
         CHIMERA_CUDA(cudaGetLastError());
         count_launch(SLOT_CI);
