@@ -999,7 +999,7 @@ struct SelFew {
 };
 // The wanted rank of the sample.  Taken from 16,384 scores on (shorter lists cost a pass of the block's loads or two, no more
 // than the sample) while the documents to be expected fill no more than 6/7 of the list.
-__device__ __forceinline__ bool select_few_applies(int n, int n_prune, int *want)
+__host__ __device__ __forceinline__ bool select_few_applies(int n, int n_prune, int *want)
 {
     const float r = (float)n_prune * ((float)SEL_SAMPLE / (float)n);
     const float w = r + 4.f * sqrtf(r) + 8.f;
@@ -1723,6 +1723,18 @@ size_t select_split_scratch_bytes(const Index &ix, const Params &p)
     return select_split_used(ix, p) ? sizeof(int32_t) * (size_t)p.B * SELS_SCRATCH : 0;
 }
 
+// The kernel with select_few costs where it does not come to that: its shared memory makes the SM change its split between kernels
+// (140 queries of 8,184 candidates 14.3 -> 16.4 us, one short list 167.7 -> 168.9 a call), and its other path is slower (6 queries of a
+// million, 9,439 wanted: 478 -> 517).  Taken where it applies to half the candidates that independent tokens would give: more than
+// that are rare, and where it does apply it takes less than half the time.
+bool select_few_used(const Index &ix, const Params &p)
+{
+    const double half = 0.5 * expected_candidates(ix, p);
+    int want;
+    return p.maxc >= 2 * SEL_SAMPLE && half >= SEL_SAMPLE &&
+           select_few_applies(half > 2 * SEL_SAMPLE ? (int)half : 2 * SEL_SAMPLE, p.n_prune, &want);
+}
+
 // scratch: select_split_scratch_bytes() bytes, or NULL (one block per query then).  many: the lists are all the candidates, not
 // a few contenders.
 int launch_select(const Index &ix, const Params &p, const int32_t *cand, const int32_t *n_cand, const int32_t *ci,
@@ -1742,8 +1754,7 @@ int launch_select(const Index &ix, const Params &p, const int32_t *cand, const i
         count_launch(SLOT_SELECT, 5);
         return CHIMERA_OK;
     }
-    // (shared memory that a short list does not need makes the SM change its split between kernels: one query 167.7 -> 168.9 us)
-    if (many) {
+    if (many && select_few_used(ix, p)) {
         CHIMERA_CUDA(allow_shared(select_kernel<true>, sizeof(SelFew)));
         launch(select_kernel<true>, (unsigned)p.B, SEL_THREADS, sizeof(SelFew), st, cand, n_cand, ci, p.maxc, p.n_prune, pruned,
                n_pruned, pruned_ci);

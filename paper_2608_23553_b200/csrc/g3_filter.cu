@@ -75,12 +75,15 @@ static int filter_codec(int64_t K)
 //     262,144 centroids, 2.2 M tokens each: 2,451 / 2,300; with four probes, 8.7 M each: 32 queries 2,746 / 3,103, two 414 / 372.
 //   others: 4 per centroid, 4 n_prune documents, 2 M a call.  21 tokens, 20,000 documents, 1.3 M tokens: 143 us with the cut, 133
 //     without; 2.6 M: 153 / 181; 100 tokens on 200,000 documents, 12 M: 263 / 756.
+double expected_candidates(const Index &ix, const Params &p)
+{
+    const double distinct = (double)ix.ivf_len / (double)ix.N, probed = (double)p.nq * p.P / (double)ix.K;
+    const double cand = probed < 1.0 ? (double)ix.N * (1.0 - pow(1.0 - probed, distinct)) : (double)ix.N;
+    return cand < (double)p.maxc ? cand : (double)p.maxc;
+}
 double expected_tokens(const Index &ix, const Params &p)
 {
-    const double len = (double)ix.T / (double)ix.N, distinct = (double)ix.ivf_len / (double)ix.N;
-    const double probed = (double)p.nq * p.P / (double)ix.K;
-    const double cand = probed < 1.0 ? (double)ix.N * (1.0 - pow(1.0 - probed, distinct)) : (double)ix.N;
-    return (cand < (double)p.maxc ? cand : (double)p.maxc) * len;
+    return expected_candidates(ix, p) * ((double)ix.T / (double)ix.N);
 }
 // Share of the centroids above each threshold: FILTER_LAMBDA tokens of a document.  Its length is that of the documents that
 // compete for the top: about halfway between the candidates' mean (somewhat above the corpus's: long documents are probed more

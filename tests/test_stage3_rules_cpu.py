@@ -1,4 +1,4 @@
-"""When stage 3 runs its first cut, starts its bounds from near tokens and keeps visits as lists: host arithmetic on the sizes, no
+"""When stage 3 runs its first cut, starts its bounds from near tokens, keeps visits as lists and selects few from many: host arithmetic on the sizes, no
 device."""
 import os
 import subprocess
@@ -39,6 +39,11 @@ def lists(routes):
 @pytest.fixture(scope="module")
 def near_first(routes):
     return lambda *a, **kw: routes(*a, **kw)[2]
+
+
+@pytest.fixture(scope="module")
+def few(routes):
+    return lambda *a, **kw: routes(*a, **kw)[3]
 
 
 def test_what_the_candidates_hold_counts_and_not_the_room_for_them(rule):
@@ -92,3 +97,17 @@ def test_bounds_start_with_near_tokens_where_that_decides(near_first):
     assert not near_first(65_536, 500_000, 50, 64, 32, 8, 2_048) and near_first(65_536, 500_000, 51, 64, 32, 8, 2_048)
     # 6-bit codes from the exact table, a query at a time
     assert not near_first(262_144, 8_800_000, 68, 256, 40, 4, 4_096) and near_first(262_144, 8_800_000, 68, 256, 32, 4, 4_096)
+
+
+def test_few_are_selected_from_many_where_the_lists_are_long_and_the_wanted_few(few):
+    mid = (65_536, 500_000, 120, 256, 32)
+    assert few(*mid, 4, 1_024) and few(*mid, 4, 4_096) and few(262_144, 8_800_000, 68, 256, 32, 4, 4_096)
+    # short lists, whatever is wanted: 8,184 documents, or 16,384 candidates to be expected of many more
+    assert not few(275, 8_184, 30, 140, 32, 7, 133) and not few(275, 16_383, 30, 140, 32, 7, 133) and few(275, 16_384, 30, 140, 32, 7, 133)
+    assert [few(65_536, n, 120, 64, 32, 4, 100) for n in (78_000, 79_000)] == [False, True]
+    # more than a list of 16,384 has room for, and longer lists with more wanted than that
+    assert not few(81_311, 1_240_245, 65, 6, 64, 17, 9_439)
+    assert [few(64, 100_000, 4, 64, 8, 16, w) for w in (4_800, 5_800)] == [True, False]
+    assert [few(64, n, 4, 64, 8, 16, 1_024) for n in (5_500_000, 5_900_000)] == [True, False]
+    # a capacity below the smallest list
+    assert not few(*mid, 4, 1_024, max_candidates=16_383) and few(*mid, 4, 1_024, max_candidates=16_384)
