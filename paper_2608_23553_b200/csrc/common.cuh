@@ -329,6 +329,8 @@ int launch_centroid_interaction(const Index &ix, const Params &p, const int32_t 
                                 cudaStream_t st);
 // pruned_ci (may be NULL): the score of each kept document, INT_MIN in the padding.
 // scratch: select_split_scratch_bytes() bytes (few queries per call: several blocks per query), or NULL.
+enum { GATHER_L2, GATHER_SHARED, GATHER_RANGES };                 // where the bits of a query's candidates are set
+int gather_form(const Index &ix, const Params &p);
 double expected_candidates(const Index &ix, const Params &p);     // of a query
 bool select_few_used(const Index &ix, const Params &p);           // a selection among all candidates is prepared for few of many
 bool select_split_used(const Index &ix, const Params &p);

@@ -40,7 +40,9 @@ mark_kernel(const int32_t *__restrict__ probes, int n_lists, const int64_t *__re
 
 // The same with the bitmap in shared memory, for small corpora: their lists set the same few words over and over, and
 // atomics on one L2 line come one after the other (10,000 documents, 128 lists of 625: 17 us, here 6.5).  grid (blocks, B): a
-// block takes every gridDim.x-th list and adds its bits to the query's bitmap at the end.
+// block takes every gridDim.x-th list and adds its bits to the query's bitmap at the end.  Its warps share a list, 256 entries
+// each, from another warp for the next list (a warp per list, the longest one took the time: one query, 400,000 documents, 1,024 lists
+// of popular centroids, stage 2b 189 us in 16 blocks, 112 so and 70 in 32).
 constexpr int MARK_SHARED_WORDS = 24 * 1024;
 __global__ void __launch_bounds__(512)
 mark_shared_kernel(const int32_t *__restrict__ probes, int n_lists, const int64_t *__restrict__ ivf_off,
@@ -51,23 +53,32 @@ mark_shared_kernel(const int32_t *__restrict__ probes, int n_lists, const int64_
     const int b = blockIdx.y;
     for (int w = threadIdx.x; w < words; w += 512) bits[w] = 0u;
     __syncthreads();
-    // a warp per list
-    for (int l = blockIdx.x + gridDim.x * (threadIdx.x >> 5); l < n_lists; l += gridDim.x * 16) {
-        const int32_t c = DBG_CID(probes[(int64_t)b * n_lists + l]);
-        const int64_t hi = ivf_off[c + 1];
-        for (int64_t e0 = ivf_off[c] + (threadIdx.x & 31); e0 < hi; e0 += 8 * 32) {
-            uint32_t d[8];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int l0 = blockIdx.x; l0 < n_lists; l0 += 32 * gridDim.x) {
+        const int l = l0 + lane * (int)gridDim.x, left = (n_lists - l0 + (int)gridDim.x - 1) / (int)gridDim.x;
+        int64_t lo = 0, hi = 0;                              // of this lane's list
+        if (l < n_lists) {
+            const int32_t c = DBG_CID(probes[(int64_t)b * n_lists + l]);
+            lo = ivf_off[c];
+            hi = ivf_off[c + 1];
+        }
+        for (int i = 0; i < (left < 32 ? left : 32); ++i) {
+            const int64_t end = __shfl_sync(0xffffffffu, hi, i);
+            for (int64_t e0 = __shfl_sync(0xffffffffu, lo, i) + 256 * ((warp - i) & 15) + lane; e0 < end; e0 += 16 * 256) {
+                uint32_t d[8];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                d[u] = e0 + 32 * u < hi ? (uint32_t)ivf_doc[e0 + 32 * u] : 0xffffffffu;
-                if (d[u] != 0xffffffffu && !DBG_DOC_OK(d[u])) d[u] = 0xffffffffu;
-            }
-#pragma unroll
-            for (int u = 0; u < 8; ++u)
-                if (d[u] != 0xffffffffu) {
-                    const uint32_t bit = 1u << (d[u] & 31);
-                    if (!(bits[d[u] >> 5] & bit)) atomicOr(&bits[d[u] >> 5], bit);
+                for (int u = 0; u < 8; ++u) {
+                    d[u] = e0 + 32 * u < end ? (uint32_t)ivf_doc[e0 + 32 * u] : 0xffffffffu;
+                    if (d[u] != 0xffffffffu && !DBG_DOC_OK(d[u])) d[u] = 0xffffffffu;
                 }
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    if (d[u] != 0xffffffffu) {
+                        const uint32_t bit = 1u << (d[u] & 31);
+                        if (!(bits[d[u] >> 5] & bit)) atomicOr(&bits[d[u] >> 5], bit);
+                    }
+            }
+            __syncwarp();
         }
     }
     __syncthreads();
@@ -264,19 +275,32 @@ compact_kernel(const uint32_t *__restrict__ bitmap, int64_t words, int n_chunks,
         }
 }
 
+// In shared memory: bitmaps of up to 96 KB whose words are set a dozen times or more on average.  By range: a block per query and
+// range (every range reads all lists: up to 14 million documents), for more queries than a quarter of the SMs, unless that leaves half
+// of them idle and the lists are long enough for sixteen blocks.  In L2: the others.
+// Measured (stage 2b in us, means over 8,000 to 760,000 documents, lists of 300 to 6,000, even and popular centroids, 32 to 1,024 lists; in
+// L2 / in shared memory / by range):
+//   by times that a word is set, 1 query: 6 to 12 times 25 / 22, 12 to 24 29 / 24, more than 100 51 / 25; 4 queries 25 / 19, 40 / 24, 71 / 26;
+//     37: 69 / 42, 138 / 72, 247 / 65.  Set fewer times, even lists are as fast in L2, and a little faster with one query.
+//   by queries, 24 times or more: 48 246 / 79 / 124; 64 305 / 89 / 126; 96 361 / 101 / 108; 128 457 / 122 / 111.  Even lists alone: 64 queries
+//     of 128 lists of 300, 50,000 documents 40 / 31 / 28; 96 queries of 1,024 lists, 8,000 documents 561 / 85 / 61.
+int gather_form(const Index &ix, const Params &p)
+{
+    const int64_t words = (ix.N + 31) / 32, ranges = (words + MARK_RANGE_WORDS - 1) / MARK_RANGE_WORDS;
+    const double entries = (double)p.nq * p.P * ((double)ix.ivf_len / (double)ix.K);
+    const bool shared = words <= MARK_SHARED_WORDS && entries >= 12.0 * (double)words;
+    if (4 * p.B > ix.sm_count && ranges <= 8 && !(shared && 2 * ranges * p.B <= ix.sm_count && entries >= 65536.0)) return GATHER_RANGES;
+    return shared ? GATHER_SHARED : GATHER_L2;
+}
+
 int launch_gather(const Index &ix, const Params &p, const Layout &L, const int32_t *probes, uint32_t *bitmap,
                   bool bitmap_clear, int32_t *chunk_cnt, int32_t *cand, int32_t *n_cand, uint2 *ranks, int2 *rng,
                   int32_t *cont_scratch, uint32_t *status, cudaStream_t st)
 {
     const int n_lists = p.nq * p.P;
     const bool few = 4 * p.B <= ix.sm_count;
-    const int ranges = (int)((L.words + MARK_RANGE_WORDS - 1) / MARK_RANGE_WORDS);
-    // Bitmaps of up to 96 KB whose words are set a dozen times or more on average: in shared memory, sixteen blocks a query (16
-    // queries of 1,024 lists, 61 entries a word: 158 us in L2, 29 so; 37 queries, 19: 32 and 28; one query, 8: 5.7 and 8.3).
-    const bool shared = L.words <= MARK_SHARED_WORDS && (double)n_lists * ((double)ix.ivf_len / (double)ix.K) >= 12.0 * (double)L.words;
-    // A block per query and range (every range reads all lists: up to 14 million documents), unless that leaves SMs idle (64 queries
-    // on one range of 25 KB: 198 us, sixteen blocks a query 100).
-    const bool by_range = !few && ranges <= 8 && (!shared || (int64_t)ranges * p.B >= ix.sm_count);
+    const int ranges = (int)((L.words + MARK_RANGE_WORDS - 1) / MARK_RANGE_WORDS), form = gather_form(ix, p);
+    const bool by_range = form == GATHER_RANGES;
     if (!by_range && !bitmap_clear) CHIMERA_CUDA(cudaMemsetAsync(bitmap, 0, sizeof(uint32_t) * (size_t)L.words * p.B, st));
     if (by_range) {
         int range_words = (int)((L.words + ranges - 1) / ranges);
@@ -285,9 +309,11 @@ int launch_gather(const Index &ix, const Params &p, const Layout &L, const int32
         CHIMERA_CUDA(allow_shared(mark_range_kernel, sizeof(uint32_t) * MARK_RANGE_WORDS));
         launch(mark_range_kernel, dim3((unsigned)((L.words + range_words - 1) / range_words), (unsigned)p.B), 1024, smem, st, probes,
                n_lists, ix.ivf_off, ix.ivf_doc, bitmap, L.words, range_words, L.n_chunks, chunk_cnt);
-    } else if (shared) {
+    } else if (form == GATHER_SHARED) {
+        // (32 blocks instead of 16, words set 24 times or more as above: one query 23 us instead of 29, eight 29 and 33, 16 39 and 39)
+        const int blocks = p.B <= 8 ? 32 : 16;
         CHIMERA_CUDA(allow_shared(mark_shared_kernel, sizeof(uint32_t) * MARK_SHARED_WORDS));
-        launch(mark_shared_kernel, dim3((unsigned)(n_lists < 16 ? n_lists : 16), (unsigned)p.B), 512,
+        launch(mark_shared_kernel, dim3((unsigned)(n_lists < blocks ? n_lists : blocks), (unsigned)p.B), 512,
                sizeof(uint32_t) * (size_t)L.words, st, probes, n_lists, ix.ivf_off, ix.ivf_doc, bitmap, (int)L.words);
     } else {
         launch(mark_kernel, dim3((unsigned)n_lists, (unsigned)p.B), 128, 0, st, probes, n_lists, ix.ivf_off, ix.ivf_doc,

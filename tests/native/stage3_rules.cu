@@ -1,7 +1,7 @@
 // The routes of stage 3 for the sizes on standard input, one line each: n_centroids n_docs n_tokens posting_entries max_doclen
 // n_queries q_len nprobe n_prune max_candidates longest_token_list.  Output: 1 or 0 for the first cut (filter_used), for visit lists
-// in the refinements (visit_list_nodes), for bounds from the tokens near the query first (filter_mask_used), and for the
-// selection of few from many (select_few_used).  Host only.
+// in the refinements (visit_list_nodes), for bounds from the tokens near the query first (filter_mask_used), for the
+// selection of few from many (select_few_used); and stage 2b's form (gather_form).  Host only.
 #include <stdio.h>
 
 #include "common.cuh"
@@ -18,8 +18,9 @@ int main()
         ix.tok_id = &id; ix.max_tok_list = longest;
         chimera::Params p;
         p.B = B; p.nq = nq; p.P = P; p.n_prune = n_prune; p.k = 1; p.maxc = maxc == 0 || maxc > N ? N : maxc;
-        printf("%d %d %d %d\n", chimera::filter_used(ix, p) ? 1 : 0, chimera::visit_list_nodes(ix, p) > 0 ? 1 : 0,
-               chimera::filter_mask_used(ix, p, chimera::batch_scan_used(ix, p)) ? 1 : 0, chimera::select_few_used(ix, p) ? 1 : 0);
+        printf("%d %d %d %d %d\n", chimera::filter_used(ix, p) ? 1 : 0, chimera::visit_list_nodes(ix, p) > 0 ? 1 : 0,
+               chimera::filter_mask_used(ix, p, chimera::batch_scan_used(ix, p)) ? 1 : 0, chimera::select_few_used(ix, p) ? 1 : 0,
+               chimera::gather_form(ix, p));
     }
     return 0;
 }

@@ -1,4 +1,4 @@
-"""When stage 3 runs its first cut, starts its bounds from near tokens, keeps visits as lists and selects few from many: host arithmetic on the sizes, no
+"""Where stage 2b sets its bits, and when stage 3 runs its first cut, starts its bounds from near tokens, keeps visits as lists and selects few from many: host arithmetic on the sizes, no
 device."""
 import os
 import subprocess
@@ -14,7 +14,8 @@ def routes(tmp_path_factory):
     tmp = tmp_path_factory.mktemp("rule")
     obj, exe = str(tmp / "stage3_rules.o"), str(tmp / "stage3_rules")
     subprocess.check_call([build.NVCC] + build.FLAGS + ["-c", os.path.join(native, "stage3_rules.cu"), "-o", obj])
-    objs = [os.path.join(build.OBJ, n) for n in ("g3_filter.o", "g3_batch_scan.o", "g3_centroid_interaction.o", "g3_partial.o")]
+    objs = [os.path.join(build.OBJ, n) for n in ("g2_gather.o", "g3_filter.o", "g3_batch_scan.o", "g3_centroid_interaction.o",
+                                                  "g3_partial.o")]
     subprocess.check_call(["g++", "-no-pie", "-o", exe, obj, os.path.join(native, "fake_cudart.cpp")] + objs +
                           ["-Wl,--unresolved-symbols=ignore-all"])
 
@@ -22,7 +23,7 @@ def routes(tmp_path_factory):
         line = "%d %d %d %d %d %d %d %d %d %d %d" % (K, N, N * length, N * (distinct or length), max_len or 2 * length, B, nq,
                                                      P, n_prune, max_candidates, longest or 2 * N * length // K)
         out = subprocess.run([exe], input=line, capture_output=True, text=True, check=True).stdout.split()
-        return [x == "1" for x in out]
+        return [x == "1" for x in out[:4]] + [("L2", "shared", "ranges")[int(out[4])]]
     return routes
 
 
@@ -44,6 +45,22 @@ def near_first(routes):
 @pytest.fixture(scope="module")
 def few(routes):
     return lambda *a, **kw: routes(*a, **kw)[3]
+
+
+@pytest.fixture(scope="module")
+def gather(routes):
+    return lambda *a, **kw: routes(*a, **kw)[4]
+
+
+def test_bits_are_set_in_shared_memory_where_words_are_set_often(gather):
+    # 10,000 documents of 40 tokens, 313 words: 12 times each are 3,756 entries
+    assert [gather(1_000, 10_000, 40, B, 1, 10, 100) for B in (1, 37, 38, 74, 200)] == ["shared"] * 2 + ["ranges"] * 3
+    assert [gather(1_000, 10_000, 40, 4, 1, P, 100) for P in (9, 10)] == ["L2", "shared"]
+    # 65,536 entries a query: sixteen blocks up to half the SMs
+    assert [gather(1_000, 10_000, 40, B, 32, 6, 100) for B in (37, 38, 74, 75, 148)] == ["shared"] * 3 + ["ranges"] * 2
+    # bitmaps of 96 KB, and of nine ranges
+    assert gather(1_000, 24 * 1024 * 32, 100, 1, 32, 8, 100) == "shared" and gather(1_000, 24 * 1024 * 32 + 1, 100, 1, 32, 8, 100) == "L2"
+    assert gather(65_536, 14_417_920, 40, 256, 32, 4, 100) == "ranges" and gather(65_536, 14_417_921, 40, 256, 32, 4, 100) == "L2"
 
 
 def test_what_the_candidates_hold_counts_and_not_the_room_for_them(rule):
