@@ -273,8 +273,10 @@ score_table_umma(const int8_t *__restrict__ cdig, const __grid_constant__ CUtens
         if (!TABLE) {
             // Only the keys are wanted, and issue binds.  Warp w reads tensor-memory lanes 32 (w % 4) ... + 31 (a centroid a
             // thread) and the 16 columns from 16 (w / 4) on: column 8 o + 2 g + b is row 8 g + 2 o + b of the tile (table_row()).
-            // Eight copies of the push take fewer instructions than a mask of the passing rows and the selects of their values (357
-            // per warp and tile with those; Mid, batch 256: 617 -> 541 us).  Rows past the end have the largest threshold.
+            // Passing rows as a mask and one push in a loop: copies of the push cost the warp whenever a single lane takes one (stage 1 of
+            // 256 queries, 8,300 centroids 226 us so and 302 with copies, 17,000 307 and 370, 65,536 677 and 679 to 696).  Both halves are
+            // combined before either is looked at (one after the other 96 registers and spills: 685).  Rows past the end have the
+            // largest threshold.
             const uint32_t c = (uint32_t)c0 + (warp & 3) * 32 + lane;
             const int group = warp >> 2;
             const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + 16 * group;
@@ -295,21 +297,28 @@ score_table_umma(const int8_t *__restrict__ cdig, const __grid_constant__ CUtens
                 }
                 tmem_ld_wait();
                 hand_back();
+                int32_t out[2][8];
 #pragma unroll
-                for (int o = 0; o < 2; ++o) {
-                    int32_t out[8];
+                for (int o = 0; o < 2; ++o)
 #pragma unroll
                     for (int x = 0; x < 8; ++x)
-                        out[x] = combine_digits(accs[o][0][x], accs[o][1][x], accs[o][2][x], accs[o][3][x], accs[o][4][x]);
-                    if (c < n_cent) {
-                        bool any = false;
+                        out[o][x] = combine_digits(accs[o][0][x], accs[o][1][x], accs[o][2][x], accs[o][3][x], accs[o][4][x]);
 #pragma unroll
-                        for (int x = 0; x < 8; ++x) any |= out[x] >= thr_v[8 * o + x];
-                        if (any) {              // about nprobe x tile_stride keys per row in all: one lane of a warp every
-                                                // few chunks, and then hardly ever two values of the lane
+                for (int o = 0; o < 2; ++o) {
+                    bool any = false;
 #pragma unroll
-                            for (int x = 0; x < 8; ++x)
-                                if (out[x] >= thr_v[8 * o + x]) push(r0 + 8 * (x >> 1) + 2 * o + (x & 1), c, out[x]);
+                    for (int x = 0; x < 8; ++x) any |= out[o][x] >= thr_v[8 * o + x];
+                    if (any && c < n_cent) {
+                        uint32_t pass = 0u;
+#pragma unroll
+                        for (int x = 0; x < 8; ++x) pass |= out[o][x] >= thr_v[8 * o + x] ? 1u << x : 0u;
+                        while (pass) {
+                            const int x = __ffs(pass) - 1;
+                            pass &= pass - 1;
+                            int32_t v = out[o][0];
+#pragma unroll
+                            for (int y = 1; y < 8; ++y) v = x == y ? out[o][y] : v;
+                            push(r0 + 8 * (x >> 1) + 2 * o + (x & 1), c, v);
                         }
                     }
                 }
@@ -364,7 +373,7 @@ score_table_umma(const int8_t *__restrict__ cdig, const __grid_constant__ CUtens
                             uint32_t pass = 0u;
 #pragma unroll
                             for (int e = 0; e < 8; ++e) pass |= out[e] >= thr_v[e] ? 1u << e : 0u;
-                            while (pass) {          // (eight copies of the push, as above, are slower here: 768 -> 796 us)
+                            while (pass) {
                                 const int e = __ffs(pass) - 1;
                                 pass &= pass - 1;
                                 int32_t v = out[0];
