@@ -103,9 +103,9 @@ NCU_CI_DRAM_PER_ALGORITHMIC_BYTE = {
     "large": (1.243, "an ncu capture (Large recipe, 1M documents, batch 16)"),
     None: (0.939, "an ncu capture (Mid corpus, batch 8)"),
 }
-# ... and the same of the launches that bound and seed stage 3 when its first cut runs.
-NCU_CUT_DRAM_PER_ALGORITHMIC_BYTE = (0.883, "an ncu capture of the form that scans by query (Mid corpus, batch 64)")
-NCU_PARTIAL_DRAM_PER_QUERY = (463.5e6 / 64.0, "an ncu capture of the visits and their sums (Mid corpus, batch 64; bytes "
+# ... and the same of the launches that bound and seed stage 3 when its first cut scans by query.
+NCU_CUT_DRAM_PER_ALGORITHMIC_BYTE = (1.336, "an ncu capture of the form that scans by query (Mid corpus, batch 16)")
+NCU_PARTIAL_DRAM_PER_QUERY = (538.0e6 / 64.0, "an ncu capture of the visits and their sums (Mid corpus, batch 64; bytes "
                                             "per query)")
 
 
@@ -646,7 +646,12 @@ def measure(pkg, cfg, corp, q, index, args, device, mode="ci", dist=None, local_
     gbs = lambda nbytes, ms: nbytes / (ms * 1e-3) / 1e9 if ms > 0 else 0.0   # noqa: E731
     # algorithmic HBM bytes of one launch of the stage-3 bound scan: the centroid id of every candidate token (4 B) +
     # 8 B per candidate document (its token offsets); the kernel's own id / range / bound traffic is not the method's
-    ci_bytes = 4.0 * mean("cand_tokens") + 8.0 * mean("cand")
+    # Where the first cut scans queries side by side, the ids and offsets of the whole corpus once per such group instead.
+    together = index.cut_plan(B, nq, P, n_prune, k, maxc) if mode == "ci" else 0
+    cuts = together > 0 and mean("kept") < mean("cand")              # (a sample of the candidates can say no)
+    by_batch = cuts and together > 1
+    ci_bytes = (-(-B // together) * (4.0 * corp.cids.numel() + 8.0 * cfg.n_docs) if by_batch
+                else 4.0 * mean("cand_tokens") + 8.0 * mean("cand"))
     # what binds it (without the first cut): one table-row lookup per candidate token; a lookup is one distinct 128-byte line
     # for the SM's load pipe, which retires one line per cycle, so the roof is SMs x SM clock row lookups per second (derived
     # from the device's SM count and the clock sampled during the timed region; not a measured peak)
@@ -666,34 +671,36 @@ def measure(pkg, cfg, corp, q, index, args, device, mode="ci", dist=None, local_
         ratio, src = NCU_CI_DRAM_PER_ALGORITHMIC_BYTE.get(cfg.name, NCU_CI_DRAM_PER_ALGORITHMIC_BYTE[None])
         frac = gbs(ci_bytes, ci_ms) / peak
         # with the first cut stage 3's bounds are many launches instead of one
-        first_cut = launches["centroid_interaction"] >= 3 * n_prof
-        if first_cut:
+        rest = ("ci_bound_kernel + ci_rest_kernel + ci_wide_rng_kernel (stage 3: one number per token, 8-bit rows of the documents "
+                "that keeps, exact rows of the seeds)")
+        if cuts:
             ratio, src = NCU_CUT_DRAM_PER_ALGORITHMIC_BYTE
         roofline = {
-            "kernel": ("filter_scan_kernel or batch_scan_kernel + ci_bound_kernel + ci_rest_kernel + ci_wide_rng_kernel (stage 3: one "
-                       "number per candidate token, 8-bit rows of the documents that keeps, exact rows of the seeds)" if first_cut else
+            "kernel": ("batch_scan_kernel + " + rest if by_batch else "filter_scan_kernel + " + rest if cuts else
                        "ci_coarse_rng_kernel (stage 3 bound scan over every candidate token)"), "bound": "hbm",
             "achieved": gbs(ci_bytes, ci_ms), "peak": peak, "peak_kind": peak_kind, "unit": "GB/s", "frac": frac,
             "frac_of_nominal_8_tb_s": gbs(ci_bytes, ci_ms) / 8000.0,       # the task quotes ~8 TB/s; context only
-            "traffic": ratio * ci_bytes + (0.0 if first_cut else float(B) * cfg.n_centroids * nq),
-            "traffic_kind": "stored ncu figure, not measured in this run: %.3f DRAM bytes per algorithmic byte from %s, "
-                            "x this launch's algorithmic bytes%s" % (ratio, src, "" if first_cut else
+            "traffic": None if by_batch else ratio * ci_bytes + (0.0 if cuts else float(B) * cfg.n_centroids * nq),
+            "traffic_kind": None if by_batch else
+                            "stored ncu figure, not measured in this run: %.3f DRAM bytes per algorithmic byte from %s, "
+                            "x this launch's algorithmic bytes%s" % (ratio, src, "" if cuts else
                                                                      ", + each query's 8-bit table once"),
             "ms_per_launch": ci_ms, "algorithmic_bytes_per_launch": ci_bytes,
-            # (bytes are counted per query; a scan of the whole batch reads the ids once for all of its queries, so with the first
-            # cut the fraction can pass the target without the memory doing so: never claimed as met there)
-            "target": {"frac": TARGET, "met": bool(frac >= TARGET and not first_cut),
-                       "note": "the task's 60 %% of HBM peak for the code-scan stages is %s: every 4-byte centroid id "
-                               "costs a random lookup, in shared memory (about 3.5 bank conflicts each 32) or of a row "
-                               "through L1/L2, which binds the kernel%s" %
-                               ("met" if frac >= TARGET and not first_cut else "NOT met",
-                                "; bytes are per query, and a scan of the whole batch reads the ids once for all queries"
-                                if first_cut else "")},
+            # (by query, with the cut: the blocks of several queries read the same ids, so the fraction can pass the target without
+            # the memory doing so: never claimed as met there)
+            "queries_together": together if cuts else None,
+            "target": {"frac": TARGET, "met": bool(frac >= TARGET and not cuts),
+                       "note": "the task's 60 %% of HBM peak for the code-scan stages is %s: every 4-byte centroid id costs a random "
+                               "lookup, %s, which binds the kernel" %
+                               ("met" if frac >= TARGET and not cuts else "NOT met",
+                                "of a row of codes through L1/L2 that serves %d queries (bytes: the corpus's ids and offsets once "
+                                "for those)" % together if by_batch else
+                                "in shared memory (about 3.5 bank conflicts each 32)" if cuts else "of a row through L1/L2")},
             "contender_fraction": mean("contenders") / max(mean("cand"), 1.0),
             # with the first cut no single rate binds its launches (the lookups of filter_scan_kernel alone run at 71 % of
             # the shared-memory wavefront peak in an ncu capture)
-            "first_cut_kept_fraction": mean("kept") / max(mean("cand"), 1.0) if first_cut else None,
-            "binding_roof": None if first_cut else
+            "first_cut_kept_fraction": mean("kept") / max(mean("cand"), 1.0) if cuts else None,
+            "binding_roof": None if cuts else
                             {"bound": "table-row lookups (one 128-byte line per SM cycle); derived from SM count x sampled SM "
                                       "clock, not a measured peak",
                              "lookups_per_launch": rows, "achieved_glookups_s": rows / (ci_ms * 1e-3) / 1e9 if ci_ms > 0 else 0.0,
