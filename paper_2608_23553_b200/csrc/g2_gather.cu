@@ -40,8 +40,8 @@ mark_kernel(const int32_t *__restrict__ probes, int n_lists, const int64_t *__re
 
 // The same with the bitmap in shared memory, for small corpora: their lists set the same few words over and over, and
 // atomics on one L2 line come one after the other (10,000 documents, 128 lists of 625: 17 us, here 6.5).  grid (blocks, B): a
-// block takes every gridDim.x-th list and adds its bits to the query's bitmap at the end.  Its warps share a list, 256 entries
-// each, from another warp for the next list (a warp per list, the longest one took the time: one query, 400,000 documents, 1,024 lists
+// block takes every gridDim.x-th list and adds its bits to the query's bitmap at the end.  Its warps take the lists in
+// pieces of 256 entries (a warp per list, the longest one took the time: one query, 400,000 documents, 1,024 lists
 // of popular centroids, stage 2b 189 us in 16 blocks, 112 so and 70 in 32).
 constexpr int MARK_SHARED_WORDS = 24 * 1024;
 __global__ void __launch_bounds__(512)
@@ -55,29 +55,39 @@ mark_shared_kernel(const int32_t *__restrict__ probes, int n_lists, const int64_
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int l0 = blockIdx.x; l0 < n_lists; l0 += 32 * gridDim.x) {
-        const int l = l0 + lane * (int)gridDim.x, left = (n_lists - l0 + (int)gridDim.x - 1) / (int)gridDim.x;
-        int64_t lo = 0, hi = 0;                              // of this lane's list
+        const int l = l0 + lane * (int)gridDim.x;
+        int64_t lo = 0;                                      // of this lane's list
+        int len = 0;
         if (l < n_lists) {
             const int32_t c = DBG_CID(probes[(int64_t)b * n_lists + l]);
             lo = ivf_off[c];
-            hi = ivf_off[c + 1];
+            len = (int)(ivf_off[c + 1] - lo);
         }
-        for (int i = 0; i < (left < 32 ? left : 32); ++i) {
-            const int64_t end = __shfl_sync(0xffffffffu, hi, i);
-            for (int64_t e0 = __shfl_sync(0xffffffffu, lo, i) + 256 * ((warp - i) & 15) + lane; e0 < end; e0 += 16 * 256) {
-                uint32_t d[8];
+        const int pieces = (len + 255) >> 8;
+        int end = pieces;                                    // of this list's pieces among those of the 32
 #pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    d[u] = e0 + 32 * u < end ? (uint32_t)ivf_doc[e0 + 32 * u] : 0xffffffffu;
-                    if (d[u] != 0xffffffffu && !DBG_DOC_OK(d[u])) d[u] = 0xffffffffu;
-                }
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, end, o);
+            if (lane >= o) end += t;
+        }
+        const int all = __shfl_sync(0xffffffffu, end, 31);
+        for (int piece = warp; piece < all; piece += 16) {
+            const int i = __ffs(__ballot_sync(0xffffffffu, end > piece)) - 1;
+            const int from = 256 * (piece - __shfl_sync(0xffffffffu, end - pieces, i)) + lane;
+            const int left = __shfl_sync(0xffffffffu, len, i) - from;
+            const int32_t *src = ivf_doc + __shfl_sync(0xffffffffu, lo, i) + from;
+            uint32_t d[8];
 #pragma unroll
-                for (int u = 0; u < 8; ++u)
-                    if (d[u] != 0xffffffffu) {
-                        const uint32_t bit = 1u << (d[u] & 31);
-                        if (!(bits[d[u] >> 5] & bit)) atomicOr(&bits[d[u] >> 5], bit);
-                    }
+            for (int u = 0; u < 8; ++u) {
+                d[u] = 32 * u < left ? (uint32_t)src[32 * u] : 0xffffffffu;
+                if (d[u] != 0xffffffffu && !DBG_DOC_OK(d[u])) d[u] = 0xffffffffu;
             }
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (d[u] != 0xffffffffu) {
+                    const uint32_t bit = 1u << (d[u] & 31);
+                    if (!(bits[d[u] >> 5] & bit)) atomicOr(&bits[d[u] >> 5], bit);
+                }
             __syncwarp();
         }
     }
