@@ -812,6 +812,23 @@ int launch_cand_ranges(const Index &ix, const Params &p, const int32_t *cand, co
     return CHIMERA_OK;
 }
 
+// Blocks per query of a scan of 8-bit rows.  Four blocks are resident per SM and the blocks of a query are adjacent in the grid, so
+// (resident blocks) / (blocks per query) queries are scanned at the same time and their 8-bit tables compete for
+// L2: enough blocks per query to keep those tables within COARSE_L2_TABLES bytes, at least enough to fill the GPU
+// when the batch is small, never more than one warp per candidate.  Measured on the Mid corpus at batch 256
+// (2 MB tables): 4 blocks per query 57 ms, 16: 23.4, 24: 18.9, 37: 16.5, 74: 16.6, 148: 16.7, 1184: 17.6; a budget
+// of 16 MB against 32 MB: Mid 16.56 / 16.52 ms, Large (8 MB tables) 36.6 / 37.2 ms; 64 MB: 21.3 and 46.7 ms.
+static int64_t coarse_blocks(const Index &ix, const Params &p)
+{
+    constexpr int64_t COARSE_L2_TABLES = 16LL << 20;
+    const int64_t resident = 4LL * ix.sm_count;
+    const int64_t want = (p.maxc + CI_WARPS - 1) / CI_WARPS;
+    int64_t per_query = (resident * ix.K * coarse_pitch(p.nq) + COARSE_L2_TABLES - 1) / COARSE_L2_TABLES;
+    const int64_t to_fill = (2 * resident + p.B - 1) / p.B;      // two waves when the batch is small
+    if (per_query < to_fill) per_query = to_fill;
+    if (per_query > want) per_query = want;
+    return per_query < 1 ? 1 : per_query;
+}
 int launch_coarse_bounds(const Index &ix, const Params &p, const uint8_t *table8, const int32_t *cand,
                          const int32_t *n_cand, int32_t *lo, int32_t *hi, const int2 *rng, const FirstCut *cut, cudaStream_t st)
 {
@@ -844,22 +861,7 @@ int launch_coarse_bounds(const Index &ix, const Params &p, const uint8_t *table8
         count_launch(SLOT_CI);
         return CHIMERA_OK;
     }
-    // Blocks per query.  Four blocks are resident per SM and the blocks of a query are adjacent in the grid, so
-    // (resident blocks) / (blocks per query) queries are scanned at the same time and their 8-bit tables compete for
-    // L2: enough blocks per query to keep those tables within COARSE_L2_TABLES bytes, at least enough to fill the GPU
-    // when the batch is small, never more than one warp per candidate.  Measured on the Mid corpus at batch 256
-    // (2 MB tables): 4 blocks per query 57 ms, 16: 23.4, 24: 18.9, 37: 16.5, 74: 16.6, 148: 16.7, 1184: 17.6; a budget
-    // of 16 MB against 32 MB: Mid 16.56 / 16.52 ms, Large (8 MB tables) 36.6 / 37.2 ms; 64 MB: 21.3 and 46.7 ms.
-    constexpr int64_t COARSE_L2_TABLES = 16LL << 20;
-    const int64_t resident = 4LL * ix.sm_count;
-    const int64_t want = (p.maxc + CI_WARPS - 1) / CI_WARPS;
-    int64_t per_query = (resident * (int64_t)table_bytes + COARSE_L2_TABLES - 1) / COARSE_L2_TABLES;
-    const int64_t to_fill = (2 * resident + p.B - 1) / p.B;      // two waves when the batch is small
-    if (per_query < to_fill) per_query = to_fill;
-    if (per_query > want) per_query = want;
-    if (per_query < 1) per_query = 1;
-    const unsigned gx = (unsigned)per_query;
-    dim3 grid(gx, (unsigned)p.B);
+    dim3 grid((unsigned)coarse_blocks(ix, p), (unsigned)p.B);
     if (use_rng) {
         if (p.nq == 32)
             launch(ci_coarse_rng_kernel<2>, grid, CI_THREADS, 0, st, table8, ix.K, rng, n_cand, p.maxc, ix.cids, lo, hi, call_cut);
@@ -907,8 +909,9 @@ int launch_kept_bounds(const Index &ix, const Params &p, const uint8_t *table8, 
         gx = (8LL * ix.sm_count + p.B - 1) / p.B;            // of one or two n_prune documents a query
         if (gx < p.n_prune / 32) gx = p.n_prune / 32;
     } else {
-        gx = (8LL * ix.sm_count + p.B - 1) / p.B;
-        if (gx < ix.sm_count / 2) gx = ix.sm_count / 2;
+        // (of all rows: half the SMs' number of blocks regardless of the tables, 19 queries of 262,144 centroids and 64-byte rows 525 -> 766 us,
+        // 31 of 51,588 and 128 1,353 -> 1,733, 14 of 107,614 and 32 284 -> 349)
+        gx = coarse_blocks(ix, p);
     }
     if (gx > want) gx = want;
     auto rest_kern = p.nq <= 32 ? ci_rest_kernel<2> : p.nq <= 64 ? ci_rest_kernel<4> : ci_rest_kernel<8>;

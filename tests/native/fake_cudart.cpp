@@ -10,6 +10,7 @@
 std::set<void *> fake_live;
 std::map<const void *, std::set<int>> fake_limits;       // dynamic shared memory allowed, of each kernel
 std::map<const void *, std::set<size_t>> fake_shared;    // ... and asked for
+unsigned fake_blocks;                                    // of the last launch in a row of its grid
 int fake_calls = 0, fake_fail_at = 0, fake_last_error = 0;
 
 static int step()
@@ -42,6 +43,7 @@ struct fake_config { unsigned grid[3], block[3]; size_t shared; };
 int cudaLaunchKernelExC(const fake_config *c, const void *kernel, void **)
 {
     fake_shared[kernel].insert(c->shared);
+    fake_blocks = c->grid[0];
     return step();
 }
 int cudaFuncSetAttribute(const void *kernel, int, int bytes)

@@ -23,7 +23,7 @@ def routes(tmp_path_factory):
         line = "%d %d %d %d %d %d %d %d %d %d %d" % (K, N, N * length, N * (distinct or length), max_len or 2 * length, B, nq,
                                                      P, n_prune, max_candidates, longest or 2 * N * length // K)
         out = subprocess.run([exe], input=line, capture_output=True, text=True, check=True).stdout.split()
-        return [x == "1" for x in out[:4]] + [("L2", "shared", "ranges")[int(out[4])]]
+        return [x == "1" for x in out[:4]] + [("L2", "shared", "ranges")[int(out[4])], int(out[5])]
     return routes
 
 
@@ -50,6 +50,14 @@ def few(routes):
 @pytest.fixture(scope="module")
 def gather(routes):
     return lambda *a, **kw: routes(*a, **kw)[4]
+
+
+@pytest.mark.parametrize("K,N,length,B,nq,P,n_prune", [(262_144, 1_279_581, 128, 19, 40, 2, 1_235), (51_588, 357_950, 114, 31, 120, 2, 251),
+                                                        (107_614, 1_572_938, 30, 14, 32, 22, 1_315), (65_536, 500_000, 120, 40, 32, 4, 1_024)])
+def test_tables_of_the_queries_looked_up_at_once_stay_in_l2(routes, K, N, length, B, nq, P, n_prune):
+    rows = 32 if nq <= 32 else 64 if nq <= 64 else 128
+    blocks = routes(K, N, length, B, nq, P, n_prune)[5]
+    assert 4 * 148 / blocks * K * rows <= 1.1 * (16 << 20) or blocks >= 4 * 148       # four blocks per SM
 
 
 def test_bits_are_set_in_shared_memory_where_words_are_set_often(gather):
