@@ -162,9 +162,11 @@ size_t filter_parts_bytes(const Index &ix, const Params &p)
 // `rank` of the m sampled rows (every step-th one) have S >= t 2^16.  With few queries the sample is split over several
 // blocks that add their histograms up in `parts_hist` ([B][groups][256 * 32], cleared before); the last one to
 // finish (`done`, likewise) reads the sum.  Also clears what the scan and the seed selection add to, and the sample's words (vote,
-// may be NULL).  table8 (may be NULL): the 8-bit rows, which hold all that is read here in a quarter of the bytes.
+// may be NULL).  Row: uint8_t, of the 8-bit table, which holds all that is read here in a quarter of the bytes, or int32_t (a choice made
+// at each load instead of by the type cost the latter a third: 120 tokens, 31 queries 59 -> 72 us).
+template <class Row>
 __global__ void __launch_bounds__(SEL_THREADS)
-filter_theta_kernel(const int32_t *__restrict__ table, const uint8_t *__restrict__ table8, int64_t K, int nq, int m, int step, int rank,
+filter_theta_kernel(const Row *__restrict__ table, int64_t K, int nq, int m, int step, int rank,
                     int32_t *__restrict__ theta, int32_t *__restrict__ hist_out, int32_t *__restrict__ n_seed,
                     int32_t *__restrict__ parts_hist, int32_t *__restrict__ done, int32_t *__restrict__ vote)
 {
@@ -180,15 +182,14 @@ filter_theta_kernel(const int32_t *__restrict__ table, const uint8_t *__restrict
         if (threadIdx.x == 0) n_seed[b] = 0;
     }
     __syncthreads();
-    const int32_t *tb = table + (int64_t)b * K * nq + col;
-    const uint8_t *tb8 = table8 + (int64_t)b * K * nq + col;
+    const Row *tb = table + (int64_t)b * K * nq + col;
     const int64_t row = (int64_t)step * nq;
     for (int r0 = blockIdx.z * 32 + warp; r0 < m; r0 += gridDim.z * 32 * 16) {
         int k[16];
 #pragma unroll
         for (int u = 0; u < 16; ++u) {
             const int r = r0 + gridDim.z * 32 * u;
-            k[u] = r >= m || col >= nq ? 0 : table8 ? (int)tb8[r * row] : tb[r * row] >> 16;
+            k[u] = r >= m || col >= nq ? 0 : sizeof(Row) == 1 ? (int)tb[r * row] : (int)tb[r * row] >> 16;
         }
 #pragma unroll
         for (int u = 0; u < 16; ++u)
@@ -1047,8 +1048,13 @@ int launch_filter_scan(const Index &ix, const Params &p, const Layout &L, bool b
     int32_t *parts_hist = (int32_t *)(ws + L.flt_parts), *done = parts_hist + (size_t)p.B * groups * 256 * 32;
     if (parts > 1)
         CHIMERA_CUDA(cudaMemsetAsync(parts_hist, 0, filter_parts_bytes(ix, p), st));
-    launch(filter_theta_kernel, dim3(groups, (unsigned)p.B, (unsigned)parts), SEL_THREADS, 0, st, table, ready ? table8 : nullptr, ix.K, p.nq, m, step, rank, theta, hist, n_seed, parts_hist, done,
-           ready ? vote : nullptr);
+    const dim3 grid(groups, (unsigned)p.B, (unsigned)parts);
+    if (ready)
+        launch(filter_theta_kernel<uint8_t>, grid, SEL_THREADS, 0, st, (const uint8_t *)table8, ix.K, p.nq, m, step, rank, theta, hist, n_seed,
+               parts_hist, done, vote);
+    else
+        launch(filter_theta_kernel<int32_t>, grid, SEL_THREADS, 0, st, table, ix.K, p.nq, m, step, rank, theta, hist, n_seed, parts_hist, done,
+               (int32_t *)nullptr);
     CHIMERA_CUDA(cudaGetLastError());
     const int us = filter_unit(ix, p, ready);
     int rc;
