@@ -266,13 +266,27 @@ compact_kernel(const uint32_t *__restrict__ bitmap, int64_t words, int n_chunks,
     if (!use_stage) {
         __syncthreads();
         const int lane = threadIdx.x & 31;
-        for (int i = threadIdx.x >> 5; i < chunk_words; i += CHUNK_THREADS / 32) {
-            const uint2 s = starts[i];
-            const int64_t at = (int64_t)s.y + __popc(s.x & ((1u << lane) - 1u));
-            if ((s.x >> lane & 1u) && at < maxc) {
-                const int32_t id = (int32_t)((((int64_t)blockIdx.x * chunk_words + i) << 5) + lane);
-                out[at] = id;
-                if (rng) rng[(int64_t)b * maxc + at] = doc_range(doc_off, id);
+        constexpr int W = 4;                                 // words in flight
+        for (int i0 = threadIdx.x >> 5; i0 < chunk_words; i0 += W * (CHUNK_THREADS / 32)) {
+            int64_t at[W];
+            int32_t id[W];
+#pragma unroll
+            for (int u = 0; u < W; ++u) {
+                const int i = i0 + u * (CHUNK_THREADS / 32);
+                const uint2 s = i < chunk_words ? starts[i] : make_uint2(0u, 0u);
+                at[u] = s.x >> lane & 1u ? (int64_t)s.y + __popc(s.x & ((1u << lane) - 1u)) : maxc;
+                id[u] = (int32_t)((((int64_t)blockIdx.x * chunk_words + i) << 5) + lane);
+            }
+#pragma unroll
+            for (int u = 0; u < W; ++u)
+                if (at[u] < maxc) out[at[u]] = id[u];
+            if (rng) {
+                int2 r[W];
+#pragma unroll
+                for (int u = 0; u < W; ++u) r[u] = at[u] < maxc ? doc_range(doc_off, id[u]) : make_int2(0, 0);
+#pragma unroll
+                for (int u = 0; u < W; ++u)
+                    if (at[u] < maxc) rng[(int64_t)b * maxc + at[u]] = r[u];
             }
         }
         return;
