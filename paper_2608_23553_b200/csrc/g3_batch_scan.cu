@@ -39,14 +39,17 @@ static int batch_groups(const Params &p) { return (p.B + batch_group(p) - 1) / b
 // When a batch is scanned this way: by the SM cycles of both forms.  Cycles a token and SM by the bytes of a row, measured on
 // 200,000 to 500,000 documents: 8 bytes 0.95, 16 1.2, 32 1.3, 64 1.4, 128 2.4, 256 4.3 (a line of the load pipe, then what L2
 // delivers).  The scan by query takes 4.3 tokens a cycle from 16-bit values and 2.2 from 6-bit codes, of the candidates only.  The
-// table has to stay in L2 beside what streams past: 32 of its 126 MB.
+// table has to stay in L2 beside what streams past: 32 of its 126 MB.  Query lengths other than 32 and 64 have no 8-bit table when the
+// step is chosen, and pay 10 to 20 us for its rows: 3 million token cycles (224 calls on 8,000 to 150,000 documents, both forms: without
+// that, 21 tokens lost up to 10 % of a call and 106 up to 9 %; with it nothing loses more than 1 %).
 bool batch_scan_used(const Index &ix, const Params &p)
 {
     if (!filter_used(ix, p) || ix.max_doclen > BS_MAX_LEN) return false;
     const int row = batch_group(p);
     if ((int64_t)row * ix.K > (32LL << 20)) return false;
     const double cycles = row == 8 ? 0.95 : row == 16 ? 1.2 : row == 32 ? 1.3 : row == 64 ? 1.4 : row == 128 ? 2.4 : 4.3;
-    return batch_groups(p) * (double)ix.T * cycles < (double)p.B * expected_tokens(ix, p) / (ix.K <= 106496 ? 4.3 : 2.2);
+    const double fixed = coarse_supported(p.nq) ? 0.0 : 3e6;
+    return batch_groups(p) * (double)ix.T * cycles + fixed < (double)p.B * expected_tokens(ix, p) / (ix.K <= 106496 ? 4.3 : 2.2);
 }
 size_t batch_table_bytes(const Index &ix, const Params &p)
 {

@@ -8,9 +8,10 @@ import oracle
 from helpers import random_corpus
 from parity import check_query, taps_to_numpy
 
-# D, q_len, centroids, documents, shortest, longest, queries, nprobe, n_prune
+# D, q_len, centroids, documents, shortest, longest, queries, nprobe, n_prune  (80,000 documents: other lengths than 32 and 64 take this
+# form from 3 million saved token cycles on, batch_scan_used)
 CALLS = [
-    (32, 21, 700, 20_000, 1, 99, 8, 8, 100),             # 8-byte rows
+    (32, 21, 700, 80_000, 1, 99, 8, 8, 100),             # 8-byte rows
     (32, 32, 900, 64 * 400 + 1, 30, 99, 16, 8, 60),      # 16; one document behind the last whole tile
     (64, 64, 1_001, 64 * 300 - 1, 40, 90, 32, 4, 60),    # 32
     (32, 32, 900, 64 * 250 + 33, 1, 120, 61, 8, 50),     # 64
@@ -18,7 +19,7 @@ CALLS = [
     (64, 32, 2_000, 12_345, 20, 80, 129, 8, 100),        # 256, half of them empty
     (32, 32, 513, 7_777, 1, 99, 259, 4, 80),             # two groups
     (32, 32, 2_049, 3_000, 900, 1_040, 24, 2, 40),       # the longest documents
-    (96, 47, 700, 9_000, 1, 90, 9, 6, 60),
+    (96, 47, 700, 80_001, 1, 90, 9, 6, 60),
 ]
 
 
